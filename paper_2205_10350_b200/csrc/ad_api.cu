@@ -12,7 +12,9 @@
 
 #include "ad_common.cuh"
 #include "attention.cuh"
+#include "attention_few.cuh"
 #include "attention_mma.cuh"
+#include "gemm_few.cuh"
 #include "gemm_simt.cuh"
 #include "gemm_tc.cuh"
 #include "gemm_tc_persistent.cuh"
@@ -63,6 +65,9 @@ struct Model {
   void* ckv_pack = nullptr;
   float* cbkv_pack = nullptr;
 };
+// Passes of at most this many packed tokens run their projections on the few-token kernel (gemm_few.cuh).
+constexpr int kFewTokens = 128;
+
 struct PassCfg {
   int M_cap = 0;     // packed-token capacity of this pass kind
   int ntile = 16;    // tokens per GEMM tile
@@ -538,6 +543,24 @@ cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw, cons
                   stages);
 }
 
+// Projection of a pass with few tokens (gemm_few.cuh).  ksplit: few::split_for of the shape, non-zero.
+template <int EPI>
+cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p, int ksplit) {
+  const dim3 grid(p.N / few::FEAT, ksplit);
+  const bf16 *w = (const bf16*)W.ptr, *xp = (const bf16*)x;
+  switch (p.K / ksplit / 256) {
+    case 1: return launch_k(few::gemm_few_kernel<EPI, 1>, grid, dim3(few::THREADS), 0, st, w, xp, p);
+    case 2: return launch_k(few::gemm_few_kernel<EPI, 2>, grid, dim3(few::THREADS), 0, st, w, xp, p);
+    case 3: return launch_k(few::gemm_few_kernel<EPI, 3>, grid, dim3(few::THREADS), 0, st, w, xp, p);
+    default: return launch_k(few::gemm_few_kernel<EPI, 4>, grid, dim3(few::THREADS), 0, st, w, xp, p);
+  }
+}
+// K split the few-token kernel takes for a projection of pass pc (0: the pass or the shape is not for it).
+int few_split(const PassCfg& pc, int epi, int N, int K) {
+  if (pc.M_cap > kFewTokens || epi == EPI_ARGMAX) return 0;
+  return few::split_for(N, K, epi == EPI_F32, pc.max_split);
+}
+
 template <int EPI>
 cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const GemmParams& p, int M_cap) {
   dim3 grid((p.N + 127) / 128, (M_cap + simt::TOK - 1) / simt::TOK);
@@ -553,7 +576,15 @@ int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int
     snprintf(nm, sizeof(nm), "%s N%d K%d", epi_name[epi & 3], W.N, W.K);
     note_launch(h, nm);
   }
-  if (h->bf16) {
+  // (p.ksplit == 0: the caller wants one full-K result whatever the pass, see ad_debug_logits)
+  const int fs = h->bf16 && (epi != EPI_F32 || p.ksplit > 0) && (epi == EPI_F32 || p.bias) ? few_split(h->pass[pk], epi, W.N, W.K) : 0;
+  if (fs > 0) {
+    switch (epi) {
+      case EPI_F32: e = launch_few<EPI_F32>(h->stream, W, X.ptr, p, fs); break;
+      case EPI_ACT: e = launch_few<EPI_ACT>(h->stream, W, X.ptr, p, fs); break;
+      default: e = launch_few<EPI_SCATTER>(h->stream, W, X.ptr, p, fs); break;
+    }
+  } else if (h->bf16) {
     p.ntile = h->pass[pk].tile_for(W.N, num_sms());
     const CUtensorMap& mx = X.map_for(pk, p.ntile);
     if (epi != EPI_F32) p.ksplit = 1;
@@ -679,6 +710,53 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   return AD_OK;
 }
 
+// Whether the few-query kernel (attention_few.cuh) serves an attention of pass pc: BF16, 64-wide heads, the keys within two
+// rounds of its warps, and a grid of at most one wave.
+bool attention_is_few(const ad_handle* h, const PassCfg& pc, int max_keys) {
+  const ad_model_cfg& c = h->cfg;
+  if (!g_fuse_attn_proj || !h->bf16 || !h->pre2 || c.d_model != c.n_heads * 64 || c.d_model % 128 || c.n_heads > few::MAX_WARPS) return false;
+  if (max_keys > 2 * few::AK * c.n_heads) return false;
+  return (long)h->cfg.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads <= num_sms();
+}
+
+// Attention with its output projection (partial sums per head in pre2) and, with wq, the query projection of x = yb.
+int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v, const int* key_base, const int* nkeys_tok,
+                  const int* nkeys_row, const Mat& wo, const Mat* wq = nullptr, const float* q_bias = nullptr) {
+  const ad_model_cfg& c = h->cfg;
+  few::FewAttnParams fp = {};
+  AttnParams& p = fp.a;
+  p.q = h->qbuf; p.k = k; p.v = v; p.q_bias = q_bias;
+  p.seg_off = pc.plan.seg_off; p.seg_len = pc.plan.seg_len;
+  p.key_base = key_base; p.nkeys_tok = nkeys_tok; p.nkeys_row = nkeys_row;
+  p.d = c.d_model; p.scale = 0.125f;
+  p.qchunks = (pc.seg_max + few::AQ - 1) / few::AQ;
+  p.wo = (const bf16*)wo.ptr; p.o_part = h->pre2; p.o_stride = (size_t)pc.M_cap * c.d_model;
+  if (wq) { fp.x = (const bf16*)h->yb.ptr; fp.wq = (const bf16*)wq->ptr; }
+  const dim3 grid(h->dims.B * p.qchunks, c.n_heads), block(32 * c.n_heads);
+  const size_t smem = few::att_few_smem(c.n_heads);
+  static bool attr_set[kMaxDevices] = {};
+  const int dev = current_device();
+  cudaError_t e = cudaSuccess;
+  if (!attr_set[dev]) {
+    const int most8 = (int)few::att_few_smem(8), most16 = (int)few::att_few_smem(16);
+    e = cudaFuncSetAttribute(few::attention_few_kernel<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most8);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(few::attention_few_kernel<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most8);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(few::attention_few_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most16);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(few::attention_few_kernel<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most16);
+    if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention attribute: ") + cudaGetErrorString(e));
+    attr_set[dev] = true;
+  }
+  note_launch(h, wq ? "q_proj+attention+out_proj" : "attention+out_proj");
+  if (c.n_heads <= 8)
+    e = wq ? launch_k(few::attention_few_kernel<true, 8>, grid, block, smem, h->stream, fp)
+           : launch_k(few::attention_few_kernel<false, 8>, grid, block, smem, h->stream, fp);
+  else
+    e = wq ? launch_k(few::attention_few_kernel<true, 16>, grid, block, smem, h->stream, fp)
+           : launch_k(few::attention_few_kernel<false, 16>, grid, block, smem, h->stream, fp);
+  if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
+  return AD_OK;
+}
+
 // y = LN(sum of the nsplit partial projections in `pre` + bias + y)
 int layernorm(ad_handle* h, const PassCfg& pc, int nsplit, const float* bias, const float* g, const float* b,
               const float* partials = nullptr) {
@@ -711,7 +789,8 @@ int gemm_to_ln(ad_handle* h, const Mat& W, const ActBuf& X, int pk, int* nsplit)
   PassCfg& pc = h->pass[pk];
   GemmParams o = {};
   o.out_f32 = h->pre;
-  o.ksplit = h->bf16 ? pc.ksplit_for(W.N, W.K, pc.tile_for(W.N, num_sms())) : 1;
+  o.ksplit = h->bf16 ? few_split(pc, EPI_F32, W.N, W.K) : 1;
+  if (o.ksplit == 0) o.ksplit = pc.ksplit_for(W.N, W.K, pc.tile_for(W.N, num_sms()));
   *nsplit = o.ksplit;
   return gemm(h, EPI_F32, W, X, pk, pc.plan.M, pc.M_cap, o);
 }
@@ -738,8 +817,12 @@ int self_attention_sublayer(ad_handle* h, int pk, const Mat& wqkv, const float* 
   p.slot = pc.plan.kv_slot;
   AD_TRY(gemm(h, EPI_SCATTER, wqkv, h->yb, pk, pc.plan.M, pc.M_cap, p));
   bool fused = false;
-  AD_TRY(attention(h, pc, h->qbuf, kbuf, vbuf, h->abuf.ptr, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk,
-                   pk == PK_VERIFY ? h->dims.max_tgt : pc.seg_max, nullptr, 0, &wo, &fused));
+  const int max_keys = pk == PK_VERIFY ? h->dims.max_tgt : pc.seg_max;
+  if (attention_is_few(h, pc, max_keys)) {
+    AD_TRY(attention_few(h, pc, kbuf, vbuf, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, wo));
+    return layernorm(h, pc, h->cfg.n_heads, bo, lng, lnb, h->pre2);
+  }
+  AD_TRY(attention(h, pc, h->qbuf, kbuf, vbuf, h->abuf.ptr, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, max_keys, nullptr, 0, &wo, &fused));
   if (fused) return layernorm(h, pc, h->cfg.n_heads, bo, lng, lnb, h->pre2);
   int ns = 1;
   AD_TRY(gemm_to_ln(h, wo, h->abuf, pk, &ns));
@@ -903,6 +986,13 @@ int decoder_pass(ad_handle* h, int pk, Model& m) {
     // projection, so it is split along K and the attention kernel adds the partial sums (and the bias) as it
     // loads its queries.
     bool fused_x = false;
+    if (attention_is_few(h, pc, c.max_src)) {
+      AD_TRY(attention_few(h, pc, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->st.cross_base, nullptr, h->st.srclen,
+                           L.co, &L.cq, L.cbq));
+      AD_TRY(layernorm(h, pc, c.n_heads, L.cbo, L.ln2g, L.ln2b, h->pre2));
+      AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b));
+      continue;
+    }
     int qs = h->bf16 && pc.M_cap <= 256 ? pc.ksplit_for(L.cq.N, L.cq.K, pc.tile_for(L.cq.N, num_sms())) : 1;
     if (qs > 1 && qs <= ATT_MAX_QSPLIT) {
       int ns_q = 1;

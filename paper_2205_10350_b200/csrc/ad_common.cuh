@@ -89,6 +89,16 @@ struct GemmParams {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Plan data.  The kernels that lay a pass out (plan_*, prepare_verify, and the accept kernel when it plans the next block)
+// never call pdl_launch(): a kernel behind one of them can only start once it has completed, and every later kernel of the
+// pass starts later still.  What they write -- PassPlan, the row state, and with it everything older, such as the encoder's
+// keys and values -- may therefore be read BEFORE pdl_wait(), off the critical path.  Read past L1, which may hold the
+// previous pass's lines.
+__device__ __forceinline__ int plan_load(const int* p) { return __ldcg(p); }
+// Early exits.  A CTA that the plan gives no work leaves before pdl_wait(), so that it does not hold an SM's resources
+// while the predecessor runs.  One CTA of the grid always waits, work or not: a grid that completed before its predecessor
+// would release its own successors too early.
+
 // Optional timeline tracing (compile with -DAD_TRACE): thread 0 of CTA (0,0,0) of every kernel stamps the
 // global nanosecond timer at entry (phase 0), after the dependency wait (phase 1), at exit (phase 2) and at
 // kernel-specific points in between (phases 3..7); the last CTA along x does the same under id + 16.

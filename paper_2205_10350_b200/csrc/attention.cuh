@@ -101,9 +101,8 @@ constexpr size_t att_smem_bytes() {
 // grid = (B * qchunks, H); block = 256 threads (8 warps, QPW queries each; a CTA covers 8 * QPW queries of one
 // row and one head and stages every K/V tile once for all of them).  QPW = 1 keeps the critical path short when
 // there are few queries; QPW = 8 amortises the K/V staging when there are thousands.
-// Global-memory round trips on the critical path: (1) the row's segment / key-range descriptors,
-// (2) the queries, their key counts and the first K/V tile together (the tile's loads are issued first and only
-// widened once the queries are in shared memory), then compute and store.
+// Global-memory round trips after the dependency wait: the queries and the first K/V tile together (the tile's loads are
+// issued first and only widened once the queries are in shared memory), then compute and store.
 // FUSE (BF16, 64-wide heads, one query per warp): the output projection of the 8 queries is done here as well (see
 // AttnParams::wo).  Warp w owns output features [w d / 8, (w + 1) d / 8); its weight fragments -- 16 rows x 64 columns
 // per group of rows, read with 16-byte loads whose eight elements are consecutive in K (the contraction index is
@@ -142,16 +141,17 @@ attention_kernel(const AttnParams p) {
         }
       }
   }
-  pdl_wait();
-  trace_mark(TR_ATTN, 1);
   const int b = blockIdx.x / p.qchunks;
   const int chunk = blockIdx.x % p.qchunks;
   const int h = blockIdx.y;
-  const int seg_len = p.seg_len[b];
-  const int seg_off = p.seg_off[b];
-  const int kbase = p.key_base[b];
-  const int row_nk = p.nkeys_row[b];         // no token of this row sees more keys than this
+  const int seg_len = plan_load(p.seg_len + b);
+  const int seg_off = plan_load(p.seg_off + b);
+  const int kbase = plan_load(p.key_base + b);
+  const int row_nk = plan_load(p.nkeys_row + b);   // no token of this row sees more keys than this
   const int i0 = chunk * QC;
+  if (i0 >= seg_len && (blockIdx.x | blockIdx.y) != 0) return;
+  pdl_wait();
+  trace_mark(TR_ATTN, 1);
   if (i0 >= seg_len) return;
   const int nq = min(QC, seg_len - i0);
   const int m0 = seg_off + i0;

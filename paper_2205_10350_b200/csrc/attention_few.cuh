@@ -1,0 +1,319 @@
+// Attention of passes with few queries per row (BF16, 64-wide heads), output projection included and, for the
+// cross-attention, the query projection as well.
+//
+// A CTA handles one head and up to 16 queries of one row.  Everything is latency: a few dozen keys, a few thousand
+// multiply-adds.  The CTA's d / 64 warps therefore split whatever there is to split: the contraction of the query
+// projection (64 input features per warp), the keys (16 per warp and round), the output features of the output projection
+// (64 per warp).  All products are warp-level MMAs on fragments read with 16-byte loads (contraction index permuted
+// identically for both operands, see gemm_few.cuh).  Weights, and for the cross-attention the keys and values (written
+// by the encoder pass long before), are requested before the dependency wait; plan data is read there too.
+//
+// The FFMA kernel it replaces for these shapes (attention.cuh: one query per warp, keys staged as FP32) took 4.4 us after
+// its dependency wait inside a 40-token step of a 512-wide model, and the cross-attention's query projection was a kernel
+// of its own (2.3 us and a kernel boundary).
+//
+// Probabilities multiply the values as a sum of two BF16 numbers (p = hi + lo), so nothing is lost against FP32
+// probabilities; queries and the output that enters the projection are rounded to BF16 exactly where a stored operand
+// would be.
+#pragma once
+
+#include "attention.cuh"
+#include "gemm_few.cuh"
+
+namespace ad {
+namespace few {
+
+constexpr int AQ = 16;            // queries per CTA = MMA M
+constexpr int AK = 16;            // keys per warp and round
+constexpr int K_LD = 96;          // key rows: 192 bytes apart (16-byte fragment loads without bank conflicts)
+constexpr int V_LD = 72;          // value rows: 144 bytes apart (ldmatrix without bank conflicts)
+constexpr int O_LD = 68;          // floats per row of a warp's partial output
+constexpr int MAX_WARPS = 16;
+
+struct FewAttnParams {
+  AttnParams a;
+  const bf16* x;        // query projection: its input [M_cap, d] (normalised hidden states) ...
+  const bf16* wq;       // ... and weights [d, d]; null: the queries are in a.q
+};
+
+inline size_t att_few_smem(int warps) {
+  const size_t kv = (size_t)warps * AK * (K_LD + V_LD) * sizeof(bf16);
+  const size_t part = (size_t)warps * AQ * O_LD * sizeof(float);      // partial query projections, later partial outputs
+  return kv + part + 2 * (size_t)warps * AQ * sizeof(float) + 2 * (size_t)AQ * K_LD * sizeof(bf16);
+}
+
+__device__ __forceinline__ void cp16(void* smem_dst, const void* gmem_src, bool there) {
+  const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem_src), "r"(there ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+  __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<uint32_t*>(&h);
+}
+// (hi, lo) BF16 pairs of two non-negative numbers: hi = bf16(v), lo = bf16(v - hi)
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = pack2(a - __low2float(h), b - __high2float(h));
+}
+
+// grid = (B * qchunks, H), qchunks = ceil(longest segment / 16); block = 32 * (d / 64) threads; dynamic smem att_few_smem.
+// MAXW: most warps of the build (8: up to 255 registers per thread, models up to 512 wide; 16: 128 registers).
+template <bool QPROJ, int MAXW>
+__global__ void __launch_bounds__(32 * MAXW, 1)
+attention_few_kernel(const FewAttnParams fp) {
+  const AttnParams& p = fp.a;
+  extern __shared__ __align__(16) uint8_t few_smem[];
+  trace_mark(TR_ATTN, 0);
+  pdl_launch();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int nw = blockDim.x >> 5, nthreads = blockDim.x;
+  const int b = blockIdx.x / p.qchunks, chunk = blockIdx.x - b * p.qchunks, h = blockIdx.y;
+  const int d = p.d;
+  const int seg_len = plan_load(p.seg_len + b);
+  const int i0 = chunk * AQ;
+  // The first CTA always waits: a grid whose CTAs all left here would let its successors run before its predecessor is done.
+  if (i0 >= seg_len) {
+    if (blockIdx.x == 0 && h == 0) pdl_wait();
+    return;
+  }
+  bf16* ks = reinterpret_cast<bf16*>(few_smem) + (size_t)warp * AK * (K_LD + V_LD);   // this warp's keys of a round ...
+  bf16* vs = ks + AK * K_LD;                                                          // ... and values
+  float* part = reinterpret_cast<float*>(few_smem + (size_t)nw * AK * (K_LD + V_LD) * sizeof(bf16));   // [nw][16][O_LD]
+  float* pm = part + (size_t)nw * AQ * O_LD;                                          // [nw][16] maxima
+  float* pl = pm + nw * AQ;                                                           // [nw][16] sums
+  bf16* qs = reinterpret_cast<bf16*>(pl + nw * AQ);                                   // [16][K_LD] queries
+  bf16* os = qs + AQ * K_LD;                                                          // [16][K_LD] outputs
+
+  // weights: rows 8 j + g of this head's query projection / of this warp's 64 output features, 64-wide slices of K
+  uint4 wf[8][2];
+  if (QPROJ) {
+    const bf16* wb = fp.wq + (size_t)(h * 64 + g) * d + warp * 64 + 8 * t;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) wf[j][c] = __ldg(reinterpret_cast<const uint4*>(wb + (size_t)(8 * j) * d + 32 * c));
+  }
+  const bf16* ob = p.wo + (size_t)(warp * 64 + g) * d + h * 64 + 8 * t;
+  if (!QPROJ) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) wf[j][c] = __ldg(reinterpret_cast<const uint4*>(ob + (size_t)(8 * j) * d + 32 * c));
+  }
+  const int m0 = plan_load(p.seg_off + b) + i0;
+  const int kbase = plan_load(p.key_base + b), row_nk = plan_load(p.nkeys_row + b);
+  const int nq = min(AQ, seg_len - i0);
+  const int r0 = min(g, nq - 1), r1 = min(g + 8, nq - 1);       // missing queries repeat the last one; never stored
+  int nk0 = row_nk, nk1 = row_nk;
+  if (p.nkeys_tok) {
+    nk0 = min(plan_load(p.nkeys_tok + m0 + r0), row_nk);
+    nk1 = min(plan_load(p.nkeys_tok + m0 + r1), row_nk);
+  }
+  const bf16* kk = reinterpret_cast<const bf16*>(p.k);
+  const bf16* vv = reinterpret_cast<const bf16*>(p.v);
+  // this warp's 16 keys of a round, 64 elements each: 128 16-byte pieces, four per lane, for keys and values each
+  auto fetch = [&](int first) {
+    const int key0 = first + warp * AK;
+    if (key0 < row_nk) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int idx = lane + 32 * i, j = idx >> 3, c = (idx & 7) * 8;
+        const bool there = key0 + j < row_nk;
+        const size_t off = (size_t)(kbase + (there ? key0 + j : 0)) * d + h * 64 + c;
+        cp16(ks + j * K_LD + c, kk + off, there);
+        cp16(vs + j * V_LD + c, vv + off, there);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (QPROJ) fetch(0);          // the encoder's keys and values: older than the plan
+  float4 qbias = make_float4(0.f, 0.f, 0.f, 0.f);
+  pdl_wait();
+  trace_mark(TR_ATTN, 1);
+  if (!QPROJ) fetch(0);
+
+  uint4 qa[2][2];               // query fragments: [32-wide chunk of the head][row g / g + 8]
+  if (QPROJ) {
+    const bf16* x0 = fp.x + (size_t)(m0 + r0) * d + warp * 64 + 8 * t;
+    const bf16* x1 = fp.x + (size_t)(m0 + r1) * d + warp * 64 + 8 * t;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      qa[c][0] = *reinterpret_cast<const uint4*>(x0 + 32 * c);
+      qa[c][1] = *reinterpret_cast<const uint4*>(x1 + 32 * c);
+    }
+    float acc[8][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { acc[j][0] = 0.f; acc[j][1] = 0.f; acc[j][2] = 0.f; acc[j][3] = 0.f; }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) mma16816(acc[j], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, wf[j][c].x, wf[j][c].y);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) mma16816(acc[j], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, wf[j][c].z, wf[j][c].w);
+    }
+    // the output projection's weights arrive while the scores are computed
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) wf[j][c] = __ldg(reinterpret_cast<const uint4*>(ob + (size_t)(8 * j) * d + 32 * c));
+    float* pw = part + (size_t)warp * AQ * O_LD;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      *reinterpret_cast<float2*>(pw + g * O_LD + 8 * j + 2 * t) = make_float2(acc[j][0], acc[j][1]);
+      *reinterpret_cast<float2*>(pw + (g + 8) * O_LD + 8 * j + 2 * t) = make_float2(acc[j][2], acc[j][3]);
+    }
+    __syncthreads();
+    for (int idx = tid; idx < AQ * 16; idx += nthreads) {
+      const int r = idx >> 4, c = (idx & 15) * 4;
+      qbias = *reinterpret_cast<const float4*>(p.q_bias + h * 64 + c);
+      float4 v = qbias;
+#pragma unroll 4
+      for (int w = 0; w < nw; ++w) {
+        const float4 o = *reinterpret_cast<const float4*>(part + ((size_t)w * AQ + r) * O_LD + c);
+        v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+      }
+      uint2 u;
+      u.x = pack2(v.x, v.y); u.y = pack2(v.z, v.w);
+      *reinterpret_cast<uint2*>(qs + r * K_LD + c) = u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      qa[c][0] = *reinterpret_cast<const uint4*>(qs + g * K_LD + 32 * c + 8 * t);
+      qa[c][1] = *reinterpret_cast<const uint4*>(qs + (g + 8) * K_LD + 32 * c + 8 * t);
+    }
+  } else {
+    const bf16* q0 = reinterpret_cast<const bf16*>(p.q) + (size_t)(m0 + r0) * d + h * 64 + 8 * t;
+    const bf16* q1 = reinterpret_cast<const bf16*>(p.q) + (size_t)(m0 + r1) * d + h * 64 + 8 * t;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      qa[c][0] = *reinterpret_cast<const uint4*>(q0 + 32 * c);
+      qa[c][1] = *reinterpret_cast<const uint4*>(q1 + 32 * c);
+    }
+  }
+
+  float o[8][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) { o[j][0] = 0.f; o[j][1] = 0.f; o[j][2] = 0.f; o[j][3] = 0.f; }
+  float mx0 = -INFINITY, mx1 = -INFINITY, den0 = 0.f, den1 = 0.f;      // den: this lane's share of the row sums
+  for (int first = 0; first < row_nk; first += AK * nw) {
+    if (first > 0) { __syncwarp(); fetch(first); }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    const int key0 = first + warp * AK;
+    if (key0 >= row_nk) break;                                         // warp-uniform; later rounds lie further out still
+    float s[2][4];
+#pragma unroll
+    for (int n = 0; n < 2; ++n) { s[n][0] = 0.f; s[n][1] = 0.f; s[n][2] = 0.f; s[n][3] = 0.f; }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const uint4 k0 = *reinterpret_cast<const uint4*>(ks + g * K_LD + 32 * c + 8 * t);
+      const uint4 k1 = *reinterpret_cast<const uint4*>(ks + (g + 8) * K_LD + 32 * c + 8 * t);
+      mma16816(s[0], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, k0.x, k0.y);
+      mma16816(s[1], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, k1.x, k1.y);
+      mma16816(s[0], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, k0.z, k0.w);
+      mma16816(s[1], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, k1.z, k1.w);
+    }
+    // element e of group n: key key0 + 8 n + 2 t + (e & 1), query row g + 8 (e >> 1)
+    float t0 = -INFINITY, t1 = -INFINITY;
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+      const int j = key0 + 8 * n + 2 * t;
+      s[n][0] = j < nk0 ? s[n][0] * p.scale : -INFINITY;
+      s[n][1] = j + 1 < nk0 ? s[n][1] * p.scale : -INFINITY;
+      s[n][2] = j < nk1 ? s[n][2] * p.scale : -INFINITY;
+      s[n][3] = j + 1 < nk1 ? s[n][3] * p.scale : -INFINITY;
+      t0 = fmaxf(t0, fmaxf(s[n][0], s[n][1]));
+      t1 = fmaxf(t1, fmaxf(s[n][2], s[n][3]));
+    }
+    t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 1)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 1));
+    t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 2)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 2));
+    const bool on0 = nk0 > key0, on1 = nk1 > key0;                     // otherwise the query sees none of these keys
+    const float n0 = on0 ? fmaxf(mx0, t0) : mx0, n1 = on1 ? fmaxf(mx1, t1) : mx1;
+    const float c0 = on0 ? expf(mx0 - n0) : 1.f, c1 = on1 ? expf(mx1 - n1) : 1.f;     // exp(-inf) = 0 at first
+    mx0 = n0; mx1 = n1;
+    uint32_t hi[4], lo[4];
+    float sum0 = 0.f, sum1 = 0.f;
+#pragma unroll
+    for (int n = 0; n < 2; ++n) {
+      const float p0 = on0 ? expf(s[n][0] - n0) : 0.f, p1 = on0 ? expf(s[n][1] - n0) : 0.f;
+      const float p2 = on1 ? expf(s[n][2] - n1) : 0.f, p3 = on1 ? expf(s[n][3] - n1) : 0.f;
+      sum0 += p0 + p1; sum1 += p2 + p3;
+      split2(p0, p1, hi[2 * n], lo[2 * n]);
+      split2(p2, p3, hi[2 * n + 1], lo[2 * n + 1]);
+    }
+    den0 = den0 * c0 + sum0;
+    den1 = den1 * c1 + sum1;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { o[j][0] *= c0; o[j][1] *= c0; o[j][2] *= c1; o[j][3] *= c1; }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      uint32_t v0, v1;
+      const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(vs + (lane & 15) * V_LD + 8 * j));
+      asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(addr));
+      mma16816(o[j], hi[0], hi[1], hi[2], hi[3], v0, v1);
+      mma16816(o[j], lo[0], lo[1], lo[2], lo[3], v0, v1);
+    }
+  }
+  // merge the warps that had keys
+  const int na = min(nw, (row_nk + AK - 1) / AK);
+  den0 += __shfl_xor_sync(0xffffffffu, den0, 1); den1 += __shfl_xor_sync(0xffffffffu, den1, 1);
+  den0 += __shfl_xor_sync(0xffffffffu, den0, 2); den1 += __shfl_xor_sync(0xffffffffu, den1, 2);
+  if (warp < na) {              // (the partial query projections in `part` were read before the last barrier)
+    float* pw = part + (size_t)warp * AQ * O_LD;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      *reinterpret_cast<float2*>(pw + g * O_LD + 8 * j + 2 * t) = make_float2(o[j][0], o[j][1]);
+      *reinterpret_cast<float2*>(pw + (g + 8) * O_LD + 8 * j + 2 * t) = make_float2(o[j][2], o[j][3]);
+    }
+    if (t == 0) {
+      pm[warp * AQ + g] = mx0; pm[warp * AQ + g + 8] = mx1;
+      pl[warp * AQ + g] = den0; pl[warp * AQ + g + 8] = den1;
+    }
+  }
+  __syncthreads();
+  for (int idx = tid; idx < AQ * 16; idx += nthreads) {
+    const int r = idx >> 4, c = (idx & 15) * 4;
+    float m = -INFINITY;
+    for (int w = 0; w < na; ++w) m = fmaxf(m, pm[w * AQ + r]);
+    float den = 0.f;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int w = 0; w < na; ++w) {
+      const float f = expf(pm[w * AQ + r] - m);                        // a warp whose keys were all masked: exp(-inf) = 0
+      den += pl[w * AQ + r] * f;
+      const float4 x = *reinterpret_cast<const float4*>(part + ((size_t)w * AQ + r) * O_LD + c);
+      v.x += x.x * f; v.y += x.y * f; v.z += x.z * f; v.w += x.w * f;
+    }
+    const float inv = 1.f / den;
+    uint2 u;
+    u.x = pack2(v.x * inv, v.y * inv); u.y = pack2(v.z * inv, v.w * inv);
+    *reinterpret_cast<uint2*>(os + r * K_LD + c) = u;
+  }
+  __syncthreads();
+  // output projection: 16 queries x this warp's 64 features, K = this head's 64 dimensions
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    qa[c][0] = *reinterpret_cast<const uint4*>(os + g * K_LD + 32 * c + 8 * t);
+    qa[c][1] = *reinterpret_cast<const uint4*>(os + (g + 8) * K_LD + 32 * c + 8 * t);
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) { o[j][0] = 0.f; o[j][1] = 0.f; o[j][2] = 0.f; o[j][3] = 0.f; }
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mma16816(o[j], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, wf[j][c].x, wf[j][c].y);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mma16816(o[j], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, wf[j][c].z, wf[j][c].w);
+  }
+  float* dst = p.o_part + (size_t)h * p.o_stride + (size_t)m0 * d + warp * 64 + 2 * t;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if (g < nq) *reinterpret_cast<float2*>(dst + (size_t)g * d + 8 * j) = make_float2(o[j][0], o[j][1]);
+    if (g + 8 < nq) *reinterpret_cast<float2*>(dst + (size_t)(g + 8) * d + 8 * j) = make_float2(o[j][2], o[j][3]);
+  }
+  trace_mark(TR_ATTN, 2);
+}
+
+}  // namespace few
+}  // namespace ad

@@ -51,16 +51,17 @@ attention_mma_kernel(const AttnParams p) {
 
   trace_mark(TR_ATTN, 0);
   pdl_launch();
-  pdl_wait();
-  trace_mark(TR_ATTN, 1);
   const int b = blockIdx.x / p.qchunks;
   const int chunk = blockIdx.x % p.qchunks;
   const int h = blockIdx.y;
-  const int seg_len = p.seg_len[b];
-  const int seg_off = p.seg_off[b];
-  const int kbase = p.key_base[b];
-  const int row_nk = p.nkeys_row[b];
+  const int seg_len = plan_load(p.seg_len + b);
+  const int seg_off = plan_load(p.seg_off + b);
+  const int kbase = plan_load(p.key_base + b);
+  const int row_nk = plan_load(p.nkeys_row + b);
   const int i0 = chunk * (16 * QT);
+  if (i0 >= seg_len && (blockIdx.x | blockIdx.y) != 0) return;
+  pdl_wait();
+  trace_mark(TR_ATTN, 1);
   if (i0 >= seg_len) return;
   const int nq = min(16 * QT, seg_len - i0);
   const int m0 = seg_off + i0;
@@ -300,16 +301,17 @@ attention_mma_wide_kernel(const AttnParams p) {
 
   trace_mark(TR_ATTN, 0);
   pdl_launch();
-  pdl_wait();
-  trace_mark(TR_ATTN, 1);
   const int b = blockIdx.x / p.qchunks;
   const int chunk = blockIdx.x % p.qchunks;
   const int h = blockIdx.y;
-  const int seg_len = p.seg_len[b];
-  const int seg_off = p.seg_off[b];
-  const int kbase = p.key_base[b];
-  const int row_nk = p.nkeys_row[b];
+  const int seg_len = plan_load(p.seg_len + b);
+  const int seg_off = plan_load(p.seg_off + b);
+  const int kbase = plan_load(p.key_base + b);
+  const int row_nk = plan_load(p.nkeys_row + b);
   const int i0 = chunk * (16 * QT);
+  if (i0 >= seg_len && (blockIdx.x | blockIdx.y) != 0) return;
+  pdl_wait();
+  trace_mark(TR_ATTN, 1);
   if (i0 >= seg_len) return;
   const int nq = min(16 * QT, seg_len - i0);
   const int m0 = seg_off + i0;

@@ -1,0 +1,146 @@
+// BF16 projections of passes with few packed tokens (up to a hundred or so), on warp-level MMAs with the weights held in
+// registers.
+//
+// With so few tokens a projection moves 1-8 MB of weights that sit in L2 and does next to no arithmetic; what it costs is
+// latency: the tcgen05 kernel (gemm_tc.cuh) needs 2.3-4 us for one after its dependency wait (TMA round trip, MMA issue,
+// tensor-memory read-out, transposition, stores).  Here a CTA owns 16 output features and its eight warps split K between
+// them, so that a warp's share of the weights is a handful of 16-byte loads per lane that are issued BEFORE the dependency
+// wait (weights never change).  After the wait a CTA does one round trip for its activations, a few dozen MMAs, one
+// exchange through shared memory (the warps' partial sums, added in warp order) and the stores.
+//
+// The contraction index is permuted identically for both operands (a lane's 16-byte piece holds eight consecutive K
+// elements, which serve as the fragments of two k16 steps), so no ldmatrix and no shared-memory staging is needed.
+#pragma once
+
+#include "ad_common.cuh"
+
+namespace ad {
+namespace few {
+
+constexpr int THREADS = 256;
+constexpr int WARPS = 8;
+constexpr int FEAT = 16;          // output features per CTA = MMA M
+constexpr int RED_LD = 20;        // floats per token row of a warp's partial sums: conflict-free, 16-byte aligned
+constexpr int MAX_CHUNKS = 4;     // 32-wide K chunks per warp: K per CTA = 256 .. 1024
+
+// D (16 x 8, FP32) += A (16 x 16, BF16, row-major) * B (16 x 8, BF16, column-major).  Not volatile: free to be scheduled.
+__device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Tokens of one round trip: 64 while a warp's slice of K is 64 wide, 32 beyond (register budget of two CTAs per SM).
+__host__ __device__ constexpr int round_tokens(int nch) { return nch <= 2 ? 64 : 32; }
+
+// K split of a projection with N output features: the smallest power of two that leaves at most 1024 of K to a CTA, more
+// while the grid stays within 128 CTAs and the split is wanted (consumer adds partial sums up).  0: shape not supported.
+inline int split_for(int N, int K, bool may_split, int max_split) {
+  if (N % FEAT || K % 256) return 0;
+  int s = 1;
+  while (K / s > 256 * MAX_CHUNKS || (may_split && (N / FEAT) * s * 2 <= 128 && K % (512 * s) == 0 && K / (2 * s) >= 512)) {
+    s *= 2;
+    if (K % (256 * s)) return 0;
+  }
+  if (s > 1 && (!may_split || s > max_split)) return 0;
+  return s;
+}
+
+// grid = (N / 16, ksplit); block = 256; K / ksplit = 256 * NCH.
+// EPI_F32: partial sums [ksplit][M_cap, N] (no bias); EPI_ACT: bias (+ ReLU) -> BF16; EPI_SCATTER: q / K / V rows.
+template <int EPI, int NCH>
+__global__ void __launch_bounds__(THREADS, 2)
+gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p) {
+  constexpr int TPR = round_tokens(NCH);
+  constexpr int NT = TPR / 8;
+  __shared__ __align__(16) float red[WARPS][TPR][RED_LD];
+  trace_mark(TR_GEMM + EPI, 0);
+  pdl_launch();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int n0 = blockIdx.x * FEAT;
+  const int kbase = blockIdx.y * (256 * NCH) + warp * (32 * NCH) + 8 * t;
+  const size_t K = (size_t)p.K;
+  uint4 wa[NCH][2];
+#pragma unroll
+  for (int c = 0; c < NCH; ++c) {
+    wa[c][0] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + g) * K + kbase + 32 * c));
+    wa[c][1] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + g + 8) * K + kbase + 32 * c));
+  }
+  const int of = (tid & 3) * 4, ot = tid >> 2;               // this thread's output: four features of one token per round
+  float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (EPI != EPI_F32) bias = *reinterpret_cast<const float4*>(p.bias + n0 + of);
+  // the plan was complete before this kernel could start (see plan_data in ad_common.cuh)
+  const int M = plan_load(p.M_ptr);
+  int slot = 0;
+  if (EPI == EPI_SCATTER && ot < M) slot = plan_load(p.slot + ot);
+  pdl_wait();
+  trace_mark(TR_GEMM + EPI, 1);
+  for (int t0 = 0; t0 < M; t0 += TPR) {
+    float acc[NT][4];
+    uint4 xb[NT][NCH];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      if (t0 + 8 * nt < M) {
+        const bf16* xr = X + (size_t)min(t0 + 8 * nt + g, p.M_cap - 1) * K + kbase;
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) xb[nt][c] = *reinterpret_cast<const uint4*>(xr + 32 * c);
+      }
+    }
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) { acc[nt][0] = 0.f; acc[nt][1] = 0.f; acc[nt][2] = 0.f; acc[nt][3] = 0.f; }
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt)
+        if (t0 + 8 * nt < M) mma16816(acc[nt], wa[c][0].x, wa[c][1].x, wa[c][0].y, wa[c][1].y, xb[nt][c].x, xb[nt][c].y);
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt)
+        if (t0 + 8 * nt < M) mma16816(acc[nt], wa[c][0].z, wa[c][1].z, wa[c][0].w, wa[c][1].w, xb[nt][c].z, xb[nt][c].w);
+    }
+    if (t0 > 0) __syncthreads();                             // the previous round has been read out
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      if (t0 + 8 * nt < M) {
+        float* r0 = &red[warp][8 * nt + 2 * t][g];
+        r0[0] = acc[nt][0]; r0[RED_LD] = acc[nt][1];
+        r0[8] = acc[nt][2]; r0[RED_LD + 8] = acc[nt][3];
+      }
+    }
+    __syncthreads();
+    const int m = t0 + ot;
+    if (ot < TPR && m < M) {
+      float4 v = *reinterpret_cast<const float4*>(&red[0][ot][of]);
+#pragma unroll
+      for (int w = 1; w < WARPS; ++w) {
+        const float4 o = *reinterpret_cast<const float4*>(&red[w][ot][of]);
+        v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+      }
+      if (EPI == EPI_F32) {
+        *reinterpret_cast<float4*>(p.out_f32 + ((size_t)blockIdx.y * p.M_cap + m) * p.N + n0 + of) = v;
+      } else {
+        v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
+        if (EPI == EPI_ACT && p.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
+        bf16* dst;
+        if (EPI == EPI_ACT) {
+          dst = reinterpret_cast<bf16*>(p.out_act) + (size_t)m * p.N + n0 + of;
+        } else {                                             // a 16-feature tile lies inside one segment
+          const int seg = n0 / p.seg_width, col = n0 - seg * p.seg_width;
+          char* base = p.seg_pair_stride ? static_cast<char*>(p.dst[seg & 1]) + (size_t)(seg >> 1) * p.seg_pair_stride
+                                         : static_cast<char*>(p.dst[seg]);
+          if (t0 > 0) slot = plan_load(p.slot + m);
+          dst = reinterpret_cast<bf16*>(base) + (size_t)(seg < p.n_direct ? m : slot) * p.seg_width + col + of;
+        }
+        __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
+        uint2 u;
+        u.x = *reinterpret_cast<unsigned int*>(&h0);
+        u.y = *reinterpret_cast<unsigned int*>(&h1);
+        *reinterpret_cast<uint2*>(dst) = u;
+      }
+    }
+  }
+  trace_mark(TR_GEMM + EPI, 2);
+}
+
+}  // namespace few
+}  // namespace ad

@@ -301,7 +301,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   const int kb_end = (int)(((long long)kb_total * (blockIdx.z + 1)) / ksplit);
   const int num_kb = kb_end - kb_begin;
   const int first_round = num_kb < stages ? num_kb : stages;
-  const bool early = (blockIdx.y == 0);   // token tile 0 always has work (M >= 1 whenever a result is read)
+  // token tile 0 always has work (M >= 1 whenever a result is read); the others leave at once when the pass does not reach them
+  const bool early = (blockIdx.y == 0);
+  const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
+  if (!early && t0 >= M) return;
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzled tiles need 1024-byte alignment
   // MMA issuers.  Issuing one tcgen05.mma costs its thread 65-80 cycles whatever the tile, so with few tokens (short
@@ -358,6 +361,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       tma_load_2d(smem_base + i * stage_bytes, &map_w, (kb_begin + i) * BLOCK_K, n0, bar);
     }
   }
+  if (EPI == EPI_SCATTER) {
+    for (int j = threadIdx.x; j < ntile; j += THREADS) slot_s[j] = (t0 + j < M) ? plan_load(p.slot + t0 + j) : 0;
+  }
   const int n = n0 + quad * 32 + lane;
   const float bias_n = (p.bias && n < p.N) ? p.bias[n] : 0.f;   // a weight as well: no dependency
 
@@ -370,13 +376,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       tma_load_2d(smem_base + i * stage_bytes + A_STAGE_BYTES, &map_x, (kb_begin + i) * BLOCK_K, t0,
                   smem_u32(&bar_full[i]));
   }
-  const int M = p.M_ptr ? *p.M_ptr : p.M_host;
-  const bool valid = early || (t0 < M);
 
-  if (valid) {
-    if (EPI == EPI_SCATTER) {
-      for (int j = threadIdx.x; j < ntile; j += THREADS) slot_s[j] = (t0 + j < M) ? p.slot[t0 + j] : 0;
-    }
+  {
     if (EPI == EPI_ARGMAX && p.draft_val) {
       for (int j = threadIdx.x; j < ntile; j += THREADS) {
         dval_s[j] = (t0 + j < M) ? p.draft_val[t0 + j] : 0.f;

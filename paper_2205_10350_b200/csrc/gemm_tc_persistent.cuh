@@ -92,9 +92,9 @@ vocab_argmax_persistent_kernel(const __grid_constant__ CUtensorMap map_w, const 
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_acc = tmem_base_slot;
   pdl_launch();
+  const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
   pdl_wait();
 
-  const int M = p.M_ptr ? *p.M_ptr : p.M_host;
   const int n_vt = (p.N + BLOCK_N_FEAT - 1) / BLOCK_N_FEAT;    // 128-row tiles: the layout of the partial arrays
   const int n_v2 = (p.N + P_VOC - 1) / P_VOC;                  // 256-row tiles of a pair
   const int n_tt = (M + P_TOK - 1) / P_TOK;                    // token tiles that hold tokens

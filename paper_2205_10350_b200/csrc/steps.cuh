@@ -183,8 +183,7 @@ __global__ void __launch_bounds__(256)
 prepare_verify_kernel(DevState st, PassPlan plan, Dims dm, int source, int k_cap, const int* override_stream,
                       int override_stride, int override_len) {
   trace_mark(TR_PREPARE, 0);
-  pdl_launch();
-  pdl_wait();
+  pdl_wait();                  // (no pdl_launch: see plan data in ad_common.cuh)
   trace_mark(TR_PREPARE, 1);
   __shared__ int s_k[256];
   __shared__ int s_off[257];
@@ -192,6 +191,7 @@ prepare_verify_kernel(DevState st, PassPlan plan, Dims dm, int source, int k_cap
   nb.source = source; nb.k_cap = k_cap; nb.override_stream = override_stream;
   nb.override_stride = override_stride; nb.override_len = override_len;
   plan_verify_block(st, plan, dm, nb, s_k, s_off);
+  __threadfence();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -200,8 +200,7 @@ prepare_verify_kernel(DevState st, PassPlan plan, Dims dm, int source, int k_cap
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 plan_draft_kernel(DevState st, PassPlan blk, PassPlan plan, Dims dm) {
-  pdl_launch();
-  pdl_wait();
+  pdl_wait();                  // (no pdl_launch: see plan data in ad_common.cuh)
   __shared__ int s_off[257];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int B = dm.B;
@@ -231,6 +230,7 @@ plan_draft_kernel(DevState st, PassPlan blk, PassPlan plan, Dims dm) {
     }
     for (int i = lane; i < k; i += 32) st.gidx[blk.seg_off[b] + i] = off + len + 1 + i;
   }
+  __threadfence();
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -239,8 +239,7 @@ plan_draft_kernel(DevState st, PassPlan blk, PassPlan plan, Dims dm) {
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 plan_encode_kernel(DevState st, PassPlan plan, Dims dm) {
-  pdl_launch();
-  pdl_wait();
+  pdl_wait();                  // (no pdl_launch: see plan data in ad_common.cuh)
   __shared__ int s_off[257];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int B = dm.B;
@@ -279,6 +278,7 @@ plan_encode_kernel(DevState st, PassPlan plan, Dims dm) {
       st.enc_slot[m] = b * dm.max_src + i;
     }
   }
+  __threadfence();
 }
 
 __global__ void set_maxlen_kernel(DevState st, Dims dm, const int* maxlen) {
@@ -369,10 +369,10 @@ layernorm_kernel(const int* __restrict__ M_ptr, const float* __restrict__ pre, i
     bv[i] = on ? reinterpret_cast<const float4*>(bta)[gi] : zero4;
     cb[i] = (on && bias) ? reinterpret_cast<const float4*>(bias)[gi] : zero4;
   }
+  const int m = blockIdx.x;
+  if (m >= plan_load(M_ptr) && m > 0) return;      // CTA 0 always waits (see early exits in ad_common.cuh)
   pdl_wait();
   trace_mark(TR_LN, 1);
-  const int m = blockIdx.x;
-  if (m >= *M_ptr) return;
   float4 xv[NG];
   float s = 0.f;
 #pragma unroll
@@ -434,10 +434,11 @@ layernorm_rows_kernel(const int* __restrict__ M_ptr, const float* __restrict__ p
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per = d >> 7;                               // float4 groups per lane (d / 128), <= 8
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int m = blockIdx.x * 8 + warp, M = plan_load(M_ptr);
+  if ((int)blockIdx.x * 8 >= M && blockIdx.x > 0) return;
   pdl_wait();
   trace_mark(TR_LN, 1);
-  const int m = blockIdx.x * 8 + warp;
-  if (m < *M_ptr) {
+  if (m < M) {
     const size_t row = (size_t)m * (d >> 2);
     float4 xv[8];
     float s = 0.f;
@@ -505,10 +506,12 @@ __global__ void __launch_bounds__(128)
 gather_rows_kernel(const int* __restrict__ M_ptr, const int* __restrict__ gidx, const ActT* __restrict__ src,
                    ActT* __restrict__ dst, int d) {
   pdl_launch();
-  pdl_wait();
   const int j = blockIdx.x;
-  if (j >= *M_ptr) return;
-  const int s = gidx[j];
+  const bool have = j < plan_load(M_ptr);
+  if (!have && j > 0) return;
+  const int s = have ? plan_load(gidx + j) : 0;
+  pdl_wait();
+  if (!have) return;
   for (int i = threadIdx.x; i < d; i += blockDim.x) dst[(size_t)j * d + i] = src[(size_t)s * d + i];
 }
 
@@ -633,11 +636,11 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
   __shared__ int s_off[257];
   __shared__ int s_last;
   trace_mark(TR_ACCEPT, 0);
-  pdl_launch();
+  if (next.source < 0) pdl_launch();     // a kernel that plans never does (see plan data in ad_common.cuh)
+  const int b = blockIdx.x;
+  const int k = plan_load(blk.seg_len + b);
   pdl_wait();
   trace_mark(TR_ACCEPT, 1);
-  const int b = blockIdx.x;
-  const int k = blk.seg_len[b];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int* pred = (to_drafts ? st.drafts : st.pred) + (size_t)b * dm.kmax;
   if (k > 0) {
@@ -730,6 +733,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
         *reinterpret_cast<float4*>(ne.y + (size_t)m * d + c) = v;
         store4(yb + (size_t)m * d + c, v);
       }
+      __threadfence();
     }
   }
   trace_mark(TR_ACCEPT, 2);
