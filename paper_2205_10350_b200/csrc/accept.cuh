@@ -1,0 +1,332 @@
+// End of a projection: final arg-max over its per-tile partials, the accept decision, and -- inside a decode loop -- the
+// commit, the choice of the next block and the layout of the pass that verifies it, all in one kernel.
+#pragma once
+
+#include "steps.cuh"
+
+namespace ad {
+
+// What the accept kernel prepares for the pass behind it (source < 0: nothing).
+struct NextPass {
+  int source;            // SRC_POLICY / SRC_OVERRIDE: plan the next verification block after the commit;
+                         // SRC_SIZES: plan the drafter's pass after the commit (block sizes, then its tokens);
+                         // SRC_KEEP (drafter's choices): plan the verification of the block just drafted
+  int k_cap;
+  const int* override_stream;
+  int override_stride, override_len;
+  PassPlan draft;        // SRC_SIZES: plan of the drafter's pass
+};
+
+constexpr int ACC_THREADS = 1024;
+constexpr int ACC_SRC = 512;            // source tokens kept in shared memory for the suffix match
+
+// Suffix match of Algorithm 1, line 3 (see warp_suffix_match) by the whole CTA: every thread looks at the end positions
+// tid, tid + 1024, ... of the source.  o(t): output token t (o(0) = [BOS]); x: source tokens; *where: shared word.
+template <typename OutTok>
+__device__ __forceinline__ int cta_suffix_match(OutTok o, int j, const int* x, int n, int bos, int* where) {
+  int found = -1;
+  for (int q = 0; q <= j; ++q) {
+    int count = 0;
+    for (int i0 = q; i0 <= n; i0 += ACC_THREADS) {
+      const int i = i0 + (int)threadIdx.x;
+      bool ok = i <= n;
+      for (int t = 0; ok && t <= q; ++t) ok = o(j - t) == (i - t == 0 ? bos : x[i - t - 1]);
+      if (ok) *where = i;
+      count += __syncthreads_count(ok);
+    }
+    if (count == 1) { found = *where; break; }
+    if (count == 0) break;
+    __syncthreads();
+  }
+  __syncthreads();
+  return found;
+}
+
+// The decision for one row:
+//   c = first block position whose greedy choice differs from the draft (Section 3.1.1; definition of c in Section 3.2),
+//   n = c + 1 (the bifurcation token is kept), n = k when nothing differs, cut at the first accepted [EOS].
+// beta >= 1: relaxed verification of Section 3.2.3 -- a position keeps its drafted token when fewer than beta other tokens
+//   score strictly higher (Eq. 8: the draft is within the top beta) and the best score exceeds the draft's by at most tau
+//   (Eq. 9; differences of log-likelihoods are differences of scores); otherwise the greedy choice.
+// to_drafts: the choices are the row's drafts and nothing is compared.
+// auto_commit (decode loop): n is committed at once (Algorithm 1 lines 6-7); the last CTA to finish updates the loop
+//   counters and the all-finished word (done_ctr: rows done in the low half, active rows in the high half; left at zero) and,
+//   with next.source >= 0, lays out the pass behind this kernel; what concerns one row alone (suffix match, drafts, sizes)
+//   is done by the row's own CTA.
+//
+// What bounds it: a chain of dependent memory round trips, so whatever older kernels wrote (row state, drafts, source) is
+// read before the dependency wait, and from the partials to the next plan everything stays in shared memory: one round trip
+// for the partials (plus the hand-over between CTAs when B > 1).
+// Batch 1, 40-token blocks: 11.4 us with the state, the match and the plan in global memory.
+// grid = B, block = 1024.
+__global__ void __launch_bounds__(ACC_THREADS)
+argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict__ part_val, const int* __restrict__ part_idx,
+                     int n_tiles, int to_drafts, int auto_commit, unsigned int* done_ctr, unsigned long long cond, int beta,
+                     float tau, const float* __restrict__ draft_val, const int* __restrict__ draft_id,
+                     const int* __restrict__ part_cnt, NextPass next) {
+  __shared__ int s_dr[256], s_pred[256], s_src[ACC_SRC];
+  __shared__ int s_k[256], s_off[257], s_len[256];
+  __shared__ int s_n, s_last_cta, s_where;
+  trace_mark(TR_ACCEPT, 0);
+  if (next.source < 0) pdl_launch();     // a kernel that plans never does (see plan data in ad_common.cuh)
+  const int b = blockIdx.x, B = dm.B;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // ---- what older kernels wrote ----
+  const int k = plan_load(blk.seg_len + b), off = plan_load(blk.seg_off + b);
+  const int len = plan_load(st.len + b), maxlen = plan_load(st.maxlen + b), old_last = plan_load(st.last + b);
+  const int old_fin = plan_load(st.fin + b);
+  int it_active = 0, it_all = 0, it_limit = 0, stat_acc = 0, stat_it = 0, stat_off = 0;
+  if (tid == 0) { stat_acc = plan_load(st.stat_acc + b); stat_it = plan_load(st.stat_it + b); stat_off = plan_load(st.stat_off + b); }
+  if (tid == ACC_THREADS - 1 && auto_commit) { it_active = plan_load(st.loop_it); it_all = plan_load(st.loop_it + 2); it_limit = plan_load(st.loop_it + 3); }
+  if (!to_drafts && tid < k) s_dr[tid] = plan_load(st.drafts + (size_t)b * dm.kmax + tid);     // k <= kmax <= 256
+  int n_src = 0;
+  const int* x = st.src + (size_t)b * dm.max_src;
+  if (next.source == SRC_POLICY) {
+    n_src = plan_load(st.srclen + b);
+    if (n_src <= ACC_SRC) {
+      for (int i = tid; i < n_src; i += ACC_THREADS) s_src[i] = plan_load(x + i);
+      x = s_src;
+    }
+  }
+  pdl_wait();
+  trace_mark(TR_ACCEPT, 1);
+
+  // ---- arg-max over the tiles of every block position: a warp per position, the lowest id wins ties ----
+  const bool relaxed = beta >= 1 && !to_drafts;
+  int* pred = (to_drafts ? st.drafts : st.pred) + (size_t)b * dm.kmax;
+  // (two positions of a warp at once, eight tiles per lane and position in flight)
+  for (int i0 = warp; i0 < k; i0 += 2 * (ACC_THREADS / 32)) {
+    float v[2] = {-INFINITY, -INFINITY};
+    int idx[2] = {0x7fffffff, 0x7fffffff}, higher[2] = {0, 0};
+    for (int t0 = 0; t0 < n_tiles; t0 += 256) {
+      float pv[2][8];
+      int pi[2][8];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = i0 + h * (ACC_THREADS / 32);
+        const size_t row = (size_t)(off + i) * n_tiles;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int t = t0 + 32 * u + lane;
+          const bool on = i < k && t < n_tiles;
+          pv[h][u] = on ? part_val[row + t] : -INFINITY;
+          pi[h][u] = on ? part_idx[row + t] : 0x7fffffff;
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (pv[h][u] > v[h] || (pv[h][u] == v[h] && pi[h][u] < idx[h])) { v[h] = pv[h][u]; idx[h] = pi[h][u]; }
+        const int i = i0 + h * (ACC_THREADS / 32);
+        if (relaxed && i < k)
+          for (int t = t0 + lane; t < min(t0 + 256, n_tiles); t += 32) higher[h] += part_cnt[(size_t)(off + i) * n_tiles + t];
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = i0 + h * (ACC_THREADS / 32);
+      if (i >= k) break;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, v[h], o);
+        const int oi = __shfl_xor_sync(0xffffffffu, idx[h], o);
+        if (ov > v[h] || (ov == v[h] && oi < idx[h])) { v[h] = ov; idx[h] = oi; }
+        if (relaxed) higher[h] += __shfl_xor_sync(0xffffffffu, higher[h], o);
+      }
+      if (lane == 0) {
+        int choice = idx[h];
+        if (relaxed) {
+          const int did = draft_id[off + i];
+          if (did >= 0 && higher[h] <= beta - 1 && v[h] - draft_val[off + i] <= tau) choice = did;
+        }
+        s_pred[i] = choice;
+        if (!(to_drafts && next.source == SRC_KEEP)) pred[i] = choice;
+      }
+    }
+  }
+  __syncthreads();
+
+  if (to_drafts) {
+    if (next.source != SRC_KEEP) return;
+    // the drafted block becomes the verification block of this row: its place among the packed tokens is known already
+    int dr = -1;
+    if (tid < k) {
+      dr = s_pred[tid];
+      if (next.override_stream) dr = len + tid < next.override_len ? next.override_stream[(size_t)b * next.override_stride + len + tid] : -1;
+      if (dr >= dm.vocab) { latch_error(st.status, AD_ERR_ARG); dr = -1; }
+      s_dr[tid] = dr;
+      st.drafts[(size_t)b * dm.kmax + tid] = dr;
+    }
+    __syncthreads();
+    if (tid < k) {
+      int tok = tid == 0 ? old_last : s_dr[tid - 1];
+      if (tok < 0 || tok >= dm.vocab) tok = dm.pad;
+      const int m = off + tid;
+      blk.tok_row[m] = b; blk.tok_pos[m] = len + tid; blk.tok_id[m] = tok;
+      blk.kv_slot[m] = b * dm.max_tgt + len + tid; blk.att_n[m] = len + tid + 1;
+    }
+    if (tid == 0) {
+      blk.key_base[b] = b * dm.max_tgt; blk.row_nk[b] = len + k;
+      if (b == 0) st.loop_it[1] = 0;
+    }
+    __threadfence();
+    trace_mark(TR_ACCEPT, 2);
+    return;
+  }
+
+  // ---- the decision ----
+  trace_mark(TR_ACCEPT, 3);
+  if (warp == 0) {
+    int n = k;
+    for (int i0 = 0; i0 < k; i0 += 32) {
+      const int i = i0 + lane;
+      const unsigned bal = __ballot_sync(0xffffffffu, i < k && (s_dr[i] < 0 || s_pred[i] != s_dr[i]));
+      if (bal) { n = i0 + __ffs(bal); break; }
+    }
+    for (int i0 = 0; i0 < n; i0 += 32) {
+      const int i = i0 + lane;
+      const unsigned bal = __ballot_sync(0xffffffffu, i < n && s_pred[i] == dm.eos);
+      if (bal) { n = i0 + __ffs(bal); break; }
+    }
+    if (lane == 0) s_n = n;
+  }
+  __syncthreads();
+  const int n = s_n;
+  if (!auto_commit) {
+    if (tid == 0) st.n_acc[b] = n;
+    return;
+  }
+
+  // ---- commit ----
+  trace_mark(TR_ACCEPT, 4);
+  const int len1 = len + n, last1 = n > 0 ? s_pred[n - 1] : old_last;
+  const int fin1 = old_fin || (n > 0 && (last1 == dm.eos || len1 >= maxlen));
+  if (tid < n) st.out_ids[(size_t)b * dm.max_tgt + len + tid] = s_pred[tid];
+  if (tid == 0) {
+    st.n_acc[b] = 0;
+    if (n > 0) {
+      st.len[b] = len1; st.last[b] = last1; st.fin[b] = fin1;
+      st.stat_acc[b] = stat_acc + n; st.stat_it[b] = stat_it + 1; st.stat_off[b] = stat_off + k;
+    }
+  }
+  // ---- this row's next block ----
+  int k1 = 0;
+  if (next.source >= 0) {
+    const bool live = !fin1 && len1 < maxlen;
+    if (next.source == SRC_POLICY) {
+      if (live) {
+        const int* old_out = st.out_ids + (size_t)b * dm.max_tgt;
+        auto o = [&](int t) { return t == 0 ? dm.bos : (t - 1 >= len ? s_pred[t - 1 - len] : __ldcg(old_out + t - 1)); };
+        const int i = cta_suffix_match(o, len1, x, n_src, dm.bos, &s_where);
+        // draft = x_{i+1..n} followed by the [PAD] slot that matches nothing; a plain step without a match
+        k1 = i >= 0 ? min(n_src - i + 1, min(next.k_cap, maxlen - len1)) : 1;
+        if (tid < k1) s_dr[tid] = (i >= 0 && i + 1 + tid <= n_src) ? x[i + tid] : -1;
+      }
+    } else {
+      k1 = live ? min(next.k_cap, maxlen - len1) : 0;
+      if (next.source == SRC_OVERRIDE && tid < k1)
+        s_dr[tid] = len1 + tid < next.override_len ? next.override_stream[(size_t)b * next.override_stride + len1 + tid] : -1;
+    }
+    if (next.source != SRC_SIZES && tid < k1) {
+      int dr = s_dr[tid];
+      // a caller-provided draft beyond the vocabulary becomes a slot that matches nothing (negative = sentinel is legal)
+      if (dr >= dm.vocab) { latch_error(st.status, AD_ERR_ARG); dr = -1; s_dr[tid] = dr; }
+      st.drafts[(size_t)b * dm.kmax + tid] = dr;
+    }
+    if (tid == 0) {
+      blk.seg_len[b] = k1; blk.key_base[b] = b * dm.max_tgt; blk.row_nk[b] = len1 + k1;
+      s_k[b] = k1; s_len[b] = len1;
+    }
+  }
+  // ---- the last row to get here sees all of them ----
+  trace_mark(TR_ACCEPT, 5);
+  __syncthreads();
+  bool all_fin = fin1 != 0, any_active = n > 0;
+  if (B > 1) {
+    if (tid == 0) {
+      __threadfence();
+      const unsigned int t = atomicAdd(done_ctr, n > 0 ? 0x10001u : 1u);
+      s_last_cta = (t & 0xffffu) == (unsigned)B - 1 ? 1 : 0;
+      if (s_last_cta) { __threadfence(); s_n = ((t >> 16) + (n > 0 ? 1u : 0u)) != 0; }
+    }
+    __syncthreads();
+    if (!s_last_cta) return;
+    any_active = s_n != 0;
+    int f = 1;
+    if (tid < B) {
+      f = __ldcg(st.fin + tid);
+      if (next.source >= 0) { s_k[tid] = __ldcg(blk.seg_len + tid); s_len[tid] = __ldcg(st.len + tid); }
+    }
+    all_fin = __syncthreads_and(f) != 0;
+  }
+  if (tid == ACC_THREADS - 1) {            // (not a thread of the warp that lays the rows out)
+    *done_ctr = 0;
+    if (any_active) *st.loop_it = it_active + 1;
+    *st.all_fin = all_fin;
+    if (cond) {
+      // the iteration runs inside a device-side `while` graph node, which repeats while its condition is non-zero: cleared
+      // when every row has finished or, as a bound that does not depend on the data, at the limit the host stored
+      st.loop_it[2] = it_all + 1;
+      cudaGraphSetConditional(cond, (all_fin || it_all + 1 >= it_limit) ? 0u : 1u);
+    }
+  }
+  if (next.source < 0) return;
+  // ---- layout of the pass behind this kernel ----
+  trace_mark(TR_ACCEPT, 6);
+  const bool draft_pass = next.source == SRC_SIZES;
+  if (warp == 0) {                         // offsets: an exclusive scan over the rows
+    int base = 0, dbase = 0;
+    for (int b0 = 0; b0 < B; b0 += 32) {
+      const int r = b0 + lane, kr = r < B ? s_k[r] : 0;
+      const int dr = kr > 0 ? s_len[r] + 1 + kr : 0;     // drafter's tokens of the row: [BOS], accepted tokens, k x [MASK]
+      int sum = kr, dsum = dr;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int a = __shfl_up_sync(0xffffffffu, sum, o), c = __shfl_up_sync(0xffffffffu, dsum, o);
+        if (lane >= o) { sum += a; dsum += c; }
+      }
+      if (r < B) {
+        blk.seg_off[r] = base + sum - kr;
+        s_off[r] = draft_pass ? dbase + dsum - dr : base + sum - kr;
+        if (draft_pass) s_k[r] = (int)((unsigned)kr | (unsigned)(base + sum - kr) << 16);   // block size and block offset (both below 65536)
+      }
+      base += __shfl_sync(0xffffffffu, sum, 31);
+      dbase += __shfl_sync(0xffffffffu, dsum, 31);
+    }
+    if (lane == 0) {
+      s_off[B] = draft_pass ? dbase : base;
+      *blk.M = base;
+      if (draft_pass) *next.draft.M = dbase;
+    }
+  }
+  __syncthreads();
+  for (int r = warp; r < B; r += ACC_THREADS / 32) {
+    const int o0 = s_off[r], lr = s_len[r];
+    if (draft_pass) {
+      const int kr = s_k[r] & 0xffff, boff = (int)((unsigned)s_k[r] >> 16), nr = kr > 0 ? lr + 1 + kr : 0;
+      const PassPlan& pl = next.draft;
+      if (lane == 0) { pl.seg_off[r] = o0; pl.seg_len[r] = nr; pl.key_base[r] = o0; pl.row_nk[r] = nr; }
+      for (int i = lane; i < nr; i += 32) {
+        const int m = o0 + i;
+        const int tok = i == 0 ? dm.bos : (i <= lr ? __ldcg(st.out_ids + (size_t)r * dm.max_tgt + i - 1) : dm.mask);
+        pl.tok_row[m] = r; pl.tok_pos[m] = i; pl.tok_id[m] = tok; pl.kv_slot[m] = m; pl.att_n[m] = nr;
+      }
+      for (int i = lane; i < kr; i += 32) st.gidx[boff + i] = o0 + lr + 1 + i;
+    } else {
+      const int kr = s_k[r];
+      const int* dr = B == 1 ? s_dr : st.drafts + (size_t)r * dm.kmax;
+      for (int i = lane; i < kr; i += 32) {
+        const int m = o0 + i;
+        int tok = B == 1 ? (i == 0 ? last1 : dr[i - 1]) : (i == 0 ? __ldcg(st.last + r) : __ldcg(dr + i - 1));
+        if (tok < 0 || tok >= dm.vocab) tok = dm.pad;
+        blk.tok_row[m] = r; blk.tok_pos[m] = lr + i; blk.tok_id[m] = tok;
+        blk.kv_slot[m] = r * dm.max_tgt + lr + i; blk.att_n[m] = lr + i + 1;
+      }
+    }
+  }
+  __threadfence();
+  trace_mark(TR_ACCEPT, 2);
+}
+
+}  // namespace ad

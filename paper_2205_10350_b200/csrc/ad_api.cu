@@ -10,6 +10,7 @@
 #include <string>
 #include <vector>
 
+#include "accept.cuh"
 #include "ad_common.cuh"
 #include "attention.cuh"
 #include "attention_few.cuh"
@@ -122,6 +123,12 @@ struct ActSet {
   void *qbuf = nullptr, *ktmp = nullptr, *vtmp = nullptr;
 };
 
+NextPass no_next_pass() {
+  NextPass n = {};
+  n.source = -1;
+  return n;
+}
+
 thread_local std::string g_create_error;
 
 }  // namespace
@@ -166,11 +173,9 @@ struct ad_handle {
   int* down = nullptr;       // result block of finalize_generate_kernel (host view) ...
   int* down_dev = nullptr;   // ... and its device view
   bool defer_status = false; // ad_encode inside ad_generate: no synchronisation of its own
-  // Decode loop with small blocks: the accept kernel of iteration i also plans and embeds the block of iteration i + 1
-  // (loop_next.source >= 0), so an iteration starts at its first projection; pass_planned tells the pass being enqueued
-  // that its plan and embedding already exist.
-  NextBlock loop_next = {-1, 0, nullptr, 0, 0};
-  bool pass_planned = false;
+  // Decode loop: the accept kernel of one pass plans the pass behind it; next_pass is what the accept kernel being enqueued
+  // shall plan (source < 0: nothing).
+  NextPass next_pass = no_next_pass();
   bool profiling = false;    // ad_debug_profile_verify: an event in front of every launch
   std::vector<std::pair<std::string, cudaEvent_t>> prof;
   // state
@@ -544,15 +549,15 @@ cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw, cons
 }
 
 // Projection of a pass with few tokens (gemm_few.cuh).  ksplit: few::split_for of the shape, non-zero.
-template <int EPI>
-cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p, int ksplit) {
+template <int EPI, bool EMB = false>
+cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p, int ksplit, const few::EmbedParams& ep = {}) {
   const dim3 grid(p.N / few::FEAT, ksplit);
   const bf16 *w = (const bf16*)W.ptr, *xp = (const bf16*)x;
   switch (p.K / ksplit / 256) {
-    case 1: return launch_k(few::gemm_few_kernel<EPI, 1>, grid, dim3(few::THREADS), 0, st, w, xp, p);
-    case 2: return launch_k(few::gemm_few_kernel<EPI, 2>, grid, dim3(few::THREADS), 0, st, w, xp, p);
-    case 3: return launch_k(few::gemm_few_kernel<EPI, 3>, grid, dim3(few::THREADS), 0, st, w, xp, p);
-    default: return launch_k(few::gemm_few_kernel<EPI, 4>, grid, dim3(few::THREADS), 0, st, w, xp, p);
+    case 1: return launch_k(few::gemm_few_kernel<EPI, 1, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    case 2: return launch_k(few::gemm_few_kernel<EPI, 2, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    case 3: return launch_k(few::gemm_few_kernel<EPI, 3, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    default: return launch_k(few::gemm_few_kernel<EPI, 4, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
   }
 }
 // K split the few-token kernel takes for a projection of pass pc (0: the pass or the shape is not for it).
@@ -567,7 +572,8 @@ cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const Gem
   return launch_k(simt::gemm_f32_kernel<EPI>, grid, dim3(128), 0, st, (const float*)w, (const float*)x, p);
 }
 
-int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int* M_ptr, int M_cap, GemmParams p) {
+// embed_of: the operand is the embedding of pass pk's tokens (first projection of a pass, few-token kernel only).
+int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int* M_ptr, int M_cap, GemmParams p, const Model* embed_of = nullptr) {
   p.K = W.K; p.N = W.N; p.M_ptr = M_ptr; p.M_cap = M_cap; p.status = h->st.status;
   cudaError_t e;
   {
@@ -582,7 +588,14 @@ int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int
     switch (epi) {
       case EPI_F32: e = launch_few<EPI_F32>(h->stream, W, X.ptr, p, fs); break;
       case EPI_ACT: e = launch_few<EPI_ACT>(h->stream, W, X.ptr, p, fs); break;
-      default: e = launch_few<EPI_SCATTER>(h->stream, W, X.ptr, p, fs); break;
+      default:
+        if (embed_of) {
+          const few::EmbedParams ep = {(const bf16*)embed_of->emb.ptr, h->pe, sqrtf((float)W.K), h->pass[pk].plan.tok_id, h->pass[pk].plan.tok_pos, h->y};
+          e = launch_few<EPI_SCATTER, true>(h->stream, W, X.ptr, p, fs, ep);
+        } else {
+          e = launch_few<EPI_SCATTER>(h->stream, W, X.ptr, p, fs);
+        }
+        break;
     }
   } else if (h->bf16) {
     p.ntile = h->pass[pk].tile_for(W.N, num_sms());
@@ -714,9 +727,9 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
 // rounds of its warps, and a grid of at most one wave.
 bool attention_is_few(const ad_handle* h, const PassCfg& pc, int max_keys) {
   const ad_model_cfg& c = h->cfg;
-  if (!g_fuse_attn_proj || !h->bf16 || !h->pre2 || c.d_model != c.n_heads * 64 || c.d_model % 128 || c.n_heads > few::MAX_WARPS) return false;
-  if (max_keys > 2 * few::AK * c.n_heads) return false;
-  return (long)h->cfg.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads <= num_sms();
+  if (!g_fuse_attn_proj || !h->bf16 || !h->pre2 || c.d_model != c.n_heads * 64 || c.d_model % 128 || c.d_model > 128 * few::MAX_WARPS) return false;
+  if (max_keys > 2 * few::AK * few::att_few_warps(c.d_model)) return false;
+  return (long)h->cfg.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * few::att_few_split(c.d_model) <= num_sms();
 }
 
 // Attention with its output projection (partial sums per head in pre2) and, with wq, the query projection of x = yb.
@@ -732,27 +745,36 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   p.qchunks = (pc.seg_max + few::AQ - 1) / few::AQ;
   p.wo = (const bf16*)wo.ptr; p.o_part = h->pre2; p.o_stride = (size_t)pc.M_cap * c.d_model;
   if (wq) { fp.x = (const bf16*)h->yb.ptr; fp.wq = (const bf16*)wq->ptr; }
-  const dim3 grid(h->dims.B * p.qchunks, c.n_heads), block(32 * c.n_heads);
-  const size_t smem = few::att_few_smem(c.n_heads);
+  const int split = few::att_few_split(c.d_model), warps = few::att_few_warps(c.d_model);
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
   cudaError_t e = cudaSuccess;
   if (!attr_set[dev]) {
-    const int most8 = (int)few::att_few_smem(8), most16 = (int)few::att_few_smem(16);
-    e = cudaFuncSetAttribute(few::attention_few_kernel<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most8);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(few::attention_few_kernel<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, most8);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(few::attention_few_kernel<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most16);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(few::attention_few_kernel<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, most16);
+    const int most = (int)few::att_few_smem(few::MAX_WARPS);
+    for (auto* kernel : {few::attention_few_kernel<false, 1>, few::attention_few_kernel<true, 1>, few::attention_few_kernel<false, 2>,
+                         few::attention_few_kernel<true, 2>})
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention attribute: ") + cudaGetErrorString(e));
     attr_set[dev] = true;
   }
   note_launch(h, wq ? "q_proj+attention+out_proj" : "attention+out_proj");
-  if (c.n_heads <= 8)
-    e = wq ? launch_k(few::attention_few_kernel<true, 8>, grid, block, smem, h->stream, fp)
-           : launch_k(few::attention_few_kernel<false, 8>, grid, block, smem, h->stream, fp);
-  else
-    e = wq ? launch_k(few::attention_few_kernel<true, 16>, grid, block, smem, h->stream, fp)
-           : launch_k(few::attention_few_kernel<false, 16>, grid, block, smem, h->stream, fp);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(h->dims.B * p.qchunks * split, c.n_heads); cfg.blockDim = dim3(32 * warps);
+  cfg.dynamicSmemBytes = few::att_few_smem(warps); cfg.stream = h->stream;
+  cudaLaunchAttribute attr[2];
+  int n_attr = 0;
+  if (g_use_pdl) {
+    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (wq && split > 1) {
+    attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+    attr[n_attr].val.clusterDim.x = split; attr[n_attr].val.clusterDim.y = 1; attr[n_attr++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n_attr;
+  auto* kernel = split == 1 ? (wq ? few::attention_few_kernel<true, 1> : few::attention_few_kernel<false, 1>)
+                            : (wq ? few::attention_few_kernel<true, 2> : few::attention_few_kernel<false, 2>);
+  e = cudaLaunchKernelEx(&cfg, kernel, fp);
   if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
   return AD_OK;
 }
@@ -808,14 +830,20 @@ int embed(ad_handle* h, const PassCfg& pc, const Model& m) {
 
 #define AD_TRY(x) do { int rc__ = (x); if (rc__ != AD_OK) return rc__; } while (0)
 
+// Embedding of a pass's tokens: a kernel of its own, unless the pass's first projection computes it (null: it is done).
+int embed_or_defer(ad_handle* h, int pk, const Model& m, const Mat& first, const Model** deferred) {
+  *deferred = h->bf16 && few_split(h->pass[pk], EPI_SCATTER, first.N, first.K) > 0 ? &m : nullptr;
+  return *deferred ? AD_OK : embed(h, h->pass[pk], m);
+}
+
 // Self-attention sublayer + FFN shared by the encoder and decoder layers.
 int self_attention_sublayer(ad_handle* h, int pk, const Mat& wqkv, const float* bqkv, const Mat& wo, const float* bo,
-                            const float* lng, const float* lnb, void* kbuf, void* vbuf) {
+                            const float* lng, const float* lnb, void* kbuf, void* vbuf, const Model* embed_of = nullptr) {
   PassCfg& pc = h->pass[pk];
   GemmParams p = {};
   p.bias = bqkv; p.dst[0] = h->qbuf; p.dst[1] = kbuf; p.dst[2] = vbuf; p.seg_width = h->cfg.d_model; p.n_direct = 1;
   p.slot = pc.plan.kv_slot;
-  AD_TRY(gemm(h, EPI_SCATTER, wqkv, h->yb, pk, pc.plan.M, pc.M_cap, p));
+  AD_TRY(gemm(h, EPI_SCATTER, wqkv, h->yb, pk, pc.plan.M, pc.M_cap, p, embed_of));
   bool fused = false;
   const int max_keys = pk == PK_VERIFY ? h->dims.max_tgt : pc.seg_max;
   if (attention_is_few(h, pc, max_keys)) {
@@ -976,12 +1004,13 @@ int decoder_pass(ad_handle* h, int pk, Model& m) {
   PassCfg& pc = h->pass[pk];
   const size_t self_layer = (size_t)h->dims.max_tgt * c.max_batch * c.d_model * h->esz;
   const size_t cross_layer = (size_t)c.max_src * c.max_batch * c.d_model * h->esz;
-  if (!(pk == PK_VERIFY && h->pass_planned)) AD_TRY(embed(h, pc, m));
+  const Model* defer = nullptr;
+  AD_TRY(embed_or_defer(h, pk, m, m.dec[0].wqkv, &defer));
   for (int l = 0; l < c.n_dec; ++l) {
     DecLayer& L = m.dec[l];
     void* kb = pk == PK_VERIFY ? (char*)h->kself + l * self_layer : h->ktmp;
     void* vb = pk == PK_VERIFY ? (char*)h->vself + l * self_layer : h->vtmp;
-    AD_TRY(self_attention_sublayer(h, pk, L.wqkv, L.bqkv, L.wo, L.bo, L.ln1g, L.ln1b, kb, vb));
+    AD_TRY(self_attention_sublayer(h, pk, L.wqkv, L.bqkv, L.wo, L.bo, L.ln1g, L.ln1b, kb, vb, l == 0 ? defer : nullptr));
     // Query projection of the cross-attention.  With few tokens a full-K walk per CTA is the slow part of the
     // projection, so it is split along K and the attention kernel adds the partial sums (and the bias) as it
     // loads its queries.
@@ -1023,10 +1052,11 @@ int encoder_pass(ad_handle* h, Model& m, bool keep_memory) {
   const ad_model_cfg& c = h->cfg;
   PassCfg& pc = h->pass[PK_ENCODE];
   const size_t cross_layer = (size_t)c.max_src * c.max_batch * c.d_model * h->esz;
-  AD_TRY(embed(h, pc, m));
+  const Model* defer = nullptr;
+  AD_TRY(embed_or_defer(h, PK_ENCODE, m, m.enc[0].wqkv, &defer));
   for (int l = 0; l < c.n_enc; ++l) {
     EncLayer& L = m.enc[l];
-    AD_TRY(self_attention_sublayer(h, PK_ENCODE, L.wqkv, L.bqkv, L.wo, L.bo, L.ln1g, L.ln1b, h->ktmp, h->vtmp));
+    AD_TRY(self_attention_sublayer(h, PK_ENCODE, L.wqkv, L.bqkv, L.wo, L.bo, L.ln1g, L.ln1b, h->ktmp, h->vtmp, l == 0 ? defer : nullptr));
     AD_TRY(ffn_sublayer(h, PK_ENCODE, L.w1, L.b1, L.w2, L.b2, L.ln2g, L.ln2b));
   }
   if (keep_memory)
@@ -1065,22 +1095,10 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
   }
   if (!partials_ready) AD_TRY(gemm(h, EPI_ARGMAX, m.emb, X, PK_VERIFY, pc.plan.M, pc.M_cap, p));
   note_launch(h, "argmax_accept");
-  NextBlock nxt = {-1, 0, nullptr, 0, 0};
-  NextEmbed ne = {};
-  if (auto_commit && !to_drafts && h->loop_next.source >= 0) {
-    nxt = h->loop_next;
-    ne.emb = m.emb.ptr; ne.pe = h->pe; ne.d = h->cfg.d_model; ne.scale = sqrtf((float)h->cfg.d_model); ne.y = h->y; ne.yb = h->yb.ptr;
-  }
-  if (h->bf16)
-    AD_CUDA(h, launch_k(argmax_accept_kernel<bf16>, dim3(h->dims.B), dim3(1024), 0, h->stream, h->st, pc.plan, h->dims, (const float*)h->part_val, (const int*)h->part_idx, h->n_vtiles,
-                        pc.M_cap, to_drafts, auto_commit, (unsigned int*)(h->st.loop_it + 1),
-                        auto_commit ? h->cond_handle : 0ull, beta, h->tau, (const float*)h->draft_val, (const int*)h->draft_id,
-                        (const int*)h->part_cnt, nxt, ne));
-  else
-    AD_CUDA(h, launch_k(argmax_accept_kernel<float>, dim3(h->dims.B), dim3(1024), 0, h->stream, h->st, pc.plan, h->dims, (const float*)h->part_val, (const int*)h->part_idx, h->n_vtiles,
-                        pc.M_cap, to_drafts, auto_commit, (unsigned int*)(h->st.loop_it + 1),
-                        auto_commit ? h->cond_handle : 0ull, beta, h->tau, (const float*)h->draft_val, (const int*)h->draft_id,
-                        (const int*)h->part_cnt, nxt, ne));
+  AD_CUDA(h, launch_k(argmax_accept_kernel, dim3(h->dims.B), dim3(ACC_THREADS), 0, h->stream, h->st, pc.plan, h->dims, (const float*)h->part_val,
+                      (const int*)h->part_idx, h->n_vtiles, to_drafts, auto_commit, (unsigned int*)(h->st.loop_it + 1),
+                      auto_commit ? h->cond_handle : 0ull, beta, h->tau, (const float*)h->draft_val, (const int*)h->draft_id,
+                      (const int*)h->part_cnt, h->next_pass));
   h->last_vocab_which = to_drafts ? 1 : 0;
   return AD_OK;
 }
@@ -1092,11 +1110,15 @@ int prepare_verify(ad_handle* h, int source, int k_cap, const int* ovr, int ovr_
   return AD_OK;
 }
 
-// Draft substep: sizes, drafter plan, drafter decoder, gather of the mask rows, projection + arg-max.
-int draft_stage(ad_handle* h, int k_cap) {
+// Draft substep: sizes and drafter plan ...
+int plan_draft(ad_handle* h, int k_cap) {
   AD_TRY(prepare_verify(h, SRC_SIZES, k_cap, nullptr, 0));
-  note_launch(h, "draft_stage");
+  note_launch(h, "plan_draft");
   AD_CUDA(h, launch_k(plan_draft_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_VERIFY].plan, h->pass[PK_DRAFT].plan, h->dims));
+  return AD_OK;
+}
+// ... then the drafter's decoder, gather of the mask rows, projection + arg-max.
+int draft_stage(ad_handle* h) {
   if (mega_applies(h, PK_DRAFT)) {      // decoder stack, gather of the mask rows and projection in one kernel
     AD_TRY(mega_launch(h, PK_DRAFT));
     return vocab_stage(h, h->nar, h->xg, 1, 0, true);
@@ -1104,7 +1126,7 @@ int draft_stage(ad_handle* h, int k_cap) {
   AD_TRY(decoder_pass(h, PK_DRAFT, h->nar));
   const int d = h->cfg.d_model;
   PassCfg& pv = h->pass[PK_VERIFY];
-  note_launch(h, "draft_stage");
+  note_launch(h, "gather_rows");
   if (h->bf16) AD_CUDA(h, launch_k(gather_rows_kernel<bf16>, dim3(pv.M_cap), dim3(128), 0, h->stream, (const int*)pv.plan.M, (const int*)h->st.gidx, (const bf16*)h->yb.ptr, (bf16*)h->xg.ptr, d));
   else AD_CUDA(h, launch_k(gather_rows_kernel<float>, dim3(pv.M_cap), dim3(128), 0, h->stream, (const int*)pv.plan.M, (const int*)h->st.gidx, (const float*)h->yb.ptr, (float*)h->xg.ptr, d));
   return vocab_stage(h, h->nar, h->xg, 1, 0);
@@ -1125,46 +1147,54 @@ int commit_stage(ad_handle* h, const int* n_dev) {
   return AD_OK;
 }
 
+// Whether the accept kernels of a decode loop plan the passes behind them (kernel-chain form of the passes only).
+bool g_fuse_plan = true;      // AD_NO_FUSED_PLAN=1: plan in kernels of their own in every iteration
+bool loop_plans_ahead(const ad_handle* h) { return g_fuse_plan && !h->mega[PK_VERIFY].on && !h->mega[PK_DRAFT].on; }
+bool loop_drafts(const ad_gen_opts& o) { return o.mode == AD_MODE_GAD && o.run_drafter; }
+int block_source(const ad_gen_opts& o, const int* ovr) { return o.mode == AD_MODE_GAD || ovr ? SRC_OVERRIDE : SRC_POLICY; }
+
+NextPass next_pass(const ad_handle* h, int source, int k_cap, const int* ovr, int ovr_len) {
+  NextPass n = no_next_pass();
+  n.source = source; n.k_cap = k_cap; n.override_stream = ovr; n.override_stride = h->cfg.max_tgt; n.override_len = ovr_len;
+  n.draft = h->pass[PK_DRAFT].plan;
+  return n;
+}
+
+// First pass of a loop that plans ahead: planned by kernels of their own.
+int plan_first_pass(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_len) {
+  if (loop_drafts(o)) return plan_draft(h, o.k);
+  return prepare_verify(h, block_source(o, ovr), o.k, ovr, ovr_len);
+}
+
 // One iteration of the decode loop: draft -> verify -> commit, all on the device.
-// Whether the loop of these options lets the accept kernel plan and embed the next block: no drafter pass in between,
-// blocks small enough for one CTA to embed, kernel-chain form of the pass.
-bool g_fuse_plan = true;      // AD_NO_FUSED_PLAN=1: plan and embed as kernels of their own in every iteration
-bool loop_plans_ahead(const ad_handle* h, const ad_gen_opts& o) {
-  return g_fuse_plan && !(o.mode == AD_MODE_GAD && o.run_drafter) && h->pass[PK_VERIFY].M_cap <= 128 && !h->mega[PK_VERIFY].on;
-}
-
-// First block of a loop that plans ahead: planned and embedded by kernels of their own, before the loop.
-int plan_first_block(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_len) {
-  AD_TRY(prepare_verify(h, (o.mode == AD_MODE_GAD || ovr) ? SRC_OVERRIDE : SRC_POLICY, o.k, ovr, ovr_len));
-  return embed(h, h->pass[PK_VERIFY], h->ar);
-}
-
 int loop_iteration(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_len) {
-  struct Shrinking {
-    PassCfg& pc;
-    Shrinking(PassCfg& p, bool on) : pc(p) { pc.shrinking = on; }
-    ~Shrinking() { pc.shrinking = false; }
-  } scope(h->pass[PK_VERIFY], o.mode == AD_MODE_IAD);
-  if (loop_plans_ahead(h, o)) {
-    // this iteration's plan and embedding exist already (plan_first_block, or the previous iteration's accept kernel)
-    h->loop_next = NextBlock{(o.mode == AD_MODE_GAD || ovr) ? SRC_OVERRIDE : SRC_POLICY, o.k, ovr, h->cfg.max_tgt, ovr_len};
-    h->pass_planned = true;
-    const int rc = verify_stage(h, 1);
-    h->pass_planned = false;
-    h->loop_next.source = -1;
-    return rc;
-  }
-  if (o.mode == AD_MODE_GAD) {
-    if (o.run_drafter) {
-      AD_TRY(draft_stage(h, o.k));
+  struct Scope {               // whatever way this function is left
+    ad_handle* h;
+    ~Scope() {
+      h->pass[PK_VERIFY].shrinking = false;
+      h->next_pass = no_next_pass();
+    }
+  } scope{h};
+  h->pass[PK_VERIFY].shrinking = o.mode == AD_MODE_IAD;
+  if (!loop_plans_ahead(h)) {
+    if (loop_drafts(o)) {
+      AD_TRY(plan_draft(h, o.k));
+      AD_TRY(draft_stage(h));
       AD_TRY(prepare_verify(h, SRC_KEEP, o.k, ovr, ovr_len));
     } else {
-      AD_TRY(prepare_verify(h, SRC_OVERRIDE, o.k, ovr, ovr_len));
+      AD_TRY(prepare_verify(h, block_source(o, ovr), o.k, ovr, ovr_len));
     }
-  } else {
-    AD_TRY(prepare_verify(h, ovr ? SRC_OVERRIDE : SRC_POLICY, o.k, ovr, ovr_len));
+    return verify_stage(h, 1);   // accept and commit in one kernel
   }
-  return verify_stage(h, 1);   // accept and commit in one kernel
+  // this iteration's first pass has been planned already (plan_first_pass, or the previous iteration's accept kernel)
+  if (loop_drafts(o)) {
+    h->next_pass = next_pass(h, SRC_KEEP, o.k, ovr, ovr_len);
+    AD_TRY(draft_stage(h));
+    h->next_pass = next_pass(h, SRC_SIZES, o.k, nullptr, 0);
+  } else {
+    h->next_pass = next_pass(h, block_source(o, ovr), o.k, ovr, ovr_len);
+  }
+  return verify_stage(h, 1);
 }
 
 int read_status(ad_handle* h) {
@@ -1484,7 +1514,8 @@ extern "C" int ad_draft_block(ad_handle* h, int32_t k_cap, int32_t* drafts, int3
   if (!h->cfg.has_drafter) return fail(h, AD_ERR_STATE, "the handle has no drafter model");
   const ad_model_cfg& c = h->cfg;
   if (k_cap < 1 || k_cap > c.kmax) return fail(h, AD_ERR_ARG, "k_cap outside 1..kmax");
-  AD_TRY(draft_stage(h, k_cap));
+  AD_TRY(plan_draft(h, k_cap));
+  AD_TRY(draft_stage(h));
   const int B = h->B;
   if (on_host) {
     if (drafts) AD_CUDA(h, cudaMemcpyAsync(drafts, h->st.drafts, sizeof(int) * (size_t)B * c.kmax, cudaMemcpyDeviceToHost, h->stream));
@@ -1625,7 +1656,7 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
     }
   }
 
-  if (loop_plans_ahead(h, *opts)) AD_TRY(plan_first_block(h, *opts, ovr, ovr_len));
+  if (loop_plans_ahead(h)) AD_TRY(plan_first_pass(h, *opts, ovr, ovr_len));
   if (device_loop) {
     // one launch runs every iteration; the data-independent bound on the iteration count travels in loop_it[3]
     h->host_flag[1] = max_iters + 1;

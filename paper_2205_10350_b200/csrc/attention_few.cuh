@@ -2,9 +2,12 @@
 // cross-attention, the query projection as well.
 //
 // A CTA handles one head and up to 16 queries of one row.  Everything is latency: a few dozen keys, a few thousand
-// multiply-adds.  The CTA's d / 64 warps therefore split whatever there is to split: the contraction of the query
-// projection (64 input features per warp), the keys (16 per warp and round), the output features of the output projection
-// (64 per warp).  All products are warp-level MMAs on fragments read with 16-byte loads (contraction index permuted
+// multiply-adds.  The CTA's warps therefore split whatever there is to split: the contraction of the query projection (64
+// input features per warp), the keys (16 per warp and round), the output features of the output projection (64 per warp).
+// Models up to 512 wide take d / 64 warps in one CTA; wider ones two CTAs of d / 128 warps (SPLIT = 2), so that both
+// projections' weights still fit the registers of eight warps: each CTA of the pair projects the queries over half of the
+// input features (the halves meet through distributed shared memory, the pair being a cluster) and the output to half of
+// the output features; the attention in between is done by both.  All products are warp-level MMAs on fragments read with 16-byte loads (contraction index permuted
 // identically for both operands, see gemm_few.cuh).  Weights, and for the cross-attention the keys and values (written
 // by the encoder pass long before), are requested before the dependency wait; plan data is read there too.
 //
@@ -28,7 +31,7 @@ constexpr int AK = 16;            // keys per warp and round
 constexpr int K_LD = 96;          // key rows: 192 bytes apart (16-byte fragment loads without bank conflicts)
 constexpr int V_LD = 72;          // value rows: 144 bytes apart (ldmatrix without bank conflicts)
 constexpr int O_LD = 68;          // floats per row of a warp's partial output
-constexpr int MAX_WARPS = 16;
+constexpr int MAX_WARPS = 8;      // per CTA
 
 struct FewAttnParams {
   AttnParams a;
@@ -39,8 +42,11 @@ struct FewAttnParams {
 inline size_t att_few_smem(int warps) {
   const size_t kv = (size_t)warps * AK * (K_LD + V_LD) * sizeof(bf16);
   const size_t part = (size_t)warps * AQ * O_LD * sizeof(float);      // partial query projections, later partial outputs
-  return kv + part + 2 * (size_t)warps * AQ * sizeof(float) + 2 * (size_t)AQ * K_LD * sizeof(bf16);
+  return kv + part + 2 * (size_t)warps * AQ * sizeof(float) + 2 * (size_t)AQ * K_LD * sizeof(bf16) + 2 * (size_t)AQ * 64 * sizeof(float);
 }
+// CTAs a head's work is split over, and warps per CTA.
+inline int att_few_split(int d) { return d > 64 * MAX_WARPS ? 2 : 1; }
+inline int att_few_warps(int d) { return d / 64 / att_few_split(d); }
 
 __device__ __forceinline__ void cp16(void* smem_dst, const void* gmem_src, bool there) {
   const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
@@ -57,10 +63,10 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
   lo = pack2(a - __low2float(h), b - __high2float(h));
 }
 
-// grid = (B * qchunks, H), qchunks = ceil(longest segment / 16); block = 32 * (d / 64) threads; dynamic smem att_few_smem.
-// MAXW: most warps of the build (8: up to 255 registers per thread, models up to 512 wide; 16: 128 registers).
-template <bool QPROJ, int MAXW>
-__global__ void __launch_bounds__(32 * MAXW, 1)
+// grid = (B * qchunks * SPLIT, H), qchunks = ceil(longest segment / 16); block = 32 * att_few_warps(d) threads; dynamic smem
+// att_few_smem; cluster (SPLIT, 1, 1) when QPROJ and SPLIT == 2.
+template <bool QPROJ, int SPLIT>
+__global__ void __launch_bounds__(32 * MAX_WARPS, 1)
 attention_few_kernel(const FewAttnParams fp) {
   const AttnParams& p = fp.a;
   extern __shared__ __align__(16) uint8_t few_smem[];
@@ -68,7 +74,9 @@ attention_few_kernel(const FewAttnParams fp) {
   pdl_launch();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int nw = blockDim.x >> 5, nthreads = blockDim.x;
-  const int b = blockIdx.x / p.qchunks, chunk = blockIdx.x - b * p.qchunks, h = blockIdx.y;
+  const int rank = SPLIT == 1 ? 0 : blockIdx.x % SPLIT, row_chunk = blockIdx.x / SPLIT;
+  const int b = row_chunk / p.qchunks, chunk = row_chunk - b * p.qchunks, h = blockIdx.y;
+  const int slice = (rank * nw + warp) * 64;      // this warp's input features of the query projection, output features of Wo
   const int d = p.d;
   const int seg_len = plan_load(p.seg_len + b);
   const int i0 = chunk * AQ;
@@ -84,23 +92,24 @@ attention_few_kernel(const FewAttnParams fp) {
   float* pl = pm + nw * AQ;                                                           // [nw][16] sums
   bf16* qs = reinterpret_cast<bf16*>(pl + nw * AQ);                                   // [16][K_LD] queries
   bf16* os = qs + AQ * K_LD;                                                          // [16][K_LD] outputs
+  // (the pair's first barrier: a CTA's shared memory may be written once it is known to run)
+  if (QPROJ && SPLIT > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  float* xq = reinterpret_cast<float*>(os + AQ * K_LD);                               // [SPLIT][16][64] the pair's query halves
 
   // weights: rows 8 j + g of this head's query projection / of this warp's 64 output features, 64-wide slices of K
-  uint4 wf[8][2];
+  uint4 wf[8][2], wqf[QPROJ ? 8 : 1][2];
   if (QPROJ) {
-    const bf16* wb = fp.wq + (size_t)(h * 64 + g) * d + warp * 64 + 8 * t;
+    const bf16* wb = fp.wq + (size_t)(h * 64 + g) * d + slice + 8 * t;
 #pragma unroll
     for (int j = 0; j < 8; ++j)
 #pragma unroll
-      for (int c = 0; c < 2; ++c) wf[j][c] = __ldg(reinterpret_cast<const uint4*>(wb + (size_t)(8 * j) * d + 32 * c));
+      for (int c = 0; c < 2; ++c) wqf[QPROJ ? j : 0][c] = __ldg(reinterpret_cast<const uint4*>(wb + (size_t)(8 * j) * d + 32 * c));
   }
-  const bf16* ob = p.wo + (size_t)(warp * 64 + g) * d + h * 64 + 8 * t;
-  if (!QPROJ) {
+  const bf16* ob = p.wo + (size_t)(slice + g) * d + h * 64 + 8 * t;
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
+  for (int j = 0; j < 8; ++j)
 #pragma unroll
-      for (int c = 0; c < 2; ++c) wf[j][c] = __ldg(reinterpret_cast<const uint4*>(ob + (size_t)(8 * j) * d + 32 * c));
-  }
+    for (int c = 0; c < 2; ++c) wf[j][c] = __ldg(reinterpret_cast<const uint4*>(ob + (size_t)(8 * j) * d + 32 * c));
   const int m0 = plan_load(p.seg_off + b) + i0;
   const int kbase = plan_load(p.key_base + b), row_nk = plan_load(p.nkeys_row + b);
   const int nq = min(AQ, seg_len - i0);
@@ -128,15 +137,14 @@ attention_few_kernel(const FewAttnParams fp) {
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   if (QPROJ) fetch(0);          // the encoder's keys and values: older than the plan
-  float4 qbias = make_float4(0.f, 0.f, 0.f, 0.f);
   pdl_wait();
   trace_mark(TR_ATTN, 1);
   if (!QPROJ) fetch(0);
 
   uint4 qa[2][2];               // query fragments: [32-wide chunk of the head][row g / g + 8]
   if (QPROJ) {
-    const bf16* x0 = fp.x + (size_t)(m0 + r0) * d + warp * 64 + 8 * t;
-    const bf16* x1 = fp.x + (size_t)(m0 + r1) * d + warp * 64 + 8 * t;
+    const bf16* x0 = fp.x + (size_t)(m0 + r0) * d + slice + 8 * t;
+    const bf16* x1 = fp.x + (size_t)(m0 + r1) * d + slice + 8 * t;
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       qa[c][0] = *reinterpret_cast<const uint4*>(x0 + 32 * c);
@@ -148,15 +156,11 @@ attention_few_kernel(const FewAttnParams fp) {
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j) mma16816(acc[j], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, wf[j][c].x, wf[j][c].y);
+      for (int j = 0; j < 8; ++j) mma16816(acc[j], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, wqf[QPROJ ? j : 0][c].x, wqf[QPROJ ? j : 0][c].y);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) mma16816(acc[j], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, wf[j][c].z, wf[j][c].w);
+      for (int j = 0; j < 8; ++j) mma16816(acc[j], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, wqf[QPROJ ? j : 0][c].z, wqf[QPROJ ? j : 0][c].w);
     }
-    // the output projection's weights arrive while the scores are computed
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) wf[j][c] = __ldg(reinterpret_cast<const uint4*>(ob + (size_t)(8 * j) * d + 32 * c));
+    trace_mark(TR_ATTN, 3);
     float* pw = part + (size_t)warp * AQ * O_LD;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -164,18 +168,39 @@ attention_few_kernel(const FewAttnParams fp) {
       *reinterpret_cast<float2*>(pw + (g + 8) * O_LD + 8 * j + 2 * t) = make_float2(acc[j][2], acc[j][3]);
     }
     __syncthreads();
+    if (SPLIT > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     for (int idx = tid; idx < AQ * 16; idx += nthreads) {
       const int r = idx >> 4, c = (idx & 15) * 4;
-      qbias = *reinterpret_cast<const float4*>(p.q_bias + h * 64 + c);
-      float4 v = qbias;
-#pragma unroll 4
+      float4 v = SPLIT == 1 ? *reinterpret_cast<const float4*>(p.q_bias + h * 64 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
       for (int w = 0; w < nw; ++w) {
         const float4 o = *reinterpret_cast<const float4*>(part + ((size_t)w * AQ + r) * O_LD + c);
         v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
       }
-      uint2 u;
-      u.x = pack2(v.x, v.y); u.y = pack2(v.z, v.w);
-      *reinterpret_cast<uint2*>(qs + r * K_LD + c) = u;
+      if (SPLIT == 1) {
+        uint2 u;
+        u.x = pack2(v.x, v.y); u.y = pack2(v.z, v.w);
+        *reinterpret_cast<uint2*>(qs + r * K_LD + c) = u;
+      } else {
+        float* mine = xq + (rank * AQ + r) * 64 + c;
+        *reinterpret_cast<float4*>(mine) = v;
+        uint32_t peer;
+        const uint32_t local = static_cast<uint32_t>(__cvta_generic_to_shared(mine));
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(local), "r"(rank ^ 1));
+        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(peer), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+      }
+    }
+    if (SPLIT > 1) {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      for (int idx = tid; idx < AQ * 16; idx += nthreads) {
+        const int r = idx >> 4, c = (idx & 15) * 4;
+        const float4 bq = *reinterpret_cast<const float4*>(p.q_bias + h * 64 + c);
+        const float4 a0 = *reinterpret_cast<const float4*>(xq + r * 64 + c), a1 = *reinterpret_cast<const float4*>(xq + (AQ + r) * 64 + c);
+        uint2 u;
+        u.x = pack2(bq.x + a0.x + a1.x, bq.y + a0.y + a1.y); u.y = pack2(bq.z + a0.z + a1.z, bq.w + a0.w + a1.w);
+        *reinterpret_cast<uint2*>(qs + r * K_LD + c) = u;
+      }
     }
     __syncthreads();
 #pragma unroll
@@ -193,6 +218,7 @@ attention_few_kernel(const FewAttnParams fp) {
     }
   }
 
+  trace_mark(TR_ATTN, 4);
   float o[8][4];
 #pragma unroll
   for (int j = 0; j < 8; ++j) { o[j][0] = 0.f; o[j][1] = 0.f; o[j][2] = 0.f; o[j][3] = 0.f; }
@@ -257,6 +283,7 @@ attention_few_kernel(const FewAttnParams fp) {
     }
   }
   // merge the warps that had keys
+  trace_mark(TR_ATTN, 5);
   const int na = min(nw, (row_nk + AK - 1) / AK);
   den0 += __shfl_xor_sync(0xffffffffu, den0, 1); den1 += __shfl_xor_sync(0xffffffffu, den1, 1);
   den0 += __shfl_xor_sync(0xffffffffu, den0, 2); den1 += __shfl_xor_sync(0xffffffffu, den1, 2);
@@ -291,6 +318,7 @@ attention_few_kernel(const FewAttnParams fp) {
     *reinterpret_cast<uint2*>(os + r * K_LD + c) = u;
   }
   __syncthreads();
+  trace_mark(TR_ATTN, 6);
   // output projection: 16 queries x this warp's 64 features, K = this head's 64 dimensions
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
@@ -306,7 +334,8 @@ attention_few_kernel(const FewAttnParams fp) {
 #pragma unroll
     for (int j = 0; j < 8; ++j) mma16816(o[j], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, wf[j][c].z, wf[j][c].w);
   }
-  float* dst = p.o_part + (size_t)h * p.o_stride + (size_t)m0 * d + warp * 64 + 2 * t;
+  trace_mark(TR_ATTN, 7);
+  float* dst = p.o_part + (size_t)h * p.o_stride + (size_t)m0 * d + slice + 2 * t;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     if (g < nq) *reinterpret_cast<float2*>(dst + (size_t)g * d + 8 * j) = make_float2(o[j][0], o[j][1]);

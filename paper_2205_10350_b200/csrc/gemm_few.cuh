@@ -47,11 +47,39 @@ inline int split_for(int N, int K, bool may_split, int max_split) {
   return s;
 }
 
+// First projection of a pass: its operand is the embedding of the planned tokens, x = emb[token] * sqrt(d) + PE[position],
+// computed where it is used; the CTAs also share the writing of the FP32 residual stream y.
+struct EmbedParams {
+  const bf16* emb;
+  const float* pe;
+  float scale;
+  const int *tok_id, *tok_pos;
+  float* y;
+};
+// Eight consecutive elements of x, rounded like a stored operand.
+__device__ __forceinline__ uint4 embed8(const EmbedParams& ep, int tok, int pos, int K, int k) {
+  const uint4 e = __ldg(reinterpret_cast<const uint4*>(ep.emb + (size_t)tok * K + k));
+  const float4 p0 = __ldg(reinterpret_cast<const float4*>(ep.pe + (size_t)pos * K + k));
+  const float4 p1 = __ldg(reinterpret_cast<const float4*>(ep.pe + (size_t)pos * K + k + 4));
+  const float pp[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+  const uint32_t w[4] = {e.x, e.y, e.z, e.w};
+  uint32_t r[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float a = __uint_as_float(w[i] << 16) * ep.scale + pp[2 * i];
+    const float b = __uint_as_float(w[i] & 0xffff0000u) * ep.scale + pp[2 * i + 1];
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    r[i] = *reinterpret_cast<const uint32_t*>(&h);
+  }
+  return make_uint4(r[0], r[1], r[2], r[3]);
+}
+
 // grid = (N / 16, ksplit); block = 256; K / ksplit = 256 * NCH.
 // EPI_F32: partial sums [ksplit][M_cap, N] (no bias); EPI_ACT: bias (+ ReLU) -> BF16; EPI_SCATTER: q / K / V rows.
-template <int EPI, int NCH>
+// EMB: the operand is the embedding (ep), X is not read; nothing depends on the predecessor until the first store.
+template <int EPI, int NCH, bool EMB>
 __global__ void __launch_bounds__(THREADS, 2)
-gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p) {
+gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, const EmbedParams ep) {
   constexpr int TPR = round_tokens(NCH);
   constexpr int NT = TPR / 8;
   __shared__ __align__(16) float red[WARPS][TPR][RED_LD];
@@ -74,7 +102,7 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p) {
   const int M = plan_load(p.M_ptr);
   int slot = 0;
   if (EPI == EPI_SCATTER && ot < M) slot = plan_load(p.slot + ot);
-  pdl_wait();
+  if (!EMB) pdl_wait();
   trace_mark(TR_GEMM + EPI, 1);
   for (int t0 = 0; t0 < M; t0 += TPR) {
     float acc[NT][4];
@@ -82,9 +110,16 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p) {
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
       if (t0 + 8 * nt < M) {
-        const bf16* xr = X + (size_t)min(t0 + 8 * nt + g, p.M_cap - 1) * K + kbase;
+        if (EMB) {
+          const int m = min(t0 + 8 * nt + g, M - 1);
+          const int tok = plan_load(ep.tok_id + m), pos = plan_load(ep.tok_pos + m);
 #pragma unroll
-        for (int c = 0; c < NCH; ++c) xb[nt][c] = *reinterpret_cast<const uint4*>(xr + 32 * c);
+          for (int c = 0; c < NCH; ++c) xb[nt][c] = embed8(ep, tok, pos, p.K, kbase + 32 * c);
+        } else {
+          const bf16* xr = X + (size_t)min(t0 + 8 * nt + g, p.M_cap - 1) * K + kbase;
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) xb[nt][c] = *reinterpret_cast<const uint4*>(xr + 32 * c);
+        }
       }
     }
 #pragma unroll
@@ -108,6 +143,7 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p) {
       }
     }
     __syncthreads();
+    if (EMB && t0 == 0) pdl_wait();
     const int m = t0 + ot;
     if (ot < TPR && m < M) {
       float4 v = *reinterpret_cast<const float4*>(&red[0][ot][of]);
@@ -136,6 +172,21 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p) {
         u.x = *reinterpret_cast<unsigned int*>(&h0);
         u.y = *reinterpret_cast<unsigned int*>(&h1);
         *reinterpret_cast<uint2*>(dst) = u;
+      }
+    }
+  }
+  if (EMB) {
+    if (M <= 0) pdl_wait();                                  // (a grid without work still ends after its predecessor)
+    const int groups = p.K >> 2;
+    for (int m = blockIdx.x; m < M; m += gridDim.x) {
+      const int tok = plan_load(ep.tok_id + m), pos = plan_load(ep.tok_pos + m);
+      for (int i = tid; i < groups; i += THREADS) {
+        const uint2 e = __ldg(reinterpret_cast<const uint2*>(ep.emb + (size_t)tok * K + 4 * i));
+        const float4 pp = __ldg(reinterpret_cast<const float4*>(ep.pe + (size_t)pos * K + 4 * i));
+        float4 v;
+        v.x = __uint_as_float(e.x << 16) * ep.scale + pp.x; v.y = __uint_as_float(e.x & 0xffff0000u) * ep.scale + pp.y;
+        v.z = __uint_as_float(e.y << 16) * ep.scale + pp.z; v.w = __uint_as_float(e.y & 0xffff0000u) * ep.scale + pp.w;
+        *reinterpret_cast<float4*>(ep.y + (size_t)m * K + 4 * i) = v;
       }
     }
   }

@@ -85,8 +85,7 @@ __device__ int warp_suffix_match(const int* out, int j, const int* src, int n, i
 // Decoder inputs of row b are (last accepted token, drafts[0..k-2]) at positions len .. len+k-1
 // (Eq. 6 / Eq. 7); a negative draft that would be fed is replaced by [PAD].
 // Executed by ALL threads of one CTA (any multiple of 32 threads); s_k / s_off: shared arrays of 256 / 257 ints.
-// The per-row state is read past L1: the caller may be the last CTA of the accept kernel, reading what the other
-// CTAs of that kernel have just committed.
+// (Inside a decode loop the accept kernel does this for the next iteration, see accept.cuh.)
 // ---------------------------------------------------------------------------------------------
 struct NextBlock {
   int source;                  // DraftSource
@@ -336,6 +335,15 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
 }
 __device__ __forceinline__ float block_sum_128(float v, float* red) { return block_sum<128>(v, red); }
 
+__device__ __forceinline__ void load4(const float* p, float (&v)[4]) {
+  const float4 f = *reinterpret_cast<const float4*>(p);
+  v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+}
+__device__ __forceinline__ void load4(const bf16* p, float (&v)[4]) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  v[0] = __uint_as_float(u.x << 16); v[1] = __uint_as_float(u.x & 0xffff0000u);
+  v[2] = __uint_as_float(u.y << 16); v[3] = __uint_as_float(u.y & 0xffff0000u);
+}
 __device__ __forceinline__ void store4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
 __device__ __forceinline__ void store4(bf16* p, float4 v) {
   __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
@@ -556,20 +564,11 @@ __device__ __forceinline__ void commit_row(const DevState& st, const PassPlan& b
 }
 
 // After every row has been committed: loop counter and the "all rows finished" word.  One thread.
-// cond != 0: the iteration runs inside a device-side `while` graph node; the node repeats while its condition
-// is non-zero, so it is cleared when every row has finished -- or, as a bound that does not depend on the data,
-// when the iteration counter st.loop_it[2] reaches the limit st.loop_it[3] the host stored before the launch.
-__device__ __forceinline__ void finish_iteration(const DevState& st, const Dims& dm, bool any_active,
-                                                 unsigned long long cond) {
+__device__ __forceinline__ void finish_iteration(const DevState& st, const Dims& dm, bool any_active) {
   int all = 1;
   for (int b = 0; b < dm.B; ++b) all &= (__ldcg(st.fin + b) != 0);
   if (any_active) *st.loop_it += 1;
   *st.all_fin = all;
-  if (cond) {
-    const int it = st.loop_it[2] + 1;
-    st.loop_it[2] = it;
-    cudaGraphSetConditional(cond, (all || it >= st.loop_it[3]) ? 0u : 1u);
-  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -599,147 +598,6 @@ draft_score_kernel(DevState st, PassPlan blk, Dims dm, const WT* __restrict__ em
 }
 
 // ---------------------------------------------------------------------------------------------
-// Final arg-max over the per-tile partials of the fused projection, then the draft compare:
-//   c = first block position whose greedy choice differs from the draft (Section 3.1.1; definition of c
-//   in Section 3.2), n = c + 1 (the bifurcation token is kept), n = k when nothing differs, cut at the
-//   first accepted [EOS].  One CTA per row, one warp per block position for the reduction; warp 0 takes the
-//   decision with ballots.
-// beta >= 1: relaxed verification of Section 3.2.3 -- a position keeps its drafted token when fewer than beta other
-//   tokens score strictly higher (Eq. 8: the draft is within the top beta) and the best score exceeds the draft's
-//   by at most tau (Eq. 9; differences of log-likelihoods are differences of scores); otherwise the greedy choice.
-// to_drafts != 0: drafter mode, the choices are written as the row's drafts and nothing is compared.
-// auto_commit != 0: the row's n_accepted is committed right away (decode loop); the last CTA to finish
-//   updates the loop counter and the all-finished word (done_ctr: rows done in the low half, active rows in
-//   the high half; left at zero).
-// next.source >= 0 (decode loop, small blocks): the LAST CTA to finish also chooses the next iteration's blocks
-//   (plan_verify_block) and embeds their tokens (y = emb[token] * sqrt(d) + PE[pos]), so that the next iteration starts
-//   at its first projection: two launches fewer per iteration.
-// grid = B, block = 1024.
-// ---------------------------------------------------------------------------------------------
-struct NextEmbed {
-  const void* emb;       // embedding matrix in the weight type
-  const float* pe;
-  int d;
-  float scale;
-  float* y;
-  void* yb;              // GEMM-operand copy in the activation type
-};
-
-template <typename WT>
-__global__ void __launch_bounds__(1024)
-argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict__ part_val,
-                     const int* __restrict__ part_idx, int n_tiles, int M_cap, int to_drafts, int auto_commit,
-                     unsigned int* done_ctr, unsigned long long cond, int beta, float tau,
-                     const float* __restrict__ draft_val, const int* __restrict__ draft_id,
-                     const int* __restrict__ part_cnt, NextBlock next, NextEmbed ne) {
-  __shared__ int s_k[256];
-  __shared__ int s_off[257];
-  __shared__ int s_last;
-  trace_mark(TR_ACCEPT, 0);
-  if (next.source < 0) pdl_launch();     // a kernel that plans never does (see plan data in ad_common.cuh)
-  const int b = blockIdx.x;
-  const int k = plan_load(blk.seg_len + b);
-  pdl_wait();
-  trace_mark(TR_ACCEPT, 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int* pred = (to_drafts ? st.drafts : st.pred) + (size_t)b * dm.kmax;
-  if (k > 0) {
-    const int off = blk.seg_off[b];
-    for (int i = warp; i < k; i += 32) {
-      const int m = off + i;
-      float v = -INFINITY;
-      int idx = 0x7fffffff;
-      int higher = 0;
-      const bool relaxed = beta >= 1 && !to_drafts;
-      for (int t = lane; t < n_tiles; t += 32) {
-        const float ov = part_val[(size_t)m * n_tiles + t];
-        const int oi = part_idx[(size_t)m * n_tiles + t];
-        if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-        if (relaxed) higher += part_cnt[(size_t)m * n_tiles + t];
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-        if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-        higher += __shfl_xor_sync(0xffffffffu, higher, o);
-      }
-      if (lane == 0) {
-        int choice = idx;
-        if (relaxed) {
-          const int did = draft_id[m];
-          if (did >= 0 && higher <= beta - 1 && v - draft_val[m] <= tau) choice = did;
-        }
-        pred[i] = choice;
-      }
-    }
-  }
-  if (to_drafts) return;
-  if (tid == 0) s_last = 0;
-  __syncthreads();
-  if (warp == 0) {
-    int n = 0;
-    if (k > 0) {
-      const int* dr = st.drafts + (size_t)b * dm.kmax;
-      n = k;
-      bool found = false;
-      for (int i0 = 0; i0 < k && !found; i0 += 32) {
-        const int i = i0 + lane;
-        const bool mism = (i < k) && (dr[i] < 0 || pred[i] != dr[i]);
-        const unsigned bal = __ballot_sync(0xffffffffu, mism);
-        if (bal) { n = i0 + __ffs(bal); found = true; }
-      }
-      found = false;
-      for (int i0 = 0; i0 < n && !found; i0 += 32) {
-        const int i = i0 + lane;
-        const bool is_eos = (i < n) && (pred[i] == dm.eos);
-        const unsigned bal = __ballot_sync(0xffffffffu, is_eos);
-        if (bal) { n = i0 + __ffs(bal); found = true; }
-      }
-    }
-    if (lane == 0) st.n_acc[b] = n;
-    if (auto_commit) {
-      __syncwarp();
-      commit_row(st, blk, dm, b, n, n, lane);
-      if (lane == 0) {
-        __threadfence();
-        const unsigned int t = atomicAdd(done_ctr, n > 0 ? 0x10001u : 1u);
-        if ((t & 0xffffu) == (unsigned)dm.B - 1) {
-          __threadfence();
-          finish_iteration(st, dm, ((t >> 16) + (n > 0 ? 1u : 0u)) != 0, cond);
-          *done_ctr = 0;
-          s_last = 1;
-        }
-      }
-    }
-  }
-  if (auto_commit && next.source >= 0) {
-    __syncthreads();
-    if (s_last) {                  // block-uniform: this CTA saw every row committed
-      __threadfence();
-      plan_verify_block(st, blk, dm, next, s_k, s_off);
-      __syncthreads();
-      // embedding of the next block's tokens (written by this CTA just above)
-      const int M = s_off[dm.B], d = ne.d, groups = d >> 2;
-      const WT* emb = reinterpret_cast<const WT*>(ne.emb);
-      WT* yb = reinterpret_cast<WT*>(ne.yb);
-      for (int idx = tid; idx < M * groups; idx += blockDim.x) {
-        const int m = idx / groups, c = (idx - m * groups) * 4;
-        const WT* er = emb + (size_t)blk.tok_id[m] * d + c;
-        const float4 pp = *reinterpret_cast<const float4*>(ne.pe + (size_t)blk.tok_pos[m] * d + c);
-        float4 v;
-        v.x = to_f32(er[0]) * ne.scale + pp.x; v.y = to_f32(er[1]) * ne.scale + pp.y;
-        v.z = to_f32(er[2]) * ne.scale + pp.z; v.w = to_f32(er[3]) * ne.scale + pp.w;
-        *reinterpret_cast<float4*>(ne.y + (size_t)m * d + c) = v;
-        store4(yb + (size_t)m * d + c, v);
-      }
-      __threadfence();
-    }
-  }
-  trace_mark(TR_ACCEPT, 2);
-}
-
-// ---------------------------------------------------------------------------------------------
 // Commit as a call of its own (ad_commit): cache-length advance or rollback.  n_in == null commits n_acc.
 // grid = 1, block = 256 (one warp per row at a time).
 // ---------------------------------------------------------------------------------------------
@@ -761,7 +619,7 @@ commit_kernel(DevState st, PassPlan blk, Dims dm, const int* n_in) {
     if (lane == 0 && nacc > 0) atomicOr(&s_active, 1);
   }
   __syncthreads();
-  if (threadIdx.x == 0) finish_iteration(st, dm, s_active != 0, 0ull);
+  if (threadIdx.x == 0) finish_iteration(st, dm, s_active != 0);
 }
 
 // Teacher-forced commit: the caller supplies the accepted tokens.  grid = 1, block = 256.

@@ -1,0 +1,63 @@
+"""Passes of few tokens (register-resident projections, attention with both projections in one kernel, loop planning in the
+accept kernel) against the checker, at the edges of their ranges: widths (one to four K chunks, one CTA or a pair per head),
+query tiles of 16, rounds of 64 and 32 tokens, the last pass size they take, keys beyond one round of the warps."""
+import numpy as np
+import pytest
+
+from oracle import ad_oracle as O
+from paper_2205_10350_b200 import synth
+from tests.parity_util import lockstep
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,ffn,batch,k,src,tgt", [
+    (256, 512, 1, 1, 3, 9),          # one token
+    (256, 768, 2, 17, 66, 70),       # one K chunk, a query tile and one more; keys in two rounds of four warps
+    (512, 2048, 1, 64, 40, 128),     # one full round of tokens, last key of the only round
+    (512, 1024, 2, 64, 129, 64),     # 128 tokens; source keys in a second round of eight warps
+    (512, 512, 1, 33, 20, 129),      # self-attention keys in a second round
+    (768, 1536, 3, 9, 30, 24),       # three K chunks, a pair of CTAs with six warps each
+    (1024, 1024, 2, 33, 17, 40),     # four K chunks, a pair of CTAs with eight warps each
+])
+def test_few_token_passes_follow_the_checker(d, ffn, batch, k, src, tgt):
+    from paper_2205_10350_b200 import binding
+    shape = synth.ModelShape(f"few_{d}_{ffn}", d, d // 64, ffn, 1003, 1, 2, "bf16")
+    w = synth.make_weights(shape, 0)
+    model = O.Model(shape, w, max_pos=256)
+    r = np.random.default_rng(d + batch + k)
+    lens = r.integers(max(1, src - 3), src + 1, size=batch).astype(np.int32)
+    lens[0] = src
+    srcs = r.integers(4, shape.vocab, size=(batch, src)).astype(np.int32)
+    dec = binding.AggressiveDecoder(shape, w, max_batch=batch, max_src=src, max_tgt=tgt, kmax=k)
+    streams = []
+    for b in range(batch):
+        g, _ = model.state(srcs[b, : lens[b]], cap=tgt).greedy(tgt)
+        row = np.full((1, tgt), 5, np.int32)
+        row[0, : len(g)] = g
+        streams.append(synth.corrupt_stream(row, [tgt], 0.95, shape.vocab, 9, b)[0])
+    stats = lockstep(dec, model, srcs, lens, streams, k, [tgt] * batch, tol=5e-2, max_steps=6)
+    print(stats)
+    assert stats["steps"] > 0
+    dec.close()
+
+
+@pytest.mark.parametrize("mode,run_drafter,k", [("IAD", False, 7), ("IAD", False, 1), ("GAD", True, 5), ("GAD", True, 12)])
+def test_loop_planned_by_the_accept_kernel_equals_one_kernel_per_plan(mode, run_drafter, k, monkeypatch):
+    """Whole loops of a ragged batch: planning inside the accept kernel and planning in kernels of their own give the same
+    tokens and the same counts, as a graph and as direct launches."""
+    from paper_2205_10350_b200 import binding
+    shape = synth.MINI_BF16
+    w, wn = synth.make_weights(shape, 0), synth.make_weights(shape, 1)
+    r = np.random.default_rng(k)
+    lens = np.array([12, 5, 1, 9, 12], np.int32)
+    src = r.integers(4, 60, size=(5, 12)).astype(np.int32)      # few ids: suffix matches that need more than one token
+    results = []
+    for env in ("0", "1"):
+        monkeypatch.setenv("AD_NO_FUSED_PLAN", env)
+        dec = binding.AggressiveDecoder(shape, w, wn if run_drafter else None, max_batch=5, max_src=12, max_tgt=16, kmax=12)
+        for graph in (True, False):
+            out, st = dec.generate(src, lens, mode=mode, k=k, max_len=[16, 3, 9, 16, 1], run_drafter=run_drafter, use_graph=graph)
+            results.append(([list(map(int, o)) for o in out], st["iterations"], st["row_iterations"], st["accepted"], st["offered"]))
+        dec.close()
+    assert all(x == results[0] for x in results[1:])
