@@ -568,8 +568,35 @@ int few_split(const PassCfg& pc, int epi, int N, int K) {
 
 template <int EPI>
 cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const GemmParams& p, int M_cap) {
-  dim3 grid((p.N + 127) / 128, (M_cap + simt::TOK - 1) / simt::TOK);
-  return launch_k(simt::gemm_f32_kernel<EPI>, grid, dim3(128), 0, st, (const float*)w, (const float*)x, p);
+  constexpr int FEAT = EPI == EPI_ARGMAX ? simt::ARGMAX_FEAT : 64;
+  constexpr size_t smem = simt::smem_bytes<FEAT>();
+  static bool attr_set[kMaxDevices] = {};
+  const int dev = current_device();
+  if (!attr_set[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(simt::gemm_f32_kernel<EPI, FEAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = true;
+  }
+  const int vec = p.K % 4 == 0 && (reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(x)) % 16 == 0;
+  const dim3 grid((p.N + FEAT - 1) / FEAT, (M_cap + simt::TOK - 1) / simt::TOK);
+  return launch_k(simt::gemm_f32_kernel<EPI, FEAT>, grid, dim3(2 * FEAT), smem, st, (const float*)w, (const float*)x, p, vec);
+}
+// The few-token FP32 kernel: passes of at most kFewTokens tokens, shapes it covers.
+bool f32_few(const PassCfg& pc, int epi, int N, int K) { return pc.M_cap <= kFewTokens && epi != EPI_ARGMAX && simt::few_fits(N, K); }
+template <int EPI>
+cudaError_t launch_simt_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p) {
+  const dim3 grid(p.N / simt::F_FEAT), block(256);
+  const float *w = (const float*)W.ptr, *xp = (const float*)x;
+  switch (p.K / 64) {
+    case 1: return launch_k(simt::gemm_f32_few_kernel<EPI, 1>, grid, block, 0, st, w, xp, p);
+    case 2: return launch_k(simt::gemm_f32_few_kernel<EPI, 2>, grid, block, 0, st, w, xp, p);
+    case 3: return launch_k(simt::gemm_f32_few_kernel<EPI, 3>, grid, block, 0, st, w, xp, p);
+    case 4: return launch_k(simt::gemm_f32_few_kernel<EPI, 4>, grid, block, 0, st, w, xp, p);
+    case 5: return launch_k(simt::gemm_f32_few_kernel<EPI, 5>, grid, block, 0, st, w, xp, p);
+    case 6: return launch_k(simt::gemm_f32_few_kernel<EPI, 6>, grid, block, 0, st, w, xp, p);
+    case 7: return launch_k(simt::gemm_f32_few_kernel<EPI, 7>, grid, block, 0, st, w, xp, p);
+    default: return launch_k(simt::gemm_f32_few_kernel<EPI, 8>, grid, block, 0, st, w, xp, p);
+  }
 }
 
 // embed_of: the operand is the embedding of pass pk's tokens (first projection of a pass, few-token kernel only).
@@ -612,8 +639,13 @@ int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int
                 : launch_tc<EPI_ARGMAX>(h->stream, W.map, mx, p, M_cap);
         break;
     }
+  } else if (p.M_ptr && f32_few(h->pass[pk], epi, W.N, W.K)) {
+    switch (epi) {
+      case EPI_F32: e = launch_simt_few<EPI_F32>(h->stream, W, X.ptr, p); break;
+      case EPI_ACT: e = launch_simt_few<EPI_ACT>(h->stream, W, X.ptr, p); break;
+      default: e = launch_simt_few<EPI_SCATTER>(h->stream, W, X.ptr, p); break;
+    }
   } else {
-    p.ntile = simt::TOK;
     switch (epi) {
       case EPI_F32: e = launch_simt<EPI_F32>(h->stream, W.ptr, X.ptr, p, M_cap); break;
       case EPI_ACT: e = launch_simt<EPI_ACT>(h->stream, W.ptr, X.ptr, p, M_cap); break;
@@ -1936,7 +1968,6 @@ extern "C" int ad_vocab_argmax(const void* x, const void* emb, int32_t dtype, in
       e = launch_tc<EPI_ARGMAX>(st, mw, mx, p, M);
     }
   } else if (dtype == AD_DTYPE_FP32) {
-    p.ntile = simt::TOK;
     e = launch_simt<EPI_ARGMAX>(st, emb, x, p, M);
   } else {
     return AD_ERR_ARG;
@@ -1961,7 +1992,6 @@ extern "C" int ad_linear(const void* x, const void* W, const float* bias, int32_
     if (!make_map(&mw, W, N, K, tc::BLOCK_N_FEAT) || !make_map(&mx, x, M, K, p.ntile)) return AD_ERR_CUDA;
     e = launch_tc<EPI_F32>(st, mw, mx, p, M);
   } else if (dtype == AD_DTYPE_FP32) {
-    p.ntile = simt::TOK;
     e = launch_simt<EPI_F32>(st, W, x, p, M);
   } else {
     return AD_ERR_ARG;

@@ -1,106 +1,224 @@
-// FP32 projection GEMM on the FP32 pipes (FFMA), for models whose weights are FP32 and whose scores have to
-// match an FP32 definition to 1e-3: no TF32, no reduced-precision operands.  Same D^T[n, m] orientation and
-// the same epilogues as the tensor-core kernel: one thread per output feature, 16 tokens per CTA, the
-// contraction index walked in ascending order.
+// FP32 projection GEMMs on the FP32 pipes (FFMA), for models whose weights are FP32 and whose scores have to match an FP32
+// definition to 1e-3: no TF32, no reduced-precision operands.  Same D^T[n, m] orientation and the same epilogues as the
+// tensor-core kernels.
+//
+// Two kernels.  gemm_f32_kernel: tiles of 64 or 128 features x 32 tokens, both operands copied asynchronously to shared memory
+// as they lie (no transposition: a thread multiplies 4 x 4 outputs by four consecutive k at a time, eight 16-byte shared
+// loads for 64 FFMA), contraction index walked in ascending order.  333 x 2048 x 512: 80 -> 21 us (the kernel before had one
+// thread per feature, 16 tokens and scalar loads).  gemm_f32_few_kernel: passes of few tokens, where that kernel's serial walk
+// along K is all latency: 16 features per CTA, K dealt to 16 half-warps, weights in registers before the dependency wait.
 #pragma once
 
 #include "ad_common.cuh"
-#include "gemm_tc.cuh"   // epilogue_chunk, warp_argmax
+#include "gemm_tc.cuh"   // warp_argmax
 
 namespace ad {
 namespace simt {
 
-constexpr int FEAT = 128;
-constexpr int TOK = 16;
-constexpr int KT = 32;
+constexpr int TOK = 32;           // tokens per tile
+constexpr int KT = 32;            // k per stage
+constexpr int LDK = KT + 4;       // rows 144 bytes apart: conflict-free 16-byte reads of consecutive rows
+constexpr int STAGES = 3;
+constexpr int ARGMAX_FEAT = 128;  // features per tile of the arg-max epilogue: the layout of the partial arrays
 
-// grid = (ceil(N / 128), ceil(M_cap / 16)); block = 128.  x: [M_cap, K] float, w: [N, K] float.
+template <int FEAT>
+constexpr size_t smem_bytes() { return sizeof(float) * (size_t)STAGES * (FEAT + TOK) * LDK; }
+
+__device__ __forceinline__ void cp16(void* s, const void* g, bool there) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(s))), "l"(g),
+               "r"(there ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp4(void* s, const void* g, bool there) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(s))), "l"(g),
+               "r"(there ? 4 : 0) : "memory");
+}
+
+// One output row of the non-arg-max epilogues.
 template <int EPI>
-__global__ void __launch_bounds__(128)
-gemm_f32_kernel(const float* __restrict__ w, const float* __restrict__ x, const GemmParams p) {
-  __shared__ float ws[KT][FEAT + 1];
-  __shared__ float xs[TOK][KT];
-  __shared__ float red_val[4][TOK];
-  __shared__ int red_idx[4][TOK];
-  __shared__ int red_cnt[4][TOK];
-
-  pdl_launch();
-  pdl_wait();
-  const int M = p.M_ptr ? *p.M_ptr : p.M_host;
-  const int t0 = blockIdx.y * TOK;
-  if (t0 >= M) return;
-  const int n0 = blockIdx.x * FEAT;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int K = p.K;
-
-  float acc[TOK];
-#pragma unroll
-  for (int j = 0; j < TOK; ++j) acc[j] = 0.f;
-
-  for (int k0 = 0; k0 < K; k0 += KT) {
-#pragma unroll
-    for (int i = 0; i < (FEAT * KT) / 128; ++i) {
-      const int idx = i * 128 + tid;
-      const int row = idx / KT, col = idx % KT;
-      const int n = n0 + row, k = k0 + col;
-      ws[col][row] = (n < p.N && k < K) ? w[(size_t)n * K + k] : 0.f;
-    }
-#pragma unroll
-    for (int i = 0; i < (TOK * KT) / 128; ++i) {
-      const int idx = i * 128 + tid;
-      const int row = idx / KT, col = idx % KT;
-      const int m = t0 + row, k = k0 + col;
-      xs[row][col] = (m < M && k < K) ? x[(size_t)m * K + k] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < KT; ++kk) {
-      const float wv = ws[kk][tid];
-#pragma unroll
-      for (int j = 0; j < TOK; ++j) acc[j] = fmaf(wv, xs[j][kk], acc[j]);
-    }
-    __syncthreads();
+__device__ __forceinline__ void store_out(const GemmParams& p, int n, int m, float v) {
+  if (EPI == EPI_F32) {
+    p.out_f32[(size_t)m * p.N + n] = v;
+  } else if (EPI == EPI_ACT) {
+    reinterpret_cast<float*>(p.out_act)[(size_t)m * p.N + n] = p.relu ? fmaxf(v, 0.f) : v;
+  } else {
+    const int s = n / p.seg_width, c = n - s * p.seg_width;
+    const int row = s < p.n_direct ? m : plan_load(p.slot + m);
+    char* base = p.seg_pair_stride ? static_cast<char*>(p.dst[s & 1]) + (size_t)(s >> 1) * p.seg_pair_stride : static_cast<char*>(p.dst[s]);
+    reinterpret_cast<float*>(base)[(size_t)row * p.seg_width + c] = v;
   }
+}
 
-  const int n = n0 + tid;
-  if (EPI == EPI_ARGMAX) {
-#pragma unroll
-    for (int j = 0; j < TOK; ++j) {
-      float v = (n < p.N) ? acc[j] : -INFINITY;
-      int i = n;
-      if (p.draft_val) {   // relaxed verification: features other than the draft that score strictly higher
-        const bool on = t0 + j < M;
-        const bool above = on && n < p.N && n != p.draft_id[t0 + j] && acc[j] > p.draft_val[t0 + j];
-        const unsigned int bal = __ballot_sync(0xffffffffu, above);
-        if (lane == 0) red_cnt[warp][j] = __popc(bal);
+// grid = (ceil(N / FEAT), ceil(M_cap / 32)); block = 2 * FEAT; dynamic smem smem_bytes<FEAT>().  x: [M_cap, K], w: [N, K].
+// vec: K is a multiple of four and both operands are 16-byte aligned.
+template <int EPI, int FEAT>
+__global__ void __launch_bounds__(2 * FEAT)
+gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p, const int vec) {
+  constexpr int THREADS = 2 * FEAT, TX = FEAT / 4;     // thread (tx, ty): features tx + TX i, tokens ty + 8 j (i, j < 4)
+  extern __shared__ __align__(16) float simt_smem[];   // [STAGES][FEAT + TOK][LDK]
+  const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
+  const int t0 = blockIdx.y * TOK, n0 = blockIdx.x * FEAT;
+  pdl_launch();
+  if (t0 >= M && blockIdx.y > 0) return;
+  pdl_wait();
+  if (t0 >= M) return;
+  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const int K = p.K, nk = (K + KT - 1) / KT;
+  auto fetch = [&](int kt) {
+    float* dst = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK;
+    const int k0 = kt * KT;
+    if (kt < nk) {
+      if (vec) {
+        for (int idx = tid; idx < (FEAT + TOK) * (KT / 4); idx += THREADS) {
+          const int r = idx / (KT / 4), c = (idx % (KT / 4)) * 4;
+          const bool is_w = r < FEAT;
+          const int row = is_w ? n0 + r : t0 + r - FEAT;
+          const bool there = row < (is_w ? p.N : M) && k0 + c < K;
+          cp16(dst + r * LDK + c, (is_w ? w : x) + (there ? (size_t)row * K + k0 + c : 0), there);
+        }
+      } else {
+        for (int idx = tid; idx < (FEAT + TOK) * KT; idx += THREADS) {
+          const int r = idx / KT, c = idx % KT;
+          const bool is_w = r < FEAT;
+          const int row = is_w ? n0 + r : t0 + r - FEAT;
+          const bool there = row < (is_w ? p.N : M) && k0 + c < K;
+          cp4(dst + r * LDK + c, (is_w ? w : x) + (there ? (size_t)row * K + k0 + c : 0), there);
+        }
       }
-      tc::warp_argmax(v, i);
-      if (lane == 0) { red_val[warp][j] = v; red_idx[warp][j] = i; }
     }
-    __syncthreads();
-    if (tid < TOK && t0 + tid < M) {
-      float v = red_val[0][tid];
-      int i = red_idx[0][tid];
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float acc[4][4];
 #pragma unroll
-      for (int wq = 1; wq < 4; ++wq) {
-        const float ov = red_val[wq][tid];
-        const int oi = red_idx[wq][tid];
-        if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll
+  for (int s = 0; s < STAGES - 1; ++s) fetch(s);
+  for (int kt = 0; kt < nk; ++kt) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+    __syncthreads();                                    // stage kt has landed, stage kt - 1 is free
+    fetch(kt + STAGES - 1);
+    const float* ws = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + tx * LDK;
+    const float* xs = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + (FEAT + ty) * LDK;
+#pragma unroll
+    for (int k = 0; k < KT; k += 4) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(ws + i * TX * LDK + k);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(xs + j * 8 * LDK + k);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+    }
+  }
+  if (EPI == EPI_ARGMAX) {
+    // FEAT == 128: a warp holds all 128 features of its four tokens; ascending ids on ties
+    const int lane = tid & 31;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int m = t0 + ty + 8 * j;
+      const bool on = m < M;                            // warp-uniform
+      float v = -INFINITY;
+      int id = 0x7fffffff, cnt = 0;
+      const float dval = p.draft_val && on ? p.draft_val[m] : 0.f;
+      const int did = p.draft_val && on ? p.draft_id[m] : -1;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int n = n0 + tx + TX * i;
+        if (n < p.N) {
+          if (acc[i][j] > v) { v = acc[i][j]; id = n; }
+          if (p.draft_val && n != did && acc[i][j] > dval) ++cnt;   // other features that score strictly higher
+        }
       }
-      p.part_val[(size_t)(t0 + tid) * gridDim.x + blockIdx.x] = v;
-      p.part_idx[(size_t)(t0 + tid) * gridDim.x + blockIdx.x] = i;
-      if (p.draft_val)
-        p.part_cnt[(size_t)(t0 + tid) * gridDim.x + blockIdx.x] =
-            red_cnt[0][tid] + red_cnt[1][tid] + red_cnt[2][tid] + red_cnt[3][tid];
+      tc::warp_argmax(v, id);
+      if (p.draft_val) cnt = __reduce_add_sync(0xffffffffu, cnt);
+      if (lane == 0 && on) {
+        const size_t o = (size_t)m * gridDim.x + blockIdx.x;
+        p.part_val[o] = v;
+        p.part_idx[o] = id;
+        if (p.draft_val) p.part_cnt[o] = cnt;
+      }
     }
   } else {
-    __shared__ int slot_s[TOK];
-    if (EPI == EPI_SCATTER) {
-      if (tid < TOK) slot_s[tid] = (t0 + tid < M) ? p.slot[t0 + tid] : 0;
-      __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int n = n0 + tx + TX * i;
+      if (n >= p.N) continue;
+      const float b = p.bias ? p.bias[n] : 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int m = t0 + ty + 8 * j;
+        if (m < M) store_out<EPI>(p, n, m, acc[i][j] + b);
+      }
     }
-    const float b = (p.bias && n < p.N) ? p.bias[n] : 0.f;
-    tc::epilogue_chunk<EPI, float>(p, n, t0, M, acc, b, p.out_f32, slot_s, 0);
+  }
+}
+
+// ---- few tokens ------------------------------------------------------------------------------------------
+constexpr int F_FEAT = 16;        // features per CTA
+constexpr int F_TOK = 16;         // tokens per round
+constexpr int F_PARTS = 16;       // half-warps of the CTA = parts of K
+constexpr int F_MAX_K = 512;
+
+inline bool few_fits(int N, int K) { return N % F_FEAT == 0 && K % 64 == 0 && K <= F_MAX_K; }
+
+// grid = N / 16, block = 256; K / 16 = 4 * NQ consecutive k per half-warp.  Lane: feature lane % 16.
+template <int EPI, int NQ>
+__global__ void __launch_bounds__(256)
+gemm_f32_few_kernel(const float* __restrict__ w, const float* x, const GemmParams p) {
+  constexpr int K = 64 * NQ;
+  __shared__ __align__(16) float xs[F_TOK][K];
+  __shared__ float red[F_PARTS][F_TOK][F_FEAT];
+  pdl_launch();
+  const int tid = threadIdx.x, f = tid & 15, part = tid >> 4, n0 = blockIdx.x * F_FEAT;
+  float4 wr[NQ];
+#pragma unroll
+  for (int i = 0; i < NQ; ++i) wr[i] = __ldg(reinterpret_cast<const float4*>(w + (size_t)(n0 + f) * K + part * 4 * NQ + 4 * i));
+  const float bias = p.bias ? p.bias[n0 + f] : 0.f;
+  const int M = plan_load(p.M_ptr);
+  pdl_wait();
+  for (int t0 = 0; t0 < M; t0 += F_TOK) {
+    if (t0 > 0) __syncthreads();
+    for (int idx = tid; idx < F_TOK * (K / 4); idx += 256) {
+      const int r = idx / (K / 4), c = (idx % (K / 4)) * 4;
+      if (t0 + r < M) cp16(&xs[r][c], x + (size_t)(t0 + r) * K + c, true);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    const int nt = min(F_TOK, M - t0);
+#pragma unroll 4
+    for (int r = 0; r < nt; ++r) {
+      float s = 0.f;
+#pragma unroll
+      for (int i = 0; i < NQ; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(&xs[r][part * 4 * NQ + 4 * i]);
+        s = fmaf(wr[i].x, v.x, s); s = fmaf(wr[i].y, v.y, s); s = fmaf(wr[i].z, v.z, s); s = fmaf(wr[i].w, v.w, s);
+      }
+      red[part][r][f] = s;
+    }
+    __syncthreads();
+    const int r = tid >> 4;                             // one output per thread
+    if (r < nt) {
+      float s = red[0][r][f];
+#pragma unroll
+      for (int q = 1; q < F_PARTS; ++q) s += red[q][r][f];
+      store_out<EPI>(p, n0 + f, t0 + r, s + bias);
+    }
   }
 }
 

@@ -241,32 +241,6 @@ __device__ __forceinline__ void warp_argmax(float& v, int& i) {
   }
 }
 
-// Applies the epilogue to 16 consecutive tokens (m0 .. m0+15) of output feature n held by this thread.
-// b is the bias of feature n (0 when there is none); slot_s holds the K/V slot of every token of the tile.
-template <int EPI, typename ActT>
-__device__ __forceinline__ void epilogue_chunk(const GemmParams& p, int n, int m0, int M, const float* acc, float b,
-                                               float* out_f32, const int* slot_s, int j0) {
-  if (n >= p.N) return;
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int m = m0 + j;
-    if (m >= M) break;
-    float v = acc[j] + b;
-    if (EPI == EPI_F32) {
-      out_f32[(size_t)m * p.N + n] = v;
-    } else if (EPI == EPI_ACT) {
-      if (p.relu) v = fmaxf(v, 0.f);
-      reinterpret_cast<ActT*>(p.out_act)[(size_t)m * p.N + n] = from_f32<ActT>(v);
-    } else if (EPI == EPI_SCATTER) {
-      const int s = n / p.seg_width, c = n - s * p.seg_width;
-      const int row = (s < p.n_direct) ? m : slot_s[j0 + j];
-      char* seg_base = p.seg_pair_stride ? static_cast<char*>(p.dst[s & 1]) + (size_t)(s >> 1) * p.seg_pair_stride
-                                         : static_cast<char*>(p.dst[s]);
-      reinterpret_cast<ActT*>(seg_base)[(size_t)row * p.seg_width + c] = from_f32<ActT>(v);
-    }
-  }
-}
-
 // grid = (ceil(N / 128), ceil(M_cap / ntile), ksplit); block = 256 threads;
 // dynamic smem = stages * stage bytes + 1024.
 //

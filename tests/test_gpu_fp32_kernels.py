@@ -1,0 +1,55 @@
+"""FP32 projection kernels at the edges of their tiles (64 / 128 features x 32 tokens x 32 k, vector and scalar copies) and of
+the few-token form (16 features, 16-token rounds, K up to 512), against the checker."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import ad_oracle as O
+from paper_2205_10350_b200 import binding, synth
+from tests.parity_util import lockstep
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+OPS = O.Ops("f32")
+
+
+@pytest.mark.parametrize("M,K,N", [(1, 1, 1), (32, 32, 64), (33, 36, 65), (31, 30, 63), (65, 130, 128), (96, 512, 200), (333, 96, 129)])
+def test_linear_tiles(M, K, N):
+    r = np.random.default_rng(M + K + N)
+    x, W = r.standard_normal((M, K)).astype(np.float32), (r.standard_normal((N, K)) * 0.1).astype(np.float32)
+    b = r.standard_normal(N).astype(np.float32)
+    y = binding.linear(torch.tensor(x, device=DEV), torch.tensor(W, device=DEV), torch.tensor(b, device=DEV))
+    assert np.abs(y.cpu().numpy() - OPS.linear(x, W.T.copy(), b)).max() < 1e-4
+
+
+@pytest.mark.parametrize("M,d,V", [(1, 128, 128), (33, 50, 129), (40, 128, 1000)])
+def test_argmax_tiles(M, d, V):
+    r = np.random.default_rng(M + V)
+    x, W = r.standard_normal((M, d)).astype(np.float32), r.standard_normal((V, d)).astype(np.float32)
+    W[V - 1] = W[V // 2]                     # equal scores: the lowest id wins
+    x[0] = 10 * W[V - 1]
+    got = binding.vocab_argmax(torch.tensor(x, device=DEV), torch.tensor(W, device=DEV)).cpu().numpy()
+    ref = OPS.linear(x, W.T.copy(), np.zeros(V, np.float32))
+    assert got[0] == V // 2
+    top = np.sort(ref, 1)
+    clear = top[:, -1] - top[:, -2] > 1e-3
+    assert np.array_equal(got[clear], ref.argmax(1)[clear])
+
+
+@pytest.mark.parametrize("d,heads,ffn,batch,k", [(64, 2, 64, 1, 1), (128, 4, 512, 2, 17), (320, 10, 448, 1, 16), (128, 2, 640, 3, 33)])
+def test_passes_follow_the_checker(d, heads, ffn, batch, k):
+    """The last shape's K = 640 is beyond the few-token form; 3 x 33 tokens take seven of its rounds."""
+    shape = synth.ModelShape(f"f32_{d}_{ffn}", d, heads, ffn, 301, 1, 2, "fp32")
+    w = synth.make_weights(shape, 0)
+    model = O.Model(shape, w, max_pos=64)
+    r = np.random.default_rng(d + k)
+    lens = np.array([11, 7, 1][:batch], np.int32)
+    src = r.integers(4, shape.vocab, size=(batch, 11)).astype(np.int32)
+    dec = binding.AggressiveDecoder(shape, w, max_batch=batch, max_src=11, max_tgt=40, kmax=k)
+    streams = r.integers(4, shape.vocab, size=(batch, 40)).astype(np.int32)
+    for b in range(batch):
+        g, _ = model.state(src[b, : lens[b]], cap=40).greedy(40)
+        streams[b, : len(g)] = np.where(r.random(len(g)) < 0.9, g, streams[b, : len(g)])
+    stats = lockstep(dec, model, src, lens, streams, k, [40] * batch, tol=1e-3, max_steps=5)
+    assert stats["steps"] > 0
+    dec.close()
