@@ -8,6 +8,8 @@
 #include <algorithm>
 #include <map>
 #include <string>
+#include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "accept.cuh"
@@ -38,11 +40,11 @@ struct ActBuf {
   void* ptr = nullptr;
   int cols = 0;
   // one map per pass kind and token tile: box rows 16, 32, 64, 128, 256 (index log2(rows) - 4), up to the pass's own tile
-  CUtensorMap map[PK_COUNT][5];
+  tc::TileMaps map[PK_COUNT];
   const CUtensorMap& map_for(int pk, int tile) const {
     int i = 0;
     while ((16 << i) < tile && i < 4) ++i;
-    return map[pk][i];
+    return map[pk].m[i];
   }
 };
 struct EncLayer {
@@ -67,54 +69,18 @@ struct Model {
   float* cbkv_pack = nullptr;
 };
 // Passes of at most this many packed tokens run their projections on the few-token kernel (gemm_few.cuh).
-constexpr int kFewTokens = 128;
+constexpr int kFewTokens = few::MAX_TOKENS;
 
 struct PassCfg {
   int M_cap = 0;     // packed-token capacity of this pass kind
   int ntile = 16;    // tokens per GEMM tile
   int seg_max = 0;   // longest segment of one row
   int max_split = 1; // largest split-K factor this pass may use (sizes the partial-sum buffer)
-  bool shrinking = false;   // set while an input-guided decode loop launches this pass: its blocks shrink every iteration
   PassPlan plan;
-  // Split-K factor of a projection that feeds the LayerNorm kernel: enough CTAs to cover the SMs when the
-  // token dimension alone gives only a handful of tiles (power of two, divides the K blocks, <= max_split).
-  // Token tile for a projection with N output features: the pass's tile, or half of a 256-token tile when the
-  // full tile would give fewer CTAs than two per SM (the K loop costs the same per CTA either way).
-  // Token tile of a projection with N output features.  Up to 64 tokens: one tile (more, smaller tiles were measured
-  // slower for a 40-token block).  Beyond that the pass's kernels are latency-bound and smaller tiles win -- more CTAs,
-  // more MMA issuers per CTA, a shorter epilogue each -- until the grids outgrow the SMs; measured per step (base model):
-  //   100 / 120 / 128 tokens: 64-token tiles 277 / 289 / 293 us against 305 / 316 / 321 us with one 128-token tile;
-  //   200 / 240 tokens: 32-token tiles 331 / 305 us, 64: 344 / 311, 128: 364 / 336, 16: 372;
-  //   320 / 400 / 512 tokens: 64-token tiles 366 / 357 / 389 us against 415 / 410 / 458 (128) and 383 / 380 / 410 (32);
-  //   800 / 1024 tokens: 64-token tiles 455 / 468 us against 477 / 486 (128);  2048 tokens: 128-token tiles 543 us, 64: 571.
-  int tile_for(int N, int n_sms) const {
-    if (M_cap <= 64) return ntile;
-    if (M_cap <= 128) return 64;
-    if (M_cap <= 256) return 32;
-    if (M_cap <= 1024) return 64;
-    // Inside an input-guided decode loop a block is what is left of the sentence: the packed token count falls with
-    // every iteration while the launch shapes stay those of the capacity, so up to 2048 tokens of capacity the loop
-    // takes the tile of the sizes it mostly runs at (batch 32, blocks of up to 64: 364 against 382 us per iteration,
-    // although one full 2048-token step costs 571 against 543 us).
-    if (shrinking && M_cap <= 2048) return 64;
-    if (ntile == 256 && ((N + 127) / 128) * ((M_cap + 255) / 256) < 2 * n_sms) return 128;
-    return ntile;
-  }
-  int ksplit_for(int N, int K, int tile) const {
-    const int tiles = ((N + 127) / 128) * ((M_cap + tile - 1) / tile);
-    const int kb = K / 64;
-    int s = 1;
-    // Up to 256 tokens: at most one CTA per SM.  (With 128-token tiles a 128-CTA grid of these one-CTA-per-SM kernels ran
-    // 16 of its CTAs as a second wave behind the 32 CTAs of the projection before it; with the 32- and 64-token tiles such
-    // passes take now the projection before it fills the SMs itself and the full-width split is as fast or faster: big
-    // model, 100 tokens, 392 against 417 us per step.)  With many tokens the grid has several waves anyway and the split
-    // keeps the K loops short.
-    // (a single token tile, up to 64 tokens: 112 -- the big model's 25-token pass loses 4 % with 128 one-K-block CTAs)
-    const int cap = M_cap <= 64 ? 112 : (M_cap <= 256 ? 148 : 160);
-    while (s * 2 <= max_split && tiles * s * 2 <= cap && kb % (s * 2) == 0) s *= 2;
-    return s;
-  }
 };
+
+// Launch shape of the tensor-core projection kernel (see tc_shape).
+struct TcShape { int ctas, budget, smem; };
 
 // A second set of activation buffers (encoder-pass sized) for work that runs on the side stream.
 struct ActSet {
@@ -185,6 +151,7 @@ struct ad_handle {
   std::string err;
   struct GraphEntry { cudaGraphExec_t exec; int launches; bool device_loop; };
   std::map<std::string, GraphEntry> graphs;
+  std::map<std::tuple<int, int, int, int>, TcShape> tc_shapes;   // launch shapes by (pass kind, N, K, split)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
   int launches = 0;          // kernels launched by the last ad_generate (direct) or per graph replay
   // Persistent decoder pass (one kernel for the decoder stack + projection): per pass kind, whether it applies and its
@@ -299,11 +266,19 @@ void pass_shapes(const ad_model_cfg& c, PassCfg* pass, int* M_all) {
   for (int k = 0; k < PK_COUNT; ++k) {
     pass[k].M_cap = B * pass[k].seg_max;
     pass[k].ntile = clampi(pow2ceil(pass[k].M_cap), 16, 256);
-    pass[k].max_split = pass[k].M_cap <= 256 ? 16 : 4;
+    pass[k].max_split = 16;
     if (pass[k].M_cap > all) all = pass[k].M_cap;
   }
   if (!c.has_drafter) { /* the drafter pass is never run; keep its shapes for sizing simplicity */ }
   *M_all = all;
+}
+
+// Floats of the partial sums of a projection with d output features over at most M tokens: a split projection has at most one
+// CTA per SM, each with at most 128 x 128 outputs (few-token kernel: at most 16 parts of 128 tokens).
+int num_sms();
+size_t partial_elems(int M, int d) {
+  const size_t all = (size_t)M * d;
+  return std::max(all, std::min(16 * all, std::max((size_t)num_sms() * 128 * 128, (size_t)16 * few::MAX_TOKENS * d)));
 }
 
 size_t layout(ad_handle* h, void* base) {
@@ -315,9 +290,7 @@ size_t layout(ad_handle* h, void* base) {
   const int M_all = h->M_all, Mv = h->pass[PK_VERIFY].M_cap;
   const int M_tmp = std::max(h->pass[PK_DRAFT].M_cap, h->pass[PK_ENCODE].M_cap);
   h->y = (float*)bp.take(sizeof(float) * (size_t)M_all * d);
-  size_t pre_elems = 0;
-  for (int k = 0; k < PK_COUNT; ++k) pre_elems = std::max(pre_elems, (size_t)h->pass[k].max_split * h->pass[k].M_cap * d);
-  h->pre = (float*)bp.take(sizeof(float) * pre_elems);
+  h->pre = (float*)bp.take(sizeof(float) * partial_elems(M_all, d));
   if (h->bf16 && c.n_heads <= 16) h->pre2 = (float*)bp.take(sizeof(float) * (size_t)c.n_heads * M_all * d);
   h->yb.ptr = bp.take(e * (size_t)M_all * d); h->yb.cols = d;
   h->abuf.ptr = bp.take(e * (size_t)M_all * d); h->abuf.cols = d;
@@ -341,7 +314,7 @@ size_t layout(ad_handle* h, void* base) {
     const int Me = h->pass[PK_ENCODE].M_cap;
     ActSet& sd = h->side;
     sd.y = (float*)bp.take(sizeof(float) * (size_t)Me * d);
-    sd.pre = (float*)bp.take(sizeof(float) * (size_t)h->pass[PK_ENCODE].max_split * Me * d);
+    sd.pre = (float*)bp.take(sizeof(float) * partial_elems(Me, d));
     if (h->bf16 && c.n_heads <= 16) sd.pre2 = (float*)bp.take(sizeof(float) * (size_t)c.n_heads * Me * d);
     sd.yb.ptr = bp.take(e * (size_t)Me * d); sd.yb.cols = d;
     sd.abuf.ptr = bp.take(e * (size_t)Me * d); sd.abuf.cols = d;
@@ -490,35 +463,56 @@ int num_sms() {
   return n[dev];
 }
 
-// Ring depth: as deep as ~200 KB of shared memory allows when the grid fits one wave; with more CTAs than SMs,
-// half of that so that two CTAs share an SM: up to twice the SM count the whole grid is then resident at once,
-// beyond that one CTA's prologue and epilogue overlap the other's K loop.
-int tc_stages(int ntile, int kb, int n_ctas) {
-  const int stage = tc::A_STAGE_BYTES + ntile * tc::BLOCK_K * 2;
-  const int budget = n_ctas > num_sms() ? 100 * 1024 : 200 * 1024;
-  int s = clampi(budget / stage, 1, tc::MAX_STAGES);
-  if (s >= kb) return kb > 0 ? kb : 1;
-  // several ring rounds: the kernel's producer count divides the depth, so avoid the prime depths 5 and 7
-  if (s == 5 || s == 7) --s;
-  return s;
+// Launch shape of the tensor-core projection kernel for passes of at most M_cap tokens: the most CTAs any token count asks for
+// and the shared memory of its ring.  Up to one CTA per SM: ~200 KB, so that the ring is as deep as it can be; with more CTAs
+// half of that, so that two CTAs share an SM: up to twice the SM count the whole grid is then resident at once, beyond that
+// one CTA's prologue and epilogue overlap the other's K loop.
+
+TcShape tc_shape(const GeoRule& r, int M_cap, bool exact) {
+  TcShape sh = {1, 0, 0};
+  auto each = [&](auto f) {
+    if (exact) { f(M_cap); return; }
+    for (int M = 1; M <= M_cap; M += M < 2048 ? 1 : 64) f(M);
+    f(M_cap);
+  };
+  each([&](int M) { sh.ctas = std::max(sh.ctas, tc::geometry_ctas(r, M)); });
+  sh.budget = (sh.ctas > num_sms() ? 100 : 200) * 1024;
+  // the ring doubles as the epilogue's transposition buffer (up to 128 rows of 132 floats) and the few-token partial sums
+  each([&](int M) {
+    const Geo g = geometry(r, M);
+    const int need = g.few ? (int)few::red_bytes(2)
+                           : std::max(tc::ring_stages(g.tile, (r.K / tc::BLOCK_K + g.ksplit - 1) / g.ksplit, sh.budget) * (tc::A_STAGE_BYTES + g.tile * tc::BLOCK_K * 2),
+                                      std::min(g.tile, 128) * 132 * 4);
+    sh.smem = std::max(sh.smem, need + 1024);
+  });
+  return sh;
 }
 
-template <int EPI>
-cudaError_t launch_tc(cudaStream_t st, const CUtensorMap& mw, const CUtensorMap& mx, const GemmParams& p, int M_cap) {
+template <int EPI, int NCH>
+cudaError_t launch_tc_n(cudaStream_t st, const CUtensorMap& mw, const tc::TileMaps& mx, const GemmParams& p, const TcShape& sh, const void* w,
+                        const void* x) {
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
   if (!attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(tc::gemm_tc_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 204 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(tc::gemm_tc_kernel<EPI, NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, 204 * 1024);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
-  const int ksplit = (EPI == EPI_F32 && p.ksplit > 1) ? p.ksplit : 1;
-  dim3 grid((p.N + 127) / 128, (M_cap + p.ntile - 1) / p.ntile, ksplit);
-  const int stages = tc_stages(p.ntile, (p.K / tc::BLOCK_K) / ksplit, grid.x * grid.y * grid.z);
-  // the ring doubles as the epilogue's transposition buffer (up to 128 rows of 132 floats)
-  const size_t ring = (size_t)stages * (tc::A_STAGE_BYTES + p.ntile * tc::BLOCK_K * 2);
-  const size_t smem = std::max(ring, (size_t)std::min(p.ntile, 128) * 132 * sizeof(float)) + 1024;
-  return launch_k(tc::gemm_tc_kernel<EPI>, grid, dim3(tc::THREADS), smem, st, mw, mx, p, stages);
+  const int nf = (p.N + tc::BLOCK_N_FEAT - 1) / tc::BLOCK_N_FEAT;
+  return launch_k(tc::gemm_tc_kernel<EPI, NCH>, dim3(nf, (sh.ctas + nf - 1) / nf), dim3(tc::THREADS), sh.smem, st, mw, mx, p, sh.budget, (const bf16*)w, (const bf16*)x);
+}
+template <int EPI>
+cudaError_t launch_tc(cudaStream_t st, const CUtensorMap& mw, const tc::TileMaps& mx, const GemmParams& p, const TcShape& sh, const void* w = nullptr,
+                      const void* x = nullptr) {
+  if (EPI != EPI_ARGMAX && p.rule.few_split > 0) {
+    switch (p.K / p.rule.few_split / 256) {
+      case 1: return launch_tc_n<EPI, EPI == EPI_ARGMAX ? 0 : 1>(st, mw, mx, p, sh, w, x);
+      case 2: return launch_tc_n<EPI, EPI == EPI_ARGMAX ? 0 : 2>(st, mw, mx, p, sh, w, x);
+      case 3: return launch_tc_n<EPI, EPI == EPI_ARGMAX ? 0 : 3>(st, mw, mx, p, sh, w, x);
+      default: return launch_tc_n<EPI, EPI == EPI_ARGMAX ? 0 : 4>(st, mw, mx, p, sh, w, x);
+    }
+  }
+  return launch_tc_n<EPI, 0>(st, mw, mx, p, sh, w, x);
 }
 
 // Projection + arg-max over many tokens: the persistent token-stationary kernel (one CTA per SM, 128-token tiles
@@ -560,11 +554,15 @@ cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmP
     default: return launch_k(few::gemm_few_kernel<EPI, 4, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
   }
 }
-// K split the few-token kernel takes for a projection of pass pc (0: the pass or the shape is not for it).
-int few_split(const PassCfg& pc, int epi, int N, int K) {
-  if (pc.M_cap > kFewTokens || epi == EPI_ARGMAX) return 0;
-  return few::split_for(N, K, epi == EPI_F32, pc.max_split);
+// Geometry rule of a projection of pass pc.  split: its consumer adds partial sums up.
+GeoRule geo_rule(const PassCfg& pc, int epi, int N, int K, bool split, bool has_bias) {
+  GeoRule r = {N, K, pc.ntile, split ? pc.max_split : 1, num_sms(), 0, 0, 0};
+  if (epi == EPI_F32 ? split : (epi != EPI_ARGMAX && has_bias)) r.few_split = few::split_for(N, K, split, pc.max_split);
+  if (r.few_split > 0) r.few_tokens = few::max_tokens(K / r.few_split / 256);
+  return r;
 }
+// Whether every projection of such a shape in pass pc runs on the few-token kernel.
+bool always_few(const PassCfg& pc, const GeoRule& r) { return r.few_split > 0 && pc.M_cap <= r.few_tokens; }
 
 template <int EPI>
 cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const GemmParams& p, int M_cap) {
@@ -579,7 +577,7 @@ cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const Gem
   }
   const int vec = p.K % 4 == 0 && (reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(x)) % 16 == 0;
   const dim3 grid((p.N + FEAT - 1) / FEAT, (M_cap + simt::TOK - 1) / simt::TOK);
-  return launch_k(simt::gemm_f32_kernel<EPI, FEAT>, grid, dim3(2 * FEAT), smem, st, (const float*)w, (const float*)x, p, vec);
+  return launch_k(simt::gemm_f32_kernel<EPI, FEAT>, grid, dim3(simt::GROUPS * FEAT), smem, st, (const float*)w, (const float*)x, p, vec);
 }
 // The few-token FP32 kernel: passes of at most kFewTokens tokens, shapes it covers.
 bool f32_few(const PassCfg& pc, int epi, int N, int K) { return pc.M_cap <= kFewTokens && epi != EPI_ARGMAX && simt::few_fits(N, K); }
@@ -600,7 +598,9 @@ cudaError_t launch_simt_few(cudaStream_t st, const Mat& W, const void* x, const 
 }
 
 // embed_of: the operand is the embedding of pass pk's tokens (first projection of a pass, few-token kernel only).
-int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int* M_ptr, int M_cap, GemmParams p, const Model* embed_of = nullptr) {
+// split: the result is partial sums that the consumer adds up (EPI_F32).
+int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int* M_ptr, int M_cap, GemmParams p, const Model* embed_of = nullptr,
+         bool split = false) {
   p.K = W.K; p.N = W.N; p.M_ptr = M_ptr; p.M_cap = M_cap; p.status = h->st.status;
   cudaError_t e;
   {
@@ -609,35 +609,34 @@ int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int
     snprintf(nm, sizeof(nm), "%s N%d K%d", epi_name[epi & 3], W.N, W.K);
     note_launch(h, nm);
   }
-  // (p.ksplit == 0: the caller wants one full-K result whatever the pass, see ad_debug_logits)
-  const int fs = h->bf16 && (epi != EPI_F32 || p.ksplit > 0) && (epi == EPI_F32 || p.bias) ? few_split(h->pass[pk], epi, W.N, W.K) : 0;
-  if (fs > 0) {
+  PassCfg& pc = h->pass[pk];
+  if (h->bf16) p.rule = geo_rule(pc, epi, W.N, W.K, split, p.bias != nullptr);
+  if (h->bf16 && always_few(pc, p.rule)) {
     switch (epi) {
-      case EPI_F32: e = launch_few<EPI_F32>(h->stream, W, X.ptr, p, fs); break;
-      case EPI_ACT: e = launch_few<EPI_ACT>(h->stream, W, X.ptr, p, fs); break;
+      case EPI_F32: e = launch_few<EPI_F32>(h->stream, W, X.ptr, p, p.rule.few_split); break;
+      case EPI_ACT: e = launch_few<EPI_ACT>(h->stream, W, X.ptr, p, p.rule.few_split); break;
       default:
         if (embed_of) {
-          const few::EmbedParams ep = {(const bf16*)embed_of->emb.ptr, h->pe, sqrtf((float)W.K), h->pass[pk].plan.tok_id, h->pass[pk].plan.tok_pos, h->y};
-          e = launch_few<EPI_SCATTER, true>(h->stream, W, X.ptr, p, fs, ep);
+          const few::EmbedParams ep = {(const bf16*)embed_of->emb.ptr, h->pe, sqrtf((float)W.K), pc.plan.tok_id, pc.plan.tok_pos, h->y};
+          e = launch_few<EPI_SCATTER, true>(h->stream, W, X.ptr, p, p.rule.few_split, ep);
         } else {
-          e = launch_few<EPI_SCATTER>(h->stream, W, X.ptr, p, fs);
+          e = launch_few<EPI_SCATTER>(h->stream, W, X.ptr, p, p.rule.few_split);
         }
         break;
     }
+  } else if (h->bf16 && epi == EPI_ARGMAX && pc.ntile == 256 && vocab_goes_persistent(W.K, W.N, M_cap, p.bias)) {
+    // (a pass with a 256-token tile also has the 128-row map of its token operand)
+    e = launch_vocab_persistent(h->stream, W.map, X.map_for(pk, tc::P_TOK), p, M_cap);
   } else if (h->bf16) {
-    p.ntile = h->pass[pk].tile_for(W.N, num_sms());
-    const CUtensorMap& mx = X.map_for(pk, p.ntile);
-    if (epi != EPI_F32) p.ksplit = 1;
+    const auto key = std::make_tuple(pk, W.N, W.K, split ? 1 : 0);
+    auto it = h->tc_shapes.find(key);
+    if (it == h->tc_shapes.end()) it = h->tc_shapes.emplace(key, tc_shape(p.rule, M_cap, false)).first;
+    const TcShape& sh = it->second;
     switch (epi) {
-      case EPI_F32: e = launch_tc<EPI_F32>(h->stream, W.map, mx, p, M_cap); break;
-      case EPI_ACT: e = launch_tc<EPI_ACT>(h->stream, W.map, mx, p, M_cap); break;
-      case EPI_SCATTER: e = launch_tc<EPI_SCATTER>(h->stream, W.map, mx, p, M_cap); break;
-      default:
-        // (a pass with a 256-token tile also has the 128-row map of its token operand)
-        e = (h->pass[pk].ntile == 256 && vocab_goes_persistent(W.K, W.N, M_cap, p.bias))
-                ? launch_vocab_persistent(h->stream, W.map, X.map_for(pk, tc::P_TOK), p, M_cap)
-                : launch_tc<EPI_ARGMAX>(h->stream, W.map, mx, p, M_cap);
-        break;
+      case EPI_F32: e = launch_tc<EPI_F32>(h->stream, W.map, X.map[pk], p, sh, W.ptr, X.ptr); break;
+      case EPI_ACT: e = launch_tc<EPI_ACT>(h->stream, W.map, X.map[pk], p, sh, W.ptr, X.ptr); break;
+      case EPI_SCATTER: e = launch_tc<EPI_SCATTER>(h->stream, W.map, X.map[pk], p, sh, W.ptr, X.ptr); break;
+      default: e = launch_tc<EPI_ARGMAX>(h->stream, W.map, X.map[pk], p, sh); break;
     }
   } else if (p.M_ptr && f32_few(h->pass[pk], epi, W.N, W.K)) {
     switch (epi) {
@@ -672,12 +671,11 @@ cudaError_t launch_attention(dim3 grid, dim3 block, cudaStream_t st, const AttnP
 
 int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, const void* v, void* out,
               const int* key_base, const int* nkeys_tok, const int* nkeys_row, int max_keys,
-              const float* q_bias = nullptr, int q_nsplit = 0, const Mat* wo = nullptr, bool* fused = nullptr) {
+              const float* q_bias = nullptr, const Partials* q_part = nullptr, const Mat* wo = nullptr, bool* fused = nullptr, bool kv_old = false) {
   const ad_model_cfg& c = h->cfg;
   AttnParams p;
   p.q = q; p.k = k; p.v = v; p.out = out;
-  p.q_part = q_nsplit > 0 ? h->pre : nullptr; p.q_bias = q_bias; p.q_nsplit = q_nsplit;
-  p.q_stride = (size_t)pc.M_cap * c.d_model;
+  p.q_part = q_part ? *q_part : Partials{}; p.M_ptr = pc.plan.M; p.q_bias = q_bias;
   p.seg_off = pc.plan.seg_off; p.seg_len = pc.plan.seg_len;
   p.key_base = key_base; p.nkeys_tok = nkeys_tok; p.nkeys_row = nkeys_row;
   p.d = c.d_model;
@@ -685,45 +683,42 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   const int dh = c.d_model / c.n_heads;
   const bool many = (long long)h->dims.B * c.n_heads * ((pc.seg_max + 7) / 8) > 3LL * num_sms();
   p.scale = 1.0f / sqrtf((float)dh);
-  // Tensor-core kernel when there are thousands of queries or rows may hold hundreds of keys (max_keys: the
-  // capacity, known on the host); the FFMA kernel spreads few queries and few keys over more CTAs.
-  if (h->bf16 && dh == 64 && max_keys >= 256) {
-    // rows may hold hundreds of keys: the keys of a row are spread over the warps of a CTA (whole 64-key tiles per warp),
-    // 1, 2 or 4 query tiles of 16 per CTA depending on how many queries a row can have
-    const int qt = pc.seg_max <= 16 ? 1 : (pc.seg_max <= 32 ? 2 : 4);
-    const int nw = qt == 4 ? 4 : 8;
-    p.qchunks = (pc.seg_max + 16 * qt - 1) / (16 * qt);
-    note_launch(h, "attention_mma_wide");
-    const dim3 mgrid(h->dims.B * p.qchunks, c.n_heads);
-    const size_t smem = (size_t)nw * AM_TILE_BYTES + AM_Q_BYTES;
-    static bool attr_set[kMaxDevices] = {};
-    const int dev = current_device();
-    cudaError_t em = cudaSuccess;
-    if (!attr_set[dev]) {
-      em = cudaFuncSetAttribute(attention_mma_wide_kernel<1, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * AM_TILE_BYTES + AM_Q_BYTES);
-      if (em == cudaSuccess) em = cudaFuncSetAttribute(attention_mma_wide_kernel<2, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * AM_TILE_BYTES + AM_Q_BYTES);
-      if (em == cudaSuccess) em = cudaFuncSetAttribute(attention_mma_wide_kernel<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * AM_TILE_BYTES + AM_Q_BYTES);
-      if (em != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention attribute: ") + cudaGetErrorString(em));
-      attr_set[dev] = true;
-    }
-    if (qt == 1) em = launch_k(attention_mma_wide_kernel<1, 8>, mgrid, dim3(256), smem, h->stream, p);
-    else if (qt == 2) em = launch_k(attention_mma_wide_kernel<2, 8>, mgrid, dim3(512), smem, h->stream, p);
-    else em = launch_k(attention_mma_wide_kernel<4, 4>, mgrid, dim3(512), smem, h->stream, p);
-    if (em != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(em));
-    return AD_OK;
-  }
-  // Tensor-core kernel when there are thousands of queries; the FFMA kernel spreads few queries and few keys over more CTAs.
-  if (h->bf16 && dh == 64 && many) {
-    // rows with few queries: warps share a 16-query tile and split the keys (2 or 4 key groups)
-    const int ng = pc.seg_max <= 16 ? 4 : (pc.seg_max <= 32 ? 2 : 1);
+  // Tensor-core kernels when there are thousands of queries or rows may hold hundreds of keys (max_keys: the capacity, known on
+  // the host); the FFMA kernel spreads few queries and few keys over more CTAs.
+  if (h->bf16 && dh == 64 && (many || max_keys >= 256) && !(max_keys >= 256 && pc.seg_max <= 32)) {
+    // Warps share a 16-query tile and split the keys (2 or 4 key groups) when rows have few queries; two groups also while
+    // 64-query CTAs would not give every SM two.
+    const long full = (long)h->dims.B * ((pc.seg_max + AM_Q - 1) / AM_Q) * c.n_heads;
+    const int ng = pc.seg_max <= 16 ? 4 : (pc.seg_max <= 32 || (full < 2 * num_sms() && max_keys > AM_KT) ? 2 : 1);
     const int qcta = AM_Q / ng;
     p.qchunks = (pc.seg_max + qcta - 1) / qcta;
     note_launch(h, "attention_mma");
     const dim3 mgrid(h->dims.B * p.qchunks, c.n_heads);
-    cudaError_t em;
-    if (ng == 4) em = launch_k(attention_mma_kernel<4>, mgrid, dim3(128), 0, h->stream, p);
-    else if (ng == 2) em = launch_k(attention_mma_kernel<2>, mgrid, dim3(128), 0, h->stream, p);
-    else em = launch_k(attention_mma_kernel<1>, mgrid, dim3(128), 0, h->stream, p);
+    auto* kernel = ng == 4 ? attention_mma_kernel<4> : (ng == 2 ? attention_mma_kernel<2> : attention_mma_kernel<1>);
+    const cudaError_t em = launch_k(kernel, mgrid, dim3(128), 0, h->stream, p, kv_old ? 1 : 0);
+    if (em != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(em));
+    return AD_OK;
+  }
+  if (h->bf16 && dh == 64 && max_keys >= 256) {
+    // few queries per row over hundreds of keys: the keys are spread over the warps of a CTA (whole 64-key tiles per warp), 1 or
+    // 2 query tiles of 16 per CTA
+    const int qt = pc.seg_max <= 16 ? 1 : 2;
+    const int threads = 32 * qt * 8, slots = att_long_slots(max_keys, threads);
+    p.qchunks = (pc.seg_max + 16 * qt - 1) / (16 * qt);
+    note_launch(h, "attention_long");
+    const dim3 mgrid(h->dims.B * p.qchunks, c.n_heads);
+    const size_t smem = att_long_smem(slots, qt);
+    static bool attr_set[kMaxDevices] = {};
+    const int dev = current_device();
+    cudaError_t em = cudaSuccess;
+    if (!attr_set[dev]) {
+      for (auto* kernel : {attention_long_kernel<1, 8>, attention_long_kernel<2, 8>})
+        if (em == cudaSuccess) em = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)att_long_smem(AL_MAX_SLOTS, 2));
+      if (em != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention attribute: ") + cudaGetErrorString(em));
+      attr_set[dev] = true;
+    }
+    auto* kernel = qt == 1 ? attention_long_kernel<1, 8> : attention_long_kernel<2, 8>;
+    em = launch_k(kernel, mgrid, dim3(threads), smem, h->stream, p, slots, kv_old ? 1 : 0);
     if (em != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(em));
     return AD_OK;
   }
@@ -760,13 +755,13 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
 bool attention_is_few(const ad_handle* h, const PassCfg& pc, int max_keys) {
   const ad_model_cfg& c = h->cfg;
   if (!g_fuse_attn_proj || !h->bf16 || !h->pre2 || c.d_model != c.n_heads * 64 || c.d_model % 128 || c.d_model > 128 * few::MAX_WARPS) return false;
-  if (max_keys > 2 * few::AK * few::att_few_warps(c.d_model)) return false;
+  if (max_keys > few::MAX_ROUNDS * few::AK * few::att_few_warps(c.d_model)) return false;
   return (long)h->cfg.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * few::att_few_split(c.d_model) <= num_sms();
 }
 
 // Attention with its output projection (partial sums per head in pre2) and, with wq, the query projection of x = yb.
 int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v, const int* key_base, const int* nkeys_tok,
-                  const int* nkeys_row, const Mat& wo, const Mat* wq = nullptr, const float* q_bias = nullptr) {
+                  const int* nkeys_row, int max_keys, const Mat& wo, const Mat* wq = nullptr, const float* q_bias = nullptr) {
   const ad_model_cfg& c = h->cfg;
   few::FewAttnParams fp = {};
   AttnParams& p = fp.a;
@@ -782,7 +777,7 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   const int dev = current_device();
   cudaError_t e = cudaSuccess;
   if (!attr_set[dev]) {
-    const int most = (int)few::att_few_smem(few::MAX_WARPS);
+    const int most = (int)few::att_few_smem(few::MAX_WARPS, few::MAX_ROUNDS);
     for (auto* kernel : {few::attention_few_kernel<false, 1>, few::attention_few_kernel<true, 1>, few::attention_few_kernel<false, 2>,
                          few::attention_few_kernel<true, 2>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
@@ -792,7 +787,8 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   note_launch(h, wq ? "q_proj+attention+out_proj" : "attention+out_proj");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(h->dims.B * p.qchunks * split, c.n_heads); cfg.blockDim = dim3(32 * warps);
-  cfg.dynamicSmemBytes = few::att_few_smem(warps); cfg.stream = h->stream;
+  fp.rounds = max_keys > few::AK * warps ? 2 : 1;
+  cfg.dynamicSmemBytes = few::att_few_smem(warps, fp.rounds); cfg.stream = h->stream;
   cudaLaunchAttribute attr[2];
   int n_attr = 0;
   if (g_use_pdl) {
@@ -811,42 +807,39 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   return AD_OK;
 }
 
-// y = LN(sum of the nsplit partial projections in `pre` + bias + y)
-int layernorm(ad_handle* h, const PassCfg& pc, int nsplit, const float* bias, const float* g, const float* b,
-              const float* partials = nullptr) {
-  const float* pre_src = partials ? partials : h->pre;
+// y = LN(sum of the partial projections + bias + y)
+int layernorm(ad_handle* h, const PassCfg& pc, const Partials& pre, const float* bias, const float* g, const float* b) {
   const int d = h->cfg.d_model;
-  dim3 grid(pc.M_cap);
-  const size_t stride = (size_t)pc.M_cap * d;
+  const LnParams p = {pc.plan.M, pre, bias, h->y, g, b, d, h->cfg.ln_eps, h->y};
   note_launch(h, "residual+layernorm");
-  cudaError_t e;
-  // many tokens: a warp per token (measured: 1024 tokens 458 us per step with a CTA per token against 467 us, 2048 tokens 582 against 543 us)
-  if (pc.M_cap >= 1536 && nsplit <= 4 && d % 128 == 0 && d <= 1024) {
-    dim3 rgrid((pc.M_cap + 7) / 8);
-    if (h->bf16) e = launch_k(layernorm_rows_kernel<bf16>, rgrid, dim3(256), 0, h->stream, (const int*)pc.plan.M, pre_src, nsplit, stride, bias,
-                              (const float*)h->y, g, b, d, h->cfg.ln_eps, h->y, (bf16*)h->yb.ptr);
-    else e = launch_k(layernorm_rows_kernel<float>, rgrid, dim3(256), 0, h->stream, (const int*)pc.plan.M, pre_src, nsplit, stride, bias,
-                      (const float*)h->y, g, b, d, h->cfg.ln_eps, h->y, (float*)h->yb.ptr);
-  } else if (h->bf16 && d > 512) e = launch_k(layernorm_kernel<bf16, 256>, grid, dim3(256), 0, h->stream, (const int*)pc.plan.M, pre_src, nsplit, stride, bias,
-                            (const float*)h->y, g, b, d, h->cfg.ln_eps, h->y, (bf16*)h->yb.ptr);
-  else if (h->bf16) e = launch_k(layernorm_kernel<bf16>, grid, dim3(128), 0, h->stream, (const int*)pc.plan.M, pre_src, nsplit, stride, bias,
-                            (const float*)h->y, g, b, d, h->cfg.ln_eps, h->y, (bf16*)h->yb.ptr);
-  else e = launch_k(layernorm_kernel<float>, grid, dim3(128), 0, h->stream, (const int*)pc.plan.M, pre_src, nsplit, stride, bias,
-                    (const float*)h->y, g, b, d, h->cfg.ln_eps, h->y, (float*)h->yb.ptr);
+  auto go = [&](auto* yb) -> cudaError_t {
+    using ActT = std::remove_pointer_t<decltype(yb)>;
+    if (pc.M_cap >= LN_ROWS && d % 128 == 0)
+      return launch_k(layernorm_many_kernel<ActT>, dim3(std::min(2 * num_sms(), (pc.M_cap + 1) / 2)), dim3(256), 0, h->stream, p, yb);
+    if (d > 512) return launch_k(layernorm_kernel<ActT, 256>, dim3(pc.M_cap), dim3(256), 0, h->stream, p, yb);
+    return launch_k(layernorm_kernel<ActT, 128>, dim3(pc.M_cap), dim3(128), 0, h->stream, p, yb);
+  };
+  const cudaError_t e = h->bf16 ? go((bf16*)h->yb.ptr) : go((float*)h->yb.ptr);
   if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("layernorm launch: ") + cudaGetErrorString(e));
   return AD_OK;
 }
+// Partial output projections of the attention kernels that carry it: one per head.
+Partials head_partials(const ad_handle* h, const PassCfg& pc) {
+  Partials q = {};
+  q.ptr = h->pre2; q.nsplit = h->cfg.n_heads; q.stride = (size_t)pc.M_cap * h->cfg.d_model;
+  return q;
+}
 
-// Projection whose consumer is the residual + LayerNorm kernel: written as split-K partial sums, bias left to
-// the consumer.  Returns the number of partials through *nsplit.
-int gemm_to_ln(ad_handle* h, const Mat& W, const ActBuf& X, int pk, int* nsplit) {
+// Projection whose consumer adds partial sums up (residual + LayerNorm, or the attention's queries); bias left to it.
+int gemm_to_partials(ad_handle* h, const Mat& W, const ActBuf& X, int pk, Partials* out) {
   PassCfg& pc = h->pass[pk];
   GemmParams o = {};
   o.out_f32 = h->pre;
-  o.ksplit = h->bf16 ? few_split(pc, EPI_F32, W.N, W.K) : 1;
-  if (o.ksplit == 0) o.ksplit = pc.ksplit_for(W.N, W.K, pc.tile_for(W.N, num_sms()));
-  *nsplit = o.ksplit;
-  return gemm(h, EPI_F32, W, X, pk, pc.plan.M, pc.M_cap, o);
+  *out = Partials{};
+  out->ptr = h->pre;
+  if (h->bf16) out->rule = geo_rule(pc, EPI_F32, W.N, W.K, true, false);
+  else out->nsplit = 1;
+  return gemm(h, EPI_F32, W, X, pk, pc.plan.M, pc.M_cap, o, nullptr, true);
 }
 
 int embed(ad_handle* h, const PassCfg& pc, const Model& m) {
@@ -864,7 +857,7 @@ int embed(ad_handle* h, const PassCfg& pc, const Model& m) {
 
 // Embedding of a pass's tokens: a kernel of its own, unless the pass's first projection computes it (null: it is done).
 int embed_or_defer(ad_handle* h, int pk, const Model& m, const Mat& first, const Model** deferred) {
-  *deferred = h->bf16 && few_split(h->pass[pk], EPI_SCATTER, first.N, first.K) > 0 ? &m : nullptr;
+  *deferred = h->bf16 && always_few(h->pass[pk], geo_rule(h->pass[pk], EPI_SCATTER, first.N, first.K, false, true)) ? &m : nullptr;
   return *deferred ? AD_OK : embed(h, h->pass[pk], m);
 }
 
@@ -879,14 +872,14 @@ int self_attention_sublayer(ad_handle* h, int pk, const Mat& wqkv, const float* 
   bool fused = false;
   const int max_keys = pk == PK_VERIFY ? h->dims.max_tgt : pc.seg_max;
   if (attention_is_few(h, pc, max_keys)) {
-    AD_TRY(attention_few(h, pc, kbuf, vbuf, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, wo));
-    return layernorm(h, pc, h->cfg.n_heads, bo, lng, lnb, h->pre2);
+    AD_TRY(attention_few(h, pc, kbuf, vbuf, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, max_keys, wo));
+    return layernorm(h, pc, head_partials(h, pc), bo, lng, lnb);
   }
-  AD_TRY(attention(h, pc, h->qbuf, kbuf, vbuf, h->abuf.ptr, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, max_keys, nullptr, 0, &wo, &fused));
-  if (fused) return layernorm(h, pc, h->cfg.n_heads, bo, lng, lnb, h->pre2);
-  int ns = 1;
-  AD_TRY(gemm_to_ln(h, wo, h->abuf, pk, &ns));
-  return layernorm(h, pc, ns, bo, lng, lnb);
+  AD_TRY(attention(h, pc, h->qbuf, kbuf, vbuf, h->abuf.ptr, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, max_keys, nullptr, nullptr, &wo, &fused));
+  if (fused) return layernorm(h, pc, head_partials(h, pc), bo, lng, lnb);
+  Partials ps;
+  AD_TRY(gemm_to_partials(h, wo, h->abuf, pk, &ps));
+  return layernorm(h, pc, ps, bo, lng, lnb);
 }
 
 int ffn_sublayer(ad_handle* h, int pk, const Mat& w1, const float* b1, const Mat& w2, const float* b2, const float* lng,
@@ -895,9 +888,9 @@ int ffn_sublayer(ad_handle* h, int pk, const Mat& w1, const float* b1, const Mat
   GemmParams a = {};
   a.bias = b1; a.relu = 1; a.out_act = h->hbuf.ptr;
   AD_TRY(gemm(h, EPI_ACT, w1, h->yb, pk, pc.plan.M, pc.M_cap, a));
-  int ns = 1;
-  AD_TRY(gemm_to_ln(h, w2, h->hbuf, pk, &ns));
-  return layernorm(h, pc, ns, b2, lng, lnb);
+  Partials ps;
+  AD_TRY(gemm_to_partials(h, w2, h->hbuf, pk, &ps));
+  return layernorm(h, pc, ps, b2, lng, lnb);
 }
 
 
@@ -1048,31 +1041,30 @@ int decoder_pass(ad_handle* h, int pk, Model& m) {
     // loads its queries.
     bool fused_x = false;
     if (attention_is_few(h, pc, c.max_src)) {
-      AD_TRY(attention_few(h, pc, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->st.cross_base, nullptr, h->st.srclen,
+      AD_TRY(attention_few(h, pc, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->st.cross_base, nullptr, h->st.srclen, c.max_src,
                            L.co, &L.cq, L.cbq));
-      AD_TRY(layernorm(h, pc, c.n_heads, L.cbo, L.ln2g, L.ln2b, h->pre2));
+      AD_TRY(layernorm(h, pc, head_partials(h, pc), L.cbo, L.ln2g, L.ln2b));
       AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b));
       continue;
     }
-    int qs = h->bf16 && pc.M_cap <= 256 ? pc.ksplit_for(L.cq.N, L.cq.K, pc.tile_for(L.cq.N, num_sms())) : 1;
-    if (qs > 1 && qs <= ATT_MAX_QSPLIT) {
-      int ns_q = 1;
-      AD_TRY(gemm_to_ln(h, L.cq, h->yb, pk, &ns_q));
+    if (h->bf16 && pc.M_cap <= 256) {
+      Partials qp;
+      AD_TRY(gemm_to_partials(h, L.cq, h->yb, pk, &qp));
       AD_TRY(attention(h, pc, nullptr, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->abuf.ptr,
-                       h->st.cross_base, nullptr, h->st.srclen, c.max_src, L.cbq, ns_q, &L.co, &fused_x));
+                       h->st.cross_base, nullptr, h->st.srclen, c.max_src, L.cbq, &qp, &L.co, &fused_x, true));
     } else {
       GemmParams q = {};
       q.bias = L.cbq; q.out_act = h->qbuf;
       AD_TRY(gemm(h, EPI_ACT, L.cq, h->yb, pk, pc.plan.M, pc.M_cap, q));
       AD_TRY(attention(h, pc, h->qbuf, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->abuf.ptr,
-                       h->st.cross_base, nullptr, h->st.srclen, c.max_src, nullptr, 0, &L.co, &fused_x));
+                       h->st.cross_base, nullptr, h->st.srclen, c.max_src, nullptr, nullptr, &L.co, &fused_x, true));
     }
     if (fused_x) {
-      AD_TRY(layernorm(h, pc, c.n_heads, L.cbo, L.ln2g, L.ln2b, h->pre2));
+      AD_TRY(layernorm(h, pc, head_partials(h, pc), L.cbo, L.ln2g, L.ln2b));
     } else {
-      int ns = 1;
-      AD_TRY(gemm_to_ln(h, L.co, h->abuf, pk, &ns));
-      AD_TRY(layernorm(h, pc, ns, L.cbo, L.ln2g, L.ln2b));
+      Partials ps;
+      AD_TRY(gemm_to_partials(h, L.co, h->abuf, pk, &ps));
+      AD_TRY(layernorm(h, pc, ps, L.cbo, L.ln2g, L.ln2b));
     }
     AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b));
   }
@@ -1203,11 +1195,9 @@ int loop_iteration(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_l
   struct Scope {               // whatever way this function is left
     ad_handle* h;
     ~Scope() {
-      h->pass[PK_VERIFY].shrinking = false;
       h->next_pass = no_next_pass();
     }
   } scope{h};
-  h->pass[PK_VERIFY].shrinking = o.mode == AD_MODE_IAD;
   if (!loop_plans_ahead(h)) {
     if (loop_drafts(o)) {
       AD_TRY(plan_draft(h, o.k));
@@ -1314,13 +1304,13 @@ extern "C" int ad_create(const ad_model_cfg* cfg, const ad_weights* w, void* wor
     for (ActBuf* b : bufs)
       for (int k = 0; k < PK_COUNT; ++k)
         for (int i = 0; i < 5 && (16 << i) <= h->pass[k].ntile; ++i)
-          ok = ok && make_map(&b->map[k][i], b->ptr, h->M_all, b->cols, 16 << i);
+          ok = ok && make_map(&b->map[k].m[i], b->ptr, h->M_all, b->cols, 16 << i);
     if (cfg->has_drafter) {
       const int Me = h->pass[PK_ENCODE].M_cap, nt = h->pass[PK_ENCODE].ntile;
       ActBuf* sbufs[3] = {&h->side.yb, &h->side.abuf, &h->side.hbuf};
       for (ActBuf* b : sbufs)
         for (int i = 0; i < 5 && (16 << i) <= nt; ++i)
-          ok = ok && make_map(&b->map[PK_ENCODE][i], b->ptr, Me, b->cols, 16 << i);
+          ok = ok && make_map(&b->map[PK_ENCODE].m[i], b->ptr, Me, b->cols, 16 << i);
     }
     if (!ok) return bail(AD_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
   }
@@ -1925,22 +1915,64 @@ extern "C" size_t ad_vocab_argmax_scratch_bytes(int32_t vocab, int32_t M) {
 
 namespace {
 
-// Arg-max over tiles for M rows without any decoding state.  grid = M, block = 32.
-__global__ void argmax_rows_kernel(const float* __restrict__ part_val, const int* __restrict__ part_idx, int n_tiles,
-                                   int M_cap, int* __restrict__ out) {
-  const int m = blockIdx.x, lane = threadIdx.x;
+// Arg-max over tiles for M rows without any decoding state: four rows per CTA, a warp each (few rows: one row per CTA, whose
+// warps share its tiles), up to eight tiles per lane in flight.  grid = ceil(M / rows), block = 128.
+__global__ void __launch_bounds__(128)
+argmax_rows_kernel(const float* __restrict__ part_val, const int* __restrict__ part_idx, int n_tiles, int M, int rows, int* __restrict__ out) {
+  __shared__ float s_v[4];
+  __shared__ int s_i[4];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int m = rows == 1 ? blockIdx.x : blockIdx.x * 4 + warp;
+  const int first = rows == 1 ? threadIdx.x : lane, step = rows == 1 ? 128 : 32;
   float v = -INFINITY;
   int idx = 0x7fffffff;
+  pdl_launch();
   pdl_wait();   // the partials come from the kernel before this one
-  for (int t = lane; t < n_tiles; t += 32) {
-    const float ov = part_val[(size_t)m * n_tiles + t];
-    const int oi = part_idx[(size_t)m * n_tiles + t];
-    if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
+  if (m < M) {
+    for (int t0 = 0; t0 < n_tiles; t0 += 8 * step) {
+      float pv[8];
+      int pi[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int t = t0 + u * step + first;
+        pv[u] = t < n_tiles ? part_val[(size_t)m * n_tiles + t] : -INFINITY;
+        pi[u] = t < n_tiles ? part_idx[(size_t)m * n_tiles + t] : 0x7fffffff;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (pv[u] > v || (pv[u] == v && pi[u] < idx)) { v = pv[u]; idx = pi[u]; }
+    }
+    tc::warp_argmax(v, idx);
+    if (rows > 1 && lane == 0) out[m] = idx;
   }
-  tc::warp_argmax(v, idx);
-  if (lane == 0) out[m] = idx;
+  if (rows == 1) {
+    if (lane == 0) { s_v[warp] = v; s_i[warp] = idx; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 4; ++w)
+        if (s_v[w] > v || (s_v[w] == v && s_i[w] < idx)) { v = s_v[w]; idx = s_i[w]; }
+      out[m] = idx;
+    }
+  }
 }
 
+}  // namespace
+
+namespace {
+// Token tile of an operator-level call: by the passes' rule.
+int op_tile(const GeoRule& r, int M) { 
+  static const int force = [] { const char* e = getenv("AD_OP_TILE"); return e ? atoi(e) : 0; }();
+  if (force) return std::min(force, r.max_tile);
+  return geometry(r, M).tile; }
+// Geometry of an operator-level call over M tokens, and the token operand's map for its tile.
+bool op_maps(GemmParams* p, tc::TileMaps* mx, const void* x, int M, int K) {
+  p->rule = GeoRule{p->N, K, clampi(pow2ceil(M), 16, 256), 1, num_sms(), 0, 0, 0};
+  const int tile = p->rule.fixed_tile = op_tile(p->rule, M);
+  int i = 0;
+  while ((16 << i) < tile) ++i;
+  memset(mx, 0, sizeof(*mx));
+  return make_map(&mx->m[i], x, M, K, tile);
+}
 }  // namespace
 
 extern "C" int ad_vocab_argmax(const void* x, const void* emb, int32_t dtype, int32_t M, int32_t d, int32_t vocab,
@@ -1957,15 +1989,16 @@ extern "C" int ad_vocab_argmax(const void* x, const void* emb, int32_t dtype, in
   cudaError_t e;
   if (dtype == AD_DTYPE_BF16) {
     if (d % 64 || M > kMaxOpTokens) return AD_ERR_ARG;
-    CUtensorMap mw, mx;
-    p.ntile = clampi(pow2ceil(M), 16, 256);
-    if (!make_map(&mw, emb, vocab, d, tc::BLOCK_N_FEAT) || !make_map(&mx, x, M, d, p.ntile)) return AD_ERR_CUDA;
+    CUtensorMap mw;
+    if (!make_map(&mw, emb, vocab, d, tc::BLOCK_N_FEAT)) return AD_ERR_CUDA;
     if (vocab_goes_persistent(d, vocab, M, nullptr)) {
       CUtensorMap mx128;
       if (!make_map(&mx128, x, M, d, tc::P_TOK)) return AD_ERR_CUDA;
       e = launch_vocab_persistent(st, mw, mx128, p, M);
     } else {
-      e = launch_tc<EPI_ARGMAX>(st, mw, mx, p, M);
+      tc::TileMaps mx;
+      if (!op_maps(&p, &mx, x, M, d)) return AD_ERR_CUDA;
+      e = launch_tc<EPI_ARGMAX>(st, mw, mx, p, tc_shape(p.rule, M, true));
     }
   } else if (dtype == AD_DTYPE_FP32) {
     e = launch_simt<EPI_ARGMAX>(st, emb, x, p, M);
@@ -1974,7 +2007,8 @@ extern "C" int ad_vocab_argmax(const void* x, const void* emb, int32_t dtype, in
   }
   if (e != cudaSuccess) return AD_ERR_CUDA;
   if (!argmax) return AD_OK;   // projection kernel alone: partials stay in scratch
-  e = launch_k(argmax_rows_kernel, dim3(M), dim3(32), 0, st, (const float*)pv, (const int*)pi, tiles, M, argmax);
+  const int rows = M <= num_sms() ? 1 : 4;
+  e = launch_k(argmax_rows_kernel, dim3((M + rows - 1) / rows), dim3(128), 0, st, (const float*)pv, (const int*)pi, tiles, M, rows, argmax);
   return e == cudaSuccess ? AD_OK : AD_ERR_CUDA;
 }
 
@@ -1987,10 +2021,10 @@ extern "C" int ad_linear(const void* x, const void* W, const float* bias, int32_
   cudaError_t e;
   if (dtype == AD_DTYPE_BF16) {
     if (K % 64 || M > kMaxOpTokens) return AD_ERR_ARG;
-    CUtensorMap mw, mx;
-    p.ntile = clampi(pow2ceil(M), 16, 256);
-    if (!make_map(&mw, W, N, K, tc::BLOCK_N_FEAT) || !make_map(&mx, x, M, K, p.ntile)) return AD_ERR_CUDA;
-    e = launch_tc<EPI_F32>(st, mw, mx, p, M);
+    CUtensorMap mw;
+    tc::TileMaps mx;
+    if (!make_map(&mw, W, N, K, tc::BLOCK_N_FEAT) || !op_maps(&p, &mx, x, M, K)) return AD_ERR_CUDA;
+    e = launch_tc<EPI_F32>(st, mw, mx, p, tc_shape(p.rule, M, true));
   } else if (dtype == AD_DTYPE_FP32) {
     e = launch_simt<EPI_F32>(st, W, x, p, M);
   } else {

@@ -50,18 +50,81 @@ enum Epi : int {
   EPI_ARGMAX = 3    // per (feature tile, token) running (max, lowest id) partials
 };
 
+// Launch geometry of the tensor-core projection kernel (gemm_tc.cuh) for M packed tokens: token tile and K split.  Evaluated
+// on the device from the M the plan holds, by the projection and by whoever adds its partial sums up, so that a pass always
+// runs at the geometry of the tokens it has, not at that of its capacity.
+//
+// Token tile: up to 64 tokens one tile; beyond that the kernels are latency-bound and smaller tiles win -- more CTAs, more MMA
+// issuers per CTA, a shorter epilogue each -- until the grids outgrow the SMs.  Measured per step (base model):
+//   100 / 120 / 128 tokens: 64-token tiles 277 / 289 / 293 us against 305 / 316 / 321 us with one 128-token tile;
+//   200 / 240 tokens: 32-token tiles 331 / 305 us, 64: 344 / 311, 128: 364 / 336, 16: 372;
+//   320 / 400 / 512 tokens: 64-token tiles 366 / 357 / 389 us against 415 / 410 / 458 (128) and 383 / 380 / 410 (32);
+//   800 / 1024 tokens: 64-token tiles 455 / 468 us against 477 / 486 (128);  2048 tokens: 128-token tiles 543 us, 64: 571;
+//   256-token tiles once they alone give two CTAs per SM.
+// A projection whose feature tiles alone outnumber the SMs (the vocabulary) is bound by its weights: one token tile as long as
+// there is one, so that they are read once (90 tokens x 50265 x 768: 19.5 us with two 64-token tiles).
+// K split (projections whose consumer adds partial sums up): as many CTAs as there are SMs at most, 112 for a single token tile
+// (the big model's 25-token pass lost 4 % with 128 one-K-block CTAs).
+struct GeoRule {
+  int N, K;
+  int max_tile;      // largest token tile that has a tensor map
+  int max_split;     // 1: no split
+  int sms;
+  int few_split;     // > 0: passes of at most few_tokens tokens run on the few-token kernel (gemm_few.cuh) with this K split
+  int few_tokens;
+  int fixed_tile;    // > 0: M is known on the host, which evaluated the rule already (operator-level calls); no split
+};
+struct Geo {
+  int tile, ksplit;
+  bool few;
+};
+__host__ __device__ inline Geo geometry(const GeoRule& r, int M) {
+  Geo g;
+  g.few = r.few_split > 0 && M <= r.few_tokens;
+  if (r.fixed_tile > 0) { g.tile = r.fixed_tile; g.ksplit = 1; return g; }
+  if (g.few) { g.tile = 0; g.ksplit = r.few_split; return g; }
+  const int nf = (r.N + 127) / 128;
+  if (M <= 64) {
+    g.tile = 16;
+    while (g.tile < M) g.tile *= 2;
+  } else if (M <= 128) {
+    g.tile = nf >= r.sms ? 128 : 64;
+  } else if (M <= 256) {
+    g.tile = 32;
+  } else if (M <= 1024) {
+    g.tile = 64;
+  } else {
+    g.tile = nf * ((M + 255) / 256) >= 2 * r.sms ? 256 : 128;
+  }
+  if (g.tile > r.max_tile) g.tile = r.max_tile;
+  const int tiles = nf * ((M + g.tile - 1) / g.tile), kb = r.K / 64, cap = M <= 64 ? 112 : r.sms;
+  g.ksplit = 1;
+  while (g.ksplit * 2 <= r.max_split && tiles * g.ksplit * 2 <= cap && kb % (g.ksplit * 2) == 0) g.ksplit *= 2;
+  return g;
+}
+// Partial sums [nsplit][.., N] of a projection: how many there are and how far apart, for whoever adds them up.
+struct Partials {
+  const float* ptr;
+  int nsplit;        // > 0: fixed, `stride` floats apart; 0: by rule and the pass's token count M, M * N floats apart
+  size_t stride;
+  GeoRule rule;
+};
+__device__ __forceinline__ void resolve_partials(const Partials& q, int M, int& nsplit, size_t& stride) {
+  nsplit = q.nsplit > 0 ? q.nsplit : geometry(q.rule, M).ksplit;
+  stride = q.nsplit > 0 ? q.stride : (size_t)M * q.rule.N;
+}
+
 struct GemmParams {
   int K;                 // contraction length
   int N;                 // output features (rows of W)
-  int ntile;             // tokens per CTA tile
   const int* M_ptr;      // device scalar: number of valid packed tokens (null: use M_host)
   int M_host;
   int M_cap;             // capacity of the token dimension of the buffers
   const float* bias;     // [N] or null
   int relu;
-  int ksplit;            // EPI_F32 only: blockIdx.z takes K range z/ksplit and writes partial z (1 = no split)
+  GeoRule rule;          // launch geometry of the tensor-core kernel
   // EPI_F32
-  float* out_f32;        // [ksplit][M_cap, N]: partial sums; the consumer adds them up
+  float* out_f32;        // [ksplit][M, N]: partial sums; the consumer adds them up
   // EPI_ACT
   void* out_act;         // [M_cap, N] float or bf16
   // EPI_SCATTER

@@ -16,11 +16,10 @@ namespace ad {
 struct AttnParams {
   const void* q;         // [M_cap, d]
   // When q_part is set the queries come straight from the split-K partial sums of their projection instead:
-  // q = round_to_activation_type(sum over q_nsplit partials [M_cap, d], q_stride elements apart, + q_bias).
-  const float* q_part;
+  // q = round_to_activation_type(sum over the partials + q_bias).
+  Partials q_part;       // (ptr null: queries in q)
+  const int* M_ptr;
   const float* q_bias;   // [d] or null
-  int q_nsplit;
-  size_t q_stride;
   const void* k;         // [slots, d]
   const void* v;         // [slots, d]
   void* out;             // [M_cap, d]
@@ -150,6 +149,9 @@ attention_kernel(const AttnParams p) {
   const int row_nk = plan_load(p.nkeys_row + b);   // no token of this row sees more keys than this
   const int i0 = chunk * QC;
   if (i0 >= seg_len && (blockIdx.x | blockIdx.y) != 0) return;
+  int q_nsplit = 0;
+  size_t q_stride = 0;
+  if (p.q_part.ptr) resolve_partials(p.q_part, plan_load(p.M_ptr), q_nsplit, q_stride);
   pdl_wait();
   trace_mark(TR_ATTN, 1);
   if (i0 >= seg_len) return;
@@ -191,11 +193,11 @@ attention_kernel(const AttnParams p) {
         const int col = h * DH + lane + 32 * rr;
         const size_t off = (size_t)(m0 + r) * d + col;
         float qv;
-        if (p.q_part) {
+        if (p.q_part.ptr) {
           qv = p.q_bias ? p.q_bias[col] : 0.f;
           float part[ATT_MAX_QSPLIT];                  // all partials in one round trip
 #pragma unroll
-          for (int sp = 0; sp < ATT_MAX_QSPLIT; ++sp) part[sp] = sp < p.q_nsplit ? p.q_part[sp * p.q_stride + off] : 0.f;
+          for (int sp = 0; sp < ATT_MAX_QSPLIT; ++sp) part[sp] = sp < q_nsplit ? p.q_part.ptr[sp * q_stride + off] : 0.f;
 #pragma unroll
           for (int sp = 0; sp < ATT_MAX_QSPLIT; ++sp) qv += part[sp];
           qv = to_f32(from_f32<ActT>(qv));     // the value a stored query would have had

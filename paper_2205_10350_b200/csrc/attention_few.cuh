@@ -37,10 +37,12 @@ struct FewAttnParams {
   AttnParams a;
   const bf16* x;        // query projection: its input [M_cap, d] (normalised hidden states) ...
   const bf16* wq;       // ... and weights [d, d]; null: the queries are in a.q
+  int rounds;           // rounds of keys the capacity may need
 };
 
-inline size_t att_few_smem(int warps) {
-  const size_t kv = (size_t)warps * AK * (K_LD + V_LD) * sizeof(bf16);
+constexpr int MAX_ROUNDS = 2;     // rounds of AK keys per warp: all resident at once
+inline size_t att_few_smem(int warps, int rounds) {
+  const size_t kv = (size_t)rounds * warps * AK * (K_LD + V_LD) * sizeof(bf16);
   const size_t part = (size_t)warps * AQ * O_LD * sizeof(float);      // partial query projections, later partial outputs
   return kv + part + 2 * (size_t)warps * AQ * sizeof(float) + 2 * (size_t)AQ * K_LD * sizeof(bf16) + 2 * (size_t)AQ * 64 * sizeof(float);
 }
@@ -87,7 +89,8 @@ attention_few_kernel(const FewAttnParams fp) {
   }
   bf16* ks = reinterpret_cast<bf16*>(few_smem) + (size_t)warp * AK * (K_LD + V_LD);   // this warp's keys of a round ...
   bf16* vs = ks + AK * K_LD;                                                          // ... and values
-  float* part = reinterpret_cast<float*>(few_smem + (size_t)nw * AK * (K_LD + V_LD) * sizeof(bf16));   // [nw][16][O_LD]
+  const int round_stride = nw * AK * (K_LD + V_LD);                                   // elements from one round to the next
+  float* part = reinterpret_cast<float*>(few_smem + (size_t)fp.rounds * round_stride * sizeof(bf16));   // [nw][16][O_LD]
   float* pm = part + (size_t)nw * AQ * O_LD;                                          // [nw][16] maxima
   float* pl = pm + nw * AQ;                                                           // [nw][16] sums
   bf16* qs = reinterpret_cast<bf16*>(pl + nw * AQ);                                   // [16][K_LD] queries
@@ -121,25 +124,26 @@ attention_few_kernel(const FewAttnParams fp) {
   }
   const bf16* kk = reinterpret_cast<const bf16*>(p.k);
   const bf16* vv = reinterpret_cast<const bf16*>(p.v);
-  // this warp's 16 keys of a round, 64 elements each: 128 16-byte pieces, four per lane, for keys and values each
-  auto fetch = [&](int first) {
-    const int key0 = first + warp * AK;
-    if (key0 < row_nk) {
+  // this warp's 16 keys of every round, 64 elements each: 128 16-byte pieces, four per lane, for keys and values each
+  auto fetch = [&]() {
+    for (int r = 0; r < fp.rounds; ++r) {
+      const int key0 = (r * nw + warp) * AK;
+      if (key0 >= row_nk) break;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int idx = lane + 32 * i, j = idx >> 3, c = (idx & 7) * 8;
         const bool there = key0 + j < row_nk;
         const size_t off = (size_t)(kbase + (there ? key0 + j : 0)) * d + h * 64 + c;
-        cp16(ks + j * K_LD + c, kk + off, there);
-        cp16(vs + j * V_LD + c, vv + off, there);
+        cp16(ks + r * round_stride + j * K_LD + c, kk + off, there);
+        cp16(vs + r * round_stride + j * V_LD + c, vv + off, there);
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  if (QPROJ) fetch(0);          // the encoder's keys and values: older than the plan
+  if (QPROJ) fetch();          // the encoder's keys and values: older than the plan
   pdl_wait();
   trace_mark(TR_ATTN, 1);
-  if (!QPROJ) fetch(0);
+  if (!QPROJ) fetch();
 
   uint4 qa[2][2];               // query fragments: [32-wide chunk of the head][row g / g + 8]
   if (QPROJ) {
@@ -223,12 +227,9 @@ attention_few_kernel(const FewAttnParams fp) {
 #pragma unroll
   for (int j = 0; j < 8; ++j) { o[j][0] = 0.f; o[j][1] = 0.f; o[j][2] = 0.f; o[j][3] = 0.f; }
   float mx0 = -INFINITY, mx1 = -INFINITY, den0 = 0.f, den1 = 0.f;      // den: this lane's share of the row sums
-  for (int first = 0; first < row_nk; first += AK * nw) {
-    if (first > 0) { __syncwarp(); fetch(first); }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncwarp();
-    const int key0 = first + warp * AK;
-    if (key0 >= row_nk) break;                                         // warp-uniform; later rounds lie further out still
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
+  for (int key0 = warp * AK; key0 < row_nk; key0 += AK * nw, ks += round_stride, vs += round_stride) {
     float s[2][4];
 #pragma unroll
     for (int n = 0; n < 2; ++n) { s[n][0] = 0.f; s[n][1] = 0.f; s[n][2] = 0.f; s[n][3] = 0.f; }

@@ -1,13 +1,12 @@
-// Attention for many queries on the tensor cores (BF16, head dimension 64).
+// Attention for many queries, or over hundreds of keys, on the tensor cores (BF16, head dimension 64).
 //
-// Same operation and masking rules as attention_kernel (attention.cuh); used when a pass has thousands of
-// queries, where the FFMA kernel is bound by its multiply-adds.  The tiles of one (row, head) pair are small
-// (at most 64 queries x 64 keys x 64 dims per step), far below the 128-row atoms of the tcgen05 path and not
-// worth a round trip through tensor memory, so the products run as warp-level m16n8k16 MMAs on register
-// fragments: S = Q K^T, online softmax on the accumulator fragments, P (rounded to BF16) reused in place as
-// the A operand of O += P V, with V read through transposing ldmatrix loads.
-//
-// grid = (B * qchunks, H), qchunks = ceil(longest segment / queries per CTA); block = 128 threads.
+// Same operation and masking rules as attention_kernel (attention.cuh).  The tiles of one (row, head) pair are small (at most
+// 64 queries x 64 keys x 64 dims per step), far below the 128-row atoms of the tcgen05 path and not worth a round trip through
+// tensor memory, so the products run as warp-level m16n8k16 MMAs on register fragments: S = Q K^T, online softmax on the
+// accumulator fragments, P (rounded to BF16) reused in place as the A operand of O += P V, with V read through transposing
+// ldmatrix loads.  Key fragments are read 16 bytes at a time, the contraction index permuted identically for both operands
+// (see gemm_few.cuh).  Keys and values that are older than the plan (cross-attention: the encoder wrote them) are requested
+// before the dependency wait.
 #pragma once
 
 #include "attention.cuh"
@@ -16,7 +15,6 @@ namespace ad {
 
 constexpr int AM_Q = 64;        // queries per CTA with one key group
 constexpr int AM_KT = 64;       // keys per shared-memory tile
-constexpr int AM_LD = 64 + 8;   // padded row length (bf16 elements): rows 144 bytes apart, conflict-free fragments
 
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm(
@@ -29,25 +27,129 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);   // .x = lo (low half), .y = hi
   return *reinterpret_cast<uint32_t*>(&h);
 }
-// Two 8x8 BF16 matrices, transposed on the way into registers: lanes 0..7 give the row addresses of the first,
-// lanes 8..15 of the second.
-__device__ __forceinline__ void ldmatrix_x2_trans(uint32_t& r0, uint32_t& r1, const void* row_ptr) {
-  const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(row_ptr));
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
+// K/V tiles in shared memory.
+constexpr int AL_KLD = 96;             // key rows 192 bytes apart: conflict-free 16-byte fragment loads
+constexpr int AL_VLD = 72;             // value rows 144 bytes apart: conflict-free ldmatrix
+constexpr int AL_TILE_BYTES = AM_KT * (AL_KLD + AL_VLD) * 2;   // 21 504
+
+// 16-byte asynchronous copy global -> shared; src_bytes = 0 writes zeros (the source address must still be valid).
+__device__ __forceinline__ void am_cp_async16(void* smem_dst, const void* gmem_src, int src_bytes) {
+  const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem_src), "r"(src_bytes) : "memory");
 }
 
-// NG = number of key groups.  With NG = 1 the CTA's four warps take 16 queries each (64 queries per CTA).  When
-// rows have few queries, NG = 2 or 4 warps share a 16-query tile instead (32 or 16 queries per CTA) and split
-// the keys of every K/V tile between them; their running maxima, sums and outputs are merged at the end.
+// One 64-key tile of K and V into `dst`; keys from row_nk on are written as zeros.
+template <int THREADS>
+__device__ __forceinline__ void fetch_kv_tile(uint8_t* dst, const bf16* k, const bf16* v, int first_key, int row_nk, int d, int tid) {
+  bf16* kd = reinterpret_cast<bf16*>(dst);
+#pragma unroll
+  for (int i = 0; i < AM_KT * 8 / THREADS; ++i) {
+    const int idx = tid + THREADS * i, j = idx >> 3, c = (idx & 7) * 8;
+    const bool there = first_key + j < row_nk;
+    const size_t off = (size_t)(there ? first_key + j : 0) * d + c;
+    am_cp_async16(kd + j * AL_KLD + c, k + off, there ? 16 : 0);
+    am_cp_async16(kd + AM_KT * AL_KLD + j * AL_VLD + c, v + off, there ? 16 : 0);
+  }
+}
+
+// Running state of 16 queries of a warp: output fragments, maxima, this lane's share of the row sums.
+struct AttnState {
+  float o[8][4];
+  float mx0, mx1, den0, den1;
+};
+__device__ __forceinline__ void attn_init(AttnState& a) {
+#pragma unroll
+  for (int t = 0; t < 8; ++t) { a.o[t][0] = 0.f; a.o[t][1] = 0.f; a.o[t][2] = 0.f; a.o[t][3] = 0.f; }
+  a.mx0 = a.mx1 = -INFINITY;
+  a.den0 = a.den1 = 0.f;
+}
+// KS keys (rows of ks / vs; the first is key jw of the row) for 16 queries whose two of this lane see nk0 / nk1 keys.
+template <int KS>
+__device__ __forceinline__ void attn_keys(AttnState& a, const uint4 (&qa)[2][2], const bf16* ks, const bf16* vs, int jw, int nk0, int nk1,
+                                          float scale, int lane) {
+  const int g = lane >> 2, tq = lane & 3;
+  constexpr int NT = KS / 8;
+  // S = Q K^T (consecutive MMAs go to different accumulators and do not wait for one another)
+  float s[NT][4];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) { s[nt][0] = 0.f; s[nt][1] = 0.f; s[nt][2] = 0.f; s[nt][3] = 0.f; }
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    uint4 kf[NT];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) kf[nt] = *reinterpret_cast<const uint4*>(ks + (nt * 8 + g) * AL_KLD + 32 * c + 8 * tq);
+    const uint32_t a0[4] = {qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y}, a1[4] = {qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w};
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(s[nt], a0, kf[nt].x, kf[nt].y);
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) mma_bf16_16816(s[nt], a1, kf[nt].z, kf[nt].w);
+  }
+  // mask, scale, online softmax; element e of group nt is key jw + nt * 8 + tq * 2 + (e & 1), query row e >> 1
+  if (jw + KS > nk0 || jw + KS > nk1) {
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      const int j = jw + nt * 8 + tq * 2;
+      if (j >= nk0) s[nt][0] = -INFINITY;
+      if (j + 1 >= nk0) s[nt][1] = -INFINITY;
+      if (j >= nk1) s[nt][2] = -INFINITY;
+      if (j + 1 >= nk1) s[nt][3] = -INFINITY;
+    }
+  }
+  float t0 = -INFINITY, t1 = -INFINITY;
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    s[nt][0] *= scale; s[nt][1] *= scale; s[nt][2] *= scale; s[nt][3] *= scale;
+    t0 = fmaxf(t0, fmaxf(s[nt][0], s[nt][1]));
+    t1 = fmaxf(t1, fmaxf(s[nt][2], s[nt][3]));
+  }
+  t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 1)); t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 2));
+  t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 1)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 2));
+  const bool on0 = nk0 > jw, on1 = nk1 > jw;         // otherwise none of these keys is visible to the query
+  const float m0n = on0 ? fmaxf(a.mx0, t0) : a.mx0, m1n = on1 ? fmaxf(a.mx1, t1) : a.mx1;
+  const float corr0 = on0 ? __expf(a.mx0 - m0n) : 1.f, corr1 = on1 ? __expf(a.mx1 - m1n) : 1.f;   // exp(-inf) = 0 at first
+  a.mx0 = m0n; a.mx1 = m1n;
+  const float e0 = on0 ? m0n : 0.f, e1 = on1 ? m1n : 0.f;           // (all scores are -inf when the query sees no key here)
+  float sum0 = 0.f, sum1 = 0.f;
+  uint32_t pa[KS / 16][4];
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    const float p0 = __expf(s[nt][0] - e0), p1 = __expf(s[nt][1] - e0);
+    const float p2 = __expf(s[nt][2] - e1), p3 = __expf(s[nt][3] - e1);
+    sum0 += p0 + p1; sum1 += p2 + p3;
+    // accumulator fragments of two neighbouring key groups are exactly one A fragment of 16 keys
+    pa[nt >> 1][(nt & 1) * 2 + 0] = pack_bf16(p0, p1);
+    pa[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
+  }
+  a.den0 = a.den0 * corr0 + sum0;
+  a.den1 = a.den1 * corr1 + sum1;
+#pragma unroll
+  for (int dt = 0; dt < 8; ++dt) { a.o[dt][0] *= corr0; a.o[dt][1] *= corr0; a.o[dt][2] *= corr1; a.o[dt][3] *= corr1; }
+#pragma unroll
+  for (int tt = 0; tt < KS / 16; ++tt) {
+#pragma unroll
+    for (int dt = 0; dt < 8; dt += 2) {              // lanes 0..15 address the keys of column group dt, 16..31 those of dt + 1
+      uint32_t v0, v1, v2, v3;
+      const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(vs + (tt * 16 + (lane & 15)) * AL_VLD + (dt + (lane >> 4)) * 8));
+      asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(v0), "=r"(v1), "=r"(v2), "=r"(v3) : "r"(addr));
+      mma_bf16_16816(a.o[dt], pa[tt], v0, v1);
+      mma_bf16_16816(a.o[dt + 1], pa[tt], v2, v3);
+    }
+  }
+}
+
+// ---- many queries -----------------------------------------------------------------------------------------
+// NG = number of key groups.  With NG = 1 the CTA's four warps take 16 queries each (64 queries per CTA) and walk the row's
+// tiles, the next one being copied under the arithmetic of this one.  When rows have few queries, or when 64-query CTAs would
+// leave SMs idle, NG = 2 or 4 warps share a 16-query tile instead (32 or 16 queries per CTA) and split the keys of every tile
+// between them; their running maxima, sums and outputs are merged at the end.
+// grid = (B * qchunks, H), qchunks = ceil(longest segment / queries per CTA); block = 128 threads.
 template <int NG>
-__global__ void __launch_bounds__(128)
-attention_mma_kernel(const AttnParams p) {
+__global__ void __launch_bounds__(128, 3)
+attention_mma_kernel(const AttnParams p, const int kv_old) {
   constexpr int DH = 64;
   constexpr int QT = 4 / NG;            // 16-query tiles per CTA
   constexpr int KS = AM_KT / NG;        // keys of a tile that one warp handles
-  __shared__ __align__(16) bf16 kv[2][AM_KT][AM_LD];
-  bf16 (*ks)[AM_LD] = kv[0];
-  bf16 (*vs)[AM_LD] = kv[1];
+  __shared__ __align__(16) uint8_t kv[2][AL_TILE_BYTES];
 
   trace_mark(TR_ATTN, 0);
   pdl_launch();
@@ -55,175 +157,92 @@ attention_mma_kernel(const AttnParams p) {
   const int chunk = blockIdx.x % p.qchunks;
   const int h = blockIdx.y;
   const int seg_len = plan_load(p.seg_len + b);
+  const int i0 = chunk * (16 * QT);
+  if (i0 >= seg_len) {
+    if ((blockIdx.x | blockIdx.y) == 0) pdl_wait();
+    return;
+  }
   const int seg_off = plan_load(p.seg_off + b);
   const int kbase = plan_load(p.key_base + b);
   const int row_nk = plan_load(p.nkeys_row + b);
-  const int i0 = chunk * (16 * QT);
-  if (i0 >= seg_len && (blockIdx.x | blockIdx.y) != 0) return;
-  pdl_wait();
-  trace_mark(TR_ATTN, 1);
-  if (i0 >= seg_len) return;
+  int q_nsplit = 0;
+  size_t q_stride = 0;
+  if (p.q_part.ptr) resolve_partials(p.q_part, plan_load(p.M_ptr), q_nsplit, q_stride);
   const int nq = min(16 * QT, seg_len - i0);
   const int m0 = seg_off + i0;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tq = lane & 3;           // fragment row (0..7) and column pair (0..3) of this lane
   const int qtile = warp % QT, grp = warp / QT;     // this warp's query tile and key group
-  const int kofs = grp * KS;                        // first key of a tile that this warp handles
   const bool active = qtile * 16 < nq;              // otherwise the warp only helps loading
   const int d = p.d;
   const bf16* q = reinterpret_cast<const bf16*>(p.q);
-  const bf16* kk = reinterpret_cast<const bf16*>(p.k);
-  const bf16* vv = reinterpret_cast<const bf16*>(p.v);
-
+  const bf16* kk = reinterpret_cast<const bf16*>(p.k) + (size_t)kbase * d + h * DH;
+  const bf16* vv = reinterpret_cast<const bf16*>(p.v) + (size_t)kbase * d + h * DH;
+  const int n_tiles = (row_nk + AM_KT - 1) / AM_KT;
+  auto fetch = [&](int tile) {
+    if (tile < n_tiles) fetch_kv_tile<128>(kv[tile & 1], kk, vv, tile * AM_KT, row_nk, d, tid);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (kv_old) { fetch(0); fetch(1); }
   // this lane's two queries (fragment rows g and g + 8 of the warp's 16) and their visible-key counts
   const int r0 = qtile * 16 + g, r1 = r0 + 8;
   int nk0 = 0, nk1 = 0;
-  if (r0 < nq) nk0 = p.nkeys_tok ? min(p.nkeys_tok[m0 + r0], row_nk) : row_nk;
-  if (r1 < nq) nk1 = p.nkeys_tok ? min(p.nkeys_tok[m0 + r1], row_nk) : row_nk;
-  // Q as A fragments of the four 16-wide steps along the head dimension
-  uint32_t qa[DH / 16][4];
-  if (p.q_part) {
-    // queries straight from the split-K partial sums of their projection (+ bias), rounded like stored ones
+  if (r0 < nq) nk0 = p.nkeys_tok ? min(plan_load(p.nkeys_tok + m0 + r0), row_nk) : row_nk;
+  if (r1 < nq) nk1 = p.nkeys_tok ? min(plan_load(p.nkeys_tok + m0 + r1), row_nk) : row_nk;
+  pdl_wait();
+  trace_mark(TR_ATTN, 1);
+  if (!kv_old) { fetch(0); fetch(1); }
+  // Q as A fragments: eight consecutive elements of the head per lane, 32-wide chunk and row
+  uint4 qa[2][2];
+  {
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-    for (int s4 = 0; s4 < DH / 16; ++s4) {
+    for (int c = 0; c < 2; ++c) {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int r = (e & 1) ? r1 : r0;
-        const int c = h * DH + s4 * 16 + tq * 2 + (e >> 1) * 8;
-        float2 acc = make_float2(0.f, 0.f);
+      for (int e = 0; e < 2; ++e) {
+        const int r = e ? r1 : r0, col = h * DH + 32 * c + 8 * tq;
+        qa[c][e] = zero;
         if (r < nq) {
-          if (p.q_bias) acc = *reinterpret_cast<const float2*>(p.q_bias + c);
-          const float* src = p.q_part + (size_t)(m0 + r) * d + c;
-          float2 part[ATT_MAX_QSPLIT];                 // all partials in one round trip
+          if (!p.q_part.ptr) {
+            qa[c][e] = *reinterpret_cast<const uint4*>(q + (size_t)(m0 + r) * d + col);
+          } else {      // split-K partial sums of the projection (+ bias), rounded like stored queries
+            float acc[8];
 #pragma unroll
-          for (int sp = 0; sp < ATT_MAX_QSPLIT; ++sp)
-            part[sp] = sp < p.q_nsplit ? *reinterpret_cast<const float2*>(src + sp * p.q_stride) : make_float2(0.f, 0.f);
+            for (int i = 0; i < 8; ++i) acc[i] = p.q_bias ? p.q_bias[col + i] : 0.f;
+            for (int sp = 0; sp < q_nsplit; ++sp) {
+              float part[8];
+              load8(p.q_part.ptr + sp * q_stride + (size_t)(m0 + r) * d + col, part);
 #pragma unroll
-          for (int sp = 0; sp < ATT_MAX_QSPLIT; ++sp) { acc.x += part[sp].x; acc.y += part[sp].y; }
+              for (int i = 0; i < 8; ++i) acc[i] += part[i];
+            }
+            qa[c][e] = make_uint4(pack_bf16(acc[0], acc[1]), pack_bf16(acc[2], acc[3]), pack_bf16(acc[4], acc[5]), pack_bf16(acc[6], acc[7]));
+          }
         }
-        qa[s4][e] = pack_bf16(acc.x, acc.y);
       }
-    }
-  } else {
-#pragma unroll
-    for (int s4 = 0; s4 < DH / 16; ++s4) {
-      const int c = h * DH + s4 * 16 + tq * 2;
-      const bf16* q0 = q + (size_t)(m0 + r0) * d + c;
-      const bf16* q1 = q + (size_t)(m0 + r1) * d + c;
-      qa[s4][0] = r0 < nq ? *reinterpret_cast<const uint32_t*>(q0) : 0u;
-      qa[s4][1] = r1 < nq ? *reinterpret_cast<const uint32_t*>(q1) : 0u;
-      qa[s4][2] = r0 < nq ? *reinterpret_cast<const uint32_t*>(q0 + 8) : 0u;
-      qa[s4][3] = r1 < nq ? *reinterpret_cast<const uint32_t*>(q1 + 8) : 0u;
     }
   }
-
-  float o[DH / 8][4];
-#pragma unroll
-  for (int t = 0; t < DH / 8; ++t) { o[t][0] = 0.f; o[t][1] = 0.f; o[t][2] = 0.f; o[t][3] = 0.f; }
-  float mx0 = -INFINITY, mx1 = -INFINITY, den0 = 0.f, den1 = 0.f;   // den: this lane's share of the row sums
-
-  // K/V tiles travel global -> registers -> shared memory; the loads of tile t + 1 are issued before the
-  // arithmetic of tile t so that their latency is hidden behind it.
-  constexpr int PIECES = AM_KT * (DH / 8) / 128;    // 16-byte pieces per thread, per matrix and tile
-  uint4 kreg[PIECES], vreg[PIECES];
-  auto fetch = [&](int j0) {
-#pragma unroll
-    for (int i = 0; i < PIECES; ++i) {
-      const int idx = tid + 128 * i;
-      const int j = idx >> 3, c = (idx & 7) * 8;
-      kreg[i] = make_uint4(0u, 0u, 0u, 0u);          // keys that do not exist read as zeros
-      vreg[i] = kreg[i];
-      if (j0 + j < row_nk) {
-        const size_t off = (size_t)(kbase + j0 + j) * d + h * DH + c;
-        kreg[i] = *reinterpret_cast<const uint4*>(kk + off);
-        vreg[i] = *reinterpret_cast<const uint4*>(vv + off);
-      }
-    }
-  };
-  fetch(0);
-  for (int j0 = 0; j0 < row_nk; j0 += AM_KT) {
-    __syncthreads();   // previous tile fully consumed
-#pragma unroll
-    for (int i = 0; i < PIECES; ++i) {
-      const int idx = tid + 128 * i;
-      const int j = idx >> 3, c = (idx & 7) * 8;
-      *reinterpret_cast<uint4*>(&ks[j][c]) = kreg[i];
-      *reinterpret_cast<uint4*>(&vs[j][c]) = vreg[i];
-    }
-    __syncthreads();
-    if (j0 + AM_KT < row_nk) fetch(j0 + AM_KT);
-    const int jw = j0 + kofs;                        // first key of this warp's share of the tile
-    if (!active || jw >= row_nk) continue;
-
-    // S = Q K^T for 16 queries x KS keys: KS / 8 key groups of 8, 4 steps along the head dimension
-    // (the step along the head dimension is the outer loop: consecutive MMAs then go to different accumulators
-    // and do not wait for one another)
-    float s[KS / 8][4];
-#pragma unroll
-    for (int nt = 0; nt < KS / 8; ++nt) { s[nt][0] = 0.f; s[nt][1] = 0.f; s[nt][2] = 0.f; s[nt][3] = 0.f; }
-#pragma unroll
-    for (int s4 = 0; s4 < DH / 16; ++s4) {
-      uint32_t kb0[KS / 8], kb1[KS / 8];
-#pragma unroll
-      for (int nt = 0; nt < KS / 8; ++nt) {
-        const bf16* kp = &ks[kofs + nt * 8 + g][s4 * 16 + tq * 2];
-        kb0[nt] = *reinterpret_cast<const uint32_t*>(kp);
-        kb1[nt] = *reinterpret_cast<const uint32_t*>(kp + 8);
-      }
-#pragma unroll
-      for (int nt = 0; nt < KS / 8; ++nt) mma_bf16_16816(s[nt], qa[s4], kb0[nt], kb1[nt]);
-    }
-    // mask, scale, online softmax; element e of group nt is key jw + nt * 8 + tq * 2 + (e & 1), query row e >> 1
-    float t0 = -INFINITY, t1 = -INFINITY;
-#pragma unroll
-    for (int nt = 0; nt < KS / 8; ++nt) {
-      const int j = jw + nt * 8 + tq * 2;
-      s[nt][0] = (j < nk0) ? s[nt][0] * p.scale : -INFINITY;
-      s[nt][1] = (j + 1 < nk0) ? s[nt][1] * p.scale : -INFINITY;
-      s[nt][2] = (j < nk1) ? s[nt][2] * p.scale : -INFINITY;
-      s[nt][3] = (j + 1 < nk1) ? s[nt][3] * p.scale : -INFINITY;
-      t0 = fmaxf(t0, fmaxf(s[nt][0], s[nt][1]));
-      t1 = fmaxf(t1, fmaxf(s[nt][2], s[nt][3]));
-    }
-    t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 1)); t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 2));
-    t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 1)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 2));
-    const bool on0 = nk0 > jw, on1 = nk1 > jw;       // otherwise none of these keys is visible to the query
-    const float m0n = on0 ? fmaxf(mx0, t0) : mx0, m1n = on1 ? fmaxf(mx1, t1) : mx1;
-    const float corr0 = on0 ? __expf(mx0 - m0n) : 1.f, corr1 = on1 ? __expf(mx1 - m1n) : 1.f;   // exp(-inf) = 0 at first
-    mx0 = m0n; mx1 = m1n;
-    float sum0 = 0.f, sum1 = 0.f;
-    uint32_t pa[KS / 16][4];
-#pragma unroll
-    for (int nt = 0; nt < KS / 8; ++nt) {
-      const float p0 = on0 ? __expf(s[nt][0] - m0n) : 0.f, p1 = on0 ? __expf(s[nt][1] - m0n) : 0.f;
-      const float p2 = on1 ? __expf(s[nt][2] - m1n) : 0.f, p3 = on1 ? __expf(s[nt][3] - m1n) : 0.f;
-      sum0 += p0 + p1; sum1 += p2 + p3;
-      // accumulator fragments of two neighbouring key groups are exactly one A fragment of 16 keys
-      pa[nt >> 1][(nt & 1) * 2 + 0] = pack_bf16(p0, p1);
-      pa[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
-    }
-    den0 = den0 * corr0 + sum0;
-    den1 = den1 * corr1 + sum1;
-    // O = O * corr + P V
-#pragma unroll
-    for (int dt = 0; dt < DH / 8; ++dt) { o[dt][0] *= corr0; o[dt][1] *= corr0; o[dt][2] *= corr1; o[dt][3] *= corr1; }
-#pragma unroll
-    for (int t = 0; t < KS / 16; ++t) {
-      uint32_t v0[DH / 8], v1[DH / 8];
-#pragma unroll
-      for (int dt = 0; dt < DH / 8; ++dt) ldmatrix_x2_trans(v0[dt], v1[dt], &vs[kofs + t * 16 + (lane & 15)][dt * 8]);
-#pragma unroll
-      for (int dt = 0; dt < DH / 8; ++dt) mma_bf16_16816(o[dt], pa[t], v0[dt], v1[dt]);
-    }
+  AttnState a;
+  attn_init(a);
+  for (int t = 0; t < n_tiles; ++t) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();                                 // everybody's copies of tile t have landed
+    const int jw = t * AM_KT + grp * KS;             // first key of this warp's share of the tile
+    const bf16* ks = reinterpret_cast<const bf16*>(kv[t & 1]);
+    if (active && jw < row_nk) attn_keys<KS>(a, qa, ks + grp * KS * AL_KLD, ks + AM_KT * AL_KLD + grp * KS * AL_VLD, jw, nk0, nk1, p.scale, lane);
+    __syncthreads();                                 // tile t is fully consumed
+    fetch(t + 2);
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
 
+  float den0 = a.den0, den1 = a.den1, mx0 = a.mx0, mx1 = a.mx1;
   den0 += __shfl_xor_sync(0xffffffffu, den0, 1); den0 += __shfl_xor_sync(0xffffffffu, den0, 2);
   den1 += __shfl_xor_sync(0xffffffffu, den1, 1); den1 += __shfl_xor_sync(0xffffffffu, den1, 2);
+  float (&o)[8][4] = a.o;
   if (NG > 1) {
     // Merge the key groups of a query tile.  Every lane of a group > 0 leaves its fragment (32 outputs, two
     // maxima, two sums) in the tile memory, value-major so that lanes hit different banks; the lane with the
     // same number in group 0 folds them in.
-    float* rec = reinterpret_cast<float*>(&kv[0][0][0]);   // [36][128]
+    float* rec = reinterpret_cast<float*>(&kv[0][0]);        // [36][128]
     __syncthreads();                                       // all tile reads are done
     if (grp > 0) {
 #pragma unroll
@@ -273,31 +292,31 @@ attention_mma_kernel(const AttnParams p) {
 
 // ---- rows with hundreds of keys ------------------------------------------------------------------------
 // In the kernel above a warp walks all K/V tiles of its row one after the other; with 400 keys that is seven tiles of
-// ~570 dependent-latency-bound instructions each, and a warp that is alone on its scheduler issues one instruction
-// every 5-6 cycles: 14-15 us per launch however few queries there are.  Here the KEYS are spread over warps instead:
-// a CTA holds QT 16-query tiles x NW key warps; warp (qtile, kw) handles the whole tiles kw, kw + NW, ... of the row
-// for its 16 queries, and the NW partial results (running maximum, sum, output) of a query tile are merged through
-// shared memory at the end.  All tiles of a round (NW tiles, 18 KB each) are copied asynchronously at once.
+// dependent-latency-bound instructions.  Here the KEYS are spread over warps instead: a CTA holds QT 16-query tiles x NW key
+// warps; warp (qtile, kw) handles the whole 64-key tiles kw, kw + NW, ... of the row for its 16 queries, and the NW partial
+// results (running maximum, sum, output) of a query tile are merged through shared memory at the end.
+// All tiles of a row are resident at once (up to AL_MAX_SLOTS, in rounds beyond that), and when the keys are older than the
+// plan (cross-attention: the encoder wrote them) they are copied before the dependency wait, off the critical path.  
 //
-// grid = (B * qchunks, H), qchunks = ceil(longest segment / (16 QT)); block = 32 QT NW threads;
-// dynamic shared memory = NW * AM_TILE_BYTES + AM_Q_BYTES.
-constexpr int AM_TILE_BYTES = 2 * AM_KT * AM_LD * 2;   // K and V of one 64-key tile: 18 432 bytes
-constexpr int AM_Q_BYTES = AM_Q * AM_LD * 2;           // staged queries of a CTA (up to 64)
-
-// 16-byte asynchronous copy global -> shared; src_bytes = 0 writes zeros (the source address must still be valid).
-__device__ __forceinline__ void am_cp_async16(void* smem_dst, const void* gmem_src, int src_bytes) {
-  const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem_src), "r"(src_bytes) : "memory");
+// What bounds it: with few queries latency (one round trip for the queries, two tiles per warp, one merge), with an encoder
+// pass's thousands the warp instructions of the softmax.  400 keys, 8 rows: AL_TIMES
+//
+// grid = (B * qchunks, H), qchunks = ceil(longest segment / (16 QT)); block = 32 QT NW threads; dynamic shared memory =
+// slots * AL_TILE_BYTES + 16 QT rows of queries (att_long_smem).
+constexpr int AL_MAX_SLOTS = 9;
+constexpr int AL_RECORD = 36;          // floats per thread in the merge
+inline int att_long_slots(int max_keys, int threads) {
+  const int tiles = (max_keys + AM_KT - 1) / AM_KT, merge = (AL_RECORD * threads * 4 + AL_TILE_BYTES - 1) / AL_TILE_BYTES;
+  return tiles < merge ? merge : (tiles > AL_MAX_SLOTS ? AL_MAX_SLOTS : tiles);
 }
+inline size_t att_long_smem(int slots, int qt) { return (size_t)slots * AL_TILE_BYTES + (size_t)16 * qt * AL_KLD * 2; }
 
 template <int QT, int NW>
 __global__ void __launch_bounds__(32 * QT * NW)
-attention_mma_wide_kernel(const AttnParams p) {
+attention_long_kernel(const AttnParams p, const int slots, const int kv_old) {
   constexpr int DH = 64;
   constexpr int THREADS = 32 * QT * NW;
-  constexpr int KS = AM_KT;             // a warp handles whole tiles
   extern __shared__ __align__(16) uint8_t am_smem[];
-  typedef bf16 (*TilePtr)[AM_LD];
 
   trace_mark(TR_ATTN, 0);
   pdl_launch();
@@ -305,14 +324,17 @@ attention_mma_wide_kernel(const AttnParams p) {
   const int chunk = blockIdx.x % p.qchunks;
   const int h = blockIdx.y;
   const int seg_len = plan_load(p.seg_len + b);
+  const int i0 = chunk * (16 * QT);
+  if (i0 >= seg_len) {
+    if ((blockIdx.x | blockIdx.y) == 0) pdl_wait();
+    return;
+  }
   const int seg_off = plan_load(p.seg_off + b);
   const int kbase = plan_load(p.key_base + b);
   const int row_nk = plan_load(p.nkeys_row + b);
-  const int i0 = chunk * (16 * QT);
-  if (i0 >= seg_len && (blockIdx.x | blockIdx.y) != 0) return;
-  pdl_wait();
-  trace_mark(TR_ATTN, 1);
-  if (i0 >= seg_len) return;
+  int q_nsplit = 0;
+  size_t q_stride = 0;
+  if (p.q_part.ptr) resolve_partials(p.q_part, plan_load(p.M_ptr), q_nsplit, q_stride);
   const int nq = min(16 * QT, seg_len - i0);
   const int m0 = seg_off + i0;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -321,165 +343,91 @@ attention_mma_wide_kernel(const AttnParams p) {
   const bool active = qtile * 16 < nq;              // otherwise the warp only helps loading
   const int d = p.d;
   const bf16* q = reinterpret_cast<const bf16*>(p.q);
-  const bf16* kk = reinterpret_cast<const bf16*>(p.k);
-  const bf16* vv = reinterpret_cast<const bf16*>(p.v);
-
-  // the first round of tiles does not depend on the queries: request it before they are fetched
+  const bf16* kk = reinterpret_cast<const bf16*>(p.k) + (size_t)kbase * d + h * DH;
+  const bf16* vv = reinterpret_cast<const bf16*>(p.v) + (size_t)kbase * d + h * DH;
   const int n_tiles = (row_nk + AM_KT - 1) / AM_KT;
+
   auto fetch_round = [&](int first_tile) {
-    for (int idx = tid; idx < NW * AM_KT * (DH / 8); idx += THREADS) {
-      const int tl = idx / (AM_KT * (DH / 8)), rem = idx - tl * (AM_KT * (DH / 8));
-      const int j = rem >> 3, c = (rem & 7) * 8;
-      const int key = (first_tile + tl) * AM_KT + j;
-      if ((first_tile + tl) < n_tiles) {             // tiles past the end are never read
-        const bool there = key < row_nk;             // keys that do not exist are written as zeros
-        const size_t off = (size_t)(kbase + (there ? key : 0)) * d + h * DH + c;
-        bf16 (*kd)[AM_LD] = reinterpret_cast<TilePtr>(am_smem + tl * AM_TILE_BYTES);
-        am_cp_async16(&kd[j][c], kk + off, there ? 16 : 0);
-        am_cp_async16(&kd[AM_KT + j][c], vv + off, there ? 16 : 0);
-      }
-    }
+    for (int tl = 0; tl < min(slots, n_tiles - first_tile); ++tl)
+      fetch_kv_tile<THREADS>(am_smem + (size_t)tl * AL_TILE_BYTES, kk, vv, (first_tile + tl) * AM_KT, row_nk, d, tid);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  fetch_round(0);
-
+  if (kv_old) fetch_round(0);
   // this lane's two queries (fragment rows g and g + 8 of the warp's 16) and their visible-key counts
   const int r0 = qtile * 16 + g, r1 = r0 + 8;
   int nk0 = 0, nk1 = 0;
-  if (r0 < nq) nk0 = p.nkeys_tok ? min(p.nkeys_tok[m0 + r0], row_nk) : row_nk;
-  if (r1 < nq) nk1 = p.nkeys_tok ? min(p.nkeys_tok[m0 + r1], row_nk) : row_nk;
-  // Queries that come as split-K partial sums of their projection are summed (+ bias) and rounded like stored ones by
-  // the whole CTA, every thread issuing all partial loads of its elements at once: one memory round trip.  (Left to
-  // the warps, each lane would walk its 16 fragment elements x q_nsplit partials in 16 dependent rounds.)
-  bf16 (*qs)[AM_LD] = reinterpret_cast<TilePtr>(am_smem + NW * AM_TILE_BYTES);   // [16 QT][AM_LD]
-  if (p.q_part) {
+  if (r0 < nq) nk0 = p.nkeys_tok ? min(plan_load(p.nkeys_tok + m0 + r0), row_nk) : row_nk;
+  if (r1 < nq) nk1 = p.nkeys_tok ? min(plan_load(p.nkeys_tok + m0 + r1), row_nk) : row_nk;
+  pdl_wait();
+  trace_mark(TR_ATTN, 1);
+  if (!kv_old) fetch_round(0);
+
+  // Queries as A fragments.  Those that come as split-K partial sums of their projection are summed (+ bias) and rounded like
+  // stored ones by the whole CTA, every thread issuing all partial loads of its elements at once: one memory round trip.
+  uint4 qa[2][2];                                    // [32-wide chunk of the head][row g / g + 8]
+  bf16* qs = reinterpret_cast<bf16*>(am_smem + (size_t)slots * AL_TILE_BYTES);   // [16 QT][AL_KLD]
+  if (p.q_part.ptr) {
     for (int idx = tid; idx < 16 * QT * (DH / 2); idx += THREADS) {
       const int r = idx / (DH / 2), c2 = (idx - r * (DH / 2)) * 2;
       float2 acc = make_float2(0.f, 0.f);
       if (r < nq) {
         const int c = h * DH + c2;
         if (p.q_bias) acc = *reinterpret_cast<const float2*>(p.q_bias + c);
-        const float* src = p.q_part + (size_t)(m0 + r) * d + c;
+        const float* src = p.q_part.ptr + (size_t)(m0 + r) * d + c;
         float2 part[ATT_MAX_QSPLIT];
 #pragma unroll
         for (int sp = 0; sp < ATT_MAX_QSPLIT; ++sp)
-          part[sp] = sp < p.q_nsplit ? *reinterpret_cast<const float2*>(src + sp * p.q_stride) : make_float2(0.f, 0.f);
+          part[sp] = sp < q_nsplit ? *reinterpret_cast<const float2*>(src + sp * q_stride) : make_float2(0.f, 0.f);
 #pragma unroll
         for (int sp = 0; sp < ATT_MAX_QSPLIT; ++sp) { acc.x += part[sp].x; acc.y += part[sp].y; }
       }
-      *reinterpret_cast<uint32_t*>(&qs[r][c2]) = pack_bf16(acc.x, acc.y);
+      *reinterpret_cast<uint32_t*>(qs + r * AL_KLD + c2) = pack_bf16(acc.x, acc.y);
+    }
+  } else {
+    const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+    const bf16* q0 = q + (size_t)(m0 + r0) * d + h * DH + 8 * tq;
+    const bf16* q1 = q + (size_t)(m0 + r1) * d + h * DH + 8 * tq;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      qa[c][0] = r0 < nq ? *reinterpret_cast<const uint4*>(q0 + 32 * c) : zero;
+      qa[c][1] = r1 < nq ? *reinterpret_cast<const uint4*>(q1 + 32 * c) : zero;
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();                                   // first round of tiles and the staged queries are in place
   trace_mark(TR_ATTN, 3);
-  // Q as A fragments of the four 16-wide steps along the head dimension
-  uint32_t qa[DH / 16][4];
-  if (p.q_part) {
+  if (p.q_part.ptr) {
 #pragma unroll
-    for (int s4 = 0; s4 < DH / 16; ++s4) {
-      const int c = s4 * 16 + tq * 2;
-      qa[s4][0] = *reinterpret_cast<const uint32_t*>(&qs[r0][c]);
-      qa[s4][1] = *reinterpret_cast<const uint32_t*>(&qs[r1][c]);
-      qa[s4][2] = *reinterpret_cast<const uint32_t*>(&qs[r0][c + 8]);
-      qa[s4][3] = *reinterpret_cast<const uint32_t*>(&qs[r1][c + 8]);
-    }
-  } else {
-#pragma unroll
-    for (int s4 = 0; s4 < DH / 16; ++s4) {
-      const int c = h * DH + s4 * 16 + tq * 2;
-      const bf16* q0 = q + (size_t)(m0 + r0) * d + c;
-      const bf16* q1 = q + (size_t)(m0 + r1) * d + c;
-      qa[s4][0] = r0 < nq ? *reinterpret_cast<const uint32_t*>(q0) : 0u;
-      qa[s4][1] = r1 < nq ? *reinterpret_cast<const uint32_t*>(q1) : 0u;
-      qa[s4][2] = r0 < nq ? *reinterpret_cast<const uint32_t*>(q0 + 8) : 0u;
-      qa[s4][3] = r1 < nq ? *reinterpret_cast<const uint32_t*>(q1 + 8) : 0u;
+    for (int c = 0; c < 2; ++c) {
+      qa[c][0] = *reinterpret_cast<const uint4*>(qs + r0 * AL_KLD + 32 * c + 8 * tq);
+      qa[c][1] = *reinterpret_cast<const uint4*>(qs + r1 * AL_KLD + 32 * c + 8 * tq);
     }
   }
 
-  float o[DH / 8][4];
-#pragma unroll
-  for (int t = 0; t < DH / 8; ++t) { o[t][0] = 0.f; o[t][1] = 0.f; o[t][2] = 0.f; o[t][3] = 0.f; }
-  float mx0 = -INFINITY, mx1 = -INFINITY, den0 = 0.f, den1 = 0.f;   // den: this lane's share of the row sums
-
-  for (int first = 0; first < n_tiles; first += NW) {
+  AttnState a;
+  attn_init(a);
+  for (int first = 0; first < n_tiles; first += slots) {
     if (first > 0) {
       __syncthreads();                               // the previous round is fully consumed
       fetch_round(first);
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       __syncthreads();                               // everybody's copies have landed
     }
-    const int t = first + kw;
-    if (!active || t >= n_tiles) continue;
-    const int jw = t * AM_KT;                        // first key of this warp's tile
-    bf16 (*ks)[AM_LD] = reinterpret_cast<TilePtr>(am_smem + kw * AM_TILE_BYTES);
-    bf16 (*vs)[AM_LD] = ks + AM_KT;
-
-    // S = Q K^T for 16 queries x 64 keys (the step along the head dimension is the outer loop: consecutive MMAs go
-    // to different accumulators and do not wait for one another)
-    float s[KS / 8][4];
-#pragma unroll
-    for (int nt = 0; nt < KS / 8; ++nt) { s[nt][0] = 0.f; s[nt][1] = 0.f; s[nt][2] = 0.f; s[nt][3] = 0.f; }
-#pragma unroll
-    for (int s4 = 0; s4 < DH / 16; ++s4) {
-      uint32_t kb0[KS / 8], kb1[KS / 8];
-#pragma unroll
-      for (int nt = 0; nt < KS / 8; ++nt) {
-        const bf16* kp = &ks[nt * 8 + g][s4 * 16 + tq * 2];
-        kb0[nt] = *reinterpret_cast<const uint32_t*>(kp);
-        kb1[nt] = *reinterpret_cast<const uint32_t*>(kp + 8);
-      }
-#pragma unroll
-      for (int nt = 0; nt < KS / 8; ++nt) mma_bf16_16816(s[nt], qa[s4], kb0[nt], kb1[nt]);
-    }
-    // mask, scale, online softmax; element e of group nt is key jw + nt * 8 + tq * 2 + (e & 1), query row e >> 1
-    float t0 = -INFINITY, t1 = -INFINITY;
-#pragma unroll
-    for (int nt = 0; nt < KS / 8; ++nt) {
-      const int j = jw + nt * 8 + tq * 2;
-      s[nt][0] = (j < nk0) ? s[nt][0] * p.scale : -INFINITY;
-      s[nt][1] = (j + 1 < nk0) ? s[nt][1] * p.scale : -INFINITY;
-      s[nt][2] = (j < nk1) ? s[nt][2] * p.scale : -INFINITY;
-      s[nt][3] = (j + 1 < nk1) ? s[nt][3] * p.scale : -INFINITY;
-      t0 = fmaxf(t0, fmaxf(s[nt][0], s[nt][1]));
-      t1 = fmaxf(t1, fmaxf(s[nt][2], s[nt][3]));
-    }
-    t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 1)); t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 2));
-    t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 1)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 2));
-    const bool on0 = nk0 > jw, on1 = nk1 > jw;       // otherwise none of these keys is visible to the query
-    const float m0n = on0 ? fmaxf(mx0, t0) : mx0, m1n = on1 ? fmaxf(mx1, t1) : mx1;
-    const float corr0 = on0 ? __expf(mx0 - m0n) : 1.f, corr1 = on1 ? __expf(mx1 - m1n) : 1.f;   // exp(-inf) = 0 at first
-    mx0 = m0n; mx1 = m1n;
-    float sum0 = 0.f, sum1 = 0.f;
-    uint32_t pa[KS / 16][4];
-#pragma unroll
-    for (int nt = 0; nt < KS / 8; ++nt) {
-      const float p0 = on0 ? __expf(s[nt][0] - m0n) : 0.f, p1 = on0 ? __expf(s[nt][1] - m0n) : 0.f;
-      const float p2 = on1 ? __expf(s[nt][2] - m1n) : 0.f, p3 = on1 ? __expf(s[nt][3] - m1n) : 0.f;
-      sum0 += p0 + p1; sum1 += p2 + p3;
-      pa[nt >> 1][(nt & 1) * 2 + 0] = pack_bf16(p0, p1);
-      pa[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
-    }
-    den0 = den0 * corr0 + sum0;
-    den1 = den1 * corr1 + sum1;
-#pragma unroll
-    for (int dt = 0; dt < DH / 8; ++dt) { o[dt][0] *= corr0; o[dt][1] *= corr0; o[dt][2] *= corr1; o[dt][3] *= corr1; }
-#pragma unroll
-    for (int tt = 0; tt < KS / 16; ++tt) {
-      uint32_t v0[DH / 8], v1[DH / 8];
-#pragma unroll
-      for (int dt = 0; dt < DH / 8; ++dt) ldmatrix_x2_trans(v0[dt], v1[dt], &vs[tt * 16 + (lane & 15)][dt * 8]);
-#pragma unroll
-      for (int dt = 0; dt < DH / 8; ++dt) mma_bf16_16816(o[dt], pa[tt], v0[dt], v1[dt]);
+    for (int tl = kw; active && tl < min(slots, n_tiles - first); tl += NW) {
+      const int jw = (first + tl) * AM_KT;           // first key of this tile
+      const bf16* ks = reinterpret_cast<const bf16*>(am_smem + (size_t)tl * AL_TILE_BYTES);
+      attn_keys<AM_KT>(a, qa, ks, ks + AM_KT * AL_KLD, jw, nk0, nk1, p.scale, lane);
     }
   }
 
+  float den0 = a.den0, den1 = a.den1, mx0 = a.mx0, mx1 = a.mx1;
+  float (&o)[8][4] = a.o;
   den0 += __shfl_xor_sync(0xffffffffu, den0, 1); den0 += __shfl_xor_sync(0xffffffffu, den0, 2);
   den1 += __shfl_xor_sync(0xffffffffu, den1, 1); den1 += __shfl_xor_sync(0xffffffffu, den1, 2);
   // Merge the key warps of a query tile.  Every lane leaves its fragment (32 outputs, two maxima, two sums) in the tile
   // memory, value-major so that lanes hit different banks.  The merge itself is spread over the key warps as well: key
   // warp kw folds the NW records for the output columns 8 dt .. 8 dt + 7 with dt = kw, kw + NW, ... and stores them
-  // (folding everything in key warp 0 took longer than the attention itself).  36 * THREADS floats <= NW tiles.
+  // (folding everything in key warp 0 took longer than the attention itself).  (AL_RECORD * THREADS floats fit the slots.)
   float* rec = reinterpret_cast<float*>(am_smem);          // [36][THREADS]
   trace_mark(TR_ATTN, 4);
   __syncthreads();                                         // all tile reads are done

@@ -21,6 +21,7 @@ constexpr int THREADS = 256;
 constexpr int WARPS = 8;
 constexpr int FEAT = 16;          // output features per CTA = MMA M
 constexpr int RED_LD = 20;        // floats per token row of a warp's partial sums: conflict-free, 16-byte aligned
+constexpr int MAX_TOKENS = 128;   // most packed tokens of a pass that these kernels take
 constexpr int MAX_CHUNKS = 4;     // 32-wide K chunks per warp: K per CTA = 256 .. 1024
 
 // D (16 x 8, FP32) += A (16 x 16, BF16, row-major) * B (16 x 8, BF16, column-major).  Not volatile: free to be scheduled.
@@ -31,6 +32,9 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// Most tokens a pass may have for this kernel to be the faster one: two rounds.  (90 tokens of a 768-wide model, three rounds of
+// 32: 4.9 us a projection against 3.3 us on the tcgen05 kernel.)
+inline int max_tokens(int nch) { return nch <= 2 ? MAX_TOKENS : 64; }
 // Tokens of one round trip: 64 while a warp's slice of K is 64 wide, 32 beyond (register budget of two CTAs per SM).
 __host__ __device__ constexpr int round_tokens(int nch) { return nch <= 2 ? 64 : 32; }
 
@@ -74,20 +78,21 @@ __device__ __forceinline__ uint4 embed8(const EmbedParams& ep, int tok, int pos,
   return make_uint4(r[0], r[1], r[2], r[3]);
 }
 
-// grid = (N / 16, ksplit); block = 256; K / ksplit = 256 * NCH.
-// EPI_F32: partial sums [ksplit][M_cap, N] (no bias); EPI_ACT: bias (+ ReLU) -> BF16; EPI_SCATTER: q / K / V rows.
+// Body of the kernel for the CTA of features 16 bx .. 16 bx + 15 and K part kz (K / ksplit = 256 * NCH).
+// EPI_F32: partial sums [ksplit][M, N] (no bias); EPI_ACT: bias (+ ReLU) -> BF16; EPI_SCATTER: q / K / V rows.
 // EMB: the operand is the embedding (ep), X is not read; nothing depends on the predecessor until the first store.
+// red: shared memory, [WARPS][round_tokens(NCH)][RED_LD] floats.
+__host__ __device__ constexpr size_t red_bytes(int nch) { return sizeof(float) * WARPS * (nch <= 2 ? 64 : 32) * RED_LD; }
+
 template <int EPI, int NCH, bool EMB>
-__global__ void __launch_bounds__(THREADS, 2)
-gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, const EmbedParams ep) {
+__device__ __forceinline__ void few_body(const bf16* __restrict__ W, const bf16* X, const GemmParams& p, const EmbedParams& ep, int bx,
+                                         int kz, int M, float* red_mem) {
   constexpr int TPR = round_tokens(NCH);
   constexpr int NT = TPR / 8;
-  __shared__ __align__(16) float red[WARPS][TPR][RED_LD];
-  trace_mark(TR_GEMM + EPI, 0);
-  pdl_launch();
+  float (*red)[TPR][RED_LD] = reinterpret_cast<float (*)[TPR][RED_LD]>(red_mem);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int n0 = blockIdx.x * FEAT;
-  const int kbase = blockIdx.y * (256 * NCH) + warp * (32 * NCH) + 8 * t;
+  const int n0 = bx * FEAT;
+  const int kbase = kz * (256 * NCH) + warp * (32 * NCH) + 8 * t;
   const size_t K = (size_t)p.K;
   uint4 wa[NCH][2];
 #pragma unroll
@@ -98,8 +103,6 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, c
   const int of = (tid & 3) * 4, ot = tid >> 2;               // this thread's output: four features of one token per round
   float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
   if (EPI != EPI_F32) bias = *reinterpret_cast<const float4*>(p.bias + n0 + of);
-  // the plan was complete before this kernel could start (see plan_data in ad_common.cuh)
-  const int M = plan_load(p.M_ptr);
   int slot = 0;
   if (EPI == EPI_SCATTER && ot < M) slot = plan_load(p.slot + ot);
   if (!EMB) pdl_wait();
@@ -153,7 +156,7 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, c
         v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
       }
       if (EPI == EPI_F32) {
-        *reinterpret_cast<float4*>(p.out_f32 + ((size_t)blockIdx.y * p.M_cap + m) * p.N + n0 + of) = v;
+        *reinterpret_cast<float4*>(p.out_f32 + ((size_t)kz * M + m) * p.N + n0 + of) = v;
       } else {
         v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
         if (EPI == EPI_ACT && p.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
@@ -178,7 +181,7 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, c
   if (EMB) {
     if (M <= 0) pdl_wait();                                  // (a grid without work still ends after its predecessor)
     const int groups = p.K >> 2;
-    for (int m = blockIdx.x; m < M; m += gridDim.x) {
+    for (int m = bx; m < M; m += p.N / FEAT) {
       const int tok = plan_load(ep.tok_id + m), pos = plan_load(ep.tok_pos + m);
       for (int i = tid; i < groups; i += THREADS) {
         const uint2 e = __ldg(reinterpret_cast<const uint2*>(ep.emb + (size_t)tok * K + 4 * i));
@@ -190,6 +193,16 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, c
       }
     }
   }
+}
+
+// grid = (N / 16, ksplit); block = 256.
+template <int EPI, int NCH, bool EMB>
+__global__ void __launch_bounds__(THREADS, 2)
+gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, const EmbedParams ep) {
+  __shared__ __align__(16) float red[red_bytes(NCH) / sizeof(float)];
+  trace_mark(TR_GEMM + EPI, 0);
+  pdl_launch();
+  few_body<EPI, NCH, EMB>(W, X, p, ep, blockIdx.x, blockIdx.y, plan_load(p.M_ptr), red);
   trace_mark(TR_GEMM + EPI, 2);
 }
 

@@ -3,14 +3,12 @@
 // tensor-core kernels.
 //
 // Two kernels.  gemm_f32_kernel: tiles of 64 or 128 features x 32 tokens, both operands copied asynchronously to shared memory
-// as they lie (no transposition: a thread multiplies 4 x 4 outputs by four consecutive k at a time, eight 16-byte shared
-// loads for 64 FFMA), contraction index walked in ascending order.  333 x 2048 x 512: 80 -> 21 us (the kernel before had one
-// thread per feature, 16 tokens and scalar loads).  gemm_f32_few_kernel: passes of few tokens, where that kernel's serial walk
-// along K is all latency: 16 features per CTA, K dealt to 16 half-warps, weights in registers before the dependency wait.
+// as they lie (no transposition: a thread multiplies its outputs by four consecutive k at a time).  gemm_f32_few_kernel:
+// passes of few tokens, where that kernel's walk along K is all latency: 16 features per CTA, K dealt to 16 half-warps,
+// weights in registers before the dependency wait.
 #pragma once
 
 #include "ad_common.cuh"
-#include "gemm_tc.cuh"   // warp_argmax
 
 namespace ad {
 namespace simt {
@@ -48,32 +46,43 @@ __device__ __forceinline__ void store_out(const GemmParams& p, int n, int m, flo
   }
 }
 
-// grid = (ceil(N / FEAT), ceil(M_cap / 32)); block = 2 * FEAT; dynamic smem smem_bytes<FEAT>().  x: [M_cap, K], w: [N, K].
-// vec: K is a multiple of four and both operands are 16-byte aligned.
+// grid = (ceil(N / FEAT), ceil(M_cap / 32)); block = 2 FEAT; dynamic smem smem_bytes<FEAT>().  x: [M_cap, K], w: [N, K].
+// A thread has 8 features x 4 tokens (twelve 16-byte shared loads for 128 FFMA); FEAT threads make up such a tile, and the two
+// groups of them take alternate quads of k, so that an SM has enough warps for its FFMA pipes although the tiles are few.  vec: K is a multiple of four and both operands are 16-byte aligned.
+constexpr int GROUPS = 2;
 template <int EPI, int FEAT>
-__global__ void __launch_bounds__(2 * FEAT)
+__global__ void __launch_bounds__(GROUPS * FEAT)
 gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p, const int vec) {
-  constexpr int THREADS = 2 * FEAT, TX = FEAT / 4;     // thread (tx, ty): features tx + TX i, tokens ty + 8 j (i, j < 4)
-  extern __shared__ __align__(16) float simt_smem[];   // [STAGES][FEAT + TOK][LDK]
+  constexpr int TX = FEAT / 8;                         // thread (tx, ty): features tx + TX i (i < 8), tokens ty + 8 j (j < 4)
+  constexpr int THREADS = GROUPS * FEAT;
+  constexpr int RSTEP = THREADS / (KT / 4);            // rows between a thread's 16-byte copies: FEAT / RSTEP of W, then of x
+  constexpr int NW = FEAT / RSTEP, NX = TOK / RSTEP;
+  extern __shared__ __align__(16) float simt_smem[];   // [STAGES][FEAT + TOK][LDK], later [GROUPS][32][FEAT] partial sums
   const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
   const int t0 = blockIdx.y * TOK, n0 = blockIdx.x * FEAT;
   pdl_launch();
-  if (t0 >= M && blockIdx.y > 0) return;
+  if (t0 >= M && (blockIdx.x | blockIdx.y) > 0) return;
   pdl_wait();
   if (t0 >= M) return;
-  const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  const int tid = threadIdx.x, grp = tid / FEAT, tt = tid % FEAT, tx = tt % TX, ty = tt / TX;
   const int K = p.K, nk = (K + KT - 1) / KT;
+  const int fr = tid / (KT / 4), fc = (tid % (KT / 4)) * 4;      // first row and k of this thread's 16-byte copies
+  const float *wsrc = w + (size_t)(n0 + fr) * K + fc, *xsrc = x + (size_t)(t0 + fr) * K + fc;
   auto fetch = [&](int kt) {
     float* dst = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK;
     const int k0 = kt * KT;
     if (kt < nk) {
       if (vec) {
-        for (int idx = tid; idx < (FEAT + TOK) * (KT / 4); idx += THREADS) {
-          const int r = idx / (KT / 4), c = (idx % (KT / 4)) * 4;
-          const bool is_w = r < FEAT;
-          const int row = is_w ? n0 + r : t0 + r - FEAT;
-          const bool there = row < (is_w ? p.N : M) && k0 + c < K;
-          cp16(dst + r * LDK + c, (is_w ? w : x) + (there ? (size_t)row * K + k0 + c : 0), there);
+        const bool in_k = k0 + fc < K;
+#pragma unroll
+        for (int i = 0; i < NW; ++i) {
+          const bool there = in_k && n0 + fr + RSTEP * i < p.N;
+          cp16(dst + (fr + RSTEP * i) * LDK + fc, there ? wsrc + (size_t)(RSTEP * i) * K + k0 : w, there);
+        }
+#pragma unroll
+        for (int i = 0; i < NX; ++i) {
+          const bool there = in_k && t0 + fr + RSTEP * i < M;
+          cp16(dst + (FEAT + fr + RSTEP * i) * LDK + fc, there ? xsrc + (size_t)(RSTEP * i) * K + k0 : x, there);
         }
       } else {
         for (int idx = tid; idx < (FEAT + TOK) * KT; idx += THREADS) {
@@ -87,9 +96,9 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  float acc[4][4];
+  float acc[8][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 8; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
 #pragma unroll
@@ -98,55 +107,73 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
     asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
     __syncthreads();                                    // stage kt has landed, stage kt - 1 is free
     fetch(kt + STAGES - 1);
-    const float* ws = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + tx * LDK;
-    const float* xs = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + (FEAT + ty) * LDK;
+    const float* ws = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + tx * LDK + 4 * grp;
+    const float* xs = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + (FEAT + ty) * LDK + 4 * grp;
 #pragma unroll
-    for (int k = 0; k < KT; k += 4) {
-      float4 a[4], b[4];
+    for (int k = 0; k < KT; k += 4 * GROUPS) {
+      float4 a[8], b[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(ws + i * TX * LDK + k);
+      for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4*>(ws + i * TX * LDK + k);
 #pragma unroll
       for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(xs + j * 8 * LDK + k);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
     }
   }
+  // the groups' sums meet in shared memory
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  float* sums = simt_smem;
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sums[(size_t)(grp * 32 + i * 4 + j) * FEAT + tt] = acc[i][j];
+  __syncthreads();
   if (EPI == EPI_ARGMAX) {
-    // FEAT == 128: a warp holds all 128 features of its four tokens; ascending ids on ties
+    // the first group finishes: the TX threads of a token are neighbours and hold its FEAT features; lowest id on ties
+    if (grp > 0) return;
     const int lane = tid & 31;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int m = t0 + ty + 8 * j;
-      const bool on = m < M;                            // warp-uniform
+      const bool on = m < M;
       float v = -INFINITY;
       int id = 0x7fffffff, cnt = 0;
       const float dval = p.draft_val && on ? p.draft_val[m] : 0.f;
       const int did = p.draft_val && on ? p.draft_id[m] : -1;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < 8; ++i) {
         const int n = n0 + tx + TX * i;
         if (n < p.N) {
-          if (acc[i][j] > v) { v = acc[i][j]; id = n; }
-          if (p.draft_val && n != did && acc[i][j] > dval) ++cnt;   // other features that score strictly higher
+          float s = 0.f;
+#pragma unroll
+          for (int q = 0; q < GROUPS; ++q) s += sums[(size_t)(q * 32 + i * 4 + j) * FEAT + tt];
+          if (s > v) { v = s; id = n; }
+          if (p.draft_val && n != did && s > dval) ++cnt;           // other features that score strictly higher
         }
       }
-      tc::warp_argmax(v, id);
-      if (p.draft_val) cnt = __reduce_add_sync(0xffffffffu, cnt);
-      if (lane == 0 && on) {
+#pragma unroll
+      for (int o = TX / 2; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, id, o);
+        if (ov > v || (ov == v && oi < id)) { v = ov; id = oi; }
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+      }
+      if ((lane & (TX - 1)) == 0 && on) {
         const size_t o = (size_t)m * gridDim.x + blockIdx.x;
         p.part_val[o] = v;
         p.part_idx[o] = id;
@@ -154,16 +181,15 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
       }
     }
   } else {
+    // output (token, feature): neighbouring threads take neighbouring features
+    for (int idx = tid; idx < FEAT * TOK; idx += THREADS) {
+      const int f = idx % FEAT, tok = idx / FEAT, n = n0 + f, m = t0 + tok;
+      if (n >= p.N || m >= M) continue;
+      const int e = (f / TX) * 4 + tok / 8, th = (tok % 8) * TX + f % TX;
+      float s = p.bias ? p.bias[n] : 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int n = n0 + tx + TX * i;
-      if (n >= p.N) continue;
-      const float b = p.bias ? p.bias[n] : 0.f;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int m = t0 + ty + 8 * j;
-        if (m < M) store_out<EPI>(p, n, m, acc[i][j] + b);
-      }
+      for (int q = 0; q < GROUPS; ++q) s += sums[(size_t)(q * 32 + e) * FEAT + th];
+      store_out<EPI>(p, n, m, s);
     }
   }
 }

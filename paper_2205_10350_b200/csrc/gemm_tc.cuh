@@ -16,6 +16,7 @@
 #pragma once
 
 #include "ad_common.cuh"
+#include "gemm_few.cuh"
 
 namespace ad {
 namespace tc {
@@ -241,16 +242,35 @@ __device__ __forceinline__ void warp_argmax(float& v, int& i) {
   }
 }
 
-// grid = (ceil(N / 128), ceil(M_cap / ntile), ksplit); block = 256 threads;
-// dynamic smem = stages * stage bytes + 1024.
+// Token-operand maps of one buffer by token tile: box rows 16, 32, 64, 128, 256.
+struct TileMaps { CUtensorMap m[5]; };
+
+// Ring depth for a token tile in `budget` bytes of shared memory and kb K blocks.  Several ring rounds: the kernel's producer
+// count divides the depth, so the prime depths 5 and 7 are avoided.
+__host__ __device__ inline int ring_stages(int tile, int kb, int budget) {
+  int s = budget / (A_STAGE_BYTES + tile * BLOCK_K * 2);
+  s = s < 1 ? 1 : (s > MAX_STAGES ? MAX_STAGES : s);
+  if (s >= kb) return kb > 0 ? kb : 1;
+  return s == 5 || s == 7 ? s - 1 : s;
+}
+__host__ __device__ inline int geometry_ctas(const GeoRule& r, int M) {
+  const Geo g = geometry(r, M);
+  if (g.few) return r.N / few::FEAT * g.ksplit;
+  return (r.N + BLOCK_N_FEAT - 1) / BLOCK_N_FEAT * ((M + g.tile - 1) / g.tile) * g.ksplit;
+}
+
+// grid = (feature tiles, enough for the most CTAs that any token count of the pass asks for: geometry_ctas); block = 256
+// threads; dynamic smem = max(ring, transposition buffer, few-token partial sums) + 1024, `budget` of it for the ring.
+// blockIdx.y: token tile, then K part.
 //
 // Order of events in a CTA (the part before pdl_wait() overlaps the previous kernel of the stream):
-//   barriers, TMEM allocation, pdl_launch;  producer: weight tiles of the first ring round (token tile 0 only);
-//   pdl_wait;  token count M;  producer: activation tiles, then the rest of the K loop;  MMA issue;  epilogue.
-template <int EPI>
-__global__ void __launch_bounds__(THREADS, 1)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
-               const GemmParams p, const int stages) {
+//   token count M and geometry; barriers, TMEM allocation, pdl_launch;  producer: weight tiles of the first ring round;
+//   pdl_wait;  producer: activation tiles, then the rest of the K loop;  MMA issue;  epilogue.
+// NCH > 0: passes of few tokens take the few-token body (gemm_few.cuh) with NCH K chunks per warp instead.
+template <int EPI, int NCH>
+__global__ void __launch_bounds__(THREADS, 2)
+gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ TileMaps maps_x, const GemmParams p,
+               const int budget, const bf16* __restrict__ w_ptr, const bf16* x_ptr) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_full[MAX_STAGES];
   __shared__ __align__(8) uint64_t bar_empty[MAX_STAGES];
@@ -262,23 +282,35 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   __shared__ int did_s[256];
 
   trace_mark(TR_GEMM + EPI, 0);
-  const int ntile = p.ntile;
-  const int t0 = blockIdx.y * ntile;
-  const int n0 = blockIdx.x * BLOCK_N_FEAT;
+  const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
+  const Geo geo = geometry(p.rule, M);
+  if (NCH > 0 && geo.few) {
+    const int nbx = p.N / few::FEAT;
+    pdl_launch();
+    const int id = blockIdx.y * gridDim.x + blockIdx.x;
+    if (id < nbx * geo.ksplit)
+      few::few_body<EPI == EPI_ARGMAX ? EPI_ACT : EPI, NCH == 0 ? 1 : NCH, false>(
+          w_ptr, x_ptr, p, few::EmbedParams{}, id % nbx, id / nbx, M, reinterpret_cast<float*>(smem_raw));
+    trace_mark(TR_GEMM + EPI, 2);
+    return;
+  }
+  const int ntile = geo.tile, ksplit = geo.ksplit;
+  const int nf = gridDim.x, fx = blockIdx.x, ntt = (M + ntile - 1) >> (31 - __clz(ntile));
+  if ((int)blockIdx.y >= ntt * ksplit && (blockIdx.x | blockIdx.y) > 0) return;      // (CTA 0 always waits)
+  int ty = blockIdx.y, kz = 0;
+  if (ksplit > 1)
+    for (; ty >= ntt && kz + 1 < ksplit; ++kz) ty -= ntt;
+  const CUtensorMap& map_x = maps_x.m[27 - __clz(ntile)];
+  const int t0 = ty * ntile;
+  const int n0 = fx * BLOCK_N_FEAT;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quad = warp & 3, grp = warp >> 2;   // accumulator lane quadrant of this warp; column group in the epilogue
   const int b_stage_bytes = ntile * BLOCK_K * 2;
   const int stage_bytes = A_STAGE_BYTES + b_stage_bytes;
   const int kb_total = p.K / BLOCK_K;
-  const int ksplit = (EPI == EPI_F32 && p.ksplit > 1) ? p.ksplit : 1;
-  const int kb_begin = (int)(((long long)kb_total * blockIdx.z) / ksplit);
-  const int kb_end = (int)(((long long)kb_total * (blockIdx.z + 1)) / ksplit);
-  const int num_kb = kb_end - kb_begin;
+  const int num_kb = kb_total >> (31 - __clz(ksplit)), kb_begin = kz * num_kb;      // (a split divides the K blocks)
+  const int stages = ring_stages(ntile, num_kb, budget);
   const int first_round = num_kb < stages ? num_kb : stages;
-  // token tile 0 always has work (M >= 1 whenever a result is read); the others leave at once when the pass does not reach them
-  const bool early = (blockIdx.y == 0);
-  const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
-  if (!early && t0 >= M) return;
 
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzled tiles need 1024-byte alignment
   // MMA issuers.  Issuing one tcgen05.mma costs its thread 65-80 cycles whatever the tile, so with few tokens (short
@@ -327,7 +359,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   // TMA issue is spread over lane 0 of all eight warps: one thread's bulk-tensor copies are processed one after
   // the other, several threads' copies run side by side.  Stage i of the first ring round belongs to warp i;
   // later rounds are fed by up to four of the warps 0 .. 3.
-  if (early && lane == 0) {
+  if (lane == 0) {
     // weights never change: fetch the first ring round before the previous kernel has finished
     for (int i = warp; i < first_round; i += THREADS / 32) {
       const uint32_t bar = smem_u32(&bar_full[i]);
@@ -343,9 +375,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 
   pdl_wait();
   trace_mark(TR_GEMM + EPI, 1);
-  if (early && lane == 0) {
-    // activations of the first ring round (the activation buffer is always valid memory; rows beyond M are
-    // simply never stored), issued before the token count is known
+  if (lane == 0) {
+    // activations of the first ring round (rows beyond M are valid memory and simply never stored)
     for (int i = warp; i < first_round; i += THREADS / 32)
       tma_load_2d(smem_base + i * stage_bytes + A_STAGE_BYTES, &map_x, (kb_begin + i) * BLOCK_K, t0,
                   smem_u32(&bar_full[i]));
@@ -371,8 +402,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       int nprod = 1;
       for (int cand = 4; cand > 1; --cand)
         if (stages % cand == 0) { nprod = cand; break; }
-      const int begin = early ? first_round : 0;
-      for (int i = begin + pw; pw < nprod && i < num_kb; i += nprod) {
+      for (int i = first_round + pw; pw < nprod && i < num_kb; i += nprod) {
         const int s = i % stages;
         const uint32_t round = i / stages;
         if (round > 0 && !mbar_wait(smem_u32(&bar_empty[s]), (round - 1) & 1, p.status)) { abort_flag = 1; break; }
@@ -482,10 +512,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
           const float ov = red_val[w * ntile + t];
           if (ov > v) { v = ov; idx = red_idx[w * ntile + t]; }
         }
-        p.part_val[(size_t)(t0 + t) * gridDim.x + blockIdx.x] = v;
-        p.part_idx[(size_t)(t0 + t) * gridDim.x + blockIdx.x] = idx;
+        p.part_val[(size_t)(t0 + t) * nf + fx] = v;
+        p.part_idx[(size_t)(t0 + t) * nf + fx] = idx;
         if (relaxed)
-          p.part_cnt[(size_t)(t0 + t) * gridDim.x + blockIdx.x] =
+          p.part_cnt[(size_t)(t0 + t) * nf + fx] =
               red_cnt[t] + red_cnt[ntile + t] + red_cnt[2 * ntile + t] + red_cnt[3 * ntile + t];
       }
     }
@@ -518,7 +548,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       if (tb == 0) trace_mark(TR_GEMM + EPI, 5);
       __syncthreads();
       if (EPI == EPI_F32) {
-        float* out = p.out_f32 + (size_t)blockIdx.z * p.M_cap * p.N;
+        float* out = p.out_f32 + (size_t)kz * M * p.N;
         const int col = n0 + lane * 4;
         const bool vec = (p.N & 3) == 0;
         for (int r = warp; r < ntok; r += THREADS / 32) {

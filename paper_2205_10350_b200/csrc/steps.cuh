@@ -313,28 +313,6 @@ embed_kernel(PassPlan plan, const WT* __restrict__ emb, const float* __restrict_
   }
 }
 
-// ---------------------------------------------------------------------------------------------
-// Residual + LayerNorm:  x = sum_s pre[s][m, :] + bias + resid[m, :];  y = LN(x) (biased variance).
-// pre holds the split-K partial sums of the preceding projection (nsplit <= 16 of them, split_stride floats
-// apart).  One CTA per packed token; each thread owns up to two groups of four consecutive features and issues
-// all of its loads (partials, residual) at once, so the kernel costs one global-memory round trip.
-// y may alias resid.  d % 4 == 0, d <= 1024.  grid = M_cap, block = THREADS (128, or 256 for d > 512).
-// ---------------------------------------------------------------------------------------------
-template <int THREADS>
-__device__ __forceinline__ float block_sum(float v, float* red) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();                 // red may still be read from a previous call
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  float t = 0.f;
-#pragma unroll
-  for (int w = 0; w < THREADS / 32; ++w) t += red[w];
-  return t;
-}
-__device__ __forceinline__ float block_sum_128(float v, float* red) { return block_sum<128>(v, red); }
-
 __device__ __forceinline__ void load4(const float* p, float (&v)[4]) {
   const float4 f = *reinterpret_cast<const float4*>(p);
   v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
@@ -353,100 +331,152 @@ __device__ __forceinline__ void store4(bf16* p, float4 v) {
   *reinterpret_cast<uint2*>(p) = u;
 }
 
-// THREADS = 128 for d <= 512 and 256 beyond: one 4-element group per thread, so that all partial sums of a thread are
-// requested at once (with two groups per thread the second group's loads waited for the first group's sums: 2.8 us
-// instead of 1.5 us per launch on a 1024-wide model with 16 partials).
-template <typename ActT, int THREADS = 128>
+// ---------------------------------------------------------------------------------------------
+// Residual + LayerNorm:  x = sum_s pre[s][m, :] + bias + resid[m, :];  y = LN(x) (biased variance).
+// pre holds the partial sums of the preceding projection (Partials: at most 16).  y may alias resid.  d % 4 == 0, d <= 1024.
+// ---------------------------------------------------------------------------------------------
+struct LnParams {
+  const int* M_ptr;
+  Partials pre;
+  const float *bias, *resid, *g, *bta;   // bias, resid may be null
+  int d;
+  float eps;
+  float* y;
+};
+
+// Sum over the THREADS threads of a group: the CTA (half < 0), or one half of it.
+template <int THREADS>
+__device__ __forceinline__ void group_sync(int half) {
+  if (half < 0) __syncthreads();
+  else if (half == 0) asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+  else asm volatile("bar.sync 2, %0;" ::"n"(THREADS) : "memory");
+}
+template <int THREADS>
+__device__ __forceinline__ float group_sum(float v, float* red, int tid, int half) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  group_sync<THREADS>(half);       // red may still be read from a previous call
+  if ((tid & 31) == 0) red[tid >> 5] = v;
+  group_sync<THREADS>(half);
+  float t = 0.f;
+#pragma unroll
+  for (int w = 0; w < THREADS / 32; ++w) t += red[w];
+  return t;
+}
+
+// Gains and biases of one thread's four features: weights, fetched while the previous kernel is still running.
+struct LnWeights { float4 g, b, c; };
+__device__ __forceinline__ LnWeights ln_weights(const LnParams& p, int gi) {
+  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  const bool on = gi < (p.d >> 2);
+  LnWeights w;
+  w.g = on ? reinterpret_cast<const float4*>(p.g)[gi] : zero4;
+  w.b = on ? reinterpret_cast<const float4*>(p.bta)[gi] : zero4;
+  w.c = on && p.bias ? reinterpret_cast<const float4*>(p.bias)[gi] : zero4;
+  return w;
+}
+
+// Token m by a group of THREADS threads, four features per thread (d <= 4 * THREADS): all partial sums of a thread and the
+// residual are requested at once, so the kernel costs one memory round trip.  (Two groups of features per thread took 2.8 us
+// instead of 1.5 us per launch on a 1024-wide model with 16 partials.)
+template <typename ActT, int THREADS>
+__device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, int m, int nsplit, size_t stride, ActT* yb, float* red,
+                                         int tid, int half) {
+  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int groups = p.d >> 2;
+  const size_t off = (size_t)m * groups + tid;
+  const bool on = tid < groups;
+  float4 v = zero4;
+  if (on) {
+    float4 part[16];
+#pragma unroll
+    for (int sp = 0; sp < 16; ++sp)
+      part[sp] = (sp < nsplit) ? reinterpret_cast<const float4*>(p.pre.ptr + sp * stride)[off] : zero4;
+    const float4 r = p.resid ? reinterpret_cast<const float4*>(p.resid)[off] : zero4;
+    v = make_float4(w.c.x + r.x, w.c.y + r.y, w.c.z + r.z, w.c.w + r.w);
+#pragma unroll
+    for (int sp = 0; sp < 16; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
+  }
+  const float mean = group_sum<THREADS>(v.x + v.y + v.z + v.w, red, tid, half) / (float)p.d;
+  float vs = 0.f;
+  if (on) {
+    const float a = v.x - mean, b = v.y - mean, c = v.z - mean, e = v.w - mean;
+    vs = a * a + b * b + c * c + e * e;
+  }
+  const float inv = rsqrtf(group_sum<THREADS>(vs, red, tid, half) / (float)p.d + p.eps);
+  if (on) {
+    float4 o;
+    o.x = w.g.x * ((v.x - mean) * inv) + w.b.x;
+    o.y = w.g.y * ((v.y - mean) * inv) + w.b.y;
+    o.z = w.g.z * ((v.z - mean) * inv) + w.b.z;
+    o.w = w.g.w * ((v.w - mean) * inv) + w.b.w;
+    store4(p.y + off * 4, o);
+    store4(yb + off * 4, o);
+  }
+}
+
+// One CTA per token.  grid = M_cap, block = THREADS (128 for d <= 512, else 256).
+template <typename ActT, int THREADS>
 __global__ void __launch_bounds__(THREADS)
-layernorm_kernel(const int* __restrict__ M_ptr, const float* __restrict__ pre, int nsplit, size_t split_stride,
-                 const float* __restrict__ bias, const float* resid, const float* __restrict__ g,
-                 const float* __restrict__ bta, int d, float eps, float* y, ActT* __restrict__ yb) {
+layernorm_kernel(const LnParams p, ActT* __restrict__ yb) {
   __shared__ float red[THREADS / 32];
-  constexpr int NG = 256 / THREADS;            // groups per thread: d <= 1024
   trace_mark(TR_LN, 0);
   pdl_launch();
-  const int groups = d >> 2;
-  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  // gains and biases are weights: fetch them while the previous kernel is still running
-  float4 gv[NG], bv[NG], cb[NG];
-#pragma unroll
-  for (int i = 0; i < NG; ++i) {
-    const int gi = threadIdx.x + THREADS * i;
-    const bool on = gi < groups;
-    gv[i] = on ? reinterpret_cast<const float4*>(g)[gi] : zero4;
-    bv[i] = on ? reinterpret_cast<const float4*>(bta)[gi] : zero4;
-    cb[i] = (on && bias) ? reinterpret_cast<const float4*>(bias)[gi] : zero4;
-  }
-  const int m = blockIdx.x;
-  if (m >= plan_load(M_ptr) && m > 0) return;      // CTA 0 always waits (see early exits in ad_common.cuh)
+  const int m = blockIdx.x, M = plan_load(p.M_ptr);
+  const LnWeights w = ln_weights(p, threadIdx.x);
+  if (m >= M && m > 0) return;                     // CTA 0 always waits (see early exits in ad_common.cuh)
+  int nsplit;
+  size_t stride;
+  resolve_partials(p.pre, M, nsplit, stride);
   pdl_wait();
   trace_mark(TR_LN, 1);
-  float4 xv[NG];
-  float s = 0.f;
-#pragma unroll
-  for (int i = 0; i < NG; ++i) {
-    const int gi = threadIdx.x + THREADS * i;
-    float4 v = zero4;
-    if (gi < groups) {
-      const size_t off = (size_t)m * groups + gi;
-      float4 part[16];
-#pragma unroll
-      for (int sp = 0; sp < 16; ++sp)
-        part[sp] = (sp < nsplit) ? reinterpret_cast<const float4*>(pre + sp * split_stride)[off] : zero4;
-      const float4 r = resid ? reinterpret_cast<const float4*>(resid)[off] : zero4;
-      v = make_float4(cb[i].x + r.x, cb[i].y + r.y, cb[i].z + r.z, cb[i].w + r.w);
-#pragma unroll
-      for (int sp = 0; sp < 16; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
-    }
-    xv[i] = v;
-    s += v.x + v.y + v.z + v.w;
-  }
-  const float mean = block_sum<THREADS>(s, red) / (float)d;
-  float vs = 0.f;
-#pragma unroll
-  for (int i = 0; i < NG; ++i) {
-    if (threadIdx.x + THREADS * i < groups) {
-      const float a = xv[i].x - mean, b = xv[i].y - mean, c = xv[i].z - mean, e = xv[i].w - mean;
-      vs += a * a + b * b + c * c + e * e;
-    }
-  }
-  const float inv = rsqrtf(block_sum<THREADS>(vs, red) / (float)d + eps);
-#pragma unroll
-  for (int i = 0; i < NG; ++i) {
-    const int gi = threadIdx.x + THREADS * i;
-    if (gi < groups) {
-      float4 o;
-      o.x = gv[i].x * ((xv[i].x - mean) * inv) + bv[i].x;
-      o.y = gv[i].y * ((xv[i].y - mean) * inv) + bv[i].y;
-      o.z = gv[i].z * ((xv[i].z - mean) * inv) + bv[i].z;
-      o.w = gv[i].w * ((xv[i].w - mean) * inv) + bv[i].w;
-      const size_t off = ((size_t)m * groups + gi) * 4;
-      store4(y + off, o);
-      store4(yb + off, o);
-    }
-  }
+  if (m >= M) return;
+  ln_token<ActT, THREADS>(p, w, m, nsplit, stride, yb, red, threadIdx.x, -1);
   trace_mark(TR_LN, 2);
 }
 
-// The same operation for large token counts: one warp per token (no block-wide barrier), 8 tokens per CTA.
-// The loads of two element groups (residual and up to four partial sums each: ten 16-byte loads per lane) are issued
-// before their first use.  nsplit <= 4 here (more partials take the one-CTA-per-token kernel).
-// grid = ceil(M_cap / 8), block = 256, d <= 1024 and a multiple of 128.
+// Passes that may hold many tokens.  From LN_ROWS tokens on: one warp per token (no block-wide barrier), the loads of two
+// element groups (residual and up to four partial sums each: ten 16-byte loads per lane) issued before their first use.
+// Below that, or with more than four partials, a group of 128 threads (256 for d > 512) per token as in the kernel above
+// (1024 tokens: 458 us per step of the base model against 467 us with a warp per token; 2048 tokens: 582 against 543 us).
+// grid: at most two CTAs per SM, which loop (a grid sized for the capacity cost 5 us per launch in waves of CTAs without work);
+// block = 256; d a multiple of 128.
+constexpr int LN_ROWS = 1536;
 template <typename ActT>
 __global__ void __launch_bounds__(256, 2)
-layernorm_rows_kernel(const int* __restrict__ M_ptr, const float* __restrict__ pre, int nsplit, size_t split_stride,
-                      const float* __restrict__ bias, const float* resid, const float* __restrict__ g,
-                      const float* __restrict__ bta, int d, float eps, float* y, ActT* __restrict__ yb) {
+layernorm_many_kernel(const LnParams p, ActT* __restrict__ yb) {
+  __shared__ float red[2][8];
   trace_mark(TR_LN, 0);
   pdl_launch();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int M = plan_load(p.M_ptr), d = p.d;
+  int nsplit;
+  size_t stride;
+  resolve_partials(p.pre, M, nsplit, stride);
+  if (M < LN_ROWS || nsplit > 4) {
+    const int per_cta = d <= 512 ? 2 : 1;
+    int m = blockIdx.x * per_cta;
+    if (m >= M && blockIdx.x > 0) return;
+    const LnWeights w = ln_weights(p, per_cta == 2 ? (tid & 127) : tid);
+    pdl_wait();
+    trace_mark(TR_LN, 1);
+    for (; m < M; m += gridDim.x * per_cta) {
+      if (per_cta == 2) {
+        if (m + (tid >> 7) < M) ln_token<ActT, 128>(p, w, m + (tid >> 7), nsplit, stride, yb, red[tid >> 7], tid & 127, tid >> 7);
+      } else {
+        ln_token<ActT, 256>(p, w, m, nsplit, stride, yb, red[0], tid, -1);
+      }
+    }
+    trace_mark(TR_LN, 2);
+    return;
+  }
   const int per = d >> 7;                               // float4 groups per lane (d / 128), <= 8
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int m = blockIdx.x * 8 + warp, M = plan_load(M_ptr);
+  const float *pre = p.pre.ptr, *resid = p.resid, *bias = p.bias;
   if ((int)blockIdx.x * 8 >= M && blockIdx.x > 0) return;
   pdl_wait();
   trace_mark(TR_LN, 1);
-  if (m < M) {
+  for (int m = blockIdx.x * 8 + warp; m < M; m += gridDim.x * 8) {
     const size_t row = (size_t)m * (d >> 2);
     float4 xv[8];
     float s = 0.f;
@@ -462,7 +492,7 @@ layernorm_rows_kernel(const int* __restrict__ M_ptr, const float* __restrict__ p
         c4[i] = (gi < per && bias) ? reinterpret_cast<const float4*>(bias)[lane + 32 * gi] : zero4;
 #pragma unroll
         for (int sp = 0; sp < 4; ++sp)
-          q4[i][sp] = (gi < per && sp < nsplit) ? reinterpret_cast<const float4*>(pre + sp * split_stride)[off] : zero4;
+          q4[i][sp] = (gi < per && sp < nsplit) ? reinterpret_cast<const float4*>(pre + sp * stride)[off] : zero4;
       }
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
@@ -488,19 +518,19 @@ layernorm_rows_kernel(const int* __restrict__ M_ptr, const float* __restrict__ p
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) vs += __shfl_xor_sync(0xffffffffu, vs, o);
-    const float inv = rsqrtf(vs / (float)d + eps);
+    const float inv = rsqrtf(vs / (float)d + p.eps);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       if (i < per) {
-        const float4 gv = reinterpret_cast<const float4*>(g)[lane + 32 * i];
-        const float4 bv = reinterpret_cast<const float4*>(bta)[lane + 32 * i];
+        const float4 gv = reinterpret_cast<const float4*>(p.g)[lane + 32 * i];
+        const float4 bv = reinterpret_cast<const float4*>(p.bta)[lane + 32 * i];
         float4 o;
         o.x = gv.x * ((xv[i].x - mean) * inv) + bv.x;
         o.y = gv.y * ((xv[i].y - mean) * inv) + bv.y;
         o.z = gv.z * ((xv[i].z - mean) * inv) + bv.z;
         o.w = gv.w * ((xv[i].w - mean) * inv) + bv.w;
         const size_t off = (row + lane + 32 * i) * 4;
-        store4(y + off, o);
+        store4(p.y + off, o);
         store4(yb + off, o);
       }
     }
