@@ -2,6 +2,7 @@
 // commit, the choice of the next block and the layout of the pass that verifies it, all in one kernel.
 #pragma once
 
+#include "gemm_tc.cuh"   // float_key
 #include "steps.cuh"
 
 namespace ad {
@@ -40,6 +41,50 @@ __device__ __forceinline__ int cta_suffix_match(OutTok o, int j, const int* x, i
   }
   __syncthreads();
   return found;
+}
+
+// Arg-max over the tiles of H block positions (i0, i0 + 32, ...) by one warp, the lowest id on ties; U tiles per lane and
+// position in flight.  COUNT: also the sum of the tiles' counts.  decide(position, maximum, id, count) runs in lane 0.
+template <int H, int U, bool COUNT, typename F>
+__device__ __forceinline__ void scan_tiles(const float* __restrict__ val, const int* __restrict__ id, const int* __restrict__ cnt, int off, int i0,
+                                           int k, int n_tiles, int lane, F decide) {
+  float v[H];
+  int idx[H], higher[H];
+#pragma unroll
+  for (int h = 0; h < H; ++h) { v[h] = -INFINITY; idx[h] = 0x7fffffff; higher[h] = 0; }
+  for (int t0 = 0; t0 < n_tiles; t0 += 32 * U) {
+    float pv[H][U];
+    int pi[H][U], pc[H][COUNT ? U : 1];
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      const int i = i0 + 32 * h;
+      const size_t row = (size_t)(off + i) * n_tiles;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int t = t0 + 32 * u + lane;
+        const bool on = i < k && t < n_tiles;
+        pv[h][u] = on ? val[row + t] : -INFINITY;
+        pi[h][u] = on ? id[row + t] : 0x7fffffff;
+        if (COUNT) pc[h][u] = on ? cnt[row + t] : 0;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < H; ++h)
+#pragma unroll
+      for (int u = 0; u < U; ++u) {                       // (a lane's tiles ascend, and so do their ids)
+        if (pv[h][u] > v[h]) { v[h] = pv[h][u]; idx[h] = pi[h][u]; }
+        if (COUNT) higher[h] += pc[h][u];
+      }
+  }
+#pragma unroll
+  for (int h = 0; h < H; ++h) {
+    if (i0 + 32 * h >= k) break;
+    const unsigned int key = tc::float_key(v[h] + 0.f);      // (-0 and +0 are equal scores)
+    const unsigned int best = __reduce_max_sync(0xffffffffu, key);
+    const unsigned int lowest = __reduce_min_sync(0xffffffffu, key == best ? (unsigned int)idx[h] : 0x7fffffffu);
+    if (COUNT) higher[h] = __reduce_add_sync(0xffffffffu, higher[h]);
+    if (lane == 0) decide(i0 + 32 * h, tc::key_float(best), (int)lowest, higher[h]);
+  }
 }
 
 // The decision for one row:
@@ -94,56 +139,21 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
   // ---- arg-max over the tiles of every block position: a warp per position, the lowest id wins ties ----
   const bool relaxed = beta >= 1 && !to_drafts;
   int* pred = (to_drafts ? st.drafts : st.pred) + (size_t)b * dm.kmax;
-  // (two positions of a warp at once, eight tiles per lane and position in flight)
-  for (int i0 = warp; i0 < k; i0 += 2 * (ACC_THREADS / 32)) {
-    float v[2] = {-INFINITY, -INFINITY};
-    int idx[2] = {0x7fffffff, 0x7fffffff}, higher[2] = {0, 0};
-    for (int t0 = 0; t0 < n_tiles; t0 += 256) {
-      float pv[2][8];
-      int pi[2][8];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int i = i0 + h * (ACC_THREADS / 32);
-        const size_t row = (size_t)(off + i) * n_tiles;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int t = t0 + 32 * u + lane;
-          const bool on = i < k && t < n_tiles;
-          pv[h][u] = on ? part_val[row + t] : -INFINITY;
-          pi[h][u] = on ? part_idx[row + t] : 0x7fffffff;
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (pv[h][u] > v[h] || (pv[h][u] == v[h] && pi[h][u] < idx[h])) { v[h] = pv[h][u]; idx[h] = pi[h][u]; }
-        const int i = i0 + h * (ACC_THREADS / 32);
-        if (relaxed && i < k)
-          for (int t = t0 + lane; t < min(t0 + 256, n_tiles); t += 32) higher[h] += part_cnt[(size_t)(off + i) * n_tiles + t];
-      }
+  auto decide = [&](int i, float v, int idx, int higher) {      // lane 0 of the position's warp
+    int choice = idx;
+    if (relaxed) {
+      const int did = draft_id[off + i];
+      if (did >= 0 && higher <= beta - 1 && v - draft_val[off + i] <= tau) choice = did;
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = i0 + h * (ACC_THREADS / 32);
-      if (i >= k) break;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, v[h], o);
-        const int oi = __shfl_xor_sync(0xffffffffu, idx[h], o);
-        if (ov > v[h] || (ov == v[h] && oi < idx[h])) { v[h] = ov; idx[h] = oi; }
-        if (relaxed) higher[h] += __shfl_xor_sync(0xffffffffu, higher[h], o);
-      }
-      if (lane == 0) {
-        int choice = idx[h];
-        if (relaxed) {
-          const int did = draft_id[off + i];
-          if (did >= 0 && higher[h] <= beta - 1 && v[h] - draft_val[off + i] <= tau) choice = did;
-        }
-        s_pred[i] = choice;
-        if (!(to_drafts && next.source == SRC_KEEP)) pred[i] = choice;
-      }
-    }
+    s_pred[i] = choice;
+    if (!(to_drafts && next.source == SRC_KEEP)) pred[i] = choice;
+  };
+  if (relaxed) {
+    for (int i = warp; i < k; i += ACC_THREADS / 32) scan_tiles<1, 8, true>(part_val, part_idx, part_cnt, off, i, k, n_tiles, lane, decide);
+  } else if (k <= ACC_THREADS / 32) {
+    if (warp < k) scan_tiles<1, 16, false>(part_val, part_idx, part_cnt, off, warp, k, n_tiles, lane, decide);
+  } else {
+    for (int i = warp; i < k; i += 2 * (ACC_THREADS / 32)) scan_tiles<2, 8, false>(part_val, part_idx, part_cnt, off, i, k, n_tiles, lane, decide);
   }
   __syncthreads();
 

@@ -113,7 +113,8 @@ struct ad_handle {
   float *y = nullptr, *pre = nullptr;
   float* pre2 = nullptr;     // per-head partial sums of an output projection fused into the attention kernel
   ActBuf yb, abuf, hbuf, xg;
-  void *qbuf = nullptr, *ktmp = nullptr, *vtmp = nullptr, *kself = nullptr, *vself = nullptr, *encmem = nullptr;
+  void *qbuf = nullptr, *ktmp = nullptr, *vtmp = nullptr, *kself = nullptr, *vself = nullptr;
+  ActBuf encmem;             // the verifier's encoder memory
   float* part_val = nullptr;
   int* part_idx = nullptr;
   int* part_cnt = nullptr;   // relaxed verification: per tile and token, other tokens scoring above the draft
@@ -136,9 +137,12 @@ struct ad_handle {
   int* up_len = nullptr;
   int* up_max = nullptr;
   int* up_ovr = nullptr;
+  int* up_ids = nullptr;     // drafts or forced tokens [B, kmax]
+  int* up_n = nullptr;       // block sizes or commit counts [B]
+  int* in_max = nullptr;     // per-row caps of ad_generate as imported
+  int* dev_view(int* host) const { return host_flag_dev + (host - host_flag); }
   int* down = nullptr;       // result block of finalize_generate_kernel (host view) ...
   int* down_dev = nullptr;   // ... and its device view
-  bool defer_status = false; // ad_encode inside ad_generate: no synchronisation of its own
   // Decode loop: the accept kernel of one pass plans the pass behind it; next_pass is what the accept kernel being enqueued
   // shall plan (source < 0: nothing).
   NextPass next_pass = no_next_pass();
@@ -149,7 +153,12 @@ struct ad_handle {
   bool encoded = false;
   int last_vocab_which = -1;
   std::string err;
-  struct GraphEntry { cudaGraphExec_t exec; int launches; bool device_loop; };
+  struct GraphEntry {
+    cudaGraphExec_t exec;
+    int launches;        // kernels per replay (whole-call graph: per loop iteration)
+    bool device_loop;    // whole-call graph ...
+    int once;            // ... and its kernels outside the loop
+  };
   std::map<std::string, GraphEntry> graphs;
   std::map<std::tuple<int, int, int, int>, TcShape> tc_shapes;   // launch shapes by (pass kind, N, K, split)
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
@@ -299,7 +308,7 @@ size_t layout(ad_handle* h, void* base) {
   h->qbuf = bp.take(e * (size_t)M_all * d);
   h->ktmp = bp.take(e * (size_t)M_tmp * d);
   h->vtmp = bp.take(e * (size_t)M_tmp * d);
-  h->encmem = bp.take(e * (size_t)h->pass[PK_ENCODE].M_cap * d);
+  h->encmem.ptr = bp.take(e * (size_t)h->pass[PK_ENCODE].M_cap * d); h->encmem.cols = d;
   const size_t self_sz = e * (size_t)c.n_dec * B * c.max_tgt * d;
   h->kself = bp.take(self_sz);
   h->vself = bp.take(self_sz);
@@ -337,6 +346,7 @@ size_t layout(ad_handle* h, void* base) {
   h->max_pos = std::max(c.max_src, c.max_tgt + 1);
   h->pe = (float*)bp.take(sizeof(float) * (size_t)h->max_pos * d);
   h->ovr = (int*)bp.take(sizeof(int) * (size_t)B * c.max_tgt);
+  h->in_max = (int*)bp.take(sizeof(int) * (size_t)B, 256);
   for (int i = 0; i < 2; ++i) {
     h->mega_maps[i] = (CUtensorMap*)bp.take(sizeof(CUtensorMap) * (size_t)(6 * c.n_dec + 1));
     h->mega_layers[i] = (mega::LayerPtrs*)bp.take(sizeof(mega::LayerPtrs) * (size_t)c.n_dec);
@@ -356,7 +366,7 @@ size_t layout(ad_handle* h, void* base) {
   s.cross_base = ints(B);
   s.gidx = ints((size_t)B * c.kmax);
   s.enc_slot = ints((size_t)B * c.max_src);
-  s.user_k = ints(B); s.user_n = ints(B); s.user_drafts = ints((size_t)B * c.kmax);
+  s.user_k = ints(B); s.user_drafts = ints((size_t)B * c.kmax);
   return align_up(bp.off, 1024);
 }
 
@@ -685,7 +695,7 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   p.scale = 1.0f / sqrtf((float)dh);
   // Tensor-core kernels when there are thousands of queries or rows may hold hundreds of keys (max_keys: the capacity, known on
   // the host); the FFMA kernel spreads few queries and few keys over more CTAs.
-  if (h->bf16 && dh == 64 && (many || max_keys >= 256) && !(max_keys >= 256 && pc.seg_max <= 32)) {
+  if (h->bf16 && dh == 64 && (many || max_keys >= 256) && !(max_keys >= 256 && pc.seg_max <= 128)) {
     // Warps share a 16-query tile and split the keys (2 or 4 key groups) when rows have few queries; two groups also while
     // 64-query CTAs would not give every SM two.
     const long full = (long)h->dims.B * ((pc.seg_max + AM_Q - 1) / AM_Q) * c.n_heads;
@@ -750,7 +760,7 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   return AD_OK;
 }
 
-// Whether the few-query kernel (attention_few.cuh) serves an attention of pass pc: BF16, 64-wide heads, the keys within two
+// Whether the few-query kernel (attention_few.cuh) serves an attention of pass pc: BF16, 64-wide heads, the keys within four
 // rounds of its warps, and a grid of at most one wave.
 bool attention_is_few(const ad_handle* h, const PassCfg& pc, int max_keys) {
   const ad_model_cfg& c = h->cfg;
@@ -787,7 +797,7 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   note_launch(h, wq ? "q_proj+attention+out_proj" : "attention+out_proj");
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(h->dims.B * p.qchunks * split, c.n_heads); cfg.blockDim = dim3(32 * warps);
-  fp.rounds = max_keys > few::AK * warps ? 2 : 1;
+  fp.rounds = (max_keys + few::AK * warps - 1) / (few::AK * warps);
   cfg.dynamicSmemBytes = few::att_few_smem(warps, fp.rounds); cfg.stream = h->stream;
   cudaLaunchAttribute attr[2];
   int n_attr = 0;
@@ -807,8 +817,9 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   return AD_OK;
 }
 
-// y = LN(sum of the partial projections + bias + y)
-int layernorm(ad_handle* h, const PassCfg& pc, const Partials& pre, const float* bias, const float* g, const float* b) {
+// y = LN(sum of the partial projections + bias + y); the GEMM-operand copy goes to `out` (default yb).
+int layernorm(ad_handle* h, const PassCfg& pc, const Partials& pre, const float* bias, const float* g, const float* b,
+              const ActBuf* out = nullptr) {
   const int d = h->cfg.d_model;
   const LnParams p = {pc.plan.M, pre, bias, h->y, g, b, d, h->cfg.ln_eps, h->y};
   note_launch(h, "residual+layernorm");
@@ -819,7 +830,8 @@ int layernorm(ad_handle* h, const PassCfg& pc, const Partials& pre, const float*
     if (d > 512) return launch_k(layernorm_kernel<ActT, 256>, dim3(pc.M_cap), dim3(256), 0, h->stream, p, yb);
     return launch_k(layernorm_kernel<ActT, 128>, dim3(pc.M_cap), dim3(128), 0, h->stream, p, yb);
   };
-  const cudaError_t e = h->bf16 ? go((bf16*)h->yb.ptr) : go((float*)h->yb.ptr);
+  void* yb = out ? out->ptr : h->yb.ptr;
+  const cudaError_t e = h->bf16 ? go((bf16*)yb) : go((float*)yb);
   if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("layernorm launch: ") + cudaGetErrorString(e));
   return AD_OK;
 }
@@ -883,14 +895,14 @@ int self_attention_sublayer(ad_handle* h, int pk, const Mat& wqkv, const float* 
 }
 
 int ffn_sublayer(ad_handle* h, int pk, const Mat& w1, const float* b1, const Mat& w2, const float* b2, const float* lng,
-                 const float* lnb) {
+                 const float* lnb, const ActBuf* out = nullptr) {
   PassCfg& pc = h->pass[pk];
   GemmParams a = {};
   a.bias = b1; a.relu = 1; a.out_act = h->hbuf.ptr;
   AD_TRY(gemm(h, EPI_ACT, w1, h->yb, pk, pc.plan.M, pc.M_cap, a));
   Partials ps;
   AD_TRY(gemm_to_partials(h, w2, h->hbuf, pk, &ps));
-  return layernorm(h, pc, ps, b2, lng, lnb);
+  return layernorm(h, pc, ps, b2, lng, lnb, out);
 }
 
 
@@ -1081,15 +1093,13 @@ int encoder_pass(ad_handle* h, Model& m, bool keep_memory) {
   for (int l = 0; l < c.n_enc; ++l) {
     EncLayer& L = m.enc[l];
     AD_TRY(self_attention_sublayer(h, PK_ENCODE, L.wqkv, L.bqkv, L.wo, L.bo, L.ln1g, L.ln1b, h->ktmp, h->vtmp, l == 0 ? defer : nullptr));
-    AD_TRY(ffn_sublayer(h, PK_ENCODE, L.w1, L.b1, L.w2, L.b2, L.ln2g, L.ln2b));
+    AD_TRY(ffn_sublayer(h, PK_ENCODE, L.w1, L.b1, L.w2, L.b2, L.ln2g, L.ln2b, keep_memory && l + 1 == c.n_enc ? &h->encmem : nullptr));
   }
-  if (keep_memory)
-    AD_CUDA(h, cudaMemcpyAsync(h->encmem, h->yb.ptr, (size_t)pc.M_cap * c.d_model * h->esz, cudaMemcpyDeviceToDevice, h->stream));
   // cross-attention keys and values of every decoder layer in one launch (segments 2l / 2l + 1 = layer l's K / V)
   GemmParams p = {};
   p.bias = m.cbkv_pack; p.dst[0] = m.kenc; p.dst[1] = m.venc; p.seg_pair_stride = cross_layer;
   p.seg_width = c.d_model; p.n_direct = 0; p.slot = h->st.enc_slot;
-  AD_TRY(gemm(h, EPI_SCATTER, m.ckv_all, h->yb, PK_ENCODE, pc.plan.M, pc.M_cap, p));
+  AD_TRY(gemm(h, EPI_SCATTER, m.ckv_all, keep_memory ? h->encmem : h->yb, PK_ENCODE, pc.plan.M, pc.M_cap, p));
   return AD_OK;
 }
 
@@ -1127,9 +1137,12 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
   return AD_OK;
 }
 
-int prepare_verify(ad_handle* h, int source, int k_cap, const int* ovr, int ovr_len) {
+// user_drafts / user_k: where SRC_USER finds the caller's block (device, or mapped host memory); null: the workspace copies.
+int prepare_verify(ad_handle* h, int source, int k_cap, const int* ovr, int ovr_len, int* user_drafts = nullptr, int* user_k = nullptr) {
+  DevState st = h->st;
+  if (user_drafts) { st.user_drafts = user_drafts; st.user_k = user_k; }
   note_launch(h, "prepare_verify");
-  AD_CUDA(h, launch_k(prepare_verify_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_VERIFY].plan, h->dims, source, k_cap, ovr,
+  AD_CUDA(h, launch_k(prepare_verify_kernel, dim3(1), dim3(256), 0, h->stream, st, h->pass[PK_VERIFY].plan, h->dims, source, k_cap, ovr,
                                                  h->cfg.max_tgt, ovr_len));
   return AD_OK;
 }
@@ -1165,9 +1178,9 @@ int verify_stage(ad_handle* h, int auto_commit) {
   return vocab_stage(h, h->ar, h->yb, 0, auto_commit);
 }
 
-int commit_stage(ad_handle* h, const int* n_dev) {
+int commit_stage(ad_handle* h, const int* n_dev, int* status_out) {
   note_launch(h, "commit_stage");
-  AD_CUDA(h, launch_k(commit_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_VERIFY].plan, h->dims, n_dev));
+  AD_CUDA(h, launch_k(commit_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_VERIFY].plan, h->dims, n_dev, status_out));
   return AD_OK;
 }
 
@@ -1219,21 +1232,47 @@ int loop_iteration(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_l
   return verify_stage(h, 1);
 }
 
-int read_status(ad_handle* h) {
-  int s = 0;
-  AD_CUDA(h, cudaMemcpyAsync(&s, h->st.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+// Waits for the stream; `status`: the mapped word a kernel before has exported the latched device error to.
+int wait_status(ad_handle* h, volatile int* status) {
   AD_CUDA(h, cudaStreamSynchronize(h->stream));
-  if (s != 0) {
-    int z = 0;
-    cudaMemcpyAsync(h->st.status, &z, sizeof(int), cudaMemcpyHostToDevice, h->stream);
-    cudaStreamSynchronize(h->stream);
-    return fail(h, s, s == AD_ERR_TIMEOUT ? "a bounded device-side wait ran out" : "device-side argument check failed");
+  const int s = *status;
+  if (s != 0) return fail(h, s, s == AD_ERR_TIMEOUT ? "a bounded device-side wait ran out" : "device-side argument check failed");
+  return AD_OK;
+}
+int read_status(ad_handle* h) {
+  AD_CUDA(h, launch_k(export_status_kernel, dim3(1), dim3(32), 0, h->stream, h->st, h->dev_view(h->host_flag + 2)));
+  return wait_status(h, h->host_flag + 2);
+}
+
+// Runs `enqueue` (launches on the handle's stream whose arguments depend only on `key`) as a graph captured on first use;
+// directly where the stream cannot be captured or every launch is being timed.
+template <typename F>
+int run_captured(ad_handle* h, const char* key, F enqueue) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (h->stream != nullptr) cudaStreamIsCapturing(h->stream, &cap);
+  if (h->stream == nullptr || cap != cudaStreamCaptureStatusNone || !g_use_graph_encode || h->profiling) return enqueue();
+  auto it = h->graphs.find(key);
+  if (it == h->graphs.end()) {
+    cudaGraph_t g = nullptr;
+    const int before = h->launches;
+    AD_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+    const int rc = enqueue();
+    const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
+    const int n = h->launches - before;
+    h->launches = before;
+    if (rc != AD_OK) { if (g) cudaGraphDestroy(g); return rc; }
+    if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+    cudaGraphExec_t exec = nullptr;
+    const cudaError_t e2 = cudaGraphInstantiate(&exec, g, 0);
+    cudaGraphDestroy(g);
+    if (e2 != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e2));
+    it = h->graphs.emplace(key, ad_handle::GraphEntry{exec, n, false, 0}).first;
   }
+  AD_CUDA(h, cudaGraphLaunch(it->second.exec, h->stream));
+  h->launches += it->second.launches;
   return AD_OK;
 }
 
-cudaMemcpyKind to_dev(int on_host) { return on_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice; }
-cudaMemcpyKind from_dev(int on_host) { return on_host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice; }
 
 void drop_graphs(ad_handle* h) {
   for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second.exec);
@@ -1305,6 +1344,8 @@ extern "C" int ad_create(const ad_model_cfg* cfg, const ad_weights* w, void* wor
       for (int k = 0; k < PK_COUNT; ++k)
         for (int i = 0; i < 5 && (16 << i) <= h->pass[k].ntile; ++i)
           ok = ok && make_map(&b->map[k].m[i], b->ptr, h->M_all, b->cols, 16 << i);
+    for (int i = 0; i < 5 && (16 << i) <= h->pass[PK_ENCODE].ntile; ++i)
+      ok = ok && make_map(&h->encmem.map[PK_ENCODE].m[i], h->encmem.ptr, h->pass[PK_ENCODE].M_cap, h->encmem.cols, 16 << i);
     if (cfg->has_drafter) {
       const int Me = h->pass[PK_ENCODE].M_cap, nt = h->pass[PK_ENCODE].ntile;
       ActBuf* sbufs[3] = {&h->side.yb, &h->side.abuf, &h->side.hbuf};
@@ -1356,12 +1397,13 @@ extern "C" int ad_create(const ad_model_cfg* cfg, const ad_weights* w, void* wor
   }
   {
     const size_t B = cfg->max_batch;
-    const size_t n_up = B * cfg->max_src + 2 * B + B * cfg->max_tgt, n_down = 4 + 4 * B + B * cfg->max_tgt;
+    const size_t n_up = B * cfg->max_src + 3 * B + B * cfg->max_tgt + B * cfg->kmax, n_down = 4 + 4 * B + B * cfg->max_tgt;
     if (cudaHostAlloc(&h->host_flag, sizeof(int) * (16 + n_up + n_down), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer(&h->host_flag_dev, h->host_flag, 0) != cudaSuccess)
       return bail(AD_ERR_CUDA, "allocating pinned host memory failed");
     h->up_src = h->host_flag + 16; h->up_len = h->up_src + B * cfg->max_src; h->up_max = h->up_len + B;
-    h->up_ovr = h->up_max + B; h->down = h->up_ovr + B * cfg->max_tgt;
+    h->up_ovr = h->up_max + B; h->up_ids = h->up_ovr + B * cfg->max_tgt; h->up_n = h->up_ids + B * cfg->kmax;
+    h->down = h->up_n + B;
     h->down_dev = h->host_flag_dev + (h->down - h->host_flag);
   }
   if (cudaEventCreate(&h->ev0) != cudaSuccess || cudaEventCreate(&h->ev1) != cudaSuccess || cudaEventCreate(&h->ev2) != cudaSuccess)
@@ -1398,9 +1440,56 @@ extern "C" int ad_sync(ad_handle* h) {
   return read_status(h);
 }
 
-extern "C" int ad_encode(ad_handle* h, const int32_t* src, int32_t src_stride, const int32_t* src_len, int32_t B,
-                         int32_t on_host) {
-  if (!h) return AD_ERR_ARG;
+namespace {
+
+// What ad_encode and ad_generate import.  maxlen / ovr may be null; limit: iteration limit of the device-side loop (0: none).
+int import_inputs(ad_handle* h, const int32_t* src, int32_t src_stride, const int32_t* src_len, int32_t B, const int32_t* maxlen,
+                  const int32_t* ovr, int ovr_stride, int ovr_width, int limit, int on_host) {
+  const ad_model_cfg& c = h->cfg;
+  ImportParams p = {src, src_len, maxlen, ovr, src_stride, std::min(src_stride, c.max_src), ovr_stride, ovr_width, limit};
+  if (on_host) {
+    // host-resident inputs go through the handle's pinned staging area, which the device reads in place (every host-array
+    // call ends synchronised, so the area is free again)
+    for (int b = 0; b < B; ++b) memcpy(h->up_src + (size_t)b * c.max_src, src + (size_t)b * src_stride, sizeof(int) * p.src_width);
+    memcpy(h->up_len, src_len, sizeof(int) * B);
+    p.src = h->dev_view(h->up_src); p.src_len = h->dev_view(h->up_len); p.src_stride = c.max_src;
+    if (maxlen) { memcpy(h->up_max, maxlen, sizeof(int) * B); p.maxlen = h->dev_view(h->up_max); }
+    if (ovr) {
+      for (int b = 0; b < B; ++b) memcpy(h->up_ovr + (size_t)b * c.max_tgt, ovr + (size_t)b * ovr_stride, sizeof(int) * ovr_width);
+      p.ovr = h->dev_view(h->up_ovr); p.ovr_stride = c.max_tgt;
+    }
+  }
+  note_launch(h, "import");
+  AD_CUDA(h, launch_k(import_kernel, dim3(B), dim3(128), 0, h->stream, h->st, h->dims, p, h->in_max, h->ovr));
+  return AD_OK;
+}
+
+// Plan of the encoder pass (which also resets every row's decoding state), then the encoder pass(es).
+int encode_stage(ad_handle* h, bool with_maxlen) {
+  const ad_model_cfg& c = h->cfg;
+  note_launch(h, "plan_encode");
+  AD_CUDA(h, launch_k(plan_encode_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_ENCODE].plan, h->dims,
+                      (const int*)(with_maxlen ? h->in_max : nullptr)));
+  if (c.has_drafter && h->side_stream) {
+    // the two encoders are independent (Section 3.2: separate models): drafter's on the side stream, verifier's here
+    AD_CUDA(h, cudaEventRecord(h->ev_fork, h->stream));
+    AD_CUDA(h, cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));
+    swap_side(h);
+    const int rc_side = encoder_pass(h, h->nar, false);
+    cudaError_t e_join = rc_side == AD_OK ? cudaEventRecord(h->ev_join, h->stream) : cudaSuccess;
+    swap_side(h);
+    if (rc_side != AD_OK) return rc_side;
+    AD_CUDA(h, e_join);
+    AD_TRY(encoder_pass(h, h->ar, true));
+    AD_CUDA(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
+    return AD_OK;
+  }
+  AD_TRY(encoder_pass(h, h->ar, true));
+  if (c.has_drafter) AD_TRY(encoder_pass(h, h->nar, false));
+  return AD_OK;
+}
+
+int check_sources(ad_handle* h, const int32_t* src, int32_t src_stride, const int32_t* src_len, int32_t B, int32_t on_host) {
   const ad_model_cfg& c = h->cfg;
   if (!src || !src_len) return fail(h, AD_ERR_ARG, "src or src_len is null");
   if (B < 1 || B > c.max_batch) return fail(h, AD_ERR_CAPACITY, "B outside 1..max_batch");
@@ -1409,76 +1498,32 @@ extern "C" int ad_encode(ad_handle* h, const int32_t* src, int32_t src_stride, c
     for (int b = 0; b < B; ++b)
       if (src_len[b] < 1 || src_len[b] > c.max_src || src_len[b] > src_stride)
         return fail(h, src_len[b] > c.max_src ? AD_ERR_CAPACITY : AD_ERR_ARG, "src_len outside 1..min(max_src, src_stride)");
+  return AD_OK;
+}
+
+}  // namespace
+
+extern "C" int ad_encode(ad_handle* h, const int32_t* src, int32_t src_stride, const int32_t* src_len, int32_t B,
+                         int32_t on_host) {
+  if (!h) return AD_ERR_ARG;
+  AD_TRY(check_sources(h, src, src_stride, src_len, B, on_host));
   // (captured graphs are keyed by the batch size, so a different B simply uses other entries)
   h->B = B;
   h->dims.B = B;
   h->encoded = false;
-  const int w = src_stride < c.max_src ? src_stride : c.max_src;
-  if (on_host) {
-    // host-resident inputs go through the handle's pinned staging area (every host-array call ends synchronised, so
-    // the area is free again): one truly asynchronous copy each instead of driver-staged pageable copies
-    for (int b = 0; b < B; ++b) memcpy(h->up_src + (size_t)b * c.max_src, src + (size_t)b * src_stride, sizeof(int) * w);
-    memcpy(h->up_len, src_len, sizeof(int) * B);
-    AD_CUDA(h, cudaMemcpyAsync(h->st.src, h->up_src, sizeof(int) * (size_t)B * c.max_src, cudaMemcpyHostToDevice, h->stream));
-    AD_CUDA(h, cudaMemcpyAsync(h->st.srclen, h->up_len, sizeof(int) * B, cudaMemcpyHostToDevice, h->stream));
-  } else {
-    AD_CUDA(h, cudaMemcpy2DAsync(h->st.src, sizeof(int) * c.max_src, src, sizeof(int) * src_stride, sizeof(int) * w, B, cudaMemcpyDeviceToDevice, h->stream));
-    AD_CUDA(h, cudaMemcpyAsync(h->st.srclen, src_len, sizeof(int) * B, cudaMemcpyDeviceToDevice, h->stream));
-  }
+  AD_TRY(import_inputs(h, src, src_stride, src_len, B, nullptr, nullptr, 0, 0, 0, on_host));
   // The encoder pass reads its inputs from fixed workspace buffers, so on a capturable stream it is captured
   // once per batch size and replayed (about fifty launches otherwise paid on the host for every sentence).
-  auto enqueue = [&]() -> int {
-    note_launch(h, "ad_encode");
-    AD_CUDA(h, launch_k(plan_encode_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_ENCODE].plan, h->dims));
-    if (c.has_drafter && h->side_stream) {
-      // the two encoders are independent (Section 3.2: separate models): drafter's on the side stream, verifier's here
-      AD_CUDA(h, cudaEventRecord(h->ev_fork, h->stream));
-      AD_CUDA(h, cudaStreamWaitEvent(h->side_stream, h->ev_fork, 0));
-      swap_side(h);
-      const int rc_side = encoder_pass(h, h->nar, false);
-      cudaError_t e_join = rc_side == AD_OK ? cudaEventRecord(h->ev_join, h->stream) : cudaSuccess;
-      swap_side(h);
-      if (rc_side != AD_OK) return rc_side;
-      AD_CUDA(h, e_join);
-      AD_TRY(encoder_pass(h, h->ar, true));
-      AD_CUDA(h, cudaStreamWaitEvent(h->stream, h->ev_join, 0));
-      return AD_OK;
-    }
-    AD_TRY(encoder_pass(h, h->ar, true));
-    if (c.has_drafter) AD_TRY(encoder_pass(h, h->nar, false));
+  char key[48];
+  snprintf(key, sizeof(key), "encode B%d h%d", B, on_host ? 1 : 0);
+  AD_TRY(run_captured(h, key, [&]() -> int {
+    AD_TRY(encode_stage(h, false));
+    if (on_host) AD_CUDA(h, launch_k(export_status_kernel, dim3(1), dim3(32), 0, h->stream, h->st, h->dev_view(h->host_flag + 2)));
     return AD_OK;
-  };
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (h->stream != nullptr) cudaStreamIsCapturing(h->stream, &cap);
-  if (h->stream != nullptr && cap == cudaStreamCaptureStatusNone && g_use_graph_encode) {
-    char key[32];
-    snprintf(key, sizeof(key), "encode B%d", B);
-    auto it = h->graphs.find(key);
-    if (it == h->graphs.end()) {
-      cudaGraph_t g = nullptr;
-      const int before = h->launches;
-      AD_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-      const int rc = enqueue();
-      const cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-      const int n = h->launches - before;
-      h->launches = before;
-      if (rc != AD_OK) { if (g) cudaGraphDestroy(g); return rc; }
-      if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("encoder graph capture: ") + cudaGetErrorString(e));
-      cudaGraphExec_t exec = nullptr;
-      const cudaError_t e2 = cudaGraphInstantiate(&exec, g, 0);
-      cudaGraphDestroy(g);
-      if (e2 != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("encoder graph instantiate: ") + cudaGetErrorString(e2));
-      it = h->graphs.emplace(key, ad_handle::GraphEntry{exec, n, false}).first;
-    }
-    AD_CUDA(h, cudaGraphLaunch(it->second.exec, h->stream));
-    h->launches += it->second.launches;
-  } else {
-    AD_TRY(enqueue());
-  }
+  }));
   h->encoded = true;
   h->last_vocab_which = -1;
-  if (on_host && !h->defer_status) return read_status(h);
-  return AD_OK;
+  return on_host ? wait_status(h, h->host_flag + 2) : AD_OK;
 }
 
 extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_t* k, int32_t* argmax,
@@ -1491,14 +1536,34 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
   if (on_host)
     for (int b = 0; b < B; ++b)
       if (k[b] < 0 || k[b] > c.kmax) return fail(h, AD_ERR_ARG, "k outside 0..kmax");
-  AD_CUDA(h, cudaMemcpyAsync(h->st.user_drafts, drafts, sizeof(int) * (size_t)B * c.kmax, to_dev(on_host), h->stream));
-  AD_CUDA(h, cudaMemcpyAsync(h->st.user_k, k, sizeof(int) * B, to_dev(on_host), h->stream));
-  AD_TRY(prepare_verify(h, SRC_USER, c.kmax, nullptr, 0));
-  AD_TRY(verify_stage(h, 0));
+  // Captured once per batch size and acceptance rule: with host arrays the whole call (the block is read from, and the result
+  // written to, mapped host memory), with device arrays everything but the copies from and to the caller's arrays.
+  char key[96];
+  snprintf(key, sizeof(key), "verify B%d h%d b%d t%a", B, on_host ? 1 : 0, h->beta, (double)h->tau);
   if (on_host) {
-    if (argmax) AD_CUDA(h, cudaMemcpyAsync(argmax, h->st.pred, sizeof(int) * (size_t)B * c.kmax, cudaMemcpyDeviceToHost, h->stream));
-    if (n_accepted) AD_CUDA(h, cudaMemcpyAsync(n_accepted, h->st.n_acc, sizeof(int) * B, cudaMemcpyDeviceToHost, h->stream));
-    return read_status(h);
+    memcpy(h->up_ids, drafts, sizeof(int) * (size_t)B * c.kmax);
+    memcpy(h->up_n, k, sizeof(int) * B);
+  } else {
+    AD_CUDA(h, cudaMemcpyAsync(h->st.user_drafts, drafts, sizeof(int) * (size_t)B * c.kmax, cudaMemcpyDeviceToDevice, h->stream));
+    AD_CUDA(h, cudaMemcpyAsync(h->st.user_k, k, sizeof(int) * B, cudaMemcpyDeviceToDevice, h->stream));
+  }
+  AD_TRY(run_captured(h, key, [&]() -> int {
+    if (on_host) AD_TRY(prepare_verify(h, SRC_USER, c.kmax, nullptr, 0, h->dev_view(h->up_ids), h->dev_view(h->up_n)));
+    else AD_TRY(prepare_verify(h, SRC_USER, c.kmax, nullptr, 0));
+    AD_TRY(verify_stage(h, 0));
+    if (on_host) {
+      note_launch(h, "ad_verify_block");
+      AD_CUDA(h, launch_k(export_host_kernel, dim3(B), dim3(64), 0, h->stream, h->st, h->dims, h->pass[PK_VERIFY].plan, 0, h->down_dev));
+    }
+    return AD_OK;
+  }));
+  h->last_vocab_which = 0;
+  if (on_host) {
+    const int rc = wait_status(h, h->down);
+    if (rc == AD_ERR_CUDA) return rc;
+    if (argmax) memcpy(argmax, h->down + 4 + B, sizeof(int) * (size_t)B * c.kmax);
+    if (n_accepted) memcpy(n_accepted, h->down + 4, sizeof(int) * B);
+    return rc;
   }
   note_launch(h, "ad_verify_block");
   AD_CUDA(h, launch_k(export_block_kernel, dim3(B), dim3(64), 0, h->stream, h->st, h->dims, argmax, n_accepted, nullptr, nullptr, h->pass[PK_VERIFY].plan));
@@ -1508,26 +1573,30 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
 extern "C" int ad_commit(ad_handle* h, const int32_t* n, int32_t on_host) {
   if (!h) return AD_ERR_ARG;
   if (!h->encoded) return fail(h, AD_ERR_STATE, "ad_commit before ad_encode");
-  const int* n_dev = nullptr;
-  if (n) {
-    AD_CUDA(h, cudaMemcpyAsync(h->st.user_n, n, sizeof(int) * h->B, to_dev(on_host), h->stream));
-    n_dev = h->st.user_n;
+  const int* n_dev = n;
+  if (n && on_host) {
+    memcpy(h->up_n, n, sizeof(int) * h->B);
+    n_dev = h->dev_view(h->up_n);
   }
-  AD_TRY(commit_stage(h, n_dev));
-  if (on_host) return read_status(h);
-  return AD_OK;
+  AD_TRY(commit_stage(h, n_dev, on_host ? h->dev_view(h->host_flag + 2) : nullptr));
+  return on_host ? wait_status(h, h->host_flag + 2) : AD_OK;
 }
 
 extern "C" int ad_force_commit(ad_handle* h, const int32_t* tokens, const int32_t* n, int32_t on_host) {
   if (!h) return AD_ERR_ARG;
   if (!h->encoded) return fail(h, AD_ERR_STATE, "ad_force_commit before ad_encode");
   if (!tokens || !n) return fail(h, AD_ERR_ARG, "tokens or n is null");
-  AD_CUDA(h, cudaMemcpyAsync(h->st.user_drafts, tokens, sizeof(int) * (size_t)h->B * h->cfg.kmax, to_dev(on_host), h->stream));
-  AD_CUDA(h, cudaMemcpyAsync(h->st.user_n, n, sizeof(int) * h->B, to_dev(on_host), h->stream));
+  const int *tok_dev = tokens, *n_dev = n;
+  if (on_host) {
+    memcpy(h->up_ids, tokens, sizeof(int) * (size_t)h->B * h->cfg.kmax);
+    memcpy(h->up_n, n, sizeof(int) * h->B);
+    tok_dev = h->dev_view(h->up_ids);
+    n_dev = h->dev_view(h->up_n);
+  }
   note_launch(h, "ad_force_commit");
-  AD_CUDA(h, launch_k(force_commit_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_VERIFY].plan, h->dims, h->st.user_drafts, h->st.user_n));
-  if (on_host) return read_status(h);
-  return AD_OK;
+  AD_CUDA(h, launch_k(force_commit_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_VERIFY].plan, h->dims, tok_dev, n_dev,
+                      on_host ? h->dev_view(h->host_flag + 2) : nullptr));
+  return on_host ? wait_status(h, h->host_flag + 2) : AD_OK;
 }
 
 extern "C" int ad_draft_block(ad_handle* h, int32_t k_cap, int32_t* drafts, int32_t* k, int32_t on_host) {
@@ -1536,13 +1605,25 @@ extern "C" int ad_draft_block(ad_handle* h, int32_t k_cap, int32_t* drafts, int3
   if (!h->cfg.has_drafter) return fail(h, AD_ERR_STATE, "the handle has no drafter model");
   const ad_model_cfg& c = h->cfg;
   if (k_cap < 1 || k_cap > c.kmax) return fail(h, AD_ERR_ARG, "k_cap outside 1..kmax");
-  AD_TRY(plan_draft(h, k_cap));
-  AD_TRY(draft_stage(h));
   const int B = h->B;
+  char key[64];
+  snprintf(key, sizeof(key), "draft B%d h%d k%d", B, on_host ? 1 : 0, k_cap);
+  AD_TRY(run_captured(h, key, [&]() -> int {
+    AD_TRY(plan_draft(h, k_cap));
+    AD_TRY(draft_stage(h));
+    if (on_host) {
+      note_launch(h, "ad_draft_block");
+      AD_CUDA(h, launch_k(export_host_kernel, dim3(B), dim3(64), 0, h->stream, h->st, h->dims, h->pass[PK_VERIFY].plan, 1, h->down_dev));
+    }
+    return AD_OK;
+  }));
+  h->last_vocab_which = 1;
   if (on_host) {
-    if (drafts) AD_CUDA(h, cudaMemcpyAsync(drafts, h->st.drafts, sizeof(int) * (size_t)B * c.kmax, cudaMemcpyDeviceToHost, h->stream));
-    if (k) AD_CUDA(h, cudaMemcpyAsync(k, h->pass[PK_VERIFY].plan.seg_len, sizeof(int) * B, cudaMemcpyDeviceToHost, h->stream));
-    return read_status(h);
+    const int rc = wait_status(h, h->down);
+    if (rc == AD_ERR_CUDA) return rc;
+    if (drafts) memcpy(drafts, h->down + 4 + B, sizeof(int) * (size_t)B * c.kmax);
+    if (k) memcpy(k, h->down + 4, sizeof(int) * B);
+    return rc;
   }
   note_launch(h, "ad_draft_block");
   AD_CUDA(h, launch_k(export_block_kernel, dim3(B), dim3(64), 0, h->stream, h->st, h->dims, nullptr, nullptr, drafts, k, h->pass[PK_VERIFY].plan));
@@ -1557,6 +1638,56 @@ extern "C" int ad_get_state(ad_handle* h, int32_t* len, int32_t* last_tok, int32
   if (finished) AD_CUDA(h, cudaMemcpyAsync(finished, h->st.fin, sizeof(int) * h->B, cudaMemcpyDeviceToHost, h->stream));
   return read_status(h);
 }
+
+namespace {
+
+// ad_generate's device work as one graph: encoder pass(es), plan of the first pass, loop (see ad_generate).
+bool build_whole_graph(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_len, bool capped, ad_handle::GraphEntry* out) {
+  const int before = h->launches;
+  cudaGraph_t g = nullptr, dummy = nullptr;
+  cudaGraphConditionalHandle ch = 0;
+  std::vector<cudaGraphNode_t> tail;
+  bool ok = cudaGraphCreate(&g, 0) == cudaSuccess && cudaGraphConditionalHandleCreate(&ch, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+  if (ok && cudaStreamBeginCaptureToGraph(h->stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    ok = encode_stage(h, capped) == AD_OK;
+    ok = ok && cudaEventRecordWithFlags(h->ev1, h->stream, cudaEventRecordExternal) == cudaSuccess;   // an event node: end of the encoders
+    if (ok && loop_plans_ahead(h)) ok = plan_first_pass(h, o, ovr, ovr_len) == AD_OK;
+    cudaStreamCaptureStatus status;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t n = 0;
+    ok = ok && cudaStreamGetCaptureInfo_v2(h->stream, &status, nullptr, nullptr, &deps, &n) == cudaSuccess;
+    if (ok) tail.assign(deps, deps + n);
+    ok = cudaStreamEndCapture(h->stream, &dummy) == cudaSuccess && ok;
+  } else {
+    ok = false;
+  }
+  out->once = h->launches - before;
+  h->launches = before;
+  if (ok) {
+    cudaGraphNodeParams np = {cudaGraphNodeTypeConditional};
+    np.conditional.handle = ch;
+    np.conditional.type = cudaGraphCondTypeWhile;
+    np.conditional.size = 1;
+    cudaGraphNode_t node;
+    ok = cudaGraphAddNode(&node, g, tail.data(), tail.size(), &np) == cudaSuccess;
+    if (ok && cudaStreamBeginCaptureToGraph(h->stream, np.conditional.phGraph_out[0], nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+      h->cond_handle = (unsigned long long)ch;
+      ok = loop_iteration(h, o, ovr, ovr_len) == AD_OK;
+      h->cond_handle = 0;
+      ok = cudaStreamEndCapture(h->stream, &dummy) == cudaSuccess && ok;
+    } else {
+      ok = false;
+    }
+  }
+  out->launches = h->launches - before;
+  h->launches = before;
+  ok = ok && cudaGraphInstantiate(&out->exec, g, 0) == cudaSuccess;
+  if (g) cudaGraphDestroy(g);
+  out->device_loop = ok;
+  return ok;
+}
+
+}  // namespace
 
 extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride, const int32_t* src_len, int32_t B,
                            const ad_gen_opts* opts, int32_t* out, int32_t out_stride, int32_t* out_len,
@@ -1581,110 +1712,67 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
     }
   }
 
+  AD_TRY(check_sources(h, src, src_stride, src_len, B, on_host));
   AD_CUDA(h, cudaEventRecord(h->ev0, h->stream));
   h->launches = 0;
-  h->defer_status = true;       // the one synchronisation at the end of this call reports device-side errors
-  const int rc_enc = ad_encode(h, src, src_stride, src_len, B, on_host);
-  h->defer_status = false;
-  if (rc_enc != AD_OK) return rc_enc;
-  if (opts->max_len) {
-    const int* ml = opts->max_len;
-    if (on_host) { memcpy(h->up_max, opts->max_len, sizeof(int) * B); ml = h->up_max; }
-    AD_CUDA(h, cudaMemcpyAsync(h->st.user_n, ml, sizeof(int) * B, to_dev(on_host), h->stream));
-    note_launch(h, "ad_generate");
-    AD_CUDA(h, launch_k(set_maxlen_kernel, dim3((B + 63) / 64), dim3(64), 0, h->stream, h->st, h->dims, h->st.user_n));
-  }
-  const int* ovr = nullptr;
-  int ovr_len = 0;   // valid leading entries of each staged override row
-  if (opts->draft_override) {
-    ovr_len = opts->override_stride < c.max_tgt ? opts->override_stride : c.max_tgt;
-    if (on_host) {
-      for (int b = 0; b < B; ++b)
-        memcpy(h->up_ovr + (size_t)b * c.max_tgt, opts->draft_override + (size_t)b * opts->override_stride, sizeof(int) * ovr_len);
-      AD_CUDA(h, cudaMemcpyAsync(h->ovr, h->up_ovr, sizeof(int) * (size_t)B * c.max_tgt, cudaMemcpyHostToDevice, h->stream));
-    } else {
-      AD_CUDA(h, cudaMemcpy2DAsync(h->ovr, sizeof(int) * c.max_tgt, opts->draft_override, sizeof(int) * opts->override_stride,
-                                   sizeof(int) * ovr_len, B, cudaMemcpyDeviceToDevice, h->stream));
-    }
-    ovr = h->ovr;
-  }
-  AD_CUDA(h, cudaEventRecord(h->ev1, h->stream));
+  h->B = B;
+  h->dims.B = B;
+  h->encoded = false;
+  const int ovr_len = opts->draft_override ? std::min(opts->override_stride, c.max_tgt) : 0;   // valid leading entries of an override row
+  const int* ovr = opts->draft_override ? h->ovr : nullptr;
+  // (the data-independent bound on the iteration count of the device-side loop travels with the inputs)
+  AD_TRY(import_inputs(h, src, src_stride, src_len, B, opts->max_len, opts->draft_override, opts->override_stride, ovr_len, max_iters + 1, on_host));
+  const bool capped = opts->max_len != nullptr;
 
   cudaGraphExec_t exec = nullptr;
   int per_iter_launches = 0;
   bool device_loop = false;
   if (opts->use_graph && h->stream != nullptr) {   // the legacy default stream cannot be captured
     char key[160];
-    snprintf(key, sizeof(key), "B%d m%d k%d o%d v%d d%d b%d t%a", B, opts->mode, opts->k, ovr ? 1 : 0, ovr_len, opts->run_drafter,
-             h->beta, (double)h->tau);
+    snprintf(key, sizeof(key), "B%d m%d k%d o%d v%d d%d c%d b%d t%a", B, opts->mode, opts->k, ovr ? 1 : 0, ovr_len, opts->run_drafter,
+             capped ? 1 : 0, h->beta, (double)h->tau);
     auto it = h->graphs.find(key);
     if (it == h->graphs.end()) {
-      const int before = h->launches;
-      // First choice: the whole loop as one graph -- a device-side `while` node whose body is one iteration and
-      // whose condition the accept/commit kernel clears; no host round trip between iterations.
-      if (g_use_devloop) {
-        cudaGraph_t g = nullptr;
-        cudaGraphConditionalHandle ch = 0;
-        bool okb = cudaGraphCreate(&g, 0) == cudaSuccess &&
-                   cudaGraphConditionalHandleCreate(&ch, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
-        cudaGraphNodeParams np = {cudaGraphNodeTypeConditional};
-        np.conditional.handle = ch;
-        np.conditional.type = cudaGraphCondTypeWhile;
-        np.conditional.size = 1;
-        cudaGraphNode_t node;
-        okb = okb && cudaGraphAddNode(&node, g, nullptr, 0, &np) == cudaSuccess;
-        if (okb) {
-          cudaGraph_t body = np.conditional.phGraph_out[0];
-          okb = cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-          if (okb) {
-            h->cond_handle = (unsigned long long)ch;
-            const int rc = loop_iteration(h, *opts, ovr, ovr_len);
-            h->cond_handle = 0;
-            cudaGraph_t dummy = nullptr;
-            const cudaError_t e = cudaStreamEndCapture(h->stream, &dummy);
-            okb = rc == AD_OK && e == cudaSuccess;
-          }
-        }
-        per_iter_launches = h->launches - before;
-        h->launches = before;
-        if (okb) okb = cudaGraphInstantiate(&exec, g, 0) == cudaSuccess;
-        if (g) cudaGraphDestroy(g);
-        if (okb) {
-          h->graphs[key] = ad_handle::GraphEntry{exec, per_iter_launches, true};
-          device_loop = true;
-        } else {
-          exec = nullptr;
-          cudaGetLastError();   // clear; fall back to one replay per iteration
-        }
+      ad_handle::GraphEntry entry = {};
+      // First choice: the whole call as one graph -- encoder pass(es), plan of the first block, and a device-side `while` node
+      // whose body is one iteration and whose condition the accept/commit kernel clears; no host round trip between them.
+      if (g_use_devloop && !build_whole_graph(h, *opts, ovr, ovr_len, capped, &entry)) {
+        entry = ad_handle::GraphEntry{};
+        cudaGetLastError();   // clear; fall back to one replay per iteration
       }
-      if (!exec) {
+      if (!entry.exec) {
+        const int before = h->launches;
         cudaGraph_t g = nullptr;
         AD_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
         const int rc = loop_iteration(h, *opts, ovr, ovr_len);
         cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-        per_iter_launches = h->launches - before;
+        entry.launches = h->launches - before;
         h->launches = before;
         if (rc != AD_OK) { if (g) cudaGraphDestroy(g); return rc; }
         if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-        e = cudaGraphInstantiate(&exec, g, 0);
+        e = cudaGraphInstantiate(&entry.exec, g, 0);
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
-        h->graphs[key] = ad_handle::GraphEntry{exec, per_iter_launches, false};
       }
-    } else {
-      exec = it->second.exec;
-      per_iter_launches = it->second.launches;
-      device_loop = it->second.device_loop;
+      it = h->graphs.emplace(key, entry).first;
     }
+    exec = it->second.exec;
+    per_iter_launches = it->second.launches;
+    device_loop = it->second.device_loop;
+    if (device_loop) h->launches += it->second.once;
   }
 
-  if (loop_plans_ahead(h)) AD_TRY(plan_first_pass(h, *opts, ovr, ovr_len));
   if (device_loop) {
-    // one launch runs every iteration; the data-independent bound on the iteration count travels in loop_it[3]
-    h->host_flag[1] = max_iters + 1;
-    AD_CUDA(h, cudaMemcpyAsync(h->st.loop_it + 3, h->host_flag + 1, sizeof(int), cudaMemcpyHostToDevice, h->stream));
     AD_CUDA(h, cudaGraphLaunch(exec, h->stream));
+  } else {
+    char key[48];
+    snprintf(key, sizeof(key), "encode B%d c%d", B, capped ? 1 : 0);
+    AD_TRY(run_captured(h, key, [&]() -> int { return encode_stage(h, capped); }));
+    AD_CUDA(h, cudaEventRecord(h->ev1, h->stream));
+    if (loop_plans_ahead(h)) AD_TRY(plan_first_pass(h, *opts, ovr, ovr_len));
   }
+  h->encoded = true;
+  h->last_vocab_which = -1;
   const int sync_every = opts->sync_every > 0 ? opts->sync_every : 1;
   int iters = 0;
   volatile int* flag = h->host_flag;
@@ -1762,8 +1850,8 @@ extern "C" int ad_debug_encoder_memory(ad_handle* h, int32_t b, float* mem, size
   const size_t n = (size_t)len * h->cfg.d_model;
   if (n > capacity_elems) return fail(h, AD_ERR_CAPACITY, "memory buffer too small");
   const size_t start = (size_t)off * h->cfg.d_model;
-  if (h->bf16) to_f32_kernel<bf16><<<64, 256, 0, h->stream>>>((const bf16*)h->encmem + start, mem, n);
-  else to_f32_kernel<float><<<64, 256, 0, h->stream>>>((const float*)h->encmem + start, mem, n);
+  if (h->bf16) to_f32_kernel<bf16><<<64, 256, 0, h->stream>>>((const bf16*)h->encmem.ptr + start, mem, n);
+  else to_f32_kernel<float><<<64, 256, 0, h->stream>>>((const float*)h->encmem.ptr + start, mem, n);
   AD_CUDA(h, cudaGetLastError());
   return AD_OK;
 }

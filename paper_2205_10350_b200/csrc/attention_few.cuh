@@ -40,7 +40,7 @@ struct FewAttnParams {
   int rounds;           // rounds of keys the capacity may need
 };
 
-constexpr int MAX_ROUNDS = 2;     // rounds of AK keys per warp: all resident at once
+constexpr int MAX_ROUNDS = 4;     // rounds of AK keys per warp, all resident at once: 512 keys with eight warps (222 KB)
 inline size_t att_few_smem(int warps, int rounds) {
   const size_t kv = (size_t)rounds * warps * AK * (K_LD + V_LD) * sizeof(bf16);
   const size_t part = (size_t)warps * AQ * O_LD * sizeof(float);      // partial query projections, later partial outputs

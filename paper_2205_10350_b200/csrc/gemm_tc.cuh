@@ -159,6 +159,46 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 16 columns of each of `n` (1, 2 or 4) accumulator regions `stride` columns apart, added up in region order.  All loads are
+// in flight before the one wait: a tensor-memory round trip per region would be paid one after the other.
+__device__ __forceinline__ void tmem_issue16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+// (orders every use of r behind the wait)
+__device__ __forceinline__ void tmem_landed16(uint32_t (&r)[16]) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                    "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
+}
+__device__ __forceinline__ void tmem_sum16(uint32_t taddr, int n, uint32_t stride, float (&acc)[16]) {
+  uint32_t r[4][16];
+  tmem_issue16(taddr, r[0]);
+  if (n > 1) tmem_issue16(taddr + stride, r[1]);
+  if (n > 2) {
+    tmem_issue16(taddr + 2 * stride, r[2]);
+    tmem_issue16(taddr + 3 * stride, r[3]);
+  }
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  tmem_landed16(r[0]);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = __uint_as_float(r[0][i]);
+  if (n > 1) {
+    tmem_landed16(r[1]);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] += __uint_as_float(r[1][i]);
+  }
+  if (n > 2) {
+    tmem_landed16(r[2]);
+    tmem_landed16(r[3]);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = (acc[i] + __uint_as_float(r[2][i])) + __uint_as_float(r[3][i]);
+  }
+}
+
 // Order-preserving map from float to unsigned: a > b  <=>  key(a) > key(b) (no NaNs expected).
 __device__ __forceinline__ unsigned int float_key(float v) {
   const unsigned int u = __float_as_uint(v);
@@ -471,13 +511,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       if (ready) {
         for (int c = grp * 16; c < ntile && c < ntok_all; c += 32) {
           float acc[16];
-          tmem_ld16(tlane + static_cast<uint32_t>(c), acc);
-          for (int r = 1; r < n_issuers; ++r) {              // the other issuers' shares of the K range
-            float more[16];
-            tmem_ld16(tlane + static_cast<uint32_t>(r * ntile + c), more);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) acc[j] += more[j];
-          }
+          tmem_sum16(tlane + static_cast<uint32_t>(c), n_issuers, (uint32_t)ntile, acc);   // (the issuers' shares of the K range)
           // columns past the last valid token hold whatever the padded activation rows produced: never stored
 #pragma unroll
           for (int j = 0; j < 16; ++j) acc[j] = n < p.N ? acc[j] + bias_n : -INFINITY;
@@ -529,13 +563,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       if (tb > 0) __syncthreads();                         // previous pass has been read out
       for (int c = grp * 16; c < sub && c < ntok; c += 32) {
         float acc[16];
-        tmem_ld16(tlane + static_cast<uint32_t>(tb + c), acc);
-        for (int r = 1; r < n_issuers; ++r) {
-          float more[16];
-          tmem_ld16(tlane + static_cast<uint32_t>(r * ntile + tb + c), more);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) acc[j] += more[j];
-        }
+        tmem_sum16(tlane + static_cast<uint32_t>(tb + c), n_issuers, (uint32_t)ntile, acc);
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
           if (c + j < ntok) {

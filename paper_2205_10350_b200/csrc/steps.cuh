@@ -31,8 +31,7 @@ struct DevState {
   int* cross_base; // [B] = b * max_src
   int* gidx;       // [B * kmax] drafter: packed token holding mask position i of row b
   int* enc_slot;   // [B * max_src] encoder: cross-K/V slot of packed source token m
-  int* user_k;     // [B] staging of caller-provided k / n
-  int* user_n;     // [B]
+  int* user_k;     // [B] staging of caller-provided k
   int* user_drafts;// [B, kmax]
   unsigned int* sync_ctr;  // [128 x 32] per-stage arrival counters of the persistent decoder pass (one per 128-byte line);
                            // every planning kernel that precedes such a pass clears them
@@ -237,7 +236,7 @@ plan_draft_kernel(DevState st, PassPlan blk, PassPlan plan, Dims dm) {
 // key counts keep it out of every attention).  Also resets the decoding state of every row.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-plan_encode_kernel(DevState st, PassPlan plan, Dims dm) {
+plan_encode_kernel(DevState st, PassPlan plan, Dims dm, const int* maxlen) {
   pdl_wait();                  // (no pdl_launch: see plan data in ad_common.cuh)
   __shared__ int s_off[257];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -257,7 +256,10 @@ plan_encode_kernel(DevState st, PassPlan plan, Dims dm) {
     *st.all_fin = 0;
   }
   for (int b = tid; b < B; b += 256) {
-    st.len[b] = 0; st.last[b] = dm.bos; st.fin[b] = 0; st.n_acc[b] = 0; st.maxlen[b] = dm.max_tgt;
+    st.len[b] = 0; st.last[b] = dm.bos; st.fin[b] = 0; st.n_acc[b] = 0;
+    int ml = maxlen ? maxlen[b] : dm.max_tgt;
+    if (ml < 1 || ml > dm.max_tgt) { latch_error(st.status, AD_ERR_ARG); ml = max(1, min(ml, dm.max_tgt)); }
+    st.maxlen[b] = ml;
     st.stat_it[b] = 0; st.stat_acc[b] = 0; st.stat_off[b] = 0;
     st.cross_base[b] = b * dm.max_src;
   }
@@ -280,14 +282,29 @@ plan_encode_kernel(DevState st, PassPlan plan, Dims dm) {
   __threadfence();
 }
 
-__global__ void set_maxlen_kernel(DevState st, Dims dm, const int* maxlen) {
+// Inputs of a call into the workspace: sources, lengths, and for ad_generate per-row caps, the draft-override stream and the
+// iteration limit of the device-side loop.  The arrays are device memory or the handle's mapped pinned staging area, which is
+// read in place: one launch instead of a copy per array.  Null pointers: that input is not part of the call.
+// grid = B, block = 128.
+struct ImportParams {
+  const int* src;
+  const int* src_len;
+  const int* maxlen;
+  const int* ovr;
+  int src_stride, src_width, ovr_stride, ovr_width, limit;
+};
+__global__ void __launch_bounds__(128)
+import_kernel(DevState st, Dims dm, ImportParams p, int* maxlen_out, int* ovr_out) {
   pdl_launch();
   pdl_wait();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < dm.B) {
-    int v = maxlen[b];
-    if (v < 1 || v > dm.max_tgt) { latch_error(st.status, AD_ERR_ARG); v = max(1, min(v, dm.max_tgt)); }
-    st.maxlen[b] = v;
+  const int b = blockIdx.x, tid = threadIdx.x;
+  for (int i = tid; i < p.src_width; i += 128) st.src[(size_t)b * dm.max_src + i] = p.src[(size_t)b * p.src_stride + i];
+  if (p.ovr)
+    for (int i = tid; i < p.ovr_width; i += 128) ovr_out[(size_t)b * dm.max_tgt + i] = p.ovr[(size_t)b * p.ovr_stride + i];
+  if (tid == 0) {
+    st.srclen[b] = p.src_len[b];
+    if (p.maxlen) maxlen_out[b] = p.maxlen[b];
+    if (b == 0 && p.limit > 0) st.loop_it[3] = p.limit;
   }
 }
 
@@ -593,6 +610,16 @@ __device__ __forceinline__ void commit_row(const DevState& st, const PassPlan& b
   }
 }
 
+// Hands the latched status word to the host (mapped memory) and clears it.  One thread.
+__device__ __forceinline__ void export_status(const DevState& st, int* status_out) {
+  *status_out = atomicExch(st.status, 0);
+}
+__global__ void export_status_kernel(DevState st, int* status_out) {
+  pdl_launch();
+  pdl_wait();
+  if (threadIdx.x == 0) export_status(st, status_out);
+}
+
 // After every row has been committed: loop counter and the "all rows finished" word.  One thread.
 __device__ __forceinline__ void finish_iteration(const DevState& st, const Dims& dm, bool any_active) {
   int all = 1;
@@ -632,7 +659,7 @@ draft_score_kernel(DevState st, PassPlan blk, Dims dm, const WT* __restrict__ em
 // grid = 1, block = 256 (one warp per row at a time).
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-commit_kernel(DevState st, PassPlan blk, Dims dm, const int* n_in) {
+commit_kernel(DevState st, PassPlan blk, Dims dm, const int* n_in, int* status_out) {
   __shared__ int s_active;
   trace_mark(TR_COMMIT, 0);
   pdl_launch();
@@ -649,12 +676,15 @@ commit_kernel(DevState st, PassPlan blk, Dims dm, const int* n_in) {
     if (lane == 0 && nacc > 0) atomicOr(&s_active, 1);
   }
   __syncthreads();
-  if (threadIdx.x == 0) finish_iteration(st, dm, s_active != 0);
+  if (threadIdx.x == 0) {
+    finish_iteration(st, dm, s_active != 0);
+    if (status_out) export_status(st, status_out);
+  }
 }
 
 // Teacher-forced commit: the caller supplies the accepted tokens.  grid = 1, block = 256.
 __global__ void __launch_bounds__(256)
-force_commit_kernel(DevState st, PassPlan blk, Dims dm, const int* tokens, const int* n_in) {
+force_commit_kernel(DevState st, PassPlan blk, Dims dm, const int* tokens, const int* n_in, int* status_out) {
   pdl_launch();
   pdl_wait();
   for (int b = threadIdx.x; b < dm.B; b += 256) {
@@ -676,6 +706,8 @@ force_commit_kernel(DevState st, PassPlan blk, Dims dm, const int* tokens, const
     }
     st.n_acc[b] = 0;
   }
+  __syncthreads();
+  if (threadIdx.x == 0 && status_out) export_status(st, status_out);
 }
 
 // Copies the block results to caller-visible arrays (device pointers).  grid = B, block = 64.
@@ -691,6 +723,20 @@ __global__ void export_block_kernel(DevState st, Dims dm, int* argmax_out, int* 
   if (threadIdx.x == 0) {
     if (n_out) n_out[b] = st.n_acc[b];
     if (k_out) k_out[b] = blk.seg_len[b];
+  }
+}
+
+// The same into mapped host memory, for calls with host-resident arrays: block[0] = status word (cleared),
+// block[4 .. 4 + B) = n_accepted (drafts: block sizes), then [B, kmax] ids.  grid = B, block = 64.
+__global__ void export_host_kernel(DevState st, Dims dm, PassPlan blk, int drafts, int* block) {
+  pdl_launch();
+  pdl_wait();
+  const int b = blockIdx.x;
+  const int* ids = (drafts ? st.drafts : st.pred) + (size_t)b * dm.kmax;
+  for (int i = threadIdx.x; i < dm.kmax; i += blockDim.x) block[4 + dm.B + (size_t)b * dm.kmax + i] = ids[i];
+  if (threadIdx.x == 0) {
+    block[4 + b] = drafts ? blk.seg_len[b] : st.n_acc[b];
+    if (b == 0) export_status(st, block);
   }
 }
 
