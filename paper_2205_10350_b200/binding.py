@@ -342,23 +342,22 @@ class AggressiveDecoder:
 
 
 def vocab_argmax(x_t, emb_t, status_t=None):
-    """Operator-level call: arg-max of x @ emb^T per row.  x_t [M, d], emb_t [V, d], both float32 or bfloat16."""
+    """Operator-level call: arg-max of x @ emb^T per row.  x_t [M, d], emb_t [V, d], both float32 or bfloat16.
+    Returns when the result is complete."""
     import torch
     lib = load()
     M, d = x_t.shape
     V = emb_t.shape[0]
-    dtype = AD_DTYPE_BF16 if x_t.dtype == torch.bfloat16 else AD_DTYPE_FP32
+    dtype = AD_DTYPE_BF16 if x_t.dtype is torch.bfloat16 else AD_DTYPE_FP32
     nbytes = lib.ad_vocab_argmax_scratch_bytes(V, M)
     scratch = torch.empty(nbytes + 256, dtype=torch.uint8, device=x_t.device)
-    base = (scratch.data_ptr() + 255) // 256 * 256
     out = torch.empty(M, dtype=torch.int32, device=x_t.device)
-    rc = lib.ad_vocab_argmax(C.c_void_p(x_t.data_ptr()), C.c_void_p(emb_t.data_ptr()), dtype, M, d, V,
-                             C.c_void_p(out.data_ptr()), C.c_void_p(base), nbytes,
-                             C.c_void_p(status_t.data_ptr()) if status_t is not None else None,
-                             C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    stream = torch.cuda.current_stream()
+    rc = lib.ad_vocab_argmax(x_t.data_ptr(), emb_t.data_ptr(), dtype, M, d, V, out.data_ptr(), (scratch.data_ptr() + 255) // 256 * 256, nbytes,
+                             status_t.data_ptr() if status_t is not None else None, stream.cuda_stream)
     if rc != AD_OK:
         raise AdError(rc, "ad_vocab_argmax")
-    torch.cuda.synchronize()
+    stream.synchronize()
     return out
 
 
@@ -376,12 +375,9 @@ def vocab_argmax_static(x_t, emb_t, out_t, status_t=None):
     import torch
     lib = load()
     M, d = x_t.shape
-    V = emb_t.shape[0]
-    dtype = AD_DTYPE_BF16 if x_t.dtype == torch.bfloat16 else AD_DTYPE_FP32
-    rc = lib.ad_vocab_argmax_static(C.c_void_p(x_t.data_ptr()), C.c_void_p(emb_t.data_ptr()), dtype, M, d, V,
-                                    C.c_void_p(out_t.data_ptr()),
-                                    C.c_void_p(status_t.data_ptr()) if status_t is not None else None,
-                                    C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    dtype = AD_DTYPE_BF16 if x_t.dtype is torch.bfloat16 else AD_DTYPE_FP32
+    rc = lib.ad_vocab_argmax_static(x_t.data_ptr(), emb_t.data_ptr(), dtype, M, d, emb_t.shape[0], out_t.data_ptr(),
+                                    status_t.data_ptr() if status_t is not None else None, torch.cuda.current_stream().cuda_stream)
     if rc != AD_OK:
         msg = lib.ad_last_error(None)
         raise AdError(rc, msg.decode() if msg else "ad_vocab_argmax_static")
@@ -389,18 +385,17 @@ def vocab_argmax_static(x_t, emb_t, out_t, status_t=None):
 
 
 def linear(x_t, W_t, bias_t=None, status_t=None):
-    """Operator-level call: y = x W^T + bias in FP32.  x_t [M, K], W_t [N, K]."""
+    """Operator-level call: y = x W^T + bias in FP32.  x_t [M, K], W_t [N, K].  Returns when the result is complete."""
     import torch
     lib = load()
     M, K = x_t.shape
     N = W_t.shape[0]
-    dtype = AD_DTYPE_BF16 if x_t.dtype == torch.bfloat16 else AD_DTYPE_FP32
+    dtype = AD_DTYPE_BF16 if x_t.dtype is torch.bfloat16 else AD_DTYPE_FP32
     y = torch.empty((M, N), dtype=torch.float32, device=x_t.device)
-    rc = lib.ad_linear(C.c_void_p(x_t.data_ptr()), C.c_void_p(W_t.data_ptr()),
-                       C.c_void_p(bias_t.data_ptr()) if bias_t is not None else None, dtype, M, K, N,
-                       C.c_void_p(y.data_ptr()), C.c_void_p(status_t.data_ptr()) if status_t is not None else None,
-                       C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    stream = torch.cuda.current_stream()
+    rc = lib.ad_linear(x_t.data_ptr(), W_t.data_ptr(), bias_t.data_ptr() if bias_t is not None else None, dtype, M, K, N, y.data_ptr(),
+                       status_t.data_ptr() if status_t is not None else None, stream.cuda_stream)
     if rc != AD_OK:
         raise AdError(rc, "ad_linear")
-    torch.cuda.synchronize()
+    stream.synchronize()
     return y

@@ -557,18 +557,29 @@ template <int EPI, bool EMB = false>
 cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p, int ksplit, const few::EmbedParams& ep = {}) {
   const dim3 grid(p.N / few::FEAT, ksplit);
   const bf16 *w = (const bf16*)W.ptr, *xp = (const bf16*)x;
-  switch (p.K / ksplit / 256) {
+  const int nch = p.K / ksplit / 256;
+  if (few::wide_fits(p.N, nch)) {
+    const dim3 wgrid(p.N / few::W_FEAT, ksplit);
+    if (nch == 3) return launch_k(few::gemm_few_wide_kernel<EPI, 3, EMB>, wgrid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    return launch_k(few::gemm_few_wide_kernel<EPI, 4, EMB>, wgrid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+  }
+  switch (nch) {
     case 1: return launch_k(few::gemm_few_kernel<EPI, 1, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
     case 2: return launch_k(few::gemm_few_kernel<EPI, 2, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
     case 3: return launch_k(few::gemm_few_kernel<EPI, 3, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
     default: return launch_k(few::gemm_few_kernel<EPI, 4, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
   }
 }
+
 // Geometry rule of a projection of pass pc.  split: its consumer adds partial sums up.
 GeoRule geo_rule(const PassCfg& pc, int epi, int N, int K, bool split, bool has_bias) {
   GeoRule r = {N, K, pc.ntile, split ? pc.max_split : 1, num_sms(), 0, 0, 0};
   if (epi == EPI_F32 ? split : (epi != EPI_ARGMAX && has_bias)) r.few_split = few::split_for(N, K, split, pc.max_split);
-  if (r.few_split > 0) r.few_tokens = few::max_tokens(K / r.few_split / 256);
+  if (r.few_split > 0) {
+    const int nch = K / r.few_split / 256;
+    // (within a larger capacity a pass of few tokens runs the 16-feature form inside the tensor-core kernel)
+    r.few_tokens = pc.M_cap <= few::MAX_TOKENS && few::wide_fits(N, nch) ? few::MAX_TOKENS : few::max_tokens(nch);
+  }
   return r;
 }
 // Whether every projection of such a shape in pass pc runs on the few-token kernel.
@@ -587,7 +598,7 @@ cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const Gem
   }
   const int vec = p.K % 4 == 0 && (reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(x)) % 16 == 0;
   const dim3 grid((p.N + FEAT - 1) / FEAT, (M_cap + simt::TOK - 1) / simt::TOK);
-  return launch_k(simt::gemm_f32_kernel<EPI, FEAT>, grid, dim3(simt::GROUPS * FEAT), smem, st, (const float*)w, (const float*)x, p, vec);
+  return launch_k(simt::gemm_f32_kernel<EPI, FEAT>, grid, dim3(2 * FEAT), smem, st, (const float*)w, (const float*)x, p, vec);
 }
 // The few-token FP32 kernel: passes of at most kFewTokens tokens, shapes it covers.
 bool f32_few(const PassCfg& pc, int epi, int N, int K) { return pc.M_cap <= kFewTokens && epi != EPI_ARGMAX && simt::few_fits(N, K); }

@@ -32,8 +32,7 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Most tokens a pass may have for this kernel to be the faster one: two rounds.  (90 tokens of a 768-wide model, three rounds of
-// 32: 4.9 us a projection against 3.3 us on the tcgen05 kernel.)
+// Most tokens a pass may have for the 16-feature kernel: two rounds.
 inline int max_tokens(int nch) { return nch <= 2 ? MAX_TOKENS : 64; }
 // Tokens of one round trip: 64 while a warp's slice of K is 64 wide, 32 beyond (register budget of two CTAs per SM).
 __host__ __device__ constexpr int round_tokens(int nch) { return nch <= 2 ? 64 : 32; }
@@ -76,6 +75,47 @@ __device__ __forceinline__ uint4 embed8(const EmbedParams& ep, int tok, int pos,
     r[i] = *reinterpret_cast<const uint32_t*>(&h);
   }
   return make_uint4(r[0], r[1], r[2], r[3]);
+}
+
+// Four output features n .. n + 3 of token m: bias, activation, store.  slot: the token's K/V row (EPI_SCATTER).
+template <int EPI>
+__device__ __forceinline__ void few_store(const GemmParams& p, int kz, int M, int m, int n, float4 v, float4 bias, int slot) {
+  if (EPI == EPI_F32) {
+    *reinterpret_cast<float4*>(p.out_f32 + ((size_t)kz * M + m) * p.N + n) = v;
+    return;
+  }
+  v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
+  if (EPI == EPI_ACT && p.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
+  bf16* dst;
+  if (EPI == EPI_ACT) {
+    dst = reinterpret_cast<bf16*>(p.out_act) + (size_t)m * p.N + n;
+  } else {
+    const int seg = n / p.seg_width, col = n - seg * p.seg_width;
+    char* base = p.seg_pair_stride ? static_cast<char*>(p.dst[seg & 1]) + (size_t)(seg >> 1) * p.seg_pair_stride
+                                   : static_cast<char*>(p.dst[seg]);
+    dst = reinterpret_cast<bf16*>(base) + (size_t)(seg < p.n_direct ? m : slot) * p.seg_width + col;
+  }
+  __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
+  uint2 u;
+  u.x = *reinterpret_cast<unsigned int*>(&h0);
+  u.y = *reinterpret_cast<unsigned int*>(&h1);
+  *reinterpret_cast<uint2*>(dst) = u;
+}
+// The embedding as FP32 residual stream, tokens first, first + step, ...
+__device__ __forceinline__ void few_embed_y(const GemmParams& p, const EmbedParams& ep, int M, int first, int step) {
+  const int groups = p.K >> 2;
+  const size_t K = (size_t)p.K;
+  for (int m = first; m < M; m += step) {
+    const int tok = plan_load(ep.tok_id + m), pos = plan_load(ep.tok_pos + m);
+    for (int i = threadIdx.x; i < groups; i += THREADS) {
+      const uint2 e = __ldg(reinterpret_cast<const uint2*>(ep.emb + (size_t)tok * K + 4 * i));
+      const float4 pp = __ldg(reinterpret_cast<const float4*>(ep.pe + (size_t)pos * K + 4 * i));
+      float4 v;
+      v.x = __uint_as_float(e.x << 16) * ep.scale + pp.x; v.y = __uint_as_float(e.x & 0xffff0000u) * ep.scale + pp.y;
+      v.z = __uint_as_float(e.y << 16) * ep.scale + pp.z; v.w = __uint_as_float(e.y & 0xffff0000u) * ep.scale + pp.w;
+      *reinterpret_cast<float4*>(ep.y + (size_t)m * K + 4 * i) = v;
+    }
+  }
 }
 
 // Body of the kernel for the CTA of features 16 bx .. 16 bx + 15 and K part kz (K / ksplit = 256 * NCH).
@@ -155,43 +195,13 @@ __device__ __forceinline__ void few_body(const bf16* __restrict__ W, const bf16*
         const float4 o = *reinterpret_cast<const float4*>(&red[w][ot][of]);
         v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
       }
-      if (EPI == EPI_F32) {
-        *reinterpret_cast<float4*>(p.out_f32 + ((size_t)kz * M + m) * p.N + n0 + of) = v;
-      } else {
-        v.x += bias.x; v.y += bias.y; v.z += bias.z; v.w += bias.w;
-        if (EPI == EPI_ACT && p.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
-        bf16* dst;
-        if (EPI == EPI_ACT) {
-          dst = reinterpret_cast<bf16*>(p.out_act) + (size_t)m * p.N + n0 + of;
-        } else {                                             // a 16-feature tile lies inside one segment
-          const int seg = n0 / p.seg_width, col = n0 - seg * p.seg_width;
-          char* base = p.seg_pair_stride ? static_cast<char*>(p.dst[seg & 1]) + (size_t)(seg >> 1) * p.seg_pair_stride
-                                         : static_cast<char*>(p.dst[seg]);
-          if (t0 > 0) slot = plan_load(p.slot + m);
-          dst = reinterpret_cast<bf16*>(base) + (size_t)(seg < p.n_direct ? m : slot) * p.seg_width + col + of;
-        }
-        __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
-        uint2 u;
-        u.x = *reinterpret_cast<unsigned int*>(&h0);
-        u.y = *reinterpret_cast<unsigned int*>(&h1);
-        *reinterpret_cast<uint2*>(dst) = u;
-      }
+      if (EPI == EPI_SCATTER && t0 > 0) slot = plan_load(p.slot + m);
+      few_store<EPI>(p, kz, M, m, n0 + of, v, bias, slot);
     }
   }
   if (EMB) {
     if (M <= 0) pdl_wait();                                  // (a grid without work still ends after its predecessor)
-    const int groups = p.K >> 2;
-    for (int m = bx; m < M; m += p.N / FEAT) {
-      const int tok = plan_load(ep.tok_id + m), pos = plan_load(ep.tok_pos + m);
-      for (int i = tid; i < groups; i += THREADS) {
-        const uint2 e = __ldg(reinterpret_cast<const uint2*>(ep.emb + (size_t)tok * K + 4 * i));
-        const float4 pp = __ldg(reinterpret_cast<const float4*>(ep.pe + (size_t)pos * K + 4 * i));
-        float4 v;
-        v.x = __uint_as_float(e.x << 16) * ep.scale + pp.x; v.y = __uint_as_float(e.x & 0xffff0000u) * ep.scale + pp.y;
-        v.z = __uint_as_float(e.y << 16) * ep.scale + pp.z; v.w = __uint_as_float(e.y & 0xffff0000u) * ep.scale + pp.w;
-        *reinterpret_cast<float4*>(ep.y + (size_t)m * K + 4 * i) = v;
-      }
-    }
+    few_embed_y(p, ep, M, bx, p.N / FEAT);
   }
 }
 
@@ -203,6 +213,113 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, c
   trace_mark(TR_GEMM + EPI, 0);
   pdl_launch();
   few_body<EPI, NCH, EMB>(W, X, p, ep, blockIdx.x, blockIdx.y, plan_load(p.M_ptr), red);
+  trace_mark(TR_GEMM + EPI, 2);
+}
+
+// The same for wider slices of K (768 and 1024 per CTA), where 16 features per CTA leave the kernel bound by the activations it
+// re-reads (90 tokens of a 768-wide model: 192 CTAs x 138 KB, three dependent rounds, 4.9 us after the wait): 32 features per
+// CTA halve that traffic, one CTA per SM has the registers for the next round's activations to be in flight under this one.
+// grid = (N / 32, ksplit); block = 256.
+constexpr int W_FEAT = 32;
+constexpr int W_TOK = 32;
+constexpr int W_LD = W_FEAT + 4;
+inline bool wide_fits(int N, int nch) { return nch >= 3 && nch <= 4 && N % W_FEAT == 0; }
+template <int EPI, int NCH, bool EMB>
+__global__ void __launch_bounds__(THREADS, 1)
+gemm_few_wide_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, const EmbedParams ep) {
+  constexpr int NT = W_TOK / 8;
+  __shared__ __align__(16) float red[WARPS][W_TOK][W_LD];
+  trace_mark(TR_GEMM + EPI, 0);
+  pdl_launch();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int n0 = blockIdx.x * W_FEAT, kz = blockIdx.y;
+  const int kbase = kz * (256 * NCH) + warp * (32 * NCH) + 8 * t;
+  const size_t K = (size_t)p.K;
+  uint4 wa[2][NCH][2];
+#pragma unroll
+  for (int f = 0; f < 2; ++f)
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+      wa[f][c][0] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + 16 * f + g) * K + kbase + 32 * c));
+      wa[f][c][1] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + 16 * f + g + 8) * K + kbase + 32 * c));
+    }
+  const int of = (tid & 7) * 4, ot = tid >> 3;               // this thread's output: four features of one token per round
+  float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (EPI != EPI_F32) bias = *reinterpret_cast<const float4*>(p.bias + n0 + of);
+  const int M = plan_load(p.M_ptr);
+  int slot = 0;
+  if (EPI == EPI_SCATTER && ot < M) slot = plan_load(p.slot + ot);
+  auto load = [&](int t0, uint4 (&xb)[NT][NCH]) {
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+      if (t0 + 8 * nt < M) {
+        const int m = min(t0 + 8 * nt + g, M - 1);
+        if (EMB) {
+          const int tok = plan_load(ep.tok_id + m), pos = plan_load(ep.tok_pos + m);
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) xb[nt][c] = embed8(ep, tok, pos, p.K, kbase + 32 * c);
+        } else {
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) xb[nt][c] = *reinterpret_cast<const uint4*>(X + (size_t)m * K + kbase + 32 * c);
+        }
+      }
+    }
+  };
+  if (!EMB) pdl_wait();
+  trace_mark(TR_GEMM + EPI, 1);
+  uint4 xb[NT][NCH], xn[NT][NCH];
+  load(0, xb);
+  for (int t0 = 0; t0 < M; t0 += W_TOK) {
+    if (t0 + W_TOK < M) load(t0 + W_TOK, xn);
+    float acc[2][NT][4];
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) { acc[f][nt][0] = 0.f; acc[f][nt][1] = 0.f; acc[f][nt][2] = 0.f; acc[f][nt][3] = 0.f; }
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+#pragma unroll
+      for (int f = 0; f < 2; ++f)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+          mma16816(acc[f][nt], wa[f][c][0].x, wa[f][c][1].x, wa[f][c][0].y, wa[f][c][1].y, xb[nt][c].x, xb[nt][c].y);
+#pragma unroll
+      for (int f = 0; f < 2; ++f)
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+          mma16816(acc[f][nt], wa[f][c][0].z, wa[f][c][1].z, wa[f][c][0].w, wa[f][c][1].w, xb[nt][c].z, xb[nt][c].w);
+    }
+    if (t0 > 0) __syncthreads();                             // the previous round has been read out
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        float* r0 = &red[warp][8 * nt + 2 * t][16 * f + g];
+        r0[0] = acc[f][nt][0]; r0[W_LD] = acc[f][nt][1];
+        r0[8] = acc[f][nt][2]; r0[W_LD + 8] = acc[f][nt][3];
+      }
+    __syncthreads();
+    if (EMB && t0 == 0) pdl_wait();
+    const int m = t0 + ot;
+    if (m < M) {
+      float4 v = *reinterpret_cast<const float4*>(&red[0][ot][of]);
+#pragma unroll
+      for (int w = 1; w < WARPS; ++w) {
+        const float4 o = *reinterpret_cast<const float4*>(&red[w][ot][of]);
+        v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+      }
+      if (EPI == EPI_SCATTER && t0 > 0) slot = plan_load(p.slot + m);
+      few_store<EPI>(p, kz, M, m, n0 + of, v, bias, slot);
+    }
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) xb[nt][c] = xn[nt][c];
+  }
+  if (EMB) {
+    if (M <= 0) pdl_wait();                                  // (a grid without work still ends after its predecessor)
+    few_embed_y(p, ep, M, blockIdx.x, gridDim.x);
+  }
   trace_mark(TR_GEMM + EPI, 2);
 }
 

@@ -9,6 +9,7 @@
 #pragma once
 
 #include "ad_common.cuh"
+#include "gemm_tc.cuh"   // warp_argmax
 
 namespace ad {
 namespace simt {
@@ -20,7 +21,7 @@ constexpr int STAGES = 3;
 constexpr int ARGMAX_FEAT = 128;  // features per tile of the arg-max epilogue: the layout of the partial arrays
 
 template <int FEAT>
-constexpr size_t smem_bytes() { return sizeof(float) * (size_t)STAGES * (FEAT + TOK) * LDK; }
+constexpr size_t smem_bytes() { return sizeof(float) * (size_t)STAGES * (FEAT + TOK) * LDK; }   // (>= the partial sums)
 
 __device__ __forceinline__ void cp16(void* s, const void* g, bool there) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(s))), "l"(g),
@@ -46,27 +47,32 @@ __device__ __forceinline__ void store_out(const GemmParams& p, int n, int m, flo
   }
 }
 
+// A warp covers 64 features x 32 tokens, 8 x 8 outputs per lane; four warps per 64 features take every fourth quad of k and
+// their sums meet in shared memory at the end.  What bounds it: shared-memory wavefronts.  A 16-byte load costs a warp four of
+// them whatever it broadcasts, so a lane's tile decides: 8 x 8 spends 64 wavefronts on 256 FFMA instructions of a warp (64 SM
+// cycles), which balances; 8 x 4 spent 48 on 128 and took F32_OLD us for 333 x 512 x 2048 (F32_NEW us now, back to back).
 // grid = (ceil(N / FEAT), ceil(M_cap / 32)); block = 2 FEAT; dynamic smem smem_bytes<FEAT>().  x: [M_cap, K], w: [N, K].
-// A thread has 8 features x 4 tokens (twelve 16-byte shared loads for 128 FFMA); FEAT threads make up such a tile, and the two
-// groups of them take alternate quads of k, so that an SM has enough warps for its FFMA pipes although the tiles are few.  vec: K is a multiple of four and both operands are 16-byte aligned.
-constexpr int GROUPS = 2;
+// vec: K is a multiple of four and both operands are 16-byte aligned.
+constexpr int GROUPS = 4;
+constexpr int SUM_LD = 33;
 template <int EPI, int FEAT>
-__global__ void __launch_bounds__(GROUPS * FEAT)
+__global__ void __launch_bounds__(2 * FEAT, FEAT == 64 ? 3 : 1)
 gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p, const int vec) {
-  constexpr int TX = FEAT / 8;                         // thread (tx, ty): features tx + TX i (i < 8), tokens ty + 8 j (j < 4)
-  constexpr int THREADS = GROUPS * FEAT;
+  constexpr int THREADS = 2 * FEAT;
   constexpr int RSTEP = THREADS / (KT / 4);            // rows between a thread's 16-byte copies: FEAT / RSTEP of W, then of x
   constexpr int NW = FEAT / RSTEP, NX = TOK / RSTEP;
-  extern __shared__ __align__(16) float simt_smem[];   // [STAGES][FEAT + TOK][LDK], later [GROUPS][32][FEAT] partial sums
+  extern __shared__ __align__(16) float simt_smem[];   // [STAGES][FEAT + TOK][LDK], later [warps][64][SUM_LD] partial sums
   const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
   const int t0 = blockIdx.y * TOK, n0 = blockIdx.x * FEAT;
   pdl_launch();
   if (t0 >= M && (blockIdx.x | blockIdx.y) > 0) return;
   pdl_wait();
   if (t0 >= M) return;
-  const int tid = threadIdx.x, grp = tid / FEAT, tt = tid % FEAT, tx = tt % TX, ty = tt / TX;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int grp = warp % GROUPS, half = warp / GROUPS;               // share of k; 64-feature part of the tile
+  const int tx = lane & 7, ty = lane >> 3;                           // features tx + 8 i, tokens ty + 4 j (i, j < 8)
   const int K = p.K, nk = (K + KT - 1) / KT;
-  const int fr = tid / (KT / 4), fc = (tid % (KT / 4)) * 4;      // first row and k of this thread's 16-byte copies
+  const int fr = tid / (KT / 4), fc = (tid % (KT / 4)) * 4;          // first row and k of this thread's 16-byte copies
   const float *wsrc = w + (size_t)(n0 + fr) * K + fc, *xsrc = x + (size_t)(t0 + fr) * K + fc;
   auto fetch = [&](int kt) {
     float* dst = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK;
@@ -96,84 +102,79 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  float acc[8][4];
+  float acc[8][8];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
 #pragma unroll
   for (int s = 0; s < STAGES - 1; ++s) fetch(s);
   for (int kt = 0; kt < nk; ++kt) {
     asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
     __syncthreads();                                    // stage kt has landed, stage kt - 1 is free
     fetch(kt + STAGES - 1);
-    const float* ws = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + tx * LDK + 4 * grp;
+    const float* ws = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + (half * 64 + tx) * LDK + 4 * grp;
     const float* xs = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + (FEAT + ty) * LDK + 4 * grp;
 #pragma unroll
     for (int k = 0; k < KT; k += 4 * GROUPS) {
-      float4 a[8], b[4];
+      float4 a[8], b[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4*>(ws + i * TX * LDK + k);
+      for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4*>(ws + i * 8 * LDK + k);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(xs + j * 8 * LDK + k);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+      for (int j = 0; j < 8; ++j) b[j] = *reinterpret_cast<const float4*>(xs + j * 4 * LDK + k);
 #pragma unroll
       for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
 #pragma unroll
       for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
 #pragma unroll
       for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
     }
   }
   // the groups' sums meet in shared memory
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  float* sums = simt_smem;
+  float* sums = simt_smem + (size_t)warp * 64 * SUM_LD + lane;
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) sums[(size_t)(grp * 32 + i * 4 + j) * FEAT + tt] = acc[i][j];
+    for (int j = 0; j < 8; ++j) sums[(i * 8 + j) * SUM_LD] = acc[i][j];
   __syncthreads();
-  if (EPI == EPI_ARGMAX) {
-    // the first group finishes: the TX threads of a token are neighbours and hold its FEAT features; lowest id on ties
-    if (grp > 0) return;
-    const int lane = tid & 31;
+  auto sum_of = [&](int f, int tok) {                   // output (feature f, token tok) of the tile
+    const float* q = simt_smem + (size_t)(f / 64) * GROUPS * 64 * SUM_LD + ((f % 64) / 8 * 8 + tok / 4) * SUM_LD + (tok % 4) * 8 + f % 8;
+    float v = q[0];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int m = t0 + ty + 8 * j;
-      const bool on = m < M;
+    for (int g = 1; g < GROUPS; ++g) v += q[(size_t)g * 64 * SUM_LD];
+    return v;
+  };
+  if (EPI == EPI_ARGMAX) {
+    for (int tok = warp; tok < TOK && t0 + tok < M; tok += THREADS / 32) {       // a warp per token; lowest id on ties
+      const int m = t0 + tok;
       float v = -INFINITY;
       int id = 0x7fffffff, cnt = 0;
-      const float dval = p.draft_val && on ? p.draft_val[m] : 0.f;
-      const int did = p.draft_val && on ? p.draft_id[m] : -1;
+      const float dval = p.draft_val ? p.draft_val[m] : 0.f;
+      const int did = p.draft_val ? p.draft_id[m] : -1;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int n = n0 + tx + TX * i;
+      for (int f = lane; f < FEAT; f += 32) {
+        const int n = n0 + f;
         if (n < p.N) {
-          float s = 0.f;
-#pragma unroll
-          for (int q = 0; q < GROUPS; ++q) s += sums[(size_t)(q * 32 + i * 4 + j) * FEAT + tt];
+          const float s = sum_of(f, tok);
           if (s > v) { v = s; id = n; }
           if (p.draft_val && n != did && s > dval) ++cnt;           // other features that score strictly higher
         }
       }
-#pragma unroll
-      for (int o = TX / 2; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, id, o);
-        if (ov > v || (ov == v && oi < id)) { v = ov; id = oi; }
-        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-      }
-      if ((lane & (TX - 1)) == 0 && on) {
+      tc::warp_argmax(v, id);
+      if (p.draft_val) cnt = __reduce_add_sync(0xffffffffu, cnt);
+      if (lane == 0) {
         const size_t o = (size_t)m * gridDim.x + blockIdx.x;
         p.part_val[o] = v;
         p.part_idx[o] = id;
@@ -184,12 +185,7 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
     // output (token, feature): neighbouring threads take neighbouring features
     for (int idx = tid; idx < FEAT * TOK; idx += THREADS) {
       const int f = idx % FEAT, tok = idx / FEAT, n = n0 + f, m = t0 + tok;
-      if (n >= p.N || m >= M) continue;
-      const int e = (f / TX) * 4 + tok / 8, th = (tok % 8) * TX + f % TX;
-      float s = p.bias ? p.bias[n] : 0.f;
-#pragma unroll
-      for (int q = 0; q < GROUPS; ++q) s += sums[(size_t)(q * 32 + e) * FEAT + th];
-      store_out<EPI>(p, n, m, s);
+      if (n < p.N && m < M) store_out<EPI>(p, n, m, sum_of(f, tok) + (p.bias ? p.bias[n] : 0.f));
     }
   }
 }
