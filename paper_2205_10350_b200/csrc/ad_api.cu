@@ -546,8 +546,8 @@ cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw, cons
   }
   const int kb = p.K / tc::BLOCK_K;
   const int stages = clampi((kSmemLimit - 1024 - kb * tc::P_A_KB_BYTES) / tc::P_B_STAGE_BYTES, 1, tc::P_MAX_STAGES);
-  const long pairs = (long)((p.N + tc::P_VOC - 1) / tc::P_VOC) * ((M_cap + tc::P_TOK - 1) / tc::P_TOK);
-  const int grid = (int)std::min<long>(pairs, num_sms());
+  const long units = (long)((p.N + tc::BLOCK_N_FEAT - 1) / tc::BLOCK_N_FEAT) * ((M_cap + tc::P_TOK - 1) / tc::P_TOK);
+  const int grid = (int)std::min<long>(units, num_sms());
   return launch_k(tc::vocab_argmax_persistent_kernel, dim3(grid), dim3(tc::P_THREADS), tc::vocab_persistent_smem(kb, stages), st, mw, mx128, p,
                   stages);
 }

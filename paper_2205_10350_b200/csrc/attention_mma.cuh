@@ -299,7 +299,8 @@ attention_mma_kernel(const AttnParams p, const int kv_old) {
 // plan (cross-attention: the encoder wrote them) they are copied before the dependency wait, off the critical path.  
 //
 // What bounds it: with few queries latency (one round trip for the queries, two tiles per warp, one merge), with an encoder
-// pass's thousands the warp instructions of the softmax.  400 keys, 8 rows: AL_TIMES
+// pass's thousands the warp instructions of the softmax.  The cross-attention of 8 rows x 25 queries over 400 keys took
+// 6.1-6.9 us after the wait with the kernel before (whole tiles per warp too, 4-byte key fragments, keys after the wait: 8 us).
 //
 // grid = (B * qchunks, H), qchunks = ceil(longest segment / (16 QT)); block = 32 QT NW threads; dynamic shared memory =
 // slots * AL_TILE_BYTES + 16 QT rows of queries (att_long_smem).

@@ -50,7 +50,7 @@ __device__ __forceinline__ void store_out(const GemmParams& p, int n, int m, flo
 // A warp covers 64 features x 32 tokens, 8 x 8 outputs per lane; four warps per 64 features take every fourth quad of k and
 // their sums meet in shared memory at the end.  What bounds it: shared-memory wavefronts.  A 16-byte load costs a warp four of
 // them whatever it broadcasts, so a lane's tile decides: 8 x 8 spends 64 wavefronts on 256 FFMA instructions of a warp (64 SM
-// cycles), which balances; 8 x 4 spent 48 on 128 and took F32_OLD us for 333 x 512 x 2048 (F32_NEW us now, back to back).
+// cycles), which balances; 8 x 4 spent 48 on 128 and took 34 us for 333 x 512 x 2048 (27 us now, back to back).
 // grid = (ceil(N / FEAT), ceil(M_cap / 32)); block = 2 FEAT; dynamic smem smem_bytes<FEAT>().  x: [M_cap, K], w: [N, K].
 // vec: K is a multiple of four and both operands are 16-byte aligned.
 constexpr int GROUPS = 4;

@@ -352,6 +352,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   const int stages = ring_stages(ntile, num_kb, budget);
   const int first_round = num_kb < stages ? num_kb : stages;
 
+  // Arg-max over a 128-token tile: the tokens are the MMA's M side (one token per tensor-memory lane, one vocabulary row per
+  // column), so that the arg-max is a scan over a thread's own columns.  With the weights on the M side the exchange between
+  // lanes takes 2.2 us of a CTA's 12 us at 90 tokens x 768.
+  const bool token_major = EPI == EPI_ARGMAX && ntile == 128 && !p.bias;
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzled tiles need 1024-byte alignment
   // MMA issuers.  Issuing one tcgen05.mma costs its thread 65-80 cycles whatever the tile, so with few tokens (short
   // MMAs) a single issuer, not the tensor pipe or shared memory, sets the pace of the K loop.  Up to four threads in
@@ -459,8 +463,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       const int j = warp - 4;
       const uint32_t idesc = make_idesc(BLOCK_N_FEAT, ntile);
       const uint32_t acc_j = tmem_acc + (uint32_t)(j * ntile);
-      const uint64_t desc_a0 = make_smem_desc(smem_base);
-      const uint64_t desc_b0 = make_smem_desc(smem_base + A_STAGE_BYTES);
+      const uint64_t desc_a0 = make_smem_desc(token_major ? smem_base + A_STAGE_BYTES : smem_base);
+      const uint64_t desc_b0 = make_smem_desc(token_major ? smem_base : smem_base + A_STAGE_BYTES);
       const uint64_t desc_step = (uint64_t)(stage_bytes >> 4);     // stage stride in the (address >> 4) field
       bool ok = true;
       int s = j % stages;
@@ -508,7 +512,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       int* red_idx = reinterpret_cast<int*>(stage + 4 * 256);   // [4][ntile]
       int* red_cnt = reinterpret_cast<int*>(stage + 8 * 256);   // [4][ntile] features scoring above the draft
       const bool relaxed = p.draft_val != nullptr;
-      if (ready) {
+      if (ready && token_major) {
+        const int tok = quad * 32 + lane;
+        const float dval = relaxed ? dval_s[tok] : 0.f;
+        const int did = relaxed ? did_s[tok] : -1;
+        float best = -INFINITY;
+        int best_n = 0x7fffffff, cnt = 0;
+        if (quad * 32 < ntok_all) {
+          for (int c = grp * 64; c < grp * 64 + 64; c += 16) {
+            float acc[16];
+            tmem_sum16(tlane + static_cast<uint32_t>(c), n_issuers, (uint32_t)ntile, acc);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const int nn = n0 + c + j;
+              const float val = nn < p.N ? acc[j] : -INFINITY;       // rows beyond the vocabulary were zero-filled
+              if (relaxed) cnt += (nn != did && val > dval) ? 1 : 0;
+              if (val > best) { best = val; best_n = nn; }
+            }
+          }
+        }
+        red_val[grp * ntile + tok] = best;
+        red_idx[grp * ntile + tok] = best_n;
+        if (relaxed) red_cnt[grp * ntile + tok] = cnt;
+      } else if (ready) {
         for (int c = grp * 16; c < ntile && c < ntok_all; c += 32) {
           float acc[16];
           tmem_sum16(tlane + static_cast<uint32_t>(c), n_issuers, (uint32_t)ntile, acc);   // (the issuers' shares of the K range)
@@ -541,16 +567,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       for (int t = threadIdx.x; t < ntok_all && ready; t += THREADS) {
         float v = red_val[t];
         int idx = red_idx[t];
-#pragma unroll
-        for (int w = 1; w < 4; ++w) {
+        const int parts = token_major ? 2 : 4;
+        for (int w = 1; w < parts; ++w) {
           const float ov = red_val[w * ntile + t];
           if (ov > v) { v = ov; idx = red_idx[w * ntile + t]; }
         }
         p.part_val[(size_t)(t0 + t) * nf + fx] = v;
         p.part_idx[(size_t)(t0 + t) * nf + fx] = idx;
-        if (relaxed)
-          p.part_cnt[(size_t)(t0 + t) * nf + fx] =
-              red_cnt[t] + red_cnt[ntile + t] + red_cnt[2 * ntile + t] + red_cnt[3 * ntile + t];
+        if (relaxed) {
+          int cnt = 0;
+          for (int w = 0; w < parts; ++w) cnt += red_cnt[w * ntile + t];
+          p.part_cnt[(size_t)(t0 + t) * nf + fx] = cnt;
+        }
       }
     }
     // Other epilogues: the tile is transposed through shared memory into rows of 128 features per token, in

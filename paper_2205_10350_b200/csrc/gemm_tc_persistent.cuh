@@ -6,14 +6,17 @@
 // one vocabulary row per column.  The arg-max over vocabulary rows is then a scan over a thread's own columns: no
 // exchange between lanes, no shared memory, no barrier.
 //
-// One CTA per SM owns a contiguous range of (token tile, vocabulary tile) pairs, the vocabulary tile running fastest:
-// 128 tokens x 256 vocabulary rows per pair.  The token tile (128 x K BF16, K <= 512) stays in shared memory for all of
-// its pairs; only vocabulary rows stream through the ring, 8 bytes of L2 traffic per output instead of 12.  Roles (512
-// threads):
-//   warps 8 .. 8+S-1, lane 0: producers of the vocabulary ring, one stage each (two 128-row boxes per stage);
-//   warp 14, lane 0:          loads the resident token tile whenever the range moves on to the next token tile;
+// One CTA per SM owns a contiguous range of (token tile, 128-row vocabulary tile) units, the vocabulary tile running fastest, and
+// takes them two at a time (128 tokens x 256 vocabulary rows; one unit where the range or the vocabulary ends).  The token tile
+// (128 x K BF16, K <= 512) stays in shared memory for all of its units; only vocabulary rows stream through the ring, 8 bytes
+// of L2 traffic per output instead of 12.  Roles (512 threads):
+//   warps 8 .. 8+S-1, lane 0: producers of the vocabulary ring, one stage each (two 128-row boxes per stage); inside a
+//                             pass the weights never change and are requested before the dependency wait;
+//   warps 8+S .. 14, lane 0:  load the resident token tile whenever the range moves on to the next token tile, K blocks dealt
+//                             to them (one thread's copies run one after the other: 128 KB by one thread took 2 us), a barrier
+//                             per K block so that the MMAs follow the copies;
 //   warp 15, lane 0:          MMA issuer; the accumulator alternates between two 256-column halves of tensor memory, so
-//                             the K loop of pair i + 1 runs while pair i is read out;
+//                             the K loop of step i + 1 runs while step i is read out;
 //   warps 0-7:                read-out: warp w owns the 32 tokens of lane quadrant w % 4 and the 128 columns w / 4 of
 //                             the half, i.e. one 128-row vocabulary tile of the partial arrays; each thread scans its
 //                             columns in ascending row order (strict comparison: lowest id wins ties) and writes the
@@ -21,6 +24,8 @@
 // Every mbarrier wait is bounded in time; a wait that runs out latches AD_ERR_TIMEOUT, raises the CTA's abort flag and
 // every role leaves its loop.  No role waits at a block-wide barrier inside the loops.
 #pragma once
+
+#include <type_traits>
 
 #include "gemm_tc.cuh"
 
@@ -45,7 +50,7 @@ inline size_t vocab_persistent_smem(int kb, int stages) {
   return (size_t)kb * P_A_KB_BYTES + (size_t)stages * P_B_STAGE_BYTES + 1024;
 }
 
-// grid = min(SMs, pairs); block = 512 threads; dynamic smem = vocab_persistent_smem(K / 64, stages).
+// grid = min(SMs, units); block = 512 threads; dynamic smem = vocab_persistent_smem(K / 64, stages).
 // map_x: box of 128 token rows x 64; map_w: box of 128 vocabulary rows x 64.  p.bias must be null.
 __global__ void __launch_bounds__(P_THREADS, 1)
 vocab_argmax_persistent_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x,
@@ -53,7 +58,7 @@ vocab_argmax_persistent_kernel(const __grid_constant__ CUtensorMap map_w, const 
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_full[P_MAX_STAGES];
   __shared__ __align__(8) uint64_t bar_empty[P_MAX_STAGES];
-  __shared__ __align__(8) uint64_t a_full, a_empty;
+  __shared__ __align__(8) uint64_t a_full[P_MAX_KB], a_empty;
   __shared__ __align__(8) uint64_t acc_full[2];
   __shared__ __align__(8) uint64_t acc_empty[2];
   __shared__ uint32_t tmem_base_slot;
@@ -72,7 +77,7 @@ vocab_argmax_persistent_kernel(const __grid_constant__ CUtensorMap map_w, const 
       mbar_init(smem_u32(&bar_full[s]), 1);
       mbar_init(smem_u32(&bar_empty[s]), 1);
     }
-    mbar_init(smem_u32(&a_full), 1);
+    for (int kb = 0; kb < KB; ++kb) mbar_init(smem_u32(&a_full[kb]), 1);
     mbar_init(smem_u32(&a_empty), 1);
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&acc_full[b]), 1);
@@ -93,94 +98,119 @@ vocab_argmax_persistent_kernel(const __grid_constant__ CUtensorMap map_w, const 
   const uint32_t tmem_acc = tmem_base_slot;
   pdl_launch();
   const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
-  pdl_wait();
 
   const int n_vt = (p.N + BLOCK_N_FEAT - 1) / BLOCK_N_FEAT;    // 128-row tiles: the layout of the partial arrays
-  const int n_v2 = (p.N + P_VOC - 1) / P_VOC;                  // 256-row tiles of a pair
   const int n_tt = (M + P_TOK - 1) / P_TOK;                    // token tiles that hold tokens
-  const long long n_pairs = (long long)n_tt * n_v2;
-  const int q_lo = (int)((n_pairs * blockIdx.x) / gridDim.x);
-  const int q_hi = (int)((n_pairs * (blockIdx.x + 1)) / gridDim.x);
-  const int my_pairs = q_hi - q_lo;
+  const long long n_units = (long long)n_tt * n_vt;
+  const int u_lo = (int)((n_units * blockIdx.x) / gridDim.x);
+  const int u_hi = (int)((n_units * (blockIdx.x + 1)) / gridDim.x);
+  // the steps of the range: from unit u, `width` (1 or 2) vocabulary tiles of token tile t
+  struct Step { int t, vt, width; };
+  auto step_at = [&](int u) {
+    Step s;
+    s.t = u / n_vt;
+    s.vt = u - s.t * n_vt;
+    s.width = (u + 1 < u_hi && s.vt + 1 < n_vt) ? 2 : 1;
+    return s;
+  };
   volatile int* abort_v = &abort_flag;
 
   if (warp >= 8 && warp < 8 + stages) {
     // ---- ring producers: producer pw owns stage pw and the K blocks pw, pw + S, ... of the CTA's whole sequence ----
     if (lane == 0) {
+      if (!p.M_ptr) pdl_wait();                            // operator-level call: the matrix may have just been written
       const int pw = warp - 8;
-      const int total_kb = my_pairs * KB;
       const uint32_t full = smem_u32(&bar_full[pw]), empty = smem_u32(&bar_empty[pw]);
       const uint32_t dst = b_base + (uint32_t)(pw * P_B_STAGE_BYTES);
-      for (int g = pw; g < total_kb; g += stages) {
-        const int it = g / KB, kb = g - it * KB;
-        const int v2 = (q_lo + it) % n_v2;
-        const uint32_t round = (uint32_t)(g / stages);
-        if (round > 0 && !mbar_wait(empty, (round - 1) & 1u, p.status)) { *abort_v = 1; break; }
-        if (*abort_v) break;
-        if (pw == 0) trace_mark_role(TR_PV_LOAD, 0);
-        mbar_expect_tx(full, (uint32_t)P_B_STAGE_BYTES);
-        // a box that starts beyond the last vocabulary row is filled with zeros and still counts its bytes
-        tma_load_2d(dst, &map_w, kb * BLOCK_K, v2 * P_VOC, full);
-        tma_load_2d(dst + A_STAGE_BYTES, &map_w, kb * BLOCK_K, v2 * P_VOC + BLOCK_N_FEAT, full);
+      int u = u_lo, first_kb = 0;                          // step at unit u starts with K block number first_kb of the sequence
+      bool ok = true;
+      for (int g = pw; ok && u < u_hi;) {
+        const Step st = step_at(u);
+        for (; g < first_kb + KB; g += stages) {
+          const uint32_t round = (uint32_t)(g / stages);
+          if (round > 0 && !mbar_wait(empty, (round - 1) & 1u, p.status)) { *abort_v = 1; ok = false; break; }
+          if (*abort_v) { ok = false; break; }
+          if (pw == 0) trace_mark_role(TR_PV_LOAD, 0);
+          const int kb = g - first_kb;
+          mbar_expect_tx(full, (uint32_t)(st.width * A_STAGE_BYTES));
+          // rows beyond the vocabulary are filled with zeros and still count their bytes
+          tma_load_2d(dst, &map_w, kb * BLOCK_K, st.vt * BLOCK_N_FEAT, full);
+          if (st.width == 2) tma_load_2d(dst + A_STAGE_BYTES, &map_w, kb * BLOCK_K, (st.vt + 1) * BLOCK_N_FEAT, full);
+        }
+        first_kb += KB;
+        u += st.width;
       }
     }
-  } else if (warp == 14) {
-    // ---- the resident token tile ----
+  } else if (warp >= 8 + stages && warp < 15) {
+    // ---- the resident token tile: loader l of n takes K blocks l, l + n, ... ----
     if (lane == 0) {
+      const int l = warp - 8 - stages, n = 7 - stages;
+      pdl_wait();
       int cur_t = -1;
       uint32_t uses = 0;
-      for (int it = 0; it < my_pairs; ++it) {
-        const int t = (q_lo + it) / n_v2;
-        if (t == cur_t) continue;
+      for (int u = u_lo; u < u_hi;) {
+        const Step st = step_at(u);
+        u += st.width;
+        if (st.t == cur_t) continue;
         // the MMAs of the previous token tile must have read it for the last time
         if (uses > 0 && !mbar_wait(smem_u32(&a_empty), (uses - 1) & 1u, p.status)) { *abort_v = 1; break; }
         if (*abort_v) break;
-        mbar_expect_tx(smem_u32(&a_full), (uint32_t)(KB * P_A_KB_BYTES));
-        for (int kb = 0; kb < KB; ++kb)
-          tma_load_2d(a_base + (uint32_t)(kb * P_A_KB_BYTES), &map_x, kb * BLOCK_K, t * P_TOK, smem_u32(&a_full));
-        cur_t = t;
+        for (int kb = l; kb < KB; kb += n) {
+          mbar_expect_tx(smem_u32(&a_full[kb]), (uint32_t)P_A_KB_BYTES);
+          tma_load_2d(a_base + (uint32_t)(kb * P_A_KB_BYTES), &map_x, kb * BLOCK_K, st.t * P_TOK, smem_u32(&a_full[kb]));
+        }
+        cur_t = st.t;
         ++uses;
       }
     }
   } else if (warp == 15) {
     // ---- MMA issuer ----
     if (lane == 0) {
-      const uint32_t idesc = make_idesc(P_TOK, P_VOC);
+      const uint32_t idesc2 = make_idesc(P_TOK, P_VOC), idesc1 = make_idesc(P_TOK, BLOCK_N_FEAT);
       const uint64_t desc_a0 = make_smem_desc(a_base);
       const uint64_t desc_b0 = make_smem_desc(b_base);
       const uint64_t a_step = (uint64_t)(P_A_KB_BYTES >> 4), b_step = (uint64_t)(P_B_STAGE_BYTES >> 4);
       bool ok = true;
-      int g = 0, cur_t = -1;
-      uint32_t uses = 0;
-      for (int it = 0; it < my_pairs && ok; ++it) {
-        const int b = it & 1;
-        const int t = (q_lo + it) / n_v2;
-        if (t != cur_t) {
-          ok = mbar_wait(smem_u32(&a_full), uses & 1u, p.status);
-          cur_t = t;
-          ++uses;
+      int cur_t = -1, it = 0, s = 0;
+      uint32_t uses = 0, phase = 0;                        // ring position of the next K block
+      // the K loop of one step; FRESH: first step of a token tile, whose K blocks arrive one by one.  (The issuing thread's own
+      // instructions set the pace: ring position by counting, no division.)
+      auto k_loop = [&](uint32_t acc, uint32_t idesc, auto fresh) {
+        uint64_t desc_a = desc_a0;
+        uint32_t accumulate = 0;
+        for (int kb = 0; kb < KB; ++kb) {
+          if (decltype(fresh)::value && !mbar_wait(smem_u32(&a_full[kb]), (uses - 1) & 1u, p.status)) return false;
+          if (!mbar_wait(smem_u32(&bar_full[s]), phase, p.status)) return false;
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint64_t desc_b = desc_b0 + b_step * (uint64_t)s;
+#pragma unroll
+          for (int k4 = 0; k4 < BLOCK_K / UMMA_K; ++k4) {
+            umma_bf16(acc, desc_a + 2 * k4, desc_b + 2 * k4, idesc, accumulate);
+            accumulate = 1u;
+          }
+          umma_commit(smem_u32(&bar_empty[s]));
+          desc_a += a_step;
+          if (++s == stages) { s = 0; phase ^= 1u; }
         }
-        // the half must have been read out (pair it - 2)
-        if (ok && it >= 2) ok = mbar_wait(smem_u32(&acc_empty[b]), (uint32_t)((it >> 1) - 1) & 1u, p.status);
+        return true;
+      };
+      for (int u = u_lo; u < u_hi && ok; ++it) {
+        const Step st = step_at(u);
+        u += st.width;
+        const int b = it & 1;
+        const bool fresh = st.t != cur_t;
+        if (fresh) { cur_t = st.t; ++uses; }
+        // the half must have been read out (step it - 2)
+        if (it >= 2) ok = mbar_wait(smem_u32(&acc_empty[b]), (uint32_t)((it >> 1) - 1) & 1u, p.status);
         if (!ok || *abort_v) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t acc = tmem_acc + (uint32_t)(b * P_VOC);
+        const uint32_t acc = tmem_acc + (uint32_t)(b * P_VOC), idesc = st.width == 2 ? idesc2 : idesc1;
         trace_mark_role(TR_PV_ISSUE, 0);
-        for (int kb = 0; kb < KB; ++kb, ++g) {
-          const int s = g % stages;
-          ok = mbar_wait(smem_u32(&bar_full[s]), (uint32_t)(g / stages) & 1u, p.status);
-          if (!ok) break;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const uint64_t desc_a = desc_a0 + a_step * (uint64_t)kb, desc_b = desc_b0 + b_step * (uint64_t)s;
-#pragma unroll
-          for (int k4 = 0; k4 < BLOCK_K / UMMA_K; ++k4)
-            umma_bf16(acc, desc_a + 2 * k4, desc_b + 2 * k4, idesc, (kb != 0 || k4 != 0) ? 1u : 0u);
-          umma_commit(smem_u32(&bar_empty[s]));
-        }
+        ok = fresh ? k_loop(acc, idesc, std::true_type{}) : k_loop(acc, idesc, std::false_type{});
         if (!ok) break;
         umma_commit(smem_u32(&acc_full[b]));
-        // last pair of this token tile: once these MMAs are done the resident tile may be replaced
-        if (it + 1 == my_pairs || (q_lo + it + 1) / n_v2 != t) umma_commit(smem_u32(&a_empty));
+        // last step of this token tile: once these MMAs are done the resident tile may be replaced
+        if (u >= u_hi || u / n_vt != st.t) umma_commit(smem_u32(&a_empty));
         trace_mark_role(TR_PV_ISSUE, 1);
       }
       if (!ok) {   // nobody must be left waiting for an accumulator that will not come
@@ -193,14 +223,15 @@ vocab_argmax_persistent_kernel(const __grid_constant__ CUtensorMap map_w, const 
     // ---- read-out: warps 0-7 ----
     const int quad = warp & 3, grp = warp >> 2;
     const bool relaxed = p.draft_val != nullptr;
-    int cur_t = -1, did = -1;
+    int cur_t = -1, did = -1, it = 0;
     float dval = 0.f;
-    for (int it = 0; it < my_pairs; ++it) {
-      const int b = it & 1;
-      const int q = q_lo + it;
-      const int t = q / n_v2, v2 = q - t * n_v2;
+    pdl_wait();
+    for (int u = u_lo; u < u_hi; ++it) {
+      const Step st = step_at(u);
+      u += st.width;
+      const int b = it & 1, t = st.t;
       const int tok = t * P_TOK + quad * 32 + lane;              // this thread's token
-      const int vt = v2 * 2 + grp;                               // this warp's 128-row tile of the partial arrays
+      const int vt = st.vt + grp;                                // this warp's 128-row tile of the partial arrays
       if (relaxed && t != cur_t) {
         dval = tok < M ? p.draft_val[tok] : 0.f;
         did = tok < M ? p.draft_id[tok] : -1;
@@ -214,6 +245,8 @@ vocab_argmax_persistent_kernel(const __grid_constant__ CUtensorMap map_w, const 
       const int n_base = vt * BLOCK_N_FEAT;
       float best = -INFINITY;
       int best_n = n_base, cnt = 0;
+      const bool mine = grp < st.width;                          // (a step of one tile has no second half)
+      if (mine)
       for (int c = 0; c < BLOCK_N_FEAT; c += 16) {
         float acc[16];
         tmem_ld16(taddr + static_cast<uint32_t>(c), acc);
@@ -230,7 +263,7 @@ vocab_argmax_persistent_kernel(const __grid_constant__ CUtensorMap map_w, const 
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
       if (threadIdx.x == 0) trace_mark_role(TR_PV_EPI, 1);
-      if (tok < M && vt < n_vt) {
+      if (mine && tok < M) {
         const size_t o = (size_t)tok * n_vt + vt;
         p.part_val[o] = best;
         p.part_idx[o] = best_n;
