@@ -20,7 +20,7 @@
 #include "gemm_few.cuh"
 #include "gemm_simt.cuh"
 #include "gemm_tc.cuh"
-#include "gemm_tc_persistent.cuh"
+#include "gemm_tc_pair.cuh"
 #include "grid_sync.cuh"
 #include "mega.cuh"
 #include "steps.cuh"
@@ -35,6 +35,7 @@ struct Mat {
   const void* ptr = nullptr;
   int N = 0, K = 0;
   CUtensorMap map;
+  CUtensorMap map64;     // embedding matrix only: boxes of 64 rows
 };
 struct ActBuf {
   void* ptr = nullptr;
@@ -410,6 +411,7 @@ int bind_model(ad_handle* h, Model& m, const ad_model_weights& w) {
   };
   auto vec = [&](const float*& t, int n) { t = vp; vp += n; };
   mat(m.emb, c.vocab, d);
+  if (h->bf16) ok = ok && make_map(&m.emb.map64, m.emb.ptr, c.vocab, d, tc::P_BOX);
   m.enc.resize(c.n_enc);
   m.dec.resize(c.n_dec);
   for (auto& L : m.enc) {
@@ -525,31 +527,36 @@ cudaError_t launch_tc(cudaStream_t st, const CUtensorMap& mw, const tc::TileMaps
   return launch_tc_n<EPI, 0>(st, mw, mx, p, sh, w, x);
 }
 
-// Projection + arg-max over many tokens: the persistent token-stationary kernel (one CTA per SM, 128-token tiles
-// resident in shared memory, read-out of one tile under the K loop of the next) once there are at least `min_pairs_per_sm`
-// (128 token x 256 vocabulary row) pairs per SM; AD_NO_PERSISTENT_VOCAB=1 keeps the one-tile-per-CTA kernel.
+// Projection + arg-max over many tokens: the persistent token-stationary kernel on pairs of SMs, once there is at least one
+// (128 token x 256 vocabulary row) piece of work per SM; AD_NO_PERSISTENT_VOCAB=1 keeps the one-tile-per-CTA kernel.
 bool vocab_goes_persistent(int K, int N, int M_cap, const float* bias) {
   static const bool enabled = [] { const char* e = getenv("AD_NO_PERSISTENT_VOCAB"); return !(e && e[0] == '1'); }();
   if (!enabled || bias || K % tc::BLOCK_K || K / tc::BLOCK_K > tc::P_MAX_KB) return false;
-  const long pairs = (long)((N + tc::P_VOC - 1) / tc::P_VOC) * ((M_cap + tc::P_TOK - 1) / tc::P_TOK);
-  return pairs >= (long)num_sms();
+  return (long)((N + tc::P_VOC - 1) / tc::P_VOC) * ((M_cap + tc::P_TOK - 1) / tc::P_TOK) >= (long)num_sms();
 }
-// mx128: the token operand's map with a 128-row box.
-cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw, const CUtensorMap& mx128, const GemmParams& p, int M_cap) {
+// mw64: the matrix' map with a 64-row box; mx128: the token operand's with a 128-row box.
+cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw64, const CUtensorMap& mx128, const GemmParams& p, int M_cap) {
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
   constexpr int kSmemLimit = 227 * 1024 - 512;   // the kernel's static shared memory is a few hundred bytes
   if (!attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(tc::vocab_argmax_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    cudaError_t e = cudaFuncSetAttribute(tc::vocab_argmax_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
   const int kb = p.K / tc::BLOCK_K;
   const int stages = clampi((kSmemLimit - 1024 - kb * tc::P_A_KB_BYTES) / tc::P_B_STAGE_BYTES, 1, tc::P_MAX_STAGES);
-  const long units = (long)((p.N + tc::BLOCK_N_FEAT - 1) / tc::BLOCK_N_FEAT) * ((M_cap + tc::P_TOK - 1) / tc::P_TOK);
-  const int grid = (int)std::min<long>(units, num_sms());
-  return launch_k(tc::vocab_argmax_persistent_kernel, dim3(grid), dim3(tc::P_THREADS), tc::vocab_persistent_smem(kb, stages), st, mw, mx128, p,
-                  stages);
+  const long units = (long)((p.N + tc::BLOCK_N_FEAT - 1) / tc::BLOCK_N_FEAT) * ((M_cap + 2 * tc::P_TOK - 1) / (2 * tc::P_TOK));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * (int)std::min<long>(units, num_sms() / 2)); cfg.blockDim = dim3(tc::P_THREADS);
+  cfg.dynamicSmemBytes = tc::vocab_pair_smem(kb, stages); cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = g_use_pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, tc::vocab_argmax_pair_kernel, mw64, mx128, p, stages);
 }
 
 // Projection of a pass with few tokens (gemm_few.cuh).  ksplit: few::split_for of the shape, non-zero.
@@ -647,7 +654,7 @@ int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int
     }
   } else if (h->bf16 && epi == EPI_ARGMAX && pc.ntile == 256 && vocab_goes_persistent(W.K, W.N, M_cap, p.bias)) {
     // (a pass with a 256-token tile also has the 128-row map of its token operand)
-    e = launch_vocab_persistent(h->stream, W.map, X.map_for(pk, tc::P_TOK), p, M_cap);
+    e = launch_vocab_persistent(h->stream, W.map64, X.map_for(pk, tc::P_TOK), p, M_cap);
   } else if (h->bf16) {
     const auto key = std::make_tuple(pk, W.N, W.K, split ? 1 : 0);
     auto it = h->tc_shapes.find(key);
@@ -2089,8 +2096,9 @@ extern "C" int ad_vocab_argmax(const void* x, const void* emb, int32_t dtype, in
   if (dtype == AD_DTYPE_BF16) {
     if (d % 64 || M > kMaxOpTokens) return AD_ERR_ARG;
     CUtensorMap mw;
-    if (!make_map(&mw, emb, vocab, d, tc::BLOCK_N_FEAT)) return AD_ERR_CUDA;
-    if (vocab_goes_persistent(d, vocab, M, nullptr)) {
+    const bool persistent = vocab_goes_persistent(d, vocab, M, nullptr);
+    if (!make_map(&mw, emb, vocab, d, persistent ? tc::P_BOX : tc::BLOCK_N_FEAT)) return AD_ERR_CUDA;
+    if (persistent) {
       CUtensorMap mx128;
       if (!make_map(&mx128, x, M, d, tc::P_TOK)) return AD_ERR_CUDA;
       e = launch_vocab_persistent(st, mw, mx128, p, M);

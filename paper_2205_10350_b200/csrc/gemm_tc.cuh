@@ -7,8 +7,8 @@
 // Both operands are K-major (row-major [rows, K]) and land in shared memory in the 128-byte-swizzled
 // canonical layout that the TMA and the MMA shared-memory descriptor agree on.
 //
-// Thread roles inside the 256-thread CTA: lane 0 of several warps issues TMA loads, lane 0 of warps 4..7 issues the
-// MMAs (up to four issuers, each with its own accumulator region in tensor memory), then all eight warps take part
+// Thread roles inside the 256-thread CTA: one lane of several warps issues TMA loads, one lane of warps 4 and 5 issues the
+// MMAs (up to two issuers, each with its own accumulator region in tensor memory), then all eight warps take part
 // in the epilogue: warp w reads the 32 TMEM lanes of quadrant w % 4 (tcgen05.ld 32x32b), adds the issuers' regions
 // up, and the two warps of a quadrant share its token columns.  The epilogue is a chain of dependent instructions
 // per thread, so halving each thread's share of it shortens the kernel.
@@ -87,11 +87,39 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* st
   return mbar_wait_budget(bar, parity, status, WAIT_BUDGET_NS);
 }
 
+// The same by a whole converged warp, which stays converged: every lane gets the same answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* status) {
+  for (int i = 0; i < 64; ++i)
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const unsigned long long t0 = global_ns();
+  for (;;) {
+    for (int i = 0; i < 64; ++i)
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, global_ns() - t0 > WAIT_BUDGET_NS)) break;
+  }
+  latch_error(status, AD_ERR_TIMEOUT);
+  return false;
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
       : "memory");
+}
+
+// Warp index as a value the compiler knows to be the same in all lanes, and one lane of a converged warp.  The MMA instructions
+// take their operands from the warp's uniform registers: issued from a branch on the lane number every one of them costs its
+// thread 65-80 cycles and more; from a converged warp behind elect.sync the paired projection below went from 64.5 to 51 us.
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(one));
+  return one != 0;
 }
 
 // Shared-memory matrix descriptor of a K-major tile whose rows are 128 bytes (64 bf16) and whose 8-row
@@ -343,7 +371,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   const CUtensorMap& map_x = maps_x.m[27 - __clz(ntile)];
   const int t0 = ty * ntile;
   const int n0 = fx * BLOCK_N_FEAT;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const int quad = warp & 3, grp = warp >> 2;   // accumulator lane quadrant of this warp; column group in the epilogue
   const int b_stage_bytes = ntile * BLOCK_K * 2;
   const int stage_bytes = A_STAGE_BYTES + b_stage_bytes;
@@ -357,17 +385,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   // lanes takes 2.2 us of a CTA's 12 us at 90 tokens x 768.
   const bool token_major = EPI == EPI_ARGMAX && ntile == 128 && !p.bias;
   const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzled tiles need 1024-byte alignment
-  // MMA issuers.  Issuing one tcgen05.mma costs its thread 65-80 cycles whatever the tile, so with few tokens (short
-  // MMAs) a single issuer, not the tensor pipe or shared memory, sets the pace of the K loop.  Up to four threads in
-  // different warps therefore issue side by side: issuer j takes the K blocks j, j + n, j + 2n, ... of this CTA and
-  // accumulates them in its own ntile-column region of tensor memory; the epilogue adds the regions up.
+  // MMA issuers.  Up to two warps issue side by side while the token tile is small: issuer j takes the K blocks j, j + n, ... of
+  // this CTA and accumulates them in its own ntile-column region of tensor memory; the epilogue adds the regions up.  (631 x 4096
+  // x 1024, 64-token tiles: one issuer 16.5 us, two 12.1, four 13.1.)
   // An issuer waits for ring phase r of a stage only after phase r - 1 has completed (a parity wait two phases ahead
   // would alias): with more than one ring round this holds when the ring depth is a multiple of the issuer count, since
   // the K block that used the stage one round earlier was then this issuer's own.
   int n_issuers = 1;
   {
-    const int cap = ntile <= 64 ? 4 : (ntile <= 128 ? 2 : 1);
-    for (int cand = 4; cand > 1; cand >>= 1)
+    const int cap = ntile <= 128 ? 2 : 1;
+    for (int cand = 2; cand > 1; cand >>= 1)
       if (cand <= cap && cand <= num_kb && (num_kb <= stages || stages % cand == 0)) { n_issuers = cand; break; }
   }
   uint32_t tmem_cols = 32;
@@ -400,12 +427,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   // never starve it.
   pdl_launch();
 
-  // TMA issue is spread over lane 0 of all eight warps: one thread's bulk-tensor copies are processed one after
+  // TMA issue is spread over all eight warps: one thread's bulk-tensor copies are processed one after
   // the other, several threads' copies run side by side.  Stage i of the first ring round belongs to warp i;
   // later rounds are fed by up to four of the warps 0 .. 3.
-  if (lane == 0) {
-    // weights never change: fetch the first ring round before the previous kernel has finished
-    for (int i = warp; i < first_round; i += THREADS / 32) {
+  // weights never change: fetch the first ring round before the previous kernel has finished
+  for (int i = warp; i < first_round; i += THREADS / 32) {
+    if (elect_one()) {
       const uint32_t bar = smem_u32(&bar_full[i]);
       mbar_expect_tx(bar, (uint32_t)stage_bytes);
       tma_load_2d(smem_base + i * stage_bytes, &map_w, (kb_begin + i) * BLOCK_K, n0, bar);
@@ -419,9 +446,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
 
   pdl_wait();
   trace_mark(TR_GEMM + EPI, 1);
-  if (lane == 0) {
-    // activations of the first ring round (rows beyond M are valid memory and simply never stored)
-    for (int i = warp; i < first_round; i += THREADS / 32)
+  // activations of the first ring round (rows beyond M are valid memory and simply never stored)
+  for (int i = warp; i < first_round; i += THREADS / 32) {
+    if (elect_one())
       tma_load_2d(smem_base + i * stage_bytes + A_STAGE_BYTES, &map_x, (kb_begin + i) * BLOCK_K, t0,
                   smem_u32(&bar_full[i]));
   }
@@ -433,7 +460,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         did_s[j] = (t0 + j < M) ? p.draft_id[t0 + j] : -1;
       }
     }
-    if (lane == 0 && warp < 4) {
+    if (warp < 4) {
       // ---- TMA producers: everything that was not issued above ----
       // The producer count divides the ring depth, so producer pw refills the same stages (pw, pw + nprod, ...) round
       // after round and every stage is refilled by one thread only.  Its parity wait on a stage's "empty" barrier is
@@ -449,17 +476,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       for (int i = first_round + pw; pw < nprod && i < num_kb; i += nprod) {
         const int s = i % stages;
         const uint32_t round = i / stages;
-        if (round > 0 && !mbar_wait(smem_u32(&bar_empty[s]), (round - 1) & 1, p.status)) { abort_flag = 1; break; }
+        if (round > 0 && !mbar_wait_warp(smem_u32(&bar_empty[s]), (round - 1) & 1, p.status)) { abort_flag = 1; break; }
         if (*reinterpret_cast<volatile int*>(&abort_flag)) break;
         const uint32_t a_dst = smem_base + s * stage_bytes;
         const uint32_t bar = smem_u32(&bar_full[s]);
-        mbar_expect_tx(bar, (uint32_t)stage_bytes);
-        tma_load_2d(a_dst, &map_w, (kb_begin + i) * BLOCK_K, n0, bar);
-        tma_load_2d(a_dst + A_STAGE_BYTES, &map_x, (kb_begin + i) * BLOCK_K, t0, bar);
+        if (elect_one()) {
+          mbar_expect_tx(bar, (uint32_t)stage_bytes);
+          tma_load_2d(a_dst, &map_w, (kb_begin + i) * BLOCK_K, n0, bar);
+          tma_load_2d(a_dst + A_STAGE_BYTES, &map_x, (kb_begin + i) * BLOCK_K, t0, bar);
+        }
+        __syncwarp();
       }
       if (warp == 0) trace_mark(TR_GEMM + EPI, 3);
-    } else if (warp >= 4 && warp - 4 < n_issuers && lane == 0) {
-      // ---- MMA issuers (lane 0 of warps 4 .. 4 + n_issuers - 1) ----
+    } else if (warp >= 4 && warp - 4 < n_issuers) {
+      // ---- MMA issuers (one lane of warps 4 .. 4 + n_issuers - 1) ----
       const int j = warp - 4;
       const uint32_t idesc = make_idesc(BLOCK_N_FEAT, ntile);
       const uint32_t acc_j = tmem_acc + (uint32_t)(j * ntile);
@@ -470,24 +500,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       int s = j % stages;
       uint32_t parity = (uint32_t)(j / stages) & 1u;
       for (int i = j; i < num_kb; i += n_issuers) {
-        ok = mbar_wait(smem_u32(&bar_full[s]), parity, p.status);
+        ok = mbar_wait_warp(smem_u32(&bar_full[s]), parity, p.status);
         if (!ok) { abort_flag = 1; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint64_t desc_a = desc_a0 + desc_step * (uint64_t)s, desc_b = desc_b0 + desc_step * (uint64_t)s;
+        if (elect_one()) {
 #pragma unroll
-        for (int k4 = 0; k4 < BLOCK_K / UMMA_K; ++k4) {
-          // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in the (address >> 4) field
-          umma_bf16(acc_j, desc_a + 2 * k4, desc_b + 2 * k4, idesc, (i != j || k4 != 0) ? 1u : 0u);
+          for (int k4 = 0; k4 < BLOCK_K / UMMA_K; ++k4) {
+            // advancing 16 bf16 = 32 bytes along K inside the swizzle row: +2 in the (address >> 4) field
+            umma_bf16(acc_j, desc_a + 2 * k4, desc_b + 2 * k4, idesc, (i != j || k4 != 0) ? 1u : 0u);
+          }
+          // the stage is handed back to the producers only if a later K block will land in it
+          if (i + stages < num_kb) umma_commit(smem_u32(&bar_empty[s]));
         }
-        // the stage is handed back to the producers only if a later K block will land in it
-        if (i + stages < num_kb) umma_commit(smem_u32(&bar_empty[s]));
+        __syncwarp();
         s += n_issuers;
         while (s >= stages) { s -= stages; parity ^= 1u; }
       }
       // one arrival per issuer: the accumulator barrier fires when every region is complete.  An issuer that gave
       // up still arrives (plainly), so that nobody waits for it; the abort flag tells the epilogue to do nothing.
-      if (ok) umma_commit(smem_u32(&bar_acc));
-      else asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_acc)) : "memory");
+      if (elect_one()) {
+        if (ok) umma_commit(smem_u32(&bar_acc));
+        else asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&bar_acc)) : "memory");
+      }
     }
     __syncwarp();
 
