@@ -564,17 +564,12 @@ template <int EPI, bool EMB = false>
 cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p, int ksplit, const few::EmbedParams& ep = {}) {
   const dim3 grid(p.N / few::FEAT, ksplit);
   const bf16 *w = (const bf16*)W.ptr, *xp = (const bf16*)x;
-  const int nch = p.K / ksplit / 256;
-  if (few::wide_fits(p.N, nch)) {
-    const dim3 wgrid(p.N / few::W_FEAT, ksplit);
-    if (nch == 3) return launch_k(few::gemm_few_wide_kernel<EPI, 3, EMB>, wgrid, dim3(few::THREADS), 0, st, w, xp, p, ep);
-    return launch_k(few::gemm_few_wide_kernel<EPI, 4, EMB>, wgrid, dim3(few::THREADS), 0, st, w, xp, p, ep);
-  }
-  switch (nch) {
+  const dim3 wgrid(p.N / few::W_FEAT, ksplit);
+  switch (p.K / ksplit / 256) {
     case 1: return launch_k(few::gemm_few_kernel<EPI, 1, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
     case 2: return launch_k(few::gemm_few_kernel<EPI, 2, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
-    case 3: return launch_k(few::gemm_few_kernel<EPI, 3, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
-    default: return launch_k(few::gemm_few_kernel<EPI, 4, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    case 3: return launch_k(few::gemm_few_wide_kernel<EPI, 3, EMB>, wgrid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    default: return launch_k(few::gemm_few_wide_kernel<EPI, 4, EMB>, wgrid, dim3(few::THREADS), 0, st, w, xp, p, ep);
   }
 }
 
@@ -585,7 +580,7 @@ GeoRule geo_rule(const PassCfg& pc, int epi, int N, int K, bool split, bool has_
   if (r.few_split > 0) {
     const int nch = K / r.few_split / 256;
     // (within a larger capacity a pass of few tokens runs the 16-feature form inside the tensor-core kernel)
-    r.few_tokens = pc.M_cap <= few::MAX_TOKENS && few::wide_fits(N, nch) ? few::MAX_TOKENS : few::max_tokens(nch);
+    r.few_tokens = pc.M_cap <= few::MAX_TOKENS ? few::MAX_TOKENS : few::max_tokens(nch);
   }
   return r;
 }
@@ -2065,15 +2060,10 @@ argmax_rows_kernel(const float* __restrict__ part_val, const int* __restrict__ p
 }  // namespace
 
 namespace {
-// Token tile of an operator-level call: by the passes' rule.
-int op_tile(const GeoRule& r, int M) { 
-  static const int force = [] { const char* e = getenv("AD_OP_TILE"); return e ? atoi(e) : 0; }();
-  if (force) return std::min(force, r.max_tile);
-  return geometry(r, M).tile; }
-// Geometry of an operator-level call over M tokens, and the token operand's map for its tile.
+// Geometry of an operator-level call over M tokens (by the passes' rule), and the token operand's map for its tile.
 bool op_maps(GemmParams* p, tc::TileMaps* mx, const void* x, int M, int K) {
   p->rule = GeoRule{p->N, K, clampi(pow2ceil(M), 16, 256), 1, num_sms(), 0, 0, 0};
-  const int tile = p->rule.fixed_tile = op_tile(p->rule, M);
+  const int tile = p->rule.fixed_tile = geometry(p->rule, M).tile;
   int i = 0;
   while ((16 << i) < tile) ++i;
   memset(mx, 0, sizeof(*mx));

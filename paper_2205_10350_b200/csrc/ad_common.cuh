@@ -54,8 +54,8 @@ enum Epi : int {
 // on the device from the M the plan holds, by the projection and by whoever adds its partial sums up, so that a pass always
 // runs at the geometry of the tokens it has, not at that of its capacity.
 //
-// Token tile: up to 64 tokens one tile; beyond that the kernels are latency-bound and smaller tiles win -- more CTAs, more MMA
-// issuers per CTA, a shorter epilogue each -- until the grids outgrow the SMs.  Measured per step (base model):
+// Token tile: up to 64 tokens one tile; beyond that the kernels are latency-bound and smaller tiles win -- more CTAs, a
+// shorter epilogue each -- until the grids outgrow the SMs.  Measured per step (base model):
 //   100 / 120 / 128 tokens: 64-token tiles 277 / 289 / 293 us against 305 / 316 / 321 us with one 128-token tile;
 //   200 / 240 tokens: 32-token tiles 331 / 305 us, 64: 344 / 311, 128: 364 / 336, 16: 372;
 //   320 / 400 / 512 tokens: 64-token tiles 366 / 357 / 389 us against 415 / 410 / 458 (128) and 383 / 380 / 410 (32);

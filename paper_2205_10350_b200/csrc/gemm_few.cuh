@@ -20,6 +20,7 @@ namespace few {
 constexpr int THREADS = 256;
 constexpr int WARPS = 8;
 constexpr int FEAT = 16;          // output features per CTA = MMA M
+constexpr int W_FEAT = 32;        // ... of the form for wide slices of K (gemm_few_wide_kernel)
 constexpr int RED_LD = 20;        // floats per token row of a warp's partial sums: conflict-free, 16-byte aligned
 constexpr int MAX_TOKENS = 128;   // most packed tokens of a pass that these kernels take
 constexpr int MAX_CHUNKS = 4;     // 32-wide K chunks per warp: K per CTA = 256 .. 1024
@@ -40,7 +41,7 @@ __host__ __device__ constexpr int round_tokens(int nch) { return nch <= 2 ? 64 :
 // K split of a projection with N output features: the smallest power of two that leaves at most 1024 of K to a CTA, more
 // while the grid stays within 128 CTAs and the split is wanted (consumer adds partial sums up).  0: shape not supported.
 inline int split_for(int N, int K, bool may_split, int max_split) {
-  if (N % FEAT || K % 256) return 0;
+  if (N % W_FEAT || K % 256) return 0;
   int s = 1;
   while (K / s > 256 * MAX_CHUNKS || (may_split && (N / FEAT) * s * 2 <= 128 && K % (512 * s) == 0 && K / (2 * s) >= 512)) {
     s *= 2;
@@ -205,7 +206,7 @@ __device__ __forceinline__ void few_body(const bf16* __restrict__ W, const bf16*
   }
 }
 
-// grid = (N / 16, ksplit); block = 256.
+// grid = (N / 16, ksplit); block = 256.  NCH = 1, 2.
 template <int EPI, int NCH, bool EMB>
 __global__ void __launch_bounds__(THREADS, 2)
 gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, const EmbedParams ep) {
@@ -219,11 +220,9 @@ gemm_few_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, c
 // The same for wider slices of K (768 and 1024 per CTA), where 16 features per CTA leave the kernel bound by the activations it
 // re-reads (90 tokens of a 768-wide model: 192 CTAs x 138 KB, three dependent rounds, 4.9 us after the wait): 32 features per
 // CTA halve that traffic, one CTA per SM has the registers for the next round's activations to be in flight under this one.
-// grid = (N / 32, ksplit); block = 256.
-constexpr int W_FEAT = 32;
+// grid = (N / 32, ksplit); block = 256.  NCH = 3, 4.
 constexpr int W_TOK = 32;
 constexpr int W_LD = W_FEAT + 4;
-inline bool wide_fits(int N, int nch) { return nch >= 3 && nch <= 4 && N % W_FEAT == 0; }
 template <int EPI, int NCH, bool EMB>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_few_wide_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams p, const EmbedParams ep) {

@@ -158,22 +158,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                : "memory");
 }
-// 32 consecutive accumulator columns of this thread's TMEM lane.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
+// 16 consecutive accumulator columns of this thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
   asm volatile(
@@ -244,34 +229,10 @@ __device__ __forceinline__ void warp_argmax_lane(float v, float& best, int& lane
   lane_of_best = __ffs(bal) - 1;
 }
 
-// Arg-max over the 32 lanes for 32 values per lane at once.  v[j] is this lane's candidate for item j; on
-// return lane L holds, for item L, the largest candidate and the lowest lane that offered it.  Each halving
-// step sends one half of the items a lane still holds to its partner and keeps the other half, so that every
+// Arg-max over the 32 lanes for 16 values per lane at once.  v[j] is this lane's candidate for item j; on
+// return lanes 2 j and 2 j + 1 hold, for item j, the largest candidate and the lowest lane that offered it.  Each
+// halving step sends one half of the items a lane still holds to its partner and keeps the other half, so that every
 // item costs about one exchange instead of five.
-__device__ __forceinline__ void warp_argmax_items(float (&v)[32], int lane, float& best, int& from) {
-  int src[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) src[j] = lane;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const bool up = (lane & o) != 0;                 // this lane keeps the upper half of its items
-#pragma unroll
-    for (int i = 0; i < o; ++i) {
-      const float keep_v = up ? v[i + o] : v[i];
-      const int keep_s = up ? src[i + o] : src[i];
-      const float send_v = up ? v[i] : v[i + o];
-      const int send_s = up ? src[i] : src[i + o];
-      const float ov = __shfl_xor_sync(0xffffffffu, send_v, o);
-      const int os = __shfl_xor_sync(0xffffffffu, send_s, o);
-      const bool take = ov > keep_v || (ov == keep_v && os < keep_s);
-      v[i] = take ? ov : keep_v;
-      src[i] = take ? os : keep_s;
-    }
-  }
-  best = v[0];
-  from = src[0];
-}
-// The same for 16 items per lane: lanes 2j and 2j+1 both end up with item j.
 __device__ __forceinline__ void warp_argmax_items16(float (&v)[16], int lane, float& best, int& from) {
   int src[16];
 #pragma unroll
