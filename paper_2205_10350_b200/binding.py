@@ -341,6 +341,23 @@ class AggressiveDecoder:
         self._check(self.lib.ad_commit(self.h, C.c_void_p(n_t.data_ptr()) if n_t is not None else None, 0), self.h)
 
 
+_stream = None          # (device, raw handle, stream object) of the last operator-level call
+
+
+def _current_stream():
+    """(stream object, raw handle) of torch's current stream.  torch.cuda.current_stream() builds an object on every call, a
+    tenth of a short operator-level call's time; the raw handle costs next to nothing, so the object is only made anew when the
+    handle is another one."""
+    import torch
+    global _stream
+    dev = torch._C._cuda_getDevice()
+    raw = torch._C._cuda_getCurrentRawStream(dev)
+    last = _stream
+    if last is None or last[0] != dev or last[1] != raw:
+        last = _stream = (dev, raw, torch.cuda.current_stream())
+    return last[2], raw
+
+
 def vocab_argmax(x_t, emb_t, status_t=None):
     """Operator-level call: arg-max of x @ emb^T per row.  x_t [M, d], emb_t [V, d], both float32 or bfloat16.
     Returns when the result is complete."""
@@ -350,11 +367,11 @@ def vocab_argmax(x_t, emb_t, status_t=None):
     V = emb_t.shape[0]
     dtype = AD_DTYPE_BF16 if x_t.dtype is torch.bfloat16 else AD_DTYPE_FP32
     nbytes = lib.ad_vocab_argmax_scratch_bytes(V, M)
-    scratch = torch.empty(nbytes + 256, dtype=torch.uint8, device=x_t.device)
-    out = torch.empty(M, dtype=torch.int32, device=x_t.device)
-    stream = torch.cuda.current_stream()
+    scratch = x_t.new_empty(nbytes + 256, dtype=torch.uint8)
+    out = x_t.new_empty(M, dtype=torch.int32)
+    stream, raw = _current_stream()
     rc = lib.ad_vocab_argmax(x_t.data_ptr(), emb_t.data_ptr(), dtype, M, d, V, out.data_ptr(), (scratch.data_ptr() + 255) // 256 * 256, nbytes,
-                             status_t.data_ptr() if status_t is not None else None, stream.cuda_stream)
+                             status_t.data_ptr() if status_t is not None else None, raw)
     if rc != AD_OK:
         raise AdError(rc, "ad_vocab_argmax")
     stream.synchronize()
@@ -377,7 +394,7 @@ def vocab_argmax_static(x_t, emb_t, out_t, status_t=None):
     M, d = x_t.shape
     dtype = AD_DTYPE_BF16 if x_t.dtype is torch.bfloat16 else AD_DTYPE_FP32
     rc = lib.ad_vocab_argmax_static(x_t.data_ptr(), emb_t.data_ptr(), dtype, M, d, emb_t.shape[0], out_t.data_ptr(),
-                                    status_t.data_ptr() if status_t is not None else None, torch.cuda.current_stream().cuda_stream)
+                                    status_t.data_ptr() if status_t is not None else None, _current_stream()[1])
     if rc != AD_OK:
         msg = lib.ad_last_error(None)
         raise AdError(rc, msg.decode() if msg else "ad_vocab_argmax_static")
@@ -391,10 +408,10 @@ def linear(x_t, W_t, bias_t=None, status_t=None):
     M, K = x_t.shape
     N = W_t.shape[0]
     dtype = AD_DTYPE_BF16 if x_t.dtype is torch.bfloat16 else AD_DTYPE_FP32
-    y = torch.empty((M, N), dtype=torch.float32, device=x_t.device)
-    stream = torch.cuda.current_stream()
+    y = x_t.new_empty((M, N), dtype=torch.float32)
+    stream, raw = _current_stream()
     rc = lib.ad_linear(x_t.data_ptr(), W_t.data_ptr(), bias_t.data_ptr() if bias_t is not None else None, dtype, M, K, N, y.data_ptr(),
-                       status_t.data_ptr() if status_t is not None else None, stream.cuda_stream)
+                       status_t.data_ptr() if status_t is not None else None, raw)
     if rc != AD_OK:
         raise AdError(rc, "ad_linear")
     stream.synchronize()

@@ -587,20 +587,29 @@ GeoRule geo_rule(const PassCfg& pc, int epi, int N, int K, bool split, bool has_
 // Whether every projection of such a shape in pass pc runs on the few-token kernel.
 bool always_few(const PassCfg& pc, const GeoRule& r) { return r.few_split > 0 && pc.M_cap <= r.few_tokens; }
 
-template <int EPI>
-cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const GemmParams& p, int M_cap) {
+template <int EPI, int TJ>
+cudaError_t launch_simt_tile(cudaStream_t st, const void* w, const void* x, const GemmParams& p, int M_cap) {
   constexpr int FEAT = EPI == EPI_ARGMAX ? simt::ARGMAX_FEAT : 64;
-  constexpr size_t smem = simt::smem_bytes<FEAT>();
+  constexpr size_t smem = simt::smem_bytes<FEAT, TJ>();
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
   if (!attr_set[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(simt::gemm_f32_kernel<EPI, FEAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(simt::gemm_f32_kernel<EPI, FEAT, TJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
   const int vec = p.K % 4 == 0 && (reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(x)) % 16 == 0;
-  const dim3 grid((p.N + FEAT - 1) / FEAT, (M_cap + simt::TOK - 1) / simt::TOK);
-  return launch_k(simt::gemm_f32_kernel<EPI, FEAT>, grid, dim3(2 * FEAT), smem, st, (const float*)w, (const float*)x, p, vec);
+  const dim3 grid((p.N + FEAT - 1) / FEAT, (M_cap + 4 * TJ - 1) / (4 * TJ));
+  return launch_k(simt::gemm_f32_kernel<EPI, FEAT, TJ>, grid, dim3(2 * FEAT), smem, st, (const float*)w, (const float*)x, p, vec);
+}
+// FP32 projection in tiles of 32 tokens, or of 16 where the fullest SM then has less to do: a small tile takes two thirds of a
+// large one's time (7 x 1536 x 512: 9.6 us against 13; 100 x 1024 x 4096: 50 against 73; with the same number of tiles for an SM
+// as before there is nothing to gain: 40 x 4096 x 1024 23 against 22).
+template <int EPI>
+cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const GemmParams& p, int M_cap) {
+  const int feat = EPI == EPI_ARGMAX ? simt::ARGMAX_FEAT : 64, sms = num_sms();
+  auto per_sm = [&](int tokens) { return ((long)((p.N + feat - 1) / feat) * ((M_cap + tokens - 1) / tokens) + sms - 1) / sms; };
+  return 2 * per_sm(16) <= 3 * per_sm(32) ? launch_simt_tile<EPI, 4>(st, w, x, p, M_cap) : launch_simt_tile<EPI, 8>(st, w, x, p, M_cap);
 }
 // The few-token FP32 kernel: passes of at most kFewTokens tokens, shapes it covers.
 bool f32_few(const PassCfg& pc, int epi, int N, int K) { return pc.M_cap <= kFewTokens && epi != EPI_ARGMAX && simt::few_fits(N, K); }

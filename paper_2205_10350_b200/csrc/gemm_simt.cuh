@@ -2,7 +2,7 @@
 // definition to 1e-3: no TF32, no reduced-precision operands.  Same D^T[n, m] orientation and the same epilogues as the
 // tensor-core kernels.
 //
-// Two kernels.  gemm_f32_kernel: tiles of 64 or 128 features x 32 tokens, both operands copied asynchronously to shared memory
+// Two kernels.  gemm_f32_kernel: tiles of 64 or 128 features x 16 or 32 tokens, both operands copied asynchronously to shared memory
 // as they lie (no transposition: a thread multiplies its outputs by four consecutive k at a time).  gemm_f32_few_kernel:
 // passes of few tokens, where that kernel's walk along K is all latency: 16 features per CTA, K dealt to 16 half-warps,
 // weights in registers before the dependency wait.
@@ -14,14 +14,17 @@
 namespace ad {
 namespace simt {
 
-constexpr int TOK = 32;           // tokens per tile
 constexpr int KT = 32;            // k per stage
 constexpr int LDK = KT + 4;       // rows 144 bytes apart: conflict-free 16-byte reads of consecutive rows
-constexpr int STAGES = 3;
+constexpr int STAGES = 4;
 constexpr int ARGMAX_FEAT = 128;  // features per tile of the arg-max epilogue: the layout of the partial arrays
 
-template <int FEAT>
-constexpr size_t smem_bytes() { return sizeof(float) * (size_t)STAGES * (FEAT + TOK) * LDK; }   // (>= the partial sums)
+// Tiles of FEAT features x 4 TJ tokens, four warps per 64 features.
+template <int FEAT, int TJ>
+constexpr size_t smem_bytes() {
+  constexpr size_t ring = sizeof(float) * (size_t)STAGES * (FEAT + 4 * TJ) * LDK, sums = sizeof(float) * (size_t)(FEAT / 16) * 8 * TJ * 33;
+  return ring > sums ? ring : sums;
+}
 
 __device__ __forceinline__ void cp16(void* s, const void* g, bool there) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(s))), "l"(g),
@@ -47,20 +50,23 @@ __device__ __forceinline__ void store_out(const GemmParams& p, int n, int m, flo
   }
 }
 
-// A warp covers 64 features x 32 tokens, 8 x 8 outputs per lane; four warps per 64 features take every fourth quad of k and
-// their sums meet in shared memory at the end.  What bounds it: shared-memory wavefronts.  A 16-byte load costs a warp four of
-// them whatever it broadcasts, so a lane's tile decides: 8 x 8 spends 64 wavefronts on 256 FFMA instructions of a warp (64 SM
-// cycles), which balances; 8 x 4 spent 48 on 128 and took 34 us for 333 x 512 x 2048 (27 us now, back to back).
-// grid = (ceil(N / FEAT), ceil(M_cap / 32)); block = 2 FEAT; dynamic smem smem_bytes<FEAT>().  x: [M_cap, K], w: [N, K].
+// A warp covers 64 features x 4 TJ tokens, 8 x TJ outputs per lane; four warps per 64 features take every fourth quad of k and
+// their sums meet in shared memory at the end.  What bounds it: instruction issue.  Shared memory is the next limit: a 16-byte
+// load of eight different rows costs a warp four wavefronts, one that four rows serve two, so a lane's tile of 8 x 8 spends 48
+// on 256 FFMA instructions of a warp (64 SM cycles); 8 x 4 spends 40 on 128.  With the loads of a step in front of its
+// multiply-adds a warp issued in 47 % of its cycles, fetching ahead (below) in 60 %: 333 x 512 x 2048 48 -> 38 us on one warp per
+// scheduler (2048 -> 512 features); 700 x 1024 x 4096 177 -> 148 us.
+// grid = (ceil(N / FEAT), ceil(M_cap / (4 TJ))); block = 2 FEAT; dynamic smem smem_bytes<FEAT, TJ>().  x: [M_cap, K], w: [N, K].
 // vec: K is a multiple of four and both operands are 16-byte aligned.
 constexpr int GROUPS = 4;
 constexpr int SUM_LD = 33;
-template <int EPI, int FEAT>
+template <int EPI, int FEAT, int TJ>
 __global__ void __launch_bounds__(2 * FEAT, FEAT == 64 ? 3 : 1)
 gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p, const int vec) {
   constexpr int THREADS = 2 * FEAT;
   constexpr int RSTEP = THREADS / (KT / 4);            // rows between a thread's 16-byte copies: FEAT / RSTEP of W, then of x
-  constexpr int NW = FEAT / RSTEP, NX = TOK / RSTEP;
+  constexpr int TOK = 4 * TJ;
+  constexpr int NW = FEAT / RSTEP, NX = (TOK + RSTEP - 1) / RSTEP;
   extern __shared__ __align__(16) float simt_smem[];   // [STAGES][FEAT + TOK][LDK], later [warps][64][SUM_LD] partial sums
   const int M = p.M_ptr ? plan_load(p.M_ptr) : p.M_host;
   const int t0 = blockIdx.y * TOK, n0 = blockIdx.x * FEAT;
@@ -70,7 +76,7 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
   if (t0 >= M) return;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = warp % GROUPS, half = warp / GROUPS;               // share of k; 64-feature part of the tile
-  const int tx = lane & 7, ty = lane >> 3;                           // features tx + 8 i, tokens ty + 4 j (i, j < 8)
+  const int tx = lane & 7, ty = lane >> 3;                           // features tx + 8 i, tokens ty + 4 j
   const int K = p.K, nk = (K + KT - 1) / KT;
   const int fr = tid / (KT / 4), fc = (tid % (KT / 4)) * 4;          // first row and k of this thread's 16-byte copies
   const float *wsrc = w + (size_t)(n0 + fr) * K + fc, *xsrc = x + (size_t)(t0 + fr) * K + fc;
@@ -87,6 +93,7 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
         }
 #pragma unroll
         for (int i = 0; i < NX; ++i) {
+          if (TOK % RSTEP && fr + RSTEP * i >= TOK) break;
           const bool there = in_k && t0 + fr + RSTEP * i < M;
           cp16(dst + (FEAT + fr + RSTEP * i) * LDK + fc, there ? xsrc + (size_t)(RSTEP * i) * K + k0 : x, there);
         }
@@ -102,58 +109,65 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  float acc[8][8];
+  float acc[8][TJ];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    for (int j = 0; j < TJ; ++j) acc[i][j] = 0.f;
 #pragma unroll
   for (int s = 0; s < STAGES - 1; ++s) fetch(s);
-  for (int kt = 0; kt < nk; ++kt) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
-    __syncthreads();                                    // stage kt has landed, stage kt - 1 is free
-    fetch(kt + STAGES - 1);
-    const float* ws = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + (half * 64 + tx) * LDK + 4 * grp;
-    const float* xs = simt_smem + (size_t)(kt % STAGES) * (FEAT + TOK) * LDK + (FEAT + ty) * LDK + 4 * grp;
+  // One step: 16 k of a stage, four per warp.  A row of W is fetched one row ahead of its use and the tokens' pieces one step ahead,
+  // so that no multiply-add waits for shared memory.
+  const float* const wbase = simt_smem + (half * 64 + tx) * LDK + 4 * grp;
+  const float* const xbase = simt_smem + (FEAT + ty) * LDK + 4 * grp;
+  constexpr int STAGE = (FEAT + TOK) * LDK;
+  float4 a, b[TJ], bn[TJ];
+  auto step = [&](float4 (&bc)[TJ], float4 (&bnext)[TJ], int at, int next) {
 #pragma unroll
-    for (int k = 0; k < KT; k += 4 * GROUPS) {
-      float4 a[8], b[8];
+    for (int i = 0; i < 8; ++i) {
+      const float4 an = *reinterpret_cast<const float4*>(i < 7 ? wbase + at + (i + 1) * 8 * LDK : wbase + next);
+      if (i < TJ) bnext[i] = *reinterpret_cast<const float4*>(xbase + next + i * 4 * LDK);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = *reinterpret_cast<const float4*>(ws + i * 8 * LDK + k);
+      for (int j = 0; j < TJ; ++j) acc[i][j] = fmaf(a.x, bc[j].x, acc[i][j]);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) b[j] = *reinterpret_cast<const float4*>(xs + j * 4 * LDK + k);
+      for (int j = 0; j < TJ; ++j) acc[i][j] = fmaf(a.y, bc[j].y, acc[i][j]);
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int j = 0; j < TJ; ++j) acc[i][j] = fmaf(a.z, bc[j].z, acc[i][j]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+      for (int j = 0; j < TJ; ++j) acc[i][j] = fmaf(a.w, bc[j].w, acc[i][j]);
+      a = an;
     }
+  };
+  static_assert(KT == 8 * GROUPS && TJ <= 8, "two steps per stage");
+  asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+  __syncthreads();
+  a = *reinterpret_cast<const float4*>(wbase);
+#pragma unroll
+  for (int j = 0; j < TJ; ++j) b[j] = *reinterpret_cast<const float4*>(xbase + j * 4 * LDK);
+  int at = 0;
+  for (int kt = 0; kt < nk; ++kt) {
+    step(b, bn, at, at + 4 * GROUPS);
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 3) : "memory");
+    __syncthreads();                                    // stage kt + 1 has landed, stage kt - 1 is free
+    fetch(kt + STAGES - 1);
+    const int next = at == (STAGES - 1) * STAGE ? 0 : at + STAGE;
+    step(bn, b, at + 4 * GROUPS, next);                 // (after the last stage: pieces that nobody uses)
+    at = next;
   }
   // the groups' sums meet in shared memory
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
-  float* sums = simt_smem + (size_t)warp * 64 * SUM_LD + lane;
+  float* sums = simt_smem + (size_t)warp * 8 * TJ * SUM_LD + lane;
 #pragma unroll
   for (int i = 0; i < 8; ++i)
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sums[(i * 8 + j) * SUM_LD] = acc[i][j];
+    for (int j = 0; j < TJ; ++j) sums[(i * TJ + j) * SUM_LD] = acc[i][j];
   __syncthreads();
   auto sum_of = [&](int f, int tok) {                   // output (feature f, token tok) of the tile
-    const float* q = simt_smem + (size_t)(f / 64) * GROUPS * 64 * SUM_LD + ((f % 64) / 8 * 8 + tok / 4) * SUM_LD + (tok % 4) * 8 + f % 8;
+    const float* q = simt_smem + (size_t)(f / 64) * GROUPS * 8 * TJ * SUM_LD + ((f % 64) / 8 * TJ + tok / 4) * SUM_LD + (tok % 4) * 8 + f % 8;
     float v = q[0];
 #pragma unroll
-    for (int g = 1; g < GROUPS; ++g) v += q[(size_t)g * 64 * SUM_LD];
+    for (int g = 1; g < GROUPS; ++g) v += q[(size_t)g * 8 * TJ * SUM_LD];
     return v;
   };
   if (EPI == EPI_ARGMAX) {

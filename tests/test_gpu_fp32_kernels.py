@@ -1,4 +1,5 @@
-"""FP32 projection kernels at the edges of their tiles (64 / 128 features x 32 tokens x 32 k, vector and scalar copies) and of
+"""FP32 projection kernels at the edges of their tiles (64 / 128 features x 16 or 32 tokens x 32 k, vector and scalar copies; the
+larger sizes are those of 32-token tiles) and of
 the few-token form (16 features, 16-token rounds, K up to 512), against the checker."""
 import numpy as np
 import pytest
@@ -13,7 +14,8 @@ DEV = "cuda:0"
 OPS = O.Ops("f32")
 
 
-@pytest.mark.parametrize("M,K,N", [(1, 1, 1), (32, 32, 64), (33, 36, 65), (31, 30, 63), (65, 130, 128), (96, 512, 200), (333, 96, 129)])
+@pytest.mark.parametrize("M,K,N", [(1, 1, 1), (32, 32, 64), (33, 36, 65), (31, 30, 63), (65, 130, 128), (96, 512, 200), (333, 96, 129),
+                                   (31, 30, 6401), (32, 32, 6400), (65, 130, 3073), (333, 512, 2048), (64, 1, 4700)])
 def test_linear_tiles(M, K, N):
     r = np.random.default_rng(M + K + N)
     x, W = r.standard_normal((M, K)).astype(np.float32), (r.standard_normal((N, K)) * 0.1).astype(np.float32)
@@ -22,7 +24,7 @@ def test_linear_tiles(M, K, N):
     assert np.abs(y.cpu().numpy() - OPS.linear(x, W.T.copy(), b)).max() < 1e-4
 
 
-@pytest.mark.parametrize("M,d,V", [(1, 128, 128), (33, 50, 129), (40, 128, 1000)])
+@pytest.mark.parametrize("M,d,V", [(1, 128, 128), (33, 50, 129), (40, 128, 1000), (31, 50, 12900), (64, 96, 9473)])
 def test_argmax_tiles(M, d, V):
     r = np.random.default_rng(M + V)
     x, W = r.standard_normal((M, d)).astype(np.float32), r.standard_normal((V, d)).astype(np.float32)
