@@ -527,25 +527,27 @@ cudaError_t launch_tc(cudaStream_t st, const CUtensorMap& mw, const tc::TileMaps
   return launch_tc_n<EPI, 0>(st, mw, mx, p, sh, w, x);
 }
 
-// Projection + arg-max over many tokens: the persistent token-stationary kernel on pairs of SMs, once there is at least one
-// (128 token x 256 vocabulary row) piece of work per SM; AD_NO_PERSISTENT_VOCAB=1 keeps the one-tile-per-CTA kernel.
+// Projection + arg-max over many tokens: the persistent kernel on pairs of SMs beyond 128 tokens (a pair's tile is 256), once there
+// is at least one (128 token x 256 vocabulary row) piece of work per SM; up to 128 tokens one tile per CTA is faster (100 tokens x
+// 50265 x 768: 18 us against 23).  AD_NO_PERSISTENT_VOCAB=1 keeps the one-tile-per-CTA kernel.
 bool vocab_goes_persistent(int K, int N, int M_cap, const float* bias) {
   static const bool enabled = [] { const char* e = getenv("AD_NO_PERSISTENT_VOCAB"); return !(e && e[0] == '1'); }();
-  if (!enabled || bias || K % tc::BLOCK_K || K / tc::BLOCK_K > tc::P_MAX_KB) return false;
+  if (!enabled || bias || K % tc::BLOCK_K || M_cap <= tc::P_TOK) return false;
   return (long)((N + tc::P_VOC - 1) / tc::P_VOC) * ((M_cap + tc::P_TOK - 1) / tc::P_TOK) >= (long)num_sms();
 }
 // mw64: the matrix' map with a 64-row box; mx128: the token operand's with a 128-row box.
-cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw64, const CUtensorMap& mx128, const GemmParams& p, int M_cap) {
+template <bool STREAM>
+cudaError_t launch_vocab_pair(cudaStream_t st, const CUtensorMap& mw64, const CUtensorMap& mx128, const GemmParams& p, int M_cap) {
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
   constexpr int kSmemLimit = 227 * 1024 - 512;   // the kernel's static shared memory is a few hundred bytes
   if (!attr_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(tc::vocab_argmax_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+    cudaError_t e = cudaFuncSetAttribute(tc::vocab_argmax_pair_kernel<STREAM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
   const int kb = p.K / tc::BLOCK_K;
-  const int stages = clampi((kSmemLimit - 1024 - kb * tc::P_A_KB_BYTES) / tc::P_B_STAGE_BYTES, 1, tc::P_MAX_STAGES);
+  const int stages = STREAM ? tc::P_MAX_STAGES : clampi((kSmemLimit - 1024 - kb * tc::P_A_KB_BYTES) / tc::P_B_STAGE_BYTES, 1, tc::P_MAX_STAGES);
   const long units = (long)((p.N + tc::BLOCK_N_FEAT - 1) / tc::BLOCK_N_FEAT) * ((M_cap + 2 * tc::P_TOK - 1) / (2 * tc::P_TOK));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * (int)std::min<long>(units, num_sms() / 2)); cfg.blockDim = dim3(tc::P_THREADS);
@@ -556,7 +558,10 @@ cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw64, co
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = g_use_pdl ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, tc::vocab_argmax_pair_kernel, mw64, mx128, p, stages);
+  return cudaLaunchKernelEx(&cfg, tc::vocab_argmax_pair_kernel<STREAM>, mw64, mx128, p, stages);
+}
+cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw64, const CUtensorMap& mx128, const GemmParams& p, int M_cap) {
+  return p.K / tc::BLOCK_K > tc::P_MAX_KB ? launch_vocab_pair<true>(st, mw64, mx128, p, M_cap) : launch_vocab_pair<false>(st, mw64, mx128, p, M_cap);
 }
 
 // Projection of a pass with few tokens (gemm_few.cuh).  ksplit: few::split_for of the shape, non-zero.

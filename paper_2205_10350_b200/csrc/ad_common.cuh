@@ -61,8 +61,9 @@ enum Epi : int {
 //   320 / 400 / 512 tokens: 64-token tiles 366 / 357 / 389 us against 415 / 410 / 458 (128) and 383 / 380 / 410 (32);
 //   800 / 1024 tokens: 64-token tiles 455 / 468 us against 477 / 486 (128);  2048 tokens: 128-token tiles 543 us, 64: 571;
 //   256-token tiles once they alone give two CTAs per SM.
-// A projection whose feature tiles alone outnumber the SMs (the vocabulary) is bound by its weights: one token tile as long as
-// there is one, so that they are read once (90 tokens x 50265 x 768: 19.5 us with two 64-token tiles).
+// A projection whose feature tiles alone outnumber the SMs (the vocabulary) fills them with one token tile, and every further one
+// reads its weights again: one 128-token tile up to 128 tokens (90 tokens x 50265 x 768: 19.5 us with two of 64), then tiles of 128
+// (400 x 768 x 50265: 56 us, 76 with 64-token tiles), of 256 beyond 1536 tokens, where L2 traffic bounds it (2048: 114 against 119 us).
 // K split (projections whose consumer adds partial sums up): as many CTAs as there are SMs at most, 112 for a single token tile
 // (the big model's 25-token pass lost 4 % with 128 one-K-block CTAs).
 struct GeoRule {
@@ -87,8 +88,10 @@ __host__ __device__ inline Geo geometry(const GeoRule& r, int M) {
   if (M <= 64) {
     g.tile = 16;
     while (g.tile < M) g.tile *= 2;
+  } else if (nf >= r.sms) {
+    g.tile = M <= 1536 ? 128 : 256;
   } else if (M <= 128) {
-    g.tile = nf >= r.sms ? 128 : 64;
+    g.tile = 64;
   } else if (M <= 256) {
     g.tile = 32;
   } else if (M <= 1024) {

@@ -1,5 +1,5 @@
 // Output projection fused with the per-tile arg-max for passes with many tokens (hundreds to thousands of packed rows): a
-// persistent, warp-specialised, token-stationary tcgen05 GEMM on pairs of SMs (cta_group::2).
+// persistent, warp-specialised tcgen05 GEMM on pairs of SMs (cta_group::2), token-stationary for K <= 512.
 //
 // Unlike gemm_tc.cuh (weights on the MMA's M side so that a handful of tokens still fill an instruction), the tokens are the M
 // side here: D[token, vocabulary row] = sum_k X[token, k] * E[row, k], one token per tensor-memory lane and one vocabulary row
@@ -7,11 +7,16 @@
 // shared memory, no barrier.
 //
 // A pair of CTAs (a cluster on two neighbouring SMs) works on 256 tokens x 256 vocabulary rows at a time: each CTA holds its 128
-// tokens (128 x K BF16, K <= 512, resident in shared memory as long as the token tile stays) and loads HALF of the vocabulary
+// tokens (128 x K BF16, resident in shared memory as long as the token tile stays) and loads HALF of the vocabulary
 // rows; the paired MMA reads both halves from both shared memories, so a K block brings 16 KB into each SM instead of the 32 KB that
 // one CTA per token tile needs.  2048 tokens x 32000 x 512, back to back: one CTA per token tile 61 us, pairs 64.5 us while the
 // MMAs were issued from a branch on the lane number, 49.5 us (1354 TFLOP/s) issued from a converged warp; 600 tokens 25.5 -> 23.6 us.
 // What bounds it now: 0.4 us per K block against 0.27 us of MMA time, plus 6 us to fill, read the last step out and tear down.
+//
+// K > 512 (STREAM): the token tile no longer fits beside a ring, so its K blocks travel through the ring with the vocabulary's, 32 KB
+// a stage.  One CTA per 128 x 128 tile, as these widths ran before, is bound by the tiles' way through L2 (11.7 TB/s): 2048 tokens x
+// 32000 x 1024 137 -> 82 us (1637 TFLOP/s), 600 x 768 x 50265 68 -> 44 us, 200 x 768 x 50265 29 -> 22 us.  Up to 512 the resident form stays 2 to 4 % ahead
+// (2048 tokens 55 against 57 us).
 //
 // The range of (token tile, 128-row vocabulary tile) units is dealt to the pairs in contiguous pieces, the vocabulary tile
 // running fastest; a pair takes two units a step, one where its piece or the vocabulary ends (the MMA is then 128 columns wide
@@ -42,7 +47,7 @@ namespace tc {
 constexpr int P_THREADS = 576;
 constexpr int P_TOK = 128;                       // tokens per CTA; MMA M = 256
 constexpr int P_VOC = 256;                       // vocabulary rows per step = MMA N
-constexpr int P_MAX_KB = 8;                      // K <= 512
+constexpr int P_MAX_KB = 8;                      // K <= 512: the token tile stays in shared memory
 constexpr int P_MAX_STAGES = 6;
 constexpr int P_BOX = 64;                        // rows per vocabulary box
 constexpr int P_BOX_BYTES = P_BOX * BLOCK_K * 2;    // 8 KiB
@@ -114,11 +119,12 @@ __device__ __forceinline__ void cluster_sync_all() {
 
 // Shared memory a launch needs for kb K blocks and `stages` ring stages.
 inline size_t vocab_pair_smem(int kb, int stages) {
-  return (size_t)kb * P_A_KB_BYTES + (size_t)stages * P_B_STAGE_BYTES + 1024;
+  return (size_t)(kb <= P_MAX_KB ? kb : stages) * P_A_KB_BYTES + (size_t)stages * P_B_STAGE_BYTES + 1024;
 }
 
 // grid = 2 x pairs; cluster (2, 1, 1); block = 576 threads; dynamic smem = vocab_pair_smem(K / 64, stages).
 // map_x: box of 128 token rows x 64; map_w: box of 64 vocabulary rows x 64.  p.bias must be null.
+template <bool STREAM>
 __global__ void __launch_bounds__(P_THREADS, 1)
 vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const GemmParams p,
                          const int stages) {
@@ -137,7 +143,8 @@ vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   const int KB = p.K / BLOCK_K;
   const uint32_t a_base = (smem_u32(smem_raw) + 1023u) & ~1023u;      // resident token tile: KB blocks of 16 KiB
-  const uint32_t b_base = a_base + (uint32_t)(KB * P_A_KB_BYTES);     // ring
+  const uint32_t b_base = STREAM ? a_base + P_A_KB_BYTES : a_base + (uint32_t)(KB * P_A_KB_BYTES);     // ring
+  constexpr uint32_t STAGE_BYTES = STREAM ? P_A_KB_BYTES + P_B_STAGE_BYTES : P_B_STAGE_BYTES;
   constexpr uint32_t TMEM_COLS = 2 * P_VOC;
 
   if (threadIdx.x == 0) {
@@ -147,7 +154,7 @@ vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
       mbar_init(smem_u32(&bar_full[s]), 1);
       mbar_init(smem_u32(&bar_empty[s]), 1);
     }
-    for (int kb = 0; kb < KB; ++kb) mbar_init(smem_u32(&a_full[kb]), 1);
+    for (int kb = 0; kb < KB && !STREAM; ++kb) mbar_init(smem_u32(&a_full[kb]), 1);
     mbar_init(smem_u32(&a_empty), 1);
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&acc_full[b]), 1);
@@ -192,7 +199,7 @@ vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
       if (!p.M_ptr) pdl_wait();                            // operator-level call: the matrix may have just been written
       const int pw = warp - 8;
       const uint32_t full = smem_u32(&bar_full[pw]), empty = smem_u32(&bar_empty[pw]), full0 = cluster_addr(full, 0);
-      const uint32_t dst = b_base + (uint32_t)(pw * P_B_STAGE_BYTES);
+      const uint32_t dst = b_base + (uint32_t)pw * STAGE_BYTES;
       int u = u_lo, first_kb = 0;                          // the step at unit u starts with K block number first_kb of the sequence
       bool ok = true;
       for (int g = pw; ok && u < u_hi;) {
@@ -206,9 +213,13 @@ vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
           const int kb = g - first_kb;
           // rows beyond the vocabulary are filled with zeros and still count their bytes
           if (elect_one()) {
-            if (rank == 0) mbar_expect_tx(full, (uint32_t)(2 * st.width * P_BOX_BYTES));
+            if (rank == 0) mbar_expect_tx(full, (uint32_t)(2 * st.width * P_BOX_BYTES + (STREAM ? 2 * P_A_KB_BYTES : 0)));
             tma_load_2d_pair(dst, &map_w, kb * BLOCK_K, row, full0);
             if (st.width == 2) tma_load_2d_pair(dst + P_BOX_BYTES, &map_w, kb * BLOCK_K, row + P_BOX, full0);
+          }
+          if (STREAM) {
+            if (g == pw) pdl_wait();
+            if (elect_one()) tma_load_2d_pair(dst - P_A_KB_BYTES, &map_x, kb * BLOCK_K, (2 * st.t + (int)rank) * P_TOK, full0);
           }
           __syncwarp();
         }
@@ -218,7 +229,7 @@ vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
     }
   } else if ((warp >= 8 + stages && warp < 15) || warp > 15) {
     // ---- the resident token tile: loader l of n takes K blocks l, l + n, ... ----
-    {
+    if (!STREAM) {
       const int l = warp > 15 ? warp - 16 : 2 + warp - 8 - stages, n = 9 - stages;
       pdl_wait();
       int cur_t = -1;
@@ -248,7 +259,7 @@ vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
       const uint32_t idesc2 = make_idesc(2 * P_TOK, P_VOC), idesc1 = make_idesc(2 * P_TOK, BLOCK_N_FEAT);
       const uint64_t desc_a0 = make_smem_desc(a_base);
       const uint64_t desc_b0 = make_smem_desc(b_base);
-      const uint64_t a_step = (uint64_t)(P_A_KB_BYTES >> 4), b_step = (uint64_t)(P_B_STAGE_BYTES >> 4);
+      const uint64_t a_step = (uint64_t)(P_A_KB_BYTES >> 4), b_step = (uint64_t)(STAGE_BYTES >> 4);
       bool ok = true;
       int cur_t = -1, it = 0, s = 0;
       uint32_t uses = 0, phase = 0;                        // ring position of the next K block
@@ -258,10 +269,11 @@ vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
         uint64_t desc_a = desc_a0;
         uint32_t accumulate = 0;
         for (int kb = 0; kb < KB; ++kb) {
-          if (decltype(fresh)::value && !mbar_wait_cluster(smem_u32(&a_full[kb]), (uses - 1) & 1u, p.status)) return false;
+          if (!STREAM && decltype(fresh)::value && !mbar_wait_cluster(smem_u32(&a_full[kb]), (uses - 1) & 1u, p.status)) return false;
           if (!mbar_wait_cluster(smem_u32(&bar_full[s]), phase, p.status)) return false;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint64_t desc_b = desc_b0 + b_step * (uint64_t)s;
+          if (STREAM) desc_a = desc_a0 + b_step * (uint64_t)s;
           if (elect_one()) {
 #pragma unroll
             for (int k4 = 0; k4 < BLOCK_K / UMMA_K; ++k4) umma_bf16_pair(acc, desc_a + 2 * k4, desc_b + 2 * k4, idesc, k4 == 0 ? accumulate : 1u);
@@ -269,7 +281,7 @@ vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid
           }
           __syncwarp();
           accumulate = 1u;
-          desc_a += a_step;
+          if (!STREAM) desc_a += a_step;
           if (++s == stages) { s = 0; phase ^= 1u; }
         }
         return true;

@@ -12,7 +12,8 @@ DEV = "cuda:0"
 
 
 @pytest.mark.parametrize("M,d,V", [(65, 768, 18945), (100, 1024, 19000), (128, 512, 18944), (127, 256, 50265), (129, 512, 19073),
-                                   (257, 448, 10001), (300, 512, 32000), (600, 512, 32000), (1025, 128, 5121), (385, 64, 12672)])
+                                   (257, 448, 10001), (300, 512, 32000), (600, 512, 32000), (1025, 128, 5121), (385, 64, 12672),
+                                   (129, 768, 19073), (300, 1024, 13000), (1025, 832, 5121)])
 def test_argmax_tiles(M, d, V):
     g = torch.Generator(DEV).manual_seed(M + V)
     x = torch.randn((M, d), generator=g, device=DEV).bfloat16()
