@@ -787,13 +787,24 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   return AD_OK;
 }
 
-// Whether the few-query kernel (attention_few.cuh) serves an attention of pass pc: BF16, 64-wide heads, the keys within four
-// rounds of its warps, and a grid of at most one wave.
-bool attention_is_few(const ad_handle* h, const PassCfg& pc, int max_keys) {
+// Whether the few-query kernel (attention_few.cuh) serves an attention of pass pk: BF16, 64-wide heads, the keys within four rounds
+// of its warps, and a grid of a few waves at most.  The grid counts what the pass could hold; CTAs of rows that have ended, of
+// blocks that are shorter and of a drafter's prefix that has not grown leave at once.  A wave costs 4 to 7 us, the projections that
+// are kernels of their own otherwise 12 us a layer, so a verification pass may need three waves at capacity, a drafter's pass
+// (on average half of its capacity) four; an encoder's rows are as long as they are announced, and there is one projection to gain:
+// one wave.  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30: 214 -> 174 us; batch 24, 12:
+// 237 -> 196; batch 20, 1: 188 -> 160; batch of 5 with drafter 442 -> 373; 1024 wide, batch 2, 40: 272 -> 226; batch 3 with drafter
+// 662 -> 600.  Beyond: base batch 32 x 64 (seven waves) 270 -> 315, 1024 wide batch 16 x 1 (four) 239 -> 284.  Wide models with fewer than eight
+// queries a row stay at one wave: their CTAs read two weight slices each for a tile that is mostly padding (768 wide, batch 12, 1: 202
+// against 210).
+bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   const ad_model_cfg& c = h->cfg;
+  const PassCfg& pc = h->pass[pk];
   if (!g_fuse_attn_proj || !h->bf16 || !h->pre2 || c.d_model != c.n_heads * 64 || c.d_model % 128 || c.d_model > 128 * few::MAX_WARPS) return false;
+  const int split = few::att_few_split(c.d_model);
   if (max_keys > few::MAX_ROUNDS * few::AK * few::att_few_warps(c.d_model)) return false;
-  return (long)h->cfg.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * few::att_few_split(c.d_model) <= num_sms();
+  const int waves = pk == PK_ENCODE || (split > 1 && pc.seg_max < 8) ? 1 : pk == PK_DRAFT ? 4 : 3;
+  return (long)c.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * split <= (long)waves * num_sms();
 }
 
 // Attention with its output projection (partial sums per head in pre2) and, with wq, the query projection of x = yb.
@@ -910,7 +921,7 @@ int self_attention_sublayer(ad_handle* h, int pk, const Mat& wqkv, const float* 
   AD_TRY(gemm(h, EPI_SCATTER, wqkv, h->yb, pk, pc.plan.M, pc.M_cap, p, embed_of));
   bool fused = false;
   const int max_keys = pk == PK_VERIFY ? h->dims.max_tgt : pc.seg_max;
-  if (attention_is_few(h, pc, max_keys)) {
+  if (attention_is_few(h, pk, max_keys)) {
     AD_TRY(attention_few(h, pc, kbuf, vbuf, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, max_keys, wo));
     return layernorm(h, pc, head_partials(h, pc), bo, lng, lnb);
   }
@@ -1079,7 +1090,7 @@ int decoder_pass(ad_handle* h, int pk, Model& m) {
     // projection, so it is split along K and the attention kernel adds the partial sums (and the bias) as it
     // loads its queries.
     bool fused_x = false;
-    if (attention_is_few(h, pc, c.max_src)) {
+    if (attention_is_few(h, pk, c.max_src)) {
       AD_TRY(attention_few(h, pc, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->st.cross_base, nullptr, h->st.srclen, c.max_src,
                            L.co, &L.cq, L.cbq));
       AD_TRY(layernorm(h, pc, head_partials(h, pc), L.cbo, L.ln2g, L.ln2b));
