@@ -272,8 +272,8 @@ def kernel_table(dec, shape, drafts, k, pk):
             N, K = (int(t[1:]) for t in name.split()[1:3])
             out_b = 4 if "f32" in name else (0 if "argmax" in name else 2)
             g["bytes"] += N * K * 2 + k * K * 2 + k * N * out_b
-        elif name.startswith("attention"):
-            g["bytes"] += 2 * 40 * d * 2 + 2 * k * d * 2 + (d * d * 2 + 8 * k * d * 4 if "out_proj" in name else 0)
+        elif "attention" in name:
+            g["bytes"] += 2 * 40 * d * 2 + 2 * k * d * 2 + (d * d * 2 + 8 * k * d * 4 if "out_proj" in name else 0) + (d * d * 2 if "q_proj" in name else 0)
         elif "layernorm" in name:
             g["bytes"] += 9 * k * d * 4 + k * d * 6
     total = sum(g["us"] for g in groups.values())
@@ -476,8 +476,8 @@ def run_ours(args, rank, world, local_rank):
     alg = step_bytes(synth.BASE, sum_src=mean_S * iters, sum_keys=float(glen.mean()) * iters, sum_k=agg["offered"], n_steps=iters) / iters
     ach = alg / (loop_us * 1e-6) / 1e9
     wv = weight_bytes(synth.BASE)
-    roofline = dict(bound="hbm", kernel="verification step: the 56-kernel chain of one loop iteration (6 decoder layers of 9 kernels, "
-                    "projection + arg-max, accept + commit + plan and embedding of the next block), graph-replayed", achieved=ach, peak=pk["hbm_gbs"], unit="GB/s",
+    roofline = dict(bound="hbm", kernel="verification step: the 50-kernel chain of one loop iteration (6 decoder layers of 8 kernels, "
+                    "projection + arg-max, accept + commit + plan of the next block), graph-replayed", achieved=ach, peak=pk["hbm_gbs"], unit="GB/s",
                     frac=ach / pk["hbm_gbs"], traffic=ncu_counter("step_block40_bytes"), peak_source=pk["source"], algorithmic_bytes=alg,
                     weight_bytes=wv, us_per_step_in_loop=loop_us, hbm_floor_us=alg / (pk["hbm_gbs"] * 1e9) * 1e6,
                     note="time = device time of the decode loops / loop iterations (weights L2-warm between the iterations of a "
@@ -597,9 +597,9 @@ def bench_extras(args, binding, dec, w, dev, pk, flush, t_src, t_len, t_max, t_o
     t_v32 = statistics.mean(_events(dec.stream, vocab32_once, 20))
     fl_v32 = 2.0 * M32 * V * d
     extras["tensor_regime"]["projection_kernel"] = dict(
-        kernel="vocab_argmax_persistent_kernel, vocabulary 32000 x 512, 2048 tokens", us=t_v32, flops=fl_v32,
+        kernel="vocab_argmax_pair_kernel, vocabulary 32000 x 512, 2048 tokens", us=t_v32, flops=fl_v32,
         tflops=fl_v32 / (t_v32 * 1e-6) / 1e12, frac_of_burst_peak=fl_v32 / (t_v32 * 1e-6) / 1e12 / pk["bf16_tflops"],
-        note="timed alone with CUDA events (weights L2-warm); ncu counters in profiles/vocab_argmax_persistent_base_M2048_ncu_full.txt")
+        note="timed alone with CUDA events (weights L2-warm)")
 
     # the other workload recipes (and shapes) through ad_generate, the CPU checker's bounded sample beside each
     if not args.skip_workloads:
