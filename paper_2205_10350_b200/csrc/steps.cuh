@@ -372,8 +372,7 @@ template <int THREADS>
 __device__ __forceinline__ float group_sum(float v, float* red, int tid, int half) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  group_sync<THREADS>(half);       // red may still be read from a previous call
-  if ((tid & 31) == 0) red[tid >> 5] = v;
+  if ((tid & 31) == 0) red[tid >> 5] = v;      // two calls in turn use two buffers: no barrier in front
   group_sync<THREADS>(half);
   float t = 0.f;
 #pragma unroll
@@ -420,7 +419,7 @@ __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, 
     const float a = v.x - mean, b = v.y - mean, c = v.z - mean, e = v.w - mean;
     vs = a * a + b * b + c * c + e * e;
   }
-  const float inv = rsqrtf(group_sum<THREADS>(vs, red, tid, half) / (float)p.d + p.eps);
+  const float inv = rsqrtf(group_sum<THREADS>(vs, red + THREADS / 32, tid, half) / (float)p.d + p.eps);
   if (on) {
     float4 o;
     o.x = w.g.x * ((v.x - mean) * inv) + w.b.x;
@@ -436,7 +435,7 @@ __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, 
 template <typename ActT, int THREADS>
 __global__ void __launch_bounds__(THREADS)
 layernorm_kernel(const LnParams p, ActT* __restrict__ yb) {
-  __shared__ float red[THREADS / 32];
+  __shared__ float red[2 * (THREADS / 32)];
   trace_mark(TR_LN, 0);
   pdl_launch();
   const int m = blockIdx.x, M = plan_load(p.M_ptr);
@@ -462,7 +461,7 @@ constexpr int LN_ROWS = 1536;
 template <typename ActT>
 __global__ void __launch_bounds__(256, 2)
 layernorm_many_kernel(const LnParams p, ActT* __restrict__ yb) {
-  __shared__ float red[2][8];
+  __shared__ float red[2][16];
   trace_mark(TR_LN, 0);
   pdl_launch();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
