@@ -237,6 +237,12 @@ int ad_debug_profile_verify(ad_handle* h, const int32_t* drafts, const int32_t* 
  * FFN1, FFN2; then the vocabulary projection.  Synchronises the stream. */
 int ad_debug_stage_timeline(ad_handle* h, uint64_t* stamps, int32_t capacity, int32_t* n_stages);
 
+/* Debug, host only: launch shapes of the tensor-core projections of a verification pass of a handle for cfg, in launch order.
+ * rows (host, capacity x 7) receives per projection {epilogue, N, K, CTAs launched, most CTAs that any token count up to
+ * max_batch * kmax asks for, bytes of dynamic shared memory launched with, most bytes asked for}; *n_rows their count.
+ * Projections that run on other kernels are left out (FP32 models: all). */
+int ad_debug_projection_shapes(const ad_model_cfg* cfg, int32_t* rows, int32_t capacity, int32_t* n_rows);
+
 /* Debug: exercises the bounded-wait mechanism that every mbarrier wait of the GEMM kernels uses (a wait gives up
  * after a time budget measured on the GPU's global timer: 20 ms in the kernels, budget_us here).  Launches one tiny
  * kernel that waits, for at most budget_us (1..65536) microseconds, on a barrier phase that nothing completes; the

@@ -161,7 +161,7 @@ struct ad_handle {
     int once;            // ... and its kernels outside the loop
   };
   std::map<std::string, GraphEntry> graphs;
-  std::map<std::tuple<int, int, int, int>, TcShape> tc_shapes;   // launch shapes by (pass kind, N, K, split)
+  std::map<std::tuple<int, int, int, int, int, int, int, int, int>, TcShape> tc_shapes;   // see cached_shape
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
   int launches = 0;          // kernels launched by the last ad_generate (direct) or per graph replay
   // Persistent decoder pass (one kernel for the decoder stack + projection): per pass kind, whether it applies and its
@@ -475,11 +475,19 @@ int num_sms() {
   return n[dev];
 }
 
+// Dynamic shared memory of a pass of M tokens: the ring doubles as the epilogue's transposition buffer (up to 128 rows of 132 floats)
+// and the few-token partial sums.
+int tc_smem_need(const GeoRule& r, int M, int budget) {
+  const Geo g = geometry(r, M);
+  const int need = g.few ? (int)few::red_bytes(2)
+                         : std::max(tc::ring_stages(g.tile, (r.K / tc::BLOCK_K + g.ksplit - 1) / g.ksplit, budget) * (tc::A_STAGE_BYTES + g.tile * tc::BLOCK_K * 2),
+                                    std::min(g.tile, 128) * 132 * 4);
+  return need + 1024;
+}
 // Launch shape of the tensor-core projection kernel for passes of at most M_cap tokens: the most CTAs any token count asks for
 // and the shared memory of its ring.  Up to one CTA per SM: ~200 KB, so that the ring is as deep as it can be; with more CTAs
 // half of that, so that two CTAs share an SM: up to twice the SM count the whole grid is then resident at once, beyond that
 // one CTA's prologue and epilogue overlap the other's K loop.
-
 TcShape tc_shape(const GeoRule& r, int M_cap, bool exact) {
   TcShape sh = {1, 0, 0};
   auto each = [&](auto f) {
@@ -489,14 +497,7 @@ TcShape tc_shape(const GeoRule& r, int M_cap, bool exact) {
   };
   each([&](int M) { sh.ctas = std::max(sh.ctas, tc::geometry_ctas(r, M)); });
   sh.budget = (sh.ctas > num_sms() ? 100 : 200) * 1024;
-  // the ring doubles as the epilogue's transposition buffer (up to 128 rows of 132 floats) and the few-token partial sums
-  each([&](int M) {
-    const Geo g = geometry(r, M);
-    const int need = g.few ? (int)few::red_bytes(2)
-                           : std::max(tc::ring_stages(g.tile, (r.K / tc::BLOCK_K + g.ksplit - 1) / g.ksplit, sh.budget) * (tc::A_STAGE_BYTES + g.tile * tc::BLOCK_K * 2),
-                                      std::min(g.tile, 128) * 132 * 4);
-    sh.smem = std::max(sh.smem, need + 1024);
-  });
+  each([&](int M) { sh.smem = std::max(sh.smem, tc_smem_need(r, M, sh.budget)); });
   return sh;
 }
 
@@ -634,6 +635,15 @@ cudaError_t launch_simt_few(cudaStream_t st, const Mat& W, const void* x, const 
   }
 }
 
+// Launch shape of a rule, worked out once per handle.  The key is everything the shape follows from: projections of equal N and K may
+// still differ in their rule (a vocabulary as large as the feed-forward width never takes the few-token kernel, FFN1 does).
+const TcShape& cached_shape(ad_handle* h, const GeoRule& r, int M_cap) {
+  const auto key = std::make_tuple(r.N, r.K, r.max_tile, r.max_split, r.sms, r.few_split, r.few_tokens, r.fixed_tile, M_cap);
+  auto it = h->tc_shapes.find(key);
+  if (it == h->tc_shapes.end()) it = h->tc_shapes.emplace(key, tc_shape(r, M_cap, false)).first;
+  return it->second;
+}
+
 // embed_of: the operand is the embedding of pass pk's tokens (first projection of a pass, few-token kernel only).
 // split: the result is partial sums that the consumer adds up (EPI_F32).
 int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int* M_ptr, int M_cap, GemmParams p, const Model* embed_of = nullptr,
@@ -665,10 +675,7 @@ int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int
     // (a pass with a 256-token tile also has the 128-row map of its token operand)
     e = launch_vocab_persistent(h->stream, W.map64, X.map_for(pk, tc::P_TOK), p, M_cap);
   } else if (h->bf16) {
-    const auto key = std::make_tuple(pk, W.N, W.K, split ? 1 : 0);
-    auto it = h->tc_shapes.find(key);
-    if (it == h->tc_shapes.end()) it = h->tc_shapes.emplace(key, tc_shape(p.rule, M_cap, false)).first;
-    const TcShape& sh = it->second;
+    const TcShape& sh = cached_shape(h, p.rule, M_cap);
     switch (epi) {
       case EPI_F32: e = launch_tc<EPI_F32>(h->stream, W.map, X.map[pk], p, sh, W.ptr, X.ptr); break;
       case EPI_ACT: e = launch_tc<EPI_ACT>(h->stream, W.map, X.map[pk], p, sh, W.ptr, X.ptr); break;
@@ -1929,6 +1936,39 @@ extern "C" int ad_debug_stage_timeline(ad_handle* h, uint64_t* stamps, int32_t c
   AD_CUDA(h, cudaStreamSynchronize(h->stream));
   AD_CUDA(h, cudaMemcpy(stamps, h->mega_timeline, sizeof(uint64_t) * 2 * (size_t)n, cudaMemcpyDeviceToHost));
   *n_stages = n;
+  return AD_OK;
+}
+
+extern "C" int ad_debug_projection_shapes(const ad_model_cfg* cfg, int32_t* rows, int32_t capacity, int32_t* n_rows) {
+  std::string why;
+  if (!rows || !n_rows || capacity < 1) return fail(nullptr, AD_ERR_ARG, "null output pointer");
+  if (check_cfg(cfg, &why) != AD_OK) return fail(nullptr, AD_ERR_ARG, why);
+  ad_handle h;
+  h.cfg = *cfg;
+  h.bf16 = cfg->dtype == AD_DTYPE_BF16;
+  h.esz = h.bf16 ? 2 : 4;
+  layout(&h, nullptr);
+  *n_rows = 0;
+  if (!h.bf16) return AD_OK;
+  const int d = cfg->d_model, F = cfg->d_ffn;
+  // the projections of a decoder pass in launch order; the query projection in both of its forms
+  struct { int epi, N, K; bool split, bias; } list[] = {
+      {EPI_SCATTER, 3 * d, d, false, true}, {EPI_F32, d, d, true, false}, {EPI_ACT, d, d, false, true}, {EPI_F32, d, d, true, false},
+      {EPI_ACT, F, d, false, true},         {EPI_F32, d, F, true, false}, {EPI_ARGMAX, cfg->vocab, d, false, false}, {EPI_F32, cfg->vocab, d, false, false}};
+  const PassCfg& pc = h.pass[PK_VERIFY];
+  for (const auto& q : list) {
+    const GeoRule r = geo_rule(pc, q.epi, q.N, q.K, q.split, q.bias);
+    if (always_few(pc, r) || (q.epi == EPI_ARGMAX && pc.ntile == 256 && vocab_goes_persistent(q.K, q.N, pc.M_cap, nullptr))) continue;
+    const TcShape& sh = cached_shape(&h, r, pc.M_cap);
+    int ctas = 0, smem = 0;
+    for (int M = 0; M <= pc.M_cap; ++M) {
+      ctas = std::max(ctas, tc::geometry_ctas(r, M));
+      smem = std::max(smem, tc_smem_need(r, M, sh.budget));
+    }
+    if (*n_rows >= capacity) return fail(nullptr, AD_ERR_CAPACITY, "ad_debug_projection_shapes: more projections than rows");
+    const int32_t row[7] = {q.epi, q.N, q.K, sh.ctas, ctas, sh.smem, smem};
+    memcpy(rows + 7 * (size_t)(*n_rows)++, row, sizeof(row));
+  }
   return AD_OK;
 }
 

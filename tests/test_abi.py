@@ -82,3 +82,18 @@ def test_null_handle_calls_are_rejected(lib):
     assert lib.ad_encode(None, None, 1, None, 1, 1) == binding.AD_ERR_ARG
     assert lib.ad_commit(None, None, 1) == binding.AD_ERR_ARG
     assert lib.ad_destroy(None) == binding.AD_ERR_ARG
+
+
+@pytest.mark.parametrize("d,heads,ffn,vocab", [(512, 8, 2048, 2048), (512, 8, 2048, 1536), (512, 8, 512, 512), (256, 4, 1024, 1024),
+                                               (256, 4, 1024, 768), (1024, 16, 4096, 3072), (768, 12, 3072, 3072), (512, 8, 2048, 32000)])
+def test_projection_launches_cover_every_token_count(lib, d, heads, ffn, vocab):
+    """Grid and shared memory of every projection of a verification pass against what its launch rule asks for at any token
+    count, for vocabularies as large as another projection's output: the two share (N, K) and nothing else."""
+    for batch, kmax in ((1, 40), (2, 64), (3, 50), (5, 40), (32, 64), (75, 61)):
+        cfg = binding.ModelCfg(d, heads, ffn, vocab, 2, 2, 1, batch, 64, 64, kmax, 0, 1, 2, 3, 1e-5, 0)
+        rows, n = (C.c_int32 * (7 * 16))(), C.c_int32()
+        assert lib.ad_debug_projection_shapes(C.byref(cfg), rows, 16, C.byref(n)) == 0
+        assert n.value >= 1
+        for i in range(n.value):
+            epi, N, K, ctas, need_ctas, smem, need_smem = rows[7 * i: 7 * i + 7]
+            assert ctas >= need_ctas and smem >= need_smem, (batch * kmax, epi, N, K, ctas, need_ctas, smem, need_smem)

@@ -42,6 +42,22 @@ def test_few_token_passes_follow_the_checker(d, ffn, batch, k, src, tgt):
     dec.close()
 
 
+def test_vocabulary_as_large_as_the_feed_forward_width():
+    """The projection onto the vocabulary and FFN1 share (N, K) in one verification pass and have different launch rules."""
+    from paper_2205_10350_b200 import binding
+    shape = synth.ModelShape("few_same_width", 256, 4, 1024, 1024, 1, 2, "bf16")
+    w = synth.make_weights(shape, 0)
+    model = O.Model(shape, w, max_pos=64)
+    src = np.random.default_rng(3).integers(4, shape.vocab, size=(3, 11)).astype(np.int32)
+    lens = np.array([11, 7, 10], np.int32)
+    for k in (50, 33, 7):                    # 150, 99 and 21 tokens of a capacity of 150
+        dec = binding.AggressiveDecoder(shape, w, max_batch=3, max_src=11, max_tgt=50, kmax=50)
+        streams = [np.resize(model.state(src[b, : lens[b]], cap=50).greedy(50)[0], 50).astype(np.int32) for b in range(3)]
+        stats = lockstep(dec, model, src, lens, streams, k, [50] * 3, tol=5e-2, max_steps=2)
+        assert stats["steps"] > 0
+        dec.close()
+
+
 @pytest.mark.parametrize("mode,run_drafter,k", [("IAD", False, 7), ("IAD", False, 1), ("GAD", True, 5), ("GAD", True, 12)])
 def test_loop_planned_by_the_accept_kernel_equals_one_kernel_per_plan(mode, run_drafter, k, monkeypatch):
     """Whole loops of a ragged batch: planning inside the accept kernel and planning in kernels of their own give the same
