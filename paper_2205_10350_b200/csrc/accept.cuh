@@ -71,8 +71,8 @@ __device__ __forceinline__ void scan_tiles(const float* __restrict__ val, const 
 #pragma unroll
     for (int h = 0; h < H; ++h)
 #pragma unroll
-      for (int u = 0; u < U; ++u) {                       // (a lane's tiles ascend, and so do their ids)
-        if (pv[h][u] > v[h]) { v[h] = pv[h][u]; idx[h] = pi[h][u]; }
+      for (int u = 0; u < U; ++u) {
+        if (pv[h][u] > v[h] || (pv[h][u] == v[h] && pi[h][u] < idx[h])) { v[h] = pv[h][u]; idx[h] = pi[h][u]; }   // (-inf included)
         if (COUNT) higher[h] += pc[h][u];
       }
   }
@@ -140,7 +140,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
   const bool relaxed = beta >= 1 && !to_drafts;
   int* pred = (to_drafts ? st.drafts : st.pred) + (size_t)b * dm.kmax;
   auto decide = [&](int i, float v, int idx, int higher) {      // lane 0 of the position's warp
-    int choice = idx;
+    int choice = idx < dm.vocab ? idx : 0;                        // a position without any ordered score (NaN) still gets an id that exists
     if (relaxed) {
       const int did = draft_id[off + i];
       if (did >= 0 && higher <= beta - 1 && v - draft_val[off + i] <= tau) choice = did;
@@ -319,7 +319,8 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
       if (lane == 0) { pl.seg_off[r] = o0; pl.seg_len[r] = nr; pl.key_base[r] = o0; pl.row_nk[r] = nr; }
       for (int i = lane; i < nr; i += 32) {
         const int m = o0 + i;
-        const int tok = i == 0 ? dm.bos : (i <= lr ? __ldcg(st.out_ids + (size_t)r * dm.max_tgt + i - 1) : dm.mask);
+        int tok = i == 0 ? dm.bos : (i <= lr ? __ldcg(st.out_ids + (size_t)r * dm.max_tgt + i - 1) : dm.mask);
+        if (!id_in_vocab(tok, dm)) { latch_error(st.status, AD_ERR_ARG); tok = dm.pad; }
         pl.tok_row[m] = r; pl.tok_pos[m] = i; pl.tok_id[m] = tok; pl.kv_slot[m] = m; pl.att_n[m] = nr;
       }
       for (int i = lane; i < kr; i += 32) st.gidx[boff + i] = o0 + lr + 1 + i;

@@ -2084,7 +2084,7 @@ namespace {
 // Arg-max over tiles for M rows without any decoding state: four rows per CTA, a warp each (few rows: one row per CTA, whose
 // warps share its tiles), up to eight tiles per lane in flight.  grid = ceil(M / rows), block = 128.
 __global__ void __launch_bounds__(128)
-argmax_rows_kernel(const float* __restrict__ part_val, const int* __restrict__ part_idx, int n_tiles, int M, int rows, int* __restrict__ out) {
+argmax_rows_kernel(const float* __restrict__ part_val, const int* __restrict__ part_idx, int n_tiles, int M, int rows, int vocab, int* __restrict__ out) {
   __shared__ float s_v[4];
   __shared__ int s_i[4];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2109,7 +2109,7 @@ argmax_rows_kernel(const float* __restrict__ part_val, const int* __restrict__ p
         if (pv[u] > v || (pv[u] == v && pi[u] < idx)) { v = pv[u]; idx = pi[u]; }
     }
     tc::warp_argmax(v, idx);
-    if (rows > 1 && lane == 0) out[m] = idx;
+    if (rows > 1 && lane == 0) out[m] = idx < vocab ? idx : 0;       // (no ordered score, NaN: still an id that exists)
   }
   if (rows == 1) {
     if (lane == 0) { s_v[warp] = v; s_i[warp] = idx; }
@@ -2117,7 +2117,7 @@ argmax_rows_kernel(const float* __restrict__ part_val, const int* __restrict__ p
     if (threadIdx.x == 0) {
       for (int w = 1; w < 4; ++w)
         if (s_v[w] > v || (s_v[w] == v && s_i[w] < idx)) { v = s_v[w]; idx = s_i[w]; }
-      out[m] = idx;
+      out[m] = idx < vocab ? idx : 0;
     }
   }
 }
@@ -2170,7 +2170,7 @@ extern "C" int ad_vocab_argmax(const void* x, const void* emb, int32_t dtype, in
   if (e != cudaSuccess) return AD_ERR_CUDA;
   if (!argmax) return AD_OK;   // projection kernel alone: partials stay in scratch
   const int rows = M <= num_sms() ? 1 : 4;
-  e = launch_k(argmax_rows_kernel, dim3((M + rows - 1) / rows), dim3(128), 0, st, (const float*)pv, (const int*)pi, tiles, M, rows, argmax);
+  e = launch_k(argmax_rows_kernel, dim3((M + rows - 1) / rows), dim3(128), 0, st, (const float*)pv, (const int*)pi, tiles, M, rows, vocab, argmax);
   return e == cudaSuccess ? AD_OK : AD_ERR_CUDA;
 }
 

@@ -183,6 +183,7 @@ gemm_f32_kernel(const float* __restrict__ w, const float* x, const GemmParams p,
         if (n < p.N) {
           const float s = sum_of(f, tok);
           if (s > v) { v = s; id = n; }
+          if (id == 0x7fffffff) id = n;                              // (the lowest one where no score compares above -inf)
           if (p.draft_val && n != did && s > dval) ++cnt;           // other features that score strictly higher
         }
       }

@@ -513,7 +513,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
         const float dval = relaxed ? dval_s[tok] : 0.f;
         const int did = relaxed ? did_s[tok] : -1;
         float best = -INFINITY;
-        int best_n = 0x7fffffff, cnt = 0;
+        int best_n = n0 + grp * 64, cnt = 0;       // (an id that exists also where no score compares above -inf)
         if (quad * 32 < ntok_all) {
           for (int c = grp * 64; c < grp * 64 + 64; c += 16) {
             float acc[16];

@@ -222,7 +222,9 @@ plan_draft_kernel(DevState st, PassPlan blk, PassPlan plan, Dims dm) {
       const int m = off + i;
       plan.tok_row[m] = b;
       plan.tok_pos[m] = i;
-      plan.tok_id[m] = (i == 0) ? dm.bos : (i <= len ? st.out_ids[(size_t)b * dm.max_tgt + i - 1] : dm.mask);
+      int tok = (i == 0) ? dm.bos : (i <= len ? st.out_ids[(size_t)b * dm.max_tgt + i - 1] : dm.mask);
+      if (!id_in_vocab(tok, dm)) { latch_error(st.status, AD_ERR_ARG); tok = dm.pad; }
+      plan.tok_id[m] = tok;
       plan.kv_slot[m] = m;
       plan.att_n[m] = n;
     }
