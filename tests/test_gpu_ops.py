@@ -114,3 +114,29 @@ def test_tensor_regime_sizes_on_sampled_rows():
     for j, m in enumerate(rows):
         i1, v1, i2, v2 = OPS.top2(lg[j])
         assert got[m] == i1 if v1 - v2 > 1e-4 else got[m] in (i1, i2)
+
+
+@pytest.mark.parametrize("dtype,M,K,N", [("bf16", 300, 512, 512), ("bf16", 40, 2048, 1536), ("fp32", 64, 256, 512)])
+def test_operator_calls_that_read_what_the_call_before_them_wrote(dtype, M, K, N):
+    """Calls issued back to back without synchronisation, each with the first result row of the call before as its bias: a call may
+    begin before the one in front of it has ended, but must not read its bias (or any other input) before that."""
+    lib = binding.load()
+    dt, code = (torch.bfloat16, binding.AD_DTYPE_BF16) if dtype == "bf16" else (torch.float32, binding.AD_DTYPE_FP32)
+    g = torch.Generator(DEV).manual_seed(N)
+    x = torch.randn((M, K), generator=g, device=DEV).to(dt)
+    W = (torch.randn((N, K), generator=g, device=DEV) * 0.02).to(dt)
+    bias = torch.randn(N, generator=g, device=DEV)
+    outs = [torch.zeros((M, N), device=DEV) for _ in range(20)]
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    torch.cuda.synchronize()
+    stream = torch.cuda.current_stream().cuda_stream
+    prev = bias
+    for y in outs:
+        assert lib.ad_linear(x.data_ptr(), W.data_ptr(), prev.data_ptr(), code, M, K, N, y.data_ptr(), st.data_ptr(), stream) == binding.AD_OK
+        prev = y
+    torch.cuda.synchronize()
+    ref = bias                                # the same calls one at a time
+    for y in outs:
+        ref = binding.linear(x, W, ref[0].clone() if ref.dim() == 2 else ref)
+        assert torch.equal(y, ref)
+    assert int(st.item()) == 0
