@@ -237,6 +237,9 @@ int ad_debug_profile_verify(ad_handle* h, const int32_t* drafts, const int32_t* 
  * FFN1, FFN2; then the vocabulary projection.  Synchronises the stream. */
 int ad_debug_stage_timeline(ad_handle* h, uint64_t* stamps, int32_t capacity, int32_t* n_stages);
 
+/* Debug: number of captured graphs that the handle keeps. */
+int ad_debug_graph_count(const ad_handle* h, int32_t* n);
+
 /* Debug, host only: launch shapes of the tensor-core projections of a verification pass of a handle for cfg, in launch order.
  * rows (host, capacity x 7) receives per projection {epilogue, N, K, CTAs launched, most CTAs that any token count up to
  * max_batch * kmax asks for, bytes of dynamic shared memory launched with, most bytes asked for}; *n_rows their count.

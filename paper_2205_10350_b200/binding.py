@@ -22,7 +22,7 @@ EXPORTS = [
     "ad_weight_counts", "ad_query_workspace", "ad_create", "ad_destroy", "ad_last_error", "ad_encode",
     "ad_verify_block", "ad_commit", "ad_force_commit", "ad_generate", "ad_draft_block", "ad_get_state", "ad_sync", "ad_set_acceptance",
     "ad_debug_logits", "ad_debug_encoder_memory", "ad_debug_stage_timeline", "ad_debug_profile_verify", "ad_vocab_argmax_scratch_bytes", "ad_vocab_argmax",
-    "ad_vocab_argmax_static", "ad_debug_projection_shapes", "ad_debug_wait_probe", "ad_debug_grid_barrier_probe",
+    "ad_vocab_argmax_static", "ad_debug_graph_count", "ad_debug_projection_shapes", "ad_debug_wait_probe", "ad_debug_grid_barrier_probe",
     "ad_linear",
 ]
 
@@ -95,6 +95,7 @@ def load():
         "ad_vocab_argmax": (C.c_int, [vp, vp, i32, i32, i32, i32, vp, vp, sz, vp, vp]),
         "ad_vocab_argmax_static": (C.c_int, [vp, vp, i32, i32, i32, i32, vp, vp, vp]),
         "ad_linear": (C.c_int, [vp, vp, vp, i32, i32, i32, i32, vp, vp, vp]),
+        "ad_debug_graph_count": (C.c_int, [vp, vp]),
         "ad_debug_projection_shapes": (C.c_int, [C.POINTER(ModelCfg), vp, i32, vp]),
         "ad_debug_wait_probe": (C.c_int, [vp, i32, vp, vp]),
         "ad_debug_grid_barrier_probe": (C.c_int, [i32, i32, i32, i32, vp, sz, vp, vp, vp]),
@@ -265,6 +266,12 @@ class AggressiveDecoder:
                                                      C.byref(n)), self.h)
         raw = names.raw
         return [(raw[i * 64: (i + 1) * 64].split(b"\0")[0].decode(), float(us[i])) for i in range(n.value)]
+
+    def debug_graph_count(self):
+        """Captured graphs that the handle keeps."""
+        n = C.c_int32()
+        self._check(self.lib.ad_debug_graph_count(self.h, C.byref(n)), self.h)
+        return n.value
 
     def debug_stage_timeline(self):
         """Per-stage (inputs visible, signalled) global-timer stamps of the last persistent decoder pass, in ns."""

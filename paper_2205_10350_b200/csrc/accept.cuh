@@ -12,9 +12,8 @@ struct NextPass {
   int source;            // SRC_POLICY / SRC_OVERRIDE: plan the next verification block after the commit;
                          // SRC_SIZES: plan the drafter's pass after the commit (block sizes, then its tokens);
                          // SRC_KEEP (drafter's choices): plan the verification of the block just drafted
-  int k_cap;
   const int* override_stream;
-  int override_stride, override_len;
+  int override_stride;
   PassPlan draft;        // SRC_SIZES: plan of the drafter's pass
 };
 
@@ -90,9 +89,9 @@ __device__ __forceinline__ void scan_tiles(const float* __restrict__ val, const 
 // The decision for one row:
 //   c = first block position whose greedy choice differs from the draft (Section 3.1.1; definition of c in Section 3.2),
 //   n = c + 1 (the bifurcation token is kept), n = k when nothing differs, cut at the first accepted [EOS].
-// beta >= 1: relaxed verification of Section 3.2.3 -- a position keeps its drafted token when fewer than beta other tokens
+// relaxed_on: relaxed verification of Section 3.2.3 -- a position keeps its drafted token when fewer than beta other tokens
 //   score strictly higher (Eq. 8: the draft is within the top beta) and the best score exceeds the draft's by at most tau
-//   (Eq. 9; differences of log-likelihoods are differences of scores); otherwise the greedy choice.
+//   (Eq. 9; differences of log-likelihoods are differences of scores); otherwise the greedy choice.  beta and tau: st.words.
 // to_drafts: the choices are the row's drafts and nothing is compared.
 // auto_commit (decode loop): n is committed at once (Algorithm 1 lines 6-7); the last CTA to finish updates the loop
 //   counters and the all-finished word (done_ctr: rows done in the low half, active rows in the high half; left at zero) and,
@@ -106,8 +105,8 @@ __device__ __forceinline__ void scan_tiles(const float* __restrict__ val, const 
 // grid = B, block = 1024.
 __global__ void __launch_bounds__(ACC_THREADS)
 argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict__ part_val, const int* __restrict__ part_idx,
-                     int n_tiles, int to_drafts, int auto_commit, unsigned int* done_ctr, unsigned long long cond, int beta,
-                     float tau, const float* __restrict__ draft_val, const int* __restrict__ draft_id,
+                     int n_tiles, int to_drafts, int auto_commit, unsigned int* done_ctr, unsigned long long cond, int relaxed_on,
+                     const float* __restrict__ draft_val, const int* __restrict__ draft_id,
                      const int* __restrict__ part_cnt, NextPass next) {
   __shared__ int s_dr[256], s_pred[256], s_src[ACC_SRC];
   __shared__ int s_k[256], s_off[257], s_len[256];
@@ -120,6 +119,9 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
   const int k = plan_load(blk.seg_len + b), off = plan_load(blk.seg_off + b);
   const int len = plan_load(st.len + b), maxlen = plan_load(st.maxlen + b), old_last = plan_load(st.last + b);
   const int old_fin = plan_load(st.fin + b);
+  const int4 words = __ldcg(reinterpret_cast<const int4*>(st.words));
+  const int k_cap = words.x, override_len = words.y, beta = words.z;
+  const float tau = __int_as_float(words.w);
   int it_active = 0, it_all = 0, it_limit = 0, stat_acc = 0, stat_it = 0, stat_off = 0;
   if (tid == 0) { stat_acc = plan_load(st.stat_acc + b); stat_it = plan_load(st.stat_it + b); stat_off = plan_load(st.stat_off + b); }
   if (tid == ACC_THREADS - 1 && auto_commit) { it_active = plan_load(st.loop_it); it_all = plan_load(st.loop_it + 2); it_limit = plan_load(st.loop_it + 3); }
@@ -137,7 +139,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
   trace_mark(TR_ACCEPT, 1);
 
   // ---- arg-max over the tiles of every block position: a warp per position, the lowest id wins ties ----
-  const bool relaxed = beta >= 1 && !to_drafts;
+  const bool relaxed = relaxed_on && !to_drafts;
   int* pred = (to_drafts ? st.drafts : st.pred) + (size_t)b * dm.kmax;
   auto decide = [&](int i, float v, int idx, int higher) {      // lane 0 of the position's warp
     int choice = idx < dm.vocab ? idx : 0;                        // a position without any ordered score (NaN) still gets an id that exists
@@ -163,7 +165,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
     int dr = -1;
     if (tid < k) {
       dr = s_pred[tid];
-      if (next.override_stream) dr = len + tid < next.override_len ? next.override_stream[(size_t)b * next.override_stride + len + tid] : -1;
+      if (next.override_stream) dr = len + tid < override_len ? next.override_stream[(size_t)b * next.override_stride + len + tid] : -1;
       if (dr >= dm.vocab) { latch_error(st.status, AD_ERR_ARG); dr = -1; }
       s_dr[tid] = dr;
       st.drafts[(size_t)b * dm.kmax + tid] = dr;
@@ -230,13 +232,13 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
         auto o = [&](int t) { return t == 0 ? dm.bos : (t - 1 >= len ? s_pred[t - 1 - len] : __ldcg(old_out + t - 1)); };
         const int i = cta_suffix_match(o, len1, x, n_src, dm.bos, &s_where);
         // draft = x_{i+1..n} followed by the [PAD] slot that matches nothing; a plain step without a match
-        k1 = i >= 0 ? min(n_src - i + 1, min(next.k_cap, maxlen - len1)) : 1;
+        k1 = i >= 0 ? min(n_src - i + 1, min(k_cap, maxlen - len1)) : 1;
         if (tid < k1) s_dr[tid] = (i >= 0 && i + 1 + tid <= n_src) ? x[i + tid] : -1;
       }
     } else {
-      k1 = live ? min(next.k_cap, maxlen - len1) : 0;
+      k1 = live ? min(k_cap, maxlen - len1) : 0;
       if (next.source == SRC_OVERRIDE && tid < k1)
-        s_dr[tid] = len1 + tid < next.override_len ? next.override_stream[(size_t)b * next.override_stride + len1 + tid] : -1;
+        s_dr[tid] = len1 + tid < override_len ? next.override_stream[(size_t)b * next.override_stride + len1 + tid] : -1;
     }
     if (next.source != SRC_SIZES && tid < k1) {
       int dr = s_dr[tid];

@@ -144,6 +144,10 @@ struct ad_handle {
   int* dev_view(int* host) const { return host_flag_dev + (host - host_flag); }
   int* down = nullptr;       // result block of finalize_generate_kernel (host view) ...
   int* down_dev = nullptr;   // ... and its device view
+  // st.words as the calls enqueued so far leave them, and whether a caller has recorded calls into a graph of its own (whose replays
+  // set the words again at times that the handle does not see).
+  int4 words = {0, 0, 0, 0};
+  bool foreign_graphs = false;
   // Decode loop: the accept kernel of one pass plans the pass behind it; next_pass is what the accept kernel being enqueued
   // shall plan (source < 0: nothing).
   NextPass next_pass = no_next_pass();
@@ -362,7 +366,7 @@ size_t layout(ad_handle* h, void* base) {
   s.out_ids = ints((size_t)B * c.max_tgt);
   s.drafts = ints((size_t)B * c.kmax); s.pred = ints((size_t)B * c.kmax); s.n_acc = ints(B);
   s.stat_it = ints(B); s.stat_acc = ints(B); s.stat_off = ints(B);
-  s.loop_it = ints(4); s.status = ints(4); s.all_fin = ints(4);
+  s.loop_it = ints(4); s.status = ints(4); s.all_fin = ints(4); s.words = ints(4);
   s.sync_ctr = (unsigned int*)ints((size_t)mega::SYNC_COUNTERS * mega::SYNC_STRIDE);
   s.cross_base = ints(B);
   s.gidx = ints((size_t)B * c.kmax);
@@ -1163,8 +1167,8 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
   PassCfg& pc = h->pass[PK_VERIFY];
   GemmParams p = {};
   p.part_val = h->part_val; p.part_idx = h->part_idx;
-  const int beta = to_drafts ? 0 : h->beta;
-  if (beta >= 1) {   // relaxed verification: the drafts' own scores first, then the projection counts against them
+  const bool relaxed = !to_drafts && h->beta >= 1;
+  if (relaxed) {     // relaxed verification: the drafts' own scores first, then the projection counts against them
     const int d = h->cfg.d_model;
     note_launch(h, "draft_score");
     const dim3 sgrid((pc.M_cap + 7) / 8);
@@ -1176,25 +1180,25 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
   note_launch(h, "argmax_accept");
   AD_CUDA(h, launch_k(argmax_accept_kernel, dim3(h->dims.B), dim3(ACC_THREADS), 0, h->stream, h->st, pc.plan, h->dims, (const float*)h->part_val,
                       (const int*)h->part_idx, h->n_vtiles, to_drafts, auto_commit, (unsigned int*)(h->st.loop_it + 1),
-                      auto_commit ? h->cond_handle : 0ull, beta, h->tau, (const float*)h->draft_val, (const int*)h->draft_id,
+                      auto_commit ? h->cond_handle : 0ull, relaxed ? 1 : 0, (const float*)h->draft_val, (const int*)h->draft_id,
                       (const int*)h->part_cnt, h->next_pass));
   h->last_vocab_which = to_drafts ? 1 : 0;
   return AD_OK;
 }
 
 // user_drafts / user_k: where SRC_USER finds the caller's block (device, or mapped host memory); null: the workspace copies.
-int prepare_verify(ad_handle* h, int source, int k_cap, const int* ovr, int ovr_len, int* user_drafts = nullptr, int* user_k = nullptr) {
+int prepare_verify(ad_handle* h, int source, const int* ovr, int* user_drafts = nullptr, int* user_k = nullptr) {
   DevState st = h->st;
   if (user_drafts) { st.user_drafts = user_drafts; st.user_k = user_k; }
   note_launch(h, "prepare_verify");
-  AD_CUDA(h, launch_k(prepare_verify_kernel, dim3(1), dim3(256), 0, h->stream, st, h->pass[PK_VERIFY].plan, h->dims, source, k_cap, ovr,
-                                                 h->cfg.max_tgt, ovr_len));
+  AD_CUDA(h, launch_k(prepare_verify_kernel, dim3(1), dim3(256), 0, h->stream, st, h->pass[PK_VERIFY].plan, h->dims, source, ovr,
+                      h->cfg.max_tgt));
   return AD_OK;
 }
 
 // Draft substep: sizes and drafter plan ...
-int plan_draft(ad_handle* h, int k_cap) {
-  AD_TRY(prepare_verify(h, SRC_SIZES, k_cap, nullptr, 0));
+int plan_draft(ad_handle* h) {
+  AD_TRY(prepare_verify(h, SRC_SIZES, nullptr));
   note_launch(h, "plan_draft");
   AD_CUDA(h, launch_k(plan_draft_kernel, dim3(1), dim3(256), 0, h->stream, h->st, h->pass[PK_VERIFY].plan, h->pass[PK_DRAFT].plan, h->dims));
   return AD_OK;
@@ -1235,21 +1239,21 @@ bool loop_plans_ahead(const ad_handle* h) { return g_fuse_plan && !h->mega[PK_VE
 bool loop_drafts(const ad_gen_opts& o) { return o.mode == AD_MODE_GAD && o.run_drafter; }
 int block_source(const ad_gen_opts& o, const int* ovr) { return o.mode == AD_MODE_GAD || ovr ? SRC_OVERRIDE : SRC_POLICY; }
 
-NextPass next_pass(const ad_handle* h, int source, int k_cap, const int* ovr, int ovr_len) {
+NextPass next_pass(const ad_handle* h, int source, const int* ovr) {
   NextPass n = no_next_pass();
-  n.source = source; n.k_cap = k_cap; n.override_stream = ovr; n.override_stride = h->cfg.max_tgt; n.override_len = ovr_len;
+  n.source = source; n.override_stream = ovr; n.override_stride = h->cfg.max_tgt;
   n.draft = h->pass[PK_DRAFT].plan;
   return n;
 }
 
 // First pass of a loop that plans ahead: planned by kernels of their own.
-int plan_first_pass(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_len) {
-  if (loop_drafts(o)) return plan_draft(h, o.k);
-  return prepare_verify(h, block_source(o, ovr), o.k, ovr, ovr_len);
+int plan_first_pass(ad_handle* h, const ad_gen_opts& o, const int* ovr) {
+  if (loop_drafts(o)) return plan_draft(h);
+  return prepare_verify(h, block_source(o, ovr), ovr);
 }
 
 // One iteration of the decode loop: draft -> verify -> commit, all on the device.
-int loop_iteration(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_len) {
+int loop_iteration(ad_handle* h, const ad_gen_opts& o, const int* ovr) {
   struct Scope {               // whatever way this function is left
     ad_handle* h;
     ~Scope() {
@@ -1258,21 +1262,21 @@ int loop_iteration(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_l
   } scope{h};
   if (!loop_plans_ahead(h)) {
     if (loop_drafts(o)) {
-      AD_TRY(plan_draft(h, o.k));
+      AD_TRY(plan_draft(h));
       AD_TRY(draft_stage(h));
-      AD_TRY(prepare_verify(h, SRC_KEEP, o.k, ovr, ovr_len));
+      AD_TRY(prepare_verify(h, SRC_KEEP, ovr));
     } else {
-      AD_TRY(prepare_verify(h, block_source(o, ovr), o.k, ovr, ovr_len));
+      AD_TRY(prepare_verify(h, block_source(o, ovr), ovr));
     }
     return verify_stage(h, 1);   // accept and commit in one kernel
   }
   // this iteration's first pass has been planned already (plan_first_pass, or the previous iteration's accept kernel)
   if (loop_drafts(o)) {
-    h->next_pass = next_pass(h, SRC_KEEP, o.k, ovr, ovr_len);
+    h->next_pass = next_pass(h, SRC_KEEP, ovr);
     AD_TRY(draft_stage(h));
-    h->next_pass = next_pass(h, SRC_SIZES, o.k, nullptr, 0);
+    h->next_pass = next_pass(h, SRC_SIZES, nullptr);
   } else {
-    h->next_pass = next_pass(h, block_source(o, ovr), o.k, ovr, ovr_len);
+    h->next_pass = next_pass(h, block_source(o, ovr), ovr);
   }
   return verify_stage(h, 1);
 }
@@ -1289,13 +1293,32 @@ int read_status(ad_handle* h) {
   return wait_status(h, h->host_flag + 2);
 }
 
+// Whether the caller is recording the handle's stream.
+bool being_captured(const ad_handle* h) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (h->stream != nullptr) cudaStreamIsCapturing(h->stream, &cap);
+  return cap != cudaStreamCaptureStatusNone;
+}
+
+// Block-level calls: the words that kernels and captured graphs read, set in stream order (calls with device arrays do not wait for
+// one another) where they are not what the last call left.
+int set_words(ad_handle* h, int k_cap, int beta, float tau) {
+  int4 w = h->words;
+  w.x = k_cap; w.z = beta;
+  memcpy(&w.w, &tau, sizeof(tau));
+  if (being_captured(h)) h->foreign_graphs = true;
+  if (!h->foreign_graphs && !memcmp(&w, &h->words, sizeof(w))) return AD_OK;
+  note_launch(h, "set_words");
+  AD_CUDA(h, launch_k(set_words_kernel, dim3(1), dim3(1), 0, h->stream, h->st, w));
+  h->words = w;
+  return AD_OK;
+}
+
 // Runs `enqueue` (launches on the handle's stream whose arguments depend only on `key`) as a graph captured on first use;
 // directly where the stream cannot be captured or every launch is being timed.
 template <typename F>
 int run_captured(ad_handle* h, const char* key, F enqueue) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (h->stream != nullptr) cudaStreamIsCapturing(h->stream, &cap);
-  if (h->stream == nullptr || cap != cudaStreamCaptureStatusNone || !g_use_graph_encode || h->profiling) return enqueue();
+  if (h->stream == nullptr || being_captured(h) || !g_use_graph_encode || h->profiling) return enqueue();
   auto it = h->graphs.find(key);
   if (it == h->graphs.end()) {
     cudaGraph_t g = nullptr;
@@ -1489,9 +1512,9 @@ namespace {
 
 // What ad_encode and ad_generate import.  maxlen / ovr may be null; limit: iteration limit of the device-side loop (0: none).
 int import_inputs(ad_handle* h, const int32_t* src, int32_t src_stride, const int32_t* src_len, int32_t B, const int32_t* maxlen,
-                  const int32_t* ovr, int ovr_stride, int ovr_width, int limit, int on_host) {
+                  const int32_t* ovr, int ovr_stride, int ovr_width, int limit, int on_host, int4 words = {}) {
   const ad_model_cfg& c = h->cfg;
-  ImportParams p = {src, src_len, maxlen, ovr, src_stride, std::min(src_stride, c.max_src), ovr_stride, ovr_width, limit};
+  ImportParams p = {src, src_len, maxlen, ovr, src_stride, std::min(src_stride, c.max_src), ovr_stride, ovr_width, limit, words};
   if (on_host) {
     // host-resident inputs go through the handle's pinned staging area, which the device reads in place (every host-array
     // call ends synchronised, so the area is free again)
@@ -1506,6 +1529,7 @@ int import_inputs(ad_handle* h, const int32_t* src, int32_t src_stride, const in
   }
   note_launch(h, "import");
   AD_CUDA(h, launch_k(import_kernel, dim3(B), dim3(128), 0, h->stream, h->st, h->dims, p, h->in_max, h->ovr));
+  if (limit > 0) h->words = words;
   return AD_OK;
 }
 
@@ -1581,10 +1605,11 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
   if (on_host)
     for (int b = 0; b < B; ++b)
       if (k[b] < 0 || k[b] > c.kmax) return fail(h, AD_ERR_ARG, "k outside 0..kmax");
-  // Captured once per batch size and acceptance rule: with host arrays the whole call (the block is read from, and the result
+  // Captured once per batch size and kind of acceptance rule (its beta and tau are words): with host arrays the whole call (the block is read from, and the result
   // written to, mapped host memory), with device arrays everything but the copies from and to the caller's arrays.
-  char key[96];
-  snprintf(key, sizeof(key), "verify B%d h%d b%d t%a", B, on_host ? 1 : 0, h->beta, (double)h->tau);
+  char key[48];
+  snprintf(key, sizeof(key), "verify B%d h%d r%d", B, on_host ? 1 : 0, h->beta >= 1 ? 1 : 0);
+  AD_TRY(set_words(h, h->words.x, h->beta, h->tau));
   if (on_host) {
     memcpy(h->up_ids, drafts, sizeof(int) * (size_t)B * c.kmax);
     memcpy(h->up_n, k, sizeof(int) * B);
@@ -1593,8 +1618,8 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
     AD_CUDA(h, cudaMemcpyAsync(h->st.user_k, k, sizeof(int) * B, cudaMemcpyDeviceToDevice, h->stream));
   }
   AD_TRY(run_captured(h, key, [&]() -> int {
-    if (on_host) AD_TRY(prepare_verify(h, SRC_USER, c.kmax, nullptr, 0, h->dev_view(h->up_ids), h->dev_view(h->up_n)));
-    else AD_TRY(prepare_verify(h, SRC_USER, c.kmax, nullptr, 0));
+    if (on_host) AD_TRY(prepare_verify(h, SRC_USER, nullptr, h->dev_view(h->up_ids), h->dev_view(h->up_n)));
+    else AD_TRY(prepare_verify(h, SRC_USER, nullptr));
     AD_TRY(verify_stage(h, 0));
     if (on_host) {
       note_launch(h, "ad_verify_block");
@@ -1651,10 +1676,11 @@ extern "C" int ad_draft_block(ad_handle* h, int32_t k_cap, int32_t* drafts, int3
   const ad_model_cfg& c = h->cfg;
   if (k_cap < 1 || k_cap > c.kmax) return fail(h, AD_ERR_ARG, "k_cap outside 1..kmax");
   const int B = h->B;
-  char key[64];
-  snprintf(key, sizeof(key), "draft B%d h%d k%d", B, on_host ? 1 : 0, k_cap);
+  char key[48];
+  snprintf(key, sizeof(key), "draft B%d h%d", B, on_host ? 1 : 0);
+  AD_TRY(set_words(h, k_cap, h->beta, h->tau));
   AD_TRY(run_captured(h, key, [&]() -> int {
-    AD_TRY(plan_draft(h, k_cap));
+    AD_TRY(plan_draft(h));
     AD_TRY(draft_stage(h));
     if (on_host) {
       note_launch(h, "ad_draft_block");
@@ -1687,7 +1713,7 @@ extern "C" int ad_get_state(ad_handle* h, int32_t* len, int32_t* last_tok, int32
 namespace {
 
 // ad_generate's device work as one graph: encoder pass(es), plan of the first pass, loop (see ad_generate).
-bool build_whole_graph(ad_handle* h, const ad_gen_opts& o, const int* ovr, int ovr_len, bool capped, ad_handle::GraphEntry* out) {
+bool build_whole_graph(ad_handle* h, const ad_gen_opts& o, const int* ovr, bool capped, ad_handle::GraphEntry* out) {
   const int before = h->launches;
   cudaGraph_t g = nullptr, dummy = nullptr;
   cudaGraphConditionalHandle ch = 0;
@@ -1696,7 +1722,7 @@ bool build_whole_graph(ad_handle* h, const ad_gen_opts& o, const int* ovr, int o
   if (ok && cudaStreamBeginCaptureToGraph(h->stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
     ok = encode_stage(h, capped) == AD_OK;
     ok = ok && cudaEventRecordWithFlags(h->ev1, h->stream, cudaEventRecordExternal) == cudaSuccess;   // an event node: end of the encoders
-    if (ok && loop_plans_ahead(h)) ok = plan_first_pass(h, o, ovr, ovr_len) == AD_OK;
+    if (ok && loop_plans_ahead(h)) ok = plan_first_pass(h, o, ovr) == AD_OK;
     cudaStreamCaptureStatus status;
     const cudaGraphNode_t* deps = nullptr;
     size_t n = 0;
@@ -1717,7 +1743,7 @@ bool build_whole_graph(ad_handle* h, const ad_gen_opts& o, const int* ovr, int o
     ok = cudaGraphAddNode(&node, g, tail.data(), tail.size(), &np) == cudaSuccess;
     if (ok && cudaStreamBeginCaptureToGraph(h->stream, np.conditional.phGraph_out[0], nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
       h->cond_handle = (unsigned long long)ch;
-      ok = loop_iteration(h, o, ovr, ovr_len) == AD_OK;
+      ok = loop_iteration(h, o, ovr) == AD_OK;
       h->cond_handle = 0;
       ok = cudaStreamEndCapture(h->stream, &dummy) == cudaSuccess && ok;
     } else {
@@ -1765,23 +1791,25 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
   h->encoded = false;
   const int ovr_len = opts->draft_override ? std::min(opts->override_stride, c.max_tgt) : 0;   // valid leading entries of an override row
   const int* ovr = opts->draft_override ? h->ovr : nullptr;
-  // (the data-independent bound on the iteration count of the device-side loop travels with the inputs)
-  AD_TRY(import_inputs(h, src, src_stride, src_len, B, opts->max_len, opts->draft_override, opts->override_stride, ovr_len, max_iters + 1, on_host));
+  // (the data-independent bound on the iteration count of the device-side loop and the words travel with the inputs)
+  int4 words = {opts->k, ovr_len, h->beta, 0};
+  memcpy(&words.w, &h->tau, sizeof(h->tau));
+  AD_TRY(import_inputs(h, src, src_stride, src_len, B, opts->max_len, opts->draft_override, opts->override_stride, ovr_len, max_iters + 1, on_host,
+                       words));
   const bool capped = opts->max_len != nullptr;
 
   cudaGraphExec_t exec = nullptr;
   int per_iter_launches = 0;
   bool device_loop = false;
   if (opts->use_graph && h->stream != nullptr) {   // the legacy default stream cannot be captured
-    char key[160];
-    snprintf(key, sizeof(key), "B%d m%d k%d o%d v%d d%d c%d b%d t%a", B, opts->mode, opts->k, ovr ? 1 : 0, ovr_len, opts->run_drafter,
-             capped ? 1 : 0, h->beta, (double)h->tau);
+    char key[64];           // (block-size cap, override width, beta and tau are words)
+    snprintf(key, sizeof(key), "B%d m%d o%d d%d c%d r%d", B, opts->mode, ovr ? 1 : 0, opts->run_drafter ? 1 : 0, capped ? 1 : 0, h->beta >= 1 ? 1 : 0);
     auto it = h->graphs.find(key);
     if (it == h->graphs.end()) {
       ad_handle::GraphEntry entry = {};
       // First choice: the whole call as one graph -- encoder pass(es), plan of the first block, and a device-side `while` node
       // whose body is one iteration and whose condition the accept/commit kernel clears; no host round trip between them.
-      if (g_use_devloop && !build_whole_graph(h, *opts, ovr, ovr_len, capped, &entry)) {
+      if (g_use_devloop && !build_whole_graph(h, *opts, ovr, capped, &entry)) {
         entry = ad_handle::GraphEntry{};
         cudaGetLastError();   // clear; fall back to one replay per iteration
       }
@@ -1789,7 +1817,7 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
         const int before = h->launches;
         cudaGraph_t g = nullptr;
         AD_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-        const int rc = loop_iteration(h, *opts, ovr, ovr_len);
+        const int rc = loop_iteration(h, *opts, ovr);
         cudaError_t e = cudaStreamEndCapture(h->stream, &g);
         entry.launches = h->launches - before;
         h->launches = before;
@@ -1814,7 +1842,7 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
     snprintf(key, sizeof(key), "encode B%d c%d", B, capped ? 1 : 0);
     AD_TRY(run_captured(h, key, [&]() -> int { return encode_stage(h, capped); }));
     AD_CUDA(h, cudaEventRecord(h->ev1, h->stream));
-    if (loop_plans_ahead(h)) AD_TRY(plan_first_pass(h, *opts, ovr, ovr_len));
+    if (loop_plans_ahead(h)) AD_TRY(plan_first_pass(h, *opts, ovr));
   }
   h->encoded = true;
   h->last_vocab_which = -1;
@@ -1828,7 +1856,7 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
         AD_CUDA(h, cudaGraphLaunch(exec, h->stream));
         h->launches += per_iter_launches;
       } else {
-        AD_TRY(loop_iteration(h, *opts, ovr, ovr_len));
+        AD_TRY(loop_iteration(h, *opts, ovr));
       }
     }
     AD_CUDA(h, cudaMemcpyAsync(h->host_flag, h->st.all_fin, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
@@ -1936,6 +1964,13 @@ extern "C" int ad_debug_stage_timeline(ad_handle* h, uint64_t* stamps, int32_t c
   AD_CUDA(h, cudaStreamSynchronize(h->stream));
   AD_CUDA(h, cudaMemcpy(stamps, h->mega_timeline, sizeof(uint64_t) * 2 * (size_t)n, cudaMemcpyDeviceToHost));
   *n_stages = n;
+  return AD_OK;
+}
+
+extern "C" int ad_debug_graph_count(const ad_handle* h, int32_t* n) {
+  if (!h || !n) return AD_ERR_ARG;
+  *n = 0;
+  for (const auto& kv : h->graphs) *n += kv.second.exec != nullptr;
   return AD_OK;
 }
 

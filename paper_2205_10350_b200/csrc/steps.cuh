@@ -28,6 +28,8 @@ struct DevState {
   int* loop_it;    // [1] iterations with at least one active row
   int* status;     // [1] latched device error
   int* all_fin;    // [1] 1 when every row is finished
+  int* words;      // [4] what a call may change from one time to the next and a captured graph must not: block-size cap, valid entries of
+                   // an override row, beta and tau (float bits) of the relaxed verification
   int* cross_base; // [B] = b * max_src
   int* gidx;       // [B * kmax] drafter: packed token holding mask position i of row b
   int* enc_slot;   // [B * max_src] encoder: cross-K/V slot of packed source token m
@@ -88,17 +90,16 @@ __device__ int warp_suffix_match(const int* out, int j, const int* src, int n, i
 // ---------------------------------------------------------------------------------------------
 struct NextBlock {
   int source;                  // DraftSource
-  int k_cap;
   const int* override_stream;
-  int override_stride, override_len;
+  int override_stride;
 };
 
 __device__ __forceinline__ void plan_verify_block(const DevState& st, const PassPlan& plan, const Dims& dm, const NextBlock& nb,
                                                   int* s_k, int* s_off) {
   const int tid = threadIdx.x, nthreads = blockDim.x, warp = tid >> 5, lane = tid & 31, nwarps = nthreads >> 5;
-  const int B = dm.B, source = nb.source, k_cap = nb.k_cap;
+  const int B = dm.B, source = nb.source, k_cap = __ldcg(st.words), override_len = __ldcg(st.words + 1);
   const int* override_stream = nb.override_stream;
-  const int override_stride = nb.override_stride, override_len = nb.override_len;
+  const int override_stride = nb.override_stride;
 
   if (source == SRC_POLICY) {
     for (int b = warp; b < B; b += nwarps) {
@@ -178,16 +179,14 @@ __device__ __forceinline__ void plan_verify_block(const DevState& st, const Pass
 
 // grid = 1, block = 256.
 __global__ void __launch_bounds__(256)
-prepare_verify_kernel(DevState st, PassPlan plan, Dims dm, int source, int k_cap, const int* override_stream,
-                      int override_stride, int override_len) {
+prepare_verify_kernel(DevState st, PassPlan plan, Dims dm, int source, const int* override_stream, int override_stride) {
   trace_mark(TR_PREPARE, 0);
   pdl_wait();                  // (no pdl_launch: see plan data in ad_common.cuh)
   trace_mark(TR_PREPARE, 1);
   __shared__ int s_k[256];
   __shared__ int s_off[257];
   NextBlock nb;
-  nb.source = source; nb.k_cap = k_cap; nb.override_stream = override_stream;
-  nb.override_stride = override_stride; nb.override_len = override_len;
+  nb.source = source; nb.override_stream = override_stream; nb.override_stride = override_stride;
   plan_verify_block(st, plan, dm, nb, s_k, s_off);
   __threadfence();
 }
@@ -284,8 +283,8 @@ plan_encode_kernel(DevState st, PassPlan plan, Dims dm, const int* maxlen) {
   __threadfence();
 }
 
-// Inputs of a call into the workspace: sources, lengths, and for ad_generate per-row caps, the draft-override stream and the
-// iteration limit of the device-side loop.  The arrays are device memory or the handle's mapped pinned staging area, which is
+// Inputs of a call into the workspace: sources, lengths, and for ad_generate per-row caps, the draft-override stream, the
+// iteration limit of the device-side loop and the words (see DevState).  The arrays are device memory or the handle's mapped pinned staging area, which is
 // read in place: one launch instead of a copy per array.  Null pointers: that input is not part of the call.
 // grid = B, block = 128.
 struct ImportParams {
@@ -293,7 +292,8 @@ struct ImportParams {
   const int* src_len;
   const int* maxlen;
   const int* ovr;
-  int src_stride, src_width, ovr_stride, ovr_width, limit;
+  int src_stride, src_width, ovr_stride, ovr_width, limit;   // limit > 0: a call of ad_generate
+  int4 words;
 };
 __global__ void __launch_bounds__(128)
 import_kernel(DevState st, Dims dm, ImportParams p, int* maxlen_out, int* ovr_out) {
@@ -306,8 +306,18 @@ import_kernel(DevState st, Dims dm, ImportParams p, int* maxlen_out, int* ovr_ou
   if (tid == 0) {
     st.srclen[b] = p.src_len[b];
     if (p.maxlen) maxlen_out[b] = p.maxlen[b];
-    if (b == 0 && p.limit > 0) st.loop_it[3] = p.limit;
+    if (b == 0 && p.limit > 0) {
+      st.loop_it[3] = p.limit;
+      *reinterpret_cast<int4*>(st.words) = p.words;
+    }
   }
+}
+
+// The words alone, for the block-level calls.  One thread.
+__global__ void set_words_kernel(DevState st, int4 words) {
+  pdl_launch();
+  pdl_wait();
+  *reinterpret_cast<int4*>(st.words) = words;
 }
 
 // ---------------------------------------------------------------------------------------------
