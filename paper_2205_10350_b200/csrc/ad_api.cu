@@ -159,11 +159,13 @@ struct ad_handle {
   int last_vocab_which = -1;
   std::string err;
   struct GraphEntry {
-    cudaGraphExec_t exec;
+    cudaGraphExec_t exec;   // null: the form has been called once, directly
     int launches;        // kernels per replay (whole-call graph: per loop iteration)
     bool device_loop;    // whole-call graph ...
     int once;            // ... and its kernels outside the loop
+    long last_use;
   };
+  long graph_uses = 0;
   std::map<std::string, GraphEntry> graphs;
   std::map<std::tuple<int, int, int, int, int, int, int, int, int>, TcShape> tc_shapes;   // see cached_shape
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
@@ -1314,13 +1316,41 @@ int set_words(ad_handle* h, int k_cap, int beta, float tau) {
   return AD_OK;
 }
 
-// Runs `enqueue` (launches on the handle's stream whose arguments depend only on `key`) as a graph captured on first use;
-// directly where the stream cannot be captured or every launch is being timed.
+// The handle's entry for `key`, made if there is none.  Forms that a program can make by calling (batch sizes above all) must not
+// pile up: beyond four per row of capacity and a few, the one that has not been used for longest goes, once nothing of it runs.
+int graph_entry(ad_handle* h, const char* key, ad_handle::GraphEntry** out) {
+  auto it = h->graphs.find(key);
+  if (it == h->graphs.end()) {
+    while (h->graphs.size() >= (size_t)4 * h->cfg.max_batch + 16) {
+      auto oldest = std::min_element(h->graphs.begin(), h->graphs.end(), [](const auto& a, const auto& b) { return a.second.last_use < b.second.last_use; });
+      if (oldest->second.exec) {
+        AD_CUDA(h, cudaStreamSynchronize(h->stream));
+        cudaGraphExecDestroy(oldest->second.exec);
+      }
+      h->graphs.erase(oldest);
+    }
+    it = h->graphs.emplace(key, ad_handle::GraphEntry{}).first;
+  }
+  it->second.last_use = ++h->graph_uses;
+  *out = &it->second;
+  return AD_OK;
+}
+
+// Runs `enqueue` (launches on the handle's stream whose arguments depend only on `key`): the first call with this key directly, so that
+// a form that is called once does not pay for a capture, later ones as a graph captured by the second.  Directly as well where the
+// stream cannot be captured or every launch is being timed.
 template <typename F>
 int run_captured(ad_handle* h, const char* key, F enqueue) {
   if (h->stream == nullptr || being_captured(h) || !g_use_graph_encode || h->profiling) return enqueue();
-  auto it = h->graphs.find(key);
-  if (it == h->graphs.end()) {
+  ad_handle::GraphEntry* entry = nullptr;
+  AD_TRY(graph_entry(h, key, &entry));
+  if (!entry->exec) {
+    if (!entry->launches) {
+      const int before = h->launches;
+      AD_TRY(enqueue());
+      entry->launches = h->launches - before;
+      return AD_OK;
+    }
     cudaGraph_t g = nullptr;
     const int before = h->launches;
     AD_CUDA(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
@@ -1334,16 +1364,18 @@ int run_captured(ad_handle* h, const char* key, F enqueue) {
     const cudaError_t e2 = cudaGraphInstantiate(&exec, g, 0);
     cudaGraphDestroy(g);
     if (e2 != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e2));
-    it = h->graphs.emplace(key, ad_handle::GraphEntry{exec, n, false, 0}).first;
+    entry->exec = exec;
+    entry->launches = n;
   }
-  AD_CUDA(h, cudaGraphLaunch(it->second.exec, h->stream));
-  h->launches += it->second.launches;
+  AD_CUDA(h, cudaGraphLaunch(entry->exec, h->stream));
+  h->launches += entry->launches;
   return AD_OK;
 }
 
 
 void drop_graphs(ad_handle* h) {
-  for (auto& kv : h->graphs) cudaGraphExecDestroy(kv.second.exec);
+  for (auto& kv : h->graphs)
+    if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
   h->graphs.clear();
 }
 
@@ -1581,8 +1613,8 @@ extern "C" int ad_encode(ad_handle* h, const int32_t* src, int32_t src_stride, c
   h->dims.B = B;
   h->encoded = false;
   AD_TRY(import_inputs(h, src, src_stride, src_len, B, nullptr, nullptr, 0, 0, 0, on_host));
-  // The encoder pass reads its inputs from fixed workspace buffers, so on a capturable stream it is captured
-  // once per batch size and replayed (about fifty launches otherwise paid on the host for every sentence).
+  // The encoder pass reads its inputs from fixed workspace buffers, so on a capturable stream it is one graph
+  // per batch size (about fifty launches otherwise paid on the host for every sentence).
   char key[48];
   snprintf(key, sizeof(key), "encode B%d h%d", B, on_host ? 1 : 0);
   AD_TRY(run_captured(h, key, [&]() -> int {
@@ -1605,7 +1637,7 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
   if (on_host)
     for (int b = 0; b < B; ++b)
       if (k[b] < 0 || k[b] > c.kmax) return fail(h, AD_ERR_ARG, "k outside 0..kmax");
-  // Captured once per batch size and kind of acceptance rule (its beta and tau are words): with host arrays the whole call (the block is read from, and the result
+  // One graph per batch size and kind of acceptance rule (its beta and tau are words): with host arrays the whole call (the block is read from, and the result
   // written to, mapped host memory), with device arrays everything but the copies from and to the caller's arrays.
   char key[48];
   snprintf(key, sizeof(key), "verify B%d h%d r%d", B, on_host ? 1 : 0, h->beta >= 1 ? 1 : 0);
@@ -1804,8 +1836,9 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
   if (opts->use_graph && h->stream != nullptr) {   // the legacy default stream cannot be captured
     char key[64];           // (block-size cap, override width, beta and tau are words)
     snprintf(key, sizeof(key), "B%d m%d o%d d%d c%d r%d", B, opts->mode, ovr ? 1 : 0, opts->run_drafter ? 1 : 0, capped ? 1 : 0, h->beta >= 1 ? 1 : 0);
-    auto it = h->graphs.find(key);
-    if (it == h->graphs.end()) {
+    ad_handle::GraphEntry* kept = nullptr;
+    AD_TRY(graph_entry(h, key, &kept));
+    if (!kept->exec) {
       ad_handle::GraphEntry entry = {};
       // First choice: the whole call as one graph -- encoder pass(es), plan of the first block, and a device-side `while` node
       // whose body is one iteration and whose condition the accept/commit kernel clears; no host round trip between them.
@@ -1827,12 +1860,13 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
         cudaGraphDestroy(g);
         if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
       }
-      it = h->graphs.emplace(key, entry).first;
+      entry.last_use = kept->last_use;
+      *kept = entry;
     }
-    exec = it->second.exec;
-    per_iter_launches = it->second.launches;
-    device_loop = it->second.device_loop;
-    if (device_loop) h->launches += it->second.once;
+    exec = kept->exec;
+    per_iter_launches = kept->launches;
+    device_loop = kept->device_loop;
+    if (device_loop) h->launches += kept->once;
   }
 
   if (device_loop) {

@@ -87,6 +87,45 @@ def test_whole_calls_with_changing_settings():
     dec.close()
 
 
+def test_a_form_that_is_called_once_is_not_captured():
+    dec = make()
+    src, lens = sources(9)
+    r = np.random.default_rng(9)
+    drafts = r.integers(4, SHAPE.vocab, size=(B, K)).astype(np.int32)
+    results = []
+    for calls, graphs in ((1, 0), (2, 3), (3, 3)):       # encode, draft, verify
+        dec.encode(src, lens)
+        d, k = dec.draft_block(5)
+        ids, n = dec.verify_block(drafts, [K, 2, 4])
+        results.append((d[:, :5].tolist(), k.tolist(), [ids[b, :c].tolist() for b, c in enumerate((K, 2, 4))], n.tolist()))
+        assert dec.debug_graph_count() == graphs, calls
+    assert results[1] == results[0] and results[2] == results[0]
+    dec.close()
+
+
+def test_captured_graphs_are_bounded():
+    """More forms of whole calls than a handle of two rows keeps graphs for: the oldest go, and come back when they are called again."""
+    cap = 4 * 2 + 16
+    dec = make(max_batch=2)
+    src, lens = sources(10)
+    stream = np.random.default_rng(11).integers(4, SHAPE.vocab, size=(B, 9)).astype(np.int32)
+    first = {}
+    for rnd in range(2):
+        for rows in (1, 2):
+            for relaxed in (0, 2):
+                dec.set_acceptance(relaxed, 0.5 if relaxed else 0.0)
+                for mode, drafter, ovr in (("IAD", False, None), ("IAD", False, stream), ("GAD", True, None), ("GAD", True, stream), ("GAD", False, stream)):
+                    for caps in (None, [7, 9]):
+                        out, _ = dec.generate(src[:rows], lens[:rows], mode=mode, k=4, max_len=None if caps is None else caps[:rows],
+                                              draft_override=None if ovr is None else ovr[:rows], run_drafter=drafter)
+                        key = (rows, relaxed, mode, drafter, ovr is None, caps is None)
+                        res = [list(map(int, o)) for o in out]
+                        assert first.setdefault(key, res) == res, key
+                        assert dec.debug_graph_count() <= cap
+    assert len(first) == 40 and dec.debug_graph_count() == cap
+    dec.close()
+
+
 def test_settings_reach_calls_with_device_arrays_in_the_order_they_were_made():
     """Calls with device arrays do not wait: each sees the acceptance rule that was set when it was made."""
     dec, one = make(), make()
