@@ -98,11 +98,28 @@ NextPass no_next_pass() {
 
 thread_local std::string g_create_error;
 
+// Switches of a handle, read from the environment when it is created.
+struct Switches {
+  bool graph_calls = true;      // AD_NO_ENCODE_GRAPH=1: launch the kernels of the block-level calls and of the encoder directly
+  bool two_stream_encode = true;   // AD_NO_CONCURRENT_ENCODERS=1: the drafter's encoder after the verifier's, on one stream
+  bool devloop = true;          // AD_NO_DEVLOOP=1: one graph replay per iteration with host polling instead of a device-side loop
+  bool fuse_attn_proj = true;   // AD_NO_ATTN_PROJ=1: attention and its output projection always as separate kernels
+  bool fuse_plan = true;        // AD_NO_FUSED_PLAN=1: plan in kernels of their own in every iteration
+  // AD_MEGA=1: run eligible decoder passes (BF16, 64-wide heads, at most 64 packed tokens) as ONE persistent kernel
+  // instead of the kernel chain.  Off by default: measured on a B200 it is slower than the chain at every shape tried
+  // (base model: 342 / 360 / 424 / 462 us per verification step for blocks of 1 / 16 / 40 / 64 tokens against 214 / 223 /
+  // 247 / 258 us; big model, 25 tokens: 537 against 323 us), because a stage that hands its result to other SMs through
+  // L2 costs about 7 us there (operand staging 1.3-3 us, MMA hand-over 0.6, tensor-memory read-out 0.3, cluster hand-shake
+  // 0.8-1.2, reduction and epilogue 1-1.7, release 0.5, propagation 0.7) against about 3.7 us per kernel of the chain.
+  bool mega = false;
+};
+
 }  // namespace
 
 struct ad_handle {
   ad_model_cfg cfg;
   cudaStream_t stream = nullptr;
+  Switches sw;
   bool bf16 = false;
   size_t esz = 4;            // bytes per activation / weight element
   Model ar, nar;
@@ -436,18 +453,16 @@ int bind_model(ad_handle* h, Model& m, const ad_model_weights& w) {
 
 // ---- kernel launch helpers -----------------------------------------------------------------------
 
-bool g_use_pdl = true;       // AD_NO_PDL=1 in the environment turns programmatic dependent launch off
-bool g_use_graph_encode = true;   // AD_NO_ENCODE_GRAPH=1: launch the encoder kernels directly
-bool g_two_stream_encode = true;   // AD_NO_CONCURRENT_ENCODERS=1: the drafter's encoder after the verifier's, on one stream
-bool g_use_devloop = true;   // AD_NO_DEVLOOP=1: one graph replay per iteration with host polling instead of a device-side loop
-bool g_fuse_attn_proj = true;   // AD_NO_ATTN_PROJ=1: attention and its output projection always as separate kernels
-// AD_MEGA=1: run eligible decoder passes (BF16, 64-wide heads, at most 64 packed tokens) as ONE persistent kernel
-// instead of the kernel chain.  Off by default: measured on a B200 it is slower than the chain at every shape tried
-// (base model: 342 / 360 / 424 / 462 us per verification step for blocks of 1 / 16 / 40 / 64 tokens against 214 / 223 /
-// 247 / 258 us; big model, 25 tokens: 537 against 323 us), because a stage that hands its result to other SMs through
-// L2 costs about 7 us there (operand staging 1.3-3 us, MMA hand-over 0.6, tensor-memory read-out 0.3, cluster hand-shake
-// 0.8-1.2, reduction and epilogue 1-1.7, release 0.5, propagation 0.7) against about 3.7 us per kernel of the chain.
-bool g_use_mega = false;
+// AD_NO_PDL=1 in the environment turns programmatic dependent launch off; a thread that times every launch turns it off for itself.
+bool env_is_1(const char* name) {
+  const char* e = getenv(name);
+  return e && e[0] == '1';
+}
+thread_local bool t_serialise_launches = false;
+bool use_pdl() {
+  static const bool off = env_is_1("AD_NO_PDL");
+  return !off && !t_serialise_launches;
+}
 
 // Launches `kernel` so that it may begin while its predecessor in the stream still runs (the kernels
 // themselves wait with griddepcontrol.wait before touching anything a predecessor writes).
@@ -459,7 +474,7 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = g_use_pdl ? 1 : 0;
+  cfg.numAttrs = use_pdl() ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(std::forward<Args>(args))...);
 }
 
@@ -564,7 +579,7 @@ cudaError_t launch_vocab_pair(cudaStream_t st, const CUtensorMap& mw64, const CU
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = g_use_pdl ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = use_pdl() ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, tc::vocab_argmax_pair_kernel<STREAM>, mw64, mx128, p, stages);
 }
 cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw64, const CUtensorMap& mx128, const GemmParams& p, int M_cap) {
@@ -779,7 +794,7 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   cudaError_t e;
 #define AD_ATT(T, D, Q) launch_attention<T, D, Q>(grid, block, h->stream, p)
   // few queries, 64-wide heads: the output projection rides along (one partial sum per head for the LayerNorm kernel)
-  const bool fuse = g_fuse_attn_proj && wo && fused && h->pre2 && h->bf16 && dh == 64 && !many && c.n_heads <= pc.max_split &&
+  const bool fuse = h->sw.fuse_attn_proj && wo && fused && h->pre2 && h->bf16 && dh == 64 && !many && c.n_heads <= pc.max_split &&
                     c.n_heads <= 16 && c.d_model % 128 == 0;
   if (fused) *fused = fuse;
   note_launch(h, fuse ? "attention+out_proj" : "attention");
@@ -813,7 +828,7 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
 bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   const ad_model_cfg& c = h->cfg;
   const PassCfg& pc = h->pass[pk];
-  if (!g_fuse_attn_proj || !h->bf16 || !h->pre2 || c.d_model != c.n_heads * 64 || c.d_model % 128 || c.d_model > 128 * few::MAX_WARPS) return false;
+  if (!h->sw.fuse_attn_proj || !h->bf16 || !h->pre2 || c.d_model != c.n_heads * 64 || c.d_model % 128 || c.d_model > 128 * few::MAX_WARPS) return false;
   const int split = few::att_few_split(c.d_model);
   if (max_keys > few::MAX_ROUNDS * few::AK * few::att_few_warps(c.d_model)) return false;
   const int waves = pk == PK_ENCODE || (split > 1 && pc.seg_max < 8) ? 1 : pk == PK_DRAFT ? 4 : 3;
@@ -852,7 +867,7 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   cfg.dynamicSmemBytes = few::att_few_smem(warps, fp.rounds); cfg.stream = h->stream;
   cudaLaunchAttribute attr[2];
   int n_attr = 0;
-  if (g_use_pdl) {
+  if (use_pdl()) {
     attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
   }
@@ -972,7 +987,7 @@ int mega_cluster_size(const ad_model_cfg& c) {
 // pass kinds (or models, or devices) it does not apply to.  Runs once, from ad_create.
 int mega_setup(ad_handle* h) {
   const ad_model_cfg& c = h->cfg;
-  if (!g_use_mega || !h->bf16 || c.d_model / c.n_heads != 64 || c.d_model % 128 || c.d_ffn % 128) return AD_OK;
+  if (!h->sw.mega || !h->bf16 || c.d_model / c.n_heads != 64 || c.d_model % 128 || c.d_ffn % 128) return AD_OK;
   if (mega::ST_PER_LAYER * c.n_dec + 1 > mega::SYNC_COUNTERS) return AD_OK;
   const int cs = mega_cluster_size(c);
   if (!cs) return AD_OK;
@@ -1078,7 +1093,7 @@ int mega_launch(ad_handle* h, int pk) {
   attr[0].val.clusterDim.x = h->mega_cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = g_use_pdl ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = use_pdl() ? 2 : 1;
   note_launch(h, "persistent_decoder_pass");
   cudaError_t e = cudaLaunchKernelEx(&cfg, mega::decoder_pass_kernel, p);
   if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("persistent decoder pass launch: ") + cudaGetErrorString(e));
@@ -1236,8 +1251,7 @@ int commit_stage(ad_handle* h, const int* n_dev, int* status_out) {
 }
 
 // Whether the accept kernels of a decode loop plan the passes behind them (kernel-chain form of the passes only).
-bool g_fuse_plan = true;      // AD_NO_FUSED_PLAN=1: plan in kernels of their own in every iteration
-bool loop_plans_ahead(const ad_handle* h) { return g_fuse_plan && !h->mega[PK_VERIFY].on && !h->mega[PK_DRAFT].on; }
+bool loop_plans_ahead(const ad_handle* h) { return h->sw.fuse_plan && !h->mega[PK_VERIFY].on && !h->mega[PK_DRAFT].on; }
 bool loop_drafts(const ad_gen_opts& o) { return o.mode == AD_MODE_GAD && o.run_drafter; }
 int block_source(const ad_gen_opts& o, const int* ovr) { return o.mode == AD_MODE_GAD || ovr ? SRC_OVERRIDE : SRC_POLICY; }
 
@@ -1341,7 +1355,7 @@ int graph_entry(ad_handle* h, const char* key, ad_handle::GraphEntry** out) {
 // stream cannot be captured or every launch is being timed.
 template <typename F>
 int run_captured(ad_handle* h, const char* key, F enqueue) {
-  if (h->stream == nullptr || being_captured(h) || !g_use_graph_encode || h->profiling) return enqueue();
+  if (h->stream == nullptr || being_captured(h) || !h->sw.graph_calls || h->profiling) return enqueue();
   ad_handle::GraphEntry* entry = nullptr;
   AD_TRY(graph_entry(h, key, &entry));
   if (!entry->exec) {
@@ -1416,18 +1430,17 @@ extern "C" int ad_create(const ad_model_cfg* cfg, const ad_weights* w, void* wor
   int dev = 0, major = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess)
     return fail(nullptr, AD_ERR_CUDA, "no CUDA device");
-  { const char* e = getenv("AD_NO_PDL"); g_use_pdl = !(e && e[0] == '1'); }
-  { const char* e = getenv("AD_NO_DEVLOOP"); g_use_devloop = !(e && e[0] == '1'); }
-  { const char* e = getenv("AD_NO_ENCODE_GRAPH"); g_use_graph_encode = !(e && e[0] == '1'); }
-  { const char* e = getenv("AD_NO_CONCURRENT_ENCODERS"); g_two_stream_encode = !(e && e[0] == '1'); }
-  { const char* e = getenv("AD_NO_ATTN_PROJ"); g_fuse_attn_proj = !(e && e[0] == '1'); }
-  { const char* e = getenv("AD_MEGA"); g_use_mega = e && e[0] == '1'; }
-  { const char* e = getenv("AD_NO_FUSED_PLAN"); g_fuse_plan = !(e && e[0] == '1'); }
   if (major != 10) return fail(nullptr, AD_ERR_CUDA, "this library contains sm_100a code only; the current device is not compute capability 10.x");
 
   ad_handle* h = new ad_handle();
   h->cfg = *cfg;
   h->stream = static_cast<cudaStream_t>(stream);
+  h->sw.devloop = !env_is_1("AD_NO_DEVLOOP");
+  h->sw.graph_calls = !env_is_1("AD_NO_ENCODE_GRAPH");
+  h->sw.two_stream_encode = !env_is_1("AD_NO_CONCURRENT_ENCODERS");
+  h->sw.fuse_attn_proj = !env_is_1("AD_NO_ATTN_PROJ");
+  h->sw.fuse_plan = !env_is_1("AD_NO_FUSED_PLAN");
+  h->sw.mega = env_is_1("AD_MEGA");
   h->bf16 = cfg->dtype == AD_DTYPE_BF16;
   h->esz = h->bf16 ? 2 : 4;
   const size_t need = layout(h, workspace);
@@ -1455,7 +1468,7 @@ extern "C" int ad_create(const ad_model_cfg* cfg, const ad_weights* w, void* wor
     }
     if (!ok) return bail(AD_ERR_CUDA, "cuTensorMapEncodeTiled failed for an activation buffer");
   }
-  if (cfg->has_drafter && g_two_stream_encode) {
+  if (cfg->has_drafter && h->sw.two_stream_encode) {
     if (cudaStreamCreateWithFlags(&h->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess)
@@ -1842,7 +1855,7 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
       ad_handle::GraphEntry entry = {};
       // First choice: the whole call as one graph -- encoder pass(es), plan of the first block, and a device-side `while` node
       // whose body is one iteration and whose condition the accept/commit kernel clears; no host round trip between them.
-      if (g_use_devloop && !build_whole_graph(h, *opts, ovr, capped, &entry)) {
+      if (h->sw.devloop && !build_whole_graph(h, *opts, ovr, capped, &entry)) {
         entry = ad_handle::GraphEntry{};
         cudaGetLastError();   // clear; fall back to one replay per iteration
       }
@@ -1968,13 +1981,12 @@ extern "C" int ad_debug_profile_verify(ad_handle* h, const int32_t* drafts, cons
                                        int32_t capacity, int32_t* n_launches) {
   if (!h || !drafts || !k || !names || !us || !n_launches || capacity < 1) return AD_ERR_ARG;
   if (!h->encoded) return fail(h, AD_ERR_STATE, "ad_debug_profile_verify before ad_encode");
-  const bool pdl = g_use_pdl;
-  g_use_pdl = false;               // serialised launches: an event between two kernels then brackets exactly one of them
+  t_serialise_launches = true;     // serialised launches: an event between two kernels then brackets exactly one of them
   h->profiling = true;
   h->prof.clear();
   const int rc = ad_verify_block(h, drafts, k, nullptr, nullptr, 1);
   h->profiling = false;
-  g_use_pdl = pdl;
+  t_serialise_launches = false;
   cudaEvent_t last = nullptr;
   if (cudaEventCreate(&last) == cudaSuccess) { cudaEventRecord(last, h->stream); h->prof.emplace_back("end", last); }
   cudaStreamSynchronize(h->stream);

@@ -126,6 +126,23 @@ def test_captured_graphs_are_bounded():
     dec.close()
 
 
+def test_switches_belong_to_the_handle(monkeypatch):
+    """A handle made with other switches in the environment does not change what an older one does: one plans its passes in kernels
+    of their own, the other in its accept kernel."""
+    src, lens = sources(12)
+    runs = []
+    handles = []
+    for own_kernels in ("0", "1"):
+        monkeypatch.setenv("AD_NO_FUSED_PLAN", own_kernels)
+        handles.append(make())
+        runs.append([(st["kernel_launches"], st["iterations"], [list(map(int, o)) for o in out]) for out, st in
+                     [h.generate(src, lens, mode="IAD", k=6, max_len=[T, 8, 13], use_graph=False) for h in handles]])
+    assert runs[0][0] == runs[1][0]                       # the first handle, before and after the second was made
+    assert runs[1][0][1:] == runs[1][1][1:] and runs[1][0][0] < runs[1][1][0]
+    for h in handles:
+        h.close()
+
+
 def test_settings_reach_calls_with_device_arrays_in_the_order_they_were_made():
     """Calls with device arrays do not wait: each sees the acceptance rule that was set when it was made."""
     dec, one = make(), make()
