@@ -609,7 +609,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
       if (EPI == EPI_F32) {
         float* out = p.out_f32 + (size_t)kz * M * p.N;
         const int col = n0 + lane * 4;
-        const bool vec = (p.N & 3) == 0;
+        const bool vec = (p.N & 3) == 0 && (reinterpret_cast<uintptr_t>(p.out_f32) & 15) == 0;      // (a caller's y: any float address)
         for (int r = warp; r < ntok; r += THREADS / 32) {
           const float4 v = *reinterpret_cast<const float4*>(stage + r * LD + lane * 4);
           float* dst = out + (size_t)(tg + r) * p.N + col;

@@ -140,3 +140,22 @@ def test_operator_calls_that_read_what_the_call_before_them_wrote(dtype, M, K, N
         ref = binding.linear(x, W, ref[0].clone() if ref.dim() == 2 else ref)
         assert torch.equal(y, ref)
     assert int(st.item()) == 0
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("shift", [1, 2, 3])
+def test_linear_into_a_result_of_any_float_alignment(dtype, shift):
+    lib = binding.load()
+    dt, code = (torch.bfloat16, binding.AD_DTYPE_BF16) if dtype == "bf16" else (torch.float32, binding.AD_DTYPE_FP32)
+    M, K, N = 33, 128, 260
+    g = torch.Generator(DEV).manual_seed(shift)
+    x, W = torch.randn((M, K), generator=g, device=DEV).to(dt), torch.randn((N, K), generator=g, device=DEV).to(dt)
+    buf, bias = torch.full((M * N + 8,), 7.0, device=DEV), torch.randn(N + 4, generator=g, device=DEV)
+    y, b = buf[shift: shift + M * N], bias[shift: shift + N]
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    torch.cuda.synchronize()
+    stream = torch.cuda.current_stream().cuda_stream
+    assert lib.ad_linear(x.data_ptr(), W.data_ptr(), b.data_ptr(), code, M, K, N, y.data_ptr(), st.data_ptr(), stream) == binding.AD_OK
+    torch.cuda.synchronize()
+    assert torch.equal(y.view(M, N), binding.linear(x, W, b.clone()))
+    assert (buf[:shift] == 7.0).all() and (buf[shift + M * N:] == 7.0).all() and int(st.item()) == 0
