@@ -34,10 +34,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// First 1024-byte boundary of a dynamic shared-memory array (launched with 1024 bytes to spare).  Nothing else aligns the array: it
-// begins wherever the kernel's static variables end.
-__device__ __forceinline__ uint8_t* aligned_1024(uint8_t* p) { return p + ((0u - smem_u32(p)) & 1023u); }
-
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
 }
@@ -304,7 +300,7 @@ template <int EPI, int NCH>
 __global__ void __launch_bounds__(THREADS, 2)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ TileMaps maps_x, const GemmParams p,
                const int budget, const bf16* __restrict__ w_ptr, const bf16* x_ptr) {
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];     // (the few-token partial sums lie at its start and are read 16 bytes at a time)
   __shared__ __align__(8) uint64_t bar_full[MAX_STAGES];
   __shared__ __align__(8) uint64_t bar_empty[MAX_STAGES];
   __shared__ __align__(8) uint64_t bar_acc;
@@ -323,7 +319,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     const int id = blockIdx.y * gridDim.x + blockIdx.x;
     if (id < nbx * geo.ksplit)
       few::few_body<EPI == EPI_ARGMAX ? EPI_ACT : EPI, NCH == 0 ? 1 : NCH, false>(
-          w_ptr, x_ptr, p, few::EmbedParams{}, id % nbx, id / nbx, M, reinterpret_cast<float*>(aligned_1024(smem_raw)));
+          w_ptr, x_ptr, p, few::EmbedParams{}, id % nbx, id / nbx, M, reinterpret_cast<float*>(smem_raw));
     trace_mark(TR_GEMM + EPI, 2);
     return;
   }
@@ -349,7 +345,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   // column), so that the arg-max is a scan over a thread's own columns.  With the weights on the M side the exchange between
   // lanes takes 2.2 us of a CTA's 12 us at 90 tokens x 768.
   const bool token_major = EPI == EPI_ARGMAX && ntile == 128 && !p.bias;
-  const uint32_t smem_base = smem_u32(aligned_1024(smem_raw));        // swizzled tiles need 1024-byte alignment
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;   // swizzled tiles need 1024-byte alignment
   // MMA issuers.  Up to two warps issue side by side while the token tile is small: issuer j takes the K blocks j, j + n, ... of
   // this CTA and accumulates them in its own ntile-column region of tensor memory; the epilogue adds the regions up.  (631 x 4096
   // x 1024, 64-token tiles: one issuer 16.5 us, two 12.1, four 13.1.)
@@ -503,7 +499,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
     // The accumulator holds one output feature per TMEM lane and one token per column.  Warp w reads lanes
     // 32 (w % 4) .. +31; the two warps of a quadrant take alternate chunks of 16 columns.  The TMA ring is free
     // once the accumulator barrier has fired and serves as staging memory.
-    float* stage = reinterpret_cast<float*>(aligned_1024(smem_raw));
+    float* stage = reinterpret_cast<float*>(smem_raw + (smem_base - smem_u32(smem_raw)));
     constexpr int LD = 132;                                // rows stay 16-byte aligned
     const int ntok_all = min(ntile, M - t0);               // valid tokens of this tile (<= 0 only if M == 0)
     const uint32_t tlane = tmem_acc + (static_cast<uint32_t>(quad * 32) << 16);

@@ -128,7 +128,7 @@ template <bool STREAM>
 __global__ void __launch_bounds__(P_THREADS, 1)
 vocab_argmax_pair_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_x, const GemmParams p,
                          const int stages) {
-  extern __shared__ uint8_t smem_raw[];
+  extern __shared__ __align__(16) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t bar_full[P_MAX_STAGES];      // first CTA's: both CTAs' rows of a stage have landed
   __shared__ __align__(8) uint64_t bar_empty[P_MAX_STAGES];     // both: the stage has been consumed
   __shared__ __align__(8) uint64_t a_full[P_MAX_KB];            // first CTA's: both CTAs' tokens of a K block have landed
