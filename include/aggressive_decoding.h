@@ -53,7 +53,8 @@ enum { AD_MODE_IAD = 0, AD_MODE_GAD = 1 };
 
 /* Plain-old-data description of one model family and of the capacities of a handle. */
 typedef struct ad_model_cfg {
-  int32_t d_model, n_heads, d_ffn, vocab, n_enc, n_dec;
+  int32_t d_model, n_heads, d_ffn, vocab, n_enc, n_dec;   /* heads 32 or 64 wide, d_model <= 1024; FP32: d_ffn % 4 == 0;
+                          BF16: d_model % 128 == 0, d_ffn % 64 == 0 */
   int32_t dtype;       /* AD_DTYPE_FP32: FP32 weights, FFMA arithmetic.  AD_DTYPE_BF16: BF16 weights and GEMM
                           operands on the tensor cores, FP32 accumulation, residual stream, LayerNorm, softmax */
   int32_t max_batch;   /* B capacity */
@@ -77,7 +78,7 @@ typedef struct ad_model_cfg {
  *       per encoder layer: bqkv [3d], bo [d], ln1 gain [d], ln1 bias [d], b1 [F], b2 [d], ln2 gain, ln2 bias
  *       per decoder layer: self bqkv [3d], self bo [d], ln1 gain, ln1 bias, cross bq [d], cross bkv [2d],
  *                          cross bo [d], ln2 gain, ln2 bias, b1 [F], b2 [d], ln3 gain, ln3 bias
- * `matrices` must be 256-byte aligned.  ad_weight_counts() gives the two element counts.
+ * `matrices` must be 256-byte aligned, `vectors` 16-byte aligned.  ad_weight_counts() gives the two element counts.
  */
 typedef struct ad_model_weights {
   const void* matrices;

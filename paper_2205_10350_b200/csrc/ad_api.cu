@@ -404,6 +404,8 @@ int check_cfg(const ad_model_cfg* c, std::string* why) {
   if (c->d_ffn <= 0 || c->vocab <= 4 || c->n_enc < 1 || c->n_dec < 1) return bad("bad model sizes");
   if (c->dtype != AD_DTYPE_FP32 && c->dtype != AD_DTYPE_BF16) return bad("dtype must be AD_DTYPE_FP32 or AD_DTYPE_BF16");
   if (c->dtype == AD_DTYPE_BF16 && (c->d_model % 128 || c->d_ffn % 64)) return bad("BF16 needs d_model to be a multiple of 128 and d_ffn a multiple of 64");
+  // (biases and gains are read 16 bytes at a time, and the vectors behind a b1 begin where it ends)
+  if (c->dtype == AD_DTYPE_FP32 && c->d_ffn % 4) return bad("FP32 needs d_ffn to be a multiple of 4");
   if (c->max_batch < 1 || c->max_batch > 256) return bad("max_batch must be 1..256");
   if (c->max_src < 1 || c->max_tgt < 1) return bad("max_src and max_tgt must be positive");
   if (c->kmax < 1 || c->kmax > 256 || c->kmax > c->max_tgt) return bad("kmax must be 1..min(256, max_tgt)");
@@ -423,6 +425,7 @@ int bind_model(ad_handle* h, Model& m, const ad_model_weights& w) {
   const ad_model_cfg& c = h->cfg;
   const int d = c.d_model, F = c.d_ffn;
   if (!w.matrices || !w.vectors) return fail(h, AD_ERR_ARG, "weight pointers are null");
+  if (reinterpret_cast<uintptr_t>(w.vectors) % 16) return fail(h, AD_ERR_ARG, "weight vectors must be 16-byte aligned");
   if (reinterpret_cast<uintptr_t>(w.matrices) % 256) return fail(h, AD_ERR_ARG, "weight matrices must be 256-byte aligned");
   const char* mp = static_cast<const char*>(w.matrices);
   const float* vp = w.vectors;

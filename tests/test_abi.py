@@ -67,6 +67,10 @@ def test_workspace_query_and_config_checks(lib):
     bad = _cfg(synth.BASE)
     bad.n_heads = 7
     assert lib.ad_query_workspace(C.byref(bad), C.byref(n)) == binding.AD_ERR_ARG
+    for d_ffn, rc in ((510, binding.AD_ERR_ARG), (508, binding.AD_OK)):      # vectors are read 16 bytes at a time
+        odd = _cfg(synth.TINY)
+        odd.d_ffn = d_ffn
+        assert lib.ad_query_workspace(C.byref(odd), C.byref(n)) == rc
     bad = _cfg(synth.BASE)
     bad.eos = 40000
     assert lib.ad_query_workspace(C.byref(bad), C.byref(n)) == binding.AD_ERR_ARG

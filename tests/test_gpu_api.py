@@ -272,3 +272,23 @@ def test_per_kernel_profile_of_a_block_changes_nothing(setup):
     assert len(prof) >= 10 and all(us > 0 for _, us in prof)
     assert names[0] == "prepare_verify" and "embed" in names and any(x.startswith("gemm_") for x in names)
     assert names[-1] in ("argmax_accept", "ad_verify_block")
+
+
+def test_weight_vectors_that_are_not_aligned_are_refused():
+    import ctypes as C
+    import torch
+    shape = synth.ModelShape("edge", 64, 2, 128, 50, 1, 1, "fp32")
+    m, v = binding.pack_weights(shape, synth.make_weights(shape, 0, std=0.1))
+    lib = binding.load()
+    cfg = binding.ModelCfg(shape.d_model, shape.n_heads, shape.d_ffn, shape.vocab, 1, 1, binding.AD_DTYPE_FP32, 1, 10, 12, 6, 0, 1, 2, 3, 1e-5, 0)
+    nbytes = C.c_size_t()
+    assert lib.ad_query_workspace(C.byref(cfg), C.byref(nbytes)) == binding.AD_OK
+    mt, vt = torch.tensor(m, device="cuda:0"), torch.zeros(v.size + 4, device="cuda:0")
+    ws = torch.empty(nbytes.value + 1024, dtype=torch.uint8, device="cuda:0")
+    base = (ws.data_ptr() + 1023) // 1024 * 1024
+    for shift, rc in ((4, binding.AD_ERR_ARG), (8, binding.AD_ERR_ARG), (16, binding.AD_OK)):
+        w, h = binding.Weights(), C.c_void_p()
+        w.ar = binding.ModelWeights(mt.data_ptr(), vt.data_ptr() + shift)
+        assert lib.ad_create(C.byref(cfg), C.byref(w), C.c_void_p(base), nbytes.value, None, C.byref(h)) == rc
+        if rc == binding.AD_OK:
+            lib.ad_destroy(h)
