@@ -19,6 +19,11 @@ pytestmark = pytest.mark.gpu
     (512, 512, 1, 33, 20, 129),      # self-attention keys in a second round
     (768, 1536, 3, 9, 30, 24),       # three K chunks, a pair of CTAs with six warps each
     (1024, 1024, 2, 33, 17, 40),     # four K chunks, a pair of CTAs with eight warps each
+    (768, 768, 1, 64, 110, 128),     # a pair of CTAs: source keys, then self-attention keys beyond one round of six warps
+    (1024, 512, 1, 64, 140, 150),    # the same with eight warps
+    (384, 768, 2, 17, 100, 24),      # six warps in one CTA, source keys in a second round
+    (640, 640, 1, 20, 90, 24),       # a pair of CTAs with five warps each, source keys in a second round
+    (896, 896, 2, 9, 20, 24),        # a pair of CTAs with seven warps each
 ])
 def test_few_token_passes_follow_the_checker(d, ffn, batch, k, src, tgt):
     from paper_2205_10350_b200 import binding

@@ -152,8 +152,7 @@ def test_setter_rejects_bad_values():
     dec.close()
 
 
-def _base_ragged_rows(ks, lens, check_rows, min_clear):
-    shape = synth.BASE
+def _base_ragged_rows(ks, lens, check_rows, min_clear, shape=synth.BASE):
     B = len(ks)
     dec, om = make(shape, 16, 16, 12, batch=B)
     r = np.random.default_rng(23)
@@ -207,3 +206,10 @@ def test_bf16_base_twelve_rows_two_token_tiles():
     vocabulary rows scoring above each draft; rows 0, 7 and 11 (the last one lies in the second, ragged 128-token tile)
     are followed by the checker."""
     _base_ragged_rows([12] * 12, [16, 11, 9, 16, 13, 16, 12, 10, 16, 15, 14, 16], {0, 7, 11}, 8)
+
+
+def test_bf16_twelve_rows_of_a_model_wider_than_512():
+    """The same 144 tokens on a 768-wide model: the token tile of the paired projection kernel travels through the ring with the
+    vocabulary's rows there, and its read-out counts as well."""
+    shape = synth.ModelShape("wide_relaxed", 768, 12, 768, 19073, 1, 1, "bf16")
+    _base_ragged_rows([12] * 12, [16, 11, 9, 16, 13, 16, 12, 10, 16, 15, 14, 16], {0, 7, 11}, 8, shape)
