@@ -807,7 +807,7 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
     e = (long)grid.x * grid.y > num_sms() ? launch_attention<bf16, 64, 1, true, 2>(grid, block, h->stream, p)
                                            : launch_attention<bf16, 64, 1, true, 1>(grid, block, h->stream, p);
   } else if (h->bf16) {
-    if (dh == 64) e = many ? AD_ATT(bf16, 64, 8) : AD_ATT(bf16, 64, 1);
+    if (dh == 64) e = AD_ATT(bf16, 64, 1);         // (many queries: the MMA kernels above)
     else e = many ? AD_ATT(bf16, 32, 8) : AD_ATT(bf16, 32, 1);
   } else {
     if (dh == 64) e = many ? AD_ATT(float, 64, 8) : AD_ATT(float, 64, 1);

@@ -51,18 +51,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Non-blocking probe of a barrier phase: returns at once with 1 if the phase has completed, else 0.
-__device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok;
-}
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -172,8 +160,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// 16 columns of each of `n` (1, 2 or 4) accumulator regions `stride` columns apart, added up in region order.  All loads are
-// in flight before the one wait: a tensor-memory round trip per region would be paid one after the other.
+// 16 columns of one or two (n) accumulator regions `stride` columns apart, added up.  Both loads are in flight before the one
+// wait: a tensor-memory round trip per region would be paid one after the other.
 __device__ __forceinline__ void tmem_issue16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -188,13 +176,9 @@ __device__ __forceinline__ void tmem_landed16(uint32_t (&r)[16]) {
                     "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]));
 }
 __device__ __forceinline__ void tmem_sum16(uint32_t taddr, int n, uint32_t stride, float (&acc)[16]) {
-  uint32_t r[4][16];
+  uint32_t r[2][16];
   tmem_issue16(taddr, r[0]);
   if (n > 1) tmem_issue16(taddr + stride, r[1]);
-  if (n > 2) {
-    tmem_issue16(taddr + 2 * stride, r[2]);
-    tmem_issue16(taddr + 3 * stride, r[3]);
-  }
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
   tmem_landed16(r[0]);
 #pragma unroll
@@ -203,12 +187,6 @@ __device__ __forceinline__ void tmem_sum16(uint32_t taddr, int n, uint32_t strid
     tmem_landed16(r[1]);
 #pragma unroll
     for (int i = 0; i < 16; ++i) acc[i] += __uint_as_float(r[1][i]);
-  }
-  if (n > 2) {
-    tmem_landed16(r[2]);
-    tmem_landed16(r[3]);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] = (acc[i] + __uint_as_float(r[2][i])) + __uint_as_float(r[3][i]);
   }
 }
 
@@ -220,15 +198,6 @@ __device__ __forceinline__ unsigned int float_key(float v) {
 __device__ __forceinline__ float key_float(unsigned int k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
-// Largest value over the warp and the lowest lane holding it: one redux and one ballot.
-__device__ __forceinline__ void warp_argmax_lane(float v, float& best, int& lane_of_best) {
-  const unsigned int k = float_key(v);
-  const unsigned int m = __reduce_max_sync(0xffffffffu, k);
-  const unsigned int bal = __ballot_sync(0xffffffffu, k == m);
-  best = key_float(m);
-  lane_of_best = __ffs(bal) - 1;
-}
-
 // Arg-max over the 32 lanes for 16 values per lane at once.  v[j] is this lane's candidate for item j; on
 // return lanes 2 j and 2 j + 1 hold, for item j, the largest candidate and the lowest lane that offered it.  Each
 // halving step sends one half of the items a lane still holds to its partner and keeps the other half, so that every
@@ -352,12 +321,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_constant_
   // An issuer waits for ring phase r of a stage only after phase r - 1 has completed (a parity wait two phases ahead
   // would alias): with more than one ring round this holds when the ring depth is a multiple of the issuer count, since
   // the K block that used the stage one round earlier was then this issuer's own.
-  int n_issuers = 1;
-  {
-    const int cap = ntile <= 128 ? 2 : 1;
-    for (int cand = 2; cand > 1; cand >>= 1)
-      if (cand <= cap && cand <= num_kb && (num_kb <= stages || stages % cand == 0)) { n_issuers = cand; break; }
-  }
+  const int n_issuers = ntile <= 128 && num_kb >= 2 && (num_kb <= stages || stages % 2 == 0) ? 2 : 1;
   uint32_t tmem_cols = 32;
   while (tmem_cols < (uint32_t)(ntile * n_issuers)) tmem_cols <<= 1;
 
