@@ -80,8 +80,8 @@ def reduce_max_sum(dist, dev, seconds_or_ms, count):
 # DRAM counters of one verification step (dram__bytes_read.sum + dram__bytes_write.sum summed over the step's
 # kernels, ncu, caches flushed before every kernel) with the digest of the kernel sources they were taken on:
 # the figures are reported only while the sources still have that digest.
-NCU_COUNTERS = dict(sources_sha256="748bbf674820a70485669346e6d0b8a7256ee158b313d80ee57d22edeb6d6edc",
-                    step_block40_bytes=102923008, projection_bytes=32858368,
+NCU_COUNTERS = dict(sources_sha256="534c420cabbaffb58020b7fb7dee77e70582493b10b549025962107d408701a6",
+                    step_block40_bytes=92233472, projection_bytes=32864768,
                     summary="profiles/verify_step_base_b1_k40_dram_traffic.txt")
 
 
@@ -288,7 +288,7 @@ def kernel_table(dec, shape, drafts, k, pk):
 
 
 def fixed_step(binding, shape, w, pk, B, k, prefix, S, reps=30, flush=None):
-    """Verification steps of one fixed shape (direct launches, verify + discard so that every repetition sees the same
+    """Verification steps of one fixed shape (a graph per block, verify + discard so that every repetition sees the same
     prefix).  Returns (microseconds L2-warm, microseconds with L2 flushed before every step or None)."""
     import torch
     dec = binding.AggressiveDecoder(shape, w, max_batch=B, max_src=S, max_tgt=max(prefix + k, 8), kmax=k)
@@ -548,7 +548,7 @@ def bench_extras(args, binding, dec, w, dev, pk, flush, t_src, t_len, t_max, t_o
                                        traffic_note="dram__bytes_read.sum + dram__bytes_write.sum of one launch (" +
                                        NCU_COUNTERS["summary"] + "); null once a kernel source has changed since the capture")
 
-    # fixed-shape verification steps, weight-streaming regime (direct launches): L2-warm and L2-flushed
+    # fixed-shape verification steps, weight-streaming regime (a graph per block): L2-warm and L2-flushed
     pts = []
     for (k, prefix) in ((16, 16), (64, 0), (1, 20)):
         warm, cold = fixed_step(binding, shape, w, pk, 1, k, prefix, 32, reps=30, flush=flush)
@@ -556,7 +556,7 @@ def bench_extras(args, binding, dec, w, dev, pk, flush, t_src, t_len, t_max, t_o
         pts.append(dict(shape=f"base, batch 1, block {k} on a {prefix}-token prefix, source 32", algorithmic_bytes=bts,
                         us_l2_warm=warm, us_l2_flushed=cold, hbm_floor_us=bts / (pk["hbm_gbs"] * 1e9) * 1e6,
                         frac_l2_warm=bts / (warm * 1e-6) / 1e9 / pk["hbm_gbs"], frac_l2_flushed=bts / (cold * 1e-6) / 1e9 / pk["hbm_gbs"]))
-    extras["step_points"] = dict(note="direct launches (no graph), verify + discard; flushed = 256 MB write before every step", points=pts)
+    extras["step_points"] = dict(note="one graph per block, verify + discard; flushed = 256 MB write before every step", points=pts)
 
     # the library's own greedy decoding (block size 1) of the same sentences
     def step_greedy():
@@ -584,7 +584,7 @@ def bench_extras(args, binding, dec, w, dev, pk, flush, t_src, t_len, t_max, t_o
                                    tensor_floor_us=flops32 / (pk["bf16_tflops"] * 1e12) * 1e6,
                                    frac_of_floor=flops32 / (pk["bf16_tflops"] * 1e12) * 1e6 / us32,
                                    frac_of_sustained=flops32 / (pk["bf16_tflops_sustained"] * 1e12) * 1e6 / us32,
-                                   note="batch 32, block 64, empty prefix, source 64; direct launches, weights L2-warm")
+                                   note="batch 32, block 64, empty prefix, source 64; one graph per block, weights L2-warm")
     # the one kernel of that step with tensor-core-sized work, timed alone: projection + arg-max partials over 2048 tokens
     x32 = torch.randn((M32, d), device=dev).bfloat16()
     nb32 = lib.ad_vocab_argmax_scratch_bytes(V, M32)

@@ -55,12 +55,14 @@ enum Epi : int {
 // runs at the geometry of the tokens it has, not at that of its capacity.
 //
 // Token tile: up to 64 tokens one tile; beyond that the kernels are latency-bound and smaller tiles win -- more CTAs, a
-// shorter epilogue each -- until the grids outgrow the SMs.  Measured per step (base model):
-//   100 / 120 / 128 tokens: 64-token tiles 277 / 289 / 293 us against 305 / 316 / 321 us with one 128-token tile;
-//   200 / 240 tokens: 32-token tiles 331 / 305 us, 64: 344 / 311, 128: 364 / 336, 16: 372;
-//   320 / 400 / 512 tokens: 64-token tiles 366 / 357 / 389 us against 415 / 410 / 458 (128) and 383 / 380 / 410 (32);
-//   800 / 1024 tokens: 64-token tiles 455 / 468 us against 477 / 486 (128);  2048 tokens: 128-token tiles 543 us, 64: 571;
-//   256-token tiles once they alone give two CTAs per SM.
+// shorter epilogue each -- until the grids outgrow the SMs.  Measured per verification step, builds that differ in the tile alone
+// (512 wide: base model, capacity 256 for the first line, 2048 for the others; 1024 wide: big model, capacity 1024):
+//   512 wide, 200 / 240 tokens: 32-token tiles 212 / 224 us, 64: 220 / 226, 128: 238 / 248, 16: 224 / 232;
+//   320 / 512 / 800 / 1024 tokens: 64-token tiles 293 / 309 / 344 / 363 us, 128: 340 / 351 / 379 / 388, 32: 334 / 362 / 435 / 455;
+//   2048 tokens: 128-token tiles 490 us, 64: 519, 256: 586 (256 is taken once it alone gives two CTAs per SM);
+//   1024 wide, 100 / 128 tokens: 64-token tiles 345 / 359 us, 128: 385 / 400, 32: 390 / 396.
+// The line at 1024 is the narrow models': 1024 wide, 128-token tiles already win there (648 us, 64: 717), and 64 at 200 (386, 32: 404).
+// Up to 128 tokens most projections take the few-token kernels and the rule is only asked for what those do not cover.
 // A projection whose feature tiles alone outnumber the SMs (the vocabulary) fills them with one token tile, and every further one
 // reads its weights again: one 128-token tile up to 128 tokens (90 tokens x 50265 x 768: 19.5 us with two of 64), then tiles of 128
 // (400 x 768 x 50265: 56 us, 76 with 64-token tiles), of 256 beyond 1536 tokens, where L2 traffic bounds it (2048: 114 against 119 us).

@@ -9,14 +9,15 @@
 // A pair of CTAs (a cluster on two neighbouring SMs) works on 256 tokens x 256 vocabulary rows at a time: each CTA holds its 128
 // tokens (128 x K BF16, resident in shared memory as long as the token tile stays) and loads HALF of the vocabulary
 // rows; the paired MMA reads both halves from both shared memories, so a K block brings 16 KB into each SM instead of the 32 KB that
-// one CTA per token tile needs.  2048 tokens x 32000 x 512, back to back: one CTA per token tile 61 us, pairs 64.5 us while the
-// MMAs were issued from a branch on the lane number, 49.5 us (1354 TFLOP/s) issued from a converged warp; 600 tokens 25.5 -> 23.6 us.
+// one CTA per token tile needs.  2048 tokens x 32000 x 512, call behind call: one CTA per token tile 61 us, pairs 64.5 us while the
+// MMAs were issued from a branch on the lane number, 49.7 us (1350 TFLOP/s) issued from a converged warp; 600 tokens 25.5 -> 23.7 us.
+// A single call between two events takes 57.8 us (1161 TFLOP/s), 600 tokens 31.
 // What bounds it now: 0.4 us per K block against 0.27 us of MMA time, plus 6 us to fill, read the last step out and tear down.
 //
 // K > 512 (STREAM): the token tile no longer fits beside a ring, so its K blocks travel through the ring with the vocabulary's, 32 KB
-// a stage.  One CTA per 128 x 128 tile, as these widths ran before, is bound by the tiles' way through L2 (11.7 TB/s): 2048 tokens x
-// 32000 x 1024 137 -> 82 us (1637 TFLOP/s), 600 x 768 x 50265 68 -> 44 us, 200 x 768 x 50265 29 -> 22 us.  Up to 512 the resident form stays 2 to 4 % ahead
-// (2048 tokens 55 against 57 us).
+// a stage.  One CTA per 128 x 128 tile, as these widths ran before, is bound by the tiles' way through L2 (11.7 TB/s).  One call between two
+// events: 2048 tokens x 32000 x 1024 137 -> 90 us (1488 TFLOP/s), 600 x 768 x 50265 65 -> 47 us, 200 x 768 x 50265 31 -> 25 us; call behind
+// call 129 -> 91, 59 -> 42 and 25 -> 19 us.  Up to 512 the resident form stays 2 to 4 % ahead.
 //
 // The range of (token tile, 128-row vocabulary tile) units is dealt to the pairs in contiguous pieces, the vocabulary tile
 // running fastest; a pair takes two units a step, one where its piece or the vocabulary ends (the MMA is then 128 columns wide

@@ -12,6 +12,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import os
 import statistics
 
 import numpy as np
@@ -37,6 +38,18 @@ def _events(stream, fn, reps, flush=None):
             evs.append((a, b))
     stream.synchronize()
     return [a.elapsed_time(b) * 1e3 for a, b in evs[3:]]
+
+
+def _back_to_back(stream, fn, reps):
+    """Device time of fn per call in microseconds, calls queued behind one another (each may begin under the one in front of it)."""
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    with torch.cuda.stream(stream):
+        a.record(stream)
+        for _ in range(reps):
+            fn()
+        b.record(stream)
+    stream.synchronize()
+    return a.elapsed_time(b) * 1e3 / reps
 
 
 def main():
@@ -104,8 +117,9 @@ def main():
         torch.cuda.synchronize()
         ts = _events(stream, fn, args.reps, flush)
         bytes_ = N * K * 2 + M * K * 2
-        out.update(M=M, K=K, N=N, us_mean=statistics.mean(ts), us_min=min(ts), weight_bytes=N * K * 2,
-                   gbs=bytes_ / (statistics.mean(ts) * 1e-6) / 1e9, status=int(status.item()))
+        us, chain = statistics.mean(ts), _back_to_back(stream, fn, 10 * args.reps)
+        out.update(M=M, K=K, N=N, us_mean=us, us_min=min(ts), us_back_to_back=chain, weight_bytes=N * K * 2, gbs=bytes_ / (us * 1e-6) / 1e9,
+                   tflops=2e-6 * M * N * K / us, tflops_back_to_back=2e-6 * M * N * K / chain, status=int(status.item()))
     else:
         shape = MODELS[args.model]
         B = args.batch
@@ -140,8 +154,7 @@ def main():
             ts = _events(stream, fn, args.reps, flush)
             dec.sync()
             out.update(model=args.model, batch=B, k=args.k, prefix=args.prefix, src=args.src,
-                       us_mean=statistics.mean(ts), us_min=min(ts), launch="direct (no graph)")
-            import os
+                       us_mean=statistics.mean(ts), us_min=min(ts), launch="direct" if os.environ.get("AD_NO_ENCODE_GRAPH") == "1" else "block as one graph")
             if os.environ.get("AD_MEGA") == "1" and os.environ.get("AD_MEGA_TIMELINE") == "1":
                 # persistent decoder pass: per stage (inputs visible, signalled) stamps of CTA 0, last step
                 tl = dec.debug_stage_timeline().astype(np.int64)
