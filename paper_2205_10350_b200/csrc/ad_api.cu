@@ -1321,11 +1321,11 @@ bool being_captured(const ad_handle* h) {
 
 // Block-level calls: the words that kernels and captured graphs read, set in stream order (calls with device arrays do not wait for
 // one another) where they are not what the last call left.
-int set_words(ad_handle* h, int k_cap, int beta, float tau) {
+int set_words(ad_handle* h, bool captured, int k_cap, int beta, float tau) {
   int4 w = h->words;
   w.x = k_cap; w.z = beta;
   memcpy(&w.w, &tau, sizeof(tau));
-  if (being_captured(h)) h->foreign_graphs = true;
+  if (captured) h->foreign_graphs = true;
   if (!h->foreign_graphs && !memcmp(&w, &h->words, sizeof(w))) return AD_OK;
   note_launch(h, "set_words");
   AD_CUDA(h, launch_k(set_words_kernel, dim3(1), dim3(1), 0, h->stream, h->st, w));
@@ -1355,10 +1355,10 @@ int graph_entry(ad_handle* h, const char* key, ad_handle::GraphEntry** out) {
 
 // Runs `enqueue` (launches on the handle's stream whose arguments depend only on `key`): the first call with this key directly, so that
 // a form that is called once does not pay for a capture, later ones as a graph captured by the second.  Directly as well where the
-// stream cannot be captured or every launch is being timed.
+// stream cannot be captured (captured: the caller is recording it) or every launch is being timed.
 template <typename F>
-int run_captured(ad_handle* h, const char* key, F enqueue) {
-  if (h->stream == nullptr || being_captured(h) || !h->sw.graph_calls || h->profiling) return enqueue();
+int run_captured(ad_handle* h, bool captured, const char* key, F enqueue) {
+  if (h->stream == nullptr || captured || !h->sw.graph_calls || h->profiling) return enqueue();
   ad_handle::GraphEntry* entry = nullptr;
   AD_TRY(graph_entry(h, key, &entry));
   if (!entry->exec) {
@@ -1633,7 +1633,7 @@ extern "C" int ad_encode(ad_handle* h, const int32_t* src, int32_t src_stride, c
   // per batch size (about fifty launches otherwise paid on the host for every sentence).
   char key[48];
   snprintf(key, sizeof(key), "encode B%d h%d", B, on_host ? 1 : 0);
-  AD_TRY(run_captured(h, key, [&]() -> int {
+  AD_TRY(run_captured(h, being_captured(h), key, [&]() -> int {
     AD_TRY(encode_stage(h, false));
     if (on_host) AD_CUDA(h, launch_k(export_status_kernel, dim3(1), dim3(32), 0, h->stream, h->st, h->dev_view(h->host_flag + 2)));
     return AD_OK;
@@ -1657,7 +1657,8 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
   // written to, mapped host memory), with device arrays everything but the copies from and to the caller's arrays.
   char key[48];
   snprintf(key, sizeof(key), "verify B%d h%d r%d", B, on_host ? 1 : 0, h->beta >= 1 ? 1 : 0);
-  AD_TRY(set_words(h, h->words.x, h->beta, h->tau));
+  const bool captured = being_captured(h);
+  AD_TRY(set_words(h, captured, h->words.x, h->beta, h->tau));
   if (on_host) {
     memcpy(h->up_ids, drafts, sizeof(int) * (size_t)B * c.kmax);
     memcpy(h->up_n, k, sizeof(int) * B);
@@ -1665,7 +1666,7 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
     AD_CUDA(h, cudaMemcpyAsync(h->st.user_drafts, drafts, sizeof(int) * (size_t)B * c.kmax, cudaMemcpyDeviceToDevice, h->stream));
     AD_CUDA(h, cudaMemcpyAsync(h->st.user_k, k, sizeof(int) * B, cudaMemcpyDeviceToDevice, h->stream));
   }
-  AD_TRY(run_captured(h, key, [&]() -> int {
+  AD_TRY(run_captured(h, captured, key, [&]() -> int {
     if (on_host) AD_TRY(prepare_verify(h, SRC_USER, nullptr, h->dev_view(h->up_ids), h->dev_view(h->up_n)));
     else AD_TRY(prepare_verify(h, SRC_USER, nullptr));
     AD_TRY(verify_stage(h, 0));
@@ -1726,8 +1727,9 @@ extern "C" int ad_draft_block(ad_handle* h, int32_t k_cap, int32_t* drafts, int3
   const int B = h->B;
   char key[48];
   snprintf(key, sizeof(key), "draft B%d h%d", B, on_host ? 1 : 0);
-  AD_TRY(set_words(h, k_cap, h->beta, h->tau));
-  AD_TRY(run_captured(h, key, [&]() -> int {
+  const bool captured = being_captured(h);
+  AD_TRY(set_words(h, captured, k_cap, h->beta, h->tau));
+  AD_TRY(run_captured(h, captured, key, [&]() -> int {
     AD_TRY(plan_draft(h));
     AD_TRY(draft_stage(h));
     if (on_host) {
@@ -1890,7 +1892,7 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
   } else {
     char key[48];
     snprintf(key, sizeof(key), "encode B%d c%d", B, capped ? 1 : 0);
-    AD_TRY(run_captured(h, key, [&]() -> int { return encode_stage(h, capped); }));
+    AD_TRY(run_captured(h, being_captured(h), key, [&]() -> int { return encode_stage(h, capped); }));
     AD_CUDA(h, cudaEventRecord(h->ev1, h->stream));
     if (loop_plans_ahead(h)) AD_TRY(plan_first_pass(h, *opts, ovr));
   }
