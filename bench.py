@@ -80,8 +80,8 @@ def reduce_max_sum(dist, dev, seconds_or_ms, count):
 # DRAM counters of one verification step (dram__bytes_read.sum + dram__bytes_write.sum summed over the step's
 # kernels, ncu, caches flushed before every kernel) with the digest of the kernel sources they were taken on:
 # the figures are reported only while the sources still have that digest.
-NCU_COUNTERS = dict(sources_sha256="534c420cabbaffb58020b7fb7dee77e70582493b10b549025962107d408701a6",
-                    step_block40_bytes=92233472, projection_bytes=32864768,
+NCU_COUNTERS = dict(sources_sha256="0e430c475d759b6a39d20977cce86ed52bcb259bc45b68ab222a16f209732ea3",
+                    step_block40_bytes=92251648, projection_bytes=32864512,
                     summary="profiles/verify_step_base_b1_k40_dram_traffic.txt")
 
 
