@@ -80,8 +80,8 @@ struct PassCfg {
   PassPlan plan;
 };
 
-// Launch shape of the tensor-core projection kernel (see tc_shape).
-struct TcShape { int ctas, budget, smem; };
+// Launch shape of the tensor-core projection kernel (see tc_shape); ksplit: the most partial sums of any token count.
+struct TcShape { int ctas, budget, smem, ksplit; };
 
 // A second set of activation buffers (encoder-pass sized) for work that runs on the side stream.
 struct ActSet {
@@ -513,13 +513,13 @@ int tc_smem_need(const GeoRule& r, int M, int budget) {
 // half of that, so that two CTAs share an SM: up to twice the SM count the whole grid is then resident at once, beyond that
 // one CTA's prologue and epilogue overlap the other's K loop.
 TcShape tc_shape(const GeoRule& r, int M_cap, bool exact) {
-  TcShape sh = {1, 0, 0};
+  TcShape sh = {1, 0, 0, 1};
   auto each = [&](auto f) {
     if (exact) { f(M_cap); return; }
     for (int M = 1; M <= M_cap; M += M < 2048 ? 1 : 64) f(M);
     f(M_cap);
   };
-  each([&](int M) { sh.ctas = std::max(sh.ctas, tc::geometry_ctas(r, M)); });
+  each([&](int M) { sh.ctas = std::max(sh.ctas, tc::geometry_ctas(r, M)); sh.ksplit = std::max(sh.ksplit, geometry(r, M).ksplit); });
   sh.budget = (sh.ctas > num_sms() ? 100 : 200) * 1024;
   each([&](int M) { sh.smem = std::max(sh.smem, tc_smem_need(r, M, sh.budget)); });
   return sh;
@@ -892,12 +892,23 @@ int layernorm(ad_handle* h, const PassCfg& pc, const Partials& pre, const float*
   const int d = h->cfg.d_model;
   const LnParams p = {pc.plan.M, pre, bias, h->y, g, b, d, h->cfg.ln_eps, h->y};
   note_launch(h, "residual+layernorm");
-  auto go = [&](auto* yb) -> cudaError_t {
+  // P, the partial sums in flight, from the most that any token count of the pass brings (it sets the registers, see layernorm_kernel)
+  const int most = pre.nsplit > 0 ? pre.nsplit : cached_shape(h, pre.rule, pc.M_cap).ksplit;
+  auto go_n = [&](auto* yb, auto threads, auto parts) -> cudaError_t {
     using ActT = std::remove_pointer_t<decltype(yb)>;
-    if (pc.M_cap >= LN_ROWS && d % 128 == 0)
-      return launch_k(layernorm_many_kernel<ActT>, dim3(std::min(2 * num_sms(), (pc.M_cap + 1) / 2)), dim3(256), 0, h->stream, p, yb);
-    if (d > 512) return launch_k(layernorm_kernel<ActT, 256>, dim3(pc.M_cap), dim3(256), 0, h->stream, p, yb);
-    return launch_k(layernorm_kernel<ActT, 128>, dim3(pc.M_cap), dim3(128), 0, h->stream, p, yb);
+    constexpr int T = decltype(threads)::value, P = decltype(parts)::value, per_cta = 256 / T;
+    // (up to six tokens an SM a CTA each: batch of 8 with drafter, 648 tokens: 7910 us a call, 7930 with CTAs that loop)
+    if (pc.M_cap > 6 * num_sms())
+      return launch_k(layernorm_many_kernel<ActT, T, P>, dim3(std::min(4 * num_sms(), (pc.M_cap + per_cta - 1) / per_cta)), dim3(256), 0, h->stream, p, yb);
+    return launch_k(layernorm_kernel<ActT, T, P>, dim3(pc.M_cap), dim3(T), 0, h->stream, p, yb);
+  };
+  auto go_t = [&](auto* yb, auto threads) -> cudaError_t {
+    if (most <= 4) return go_n(yb, threads, std::integral_constant<int, 4>());
+    if (most <= 8) return go_n(yb, threads, std::integral_constant<int, 8>());
+    return go_n(yb, threads, std::integral_constant<int, 16>());
+  };
+  auto go = [&](auto* yb) -> cudaError_t {
+    return d > 512 ? go_t(yb, std::integral_constant<int, 256>()) : go_t(yb, std::integral_constant<int, 128>());
   };
   void* yb = out ? out->ptr : h->yb.ptr;
   const cudaError_t e = h->bf16 ? go((bf16*)yb) : go((float*)yb);

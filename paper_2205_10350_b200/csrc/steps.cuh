@@ -404,10 +404,10 @@ __device__ __forceinline__ LnWeights ln_weights(const LnParams& p, int gi) {
   return w;
 }
 
-// Token m by a group of THREADS threads, four features per thread (d <= 4 * THREADS): all partial sums of a thread and the
-// residual are requested at once, so the kernel costs one memory round trip.  (Two groups of features per thread took 2.8 us
-// instead of 1.5 us per launch on a 1024-wide model with 16 partials.)
-template <typename ActT, int THREADS>
+// Token m by a group of THREADS threads, four features per thread (d <= 4 * THREADS): the residual and P partial sums of a thread are
+// requested at once, so that with P no smaller than their number the kernel costs one memory round trip.  (Two groups of features per
+// thread took 2.8 us instead of 1.5 us per launch on a 1024-wide model with 16 partials.)
+template <typename ActT, int THREADS, int P>
 __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, int m, int nsplit, size_t stride, ActT* yb, float* red,
                                          int tid, int half) {
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -416,14 +416,22 @@ __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, 
   const bool on = tid < groups;
   float4 v = zero4;
   if (on) {
-    float4 part[16];
+    const float4* pre = reinterpret_cast<const float4*>(p.pre.ptr) + off;
+    const size_t step = stride >> 2;               // (stride is a multiple of d, d of 4)
+    float4 part[P];
 #pragma unroll
-    for (int sp = 0; sp < 16; ++sp)
-      part[sp] = (sp < nsplit) ? reinterpret_cast<const float4*>(p.pre.ptr + sp * stride)[off] : zero4;
+    for (int sp = 0; sp < P; ++sp) part[sp] = sp < nsplit ? pre[sp * step] : zero4;
     const float4 r = p.resid ? reinterpret_cast<const float4*>(p.resid)[off] : zero4;
     v = make_float4(w.c.x + r.x, w.c.y + r.y, w.c.z + r.z, w.c.w + r.w);
 #pragma unroll
-    for (int sp = 0; sp < 16; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
+    for (int sp = 0; sp < P; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
+#pragma unroll 1
+    for (int s0 = P; s0 < nsplit; s0 += P) {
+#pragma unroll
+      for (int sp = 0; sp < P; ++sp) part[sp] = s0 + sp < nsplit ? pre[(s0 + sp) * step] : zero4;
+#pragma unroll
+      for (int sp = 0; sp < P; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
+    }
   }
   const float mean = group_sum<THREADS>(v.x + v.y + v.z + v.w, red, tid, half) / (float)p.d;
   float vs = 0.f;
@@ -444,8 +452,12 @@ __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, 
 }
 
 // One CTA per token.  grid = M_cap, block = THREADS (128 for d <= 512, else 256).
-template <typename ActT, int THREADS>
-__global__ void __launch_bounds__(THREADS)
+// What bounds it: one memory round trip (1.0-1.3 us), and what it keeps from the projection behind it, whose CTAs (32 K registers and up to
+// 200 KB of shared memory each) want to be on the SM before this kernel's wait is over.  With room for 16 partial sums whatever their number
+// (96 registers) the CTAs of a few hundred tokens filled the register files; now 46, 64 or 96-112 registers for up to 4, 8 or 16.
+// Whole calls: 768 wide, batch 16 5090 -> 4805 us; 512 wide, batch 24 with drafter 6310 -> 6000, batch 32 5385 -> 5170; batch 1 1177 -> 1135.
+template <typename ActT, int THREADS, int P>
+__global__ void __launch_bounds__(THREADS, (P <= 4 ? 1280 : P <= 8 ? 1024 : 512) / THREADS)
 layernorm_kernel(const LnParams p, ActT* __restrict__ yb) {
   __shared__ float red[2 * (THREADS / 32)];
   trace_mark(TR_LN, 0);
@@ -459,110 +471,30 @@ layernorm_kernel(const LnParams p, ActT* __restrict__ yb) {
   pdl_wait();
   trace_mark(TR_LN, 1);
   if (m >= M) return;
-  ln_token<ActT, THREADS>(p, w, m, nsplit, stride, yb, red, threadIdx.x, -1);
+  ln_token<ActT, THREADS, P>(p, w, m, nsplit, stride, yb, red, threadIdx.x, -1);
   trace_mark(TR_LN, 2);
 }
 
-// Passes that may hold many tokens.  From LN_ROWS tokens on: one warp per token (no block-wide barrier), the loads of two
-// element groups (residual and up to four partial sums each: ten 16-byte loads per lane) issued before their first use.
-// Below that, or with more than four partials, a group of 128 threads (256 for d > 512) per token as in the kernel above
-// (1024 tokens: 458 us per step of the base model against 467 us with a warp per token; 2048 tokens: 582 against 543 us).
-// grid: at most two CTAs per SM, which loop (a grid sized for the capacity cost 5 us per launch in waves of CTAs without work);
-// block = 256; d a multiple of 128.
-constexpr int LN_ROWS = 1536;
-template <typename ActT>
-__global__ void __launch_bounds__(256, 2)
+// Passes that may hold many tokens: two tokens (one for d > 512) per CTA and turn.  grid: at most four CTAs per SM, which loop (a grid sized
+// for the capacity cost 5 us per launch in waves of CTAs without work); block = 256.
+template <typename ActT, int THREADS, int P>
+__global__ void __launch_bounds__(256, P <= 8 ? 4 : 2)
 layernorm_many_kernel(const LnParams p, ActT* __restrict__ yb) {
-  __shared__ float red[2][16];
+  constexpr int TOKENS = 256 / THREADS;
+  __shared__ float red[TOKENS][2 * (THREADS / 32)];
   trace_mark(TR_LN, 0);
   pdl_launch();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int M = plan_load(p.M_ptr), d = p.d;
+  const int M = plan_load(p.M_ptr);
+  int m = blockIdx.x * TOKENS;
+  if (m >= M && blockIdx.x > 0) return;
+  const int half = TOKENS == 1 ? 0 : threadIdx.x / THREADS, tid = threadIdx.x % THREADS;
+  const LnWeights w = ln_weights(p, tid);
   int nsplit;
   size_t stride;
   resolve_partials(p.pre, M, nsplit, stride);
-  if (M < LN_ROWS || nsplit > 4) {
-    const int per_cta = d <= 512 ? 2 : 1;
-    int m = blockIdx.x * per_cta;
-    if (m >= M && blockIdx.x > 0) return;
-    const LnWeights w = ln_weights(p, per_cta == 2 ? (tid & 127) : tid);
-    pdl_wait();
-    trace_mark(TR_LN, 1);
-    for (; m < M; m += gridDim.x * per_cta) {
-      if (per_cta == 2) {
-        if (m + (tid >> 7) < M) ln_token<ActT, 128>(p, w, m + (tid >> 7), nsplit, stride, yb, red[tid >> 7], tid & 127, tid >> 7);
-      } else {
-        ln_token<ActT, 256>(p, w, m, nsplit, stride, yb, red[0], tid, -1);
-      }
-    }
-    trace_mark(TR_LN, 2);
-    return;
-  }
-  const int per = d >> 7;                               // float4 groups per lane (d / 128), <= 8
-  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  const float *pre = p.pre.ptr, *resid = p.resid, *bias = p.bias;
-  if ((int)blockIdx.x * 8 >= M && blockIdx.x > 0) return;
   pdl_wait();
   trace_mark(TR_LN, 1);
-  for (int m = blockIdx.x * 8 + warp; m < M; m += gridDim.x * 8) {
-    const size_t row = (size_t)m * (d >> 2);
-    float4 xv[8];
-    float s = 0.f;
-#pragma unroll
-    for (int pair = 0; pair < 4; ++pair) {
-      if (pair * 2 >= per) break;
-      float4 r4[2], c4[2], q4[2][4];
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int gi = pair * 2 + i;
-        const size_t off = row + lane + 32 * gi;
-        r4[i] = (gi < per && resid) ? reinterpret_cast<const float4*>(resid)[off] : zero4;
-        c4[i] = (gi < per && bias) ? reinterpret_cast<const float4*>(bias)[lane + 32 * gi] : zero4;
-#pragma unroll
-        for (int sp = 0; sp < 4; ++sp)
-          q4[i][sp] = (gi < per && sp < nsplit) ? reinterpret_cast<const float4*>(pre + sp * stride)[off] : zero4;
-      }
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const int gi = pair * 2 + i;
-        float4 v = r4[i];
-        v.x += c4[i].x; v.y += c4[i].y; v.z += c4[i].z; v.w += c4[i].w;
-#pragma unroll
-        for (int sp = 0; sp < 4; ++sp) { v.x += q4[i][sp].x; v.y += q4[i][sp].y; v.z += q4[i][sp].z; v.w += q4[i][sp].w; }
-        xv[gi] = v;
-        s += v.x + v.y + v.z + v.w;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    const float mean = s / (float)d;
-    float vs = 0.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (i < per) {
-        const float a = xv[i].x - mean, b = xv[i].y - mean, c = xv[i].z - mean, e = xv[i].w - mean;
-        vs += a * a + b * b + c * c + e * e;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) vs += __shfl_xor_sync(0xffffffffu, vs, o);
-    const float inv = rsqrtf(vs / (float)d + p.eps);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      if (i < per) {
-        const float4 gv = reinterpret_cast<const float4*>(p.g)[lane + 32 * i];
-        const float4 bv = reinterpret_cast<const float4*>(p.bta)[lane + 32 * i];
-        float4 o;
-        o.x = gv.x * ((xv[i].x - mean) * inv) + bv.x;
-        o.y = gv.y * ((xv[i].y - mean) * inv) + bv.y;
-        o.z = gv.z * ((xv[i].z - mean) * inv) + bv.z;
-        o.w = gv.w * ((xv[i].w - mean) * inv) + bv.w;
-        const size_t off = (row + lane + 32 * i) * 4;
-        store4(p.y + off, o);
-        store4(yb + off, o);
-      }
-    }
-  }
+  for (m += half; m < M; m += gridDim.x * TOKENS) ln_token<ActT, THREADS, P>(p, w, m, nsplit, stride, yb, red[half], tid, TOKENS == 1 ? -1 : half);
   trace_mark(TR_LN, 2);
 }
 
