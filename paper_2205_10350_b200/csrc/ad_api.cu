@@ -753,7 +753,10 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   p.scale = 1.0f / sqrtf((float)dh);
   // Tensor-core kernels when there are thousands of queries or rows may hold hundreds of keys (max_keys: the capacity, known on
   // the host); the FFMA kernel spreads few queries and few keys over more CTAs.
-  if (h->bf16 && dh == 64 && (many || max_keys >= 256) && !(max_keys >= 256 && pc.seg_max <= 128)) {
+  // An encoder's rows are all queries: 512 wide, batch 2, 200 tokens 765 us a call with the FFMA kernel, 608 with the MMA one; batch 3, 128
+  // tokens 780 -> 692; 768 wide, batch 2, 90 tokens 767 -> 725.
+  const bool encode = &pc == &h->pass[PK_ENCODE];
+  if (h->bf16 && dh == 64 && (many || encode || max_keys >= 256) && (encode || !(max_keys >= 256 && pc.seg_max <= 128))) {
     // Warps share a 16-query tile and split the keys (2 or 4 key groups) when rows have few queries; two groups also while
     // 64-query CTAs would not give every SM two.
     const long full = (long)h->dims.B * ((pc.seg_max + AM_Q - 1) / AM_Q) * c.n_heads;
@@ -823,7 +826,8 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
 // blocks that are shorter and of a drafter's prefix that has not grown leave at once.  A wave costs 4 to 7 us, the projections that
 // are kernels of their own otherwise 12 us a layer, so a verification pass may need three waves at capacity, a drafter's pass
 // (on average half of its capacity) four; an encoder's rows are as long as they are announced, and there is one projection to gain:
-// one wave.  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30: 214 -> 174 us; batch 24, 12:
+// one and a half (batch 5, 75 tokens, 12 layers: 742 us a call, 764 with the MMA kernel and a projection behind it), beyond 512 wide one
+// (768 wide, batch 2, 90 tokens: 757 us with two, 725 with the MMA kernel).  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30: 214 -> 174 us; batch 24, 12:
 // 237 -> 196; batch 20, 1: 188 -> 160; batch of 5 with drafter 442 -> 373; 1024 wide, batch 2, 40: 272 -> 226; batch 3 with drafter
 // 662 -> 600.  Beyond: base batch 32 x 64 (seven waves) 270 -> 315, 1024 wide batch 16 x 1 (four) 239 -> 284.  Wide models with fewer than eight
 // queries a row stay at one wave: their CTAs read two weight slices each for a tile that is mostly padding (768 wide, batch 12, 1: 202
@@ -834,8 +838,9 @@ bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   if (!h->sw.fuse_attn_proj || !h->bf16 || !h->pre2 || c.d_model != c.n_heads * 64 || c.d_model % 128 || c.d_model > 128 * few::MAX_WARPS) return false;
   const int split = few::att_few_split(c.d_model);
   if (max_keys > few::MAX_ROUNDS * few::AK * few::att_few_warps(c.d_model)) return false;
-  const int waves = pk == PK_ENCODE || (split > 1 && pc.seg_max < 8) ? 1 : pk == PK_DRAFT ? 4 : 3;
-  return (long)c.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * split <= (long)waves * num_sms();
+  // (in half waves)
+  const int waves = pk == PK_ENCODE ? (split > 1 ? 2 : 3) : split > 1 && pc.seg_max < 8 ? 2 : pk == PK_DRAFT ? 8 : 6;
+  return 2L * c.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * split <= (long)waves * num_sms();
 }
 
 // Attention with its output projection (partial sums per head in pre2) and, with wq, the query projection of x = yb.

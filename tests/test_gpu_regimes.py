@@ -135,3 +135,29 @@ def test_decode_loop_as_one_graph_equals_direct_launches_at_every_pass_size(B, k
     print(f"B={B} k={k} S={S} {mode}: {sa['iterations']} iterations, {same}/{B} rows identical to block-size-1 decoding")
     assert same >= B - max(1, B // 4)          # near-ties may move a few rows off; a broken loop moves all of them
     dec.close()
+
+
+# last and first capacity on either side of the lines between the encoder's attention kernels
+ENCODE_CASES = [("base", synth.BASE, 5, 80), ("base", synth.BASE, 5, 81), ("base", synth.BASE, 2, 200), ("bart", synth.BART_BASE_SIZED, 2, 97),
+                ("bart", synth.BART_BASE_SIZED, 2, 50)]
+
+
+@pytest.mark.parametrize("name,shape,B,S", ENCODE_CASES, ids=[f"{c[0]}-{c[2]}x{c[3]}" for c in ENCODE_CASES])
+def test_encoder_rows_agree_with_single_row_passes(name, shape, B, S):
+    """The encoder memory of the longest and the shortest row of a ragged batch against the same rows encoded alone (unit-variance rows;
+    the bar is the one of the comparison with the checker)."""
+    r = np.random.default_rng(B * 1000 + S)
+    w = synth.make_weights(shape, 0)
+    src = r.integers(4, shape.vocab, size=(B, S)).astype(np.int32)
+    lens = r.integers(1, S + 1, size=B).astype(np.int32)
+    lens[B - 1] = S
+    dec = binding.AggressiveDecoder(shape, w, max_batch=B, max_src=S, max_tgt=4, kmax=4)
+    dec.encode(src, lens)
+    for b in {int(np.argmin(lens)), B - 1}:
+        n = int(lens[b])
+        one = binding.AggressiveDecoder(shape, w, max_batch=1, max_src=n, max_tgt=4, kmax=4)
+        one.encode(src[b: b + 1, :n], lens[b: b + 1])
+        diff = np.abs(dec.debug_encoder_memory(b, n) - one.debug_encoder_memory(0, n)).max()
+        one.close()
+        assert diff <= 5e-2
+    dec.close()
