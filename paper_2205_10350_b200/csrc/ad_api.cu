@@ -668,6 +668,34 @@ const TcShape& cached_shape(ad_handle* h, const GeoRule& r, int M_cap) {
   return it->second;
 }
 
+// Whether a decoder pass reads more weights than stay in L2 (126 MB, shared with everything else) from one pass to the next.  Its kernels
+// then fetch them from HBM, and can begin to when an SM has room for them, one kernel ahead at most: the feed-forward projections, 128 CTAs
+// that fill an SM's registers each, waited 1.2 us for theirs.  So the QKV projection of a layer, three to four kernels ahead, brings
+// the layer's feed-forward weights into L2, its first feed-forward projection the next layer's attention weights.  Whole calls: 1024 wide
+// (242 MB a pass), batch 4 greedy 7730 -> 7580 us, batch 1 with drafter 3810 -> 3760; 768 wide (176 MB) 2287 -> 2267.  The embedding matrix
+// fetched ahead in the last layers, or the first layer's weights at the end of the vocabulary kernel, gained nothing or lost it again.
+bool weights_stream(const ad_handle* h) {
+  const ad_model_cfg& c = h->cfg;
+  const size_t d = c.d_model;
+  return h->bf16 && h->esz * ((size_t)c.n_dec * (6 * d * d + 2 * d * c.d_ffn) + (size_t)c.vocab * d) > (size_t)100 << 20;
+}
+Prefetch attention_weights(const ad_handle* h, const Model& m, int l) {
+  Prefetch f = {};
+  if (!weights_stream(h) || l >= h->cfg.n_dec) return f;
+  const uint32_t dd = (uint32_t)(h->esz * h->cfg.d_model * h->cfg.d_model);
+  f.ptr[0] = (const char*)m.dec[l].wqkv.ptr; f.bytes[0] = 5 * dd;      // wqkv, wo, cq: one behind the other
+  f.ptr[1] = (const char*)m.dec[l].co.ptr; f.bytes[1] = dd;
+  return f;
+}
+Prefetch ffn_weights(const ad_handle* h, const Model& m, int l) {
+  Prefetch f = {};
+  if (!weights_stream(h)) return f;
+  const uint32_t df = (uint32_t)(h->esz * h->cfg.d_model * h->cfg.d_ffn);
+  f.ptr[0] = (const char*)m.dec[l].w1.ptr; f.bytes[0] = df;
+  f.ptr[1] = (const char*)m.dec[l].w2.ptr; f.bytes[1] = df;
+  return f;
+}
+
 // embed_of: the operand is the embedding of pass pk's tokens (first projection of a pass, few-token kernel only).
 // split: the result is partial sums that the consumer adds up (EPI_F32).
 int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int* M_ptr, int M_cap, GemmParams p, const Model* embed_of = nullptr,
@@ -960,9 +988,10 @@ int embed_or_defer(ad_handle* h, int pk, const Model& m, const Mat& first, const
 
 // Self-attention sublayer + FFN shared by the encoder and decoder layers.
 int self_attention_sublayer(ad_handle* h, int pk, const Mat& wqkv, const float* bqkv, const Mat& wo, const float* bo,
-                            const float* lng, const float* lnb, void* kbuf, void* vbuf, const Model* embed_of = nullptr) {
+                            const float* lng, const float* lnb, void* kbuf, void* vbuf, const Model* embed_of = nullptr, const Prefetch& next = {}) {
   PassCfg& pc = h->pass[pk];
   GemmParams p = {};
+  p.next = next;
   p.bias = bqkv; p.dst[0] = h->qbuf; p.dst[1] = kbuf; p.dst[2] = vbuf; p.seg_width = h->cfg.d_model; p.n_direct = 1;
   p.slot = pc.plan.kv_slot;
   AD_TRY(gemm(h, EPI_SCATTER, wqkv, h->yb, pk, pc.plan.M, pc.M_cap, p, embed_of));
@@ -980,9 +1009,10 @@ int self_attention_sublayer(ad_handle* h, int pk, const Mat& wqkv, const float* 
 }
 
 int ffn_sublayer(ad_handle* h, int pk, const Mat& w1, const float* b1, const Mat& w2, const float* b2, const float* lng,
-                 const float* lnb, const ActBuf* out = nullptr) {
+                 const float* lnb, const ActBuf* out = nullptr, const Prefetch& next = {}) {
   PassCfg& pc = h->pass[pk];
   GemmParams a = {};
+  a.next = next;
   a.bias = b1; a.relu = 1; a.out_act = h->hbuf.ptr;
   AD_TRY(gemm(h, EPI_ACT, w1, h->yb, pk, pc.plan.M, pc.M_cap, a));
   Partials ps;
@@ -1132,7 +1162,8 @@ int decoder_pass(ad_handle* h, int pk, Model& m) {
     DecLayer& L = m.dec[l];
     void* kb = pk == PK_VERIFY ? (char*)h->kself + l * self_layer : h->ktmp;
     void* vb = pk == PK_VERIFY ? (char*)h->vself + l * self_layer : h->vtmp;
-    AD_TRY(self_attention_sublayer(h, pk, L.wqkv, L.bqkv, L.wo, L.bo, L.ln1g, L.ln1b, kb, vb, l == 0 ? defer : nullptr));
+    AD_TRY(self_attention_sublayer(h, pk, L.wqkv, L.bqkv, L.wo, L.bo, L.ln1g, L.ln1b, kb, vb, l == 0 ? defer : nullptr, ffn_weights(h, m, l)));
+    const Prefetch next = attention_weights(h, m, l + 1);
     // Query projection of the cross-attention.  With few tokens a full-K walk per CTA is the slow part of the
     // projection, so it is split along K and the attention kernel adds the partial sums (and the bias) as it
     // loads its queries.
@@ -1141,7 +1172,7 @@ int decoder_pass(ad_handle* h, int pk, Model& m) {
       AD_TRY(attention_few(h, pc, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->st.cross_base, nullptr, h->st.srclen, c.max_src,
                            L.co, &L.cq, L.cbq));
       AD_TRY(layernorm(h, pc, head_partials(h, pc), L.cbo, L.ln2g, L.ln2b));
-      AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b));
+      AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b, nullptr, next));
       continue;
     }
     if (h->bf16 && pc.M_cap <= 256) {
@@ -1163,7 +1194,7 @@ int decoder_pass(ad_handle* h, int pk, Model& m) {
       AD_TRY(gemm_to_partials(h, L.co, h->abuf, pk, &ps));
       AD_TRY(layernorm(h, pc, ps, L.cbo, L.ln2g, L.ln2b));
     }
-    AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b));
+    AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b, nullptr, next));
   }
   return AD_OK;
 }

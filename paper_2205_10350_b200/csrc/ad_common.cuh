@@ -119,6 +119,12 @@ __device__ __forceinline__ void resolve_partials(const Partials& q, int M, int& 
   stride = q.nsplit > 0 ? q.stride : (size_t)M * q.rule.N;
 }
 
+// Weights that kernels further down the chain will read, to be brought into L2 (see prefetch_share).
+struct Prefetch {
+  const char* ptr[2];
+  uint32_t bytes[2];     // multiples of 16; 0: nothing
+};
+
 struct GemmParams {
   int K;                 // contraction length
   int N;                 // output features (rows of W)
@@ -147,6 +153,7 @@ struct GemmParams {
   const int* draft_id;     // [M_cap] (negative: no draft at this position)
   int* part_cnt;           // [M_cap, n_tiles]
   int* status;           // device status word (latches AD_ERR_TIMEOUT), may be null
+  Prefetch next;         // few-token kernel for wide slices of K: what to bring into L2
 };
 
 // Programmatic dependent launch: a kernel launched with the programmatic-serialization attribute may start
@@ -208,6 +215,17 @@ __device__ __forceinline__ void trace_mark_role(int, int) {}
 #endif
 enum TraceId { TR_GEMM = 0, TR_ATTN = 8, TR_LN = 9, TR_EMBED = 10, TR_PREPARE = 11, TR_ACCEPT = 12, TR_COMMIT = 13,
                TR_PV_ISSUE = 20, TR_PV_EPI = 21, TR_PV_LOAD = 22 };
+
+// Share i of n of what is to be brought into L2, in pieces that one thread hands to the SM's bulk-copy unit; nothing waits for them.
+// To be shared by a hundred CTAs: one CTA alone (the accept kernel was tried) gets no more than its SM's share of the way into L2 and stays
+// until all is through.
+constexpr uint32_t PF_PIECE = 8192;
+__device__ __forceinline__ void prefetch_share(const Prefetch& f, uint32_t i, uint32_t n) {
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+    for (uint32_t o = i * PF_PIECE; o < f.bytes[r]; o += n * PF_PIECE)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(f.ptr[r] + o), "r"(min(PF_PIECE, f.bytes[r] - o)) : "memory");
+}
 
 __device__ __forceinline__ void latch_error(int* status, int code) {
   if (status) atomicCAS(status, 0, code);

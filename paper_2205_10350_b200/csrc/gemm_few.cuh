@@ -242,6 +242,7 @@ gemm_few_wide_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams
       wa[f][c][0] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + 16 * f + g) * K + kbase + 32 * c));
       wa[f][c][1] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + 16 * f + g + 8) * K + kbase + 32 * c));
     }
+  if (tid == THREADS - 1) prefetch_share(p.next, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   const int of = (tid & 7) * 4, ot = tid >> 3;               // this thread's output: four features of one token per round
   float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
   if (EPI != EPI_F32) bias = *reinterpret_cast<const float4*>(p.bias + n0 + of);
