@@ -2,6 +2,8 @@
 // commit, the choice of the next block and the layout of the pass that verifies it, all in one kernel.
 #pragma once
 
+#include <type_traits>
+
 #include "gemm_tc.cuh"   // float_key
 #include "steps.cuh"
 
@@ -38,7 +40,6 @@ __device__ __forceinline__ int cta_suffix_match(OutTok o, int j, const int* x, i
     if (count == 0) break;
     __syncthreads();
   }
-  __syncthreads();
   return found;
 }
 
@@ -102,15 +103,22 @@ __device__ __forceinline__ void scan_tiles(const float* __restrict__ val, const 
 // read before the dependency wait, and from the partials to the next plan everything stays in shared memory: one round trip
 // for the partials (plus the hand-over between CTAs when B > 1).
 // Batch 1, 40-token blocks: 11.4 us with the state, the match and the plan in global memory.
-// grid = B, block = 1024.
+// CLUSTER (2 to ACC_CLUSTER rows of a decode loop): the rows' CTAs are a cluster; each tells the others its next block's size through
+// distributed shared memory and lays its own row out.  Through global memory (a counter, fences, the last CTA reads what the others wrote
+// and lays out all rows: 3.3 us and 1.8 us) an iteration takes 2.2 us longer with 4 rows, 3 us with 8.  More rows take that way still.
+// grid = B, block = 1024; CLUSTER: cluster (B, 1, 1).
+constexpr int ACC_CLUSTER = 16;
+template <bool CLUSTER>
 __global__ void __launch_bounds__(ACC_THREADS)
 argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict__ part_val, const int* __restrict__ part_idx,
                      int n_tiles, int to_drafts, int auto_commit, unsigned int* done_ctr, unsigned long long cond, int relaxed_on,
                      const float* __restrict__ draft_val, const int* __restrict__ draft_id,
                      const int* __restrict__ part_cnt, NextPass next) {
   __shared__ int s_dr[256], s_pred[256], s_src[ACC_SRC];
-  __shared__ int s_k[256], s_off[257], s_len[256];
+  __shared__ int s_k[256], s_off[256], s_boff[256], s_len[256];
+  __shared__ int s_next[256], s_row[CLUSTER ? ACC_CLUSTER : 1];   // the next block's drafts; per row: 1 finished, 2 took part
   __shared__ int s_n, s_last_cta, s_where;
+  if (CLUSTER) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");      // (a CTA's shared memory may be written once it is known to run)
   trace_mark(TR_ACCEPT, 0);
   if (next.source < 0) pdl_launch();     // a kernel that plans never does (see plan data in ad_common.cuh)
   const int b = blockIdx.x, B = dm.B;
@@ -189,22 +197,17 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
 
   // ---- the decision ----
   trace_mark(TR_ACCEPT, 3);
-  if (warp == 0) {
-    int n = k;
-    for (int i0 = 0; i0 < k; i0 += 32) {
-      const int i = i0 + lane;
-      const unsigned bal = __ballot_sync(0xffffffffu, i < k && (s_dr[i] < 0 || s_pred[i] != s_dr[i]));
-      if (bal) { n = i0 + __ffs(bal); break; }
-    }
-    for (int i0 = 0; i0 < n; i0 += 32) {
-      const int i = i0 + lane;
-      const unsigned bal = __ballot_sync(0xffffffffu, i < n && s_pred[i] == dm.eos);
-      if (bal) { n = i0 + __ffs(bal); break; }
-    }
-    if (lane == 0) s_n = n;
+  int n = k;                               // (every warp for itself)
+  for (int i0 = 0; i0 < k; i0 += 32) {
+    const int i = i0 + lane;
+    const unsigned bal = __ballot_sync(0xffffffffu, i < k && (s_dr[i] < 0 || s_pred[i] != s_dr[i]));
+    if (bal) { n = i0 + __ffs(bal); break; }
   }
-  __syncthreads();
-  const int n = s_n;
+  for (int i0 = 0; i0 < n; i0 += 32) {
+    const int i = i0 + lane;
+    const unsigned bal = __ballot_sync(0xffffffffu, i < n && s_pred[i] == dm.eos);
+    if (bal) { n = i0 + __ffs(bal); break; }
+  }
   if (!auto_commit) {
     if (tid == 0) st.n_acc[b] = n;
     return;
@@ -233,29 +236,48 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
         const int i = cta_suffix_match(o, len1, x, n_src, dm.bos, &s_where);
         // draft = x_{i+1..n} followed by the [PAD] slot that matches nothing; a plain step without a match
         k1 = i >= 0 ? min(n_src - i + 1, min(k_cap, maxlen - len1)) : 1;
-        if (tid < k1) s_dr[tid] = (i >= 0 && i + 1 + tid <= n_src) ? x[i + tid] : -1;
+        if (tid < k1) s_next[tid] = (i >= 0 && i + 1 + tid <= n_src) ? x[i + tid] : -1;
       }
     } else {
       k1 = live ? min(k_cap, maxlen - len1) : 0;
       if (next.source == SRC_OVERRIDE && tid < k1)
-        s_dr[tid] = len1 + tid < override_len ? next.override_stream[(size_t)b * next.override_stride + len1 + tid] : -1;
+        s_next[tid] = len1 + tid < override_len ? next.override_stream[(size_t)b * next.override_stride + len1 + tid] : -1;
     }
     if (next.source != SRC_SIZES && tid < k1) {
-      int dr = s_dr[tid];
+      int dr = s_next[tid];
       // a caller-provided draft beyond the vocabulary becomes a slot that matches nothing (negative = sentinel is legal)
-      if (dr >= dm.vocab) { latch_error(st.status, AD_ERR_ARG); dr = -1; s_dr[tid] = dr; }
+      if (dr >= dm.vocab) { latch_error(st.status, AD_ERR_ARG); dr = -1; s_next[tid] = dr; }
       st.drafts[(size_t)b * dm.kmax + tid] = dr;
     }
     if (tid == 0) {
       blk.seg_len[b] = k1; blk.key_base[b] = b * dm.max_tgt; blk.row_nk[b] = len1 + k1;
-      s_k[b] = k1; s_len[b] = len1;
+      if (!CLUSTER) { s_k[b] = k1; s_len[b] = len1; }
     }
   }
-  // ---- the last row to get here sees all of them ----
+  // ---- what the rows have to tell one another; without a cluster the last row to get here sees all of them ----
   trace_mark(TR_ACCEPT, 5);
-  __syncthreads();
   bool all_fin = fin1 != 0, any_active = n > 0;
-  if (B > 1) {
+  if (CLUSTER) {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (tid < B) {
+      auto tell = [&](int* mine, int v) {
+        uint32_t a;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(mine))), "r"(tid));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+      };
+      tell(s_k + b, k1); tell(s_len + b, len1); tell(s_row + b, (fin1 ? 1 : 0) | (n > 0 ? 2 : 0));
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const int row = lane < B ? s_row[lane] : 1;
+    all_fin = __all_sync(0xffffffffu, row & 1);
+    any_active = __any_sync(0xffffffffu, row & 2);
+  } else {
+    __syncthreads();
+  }
+  if (!CLUSTER && B > 1) {
     if (tid == 0) {
       __threadfence();
       const unsigned int t = atomicAdd(done_ctr, n > 0 ? 0x10001u : 1u);
@@ -272,7 +294,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
     }
     all_fin = __syncthreads_and(f) != 0;
   }
-  if (tid == ACC_THREADS - 1) {            // (not a thread of the warp that lays the rows out)
+  if (tid == ACC_THREADS - 1 && (!CLUSTER || b == 0)) {            // (not a thread of the warp that lays the rows out)
     *done_ctr = 0;
     if (any_active) *st.loop_it = it_active + 1;
     *st.all_fin = all_fin;
@@ -287,56 +309,75 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
   // ---- layout of the pass behind this kernel ----
   trace_mark(TR_ACCEPT, 6);
   const bool draft_pass = next.source == SRC_SIZES;
-  if (warp == 0) {                         // offsets: an exclusive scan over the rows
-    int base = 0, dbase = 0;
-    for (int b0 = 0; b0 < B; b0 += 32) {
-      const int r = b0 + lane, kr = r < B ? s_k[r] : 0;
-      const int dr = kr > 0 ? s_len[r] + 1 + kr : 0;     // drafter's tokens of the row: [BOS], accepted tokens, k x [MASK]
-      int sum = kr, dsum = dr;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int a = __shfl_up_sync(0xffffffffu, sum, o), c = __shfl_up_sync(0xffffffffu, dsum, o);
-        if (lane >= o) { sum += a; dsum += c; }
-      }
-      if (r < B) {
-        blk.seg_off[r] = base + sum - kr;
-        s_off[r] = draft_pass ? dbase + dsum - dr : base + sum - kr;
-        if (draft_pass) s_k[r] = (int)((unsigned)kr | (unsigned)(base + sum - kr) << 16);   // block size and block offset (both below 65536)
-      }
-      base += __shfl_sync(0xffffffffu, sum, 31);
-      dbase += __shfl_sync(0xffffffffu, dsum, 31);
-    }
-    if (lane == 0) {
-      s_off[B] = draft_pass ? dbase : base;
-      *blk.M = base;
-      if (draft_pass) *next.draft.M = dbase;
-    }
-  }
-  __syncthreads();
-  for (int r = warp; r < B; r += ACC_THREADS / 32) {
-    const int o0 = s_off[r], lr = s_len[r];
+  // drafter's tokens of a row: [BOS], accepted tokens, k x [MASK]
+  auto draft_tokens = [&](int r) { return s_k[r] > 0 ? s_len[r] + 1 + s_k[r] : 0; };
+  // tokens of row r from o0 on (block offset boff), by the lanes of a group; alone: the row is this CTA's own
+  auto lay_out = [&](int r, int o0, int boff, int first, int step, auto alone) {
+    constexpr bool ALONE = decltype(alone)::value;
+    const int lr = s_len[r], kr = s_k[r];
     if (draft_pass) {
-      const int kr = s_k[r] & 0xffff, boff = (int)((unsigned)s_k[r] >> 16), nr = kr > 0 ? lr + 1 + kr : 0;
+      const int nr = draft_tokens(r);
       const PassPlan& pl = next.draft;
-      if (lane == 0) { pl.seg_off[r] = o0; pl.seg_len[r] = nr; pl.key_base[r] = o0; pl.row_nk[r] = nr; }
-      for (int i = lane; i < nr; i += 32) {
+      if (first == 0) { pl.seg_off[r] = o0; pl.seg_len[r] = nr; pl.key_base[r] = o0; pl.row_nk[r] = nr; }
+      for (int i = first; i < nr; i += step) {
         const int m = o0 + i;
-        int tok = i == 0 ? dm.bos : (i <= lr ? __ldcg(st.out_ids + (size_t)r * dm.max_tgt + i - 1) : dm.mask);
+        int tok = i == 0 ? dm.bos : i > lr ? dm.mask : ALONE && i > len ? s_pred[i - 1 - len] : __ldcg(st.out_ids + (size_t)r * dm.max_tgt + i - 1);
         if (!id_in_vocab(tok, dm)) { latch_error(st.status, AD_ERR_ARG); tok = dm.pad; }
         pl.tok_row[m] = r; pl.tok_pos[m] = i; pl.tok_id[m] = tok; pl.kv_slot[m] = m; pl.att_n[m] = nr;
       }
-      for (int i = lane; i < kr; i += 32) st.gidx[boff + i] = o0 + lr + 1 + i;
+      for (int i = first; i < kr; i += step) st.gidx[boff + i] = o0 + lr + 1 + i;
     } else {
-      const int kr = s_k[r];
-      const int* dr = B == 1 ? s_dr : st.drafts + (size_t)r * dm.kmax;
-      for (int i = lane; i < kr; i += 32) {
+      const int* dr = st.drafts + (size_t)r * dm.kmax;
+      for (int i = first; i < kr; i += step) {
         const int m = o0 + i;
-        int tok = B == 1 ? (i == 0 ? last1 : dr[i - 1]) : (i == 0 ? __ldcg(st.last + r) : __ldcg(dr + i - 1));
+        int tok = ALONE ? (i == 0 ? last1 : s_next[i - 1]) : (i == 0 ? __ldcg(st.last + r) : __ldcg(dr + i - 1));
         if (tok < 0 || tok >= dm.vocab) tok = dm.pad;
         blk.tok_row[m] = r; blk.tok_pos[m] = lr + i; blk.tok_id[m] = tok;
         blk.kv_slot[m] = r * dm.max_tgt + lr + i; blk.att_n[m] = lr + i + 1;
       }
     }
+  };
+  if (CLUSTER || B == 1) {
+    // (at most 16 rows: every warp adds up those in front of its own)
+    const int kr = lane < B ? s_k[lane] : 0, dr = lane < B && draft_pass ? draft_tokens(lane) : 0;
+    const int boff = __reduce_add_sync(0xffffffffu, lane < b ? kr : 0), all = __reduce_add_sync(0xffffffffu, kr);
+    const int doff = __reduce_add_sync(0xffffffffu, lane < b ? dr : 0), dall = __reduce_add_sync(0xffffffffu, dr);
+    const int o0 = draft_pass ? doff : boff;
+    if (tid == 0) {
+      blk.seg_off[b] = boff;
+      if (b == 0) {
+        *blk.M = all;
+        if (draft_pass) *next.draft.M = dall;
+      }
+    }
+    lay_out(b, o0, boff, tid, ACC_THREADS, std::true_type());
+  } else {
+    if (warp == 0) {                       // offsets: an exclusive scan over the rows
+      int base = 0, dbase = 0;
+      for (int b0 = 0; b0 < B; b0 += 32) {
+        const int r = b0 + lane, kr = r < B ? s_k[r] : 0;
+        const int dr = r < B ? draft_tokens(r) : 0;
+        int sum = kr, dsum = dr;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int a = __shfl_up_sync(0xffffffffu, sum, o), c = __shfl_up_sync(0xffffffffu, dsum, o);
+          if (lane >= o) { sum += a; dsum += c; }
+        }
+        if (r < B) {
+          blk.seg_off[r] = base + sum - kr;
+          s_off[r] = draft_pass ? dbase + dsum - dr : base + sum - kr;
+          s_boff[r] = base + sum - kr;
+        }
+        base += __shfl_sync(0xffffffffu, sum, 31);
+        dbase += __shfl_sync(0xffffffffu, dsum, 31);
+      }
+      if (lane == 0) {
+        *blk.M = base;
+        if (draft_pass) *next.draft.M = dbase;
+      }
+    }
+    __syncthreads();
+    for (int r = warp; r < B; r += ACC_THREADS / 32) lay_out(r, s_off[r], s_boff[r], lane, 32, std::false_type());
   }
   __threadfence();
   trace_mark(TR_ACCEPT, 2);

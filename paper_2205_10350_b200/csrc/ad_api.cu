@@ -1245,10 +1245,34 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
   }
   if (!partials_ready) AD_TRY(gemm(h, EPI_ARGMAX, m.emb, X, PK_VERIFY, pc.plan.M, pc.M_cap, p));
   note_launch(h, "argmax_accept");
-  AD_CUDA(h, launch_k(argmax_accept_kernel, dim3(h->dims.B), dim3(ACC_THREADS), 0, h->stream, h->st, pc.plan, h->dims, (const float*)h->part_val,
-                      (const int*)h->part_idx, h->n_vtiles, to_drafts, auto_commit, (unsigned int*)(h->st.loop_it + 1),
-                      auto_commit ? h->cond_handle : 0ull, relaxed ? 1 : 0, (const float*)h->draft_val, (const int*)h->draft_id,
-                      (const int*)h->part_cnt, h->next_pass));
+  // the rows of a decode loop as a cluster (up to 8 CTAs everywhere, 16 on this device)
+  const int B = h->dims.B;
+  const bool cluster = auto_commit && !to_drafts && B > 1 && B <= ACC_CLUSTER;
+  if (cluster && B > 8) {
+    static bool attr_set[kMaxDevices] = {};
+    const int dev = current_device();
+    if (!attr_set[dev]) {
+      AD_CUDA(h, cudaFuncSetAttribute(argmax_accept_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      attr_set[dev] = true;
+    }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(B); cfg.blockDim = dim3(ACC_THREADS); cfg.stream = h->stream;
+  cudaLaunchAttribute attr[2];
+  int n_attr = 0;
+  if (use_pdl()) {
+    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster) {
+    attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+    attr[n_attr].val.clusterDim.x = B; attr[n_attr].val.clusterDim.y = 1; attr[n_attr++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr; cfg.numAttrs = n_attr;
+  AD_CUDA(h, cudaLaunchKernelEx(&cfg, cluster ? argmax_accept_kernel<true> : argmax_accept_kernel<false>, h->st, pc.plan, h->dims, (const float*)h->part_val,
+                                (const int*)h->part_idx, h->n_vtiles, to_drafts, auto_commit, (unsigned int*)(h->st.loop_it + 1),
+                                auto_commit ? h->cond_handle : 0ull, relaxed ? 1 : 0, (const float*)h->draft_val, (const int*)h->draft_id,
+                                (const int*)h->part_cnt, h->next_pass));
   h->last_vocab_which = to_drafts ? 1 : 0;
   return AD_OK;
 }

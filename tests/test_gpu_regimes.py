@@ -161,3 +161,27 @@ def test_encoder_rows_agree_with_single_row_passes(name, shape, B, S):
         one.close()
         assert diff <= 5e-2
     dec.close()
+
+
+@pytest.mark.parametrize("B", [2, 8, 9, 16, 17])
+def test_rows_of_a_loop_end_like_single_rows(B):
+    """Decode loops around the numbers of rows whose accept kernels are one cluster (8 CTAs everywhere, up to 16 here, none beyond): tokens,
+    iterations and offered drafts of every row as in a loop of its own.  FP32: the arithmetic leaves no doubt."""
+    shape = synth.TINY
+    w, wn = synth.make_weights(shape, 0), synth.make_weights(shape, 1)
+    r = np.random.default_rng(B)
+    S, T = 12, 14
+    src = r.integers(4, shape.vocab, size=(B, S)).astype(np.int32)
+    lens = r.integers(2, S + 1, size=B).astype(np.int32)
+    cap = r.integers(1, T + 1, size=B).astype(np.int32)
+    many = binding.AggressiveDecoder(shape, w, wn, max_batch=B, max_src=S, max_tgt=T, kmax=6)
+    one = binding.AggressiveDecoder(shape, w, wn, max_batch=1, max_src=S, max_tgt=T, kmax=6)
+    for opts in (dict(mode="IAD", k=6), dict(mode="GAD", k=5, run_drafter=True)):
+        out, st = many.generate(src, lens, max_len=cap, **opts)
+        alone = [one.generate(src[b: b + 1], lens[b: b + 1], max_len=cap[b: b + 1], **opts) for b in range(B)]
+        assert all(np.array_equal(out[b], alone[b][0][0]) for b in range(B))
+        assert st["iterations"] == max(a[1]["iterations"] for a in alone)
+        for key in ("row_iterations", "accepted", "offered"):
+            assert st[key] == sum(a[1][key] for a in alone)
+    many.close()
+    one.close()
