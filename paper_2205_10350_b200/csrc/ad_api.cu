@@ -2285,7 +2285,12 @@ namespace {
 // Geometry of an operator-level call over M tokens (by the passes' rule), and the token operand's map for its tile.
 bool op_maps(GemmParams* p, tc::TileMaps* mx, const void* x, int M, int K) {
   p->rule = GeoRule{p->N, K, clampi(pow2ceil(M), 16, 256), 1, num_sms(), 0, 0, 0};
-  const int tile = p->rule.fixed_tile = geometry(p->rule, M).tile;
+  int tile = geometry(p->rule, M).tile;
+  // No K split here: tiles of half the tokens while they leave SMs without work (1800 x 2048 x 512, 60 CTAs with the passes' 128-token
+  // tiles: a call 25.5 us, 23.6 with 64; 1100 tokens 24.8, 22.7 with 64, 22.1 with 32; 100 x 4096 x 1024 26.1, 24.8 with 32).
+  const int nf = (p->N + tc::BLOCK_N_FEAT - 1) / tc::BLOCK_N_FEAT;
+  while (tile > 32 && 2 * nf * ((M + tile - 1) / tile) <= num_sms()) tile /= 2;
+  p->rule.fixed_tile = tile;
   int i = 0;
   while ((16 << i) < tile) ++i;
   memset(mx, 0, sizeof(*mx));

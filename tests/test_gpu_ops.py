@@ -159,3 +159,15 @@ def test_linear_into_a_result_of_any_float_alignment(dtype, shift):
     torch.cuda.synchronize()
     assert torch.equal(y.view(M, N), binding.linear(x, W, b.clone()))
     assert (buf[:shift] == 7.0).all() and (buf[shift + M * N:] == 7.0).all() and int(st.item()) == 0
+
+
+@pytest.mark.parametrize("M,K,N", [(2304, 512, 512), (2305, 512, 512), (1152, 2048, 512), (1153, 320, 500), (33, 4096, 1024), (97, 64, 130)])
+def test_projection_tiles_on_either_side_of_their_lines(M, K, N):
+    """Token counts around which an operator-level projection takes tiles of 128, 64 and 32 tokens (four 128-row weight tiles on 148 SMs), and
+    ragged ones.  FP32 sums of exact products: K additions of terms of the result's size."""
+    x, W, b = _data(M, K, N, True, seed=M + K)
+    st = torch.zeros(1, dtype=torch.int32, device=DEV)
+    y = binding.linear(torch.tensor(x, device=DEV).bfloat16(), torch.tensor(W, device=DEV).bfloat16(), torch.tensor(b, device=DEV), st).cpu().numpy()
+    ref = x.astype(np.float64) @ W.T.astype(np.float64) + b
+    assert int(st.item()) == 0
+    assert np.abs(y - ref).max() <= 2.0 ** -24 * K * np.abs(x).max() * np.abs(W).max() * 8
