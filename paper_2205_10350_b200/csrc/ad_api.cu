@@ -595,6 +595,19 @@ cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmP
   const dim3 grid(p.N / few::FEAT, ksplit);
   const bf16 *w = (const bf16*)W.ptr, *xp = (const bf16*)x;
   const dim3 wgrid(p.N / few::W_FEAT, ksplit);
+  // A quarter of the SM's memory as shared memory, enough for one CTA of the 16-feature forms (41 KB each): left to itself the runtime
+  // makes room for two, and the 96 to 128 CTAs of a grid share 64 SMs while others stand by (the weights and activations of both then queue
+  // for one L1).  Whole calls, the runtime's choice -> this: 512 wide, batch 1 1124 -> 1075 us, batch 2 with drafter 4360 -> 3950, batch 8
+  // 3560 -> 3520; 12+2, batch 1 960 -> 906.  43 % (two CTAs fit again): 1120, 4300, 3530, 961.
+  static bool attr_set[kMaxDevices] = {};
+  const int dev = current_device();
+  if (!attr_set[dev]) {
+    for (auto* kernel : {few::gemm_few_kernel<EPI, 1, EMB>, few::gemm_few_kernel<EPI, 2, EMB>}) {
+      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
+      if (e != cudaSuccess) return e;
+    }
+    attr_set[dev] = true;
+  }
   switch (p.K / ksplit / 256) {
     case 1: return launch_k(few::gemm_few_kernel<EPI, 1, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
     case 2: return launch_k(few::gemm_few_kernel<EPI, 2, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);

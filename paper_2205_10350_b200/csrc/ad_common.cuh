@@ -174,6 +174,14 @@ __device__ __forceinline__ int plan_load(const int* p) { return __ldcg(p); }
 // while the predecessor runs.  One CTA of the grid always waits, work or not: a grid that completed before its predecessor
 // would release its own successors too early.
 
+// 16 bytes of weights that one CTA reads once, kept out of L1 (whole calls: batch 1 1133 -> 1124 us, batch 8 3587 -> 3548; not for the
+// attention's weights, which the CTAs of a row's other query chunks read again: batch 8 with drafter 7865 -> 8090).
+__device__ __forceinline__ uint4 weight_load_once(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 // Optional timeline tracing (compile with -DAD_TRACE): thread 0 of CTA (0,0,0) of every kernel stamps the
 // global nanosecond timer at entry (phase 0), after the dependency wait (phase 1), at exit (phase 2) and at
 // kernel-specific points in between (phases 3..7); the last CTA along x does the same under id + 16.

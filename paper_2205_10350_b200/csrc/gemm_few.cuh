@@ -138,8 +138,8 @@ __device__ __forceinline__ void few_body(const bf16* __restrict__ W, const bf16*
   uint4 wa[NCH][2];
 #pragma unroll
   for (int c = 0; c < NCH; ++c) {
-    wa[c][0] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + g) * K + kbase + 32 * c));
-    wa[c][1] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + g + 8) * K + kbase + 32 * c));
+    wa[c][0] = weight_load_once(W + (size_t)(n0 + g) * K + kbase + 32 * c);
+    wa[c][1] = weight_load_once(W + (size_t)(n0 + g + 8) * K + kbase + 32 * c);
   }
   const int of = (tid & 3) * 4, ot = tid >> 2;               // this thread's output: four features of one token per round
   float4 bias = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -239,8 +239,8 @@ gemm_few_wide_kernel(const bf16* __restrict__ W, const bf16* X, const GemmParams
   for (int f = 0; f < 2; ++f)
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
-      wa[f][c][0] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + 16 * f + g) * K + kbase + 32 * c));
-      wa[f][c][1] = __ldg(reinterpret_cast<const uint4*>(W + (size_t)(n0 + 16 * f + g + 8) * K + kbase + 32 * c));
+      wa[f][c][0] = weight_load_once(W + (size_t)(n0 + 16 * f + g) * K + kbase + 32 * c);
+      wa[f][c][1] = weight_load_once(W + (size_t)(n0 + 16 * f + g + 8) * K + kbase + 32 * c);
     }
   if (tid == THREADS - 1) prefetch_share(p.next, blockIdx.y * gridDim.x + blockIdx.x, gridDim.x * gridDim.y);
   const int of = (tid & 7) * 4, ot = tid >> 3;               // this thread's output: four features of one token per round
