@@ -656,19 +656,35 @@ cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const Gem
 }
 // The few-token FP32 kernel: passes of at most kFewTokens tokens, shapes it covers.
 bool f32_few(const PassCfg& pc, int epi, int N, int K) { return pc.M_cap <= kFewTokens && epi != EPI_ARGMAX && simt::few_fits(N, K); }
+// Most shared memory that leaves room for one CTA of `kernel` an SM, as the share of the SM's memory to prefer (see launch_few: CTAs of a
+// small grid that share SMs while others stand by).  With both FP32 kernels of a sublayer one an SM, whole calls of the 128-wide model: batch 6
+// 1565 -> 1520 us, batch 2 with drafter 1251 -> 1229, batch 1 551 -> 549.
+template <typename K>
+cudaError_t one_cta_per_sm(K* kernel, size_t smem_bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)((smem_bytes + 1024) * 100 / (228 * 1024)) + 1);
+}
+template <int EPI, int NQ>
+cudaError_t launch_simt_few_n(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p) {
+  static bool attr_set[kMaxDevices] = {};
+  const int dev = current_device();
+  if (!attr_set[dev]) {
+    const cudaError_t e = one_cta_per_sm(simt::gemm_f32_few_kernel<EPI, NQ>, sizeof(float) * simt::F_TOK * (64 * NQ + simt::F_PARTS * simt::F_FEAT));
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = true;
+  }
+  return launch_k(simt::gemm_f32_few_kernel<EPI, NQ>, dim3(p.N / simt::F_FEAT), dim3(256), 0, st, (const float*)W.ptr, (const float*)x, p);
+}
 template <int EPI>
 cudaError_t launch_simt_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p) {
-  const dim3 grid(p.N / simt::F_FEAT), block(256);
-  const float *w = (const float*)W.ptr, *xp = (const float*)x;
   switch (p.K / 64) {
-    case 1: return launch_k(simt::gemm_f32_few_kernel<EPI, 1>, grid, block, 0, st, w, xp, p);
-    case 2: return launch_k(simt::gemm_f32_few_kernel<EPI, 2>, grid, block, 0, st, w, xp, p);
-    case 3: return launch_k(simt::gemm_f32_few_kernel<EPI, 3>, grid, block, 0, st, w, xp, p);
-    case 4: return launch_k(simt::gemm_f32_few_kernel<EPI, 4>, grid, block, 0, st, w, xp, p);
-    case 5: return launch_k(simt::gemm_f32_few_kernel<EPI, 5>, grid, block, 0, st, w, xp, p);
-    case 6: return launch_k(simt::gemm_f32_few_kernel<EPI, 6>, grid, block, 0, st, w, xp, p);
-    case 7: return launch_k(simt::gemm_f32_few_kernel<EPI, 7>, grid, block, 0, st, w, xp, p);
-    default: return launch_k(simt::gemm_f32_few_kernel<EPI, 8>, grid, block, 0, st, w, xp, p);
+    case 1: return launch_simt_few_n<EPI, 1>(st, W, x, p);
+    case 2: return launch_simt_few_n<EPI, 2>(st, W, x, p);
+    case 3: return launch_simt_few_n<EPI, 3>(st, W, x, p);
+    case 4: return launch_simt_few_n<EPI, 4>(st, W, x, p);
+    case 5: return launch_simt_few_n<EPI, 5>(st, W, x, p);
+    case 6: return launch_simt_few_n<EPI, 6>(st, W, x, p);
+    case 7: return launch_simt_few_n<EPI, 7>(st, W, x, p);
+    default: return launch_simt_few_n<EPI, 8>(st, W, x, p);
   }
 }
 
@@ -772,6 +788,10 @@ cudaError_t launch_attention(dim3 grid, dim3 block, cudaStream_t st, const AttnP
   const int dev = current_device();
   if (!attr_set[dev] && smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(attention_kernel<T, D, Q, FUSE, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+  }
+  if (!attr_set[dev] && std::is_same<T, float>::value && Q == 1) {
+    const cudaError_t e = one_cta_per_sm(attention_kernel<T, D, Q, FUSE, MINB>, smem + sizeof(bf16) * ATT_WARPS * 96);
     if (e != cudaSuccess) return e;
   }
   attr_set[dev] = true;
