@@ -923,8 +923,9 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   cudaError_t e = cudaSuccess;
   if (!attr_set[dev]) {
     const int most = (int)few::att_few_smem(few::MAX_WARPS, few::MAX_ROUNDS);
-    for (auto* kernel : {few::attention_few_kernel<false, 1>, few::attention_few_kernel<true, 1>, few::attention_few_kernel<false, 2>,
-                         few::attention_few_kernel<true, 2>})
+    for (auto* kernel : {few::attention_few_kernel<false, 1, false>, few::attention_few_kernel<true, 1, false>, few::attention_few_kernel<false, 2, false>,
+                         few::attention_few_kernel<true, 2, false>, few::attention_few_kernel<false, 1, true>, few::attention_few_kernel<true, 1, true>,
+                         few::attention_few_kernel<false, 2, true>, few::attention_few_kernel<true, 2, true>})
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention attribute: ") + cudaGetErrorString(e));
     attr_set[dev] = true;
@@ -945,8 +946,12 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
     attr[n_attr].val.clusterDim.x = split; attr[n_attr].val.clusterDim.y = 1; attr[n_attr++].val.clusterDim.z = 1;
   }
   cfg.attrs = attr; cfg.numAttrs = n_attr;
-  auto* kernel = split == 1 ? (wq ? few::attention_few_kernel<true, 1> : few::attention_few_kernel<false, 1>)
-                            : (wq ? few::attention_few_kernel<true, 2> : few::attention_few_kernel<false, 2>);
+  auto pick = [&](auto scores_first) {
+    constexpr bool F = decltype(scores_first)::value;
+    return split == 1 ? (wq ? few::attention_few_kernel<true, 1, F> : few::attention_few_kernel<false, 1, F>)
+                      : (wq ? few::attention_few_kernel<true, 2, F> : few::attention_few_kernel<false, 2, F>);
+  };
+  auto* kernel = fp.rounds > 2 ? pick(std::true_type()) : pick(std::false_type());
   e = cudaLaunchKernelEx(&cfg, kernel, fp);
   if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
   return AD_OK;

@@ -67,7 +67,9 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
 
 // grid = (B * qchunks * SPLIT, H), qchunks = ceil(longest segment / 16); block = 32 * att_few_warps(d) threads; dynamic smem
 // att_few_smem; cluster (SPLIT, 1, 1) when QPROJ and SPLIT == 2.
-template <bool QPROJ, int SPLIT>
+// SCORES_FIRST: three or four rounds of keys.  Whole calls, round after round -> this: 512 wide, batch 8 with drafter, 400 keys 7858 -> 7780 us;
+// 768 wide, batch 4, 300 keys 2478 -> 2460.  With one or two rounds it is slower (batch 1 1132 -> 1139, 768 wide, batch 3, 150 keys 2250 -> 2275).
+template <bool QPROJ, int SPLIT, bool SCORES_FIRST>
 __global__ void __launch_bounds__(32 * MAX_WARPS, 1)
 attention_few_kernel(const FewAttnParams fp) {
   const AttnParams& p = fp.a;
@@ -229,58 +231,119 @@ attention_few_kernel(const FewAttnParams fp) {
   float mx0 = -INFINITY, mx1 = -INFINITY, den0 = 0.f, den1 = 0.f;      // den: this lane's share of the row sums
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncwarp();
-  for (int key0 = warp * AK; key0 < row_nk; key0 += AK * nw, ks += round_stride, vs += round_stride) {
-    float s[2][4];
-#pragma unroll
-    for (int n = 0; n < 2; ++n) { s[n][0] = 0.f; s[n][1] = 0.f; s[n][2] = 0.f; s[n][3] = 0.f; }
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const uint4 k0 = *reinterpret_cast<const uint4*>(ks + g * K_LD + 32 * c + 8 * t);
-      const uint4 k1 = *reinterpret_cast<const uint4*>(ks + (g + 8) * K_LD + 32 * c + 8 * t);
-      mma16816(s[0], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, k0.x, k0.y);
-      mma16816(s[1], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, k1.x, k1.y);
-      mma16816(s[0], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, k0.z, k0.w);
-      mma16816(s[1], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, k1.z, k1.w);
-    }
-    // element e of group n: key key0 + 8 n + 2 t + (e & 1), query row g + 8 (e >> 1)
+  if (SCORES_FIRST) {
+    // scores of all rounds first: their MMAs do not depend on one another, and the maximum is known before the first exponential
+    float s[MAX_ROUNDS][2][4];
     float t0 = -INFINITY, t1 = -INFINITY;
 #pragma unroll
-    for (int n = 0; n < 2; ++n) {
-      const int j = key0 + 8 * n + 2 * t;
-      s[n][0] = j < nk0 ? s[n][0] * p.scale : -INFINITY;
-      s[n][1] = j + 1 < nk0 ? s[n][1] * p.scale : -INFINITY;
-      s[n][2] = j < nk1 ? s[n][2] * p.scale : -INFINITY;
-      s[n][3] = j + 1 < nk1 ? s[n][3] * p.scale : -INFINITY;
-      t0 = fmaxf(t0, fmaxf(s[n][0], s[n][1]));
-      t1 = fmaxf(t1, fmaxf(s[n][2], s[n][3]));
+    for (int r = 0; r < MAX_ROUNDS; ++r) {
+      const int key0 = (r * nw + warp) * AK;
+      if (key0 >= row_nk) break;
+      const bf16* kr = ks + r * round_stride;
+#pragma unroll
+      for (int n = 0; n < 2; ++n) { s[r][n][0] = 0.f; s[r][n][1] = 0.f; s[r][n][2] = 0.f; s[r][n][3] = 0.f; }
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const uint4 k0 = *reinterpret_cast<const uint4*>(kr + g * K_LD + 32 * c + 8 * t);
+        const uint4 k1 = *reinterpret_cast<const uint4*>(kr + (g + 8) * K_LD + 32 * c + 8 * t);
+        mma16816(s[r][0], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, k0.x, k0.y);
+        mma16816(s[r][1], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, k1.x, k1.y);
+        mma16816(s[r][0], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, k0.z, k0.w);
+        mma16816(s[r][1], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, k1.z, k1.w);
+      }
+      // element e of group n: key key0 + 8 n + 2 t + (e & 1), query row g + 8 (e >> 1)
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        const int j = key0 + 8 * n + 2 * t;
+        s[r][n][0] = j < nk0 ? s[r][n][0] * p.scale : -INFINITY;
+        s[r][n][1] = j + 1 < nk0 ? s[r][n][1] * p.scale : -INFINITY;
+        s[r][n][2] = j < nk1 ? s[r][n][2] * p.scale : -INFINITY;
+        s[r][n][3] = j + 1 < nk1 ? s[r][n][3] * p.scale : -INFINITY;
+        t0 = fmaxf(t0, fmaxf(s[r][n][0], s[r][n][1]));
+        t1 = fmaxf(t1, fmaxf(s[r][n][2], s[r][n][3]));
+      }
     }
     t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 1)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 1));
     t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 2)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 2));
-    const bool on0 = nk0 > key0, on1 = nk1 > key0;                     // otherwise the query sees none of these keys
-    const float n0 = on0 ? fmaxf(mx0, t0) : mx0, n1 = on1 ? fmaxf(mx1, t1) : mx1;
-    const float c0 = on0 ? expf(mx0 - n0) : 1.f, c1 = on1 ? expf(mx1 - n1) : 1.f;     // exp(-inf) = 0 at first
-    mx0 = n0; mx1 = n1;
-    uint32_t hi[4], lo[4];
-    float sum0 = 0.f, sum1 = 0.f;
+    const bool on0 = nk0 > warp * AK, on1 = nk1 > warp * AK;             // otherwise the query sees none of this warp's keys
+    if (on0) mx0 = t0;
+    if (on1) mx1 = t1;
 #pragma unroll
-    for (int n = 0; n < 2; ++n) {
-      const float p0 = on0 ? expf(s[n][0] - n0) : 0.f, p1 = on0 ? expf(s[n][1] - n0) : 0.f;
-      const float p2 = on1 ? expf(s[n][2] - n1) : 0.f, p3 = on1 ? expf(s[n][3] - n1) : 0.f;
-      sum0 += p0 + p1; sum1 += p2 + p3;
-      split2(p0, p1, hi[2 * n], lo[2 * n]);
-      split2(p2, p3, hi[2 * n + 1], lo[2 * n + 1]);
+    for (int r = 0; r < MAX_ROUNDS; ++r) {
+      if ((r * nw + warp) * AK >= row_nk) break;
+      const bf16* vr = vs + r * round_stride;
+      uint32_t hi[4], lo[4];
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        const float p0 = on0 ? expf(s[r][n][0] - mx0) : 0.f, p1 = on0 ? expf(s[r][n][1] - mx0) : 0.f;
+        const float p2 = on1 ? expf(s[r][n][2] - mx1) : 0.f, p3 = on1 ? expf(s[r][n][3] - mx1) : 0.f;
+        den0 += p0 + p1; den1 += p2 + p3;
+        split2(p0, p1, hi[2 * n], lo[2 * n]);
+        split2(p2, p3, hi[2 * n + 1], lo[2 * n + 1]);
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        uint32_t v0, v1;
+        const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(vr + (lane & 15) * V_LD + 8 * j));
+        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(addr));
+        mma16816(o[j], hi[0], hi[1], hi[2], hi[3], v0, v1);
+        mma16816(o[j], lo[0], lo[1], lo[2], lo[3], v0, v1);
+      }
     }
-    den0 = den0 * c0 + sum0;
-    den1 = den1 * c1 + sum1;
+  } else {
+    for (int key0 = warp * AK; key0 < row_nk; key0 += AK * nw, ks += round_stride, vs += round_stride) {
+      float s[2][4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) { o[j][0] *= c0; o[j][1] *= c0; o[j][2] *= c1; o[j][3] *= c1; }
+      for (int n = 0; n < 2; ++n) { s[n][0] = 0.f; s[n][1] = 0.f; s[n][2] = 0.f; s[n][3] = 0.f; }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      uint32_t v0, v1;
-      const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(vs + (lane & 15) * V_LD + 8 * j));
-      asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(addr));
-      mma16816(o[j], hi[0], hi[1], hi[2], hi[3], v0, v1);
-      mma16816(o[j], lo[0], lo[1], lo[2], lo[3], v0, v1);
+      for (int c = 0; c < 2; ++c) {
+        const uint4 k0 = *reinterpret_cast<const uint4*>(ks + g * K_LD + 32 * c + 8 * t);
+        const uint4 k1 = *reinterpret_cast<const uint4*>(ks + (g + 8) * K_LD + 32 * c + 8 * t);
+        mma16816(s[0], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, k0.x, k0.y);
+        mma16816(s[1], qa[c][0].x, qa[c][1].x, qa[c][0].y, qa[c][1].y, k1.x, k1.y);
+        mma16816(s[0], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, k0.z, k0.w);
+        mma16816(s[1], qa[c][0].z, qa[c][1].z, qa[c][0].w, qa[c][1].w, k1.z, k1.w);
+      }
+      // element e of group n: key key0 + 8 n + 2 t + (e & 1), query row g + 8 (e >> 1)
+      float t0 = -INFINITY, t1 = -INFINITY;
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        const int j = key0 + 8 * n + 2 * t;
+        s[n][0] = j < nk0 ? s[n][0] * p.scale : -INFINITY;
+        s[n][1] = j + 1 < nk0 ? s[n][1] * p.scale : -INFINITY;
+        s[n][2] = j < nk1 ? s[n][2] * p.scale : -INFINITY;
+        s[n][3] = j + 1 < nk1 ? s[n][3] * p.scale : -INFINITY;
+        t0 = fmaxf(t0, fmaxf(s[n][0], s[n][1]));
+        t1 = fmaxf(t1, fmaxf(s[n][2], s[n][3]));
+      }
+      t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 1)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 1));
+      t0 = fmaxf(t0, __shfl_xor_sync(0xffffffffu, t0, 2)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 2));
+      const bool on0 = nk0 > key0, on1 = nk1 > key0;                     // otherwise the query sees none of these keys
+      const float n0 = on0 ? fmaxf(mx0, t0) : mx0, n1 = on1 ? fmaxf(mx1, t1) : mx1;
+      const float c0 = on0 ? expf(mx0 - n0) : 1.f, c1 = on1 ? expf(mx1 - n1) : 1.f;     // exp(-inf) = 0 at first
+      mx0 = n0; mx1 = n1;
+      uint32_t hi[4], lo[4];
+      float sum0 = 0.f, sum1 = 0.f;
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        const float p0 = on0 ? expf(s[n][0] - n0) : 0.f, p1 = on0 ? expf(s[n][1] - n0) : 0.f;
+        const float p2 = on1 ? expf(s[n][2] - n1) : 0.f, p3 = on1 ? expf(s[n][3] - n1) : 0.f;
+        sum0 += p0 + p1; sum1 += p2 + p3;
+        split2(p0, p1, hi[2 * n], lo[2 * n]);
+        split2(p2, p3, hi[2 * n + 1], lo[2 * n + 1]);
+      }
+      den0 = den0 * c0 + sum0;
+      den1 = den1 * c1 + sum1;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { o[j][0] *= c0; o[j][1] *= c0; o[j][2] *= c1; o[j][3] *= c1; }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        uint32_t v0, v1;
+        const uint32_t addr = static_cast<uint32_t>(__cvta_generic_to_shared(vs + (lane & 15) * V_LD + 8 * j));
+        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(addr));
+        mma16816(o[j], hi[0], hi[1], hi[2], hi[3], v0, v1);
+        mma16816(o[j], lo[0], lo[1], lo[2], lo[3], v0, v1);
+      }
     }
   }
   // merge the warps that had keys

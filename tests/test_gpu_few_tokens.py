@@ -82,3 +82,21 @@ def test_loop_planned_by_the_accept_kernel_equals_one_kernel_per_plan(mode, run_
             results.append(([list(map(int, o)) for o in out], st["iterations"], st["row_iterations"], st["accepted"], st["offered"]))
         dec.close()
     assert all(x == results[0] for x in results[1:])
+
+
+@pytest.mark.parametrize("d,batch,k,src", [(256, 2, 17, 129), (256, 1, 5, 192), (512, 1, 16, 257), (512, 2, 9, 400), (768, 1, 17, 200), (1024, 1, 3, 512)])
+def test_source_keys_in_three_and_four_rounds(d, batch, k, src):
+    """Cross-attention over so many keys that a warp has three or four rounds of them: first and last key count of a round, ragged rows of
+    which one ends in the first round."""
+    from paper_2205_10350_b200 import binding
+    shape = synth.ModelShape(f"rounds_{d}", d, d // 64, 512, 1003, 1, 1, "bf16")
+    w = synth.make_weights(shape, 0)
+    model = O.Model(shape, w, max_pos=512)
+    r = np.random.default_rng(d + src)
+    lens = np.array([src, 7][:batch], np.int32)
+    srcs = r.integers(4, shape.vocab, size=(batch, src)).astype(np.int32)
+    dec = binding.AggressiveDecoder(shape, w, max_batch=batch, max_src=src, max_tgt=k, kmax=k)
+    streams = [r.integers(4, shape.vocab, size=k).astype(np.int32) for _ in range(batch)]
+    stats = lockstep(dec, model, srcs, lens, streams, k, [k] * batch, tol=5e-2, max_steps=3)
+    assert stats["steps"] > 0
+    dec.close()
