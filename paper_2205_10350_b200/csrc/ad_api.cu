@@ -814,10 +814,17 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   p.scale = 1.0f / sqrtf((float)dh);
   // Tensor-core kernels when there are thousands of queries or rows may hold hundreds of keys (max_keys: the capacity, known on
   // the host); the FFMA kernel spreads few queries and few keys over more CTAs.
-  // An encoder's rows are all queries: 512 wide, batch 2, 200 tokens 765 us a call with the FFMA kernel, 608 with the MMA one; batch 3, 128
-  // tokens 780 -> 692; 768 wide, batch 2, 90 tokens 767 -> 725.
-  const bool encode = &pc == &h->pass[PK_ENCODE];
-  if (h->bf16 && dh == 64 && (many || encode || max_keys >= 256) && (encode || !(max_keys >= 256 && pc.seg_max <= 128))) {
+  // An encoder's rows are all queries: between the two it keeps the FFMA kernel, which has the output projection in it, only for rows of one
+  // key tile in at most one and a half waves of its CTAs (two for rows of at most eight, half of an MMA tile).  Calls of four layers, FFMA -> MMA, us:
+  // 768 wide 8 x 8 tokens 113 -> 120, 2 x 64 171 -> 176, 4 x 17 127 -> 138, but 4 x 48 153 -> 146, 2 x 90 171 -> 147, 1 x 200 274 -> 173; 1024 wide
+  // 3 x 50 215 -> 184, 1 x 150 273 -> 190; 512 wide 5 x 81 190 -> 146, 16 x 17 143 -> 128, 32 x 8 125 -> 129.
+  const long ffma_ctas = (long)h->dims.B * ((pc.seg_max + 7) / 8) * c.n_heads;
+  const bool encode_mma = &pc == &h->pass[PK_ENCODE] && (pc.seg_max > ATT_KT || 2 * ffma_ctas > (pc.seg_max <= 8 ? 4 : 3) * (long)num_sms());
+  if (h->bf16 && dh == 64 && (many || encode_mma || max_keys >= 256) && !(max_keys >= 256 && pc.seg_max <= 128)) {
+    // What the FFMA kernel would do with FP32 probabilities keeps them (two BF16 numbers each; 0 to 5 us of such a call more than with one):
+    // memory of one layer dominated by its attention, 27 sizes of 256 to 1024 wide: error against 64 bits within 0.03 % of the FFMA kernel's,
+    // 0.3 to 1.8 % above it with probabilities rounded to BF16.
+    const bool split_p = !many && max_keys < 256;
     // Warps share a 16-query tile and split the keys (2 or 4 key groups) when rows have few queries; two groups also while
     // 64-query CTAs would not give every SM two.
     const long full = (long)h->dims.B * ((pc.seg_max + AM_Q - 1) / AM_Q) * c.n_heads;
@@ -826,7 +833,11 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
     p.qchunks = (pc.seg_max + qcta - 1) / qcta;
     note_launch(h, "attention_mma");
     const dim3 mgrid(h->dims.B * p.qchunks, c.n_heads);
-    auto* kernel = ng == 4 ? attention_mma_kernel<4> : (ng == 2 ? attention_mma_kernel<2> : attention_mma_kernel<1>);
+    auto pick = [&](auto split) {
+      constexpr bool S = decltype(split)::value;
+      return ng == 4 ? attention_mma_kernel<4, S> : (ng == 2 ? attention_mma_kernel<2, S> : attention_mma_kernel<1, S>);
+    };
+    auto* kernel = split_p ? pick(std::true_type()) : pick(std::false_type());
     const cudaError_t em = launch_k(kernel, mgrid, dim3(128), 0, h->stream, p, kv_old ? 1 : 0);
     if (em != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(em));
     return AD_OK;
@@ -886,13 +897,15 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
 // of its warps, and a grid of a few waves at most.  The grid counts what the pass could hold; CTAs of rows that have ended, of
 // blocks that are shorter and of a drafter's prefix that has not grown leave at once.  A wave costs 4 to 7 us, the projections that
 // are kernels of their own otherwise 12 us a layer, so a verification pass may need three waves at capacity, a drafter's pass
-// (on average half of its capacity) four; an encoder's rows are as long as they are announced, and there is one projection to gain:
-// one and a half (batch 5, 75 tokens, 12 layers: 742 us a call, 764 with the MMA kernel and a projection behind it), beyond 512 wide one
-// (768 wide, batch 2, 90 tokens: 757 us with two, 725 with the MMA kernel).  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30: 214 -> 174 us; batch 24, 12:
-// 237 -> 196; batch 20, 1: 188 -> 160; batch of 5 with drafter 442 -> 373; 1024 wide, batch 2, 40: 272 -> 226; batch 3 with drafter
-// 662 -> 600.  Beyond: base batch 32 x 64 (seven waves) 270 -> 315, 1024 wide batch 16 x 1 (four) 239 -> 284.  Wide models with fewer than eight
-// queries a row stay at one wave: their CTAs read two weight slices each for a tile that is mostly padding (768 wide, batch 12, 1: 202
-// against 210).
+// (on average half of its capacity) four.  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30:
+// 214 -> 174 us; batch 24, 12: 237 -> 196; batch 20, 1: 188 -> 160; batch of 5 with drafter 442 -> 373; 1024 wide, batch 2, 40: 272 -> 226;
+// batch 3 with drafter 662 -> 600.  Beyond: base batch 32 x 64 (seven waves) 270 -> 315, 1024 wide batch 16 x 1 (four) 239 -> 284.  Wide
+// models with fewer than eight queries a row stay at one wave: their CTAs read two weight slices each for a tile that is mostly padding
+// (768 wide, batch 12, 1: 202 against 210).
+// An encoder's rows are as long as they are announced, and there is one projection to gain: one and a half.  Calls of four layers, 512 wide,
+// kernel without it -> with it, us: 3 x 112 tokens 143 -> 137, 4 x 96 143 -> 134, 5 x 75 144 -> 137, 8 x 48 140 -> 132, 24 x 16 139 -> 131.  One wave
+// beyond 512 wide (768 wide 2 x 90 147 -> 156, 3 x 64 147 -> 152), for rows of at most eight (512 wide 24 x 8 116 -> 118, 24 x 4 122 -> 125; 256 wide
+// the CTAs are small and gain: 40 x 8 111 -> 105) and with 256 keys or more (1 x 304 140 -> 147).
 bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   const ad_model_cfg& c = h->cfg;
   const PassCfg& pc = h->pass[pk];
@@ -900,7 +913,8 @@ bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   const int split = few::att_few_split(c.d_model);
   if (max_keys > few::MAX_ROUNDS * few::AK * few::att_few_warps(c.d_model)) return false;
   // (in half waves)
-  const int waves = pk == PK_ENCODE ? (split > 1 ? 2 : 3) : split > 1 && pc.seg_max < 8 ? 2 : pk == PK_DRAFT ? 8 : 6;
+  const bool one_wave = pk == PK_ENCODE ? split > 1 || max_keys >= 256 || (pc.seg_max <= 8 && c.d_model > 256) : split > 1 && pc.seg_max < 8;
+  const int waves = one_wave ? 2 : pk == PK_ENCODE ? 3 : pk == PK_DRAFT ? 8 : 6;
   return 2L * c.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * split <= (long)waves * num_sms();
 }
 

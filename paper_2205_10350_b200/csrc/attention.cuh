@@ -49,6 +49,14 @@ __device__ __forceinline__ void att_mma_bf16(float (&c)[4], uint32_t a0, uint32_
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
+// (hi, lo) BF16 pairs of two non-negative numbers: hi = bf16(v), lo = bf16(v - hi)
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(a - __low2float(h), b - __high2float(h));
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
 // Eight consecutive elements (16-byte aligned for bf16, 32-byte for float) as floats.
 __device__ __forceinline__ void load8(const bf16* p, float* out) {
   const uint4 u = *reinterpret_cast<const uint4*>(p);

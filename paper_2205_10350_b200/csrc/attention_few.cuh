@@ -58,12 +58,6 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
 }
-// (hi, lo) BF16 pairs of two non-negative numbers: hi = bf16(v), lo = bf16(v - hi)
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  hi = *reinterpret_cast<const uint32_t*>(&h);
-  lo = pack2(a - __low2float(h), b - __high2float(h));
-}
 
 // grid = (B * qchunks * SPLIT, H), qchunks = ceil(longest segment / 16); block = 32 * att_few_warps(d) threads; dynamic smem
 // att_few_smem; cluster (SPLIT, 1, 1) when QPROJ and SPLIT == 2.

@@ -3,8 +3,8 @@
 // Same operation and masking rules as attention_kernel (attention.cuh).  The tiles of one (row, head) pair are small (at most
 // 64 queries x 64 keys x 64 dims per step), far below the 128-row atoms of the tcgen05 path and not worth a round trip through
 // tensor memory, so the products run as warp-level m16n8k16 MMAs on register fragments: S = Q K^T, online softmax on the
-// accumulator fragments, P (rounded to BF16) reused in place as the A operand of O += P V, with V read through transposing
-// ldmatrix loads.  Key fragments are read 16 bytes at a time, the contraction index permuted identically for both operands
+// accumulator fragments, P (rounded to BF16, or as a sum of two BF16 numbers) reused in place as the A operand of O += P V, with V
+// read through transposing ldmatrix loads.  Key fragments are read 16 bytes at a time, the contraction index permuted identically for both operands
 // (see gemm_few.cuh).  Keys and values that are older than the plan (cross-attention: the encoder wrote them) are requested
 // before the dependency wait.
 #pragma once
@@ -27,6 +27,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);   // .x = lo (low half), .y = hi
   return *reinterpret_cast<uint32_t*>(&h);
 }
+template <bool SPLIT_P>
+__device__ __forceinline__ float exp_p(float x) { return SPLIT_P ? expf(x) : __expf(x); }
 // K/V tiles in shared memory.
 constexpr int AL_KLD = 96;             // key rows 192 bytes apart: conflict-free 16-byte fragment loads
 constexpr int AL_VLD = 72;             // value rows 144 bytes apart: conflict-free ldmatrix
@@ -64,7 +66,8 @@ __device__ __forceinline__ void attn_init(AttnState& a) {
   a.den0 = a.den1 = 0.f;
 }
 // KS keys (rows of ks / vs; the first is key jw of the row) for 16 queries whose two of this lane see nk0 / nk1 keys.
-template <int KS>
+// SPLIT_P: probabilities from expf, multiplied as a sum of two BF16 numbers; otherwise from __expf, rounded to BF16.
+template <int KS, bool SPLIT_P>
 __device__ __forceinline__ void attn_keys(AttnState& a, const uint4 (&qa)[2][2], const bf16* ks, const bf16* vs, int jw, int nk0, int nk1,
                                           float scale, int lane) {
   const int g = lane >> 2, tq = lane & 3;
@@ -106,19 +109,25 @@ __device__ __forceinline__ void attn_keys(AttnState& a, const uint4 (&qa)[2][2],
   t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 1)); t1 = fmaxf(t1, __shfl_xor_sync(0xffffffffu, t1, 2));
   const bool on0 = nk0 > jw, on1 = nk1 > jw;         // otherwise none of these keys is visible to the query
   const float m0n = on0 ? fmaxf(a.mx0, t0) : a.mx0, m1n = on1 ? fmaxf(a.mx1, t1) : a.mx1;
-  const float corr0 = on0 ? __expf(a.mx0 - m0n) : 1.f, corr1 = on1 ? __expf(a.mx1 - m1n) : 1.f;   // exp(-inf) = 0 at first
+  const float corr0 = on0 ? exp_p<SPLIT_P>(a.mx0 - m0n) : 1.f, corr1 = on1 ? exp_p<SPLIT_P>(a.mx1 - m1n) : 1.f;   // exp(-inf) = 0 at first
   a.mx0 = m0n; a.mx1 = m1n;
   const float e0 = on0 ? m0n : 0.f, e1 = on1 ? m1n : 0.f;           // (all scores are -inf when the query sees no key here)
   float sum0 = 0.f, sum1 = 0.f;
-  uint32_t pa[KS / 16][4];
+  uint32_t pa[KS / 16][4], pl[SPLIT_P ? KS / 16 : 1][4];
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt) {
-    const float p0 = __expf(s[nt][0] - e0), p1 = __expf(s[nt][1] - e0);
-    const float p2 = __expf(s[nt][2] - e1), p3 = __expf(s[nt][3] - e1);
+    const float p0 = exp_p<SPLIT_P>(s[nt][0] - e0), p1 = exp_p<SPLIT_P>(s[nt][1] - e0);
+    const float p2 = exp_p<SPLIT_P>(s[nt][2] - e1), p3 = exp_p<SPLIT_P>(s[nt][3] - e1);
     sum0 += p0 + p1; sum1 += p2 + p3;
     // accumulator fragments of two neighbouring key groups are exactly one A fragment of 16 keys
-    pa[nt >> 1][(nt & 1) * 2 + 0] = pack_bf16(p0, p1);
-    pa[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
+    const int i = (nt & 1) * 2;
+    if (SPLIT_P) {
+      split2(p0, p1, pa[nt >> 1][i], pl[SPLIT_P ? nt >> 1 : 0][i]);
+      split2(p2, p3, pa[nt >> 1][i + 1], pl[SPLIT_P ? nt >> 1 : 0][i + 1]);
+    } else {
+      pa[nt >> 1][i] = pack_bf16(p0, p1);
+      pa[nt >> 1][i + 1] = pack_bf16(p2, p3);
+    }
   }
   a.den0 = a.den0 * corr0 + sum0;
   a.den1 = a.den1 * corr1 + sum1;
@@ -133,6 +142,10 @@ __device__ __forceinline__ void attn_keys(AttnState& a, const uint4 (&qa)[2][2],
       asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(v0), "=r"(v1), "=r"(v2), "=r"(v3) : "r"(addr));
       mma_bf16_16816(a.o[dt], pa[tt], v0, v1);
       mma_bf16_16816(a.o[dt + 1], pa[tt], v2, v3);
+      if (SPLIT_P) {
+        mma_bf16_16816(a.o[dt], pl[SPLIT_P ? tt : 0], v0, v1);
+        mma_bf16_16816(a.o[dt + 1], pl[SPLIT_P ? tt : 0], v2, v3);
+      }
     }
   }
 }
@@ -143,7 +156,7 @@ __device__ __forceinline__ void attn_keys(AttnState& a, const uint4 (&qa)[2][2],
 // leave SMs idle, NG = 2 or 4 warps share a 16-query tile instead (32 or 16 queries per CTA) and split the keys of every tile
 // between them; their running maxima, sums and outputs are merged at the end.
 // grid = (B * qchunks, H), qchunks = ceil(longest segment / queries per CTA); block = 128 threads.
-template <int NG>
+template <int NG, bool SPLIT_P>
 __global__ void __launch_bounds__(128, 3)
 attention_mma_kernel(const AttnParams p, const int kv_old) {
   constexpr int DH = 64;
@@ -228,7 +241,7 @@ attention_mma_kernel(const AttnParams p, const int kv_old) {
     __syncthreads();                                 // everybody's copies of tile t have landed
     const int jw = t * AM_KT + grp * KS;             // first key of this warp's share of the tile
     const bf16* ks = reinterpret_cast<const bf16*>(kv[t & 1]);
-    if (active && jw < row_nk) attn_keys<KS>(a, qa, ks + grp * KS * AL_KLD, ks + AM_KT * AL_KLD + grp * KS * AL_VLD, jw, nk0, nk1, p.scale, lane);
+    if (active && jw < row_nk) attn_keys<KS, SPLIT_P>(a, qa, ks + grp * KS * AL_KLD, ks + AM_KT * AL_KLD + grp * KS * AL_VLD, jw, nk0, nk1, p.scale, lane);
     __syncthreads();                                 // tile t is fully consumed
     fetch(t + 2);
   }
@@ -260,8 +273,8 @@ attention_mma_kernel(const AttnParams p, const int kv_old) {
       const float om0 = rec[32 * 128 + src], om1 = rec[33 * 128 + src];
       const float n0 = fmaxf(mx0, om0), n1 = fmaxf(mx1, om1);
       // a row that saw no key at all keeps maximum -inf on both sides: factors 0, nothing to add
-      const float a0 = n0 == -INFINITY ? 0.f : __expf(mx0 - n0), b0 = n0 == -INFINITY ? 0.f : __expf(om0 - n0);
-      const float a1 = n1 == -INFINITY ? 0.f : __expf(mx1 - n1), b1 = n1 == -INFINITY ? 0.f : __expf(om1 - n1);
+      const float a0 = n0 == -INFINITY ? 0.f : exp_p<SPLIT_P>(mx0 - n0), b0 = n0 == -INFINITY ? 0.f : exp_p<SPLIT_P>(om0 - n0);
+      const float a1 = n1 == -INFINITY ? 0.f : exp_p<SPLIT_P>(mx1 - n1), b1 = n1 == -INFINITY ? 0.f : exp_p<SPLIT_P>(om1 - n1);
       den0 = den0 * a0 + rec[34 * 128 + src] * b0;
       den1 = den1 * a1 + rec[35 * 128 + src] * b1;
 #pragma unroll
@@ -417,7 +430,7 @@ attention_long_kernel(const AttnParams p, const int slots, const int kv_old) {
     for (int tl = kw; active && tl < min(slots, n_tiles - first); tl += NW) {
       const int jw = (first + tl) * AM_KT;           // first key of this tile
       const bf16* ks = reinterpret_cast<const bf16*>(am_smem + (size_t)tl * AL_TILE_BYTES);
-      attn_keys<AM_KT>(a, qa, ks, ks + AM_KT * AL_KLD, jw, nk0, nk1, p.scale, lane);
+      attn_keys<AM_KT, false>(a, qa, ks, ks + AM_KT * AL_KLD, jw, nk0, nk1, p.scale, lane);
     }
   }
 
