@@ -591,7 +591,7 @@ cudaError_t launch_vocab_persistent(cudaStream_t st, const CUtensorMap& mw64, co
 
 // Projection of a pass with few tokens (gemm_few.cuh).  ksplit: few::split_for of the shape, non-zero.
 template <int EPI, bool EMB = false>
-cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p, int ksplit, const few::EmbedParams& ep = {}) {
+cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p, int ksplit, bool decoder, const few::EmbedParams& ep = {}) {
   const dim3 grid(p.N / few::FEAT, ksplit);
   const bf16 *w = (const bf16*)W.ptr, *xp = (const bf16*)x;
   const dim3 wgrid(p.N / few::W_FEAT, ksplit);
@@ -611,8 +611,12 @@ cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmP
   switch (p.K / ksplit / 256) {
     case 1: return launch_k(few::gemm_few_kernel<EPI, 1, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
     case 2: return launch_k(few::gemm_few_kernel<EPI, 2, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
-    case 3: return launch_k(few::gemm_few_wide_kernel<EPI, 3, EMB>, wgrid, dim3(few::THREADS), 0, st, w, xp, p, ep);
-    default: return launch_k(few::gemm_few_wide_kernel<EPI, 4, EMB>, wgrid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    case 3:
+      return launch_k(decoder ? few::gemm_few_wide_kernel<EPI, 3, EMB, true> : few::gemm_few_wide_kernel<EPI, 3, EMB, false>, wgrid,
+                      dim3(few::THREADS), 0, st, w, xp, p, ep);
+    default:
+      return launch_k(decoder ? few::gemm_few_wide_kernel<EPI, 4, EMB, true> : few::gemm_few_wide_kernel<EPI, 4, EMB, false>, wgrid,
+                      dim3(few::THREADS), 0, st, w, xp, p, ep);
   }
 }
 
@@ -740,15 +744,17 @@ int gemm(ad_handle* h, int epi, const Mat& W, const ActBuf& X, int pk, const int
   PassCfg& pc = h->pass[pk];
   if (h->bf16) p.rule = geo_rule(pc, epi, W.N, W.K, split, p.bias != nullptr);
   if (h->bf16 && always_few(pc, p.rule)) {
+    const int split = p.rule.few_split;
+    const bool decoder = pk != PK_ENCODE;
     switch (epi) {
-      case EPI_F32: e = launch_few<EPI_F32>(h->stream, W, X.ptr, p, p.rule.few_split); break;
-      case EPI_ACT: e = launch_few<EPI_ACT>(h->stream, W, X.ptr, p, p.rule.few_split); break;
+      case EPI_F32: e = launch_few<EPI_F32>(h->stream, W, X.ptr, p, split, decoder); break;
+      case EPI_ACT: e = launch_few<EPI_ACT>(h->stream, W, X.ptr, p, split, decoder); break;
       default:
         if (embed_of) {
           const few::EmbedParams ep = {(const bf16*)embed_of->emb.ptr, h->pe, sqrtf((float)W.K), pc.plan.tok_id, pc.plan.tok_pos, h->y};
-          e = launch_few<EPI_SCATTER, true>(h->stream, W, X.ptr, p, p.rule.few_split, ep);
+          e = launch_few<EPI_SCATTER, true>(h->stream, W, X.ptr, p, split, decoder, ep);
         } else {
-          e = launch_few<EPI_SCATTER>(h->stream, W, X.ptr, p, p.rule.few_split);
+          e = launch_few<EPI_SCATTER>(h->stream, W, X.ptr, p, split, decoder);
         }
         break;
     }
