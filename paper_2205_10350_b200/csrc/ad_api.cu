@@ -985,6 +985,7 @@ int layernorm(ad_handle* h, const PassCfg& pc, const Partials& pre, const float*
   note_launch(h, "residual+layernorm");
   // P, the partial sums in flight, from the most that any token count of the pass brings (it sets the registers, see layernorm_kernel)
   const int most = pre.nsplit > 0 ? pre.nsplit : cached_shape(h, pre.rule, pc.M_cap).ksplit;
+  if (most > 16) return fail(h, AD_ERR_ARG, "layernorm: more than 16 partial sums");
   auto go_n = [&](auto* yb, auto threads, auto parts) -> cudaError_t {
     using ActT = std::remove_pointer_t<decltype(yb)>;
     constexpr int T = decltype(threads)::value, P = decltype(parts)::value, per_cta = 256 / T;

@@ -404,9 +404,10 @@ __device__ __forceinline__ LnWeights ln_weights(const LnParams& p, int gi) {
   return w;
 }
 
-// Token m by a group of THREADS threads, four features per thread (d <= 4 * THREADS): the residual and P partial sums of a thread are
-// requested at once, so that with P no smaller than their number the kernel costs one memory round trip.  (Two groups of features per
-// thread took 2.8 us instead of 1.5 us per launch on a 1024-wide model with 16 partials.)
+// Token m by a group of THREADS threads, four features per thread (d <= 4 * THREADS): the residual and all partial sums of a thread
+// (P of them at most) are requested at once, so that the kernel costs one memory round trip.  (Two groups of features per thread took
+// 2.8 us instead of 1.5 us per launch on a 1024-wide model with 16 partials; 9 to 16 partials in two turns of eight, with 64
+// registers: whole calls 768 wide +2.5 %, 1024 wide +3 %.)
 template <typename ActT, int THREADS, int P>
 __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, int m, int nsplit, size_t stride, ActT* yb, float* red,
                                          int tid, int half) {
@@ -420,18 +421,11 @@ __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, 
     const size_t step = stride >> 2;               // (stride is a multiple of d, d of 4)
     float4 part[P];
 #pragma unroll
-    for (int sp = 0; sp < P; ++sp) part[sp] = sp < nsplit ? pre[sp * step] : zero4;
+    for (int sp = 0; sp < P; ++sp, pre += step) part[sp] = sp < nsplit ? *pre : zero4;
     const float4 r = p.resid ? reinterpret_cast<const float4*>(p.resid)[off] : zero4;
     v = make_float4(w.c.x + r.x, w.c.y + r.y, w.c.z + r.z, w.c.w + r.w);
 #pragma unroll
     for (int sp = 0; sp < P; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
-#pragma unroll 1
-    for (int s0 = P; s0 < nsplit; s0 += P) {
-#pragma unroll
-      for (int sp = 0; sp < P; ++sp) part[sp] = s0 + sp < nsplit ? pre[(s0 + sp) * step] : zero4;
-#pragma unroll
-      for (int sp = 0; sp < P; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
-    }
   }
   const float mean = group_sum<THREADS>(v.x + v.y + v.z + v.w, red, tid, half) / (float)p.d;
   float vs = 0.f;
@@ -454,8 +448,9 @@ __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, 
 // One CTA per token.  grid = M_cap, block = THREADS (128 for d <= 512, else 256).
 // What bounds it: one memory round trip (1.0-1.3 us), and what it keeps from the projection behind it, whose CTAs (32 K registers and up to
 // 200 KB of shared memory each) want to be on the SM before this kernel's wait is over.  With room for 16 partial sums whatever their number
-// (96 registers) the CTAs of a few hundred tokens filled the register files; now 46, 64 or 96-112 registers for up to 4, 8 or 16.
-// Whole calls: 768 wide, batch 16 5090 -> 4805 us; 512 wide, batch 24 with drafter 6310 -> 6000, batch 32 5385 -> 5170; batch 1 1177 -> 1135.
+// (96 registers) the CTAs of a few hundred tokens filled the register files; now 48 or 64 for up to 4 or 8, 96 only for more (12 and 16
+// heads).  Whole calls: 768 wide, batch 16 5090 -> 4805 us; 512 wide, batch 24 with drafter 6310 -> 6000, batch 32 5385 -> 5170; batch 1
+// 1177 -> 1135.  With a tail loop for sums beyond P, which no pass has, it was 128 registers and 0.3 to 0.6 % of every decode call more.
 template <typename ActT, int THREADS, int P>
 __global__ void __launch_bounds__(THREADS, (P <= 4 ? 1280 : P <= 8 ? 1024 : 512) / THREADS)
 layernorm_kernel(const LnParams p, ActT* __restrict__ yb) {

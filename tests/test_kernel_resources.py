@@ -1,0 +1,34 @@
+"""Registers and spills of the small kernels that a pass runs between its projections, as the compiler reports them.
+
+They are bound by one memory round trip each, and the registers they hold are kept from the projection behind them."""
+import os
+import re
+import subprocess
+
+import pytest
+
+from paper_2205_10350_b200 import build
+
+NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+pytestmark = pytest.mark.skipif(not os.path.exists(NVCC), reason="no CUDA compiler")
+
+
+def _report(tmp_path, kernels):
+    """{kernel's symbol: (registers, bytes spilled)} of the kernels named."""
+    src = tmp_path / "kernels.cu"
+    src.write_text('#include "accept.cuh"\nusing namespace ad;\nvoid* kernels[] = {%s};\n' % ", ".join(f"(void*){k}" for k in kernels))
+    r = subprocess.run([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-rdc=true", "-I", build.CSRC, "-Xptxas", "-v",
+                        "-c", str(src), "-o", str(tmp_path / "kernels.o")], check=True, capture_output=True, text=True)
+    found = re.findall(r"Compiling entry function '(\S+)'.*?(\d+) bytes spill stores.*?Used (\d+) registers", r.stdout + r.stderr, re.S)
+    names = {re.match(r"\w+", k).group() for k in kernels}
+    return {sym: (int(regs), int(spill)) for sym, spill, regs in found if any(re.match(rf"_ZN2ad\d+{n}I", sym) for n in names)}
+
+
+def test_layernorm_holds_what_its_partial_sums_need(tmp_path):
+    limits = {"layernorm_kernel": {4: 48, 8: 64, 16: 96}, "layernorm_many_kernel": {4: 64, 8: 64, 16: 112}}
+    cases = [(n, t, p) for n in limits for t in (128, 256) for p in (4, 8, 16)]
+    found = _report(tmp_path, [f"{n}<{a}, {t}, {p}>" for n, t, p in cases for a in ("bf16", "float")])
+    assert len(found) == 2 * len(cases)
+    for sym, (regs, spill) in found.items():
+        name, p = re.search(r"(layernorm\w*kernel)I.*?Li\d+ELi(\d+)E", sym).groups()
+        assert spill == 0 and regs <= limits[name][int(p)], f"{sym}: {regs} registers, {spill} bytes spilled"
