@@ -469,16 +469,28 @@ bool use_pdl() {
 
 // Launches `kernel` so that it may begin while its predecessor in the stream still runs (the kernels
 // themselves wait with griddepcontrol.wait before touching anything a predecessor writes).
+// shared_share: share of an SM's memory to prefer as shared memory, in percent (negative: the runtime's choice).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+cudaError_t launch_shared(int shared_share, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  int n_attr = 0;
+  if (use_pdl()) {
+    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (shared_share >= 0) {
+    attr[n_attr].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[n_attr++].val.sharedMemCarveout = shared_share;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = use_pdl() ? 1 : 0;
+  cfg.numAttrs = n_attr;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(std::forward<Args>(args))...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_shared(-1, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // Per-device caches (a process may hold handles on several GPUs): SM count, and which kernels already had their
@@ -498,6 +510,10 @@ int num_sms() {
   }
   return n[dev];
 }
+
+// Share of an SM's memory that leaves room for one CTA of smem_bytes and not for two.  Left to itself the runtime makes room for two, and
+// the CTAs of a small grid share SMs while others stand by (weights and activations of both then queue for one L1).
+int one_cta_share(size_t smem_bytes) { return (int)((smem_bytes + 1024) * 100 / (228 * 1024)) + 1; }
 
 // Dynamic shared memory of a pass of M tokens: the ring doubles as the epilogue's transposition buffer (up to 128 rows of 132 floats)
 // and the few-token partial sums.
@@ -595,22 +611,14 @@ cudaError_t launch_few(cudaStream_t st, const Mat& W, const void* x, const GemmP
   const dim3 grid(p.N / few::FEAT, ksplit);
   const bf16 *w = (const bf16*)W.ptr, *xp = (const bf16*)x;
   const dim3 wgrid(p.N / few::W_FEAT, ksplit);
-  // A quarter of the SM's memory as shared memory, enough for one CTA of the 16-feature forms (41 KB each): left to itself the runtime
-  // makes room for two, and the 96 to 128 CTAs of a grid share 64 SMs while others stand by (the weights and activations of both then queue
-  // for one L1).  Whole calls, the runtime's choice -> this: 512 wide, batch 1 1124 -> 1075 us, batch 2 with drafter 4360 -> 3950, batch 8
-  // 3560 -> 3520; 12+2, batch 1 960 -> 906.  43 % (two CTAs fit again): 1120, 4300, 3530, 961.
-  static bool attr_set[kMaxDevices] = {};
-  const int dev = current_device();
-  if (!attr_set[dev]) {
-    for (auto* kernel : {few::gemm_few_kernel<EPI, 1, EMB>, few::gemm_few_kernel<EPI, 2, EMB>}) {
-      const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
-      if (e != cudaSuccess) return e;
-    }
-    attr_set[dev] = true;
-  }
+  // One CTA of the 16-feature forms an SM where there are no more CTAs than SMs.  Whole calls, the runtime's choice -> this: 512 wide,
+  // batch 1 1124 -> 1075 us, batch 2 with drafter 4360 -> 3950, batch 8 3560 -> 3520; 12+2, batch 1 960 -> 906.  Room for two again: 1120,
+  // 4300, 3530, 961.  Larger grids would take turns: encoder calls of four layers, 512 wide, batch 1, 25 tokens: 89.1 us with one CTA an SM
+  // for the 384 CTAs of the cross-attention's keys and values, 87.1 with the runtime's choice; feed-forward width 4096 (256 CTAs) 93.7, 86.7.
+  const int share = (long)grid.x * grid.y <= num_sms() ? one_cta_share(few::red_bytes(2)) : -1;
   switch (p.K / ksplit / 256) {
-    case 1: return launch_k(few::gemm_few_kernel<EPI, 1, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
-    case 2: return launch_k(few::gemm_few_kernel<EPI, 2, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    case 1: return launch_shared(share, few::gemm_few_kernel<EPI, 1, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
+    case 2: return launch_shared(share, few::gemm_few_kernel<EPI, 2, EMB>, grid, dim3(few::THREADS), 0, st, w, xp, p, ep);
     case 3:
       return launch_k(decoder ? few::gemm_few_wide_kernel<EPI, 3, EMB, true> : few::gemm_few_wide_kernel<EPI, 3, EMB, false>, wgrid,
                       dim3(few::THREADS), 0, st, w, xp, p, ep);
@@ -660,23 +668,14 @@ cudaError_t launch_simt(cudaStream_t st, const void* w, const void* x, const Gem
 }
 // The few-token FP32 kernel: passes of at most kFewTokens tokens, shapes it covers.
 bool f32_few(const PassCfg& pc, int epi, int N, int K) { return pc.M_cap <= kFewTokens && epi != EPI_ARGMAX && simt::few_fits(N, K); }
-// Most shared memory that leaves room for one CTA of `kernel` an SM, as the share of the SM's memory to prefer (see launch_few: CTAs of a
-// small grid that share SMs while others stand by).  With both FP32 kernels of a sublayer one an SM, whole calls of the 128-wide model: batch 6
-// 1565 -> 1520 us, batch 2 with drafter 1251 -> 1229, batch 1 551 -> 549.
-template <typename K>
-cudaError_t one_cta_per_sm(K* kernel, size_t smem_bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)((smem_bytes + 1024) * 100 / (228 * 1024)) + 1);
-}
+// The FP32 kernels of a sublayer (this one and the attention with one query per warp) keep to one CTA an SM whatever their grid: where only
+// one of two neighbours does, the change from one share to the other costs more than a second CTA gains.  Whole calls, both at one CTA an
+// SM -> the attention at the runtime's choice once it has more CTAs than SMs: 128 wide, batch 32 2264 -> 2458 us; 256 wide, batch 12
+// 3223 -> 3530; 512 wide, batch 6 3692 -> 3775, 12 4955 -> 5460, 24 6754 -> 6910.
 template <int EPI, int NQ>
 cudaError_t launch_simt_few_n(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p) {
-  static bool attr_set[kMaxDevices] = {};
-  const int dev = current_device();
-  if (!attr_set[dev]) {
-    const cudaError_t e = one_cta_per_sm(simt::gemm_f32_few_kernel<EPI, NQ>, sizeof(float) * simt::F_TOK * (64 * NQ + simt::F_PARTS * simt::F_FEAT));
-    if (e != cudaSuccess) return e;
-    attr_set[dev] = true;
-  }
-  return launch_k(simt::gemm_f32_few_kernel<EPI, NQ>, dim3(p.N / simt::F_FEAT), dim3(256), 0, st, (const float*)W.ptr, (const float*)x, p);
+  const int share = one_cta_share(sizeof(float) * simt::F_TOK * (64 * NQ + simt::F_PARTS * simt::F_FEAT));
+  return launch_shared(share, simt::gemm_f32_few_kernel<EPI, NQ>, dim3(p.N / simt::F_FEAT), dim3(256), 0, st, (const float*)W.ptr, (const float*)x, p);
 }
 template <int EPI>
 cudaError_t launch_simt_few(cudaStream_t st, const Mat& W, const void* x, const GemmParams& p) {
@@ -796,12 +795,9 @@ cudaError_t launch_attention(dim3 grid, dim3 block, cudaStream_t st, const AttnP
     cudaError_t e = cudaFuncSetAttribute(attention_kernel<T, D, Q, FUSE, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  if (!attr_set[dev] && std::is_same<T, float>::value && Q == 1) {
-    const cudaError_t e = one_cta_per_sm(attention_kernel<T, D, Q, FUSE, MINB>, smem + sizeof(bf16) * ATT_WARPS * 96);
-    if (e != cudaSuccess) return e;
-  }
   attr_set[dev] = true;
-  return launch_k(attention_kernel<T, D, Q, FUSE, MINB>, grid, block, smem, st, p);
+  const int share = std::is_same<T, float>::value && Q == 1 ? one_cta_share(smem + sizeof(bf16) * ATT_WARPS * 96) : -1;
+  return launch_shared(share, attention_kernel<T, D, Q, FUSE, MINB>, grid, block, smem, st, p);
 }
 
 int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, const void* v, void* out,
