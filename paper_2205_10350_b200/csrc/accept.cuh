@@ -94,26 +94,31 @@ __device__ __forceinline__ void scan_tiles(const float* __restrict__ val, const 
 //   score strictly higher (Eq. 8: the draft is within the top beta) and the best score exceeds the draft's by at most tau
 //   (Eq. 9; differences of log-likelihoods are differences of scores); otherwise the greedy choice.  beta and tau: st.words.
 // to_drafts: the choices are the row's drafts and nothing is compared.
-// auto_commit (decode loop): n is committed at once (Algorithm 1 lines 6-7); the last CTA to finish updates the loop
-//   counters and the all-finished word (done_ctr: rows done in the low half, active rows in the high half; left at zero) and,
-//   with next.source >= 0, lays out the pass behind this kernel; what concerns one row alone (suffix match, drafts, sizes)
-//   is done by the row's own CTA.
+// auto_commit (decode loop): n is committed at once (Algorithm 1 lines 6-7); what concerns one row alone (suffix match, drafts,
+//   sizes) is done by the row's own CTA.  The loop counters, the all-finished word and, with next.source >= 0, the layout of the
+//   pass behind this kernel need all rows; how these meet is the kernel's form:
+//   ACC_ONE        there is one row;
+//   ACC_CLUSTERED  2 to ACC_CLUSTER rows of a decode loop, as many as the device places as one cluster: each CTA tells the others its next
+//                  block's size through distributed shared memory and lays its own row out, row 0's updates the loop words;
+//   ACC_ROWS       through global memory: the last CTA to finish (done_ctr: rows done in the low half, active rows in the high
+//                  half; left at zero) reads what the others wrote, updates the loop words and lays out all rows (3.3 us and 1.8 us: an
+//                  iteration takes 2.2 us longer than with a cluster with 4 rows, 3 us with 8).
+//   (Calls that commit nothing need no other row and run as one of the first and the last.)
 //
 // What bounds it: a chain of dependent memory round trips, so whatever older kernels wrote (row state, drafts, source) is
 // read before the dependency wait, and from the partials to the next plan everything stays in shared memory: one round trip
 // for the partials (plus the hand-over between CTAs when B > 1).
 // Batch 1, 40-token blocks: 11.4 us with the state, the match and the plan in global memory.
-// CLUSTER (2 to ACC_CLUSTER rows of a decode loop): the rows' CTAs are a cluster; each tells the others its next block's size through
-// distributed shared memory and lays its own row out.  Through global memory (a counter, fences, the last CTA reads what the others wrote
-// and lays out all rows: 3.3 us and 1.8 us) an iteration takes 2.2 us longer with 4 rows, 3 us with 8.  More rows take that way still.
-// grid = B, block = 1024; CLUSTER: cluster (B, 1, 1).
+// grid = B, block = 1024; ACC_CLUSTERED: cluster (B, 1, 1).
 constexpr int ACC_CLUSTER = 16;
-template <bool CLUSTER>
+enum AcceptForm { ACC_ONE, ACC_CLUSTERED, ACC_ROWS };
+template <AcceptForm FORM>
 __global__ void __launch_bounds__(ACC_THREADS)
 argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict__ part_val, const int* __restrict__ part_idx,
                      int n_tiles, int to_drafts, int auto_commit, unsigned int* done_ctr, unsigned long long cond, int relaxed_on,
                      const float* __restrict__ draft_val, const int* __restrict__ draft_id,
                      const int* __restrict__ part_cnt, NextPass next) {
+  constexpr bool CLUSTER = FORM == ACC_CLUSTERED;
   __shared__ int s_dr[256], s_pred[256], s_src[ACC_SRC];
   __shared__ int s_k[256], s_off[256], s_boff[256], s_len[256];
   __shared__ int s_next[256], s_row[CLUSTER ? ACC_CLUSTER : 1];   // the next block's drafts; per row: 1 finished, 2 took part
@@ -130,9 +135,11 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
   const int4 words = __ldcg(reinterpret_cast<const int4*>(st.words));
   const int k_cap = words.x, override_len = words.y, beta = words.z;
   const float tau = __int_as_float(words.w);
-  int it_active = 0, it_all = 0, it_limit = 0, stat_acc = 0, stat_it = 0, stat_off = 0;
-  if (tid == 0) { stat_acc = plan_load(st.stat_acc + b); stat_it = plan_load(st.stat_it + b); stat_off = plan_load(st.stat_off + b); }
-  if (tid == ACC_THREADS - 1 && auto_commit) { it_active = plan_load(st.loop_it); it_all = plan_load(st.loop_it + 2); it_limit = plan_load(st.loop_it + 3); }
+  // the first thread's row counters, the last one's loop counters
+  const bool counts = tid == 0 || (tid == ACC_THREADS - 1 && auto_commit);
+  const int ctr0 = counts ? plan_load(tid == 0 ? st.stat_acc + b : st.loop_it) : 0;
+  const int ctr1 = counts ? plan_load(tid == 0 ? st.stat_it + b : st.loop_it + 2) : 0;
+  const int ctr2 = counts ? plan_load(tid == 0 ? st.stat_off + b : st.loop_it + 3) : 0;
   if (!to_drafts && tid < k) s_dr[tid] = plan_load(st.drafts + (size_t)b * dm.kmax + tid);     // k <= kmax <= 256
   int n_src = 0;
   const int* x = st.src + (size_t)b * dm.max_src;
@@ -222,7 +229,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
     st.n_acc[b] = 0;
     if (n > 0) {
       st.len[b] = len1; st.last[b] = last1; st.fin[b] = fin1;
-      st.stat_acc[b] = stat_acc + n; st.stat_it[b] = stat_it + 1; st.stat_off[b] = stat_off + k;
+      st.stat_acc[b] = ctr0 + n; st.stat_it[b] = ctr1 + 1; st.stat_off[b] = ctr2 + k;
     }
   }
   // ---- this row's next block ----
@@ -277,7 +284,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
   } else {
     __syncthreads();
   }
-  if (!CLUSTER && B > 1) {
+  if (FORM == ACC_ROWS) {
     if (tid == 0) {
       __threadfence();
       const unsigned int t = atomicAdd(done_ctr, n > 0 ? 0x10001u : 1u);
@@ -294,15 +301,15 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
     }
     all_fin = __syncthreads_and(f) != 0;
   }
-  if (tid == ACC_THREADS - 1 && (!CLUSTER || b == 0)) {            // (not a thread of the warp that lays the rows out)
+  if (tid == ACC_THREADS - 1 && (!CLUSTER || b == 0)) {            // (not a thread of the warp that adds up many rows' offsets)
     *done_ctr = 0;
-    if (any_active) *st.loop_it = it_active + 1;
+    if (any_active) *st.loop_it = ctr0 + 1;
     *st.all_fin = all_fin;
     if (cond) {
       // the iteration runs inside a device-side `while` graph node, which repeats while its condition is non-zero: cleared
       // when every row has finished or, as a bound that does not depend on the data, at the limit the host stored
-      st.loop_it[2] = it_all + 1;
-      cudaGraphSetConditional(cond, (all_fin || it_all + 1 >= it_limit) ? 0u : 1u);
+      st.loop_it[2] = ctr1 + 1;
+      cudaGraphSetConditional(cond, (all_fin || ctr1 + 1 >= ctr2) ? 0u : 1u);
     }
   }
   if (next.source < 0) return;
@@ -337,7 +344,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
       }
     }
   };
-  if (CLUSTER || B == 1) {
+  if constexpr (FORM != ACC_ROWS) {
     // (at most 16 rows: every warp adds up those in front of its own)
     const int kr = lane < B ? s_k[lane] : 0, dr = lane < B && draft_pass ? draft_tokens(lane) : 0;
     const int boff = __reduce_add_sync(0xffffffffu, lane < b ? kr : 0), all = __reduce_add_sync(0xffffffffu, kr);

@@ -105,6 +105,7 @@ struct Switches {
   bool devloop = true;          // AD_NO_DEVLOOP=1: one graph replay per iteration with host polling instead of a device-side loop
   bool fuse_attn_proj = true;   // AD_NO_ATTN_PROJ=1: attention and its output projection always as separate kernels
   bool fuse_plan = true;        // AD_NO_FUSED_PLAN=1: plan in kernels of their own in every iteration
+  int accept_cluster = ACC_CLUSTER;   // AD_ACCEPT_CLUSTER=n: rows of a loop meet in a cluster up to n of them (0: always through global memory)
   // AD_MEGA=1: run eligible decoder passes (BF16, 64-wide heads, at most 64 packed tokens) as ONE persistent kernel
   // instead of the kernel chain.  Off by default: measured on a B200 it is slower than the chain at every shape tried
   // (base model: 342 / 360 / 424 / 462 us per verification step for blocks of 1 / 16 / 40 / 64 tokens against 214 / 223 /
@@ -145,6 +146,7 @@ struct ad_handle {
   int beta = 0;              // 0: exact-match verification; >= 1: relaxed verification (Section 3.2.3)
   float tau = 0.f;
   int n_vtiles = 0;
+  int accept_rows = 0;       // rows of a loop up to which the accept kernel is one cluster
   float* pe = nullptr;
   int max_pos = 0;
   int* ovr = nullptr;        // [B, max_tgt] staged draft-override stream
@@ -1283,6 +1285,28 @@ void swap_side(ad_handle* h) {
   std::swap(h->stream, h->side_stream);
 }
 
+// Most rows, up to `most`, whose accept kernels this device places as one cluster (0: none).  A CTA takes an SM's registers, so a cluster needs
+// that many SMs of one GPC, which a partitioned GPU may not have; beyond eight the device has to allow it too.
+int accept_cluster_rows(int most) {
+  auto* kernel = argmax_accept_kernel<ACC_CLUSTERED>;
+  if (most > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    most = 8;
+  }
+  for (; most > 1; --most) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(most); cfg.blockDim = dim3(ACC_THREADS);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = most; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0) return most;
+    cudaGetLastError();
+  }
+  return 0;
+}
+
 // Output projection fused with arg-max over X (yb for the verifier, the gathered mask rows for the drafter),
 // then the final reduction and (verifier) the draft compare.
 int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto_commit, bool partials_ready = false) {
@@ -1300,17 +1324,8 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
   }
   if (!partials_ready) AD_TRY(gemm(h, EPI_ARGMAX, m.emb, X, PK_VERIFY, pc.plan.M, pc.M_cap, p));
   note_launch(h, "argmax_accept");
-  // the rows of a decode loop as a cluster (up to 8 CTAs everywhere, 16 on this device)
   const int B = h->dims.B;
-  const bool cluster = auto_commit && !to_drafts && B > 1 && B <= ACC_CLUSTER;
-  if (cluster && B > 8) {
-    static bool attr_set[kMaxDevices] = {};
-    const int dev = current_device();
-    if (!attr_set[dev]) {
-      AD_CUDA(h, cudaFuncSetAttribute(argmax_accept_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-      attr_set[dev] = true;
-    }
-  }
+  const bool cluster = auto_commit && !to_drafts && B > 1 && B <= h->accept_rows;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(B); cfg.blockDim = dim3(ACC_THREADS); cfg.stream = h->stream;
   cudaLaunchAttribute attr[2];
@@ -1324,7 +1339,8 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
     attr[n_attr].val.clusterDim.x = B; attr[n_attr].val.clusterDim.y = 1; attr[n_attr++].val.clusterDim.z = 1;
   }
   cfg.attrs = attr; cfg.numAttrs = n_attr;
-  AD_CUDA(h, cudaLaunchKernelEx(&cfg, cluster ? argmax_accept_kernel<true> : argmax_accept_kernel<false>, h->st, pc.plan, h->dims, (const float*)h->part_val,
+  auto* kernel = cluster ? argmax_accept_kernel<ACC_CLUSTERED> : B == 1 ? argmax_accept_kernel<ACC_ONE> : argmax_accept_kernel<ACC_ROWS>;
+  AD_CUDA(h, cudaLaunchKernelEx(&cfg, kernel, h->st, pc.plan, h->dims, (const float*)h->part_val,
                                 (const int*)h->part_idx, h->n_vtiles, to_drafts, auto_commit, (unsigned int*)(h->st.loop_it + 1),
                                 auto_commit ? h->cond_handle : 0ull, relaxed ? 1 : 0, (const float*)h->draft_val, (const int*)h->draft_id,
                                 (const int*)h->part_cnt, h->next_pass));
@@ -1570,6 +1586,7 @@ extern "C" int ad_create(const ad_model_cfg* cfg, const ad_weights* w, void* wor
   h->sw.fuse_attn_proj = !env_is_1("AD_NO_ATTN_PROJ");
   h->sw.fuse_plan = !env_is_1("AD_NO_FUSED_PLAN");
   h->sw.mega = env_is_1("AD_MEGA");
+  if (const char* e = getenv("AD_ACCEPT_CLUSTER")) h->sw.accept_cluster = clampi(atoi(e), 0, ACC_CLUSTER);
   h->bf16 = cfg->dtype == AD_DTYPE_BF16;
   h->esz = h->bf16 ? 2 : 4;
   const size_t need = layout(h, workspace);
@@ -1603,6 +1620,7 @@ extern "C" int ad_create(const ad_model_cfg* cfg, const ad_weights* w, void* wor
         cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess)
       return bail(AD_ERR_CUDA, "creating the side stream failed");
   }
+  h->accept_rows = accept_cluster_rows(std::min(cfg->max_batch, h->sw.accept_cluster));
   // Cache, scratch and state start from zero so that no stale bit pattern is ever read as a number.
   if (cudaMemsetAsync(workspace, 0, need, h->stream) != cudaSuccess) return bail(AD_ERR_CUDA, "clearing the workspace failed");
   // Gather the cross-attention key/value projections of all decoder layers (see Model::ckv_all).

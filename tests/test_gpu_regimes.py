@@ -185,3 +185,40 @@ def test_rows_of_a_loop_end_like_single_rows(B):
             assert st[key] == sum(a[1][key] for a in alone)
     many.close()
     one.close()
+
+
+def _loop_results(dec, src, lens, cap, stream, relaxed):
+    runs = [dict(mode="IAD", k=6), dict(mode="GAD", k=5, run_drafter=True), dict(mode="GAD", k=6, draft_override=stream)]
+    out = []
+    for beta in ((0, 2) if relaxed else (0,)):
+        dec.set_acceptance(beta, 0.5)
+        for opts in runs:
+            rows, st = dec.generate(src, lens, max_len=cap, **opts)
+            out.append(([r.tolist() for r in rows], [st[key] for key in ("iterations", "row_iterations", "accepted", "offered")]))
+    return out
+
+
+@pytest.mark.parametrize("B", [2, 7, 8, 9, 16, 17])
+def test_rows_of_a_loop_meet_in_a_cluster_or_through_global_memory(B, monkeypatch):
+    """BF16 loops with drafts from the source, the drafter and the caller, exact and relaxed: the same tokens and counts whether the rows'
+    accept kernels are one cluster as large as the device places it, one of at most eight rows, or meet through global memory as on a
+    device that places none."""
+    shape = synth.MINI_BF16
+    w, wn = synth.make_weights(shape, 0), synth.make_weights(shape, 1)
+    r = np.random.default_rng(100 + B)
+    S, T = 12, 14
+    src = r.integers(4, 60, size=(B, S)).astype(np.int32)
+    lens = r.integers(2, S + 1, size=B).astype(np.int32)
+    cap = r.integers(1, T + 1, size=B).astype(np.int32)
+    stream = r.integers(4, shape.vocab, size=(B, T)).astype(np.int32)
+    results = []
+    for limit in (None, "8", "0"):
+        if limit is not None:
+            monkeypatch.setenv("AD_ACCEPT_CLUSTER", limit)      # read when a handle is created
+        dec = binding.AggressiveDecoder(shape, w, wn, max_batch=B, max_src=S, max_tgt=T, kmax=6)
+        greedy, _ = dec.generate(src, lens, max_len=cap, k=1)
+        for b in range(0, B, 2):                                # long accepted blocks in every other row
+            stream[b, : len(greedy[b])] = greedy[b]
+        results.append(_loop_results(dec, src, lens, cap, stream, relaxed=True))
+        dec.close()
+    assert results[1] == results[0] and results[2] == results[0]

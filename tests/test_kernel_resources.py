@@ -32,3 +32,10 @@ def test_layernorm_holds_what_its_partial_sums_need(tmp_path):
     for sym, (regs, spill) in found.items():
         name, p = re.search(r"(layernorm\w*kernel)I.*?Li\d+ELi(\d+)E", sym).groups()
         assert spill == 0 and regs <= limits[name][int(p)], f"{sym}: {regs} registers, {spill} bytes spilled"
+
+
+def test_accept_kernels_fit_a_thousand_threads_without_spills(tmp_path):
+    found = _report(tmp_path, [f"argmax_accept_kernel<{form}>" for form in ("ACC_ONE", "ACC_CLUSTERED", "ACC_ROWS")])
+    assert len(found) == 3
+    for sym, (regs, spill) in found.items():
+        assert spill == 0 and regs <= 64, f"{sym}: {regs} registers, {spill} bytes spilled"
