@@ -716,15 +716,15 @@ bool weights_stream(const ad_handle* h) {
 Prefetch attention_weights(const ad_handle* h, const Model& m, int l) {
   Prefetch f = {};
   if (!weights_stream(h) || l >= h->cfg.n_dec) return f;
-  const uint32_t dd = (uint32_t)(h->esz * h->cfg.d_model * h->cfg.d_model);
-  f.ptr[0] = (const char*)m.dec[l].wqkv.ptr; f.bytes[0] = 5 * dd;      // wqkv, wo, cq: one behind the other
-  f.ptr[1] = (const char*)m.dec[l].co.ptr; f.bytes[1] = dd;
+  const size_t dd = h->esz * h->cfg.d_model * h->cfg.d_model;
+  f.ptr[0] = (const char*)m.dec[l].wqkv.ptr; f.bytes[0] = prefetch_bytes(5 * dd);      // wqkv, wo, cq: one behind the other
+  f.ptr[1] = (const char*)m.dec[l].co.ptr; f.bytes[1] = prefetch_bytes(dd);
   return f;
 }
 Prefetch ffn_weights(const ad_handle* h, const Model& m, int l) {
   Prefetch f = {};
   if (!weights_stream(h)) return f;
-  const uint32_t df = (uint32_t)(h->esz * h->cfg.d_model * h->cfg.d_ffn);
+  const uint32_t df = prefetch_bytes(h->esz * h->cfg.d_model * h->cfg.d_ffn);
   f.ptr[0] = (const char*)m.dec[l].w1.ptr; f.bytes[0] = df;
   f.ptr[1] = (const char*)m.dec[l].w2.ptr; f.bytes[1] = df;
   return f;

@@ -122,8 +122,12 @@ __device__ __forceinline__ void resolve_partials(const Partials& q, int M, int& 
 // Weights that kernels further down the chain will read, to be brought into L2 (see prefetch_share).
 struct Prefetch {
   const char* ptr[2];
-  uint32_t bytes[2];     // multiples of 16; 0: nothing
+  uint32_t bytes[2];     // multiples of 16 (see prefetch_bytes); 0: nothing
 };
+// What to prefetch of a matrix: all of it, or nothing of one that would push a quarter of L2 and more out (whose offsets, moreover, might not
+// be numbers of 32 bits).
+constexpr size_t PF_MAX = (size_t)32 << 20;
+__host__ __device__ constexpr uint32_t prefetch_bytes(size_t bytes) { return bytes <= PF_MAX ? (uint32_t)bytes : 0u; }
 
 struct GemmParams {
   int K;                 // contraction length

@@ -1,4 +1,4 @@
-"""Registers and spills of the small kernels that a pass runs between its projections, as the compiler reports them.
+"""Registers and spills of the small kernels that a pass runs between its projections, as the compiler reports them, and sizes of prefetches.
 
 They are bound by one memory round trip each, and the registers they hold are kept from the projection behind them."""
 import os
@@ -39,3 +39,24 @@ def test_accept_kernels_fit_a_thousand_threads_without_spills(tmp_path):
     assert len(found) == 3
     for sym, (regs, spill) in found.items():
         assert spill == 0 and regs <= 64, f"{sym}: {regs} registers, {spill} bytes spilled"
+
+
+def test_prefetches_end(tmp_path):
+    """The pieces of a prefetch are counted in 32 bits: the step beyond the last one must not wrap around, for every number of CTAs."""
+    src = tmp_path / "prefetch.cu"
+    src.write_text("""
+#include "ad_common.cuh"
+using namespace ad;
+int main() {
+  const size_t sizes[] = {0, 16, 2048u * 1024, 5u << 21, PF_MAX, PF_MAX + 16, (size_t)1 << 31, ((size_t)1 << 32) - 16, (size_t)1 << 33};
+  for (size_t s : sizes)
+    for (uint32_t n = 1; n <= 1024; ++n) {
+      const uint32_t b = prefetch_bytes(s);
+      if (b > s || (uint64_t)b + (uint64_t)n * PF_PIECE > 0xffffffffull || b % 16) return 1;
+    }
+  return prefetch_bytes(PF_MAX) == PF_MAX && prefetch_bytes(((size_t)1 << 32) + 64) == 0 ? 0 : 1;
+}
+""")
+    exe = tmp_path / "prefetch"
+    subprocess.run([NVCC, "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-I", build.CSRC, str(src), "-o", str(exe)], check=True)
+    assert subprocess.run([str(exe)]).returncode == 0
