@@ -100,3 +100,54 @@ def test_source_keys_in_three_and_four_rounds(d, batch, k, src):
     stats = lockstep(dec, model, srcs, lens, streams, k, [k] * batch, tol=5e-2, max_steps=3)
     assert stats["steps"] > 0
     dec.close()
+
+
+def _needle_model(d):
+    """One layer whose self-attention drops everything else for one token, wherever that token is visible."""
+    shape = synth.ModelShape(f"needle_{d}", d, d // 64, 512, 1003, 1, 1, "bf16")
+    w = synth.make_weights(shape, 0)
+    needle, feature = 77, 5
+    w["emb"][:, feature] = 0.0
+    w["emb"][needle, feature] = 16.0 / np.sqrt(d)             # 16 once scaled; the positional part adds at most 1
+    p = "dec.0.self"
+    w[f"{p}.o.W"] = synth.round_to_bf16(w[f"{p}.o.W"] * 10.0)
+    for h in range(shape.n_heads):
+        w[f"{p}.k.W"][feature, h * 64 + 7] = 1.0
+        w[f"{p}.q.b"][h * 64 + 7] = 4.0                       # score 8 against at most 0.5 or so: 0.9 of the weight among 400 keys
+        w[f"{p}.v.W"][feature, h * 64 + 9: h * 64 + 17] = 0.5
+    w["emb"] = synth.round_to_bf16(w["emb"])
+    return shape, w, needle
+
+
+def _blocks(T, k):
+    return [(i, min(k, T - i)) for i in range(0, T, k)]
+
+
+@pytest.mark.parametrize("d,T,k,keys", [(256, 200, 17, (15, 16, 63, 64, 65, 80, 127, 128, 129, 191, 192, 198)),
+                                        (256, 180, 9, (64, 112, 128, 176)), (512, 400, 33, (127, 128, 255, 256, 271, 383, 384, 398))])
+def test_verified_blocks_see_their_own_keys_in_three_and_four_rounds(d, T, k, keys):
+    """Self-attention of blocks over a prefix that reaches three and four rounds of keys per warp, every query with its own number of them:
+    a token that takes the whole attention sits on either side of the first key of a warp and of a round, so a query that saw one key
+    too many or too few there would choose among other scores altogether."""
+    from paper_2205_10350_b200 import binding
+    shape, w, needle = _needle_model(d)
+    model = O.Model(shape, w, max_pos=512)
+    r = np.random.default_rng(d + k)
+    src = r.integers(100, shape.vocab, size=(1, 9)).astype(np.int32)
+    dec = binding.AggressiveDecoder(shape, w, max_batch=1, max_src=9, max_tgt=T, kmax=k)
+    st = model.state(src[0], cap=T)
+    for key in keys:
+        toks = r.integers(100, shape.vocab, size=T).astype(np.int32)
+        toks[key - 1] = needle                                # (key 0 is [BOS])
+        st.reset()
+        dec.encode(src, [9])
+        last = model.bos
+        for at, n in _blocks(T, k):
+            want = st.verify_block(last, toks[at: at + n], want_logits=True)["logits"]
+            dec.verify_block(toks[None, at: at + n], [n])
+            err = np.abs(dec.debug_logits(n) - want).max(1)
+            assert err.max() <= 5e-2, f"token at key {key}, block from {at}: scores differ by {err.max():.3f} at query {int(err.argmax())}"
+            st.commit(n)
+            dec.force_commit(toks[None, at: at + n], [n])
+            last = int(toks[at + n - 1])
+    dec.close()

@@ -137,9 +137,16 @@ def test_decode_loop_as_one_graph_equals_direct_launches_at_every_pass_size(B, k
     dec.close()
 
 
-# last and first capacity on either side of the lines between the encoder's attention kernels
-ENCODE_CASES = [("base", synth.BASE, 5, 80), ("base", synth.BASE, 5, 81), ("base", synth.BASE, 2, 200), ("bart", synth.BART_BASE_SIZED, 2, 97),
-                ("bart", synth.BART_BASE_SIZED, 2, 50)]
+# last and first capacity on either side of the lines between the encoder's attention kernels (148 SMs): few-query to MMA or FFMA kernel, FFMA to
+# MMA kernel (more than one key tile, more CTAs), MMA kernel to the same for many queries, and 256 keys and more
+ENCODE_CASES = [("base", synth.BASE, 5, 80), ("base", synth.BASE, 5, 81), ("base", synth.BASE, 2, 200), ("base", synth.BASE, 2, 208),
+                ("base", synth.BASE, 2, 209), ("base", synth.BASE, 2, 216), ("base", synth.BASE, 2, 217), ("base", synth.BASE, 1, 288),
+                ("base", synth.BASE, 1, 289), ("bart", synth.BART_BASE_SIZED, 2, 48), ("bart", synth.BART_BASE_SIZED, 2, 49),
+                ("bart", synth.BART_BASE_SIZED, 2, 64), ("bart", synth.BART_BASE_SIZED, 2, 65), ("bart", synth.BART_BASE_SIZED, 2, 97),
+                ("bart", synth.BART_BASE_SIZED, 2, 50), ("bart", synth.BART_BASE_SIZED, 2, 144), ("bart", synth.BART_BASE_SIZED, 2, 145),
+                ("bart", synth.BART_BASE_SIZED, 9, 16), ("bart", synth.BART_BASE_SIZED, 10, 16), ("bart", synth.BART_BASE_SIZED, 24, 8),
+                ("bart", synth.BART_BASE_SIZED, 25, 8), ("big", synth.BIG, 2, 32), ("big", synth.BIG, 2, 33), ("big", synth.BIG, 2, 48),
+                ("big", synth.BIG, 2, 49)]
 
 
 @pytest.mark.parametrize("name,shape,B,S", ENCODE_CASES, ids=[f"{c[0]}-{c[2]}x{c[3]}" for c in ENCODE_CASES])
