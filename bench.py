@@ -80,8 +80,8 @@ def reduce_max_sum(dist, dev, seconds_or_ms, count):
 # DRAM counters of one verification step (dram__bytes_read.sum + dram__bytes_write.sum summed over the step's
 # kernels, ncu, caches flushed before every kernel) with the digest of the kernel sources they were taken on:
 # the figures are reported only while the sources still have that digest.
-NCU_COUNTERS = dict(sources_sha256="0e430c475d759b6a39d20977cce86ed52bcb259bc45b68ab222a16f209732ea3",
-                    step_block40_bytes=92251648, projection_bytes=32864512,
+NCU_COUNTERS = dict(sources_sha256="ff6c87ba9bd82031411d5a2cbc3261707e3b9060e8f308fdf8da8da760bda6b5",
+                    step_block40_bytes=92147456, projection_bytes=32865024,
                     summary="profiles/verify_step_base_b1_k40_dram_traffic.txt")
 
 
