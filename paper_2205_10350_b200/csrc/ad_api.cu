@@ -922,6 +922,18 @@ bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   return 2L * c.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * split <= (long)waves * num_sms();
 }
 
+// Forms of the few-query kernel: query projection + 2 (pair of CTAs) + 4 (three or four rounds of keys) + 8 (looping grid).
+typedef void (*AttentionFewKernel)(const few::FewAttnParams);
+const AttentionFewKernel kAttentionFew[16] = {
+    few::attention_few_kernel<false, 1, false, false>, few::attention_few_kernel<true, 1, false, false>,
+    few::attention_few_kernel<false, 2, false, false>, few::attention_few_kernel<true, 2, false, false>,
+    few::attention_few_kernel<false, 1, true, false>,  few::attention_few_kernel<true, 1, true, false>,
+    few::attention_few_kernel<false, 2, true, false>,  few::attention_few_kernel<true, 2, true, false>,
+    few::attention_few_kernel<false, 1, false, true>,  few::attention_few_kernel<true, 1, false, true>,
+    few::attention_few_kernel<false, 2, false, true>,  few::attention_few_kernel<true, 2, false, true>,
+    few::attention_few_kernel<false, 1, true, true>,   few::attention_few_kernel<true, 1, true, true>,
+    few::attention_few_kernel<false, 2, true, true>,   few::attention_few_kernel<true, 2, true, true>};
+
 // Attention with its output projection (partial sums per head in pre2) and, with wq, the query projection of x = yb.
 int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v, const int* key_base, const int* nkeys_tok,
                   const int* nkeys_row, int max_keys, const Mat& wo, const Mat* wq = nullptr, const float* q_bias = nullptr) {
@@ -940,19 +952,22 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   const int dev = current_device();
   cudaError_t e = cudaSuccess;
   if (!attr_set[dev]) {
-    const int most = (int)few::att_few_smem(few::MAX_WARPS, few::MAX_ROUNDS);
-    for (auto* kernel : {few::attention_few_kernel<false, 1, false>, few::attention_few_kernel<true, 1, false>, few::attention_few_kernel<false, 2, false>,
-                         few::attention_few_kernel<true, 2, false>, few::attention_few_kernel<false, 1, true>, few::attention_few_kernel<true, 1, true>,
-                         few::attention_few_kernel<false, 2, true>, few::attention_few_kernel<true, 2, true>})
+    const int most = (int)few::att_few_smem(few::MAX_WARPS, few::MAX_ROUNDS, true);
+    for (auto* kernel : kAttentionFew)
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention attribute: ") + cudaGetErrorString(e));
     attr_set[dev] = true;
   }
   note_launch(h, wq ? "q_proj+attention+out_proj" : "attention+out_proj");
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(h->dims.B * p.qchunks * split, c.n_heads); cfg.blockDim = dim3(32 * warps);
+  // (CTAs of up to four warps fit an SM twice and keep their waves: 256 wide, encoder calls of four layers, 10 x 60 tokens 114 -> 125 us as a loop)
+  const long ctas = (long)c.max_batch * p.qchunks * c.n_heads * split;
+  const bool loop = ctas > num_sms() && warps > 4 && c.n_heads * split <= num_sms();
+  fp.rows = h->dims.B;
+  const int groups = loop ? std::min(h->dims.B * p.qchunks, num_sms() / (c.n_heads * split)) : h->dims.B * p.qchunks;
+  cfg.gridDim = dim3(groups * split, c.n_heads); cfg.blockDim = dim3(32 * warps);
   fp.rounds = (max_keys + few::AK * warps - 1) / (few::AK * warps);
-  cfg.dynamicSmemBytes = few::att_few_smem(warps, fp.rounds); cfg.stream = h->stream;
+  cfg.dynamicSmemBytes = few::att_few_smem(warps, fp.rounds, loop && wq && split > 1); cfg.stream = h->stream;
   cudaLaunchAttribute attr[2];
   int n_attr = 0;
   if (use_pdl()) {
@@ -964,12 +979,7 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
     attr[n_attr].val.clusterDim.x = split; attr[n_attr].val.clusterDim.y = 1; attr[n_attr++].val.clusterDim.z = 1;
   }
   cfg.attrs = attr; cfg.numAttrs = n_attr;
-  auto pick = [&](auto scores_first) {
-    constexpr bool F = decltype(scores_first)::value;
-    return split == 1 ? (wq ? few::attention_few_kernel<true, 1, F> : few::attention_few_kernel<false, 1, F>)
-                      : (wq ? few::attention_few_kernel<true, 2, F> : few::attention_few_kernel<false, 2, F>);
-  };
-  auto* kernel = fp.rounds > 2 ? pick(std::true_type()) : pick(std::false_type());
+  auto* kernel = kAttentionFew[(wq ? 1 : 0) + (split - 1) * 2 + (fp.rounds > 2 ? 4 : 0) + (loop ? 8 : 0)];
   e = cudaLaunchKernelEx(&cfg, kernel, fp);
   if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("attention launch: ") + cudaGetErrorString(e));
   return AD_OK;

@@ -151,3 +151,43 @@ def test_verified_blocks_see_their_own_keys_in_three_and_four_rounds(d, T, k, ke
             dec.force_commit(toks[None, at: at + n], [n])
             last = int(toks[at + n - 1])
     dec.close()
+
+
+@pytest.mark.parametrize("d,batch,k,src,rows", [
+    (512, 23, 1, 20, (0, 9, 22)),       # an item a row, more items than groups of CTAs by a handful
+    (512, 10, 33, 130, (0, 4, 9)),      # three items a row of which some are short, source keys in two rounds
+    (512, 40, 1, 260, (0, 31, 32, 39)), # more rows than lanes; source keys in three rounds
+    (384, 35, 2, 10, (0, 17, 34)),      # six warps; the last lane's share of the rows is not full
+    (768, 4, 33, 100, (0, 1, 3)),       # pairs of CTAs whose halves of the queries meet once an item, keys in two rounds
+    (1024, 3, 40, 300, (0, 2)),         # the same with keys in three rounds
+])
+def test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, rows):
+    """Attention of passes with more pieces of 16 queries than the device holds CTAs: one verified block of a ragged batch, idle rows among
+    the others, at an empty prefix and behind a committed one; sampled rows against the checker."""
+    from paper_2205_10350_b200 import binding
+    shape = synth.ModelShape(f"loop_{d}", d, d // 64, 512, 1003, 1, 2, "bf16")
+    w = synth.make_weights(shape, 0)
+    model = O.Model(shape, w, max_pos=320)
+    r = np.random.default_rng(d + batch + k)
+    lens = r.integers(max(1, src // 3), src + 1, size=batch).astype(np.int32)
+    lens[rows[-1]] = src
+    srcs = r.integers(4, shape.vocab, size=(batch, src)).astype(np.int32)
+    dec = binding.AggressiveDecoder(shape, w, max_batch=batch, max_src=src, max_tgt=2 * k + 1, kmax=k)
+    dec.encode(srcs, lens)
+    states = {b: model.state(srcs[b, : lens[b]], cap=2 * k + 1) for b in rows}
+    last = {b: model.bos for b in rows}
+    for turn in range(2):
+        drafts = r.integers(4, shape.vocab, size=(batch, k)).astype(np.int32)
+        n = np.where(r.random(batch) < 0.2, 0, r.integers(1, k + 1, size=batch)).astype(np.int32)
+        n[list(rows)] = [k] + [max(1, k - 5)] * (len(rows) - 2) + [k]
+        dec.verify_block(drafts, n)
+        lg = dec.debug_logits(int(n.sum()))
+        off = np.concatenate([[0], np.cumsum(n)])
+        for b in rows:
+            want = states[b].verify_block(last[b], drafts[b, : n[b]], want_logits=True)["logits"]
+            err = np.abs(lg[off[b]: off[b + 1]] - want).max()
+            assert err <= 5e-2, f"row {b}, turn {turn}: scores differ by {err:.3f}"
+            states[b].commit(int(n[b]))
+            last[b] = int(drafts[b, n[b] - 1])
+        dec.force_commit(drafts, n)
+    dec.close()
