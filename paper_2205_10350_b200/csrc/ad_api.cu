@@ -71,6 +71,10 @@ struct Model {
 };
 // Passes of at most this many packed tokens run their projections on the few-token kernel (gemm_few.cuh).
 constexpr int kFewTokens = few::MAX_TOKENS;
+// Encoder passes of at most this many have the embedding in their first projection; beyond, the projection's CTAs, each of which computes all of it
+// (its loads are three times the operand), take longer than a kernel in front of them.  Encoder calls of four layers, in the projection -> a kernel:
+// 512 wide, 1 x 80 tokens 111 -> 108 us, 2 x 50 116 -> 111, 4 x 32 121 -> 116; 768 wide, 1 x 97 161 -> 157; 1024 wide, 1 x 128 200 -> 190.
+constexpr int kFusedEmbed = 64;
 
 struct PassCfg {
   int M_cap = 0;     // packed-token capacity of this pass kind
@@ -635,9 +639,8 @@ GeoRule geo_rule(const PassCfg& pc, int epi, int N, int K, bool split, bool has_
   GeoRule r = {N, K, pc.ntile, split ? pc.max_split : 1, num_sms(), 0, 0, 0};
   if (epi == EPI_F32 ? split : (epi != EPI_ARGMAX && has_bias)) r.few_split = few::split_for(N, K, split, pc.max_split);
   if (r.few_split > 0) {
-    const int nch = K / r.few_split / 256;
     // (within a larger capacity a pass of few tokens runs the 16-feature form inside the tensor-core kernel)
-    r.few_tokens = pc.M_cap <= few::MAX_TOKENS ? few::MAX_TOKENS : few::max_tokens(nch);
+    r.few_tokens = pc.M_cap <= few::MAX_TOKENS ? few::MAX_TOKENS : few::INNER_TOKENS;
   }
   return r;
 }
@@ -1049,7 +1052,8 @@ int embed(ad_handle* h, const PassCfg& pc, const Model& m) {
 
 // Embedding of a pass's tokens: a kernel of its own, unless the pass's first projection computes it (null: it is done).
 int embed_or_defer(ad_handle* h, int pk, const Model& m, const Mat& first, const Model** deferred) {
-  *deferred = h->bf16 && always_few(h->pass[pk], geo_rule(h->pass[pk], EPI_SCATTER, first.N, first.K, false, true)) ? &m : nullptr;
+  const bool fits = pk != PK_ENCODE || h->pass[pk].M_cap <= kFusedEmbed;
+  *deferred = h->bf16 && fits && always_few(h->pass[pk], geo_rule(h->pass[pk], EPI_SCATTER, first.N, first.K, false, true)) ? &m : nullptr;
   return *deferred ? AD_OK : embed(h, h->pass[pk], m);
 }
 

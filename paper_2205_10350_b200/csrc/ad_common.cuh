@@ -62,7 +62,9 @@ enum Epi : int {
 //   2048 tokens: 128-token tiles 490 us, 64: 519, 256: 586 (256 is taken once it alone gives two CTAs per SM);
 //   1024 wide, 100 / 128 tokens: 64-token tiles 345 / 359 us, 128: 385 / 400, 32: 390 / 396.
 // The line at 1024 is the narrow models': 1024 wide, 128-token tiles already win there (648 us, 64: 717), and 64 at 200 (386, 32: 404).
-// Up to 128 tokens most projections take the few-token kernels and the rule is only asked for what those do not cover.
+// 65 to 128 tokens inside a larger capacity: 32-token tiles too.  Whole calls of 512 wide models whose passes are of this size, the 16-feature form
+// of the few-token kernel in two rounds -> 64-token tiles -> 32: batch 3 with drafter 4560 -> 4236 -> 4073 us, batch 5 with drafter 4610 -> 4415 -> 4304.
+// Passes that never have more than 128 tokens take the few-token kernels and the rule is only asked for what those do not cover.
 // A projection whose feature tiles alone outnumber the SMs (the vocabulary) fills them with one token tile, and every further one
 // reads its weights again: one 128-token tile up to 128 tokens (90 tokens x 50265 x 768: 19.5 us with two of 64), then tiles of 128
 // (400 x 768 x 50265: 56 us, 76 with 64-token tiles), of 256 beyond 1536 tokens, where L2 traffic bounds it (2048: 114 against 119 us).
@@ -92,8 +94,6 @@ __host__ __device__ inline Geo geometry(const GeoRule& r, int M) {
     while (g.tile < M) g.tile *= 2;
   } else if (nf >= r.sms) {
     g.tile = M <= 1536 ? 128 : 256;
-  } else if (M <= 128) {
-    g.tile = 64;
   } else if (M <= 256) {
     g.tile = 32;
   } else if (M <= 1024) {

@@ -22,7 +22,8 @@ constexpr int WARPS = 8;
 constexpr int FEAT = 16;          // output features per CTA = MMA M
 constexpr int W_FEAT = 32;        // ... of the form for wide slices of K (gemm_few_wide_kernel)
 constexpr int RED_LD = 20;        // floats per token row of a warp's partial sums: conflict-free, 16-byte aligned
-constexpr int MAX_TOKENS = 128;   // most packed tokens of a pass that these kernels take
+constexpr int MAX_TOKENS = 128;   // most packed tokens of a pass that these kernels take ...
+constexpr int INNER_TOKENS = 64;  // ... where its capacity is larger: one round
 constexpr int MAX_CHUNKS = 4;     // 32-wide K chunks per warp: K per CTA = 256 .. 1024
 
 // D (16 x 8, FP32) += A (16 x 16, BF16, row-major) * B (16 x 8, BF16, column-major).  Not volatile: free to be scheduled.
@@ -33,8 +34,6 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Most tokens a pass may have for the 16-feature kernel: two rounds.
-inline int max_tokens(int nch) { return nch <= 2 ? MAX_TOKENS : 64; }
 // Tokens of one round trip: 64 while a warp's slice of K is 64 wide, 32 beyond (register budget of two CTAs per SM).
 __host__ __device__ constexpr int round_tokens(int nch) { return nch <= 2 ? 64 : 32; }
 
