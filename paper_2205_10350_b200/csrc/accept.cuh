@@ -11,12 +11,16 @@ namespace ad {
 
 // What the accept kernel prepares for the pass behind it (source < 0: nothing).
 struct NextPass {
+  static constexpr int BODIES = BodyPick::BODIES;
+  typedef BodyPick Pick;
   int source;            // SRC_POLICY / SRC_OVERRIDE: plan the next verification block after the commit;
                          // SRC_SIZES: plan the drafter's pass after the commit (block sizes, then its tokens);
                          // SRC_KEEP (drafter's choices): plan the verification of the block just drafted
   const int* override_stream;
   int override_stride;
   PassPlan draft;        // SRC_SIZES: plan of the drafter's pass
+  Pick pick;
+  int launches;          // kernels of this iteration
 };
 
 constexpr int ACC_THREADS = 1024;
@@ -309,6 +313,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
       // the iteration runs inside a device-side `while` graph node, which repeats while its condition is non-zero: cleared
       // when every row has finished or, as a bound that does not depend on the data, at the limit the host stored
       st.loop_it[2] = ctr1 + 1;
+      atomicAdd(st.loop_it + 4, next.launches);
       cudaGraphSetConditional(cond, (all_fin || ctr1 + 1 >= ctr2) ? 0u : 1u);
     }
   }
@@ -355,6 +360,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
       if (b == 0) {
         *blk.M = all;
         if (draft_pass) *next.draft.M = dall;
+        pick_body(next.pick, all);
       }
     }
     lay_out(b, o0, boff, tid, ACC_THREADS, std::true_type());
@@ -381,6 +387,7 @@ argmax_accept_kernel(DevState st, PassPlan blk, Dims dm, const float* __restrict
       if (lane == 0) {
         *blk.M = base;
         if (draft_pass) *next.draft.M = dbase;
+        pick_body(next.pick, base);
       }
     }
     __syncthreads();

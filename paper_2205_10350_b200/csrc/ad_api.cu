@@ -1,5 +1,6 @@
 // Host side of the verification-step library: handle, workspace layout, kernel sequencing, CUDA-graph
 // replay of the decode loop, and the extern "C" entry points declared in include/aggressive_decoding.h.
+#include <limits.h>
 #include <math.h>
 #include <stdio.h>
 #include <stdlib.h>
@@ -81,7 +82,10 @@ struct PassCfg {
   int ntile = 16;    // tokens per GEMM tile
   int seg_max = 0;   // longest segment of one row
   int max_split = 1; // largest split-K factor this pass may use (sizes the partial-sum buffer)
+  int few_cap = few::MAX_TOKENS;   // capacities up to which every pass runs its projections on the few-token kernels
   PassPlan plan;
+  // Most pieces of up to q tokens of one row that a pass over `rows` rows can have.
+  long pieces(int rows, int q) const { return std::min((long)rows * ((seg_max + q - 1) / q), (long)std::min(rows, M_cap) + M_cap / q); }
 };
 
 // Launch shape of the tensor-core projection kernel (see tc_shape); ksplit: the most partial sums of any token count.
@@ -109,6 +113,7 @@ struct Switches {
   bool devloop = true;          // AD_NO_DEVLOOP=1: one graph replay per iteration with host polling instead of a device-side loop
   bool fuse_attn_proj = true;   // AD_NO_ATTN_PROJ=1: attention and its output projection always as separate kernels
   bool fuse_plan = true;        // AD_NO_FUSED_PLAN=1: plan in kernels of their own in every iteration
+  bool few_body = true;         // AD_NO_FEW_BODY=1: one body for every iteration of a device-side loop
   int accept_cluster = ACC_CLUSTER;   // AD_ACCEPT_CLUSTER=n: rows of a loop meet in a cluster up to n of them (0: always through global memory)
   // AD_MEGA=1: run eligible decoder passes (BF16, 64-wide heads, at most 64 packed tokens) as ONE persistent kernel
   // instead of the kernel chain.  Off by default: measured on a B200 it is slower than the chain at every shape tried
@@ -183,7 +188,7 @@ struct ad_handle {
   std::string err;
   struct GraphEntry {
     cudaGraphExec_t exec;   // null: the form has been called once, directly
-    int launches;        // kernels per replay (whole-call graph: per loop iteration)
+    int launches;        // kernels per replay (a device-side loop counts its own)
     bool device_loop;    // whole-call graph ...
     int once;            // ... and its kernels outside the loop
     long last_use;
@@ -204,6 +209,8 @@ struct ad_handle {
   float* mega_stats[2] = {nullptr, nullptr};
   unsigned long long* mega_timeline = nullptr;
   unsigned long long cond_handle = 0;   // non-zero only while the body of a device-side `while` node is captured
+  NextPass::Pick pick = {};             // set only while a loop whose body comes in several forms is captured
+  int body_launches = 0;                // h->launches where the body being captured begins
 };
 
 namespace {
@@ -391,7 +398,7 @@ size_t layout(ad_handle* h, void* base) {
   s.out_ids = ints((size_t)B * c.max_tgt);
   s.drafts = ints((size_t)B * c.kmax); s.pred = ints((size_t)B * c.kmax); s.n_acc = ints(B);
   s.stat_it = ints(B); s.stat_acc = ints(B); s.stat_off = ints(B);
-  s.loop_it = ints(4); s.status = ints(4); s.all_fin = ints(4); s.words = ints(4);
+  s.loop_it = ints(8); s.status = ints(4); s.all_fin = ints(4); s.words = ints(4);
   s.sync_ctr = (unsigned int*)ints((size_t)mega::SYNC_COUNTERS * mega::SYNC_STRIDE);
   s.cross_base = ints(B);
   s.gidx = ints((size_t)B * c.kmax);
@@ -640,7 +647,7 @@ GeoRule geo_rule(const PassCfg& pc, int epi, int N, int K, bool split, bool has_
   if (epi == EPI_F32 ? split : (epi != EPI_ARGMAX && has_bias)) r.few_split = few::split_for(N, K, split, pc.max_split);
   if (r.few_split > 0) {
     // (within a larger capacity a pass of few tokens runs the 16-feature form inside the tensor-core kernel)
-    r.few_tokens = pc.M_cap <= few::MAX_TOKENS ? few::MAX_TOKENS : few::INNER_TOKENS;
+    r.few_tokens = pc.M_cap <= pc.few_cap ? pc.few_cap : few::INNER_TOKENS;
   }
   return r;
 }
@@ -817,7 +824,7 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   p.d = c.d_model;
   // one query per warp while the grid stays within a couple of waves, eight when there are many queries
   const int dh = c.d_model / c.n_heads;
-  const bool many = (long long)h->dims.B * c.n_heads * ((pc.seg_max + 7) / 8) > 3LL * num_sms();
+  const bool many = pc.pieces(h->dims.B, 8) * c.n_heads > 3L * num_sms();
   p.scale = 1.0f / sqrtf((float)dh);
   // Tensor-core kernels when there are thousands of queries or rows may hold hundreds of keys (max_keys: the capacity, known on
   // the host); the FFMA kernel spreads few queries and few keys over more CTAs.
@@ -901,14 +908,15 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
 }
 
 // Whether the few-query kernel (attention_few.cuh) serves an attention of pass pk: BF16, 64-wide heads, the keys within four rounds
-// of its warps, and a grid of a few waves at most.  The grid counts what the pass could hold; CTAs of rows that have ended, of
-// blocks that are shorter and of a drafter's prefix that has not grown leave at once.  A wave costs 4 to 7 us, the projections that
-// are kernels of their own otherwise 12 us a layer, so a verification pass may need three waves at capacity, a drafter's pass
-// (on average half of its capacity) four.  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30:
+// of its warps, and work for a few waves of CTAs at most, counted by what the pass could hold (rows that have ended, shorter blocks and a
+// drafter's prefix that has not grown leave less).  A wave costs 4 to 7 us, the projections that
+// are kernels of their own otherwise 12 us a layer, so a verification pass may need two and a half waves at capacity (three where CTAs do not loop,
+// four beyond 512 wide), a drafter's pass (on average half of its capacity) four.  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30:
 // 214 -> 174 us; batch 24, 12: 237 -> 196; batch 20, 1: 188 -> 160; batch of 5 with drafter 442 -> 373; 1024 wide, batch 2, 40: 272 -> 226;
 // batch 3 with drafter 662 -> 600.  Beyond: base batch 32 x 64 (seven waves) 270 -> 315, 1024 wide batch 16 x 1 (four) 239 -> 284.  Wide
 // models with fewer than eight queries a row stay at one wave: their CTAs read two weight slices each for a tile that is mostly padding
-// (768 wide, batch 12, 1: 202 against 210).
+// (768 wide, batch 12, 1: 202 against 210).  Looping grids, waves 2 / 2.5 / 3 / 3.5 / 4 / 4.5, whole calls: 512 wide, batch 20 5068 / 5046 / 5073 / 5147 / 5350 / 5443,
+// batch 16, relaxed 2379 / 2375 / 2482 / 2483 / 2481 / 2480; from 3 on, 1024 wide, batch 8 5350 / 4873 / 5028 / 5078, 768 wide, batch 16 4786 / 4781 / 4409 / 4479.
 // An encoder's rows are as long as they are announced, and there is one projection to gain: one and a half.  Calls of four layers, 512 wide,
 // kernel without it -> with it, us: 3 x 112 tokens 143 -> 137, 4 x 96 143 -> 134, 5 x 75 144 -> 137, 8 x 48 140 -> 132, 24 x 16 139 -> 131.  One wave
 // beyond 512 wide (768 wide 2 x 90 147 -> 156, 3 x 64 147 -> 152), for rows of at most eight (512 wide 24 x 8 116 -> 118, 24 x 4 122 -> 125; 256 wide
@@ -921,8 +929,8 @@ bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   if (max_keys > few::MAX_ROUNDS * few::AK * few::att_few_warps(c.d_model)) return false;
   // (in half waves)
   const bool one_wave = pk == PK_ENCODE ? split > 1 || max_keys >= 256 || (pc.seg_max <= 8 && c.d_model > 256) : split > 1 && pc.seg_max < 8;
-  const int waves = one_wave ? 2 : pk == PK_ENCODE ? 3 : pk == PK_DRAFT ? 8 : 6;
-  return 2L * c.max_batch * ((pc.seg_max + few::AQ - 1) / few::AQ) * c.n_heads * split <= (long)waves * num_sms();
+  const int waves = one_wave ? 2 : pk == PK_ENCODE ? 3 : pk == PK_DRAFT || split > 1 ? 8 : few::att_few_warps(c.d_model) > 4 ? 5 : 6;
+  return 2 * pc.pieces(c.max_batch, few::AQ) * c.n_heads * split <= (long)waves * num_sms();
 }
 
 // Forms of the few-query kernel: query projection + 2 (pair of CTAs) + 4 (three or four rounds of keys) + 8 (looping grid).
@@ -964,10 +972,10 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   note_launch(h, wq ? "q_proj+attention+out_proj" : "attention+out_proj");
   cudaLaunchConfig_t cfg = {};
   // (CTAs of up to four warps fit an SM twice and keep their waves: 256 wide, encoder calls of four layers, 10 x 60 tokens 114 -> 125 us as a loop)
-  const long ctas = (long)c.max_batch * p.qchunks * c.n_heads * split;
+  const long items = pc.pieces(c.max_batch, few::AQ), ctas = items * c.n_heads * split;
   const bool loop = ctas > num_sms() && warps > 4 && c.n_heads * split <= num_sms();
   fp.rows = h->dims.B;
-  const int groups = loop ? std::min(h->dims.B * p.qchunks, num_sms() / (c.n_heads * split)) : h->dims.B * p.qchunks;
+  const int groups = loop ? (int)std::min(items, (long)num_sms() / (c.n_heads * split)) : h->dims.B * p.qchunks;
   cfg.gridDim = dim3(groups * split, c.n_heads); cfg.blockDim = dim3(32 * warps);
   fp.rounds = (max_keys + few::AK * warps - 1) / (few::AK * warps);
   cfg.dynamicSmemBytes = few::att_few_smem(warps, fp.rounds, loop && wq && split > 1); cfg.stream = h->stream;
@@ -1340,6 +1348,8 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
   note_launch(h, "argmax_accept");
   const int B = h->dims.B;
   const bool cluster = auto_commit && !to_drafts && B > 1 && B <= h->accept_rows;
+  NextPass next = h->next_pass;
+  next.launches = h->launches - h->body_launches;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(B); cfg.blockDim = dim3(ACC_THREADS); cfg.stream = h->stream;
   cudaLaunchAttribute attr[2];
@@ -1357,7 +1367,7 @@ int vocab_stage(ad_handle* h, Model& m, const ActBuf& X, int to_drafts, int auto
   AD_CUDA(h, cudaLaunchKernelEx(&cfg, kernel, h->st, pc.plan, h->dims, (const float*)h->part_val,
                                 (const int*)h->part_idx, h->n_vtiles, to_drafts, auto_commit, (unsigned int*)(h->st.loop_it + 1),
                                 auto_commit ? h->cond_handle : 0ull, relaxed ? 1 : 0, (const float*)h->draft_val, (const int*)h->draft_id,
-                                (const int*)h->part_cnt, h->next_pass));
+                                (const int*)h->part_cnt, next));
   h->last_vocab_which = to_drafts ? 1 : 0;
   return AD_OK;
 }
@@ -1368,8 +1378,57 @@ int prepare_verify(ad_handle* h, int source, const int* ovr, int* user_drafts = 
   if (user_drafts) { st.user_drafts = user_drafts; st.user_k = user_k; }
   note_launch(h, "prepare_verify");
   AD_CUDA(h, launch_k(prepare_verify_kernel, dim3(1), dim3(256), 0, h->stream, st, h->pass[PK_VERIFY].plan, h->dims, source, ovr,
-                      h->cfg.max_tgt));
+                      h->cfg.max_tgt, h->pick));
   return AD_OK;
+}
+
+// Whether the accept kernels of a decode loop plan the passes behind them (kernel-chain form of the passes only).
+bool loop_plans_ahead(const ad_handle* h) { return h->sw.fuse_plan && !h->mega[PK_VERIFY].on && !h->mega[PK_DRAFT].on; }
+// The body of a decode loop comes in up to three forms, each laid out for a verification pass of at most cap[i] tokens; an iteration takes the first
+// one that holds the tokens planned for it (the choice is a graph node and costs 3.5 us).  A batch begins with hundreds of tokens and ends with a handful, for which
+// the kernels and grids that a large capacity asks for are the wrong ones: 512 wide, batch 32, blocks of 64, an iteration of 9 to 128 tokens took 220 to 320 us,
+// of a handle made for so few 130 to 180.  First the few-token kernels, up to 64 tokens (96 beyond 512 wide, see geometry); then, where the whole capacity is too
+// much for the few-query attention, as many tokens as it takes; then all.  Calls of the input-guided policy, whose blocks are mostly short, keep the
+// few-token kernels as their only form up to 128 tokens, others up to 96.  Whole calls, one form -> several: 512 wide, batch 32 4840 -> 4437 us, batch 20 5740 -> 5104,
+// batch 12 2678 -> 2590, batch 8 3112 -> 3046, batch 5 with drafter 4440 -> 4300; 768 wide, batch 6 4209 -> 4005, batch 16 4814 -> 4461; 1024 wide, batch 8 5465 -> 5071, with
+// drafter 10890 -> 9975.
+struct LoopBodies { int n, cap[NextPass::BODIES]; };
+// While one lives, pass pk is laid out for at most `cap` tokens (few_cap: see PassCfg).
+struct PassLayout {
+  ad_handle* h;
+  int pk;
+  PassCfg kept;
+  PassLayout(ad_handle* h, int pk, int cap, int few_cap) : h(h), pk(pk), kept(h->pass[pk]) {
+    PassCfg& pc = h->pass[pk];
+    pc.M_cap = std::min(pc.M_cap, cap);
+    pc.ntile = clampi(pow2ceil(pc.M_cap), 16, 256);
+    pc.few_cap = few_cap;
+  }
+  ~PassLayout() { h->pass[pk] = kept; }
+};
+PassLayout body_layout(ad_handle* h, const LoopBodies& b, int i) {
+  return PassLayout(h, PK_VERIFY, b.cap[i], b.n > 1 && i > 0 ? 0 : kFewTokens);
+}
+LoopBodies loop_bodies(ad_handle* h, bool policy) {
+  const PassCfg& pc = h->pass[PK_VERIFY];
+  const int d = h->cfg.d_model, full = pc.M_cap;
+  LoopBodies b = {1, {full, 0, 0}};
+  const int few = d <= 512 ? 64 : 96;
+  if (!h->bf16 || !h->sw.few_body || !loop_plans_ahead(h) || few::split_for(3 * d, d, false, 1) == 0) return b;
+  if (full <= (policy ? kFewTokens : 96)) return b;
+  b.n = 0;
+  b.cap[b.n++] = few;
+  if (!attention_is_few(h, PK_VERIFY, h->cfg.max_src)) {
+    int cap = few;
+    for (int c = few + 16; c < full; c += 16) {
+      const PassLayout at(h, PK_VERIFY, c, 0);
+      if (!attention_is_few(h, PK_VERIFY, h->cfg.max_src)) break;
+      cap = c;
+    }
+    if (cap > few) b.cap[b.n++] = cap;
+  }
+  b.cap[b.n++] = full;
+  return b;
 }
 
 // Draft substep: sizes and drafter plan ...
@@ -1409,8 +1468,6 @@ int commit_stage(ad_handle* h, const int* n_dev, int* status_out) {
   return AD_OK;
 }
 
-// Whether the accept kernels of a decode loop plan the passes behind them (kernel-chain form of the passes only).
-bool loop_plans_ahead(const ad_handle* h) { return h->sw.fuse_plan && !h->mega[PK_VERIFY].on && !h->mega[PK_DRAFT].on; }
 bool loop_drafts(const ad_gen_opts& o) { return o.mode == AD_MODE_GAD && o.run_drafter; }
 int block_source(const ad_gen_opts& o, const int* ovr) { return o.mode == AD_MODE_GAD || ovr ? SRC_OVERRIDE : SRC_POLICY; }
 
@@ -1418,6 +1475,7 @@ NextPass next_pass(const ad_handle* h, int source, const int* ovr) {
   NextPass n = no_next_pass();
   n.source = source; n.override_stream = ovr; n.override_stride = h->cfg.max_tgt;
   n.draft = h->pass[PK_DRAFT].plan;
+  if (source != SRC_KEEP) n.pick = h->pick;
   return n;
 }
 
@@ -1599,6 +1657,7 @@ extern "C" int ad_create(const ad_model_cfg* cfg, const ad_weights* w, void* wor
   h->sw.two_stream_encode = !env_is_1("AD_NO_CONCURRENT_ENCODERS");
   h->sw.fuse_attn_proj = !env_is_1("AD_NO_ATTN_PROJ");
   h->sw.fuse_plan = !env_is_1("AD_NO_FUSED_PLAN");
+  h->sw.few_body = !env_is_1("AD_NO_FEW_BODY");
   h->sw.mega = env_is_1("AD_MEGA");
   if (const char* e = getenv("AD_ACCEPT_CLUSTER")) h->sw.accept_cluster = clampi(atoi(e), 0, ACC_CLUSTER);
   h->bf16 = cfg->dtype == AD_DTYPE_BF16;
@@ -1811,11 +1870,20 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
   if (on_host)
     for (int b = 0; b < B; ++b)
       if (k[b] < 0 || k[b] > c.kmax) return fail(h, AD_ERR_ARG, "k outside 0..kmax");
-  // One graph per batch size and kind of acceptance rule (its beta and tau are words): with host arrays the whole call (the block is read from, and the result
+  // With host arrays the tokens are known here, and the pass is laid out for so many (see LoopBodies).
+  const bool captured = being_captured(h);
+  LoopBodies bodies = {1, {h->pass[PK_VERIFY].M_cap}};
+  int layout_of = 0;
+  if (on_host && !captured) {
+    long tokens = 0;
+    for (int b = 0; b < B; ++b) tokens += k[b];
+    bodies = loop_bodies(h, false);
+    while (layout_of + 1 < bodies.n && tokens > bodies.cap[layout_of]) ++layout_of;
+  }
+  // One graph per batch size, layout and kind of acceptance rule (its beta and tau are words): with host arrays the whole call (the block is read from, and the result
   // written to, mapped host memory), with device arrays everything but the copies from and to the caller's arrays.
   char key[48];
-  snprintf(key, sizeof(key), "verify B%d h%d r%d", B, on_host ? 1 : 0, h->beta >= 1 ? 1 : 0);
-  const bool captured = being_captured(h);
+  snprintf(key, sizeof(key), "verify B%d h%d r%d f%d", B, on_host ? 1 : 0, h->beta >= 1 ? 1 : 0, layout_of);
   AD_TRY(set_words(h, captured, h->words.x, h->beta, h->tau));
   if (on_host) {
     memcpy(h->up_ids, drafts, sizeof(int) * (size_t)B * c.kmax);
@@ -1825,6 +1893,7 @@ extern "C" int ad_verify_block(ad_handle* h, const int32_t* drafts, const int32_
     AD_CUDA(h, cudaMemcpyAsync(h->st.user_k, k, sizeof(int) * B, cudaMemcpyDeviceToDevice, h->stream));
   }
   AD_TRY(run_captured(h, captured, key, [&]() -> int {
+    const PassLayout layout = body_layout(h, bodies, layout_of);
     if (on_host) AD_TRY(prepare_verify(h, SRC_USER, nullptr, h->dev_view(h->up_ids), h->dev_view(h->up_n)));
     else AD_TRY(prepare_verify(h, SRC_USER, nullptr));
     AD_TRY(verify_stage(h, 0));
@@ -1921,12 +1990,18 @@ extern "C" int ad_get_state(ad_handle* h, int32_t* len, int32_t* last_tok, int32
 namespace {
 
 // ad_generate's device work as one graph: encoder pass(es), plan of the first pass, loop (see ad_generate).
-bool build_whole_graph(ad_handle* h, const ad_gen_opts& o, const int* ovr, bool capped, ad_handle::GraphEntry* out) {
+bool build_whole_graph(ad_handle* h, const ad_gen_opts& o, const int* ovr, bool capped, const LoopBodies& bodies, ad_handle::GraphEntry* out) {
   const int before = h->launches;
   cudaGraph_t g = nullptr, dummy = nullptr;
   cudaGraphConditionalHandle ch = 0;
   std::vector<cudaGraphNode_t> tail;
   bool ok = cudaGraphCreate(&g, 0) == cudaSuccess && cudaGraphConditionalHandleCreate(&ch, g, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+  if (ok && bodies.n > 1) {
+    cudaGraphConditionalHandle pick = 0;
+    ok = cudaGraphConditionalHandleCreate(&pick, g, 0, cudaGraphCondAssignDefault) == cudaSuccess;
+    h->pick.node = (unsigned long long)pick;
+    for (int i = 0; i + 1 < NextPass::BODIES; ++i) h->pick.cap[i] = i + 1 < bodies.n ? bodies.cap[i] : INT_MAX;
+  }
   if (ok && cudaStreamBeginCaptureToGraph(h->stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
     ok = encode_stage(h, capped) == AD_OK;
     ok = ok && cudaEventRecordWithFlags(h->ev1, h->stream, cudaEventRecordExternal) == cudaSuccess;   // an event node: end of the encoders
@@ -1949,17 +2024,32 @@ bool build_whole_graph(ad_handle* h, const ad_gen_opts& o, const int* ovr, bool 
     np.conditional.size = 1;
     cudaGraphNode_t node;
     ok = cudaGraphAddNode(&node, g, tail.data(), tail.size(), &np) == cudaSuccess;
-    if (ok && cudaStreamBeginCaptureToGraph(h->stream, np.conditional.phGraph_out[0], nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+    const cudaGraph_t body = ok ? np.conditional.phGraph_out[0] : nullptr;
+    auto capture_body = [&](cudaGraph_t into) {
+      if (cudaStreamBeginCaptureToGraph(h->stream, into, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return false;
       h->cond_handle = (unsigned long long)ch;
-      ok = loop_iteration(h, o, ovr) == AD_OK;
+      h->body_launches = h->launches;
+      bool done = loop_iteration(h, o, ovr) == AD_OK;
       h->cond_handle = 0;
-      ok = cudaStreamEndCapture(h->stream, &dummy) == cudaSuccess && ok;
-    } else {
-      ok = false;
+      h->launches = before;
+      return cudaStreamEndCapture(h->stream, &dummy) == cudaSuccess && done;
+    };
+    if (ok && bodies.n > 1) {
+      cudaGraphNodeParams sp = {cudaGraphNodeTypeConditional};
+      sp.conditional.handle = (cudaGraphConditionalHandle)h->pick.node;
+      sp.conditional.type = cudaGraphCondTypeSwitch;
+      sp.conditional.size = bodies.n;
+      cudaGraphNode_t pick;
+      ok = cudaGraphAddNode(&pick, body, nullptr, 0, &sp) == cudaSuccess;
+      for (int i = 0; i < bodies.n && ok; ++i) {
+        const PassLayout layout = body_layout(h, bodies, i);
+        ok = capture_body(sp.conditional.phGraph_out[i]);
+      }
+    } else if (ok) {
+      ok = capture_body(body);
     }
   }
-  out->launches = h->launches - before;
-  h->launches = before;
+  h->pick = {};
   ok = ok && cudaGraphInstantiate(&out->exec, g, 0) == cudaSuccess;
   if (g) cudaGraphDestroy(g);
   out->device_loop = ok;
@@ -2018,9 +2108,13 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
       ad_handle::GraphEntry entry = {};
       // First choice: the whole call as one graph -- encoder pass(es), plan of the first block, and a device-side `while` node
       // whose body is one iteration and whose condition the accept/commit kernel clears; no host round trip between them.
-      if (h->sw.devloop && !build_whole_graph(h, *opts, ovr, capped, &entry)) {
+      // (a driver that does not know such a node: one body; no `while` node either: one replay per iteration)
+      const LoopBodies one = {1, {h->pass[PK_VERIFY].M_cap}}, bodies = loop_bodies(h, !loop_drafts(*opts) && block_source(*opts, ovr) == SRC_POLICY);
+      for (const LoopBodies* b : {&bodies, &one}) {
+        if (!h->sw.devloop || (b == &one && bodies.n == 1)) break;
+        if (build_whole_graph(h, *opts, ovr, capped, *b, &entry)) break;
         entry = ad_handle::GraphEntry{};
-        cudaGetLastError();   // clear; fall back to one replay per iteration
+        cudaGetLastError();
       }
       if (!entry.exec) {
         const int before = h->launches;
@@ -2081,7 +2175,7 @@ extern "C" int ad_generate(ad_handle* h, const int32_t* src, int32_t src_stride,
                       on_host ? nullptr : out_len, h->down_dev));
   AD_CUDA(h, cudaStreamSynchronize(h->stream));
   const int* blk = h->down;
-  if (device_loop) h->launches += per_iter_launches * blk[0];
+  if (device_loop) h->launches += blk[3];
   if (on_host) {
     const int w = out_stride < c.max_tgt ? out_stride : c.max_tgt;
     for (int b = 0; b < B; ++b) {

@@ -25,7 +25,8 @@ struct DevState {
   int* stat_it;    // [B] iterations the row took part in
   int* stat_acc;   // [B] tokens accepted
   int* stat_off;   // [B] block sizes offered
-  int* loop_it;    // [1] iterations with at least one active row
+  int* loop_it;    // [0] iterations with at least one active row, [1] rows-done counter of the accept kernel, [2] iterations of the device-side loop,
+                   // [3] their limit, [4] the kernels they launched
   int* status;     // [1] latched device error
   int* all_fin;    // [1] 1 when every row is finished
   int* words;      // [4] what a call may change from one time to the next and a captured graph must not: block-size cap, valid entries of
@@ -177,9 +178,19 @@ __device__ __forceinline__ void plan_verify_block(const DevState& st, const Pass
   }
 }
 
+// A decode loop whose body comes in several forms (each for at most so many tokens): picks the first one that holds the pass that has been planned.
+struct BodyPick {
+  static constexpr int BODIES = 3;
+  unsigned long long node;   // 0: there is one form
+  int cap[BODIES - 1];
+};
+__device__ __forceinline__ void pick_body(const BodyPick& p, int tokens) {
+  if (p.node) cudaGraphSetConditional(p.node, tokens <= p.cap[0] ? 0u : tokens <= p.cap[1] ? 1u : 2u);
+}
+
 // grid = 1, block = 256.
 __global__ void __launch_bounds__(256)
-prepare_verify_kernel(DevState st, PassPlan plan, Dims dm, int source, const int* override_stream, int override_stride) {
+prepare_verify_kernel(DevState st, PassPlan plan, Dims dm, int source, const int* override_stream, int override_stride, BodyPick pick) {
   trace_mark(TR_PREPARE, 0);
   pdl_wait();                  // (no pdl_launch: see plan data in ad_common.cuh)
   trace_mark(TR_PREPARE, 1);
@@ -188,6 +199,7 @@ prepare_verify_kernel(DevState st, PassPlan plan, Dims dm, int source, const int
   NextBlock nb;
   nb.source = source; nb.override_stream = override_stream; nb.override_stride = override_stride;
   plan_verify_block(st, plan, dm, nb, s_k, s_off);
+  if (threadIdx.x == 0) pick_body(pick, s_off[dm.B]);
   __threadfence();
 }
 
@@ -254,6 +266,7 @@ plan_encode_kernel(DevState st, PassPlan plan, Dims dm, const int* maxlen) {
     *plan.M = acc;
     *st.loop_it = 0;
     st.loop_it[2] = 0;
+    st.loop_it[4] = 0;
     *st.all_fin = 0;
   }
   for (int b = tid; b < B; b += 256) {
@@ -681,7 +694,7 @@ __global__ void export_host_kernel(DevState st, Dims dm, PassPlan blk, int draft
 // End of ad_generate: everything the host needs, gathered into one block (device pointer of pinned, mapped host memory
 // or a device buffer), so that the call ends with ONE synchronisation and no further copies:
 //   block[0] = iterations the device-side loop ran, block[1] = latched status word (cleared here),
-//   block[2] = iterations with an active row, block[3] = B,
+//   block[2] = iterations with an active row, block[3] = kernels that the device-side loop launched,
 //   block[4 + 4 b ..] = {row iterations, accepted, offered, output length} of row b,
 //   block[4 + 4 B + b * max_tgt ..] = output ids of row b (only when out_dev is null: host-resident results).
 // out_dev / out_len_dev (device pointers, may be null): the caller's result arrays when they live on the device.
@@ -698,7 +711,7 @@ finalize_generate_kernel(DevState st, Dims dm, int* out_dev, int out_stride, int
       block[1] = *st.status;
       *st.status = 0;
       block[2] = st.loop_it[0];
-      block[3] = dm.B;
+      block[3] = st.loop_it[4];
     }
     int* row = block + 4 + 4 * b;
     row[0] = st.stat_it[b]; row[1] = st.stat_acc[b]; row[2] = st.stat_off[b]; row[3] = len;
