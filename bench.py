@@ -274,6 +274,8 @@ def kernel_table(dec, shape, drafts, k, pk):
             g["bytes"] += N * K * 2 + k * K * 2 + k * N * out_b
         elif "attention" in name:
             g["bytes"] += 2 * 40 * d * 2 + 2 * k * d * 2 + (d * d * 2 + 8 * k * d * 4 if "out_proj" in name else 0) + (d * d * 2 if "q_proj" in name else 0)
+        elif name == "ffn":
+            g["bytes"] += 2 * d * F * 2 + k * d * 2 + (F // 64) * k * d * 4
         elif "layernorm" in name:
             g["bytes"] += 9 * k * d * 4 + k * d * 6
     total = sum(g["us"] for g in groups.values())

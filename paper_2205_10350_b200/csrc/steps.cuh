@@ -417,6 +417,27 @@ __device__ __forceinline__ LnWeights ln_weights(const LnParams& p, int gi) {
   return w;
 }
 
+// Normalisation of a token whose features a group of THREADS threads holds, four each at off (`on`: this thread has some).
+template <typename ActT, int THREADS>
+__device__ __forceinline__ void ln_finish(const LnParams& p, const LnWeights& w, size_t off, bool on, float4 v, ActT* yb, float* red, int tid, int half) {
+  const float mean = group_sum<THREADS>(v.x + v.y + v.z + v.w, red, tid, half) / (float)p.d;
+  float vs = 0.f;
+  if (on) {
+    const float a = v.x - mean, b = v.y - mean, c = v.z - mean, e = v.w - mean;
+    vs = a * a + b * b + c * c + e * e;
+  }
+  const float inv = rsqrtf(group_sum<THREADS>(vs, red + THREADS / 32, tid, half) / (float)p.d + p.eps);
+  if (on) {
+    float4 o;
+    o.x = w.g.x * ((v.x - mean) * inv) + w.b.x;
+    o.y = w.g.y * ((v.y - mean) * inv) + w.b.y;
+    o.z = w.g.z * ((v.z - mean) * inv) + w.b.z;
+    o.w = w.g.w * ((v.w - mean) * inv) + w.b.w;
+    store4(p.y + off * 4, o);
+    store4(yb + off * 4, o);
+  }
+}
+
 // Token m by a group of THREADS threads, four features per thread (d <= 4 * THREADS): the residual and all partial sums of a thread
 // (P of them at most) are requested at once, so that the kernel costs one memory round trip.  (Two groups of features per thread took
 // 2.8 us instead of 1.5 us per launch on a 1024-wide model with 16 partials; 9 to 16 partials in two turns of eight, with 64
@@ -440,24 +461,8 @@ __device__ __forceinline__ void ln_token(const LnParams& p, const LnWeights& w, 
 #pragma unroll
     for (int sp = 0; sp < P; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
   }
-  const float mean = group_sum<THREADS>(v.x + v.y + v.z + v.w, red, tid, half) / (float)p.d;
-  float vs = 0.f;
-  if (on) {
-    const float a = v.x - mean, b = v.y - mean, c = v.z - mean, e = v.w - mean;
-    vs = a * a + b * b + c * c + e * e;
-  }
-  const float inv = rsqrtf(group_sum<THREADS>(vs, red + THREADS / 32, tid, half) / (float)p.d + p.eps);
-  if (on) {
-    float4 o;
-    o.x = w.g.x * ((v.x - mean) * inv) + w.b.x;
-    o.y = w.g.y * ((v.y - mean) * inv) + w.b.y;
-    o.z = w.g.z * ((v.z - mean) * inv) + w.b.z;
-    o.w = w.g.w * ((v.w - mean) * inv) + w.b.w;
-    store4(p.y + off * 4, o);
-    store4(yb + off * 4, o);
-  }
+  ln_finish<ActT, THREADS>(p, w, off, on, v, yb, red, tid, half);
 }
-
 // One CTA per token.  grid = M_cap, block = THREADS (128 for d <= 512, else 256).
 // What bounds it: one memory round trip (1.0-1.3 us), and what it keeps from the projection behind it, whose CTAs (32 K registers and up to
 // 200 KB of shared memory each) want to be on the SM before this kernel's wait is over.  With room for 16 partial sums whatever their number
@@ -480,6 +485,47 @@ layernorm_kernel(const LnParams p, ActT* __restrict__ yb) {
   trace_mark(TR_LN, 1);
   if (m >= M) return;
   ln_token<ActT, THREADS, P>(p, w, m, nsplit, stride, yb, red, threadIdx.x, -1);
+  trace_mark(TR_LN, 2);
+}
+
+// 17 to 32 partial sums, d <= 512: two halves of a CTA add up to 16 each.  One CTA per token; grid = M_cap, block = 256.  What bounds it is the 64 KB that
+// a token's sums are (512 wide): half a microsecond on one SM.
+template <typename ActT>
+__global__ void __launch_bounds__(256, 2)
+layernorm_parts_kernel(const LnParams p, ActT* __restrict__ yb) {
+  __shared__ float red[2 * 4];
+  __shared__ __align__(16) float4 other[128];
+  trace_mark(TR_LN, 0);
+  pdl_launch();
+  const int m = blockIdx.x, M = plan_load(p.M_ptr), half = threadIdx.x >> 7, tid = threadIdx.x & 127;
+  const LnWeights w = ln_weights(p, tid);
+  if (m >= M && m > 0) return;                     // CTA 0 always waits (see early exits in ad_common.cuh)
+  pdl_wait();
+  trace_mark(TR_LN, 1);
+  if (m >= M) return;
+  const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  const size_t off = (size_t)m * (p.d >> 2) + tid, step = p.pre.stride >> 2;
+  const bool on = tid < (p.d >> 2);
+  float4 v = zero4;
+  if (on) {
+    const int n = p.pre.nsplit, first = half * 16;
+    const float4* pre = reinterpret_cast<const float4*>(p.pre.ptr) + off + first * step;
+    float4 part[16];
+#pragma unroll
+    for (int sp = 0; sp < 16; ++sp, pre += step) part[sp] = first + sp < n ? *pre : zero4;
+    if (half == 0) {
+      const float4 r = p.resid ? reinterpret_cast<const float4*>(p.resid)[off] : zero4;
+      v = make_float4(w.c.x + r.x, w.c.y + r.y, w.c.z + r.z, w.c.w + r.w);
+    }
+#pragma unroll
+    for (int sp = 0; sp < 16; ++sp) { v.x += part[sp].x; v.y += part[sp].y; v.z += part[sp].z; v.w += part[sp].w; }
+  }
+  if (half == 1) other[tid] = v;
+  __syncthreads();
+  if (half == 1) return;
+  const float4 o = other[tid];
+  v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+  ln_finish<ActT, 128>(p, w, off, on, v, yb, red, tid, 0);
   trace_mark(TR_LN, 2);
 }
 

@@ -191,3 +191,14 @@ def test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, r
             last[b] = int(drafts[b, n[b] - 1])
         dec.force_commit(drafts, n)
     dec.close()
+
+
+@pytest.mark.parametrize("d,ffn,batch,k", [
+    (128, 64, 1, 3),         # one slice of hidden features, two warps
+    (256, 1024, 3, 5),       # 16 partial sums, 15 tokens: less than a tile
+    (256, 2048, 1, 17),      # 32 partial sums, a tile and one token
+    (384, 1536, 2, 40),      # 24 partial sums, six warps; five tiles
+    (512, 1088, 2, 64),      # 17 partial sums; eight tiles, two for each CTA
+])
+def test_feed_forward_sublayer_in_one_kernel_follows_the_checker(d, ffn, batch, k):
+    test_few_token_passes_follow_the_checker(d, ffn, batch, k, 9, k + 8)
