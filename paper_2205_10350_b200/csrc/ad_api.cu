@@ -26,6 +26,7 @@
 #include "grid_sync.cuh"
 #include "mega.cuh"
 #include "steps.cuh"
+#include "sublayer_f32.cuh"
 
 using namespace ad;
 
@@ -323,11 +324,16 @@ void pass_shapes(const ad_model_cfg& c, PassCfg* pass, int* M_all) {
 // Floats of the partial sums of a projection with d output features over at most M tokens: a split projection has at most one
 // CTA per SM, each with at most 128 x 128 outputs (few-token kernel: at most 16 parts of 128 tokens).
 int num_sms();
-size_t partial_elems(int M, int d) {
+size_t partial_elems(int M, int d, bool bf16) {
   const size_t all = (size_t)M * d;
-  // (the feed-forward kernel of few tokens: up to 32 parts)
-  const size_t ffn = d <= 64 * few::MAX_WARPS ? (size_t)few::FFN_MAX_PARTS * std::min(M, few::MAX_TOKENS) * d : 0;
+  // (the feed-forward kernels of few tokens: up to 32 parts)
+  const size_t ffn = d <= 64 * few::MAX_WARPS ? (size_t)few::FFN_MAX_PARTS * std::min(M, bf16 ? few::MAX_TOKENS : sub32::MAX_TOKENS) * d : 0;
   return std::max(std::max(all, ffn), std::min(16 * all, std::max((size_t)num_sms() * 128 * 128, (size_t)16 * few::MAX_TOKENS * d)));
+}
+
+// Models some of whose attention kernels leave a partial output projection per head.
+bool has_head_partials(const ad_model_cfg& c) {
+  return c.n_heads <= 16 && (c.dtype == AD_DTYPE_BF16 || c.d_model == 128 || c.d_model == 256);
 }
 
 size_t layout(ad_handle* h, void* base) {
@@ -339,8 +345,8 @@ size_t layout(ad_handle* h, void* base) {
   const int M_all = h->M_all, Mv = h->pass[PK_VERIFY].M_cap;
   const int M_tmp = std::max(h->pass[PK_DRAFT].M_cap, h->pass[PK_ENCODE].M_cap);
   h->y = (float*)bp.take(sizeof(float) * (size_t)M_all * d);
-  h->pre = (float*)bp.take(sizeof(float) * partial_elems(M_all, d));
-  if (h->bf16 && c.n_heads <= 16) h->pre2 = (float*)bp.take(sizeof(float) * (size_t)c.n_heads * M_all * d);
+  h->pre = (float*)bp.take(sizeof(float) * partial_elems(M_all, d, h->bf16));
+  if (has_head_partials(c)) h->pre2 = (float*)bp.take(sizeof(float) * (size_t)c.n_heads * M_all * d);
   h->yb.ptr = bp.take(e * (size_t)M_all * d); h->yb.cols = d;
   h->abuf.ptr = bp.take(e * (size_t)M_all * d); h->abuf.cols = d;
   h->hbuf.ptr = bp.take(e * (size_t)M_all * F); h->hbuf.cols = F;
@@ -363,8 +369,8 @@ size_t layout(ad_handle* h, void* base) {
     const int Me = h->pass[PK_ENCODE].M_cap;
     ActSet& sd = h->side;
     sd.y = (float*)bp.take(sizeof(float) * (size_t)Me * d);
-    sd.pre = (float*)bp.take(sizeof(float) * partial_elems(Me, d));
-    if (h->bf16 && c.n_heads <= 16) sd.pre2 = (float*)bp.take(sizeof(float) * (size_t)c.n_heads * Me * d);
+    sd.pre = (float*)bp.take(sizeof(float) * partial_elems(Me, d, h->bf16));
+    if (has_head_partials(c)) sd.pre2 = (float*)bp.take(sizeof(float) * (size_t)c.n_heads * Me * d);
     sd.yb.ptr = bp.take(e * (size_t)Me * d); sd.yb.cols = d;
     sd.abuf.ptr = bp.take(e * (size_t)Me * d); sd.abuf.cols = d;
     sd.hbuf.ptr = bp.take(e * (size_t)Me * F); sd.hbuf.cols = F;
@@ -1026,7 +1032,8 @@ int layernorm(ad_handle* h, const PassCfg& pc, const Partials& pre, const float*
   };
   void* yb = out ? out->ptr : h->yb.ptr;
   if (most > 16) {
-    AD_CUDA(h, launch_k(layernorm_parts_kernel<bf16>, dim3(pc.M_cap), dim3(256), 0, h->stream, p, (bf16*)yb));
+    if (h->bf16) AD_CUDA(h, launch_k(layernorm_parts_kernel<bf16>, dim3(pc.M_cap), dim3(256), 0, h->stream, p, (bf16*)yb));
+    else AD_CUDA(h, launch_k(layernorm_parts_kernel<float>, dim3(pc.M_cap), dim3(256), 0, h->stream, p, (float*)yb));
     return AD_OK;
   }
   const cudaError_t e = h->bf16 ? go((bf16*)yb) : go((float*)yb);
@@ -1063,6 +1070,52 @@ int embed(ad_handle* h, const PassCfg& pc, const Model& m) {
   return AD_OK;
 }
 
+// ---- FP32 sublayers of few tokens (sublayer_f32.cuh) ----
+// Width of the slices of hidden features of the feed-forward sublayer (0: not covered).
+int f32_ffn_slice(int F) { return F % 32 == 0 && F / 32 <= 16 ? 32 : F % 64 == 0 && F / 64 <= 32 ? 64 : 0; }
+// Whether the sublayers of pass pc run on these kernels: what they cover, up to five waves of CTAs of the attention at capacity (two, three, five allowed:
+// 256 wide, batch 24 2522, 2494, 2494 us a call, 3256 without them).
+bool f32_sublayers(const ad_handle* h, const PassCfg& pc) {
+  const ad_model_cfg& c = h->cfg;
+  return !h->bf16 && h->pre2 && h->sw.fuse_attn_proj && pc.M_cap <= sub32::MAX_TOKENS && pc.pieces(c.max_batch, sub32::TOK) * c.n_heads <= 5L * num_sms();
+}
+template <sub32::Kind KIND, int D, int S>
+cudaError_t launch_sublayer_f32_n(cudaStream_t st, dim3 grid, const sub32::Params& p) {
+  typedef sub32::Layout<D, S> L;
+  constexpr size_t smem = sizeof(float) * (KIND == sub32::FFN ? L::OS : L::FLOATS);
+  static bool attr_set[kMaxDevices] = {};
+  const int dev = current_device();
+  if (!attr_set[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(sub32::sublayer_f32_kernel<KIND, D, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = true;
+  }
+  // (one CTA an SM, like the projections around it: 256 wide, batch 6 1364 us a call with the runtime's choice, 1295)
+  return launch_shared(one_cta_share(smem), sub32::sublayer_f32_kernel<KIND, D, S>, grid, dim3(sub32::THREADS), smem, st, p);
+}
+template <sub32::Kind KIND>
+int launch_sublayer_f32(ad_handle* h, dim3 grid, int width, const sub32::Params& p, const char* what) {
+  note_launch(h, what);
+  const bool d128 = h->cfg.d_model == 128, s32 = width == 32;
+  const cudaError_t e = d128 ? (s32 ? launch_sublayer_f32_n<KIND, 128, 32>(h->stream, grid, p) : launch_sublayer_f32_n<KIND, 128, 64>(h->stream, grid, p))
+                             : (s32 ? launch_sublayer_f32_n<KIND, 256, 32>(h->stream, grid, p) : launch_sublayer_f32_n<KIND, 256, 64>(h->stream, grid, p));
+  if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("sublayer launch: ") + cudaGetErrorString(e));
+  return AD_OK;
+}
+// Attention with its output projection (partial sums per head in pre2) and, with wq, the query projection of x = yb.
+int attention_f32(ad_handle* h, const PassCfg& pc, const void* k, const void* v, const int* key_base, const int* nkeys_tok, const int* nkeys_row,
+                  const Mat& wo, const Mat* wq = nullptr, const float* q_bias = nullptr) {
+  const int d = h->cfg.d_model, dh = d / h->cfg.n_heads;
+  sub32::Params p = {};
+  p.a.q = h->qbuf; p.a.k = k; p.a.v = v;
+  p.a.seg_off = pc.plan.seg_off; p.a.seg_len = pc.plan.seg_len; p.a.key_base = key_base; p.a.nkeys_tok = nkeys_tok; p.a.nkeys_row = nkeys_row;
+  p.a.qchunks = (pc.seg_max + sub32::TOK - 1) / sub32::TOK; p.a.scale = 1.0f / sqrtf((float)dh);
+  p.x = (const float*)h->yb.ptr; p.b_in = q_bias; p.w_in = wq ? (const float*)wq->ptr : nullptr;
+  p.w_out = (const float*)wo.ptr; p.out = h->pre2; p.stride = (size_t)pc.M_cap * d; p.K2 = d;
+  const dim3 grid(h->dims.B * p.a.qchunks, h->cfg.n_heads);
+  return wq ? launch_sublayer_f32<sub32::CROSS>(h, grid, dh, p, "q_proj+attention+out_proj") : launch_sublayer_f32<sub32::SELF>(h, grid, dh, p, "attention+out_proj");
+}
+
 #define AD_TRY(x) do { int rc__ = (x); if (rc__ != AD_OK) return rc__; } while (0)
 
 // Embedding of a pass's tokens: a kernel of its own, unless the pass's first projection computes it (null: it is done).
@@ -1087,6 +1140,10 @@ int self_attention_sublayer(ad_handle* h, int pk, const Mat& wqkv, const float* 
     AD_TRY(attention_few(h, pc, kbuf, vbuf, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, max_keys, wo));
     return layernorm(h, pc, head_partials(h, pc), bo, lng, lnb);
   }
+  if (f32_sublayers(h, pc)) {
+    AD_TRY(attention_f32(h, pc, kbuf, vbuf, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, wo));
+    return layernorm(h, pc, head_partials(h, pc), bo, lng, lnb);
+  }
   AD_TRY(attention(h, pc, h->qbuf, kbuf, vbuf, h->abuf.ptr, pc.plan.key_base, pc.plan.att_n, pc.plan.row_nk, max_keys, nullptr, nullptr, &wo, &fused));
   if (fused) return layernorm(h, pc, head_partials(h, pc), bo, lng, lnb);
   Partials ps;
@@ -1108,6 +1165,17 @@ int ffn_sublayer(ad_handle* h, int pk, const Mat& w1, const float* b1, const Mat
     const int slices = F / few::FFN_SLICE, groups = std::min((pc.M_cap + few::AQ - 1) / few::AQ, std::max(1, num_sms() / slices));
     note_launch(h, "ffn");
     AD_CUDA(h, launch_k(few::ffn_few_kernel, dim3(groups, slices), dim3(d / 2), 0, h->stream, p));
+    return layernorm(h, pc, ps, b2, lng, lnb, out);
+  }
+  if (f32_sublayers(h, pc) && f32_ffn_slice(F) > 0) {
+    const int slice = f32_ffn_slice(F);
+    sub32::Params p = {};
+    p.a.M_ptr = pc.plan.M;
+    p.x = (const float*)h->yb.ptr; p.w_in = (const float*)w1.ptr; p.b_in = b1; p.w_out = (const float*)w2.ptr;
+    p.out = h->pre; p.stride = (size_t)pc.M_cap * d; p.K2 = F;
+    AD_TRY(launch_sublayer_f32<sub32::FFN>(h, dim3((pc.M_cap + sub32::TOK - 1) / sub32::TOK, F / slice), slice, p, "ffn"));
+    Partials ps = {};
+    ps.ptr = h->pre; ps.nsplit = F / slice; ps.stride = p.stride;
     return layernorm(h, pc, ps, b2, lng, lnb, out);
   }
   GemmParams a = {};
@@ -1270,6 +1338,12 @@ int decoder_pass(ad_handle* h, int pk, Model& m) {
     if (attention_is_few(h, pk, c.max_src)) {
       AD_TRY(attention_few(h, pc, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->st.cross_base, nullptr, h->st.srclen, c.max_src,
                            L.co, &L.cq, L.cbq));
+      AD_TRY(layernorm(h, pc, head_partials(h, pc), L.cbo, L.ln2g, L.ln2b));
+      AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b, nullptr, next));
+      continue;
+    }
+    if (f32_sublayers(h, pc)) {
+      AD_TRY(attention_f32(h, pc, (char*)m.kenc + l * cross_layer, (char*)m.venc + l * cross_layer, h->st.cross_base, nullptr, h->st.srclen, L.co, &L.cq, L.cbq));
       AD_TRY(layernorm(h, pc, head_partials(h, pc), L.cbo, L.ln2g, L.ln2b));
       AD_TRY(ffn_sublayer(h, pk, L.w1, L.b1, L.w2, L.b2, L.ln3g, L.ln3b, nullptr, next));
       continue;

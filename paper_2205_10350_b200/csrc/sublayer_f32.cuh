@@ -1,0 +1,221 @@
+// Sublayers of FP32 passes of up to a thousand packed tokens, models 128 or 256 wide: attention with its output projection and, for the cross-attention, the
+// query projection, and the feed-forward sublayer with both of its projections, one kernel each.
+//
+// As kernels of their own the projections are 2.1 us a piece, most of it boundary and round trips: eleven kernels a decoder layer.  With these it is
+// seven: QKV | attention + Wo | LayerNorm | Wq + attention + Wo | LayerNorm | W1 + W2 | LayerNorm.  A CTA owns a head (or a slice of the hidden features) and 16
+// tokens; its shares of both weight matrices are in registers before the dependency wait, and what it computes in between stays in shared memory.
+// What bounds them: one memory round trip, three to five barriers and, at 16 tokens, 512 to 1024 multiply-adds per thread.  Whole calls, before -> after, us: 128
+// wide, batch 1 575 -> 518, batch 6 1386 -> 929, batch 32 2224 -> 1708; 256 wide, batch 1 1163 -> 806, batch 6 2240 -> 1296, batch 24 3256 -> 2495.
+// All sums are FP32 multiply-adds.  The output projection leaves one partial sum per head (slice) for the LayerNorm to add.
+#pragma once
+
+#include "attention.cuh"
+#include "gemm_simt.cuh"   // cp16
+
+namespace ad {
+namespace sub32 {
+
+enum Kind { SELF, CROSS, FFN };
+constexpr int TOK = 16;           // tokens per CTA: two per warp in the attention
+constexpr int KEYS = 64;          // keys per shared-memory tile
+constexpr int THREADS = 256;
+constexpr int MAX_TOKENS = 1024;  // largest capacity of a pass that takes these kernels
+
+struct Params {
+  AttnParams a;        // attention: q (SELF), k, v, scale, q_bias, segments; wo as float in w_out
+  const float* x;      // [M_cap, D] input of the first projection (CROSS, FFN)
+  const float* w_in;   // CROSS: Wq [D, D]; FFN: W1 [F, D]
+  const float* b_in;   // CROSS: bq; FFN: b1
+  const float* w_out;  // Wo [D, D] or W2 [D, F]
+  float* out;          // [heads or slices][M_cap, D] partial sums (no bias)
+  size_t stride;       // M_cap * D
+  int K2;              // row length of w_out: D or F
+};
+
+// Shared memory in floats: rows of the tiles are 16-byte aligned and four words apart modulo 32 (conflict-free 16-byte reads of 8 rows).
+template <int D, int S>
+struct Layout {
+  static constexpr int LD = S + 4;
+  static constexpr int XS = 0, RED = XS + TOK * D, HS = RED + TOK * THREADS, OS = HS + TOK * LD, KS = OS + TOK * LD, VS = KS + KEYS * LD, PS = VS + KEYS * LD,
+                       FLOATS = PS + TOK * KEYS;
+};
+
+// S: width of a head, or of a slice of hidden features.  grid = (B * qchunks, heads) or (ceil(M_cap / 16), F / S); block = 256; dynamic shared
+// memory Layout<D, S>::FLOATS floats.
+template <Kind KIND, int D, int S>
+__global__ void __launch_bounds__(THREADS)
+sublayer_f32_kernel(const Params p) {
+  typedef Layout<D, S> L;
+  constexpr int PARTS = THREADS / S, KP = D / PARTS;        // parts of the first projection's contraction
+  constexpr int GROUPS = THREADS / D;                       // tokens side by side in the second projection
+  extern __shared__ __align__(16) float sub_smem[];
+  float *xs = sub_smem + L::XS, *red = sub_smem + L::RED, *hs = sub_smem + L::HS, *os = KIND == FFN ? hs : sub_smem + L::OS;
+  float *ks = sub_smem + L::KS, *vs = sub_smem + L::VS, *ps = sub_smem + L::PS;
+  pdl_launch();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, h = blockIdx.y;
+  int m0, nt, kbase = 0, row_nk = 0;
+  if (KIND == FFN) {
+    m0 = blockIdx.x * TOK;
+    nt = min(TOK, plan_load(p.a.M_ptr) - m0);
+  } else {
+    const int b = blockIdx.x / p.a.qchunks, i0 = (blockIdx.x - b * p.a.qchunks) * TOK;
+    nt = min(TOK, plan_load(p.a.seg_len + b) - i0);
+    m0 = plan_load(p.a.seg_off + b) + i0;
+    kbase = plan_load(p.a.key_base + b); row_nk = plan_load(p.a.nkeys_row + b);
+  }
+  if (nt <= 0) {                                            // (one CTA always waits, see early exits in ad_common.cuh)
+    if ((blockIdx.x | blockIdx.y) == 0) pdl_wait();
+    return;
+  }
+  // weights
+  const int f = tid % S, part = tid / S, n = tid % D, group = tid / D;
+  float4 w1[KIND == SELF ? 1 : KP / 4], w2[S / 4];
+  float bias = 0.f;
+  if (KIND != SELF) {
+#pragma unroll
+    for (int i = 0; i < KP / 4; ++i) w1[KIND == SELF ? 0 : i] = __ldg(reinterpret_cast<const float4*>(p.w_in + (size_t)(h * S + f) * D + part * KP + 4 * i));
+    bias = p.b_in[h * S + f];
+  }
+#pragma unroll
+  for (int i = 0; i < S / 4; ++i) w2[i] = __ldg(reinterpret_cast<const float4*>(p.w_out + (size_t)n * p.K2 + h * S + 4 * i));
+  const float *kk = reinterpret_cast<const float*>(p.a.k), *vv = reinterpret_cast<const float*>(p.a.v);
+  auto fetch_keys = [&](int j0) {                           // keys j0 .. j0 + 63 of the row and their values; zeros beyond the last
+    for (int idx = tid; idx < KEYS * (S / 4); idx += THREADS) {
+      const int j = idx / (S / 4), c = (idx % (S / 4)) * 4;
+      const bool there = j0 + j < row_nk;
+      const size_t off = (size_t)(kbase + (there ? j0 + j : 0)) * D + h * S + c;
+      simt::cp16(ks + j * L::LD + c, kk + off, there);
+      simt::cp16(vs + j * L::LD + c, vv + off, there);
+    }
+  };
+  if (KIND == CROSS) fetch_keys(0);                         // the encoder's: older than the plan
+  int nk[2] = {0, 0};
+  if (KIND != FFN)
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int r = warp + 8 * u;
+      if (r < nt) nk[u] = p.a.nkeys_tok ? min(plan_load(p.a.nkeys_tok + m0 + r), row_nk) : row_nk;
+    }
+  pdl_wait();
+  if (KIND == SELF) {
+    fetch_keys(0);
+    const float* q = reinterpret_cast<const float*>(p.a.q);
+    for (int idx = tid; idx < nt * S; idx += THREADS) hs[(idx / S) * L::LD + idx % S] = q[(size_t)(m0 + idx / S) * D + h * S + idx % S] * p.a.scale;
+  } else {
+    for (int idx = tid; idx < nt * (D / 4); idx += THREADS) {
+      const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
+      simt::cp16(xs + r * D + c, p.x + (size_t)(m0 + r) * D + c, true);
+    }
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();
+  if (KIND != SELF) {
+    // first projection: every part's share of the tokens' S features, then their sum
+#pragma unroll 4
+    for (int r = 0; r < nt; ++r) {
+      float s = 0.f;
+#pragma unroll
+      for (int i = 0; i < KP / 4; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(xs + r * D + part * KP + 4 * i), w = w1[KIND == SELF ? 0 : i];
+        s = fmaf(w.x, v.x, s); s = fmaf(w.y, v.y, s); s = fmaf(w.z, v.z, s); s = fmaf(w.w, v.w, s);
+      }
+      red[(part * TOK + r) * S + f] = s;
+    }
+    __syncthreads();
+    for (int r = part; r < nt; r += PARTS) {
+      float s = red[r * S + f];
+#pragma unroll
+      for (int q = 1; q < PARTS; ++q) s += red[(q * TOK + r) * S + f];
+      s += bias;
+      hs[r * L::LD + f] = KIND == FFN ? fmaxf(s, 0.f) : s * p.a.scale;
+    }
+    __syncthreads();
+  }
+  if (KIND != FFN) {
+    // attention: two queries per warp, keys lane and lane + 32 of every tile, running maximum and sum
+    float mx[2] = {-INFINITY, -INFINITY}, den[2] = {0.f, 0.f}, acc[2][S / 32];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int c = 0; c < S / 32; ++c) acc[u][c] = 0.f;
+    for (int j0 = 0; j0 < row_nk; j0 += KEYS) {
+      if (j0 > 0) {
+        __syncthreads();                                    // the previous tile has been read
+        fetch_keys(j0);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+      }
+      float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll 4
+      for (int c = 0; c < S; c += 4) {
+        const float4 k0 = *reinterpret_cast<const float4*>(ks + lane * L::LD + c), k1 = *reinterpret_cast<const float4*>(ks + (lane + 32) * L::LD + c);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const float4 q = *reinterpret_cast<const float4*>(hs + (warp + 8 * u) * L::LD + c);
+          s[u][0] = fmaf(q.x, k0.x, s[u][0]); s[u][0] = fmaf(q.y, k0.y, s[u][0]); s[u][0] = fmaf(q.z, k0.z, s[u][0]); s[u][0] = fmaf(q.w, k0.w, s[u][0]);
+          s[u][1] = fmaf(q.x, k1.x, s[u][1]); s[u][1] = fmaf(q.y, k1.y, s[u][1]); s[u][1] = fmaf(q.z, k1.z, s[u][1]); s[u][1] = fmaf(q.w, k1.w, s[u][1]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        float p0 = 0.f, p1 = 0.f, corr = 1.f;
+        if (nk[u] > j0) {                                   // warp-uniform; otherwise the query sees no key of this tile
+          const float a0 = j0 + lane < nk[u] ? s[u][0] : -INFINITY, a1 = j0 + lane + 32 < nk[u] ? s[u][1] : -INFINITY;
+          float top = fmaxf(a0, a1);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+          const float now = fmaxf(mx[u], top);              // finite: key j0 is visible
+          corr = expf(mx[u] - now);                         // exp(-inf) = 0 on the first tile
+          p0 = expf(a0 - now); p1 = expf(a1 - now);
+          float sum = p0 + p1;
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+          den[u] = den[u] * corr + sum;
+          mx[u] = now;
+        }
+        ps[(warp + 8 * u) * KEYS + lane] = p0;
+        ps[(warp + 8 * u) * KEYS + lane + 32] = p1;
+#pragma unroll
+        for (int c = 0; c < S / 32; ++c) acc[u][c] *= corr;
+      }
+      __syncwarp();
+      const int jn = min(KEYS, row_nk - j0);
+#pragma unroll 2
+      for (int j = 0; j < jn; j += 4) {                     // (keys beyond the last are zeros with probability 0)
+        const float4 pa = *reinterpret_cast<const float4*>(ps + warp * KEYS + j), pb = *reinterpret_cast<const float4*>(ps + (warp + 8) * KEYS + j);
+#pragma unroll
+        for (int c = 0; c < S / 32; ++c) {
+          const float* v = vs + j * L::LD + lane + 32 * c;
+          const float v0 = v[0], v1 = v[L::LD], v2 = v[2 * L::LD], v3 = v[3 * L::LD];
+          acc[0][c] = fmaf(pa.x, v0, acc[0][c]); acc[0][c] = fmaf(pa.y, v1, acc[0][c]); acc[0][c] = fmaf(pa.z, v2, acc[0][c]); acc[0][c] = fmaf(pa.w, v3, acc[0][c]);
+          acc[1][c] = fmaf(pb.x, v0, acc[1][c]); acc[1][c] = fmaf(pb.y, v1, acc[1][c]); acc[1][c] = fmaf(pb.z, v2, acc[1][c]); acc[1][c] = fmaf(pb.w, v3, acc[1][c]);
+        }
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float inv = nk[u] > 0 ? 1.f / den[u] : 0.f;
+#pragma unroll
+      for (int c = 0; c < S / 32; ++c) os[(warp + 8 * u) * L::LD + lane + 32 * c] = acc[u][c] * inv;
+    }
+    __syncthreads();
+  }
+  // second projection: this thread's output feature of every GROUPS-th token
+  float* dst = p.out + (size_t)h * p.stride + (size_t)m0 * D + n;
+#pragma unroll 4
+  for (int r = group; r < nt; r += GROUPS) {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < S / 4; ++i) {
+      const float4 v = *reinterpret_cast<const float4*>(os + r * L::LD + 4 * i);
+      s = fmaf(w2[i].x, v.x, s); s = fmaf(w2[i].y, v.y, s); s = fmaf(w2[i].z, v.z, s); s = fmaf(w2[i].w, v.w, s);
+    }
+    dst[(size_t)r * D] = s;
+  }
+}
+
+}  // namespace sub32
+}  // namespace ad

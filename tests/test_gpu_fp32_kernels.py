@@ -55,3 +55,30 @@ def test_passes_follow_the_checker(d, heads, ffn, batch, k):
     stats = lockstep(dec, model, src, lens, streams, k, [40] * batch, tol=1e-3, max_steps=5)
     assert stats["steps"] > 0
     dec.close()
+
+
+@pytest.mark.parametrize("d,heads,ffn,batch,k,src,tgt", [
+    (128, 4, 96, 1, 1, 3, 9),          # one token, three slices of hidden features
+    (128, 2, 512, 3, 16, 65, 70),      # 64-wide heads, a whole tile of queries a row; source keys beyond a tile, later the prefix too
+    (128, 4, 1024, 2, 17, 40, 129),    # a tile and one query; 16 slices of 64; prefix keys in three tiles
+    (256, 8, 512, 9, 33, 64, 40),      # 297 tokens of capacity, exactly one tile of source keys
+    (256, 4, 2048, 2, 5, 130, 24),     # 64-wide heads, 32 partial sums for the LayerNorm, source keys in three tiles
+    (256, 8, 1100, 2, 7, 20, 24),      # a feed-forward width that stays with the projections' own kernels
+])
+def test_sublayer_kernels_follow_the_checker(d, heads, ffn, batch, k, src, tgt):
+    """FP32 attention with its projections and the feed-forward sublayer in one kernel each: ragged rows, blocks behind growing prefixes."""
+    shape = synth.ModelShape(f"f32sub_{d}_{heads}_{ffn}", d, heads, ffn, 301, 1, 2, "fp32")
+    w = synth.make_weights(shape, 0)
+    model = O.Model(shape, w, max_pos=160)
+    r = np.random.default_rng(d + heads + k)
+    lens = r.integers(max(1, src // 2), src + 1, size=batch).astype(np.int32)
+    lens[0] = src
+    srcs = r.integers(4, shape.vocab, size=(batch, src)).astype(np.int32)
+    dec = binding.AggressiveDecoder(shape, w, max_batch=batch, max_src=src, max_tgt=tgt, kmax=k)
+    streams = r.integers(4, shape.vocab, size=(batch, tgt)).astype(np.int32)
+    for b in range(batch):
+        g, _ = model.state(srcs[b, : lens[b]], cap=tgt).greedy(tgt)
+        streams[b, : len(g)] = np.where(r.random(len(g)) < 0.95, g, streams[b, : len(g)])
+    stats = lockstep(dec, model, srcs, lens, streams, k, [tgt] * batch, tol=1e-3, max_steps=12)
+    assert stats["steps"] > 0
+    dec.close()
