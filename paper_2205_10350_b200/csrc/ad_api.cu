@@ -327,7 +327,8 @@ int num_sms();
 size_t partial_elems(int M, int d, bool bf16) {
   const size_t all = (size_t)M * d;
   // (the feed-forward kernels of few tokens: up to 32 parts)
-  const size_t ffn = d <= 64 * few::MAX_WARPS ? (size_t)few::FFN_MAX_PARTS * std::min(M, bf16 ? few::MAX_TOKENS : sub32::MAX_TOKENS) * d : 0;
+  const size_t rows = bf16 ? std::min(few::FFN_MAX_PARTS * (size_t)M, (size_t)few::FFN_MAX_ROWS) : few::FFN_MAX_PARTS * (size_t)std::min(M, sub32::MAX_TOKENS);
+  const size_t ffn = d <= 64 * few::MAX_WARPS ? rows * d : 0;
   return std::max(std::max(all, ffn), std::min(16 * all, std::max((size_t)num_sms() * 128 * 128, (size_t)16 * few::MAX_TOKENS * d)));
 }
 
@@ -1155,10 +1156,11 @@ int ffn_sublayer(ad_handle* h, int pk, const Mat& w1, const float* b1, const Mat
                  const float* lnb, const ActBuf* out = nullptr, const Prefetch& next = {}) {
   PassCfg& pc = h->pass[pk];
   const int d = h->cfg.d_model, F = h->cfg.d_ffn;
-  // Passes that are always of few tokens, up to 512 wide: both projections in one kernel (wider models would bring 48 partial sums and more).  Whole
+  // Passes of few tokens, up to 512 wide: both projections in one kernel (wider models would bring 48 partial sums and more).  Whole
   // calls, two kernels -> this: 512 wide, batch 1 1201 -> 1168 us, batch 16 token by token 4880 -> 4742, batch 3, relaxed, 75 tokens 1597 -> 1535, batch 2 with
-  // drafter 2689 -> 2605; encoder calls of four layers, 1 x 64 tokens 92 -> 85, 2 x 50 112 -> 100, 4 x 32 117 -> 103; 256 wide, 2 x 60 100 -> 80.
-  if (h->bf16 && few::ffn_few_fits(d, F) && pc.M_cap <= pc.few_cap) {
+  // drafter 2689 -> 2605; encoder calls of four layers, 1 x 64 tokens 92 -> 85, 2 x 50 112 -> 100, 4 x 32 117 -> 103, 1 x 140 112 -> 109, 1 x 200 118 -> 122; 256 wide (16
+  // partial sums) 2 x 60 100 -> 80, 4 x 60 104 -> 92.
+  if (h->bf16 && few::ffn_few_fits(d, F, pc.M_cap)) {
     const few::FfnFewParams p = {pc.plan.M, (const bf16*)h->yb.ptr, (const bf16*)w1.ptr, (const bf16*)w2.ptr, b1, h->pre, (size_t)pc.M_cap * d, d, F};
     Partials ps = {};
     ps.ptr = h->pre; ps.nsplit = F / few::FFN_SLICE; ps.stride = p.stride;

@@ -17,7 +17,10 @@ namespace few {
 
 constexpr int FFN_SLICE = 64;            // hidden features per CTA
 constexpr int FFN_MAX_PARTS = 32;
-inline bool ffn_few_fits(int d, int F) { return d % 128 == 0 && d <= 64 * MAX_WARPS && F % FFN_SLICE == 0 && F / FFN_SLICE <= FFN_MAX_PARTS; }
+constexpr int FFN_MAX_ROWS = 160 * 32;   // most rows of partial sums: what the LayerNorm has to read outgrows the kernel that was saved
+inline bool ffn_few_fits(int d, int F, int M_cap) {
+  return d % 128 == 0 && d <= 64 * MAX_WARPS && F % FFN_SLICE == 0 && F / FFN_SLICE <= FFN_MAX_PARTS && (long)M_cap * (F / FFN_SLICE) <= FFN_MAX_ROWS;
+}
 
 struct FfnFewParams {
   const int* M_ptr;
