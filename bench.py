@@ -80,8 +80,8 @@ def reduce_max_sum(dist, dev, seconds_or_ms, count):
 # DRAM counters of one verification step (dram__bytes_read.sum + dram__bytes_write.sum summed over the step's
 # kernels, ncu, caches flushed before every kernel) with the digest of the kernel sources they were taken on:
 # the figures are reported only while the sources still have that digest.
-NCU_COUNTERS = dict(sources_sha256="ff6c87ba9bd82031411d5a2cbc3261707e3b9060e8f308fdf8da8da760bda6b5",
-                    step_block40_bytes=92147456, projection_bytes=32865024,
+NCU_COUNTERS = dict(sources_sha256="3edca787c6f90918e863d1d9b9fb98ca6079f7ac1435daa2e86755136dcf4c49",
+                    step_block40_bytes=104927488, projection_bytes=32865024,
                     summary="profiles/verify_step_base_b1_k40_dram_traffic.txt")
 
 
@@ -478,7 +478,7 @@ def run_ours(args, rank, world, local_rank):
     alg = step_bytes(synth.BASE, sum_src=mean_S * iters, sum_keys=float(glen.mean()) * iters, sum_k=agg["offered"], n_steps=iters) / iters
     ach = alg / (loop_us * 1e-6) / 1e9
     wv = weight_bytes(synth.BASE)
-    roofline = dict(bound="hbm", kernel="verification step: the 50-kernel chain of one loop iteration (6 decoder layers of 8 kernels, "
+    roofline = dict(bound="hbm", kernel="verification step: the 44-kernel chain of one loop iteration (6 decoder layers of 7 kernels, "
                     "projection + arg-max, accept + commit + plan of the next block), graph-replayed", achieved=ach, peak=pk["hbm_gbs"], unit="GB/s",
                     frac=ach / pk["hbm_gbs"], traffic=ncu_counter("step_block40_bytes"), peak_source=pk["source"], algorithmic_bytes=alg,
                     weight_bytes=wv, us_per_step_in_loop=loop_us, hbm_floor_us=alg / (pk["hbm_gbs"] * 1e9) * 1e6,
