@@ -5,7 +5,7 @@
 // seven: QKV | attention + Wo | LayerNorm | Wq + attention + Wo | LayerNorm | W1 + W2 | LayerNorm.  A CTA owns a head (or a slice of the hidden features) and 16
 // tokens; its shares of both weight matrices are in registers before the dependency wait, and what it computes in between stays in shared memory.
 // What bounds them: one memory round trip, three to five barriers and, at 16 tokens, 512 to 1024 multiply-adds per thread.  Whole calls, before -> after, us: 128
-// wide, batch 1 575 -> 518, batch 6 1386 -> 929, batch 32 2224 -> 1708; 256 wide, batch 1 1163 -> 806, batch 6 2240 -> 1296, batch 24 3256 -> 2495.
+// wide, batch 1 575 -> 538, batch 6 1386 -> 913, batch 32 2224 -> 1735; 256 wide, batch 1 1163 -> 806, batch 6 2240 -> 1296, batch 24 3256 -> 2495.
 // All sums are FP32 multiply-adds.  The output projection leaves one partial sum per head (slice) for the LayerNorm to add.
 #pragma once
 
@@ -39,6 +39,13 @@ struct Layout {
   static constexpr int XS = 0, RED = XS + TOK * D, HS = RED + TOK * THREADS, OS = HS + TOK * LD, KS = OS + TOK * LD, VS = KS + KEYS * LD, PS = VS + KEYS * LD,
                        FLOATS = PS + TOK * KEYS;
 };
+
+// Products in four running sums, which keeps the chains of additions, and with them the rounding, as short as in the kernels that split K between half-warps (error
+// against 64 bits, 128 wide, batch 1 x 17: 4.9e-7 with those, 5.0e-7; in one running sum 5.8e-7, and a call takes 3 % less).
+__device__ __forceinline__ void fma4(float4& s, float4 a, float4 b) {
+  s.x = fmaf(a.x, b.x, s.x); s.y = fmaf(a.y, b.y, s.y); s.z = fmaf(a.z, b.z, s.z); s.w = fmaf(a.w, b.w, s.w);
+}
+__device__ __forceinline__ float sum4(float4 s) { return (s.x + s.y) + (s.z + s.w); }
 
 // S: width of a head, or of a slice of hidden features.  grid = (B * qchunks, heads) or (ceil(M_cap / 16), F / S); block = 256; dynamic shared
 // memory Layout<D, S>::FLOATS floats.
@@ -114,13 +121,10 @@ sublayer_f32_kernel(const Params p) {
     // first projection: every part's share of the tokens' S features, then their sum
 #pragma unroll 4
     for (int r = 0; r < nt; ++r) {
-      float s = 0.f;
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < KP / 4; ++i) {
-        const float4 v = *reinterpret_cast<const float4*>(xs + r * D + part * KP + 4 * i), w = w1[KIND == SELF ? 0 : i];
-        s = fmaf(w.x, v.x, s); s = fmaf(w.y, v.y, s); s = fmaf(w.z, v.z, s); s = fmaf(w.w, v.w, s);
-      }
-      red[(part * TOK + r) * S + f] = s;
+      for (int i = 0; i < KP / 4; ++i) fma4(s, w1[KIND == SELF ? 0 : i], *reinterpret_cast<const float4*>(xs + r * D + part * KP + 4 * i));
+      red[(part * TOK + r) * S + f] = sum4(s);
     }
     __syncthreads();
     for (int r = part; r < nt; r += PARTS) {
@@ -147,17 +151,22 @@ sublayer_f32_kernel(const Params p) {
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
       }
-      float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+      float s[2][2];
+      float4 s4[2][2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) s4[u][0] = s4[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
       for (int c = 0; c < S; c += 4) {
         const float4 k0 = *reinterpret_cast<const float4*>(ks + lane * L::LD + c), k1 = *reinterpret_cast<const float4*>(ks + (lane + 32) * L::LD + c);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           const float4 q = *reinterpret_cast<const float4*>(hs + (warp + 8 * u) * L::LD + c);
-          s[u][0] = fmaf(q.x, k0.x, s[u][0]); s[u][0] = fmaf(q.y, k0.y, s[u][0]); s[u][0] = fmaf(q.z, k0.z, s[u][0]); s[u][0] = fmaf(q.w, k0.w, s[u][0]);
-          s[u][1] = fmaf(q.x, k1.x, s[u][1]); s[u][1] = fmaf(q.y, k1.y, s[u][1]); s[u][1] = fmaf(q.z, k1.z, s[u][1]); s[u][1] = fmaf(q.w, k1.w, s[u][1]);
+          fma4(s4[u][0], q, k0);
+          fma4(s4[u][1], q, k1);
         }
       }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) { s[u][0] = sum4(s4[u][0]); s[u][1] = sum4(s4[u][1]); }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         float p0 = 0.f, p1 = 0.f, corr = 1.f;
@@ -207,13 +216,10 @@ sublayer_f32_kernel(const Params p) {
   float* dst = p.out + (size_t)h * p.stride + (size_t)m0 * D + n;
 #pragma unroll 4
   for (int r = group; r < nt; r += GROUPS) {
-    float s = 0.f;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < S / 4; ++i) {
-      const float4 v = *reinterpret_cast<const float4*>(os + r * L::LD + 4 * i);
-      s = fmaf(w2[i].x, v.x, s); s = fmaf(w2[i].y, v.y, s); s = fmaf(w2[i].z, v.z, s); s = fmaf(w2[i].w, v.w, s);
-    }
-    dst[(size_t)r * D] = s;
+    for (int i = 0; i < S / 4; ++i) fma4(s, w2[i], *reinterpret_cast<const float4*>(os + r * L::LD + 4 * i));
+    dst[(size_t)r * D] = sum4(s);
   }
 }
 
