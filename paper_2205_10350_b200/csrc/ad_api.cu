@@ -84,7 +84,8 @@ struct PassCfg {
   int ntile = 16;    // tokens per GEMM tile
   int seg_max = 0;   // longest segment of one row
   int max_split = 1; // largest split-K factor this pass may use (sizes the partial-sum buffer)
-  int few_cap = few::MAX_TOKENS;   // capacities up to which every pass runs its projections on the few-token kernels
+  int few_cap = few::MAX_TOKENS;   // capacities up to which every pass runs its projections on the few-token kernels; 0: one of several layouts, picked
+                                   // by the tokens that are there, and not the first (see LoopBodies)
   PassPlan plan;
   // Most pieces of up to q tokens of one row that a pass over `rows` rows can have.
   long pieces(int rows, int q) const { return std::min((long)rows * ((seg_max + q - 1) / q), (long)std::min(rows, M_cap) + M_cap / q); }
@@ -822,6 +823,11 @@ cudaError_t launch_attention(dim3 grid, dim3 block, cudaStream_t st, const AttnP
   return launch_shared(share, attention_kernel<T, D, Q, FUSE, MINB>, grid, block, smem, st, p);
 }
 
+// Whether a pass of a model up to 512 wide has, at its capacity, work for at most three waves of the few-query kernel's CTAs (attention_few.cuh).
+bool within_three_waves(const ad_handle* h, const PassCfg& pc) {
+  return few::att_few_split(h->cfg.d_model) == 1 && pc.pieces(h->cfg.max_batch, few::AQ) * h->cfg.n_heads <= 3L * num_sms();
+}
+
 int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, const void* v, void* out,
               const int* key_base, const int* nkeys_tok, const int* nkeys_row, int max_keys,
               const float* q_bias = nullptr, const Partials* q_part = nullptr, const Mat* wo = nullptr, bool* fused = nullptr, bool kv_old = false) {
@@ -848,7 +854,8 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
     // What the FFMA kernel would do with FP32 probabilities keeps them (two BF16 numbers each; 0 to 5 us of such a call more than with one):
     // memory of one layer dominated by its attention, 27 sizes of 256 to 1024 wide: error against 64 bits within 0.03 % of the FFMA kernel's,
     // 0.3 to 1.8 % above it with probabilities rounded to BF16.
-    const bool split_p = !many && max_keys < 256;
+    // So do verification passes that the few-query kernel takes where their tokens are not known (see attention_is_few).
+    const bool split_p = (!many || (&pc == &h->pass[PK_VERIFY] && within_three_waves(h, pc))) && max_keys < 256;
     // Warps share a 16-query tile and split the keys (2 or 4 key groups) when rows have few queries; two groups also while
     // 64-query CTAs would not give every SM two.
     const long full = (long)h->dims.B * ((pc.seg_max + AM_Q - 1) / AM_Q) * c.n_heads;
@@ -920,13 +927,18 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
 // Whether the few-query kernel (attention_few.cuh) serves an attention of pass pk: BF16, 64-wide heads, the keys within four rounds
 // of its warps, and work for a few waves of CTAs at most, counted by what the pass could hold (rows that have ended, shorter blocks and a
 // drafter's prefix that has not grown leave less).  A wave costs 4 to 7 us, the projections that
-// are kernels of their own otherwise 12 us a layer, so a verification pass may need two and a half waves at capacity (three where CTAs do not loop,
-// four beyond 512 wide), a drafter's pass (on average half of its capacity) four.  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30:
+// are kernels of their own otherwise 12 us a layer, so a verification pass may need three waves at capacity (four beyond 512 wide), a drafter's pass (on
+// average half of its capacity) four.  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30:
 // 214 -> 174 us; batch 24, 12: 237 -> 196; batch 20, 1: 188 -> 160; batch of 5 with drafter 442 -> 373; 1024 wide, batch 2, 40: 272 -> 226;
 // batch 3 with drafter 662 -> 600.  Beyond: base batch 32 x 64 (seven waves) 270 -> 315, 1024 wide batch 16 x 1 (four) 239 -> 284.  Wide
 // models with fewer than eight queries a row stay at one wave: their CTAs read two weight slices each for a tile that is mostly padding
 // (768 wide, batch 12, 1: 202 against 210).  Looping grids, waves 2 / 2.5 / 3 / 3.5 / 4 / 4.5, whole calls: 512 wide, batch 20 5068 / 5046 / 5073 / 5147 / 5350 / 5443,
 // batch 16, relaxed 2379 / 2375 / 2482 / 2483 / 2481 / 2480; from 3 on, 1024 wide, batch 8 5350 / 4873 / 5028 / 5078, 768 wide, batch 16 4786 / 4781 / 4409 / 4479.
+// Layouts that the tokens pick hold as many as they are made for, and with 384 and 512 wide models two and a half waves are the line there; the MMA kernel
+// beyond keeps FP32's probabilities up to three waves, as this one does (split_p in attention).  It does so for fewer than 256 keys, with more the line stays at three waves.
+// A layout that has to hold whatever comes (device arrays) is mostly emptier than its capacity: verified blocks, two and a half waves for it as well -> three, 512 wide,
+// rows x tokens of a capacity of 12 x 64: 12 x 4 218 -> 181 us, 12 x 20 262 -> 256, 12 x 45 319 -> 305, 12 x 64 330 -> 355.  Whole calls, probabilities rounded to BF16 in that
+// band -> not: 512 wide, relaxed, 12 x 64 2007 -> 2015, 16 x 40 2001 -> 2029, 24 x 30 2492 -> 2504, 300 source tokens, 12 x 60 (three waves) 2327 -> 2375.
 // An encoder's rows are as long as they are announced, and there is one projection to gain: one and a half.  Calls of four layers, 512 wide,
 // kernel without it -> with it, us: 3 x 112 tokens 143 -> 137, 4 x 96 143 -> 134, 5 x 75 144 -> 137, 8 x 48 140 -> 132, 24 x 16 139 -> 131.  One wave
 // beyond 512 wide (768 wide 2 x 90 147 -> 156, 3 x 64 147 -> 152), for rows of at most eight (512 wide 24 x 8 116 -> 118, 24 x 4 122 -> 125; 256 wide
@@ -939,7 +951,8 @@ bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   if (max_keys > few::MAX_ROUNDS * few::AK * few::att_few_warps(c.d_model)) return false;
   // (in half waves)
   const bool one_wave = pk == PK_ENCODE ? split > 1 || max_keys >= 256 || (pc.seg_max <= 8 && c.d_model > 256) : split > 1 && pc.seg_max < 8;
-  const int waves = one_wave ? 2 : pk == PK_ENCODE ? 3 : pk == PK_DRAFT || split > 1 ? 8 : few::att_few_warps(c.d_model) > 4 ? 5 : 6;
+  const bool half_less = pc.few_cap == 0 && few::att_few_warps(c.d_model) > 4 && std::max(c.max_src, c.max_tgt) < 256;
+  const int waves = one_wave ? 2 : pk == PK_ENCODE ? 3 : pk == PK_DRAFT || split > 1 ? 8 : half_less ? 5 : 6;
   return 2 * pc.pieces(c.max_batch, few::AQ) * c.n_heads * split <= (long)waves * num_sms();
 }
 
@@ -1514,13 +1527,13 @@ LoopBodies loop_bodies(ad_handle* h, bool policy) {
   if (full <= (policy ? kFewTokens : 96)) return b;
   b.n = 0;
   b.cap[b.n++] = few;
-  if (!attention_is_few(h, PK_VERIFY, h->cfg.max_src)) {
+  auto takes_few = [&](int cap) {
+    const PassLayout at(h, PK_VERIFY, cap, 0);
+    return attention_is_few(h, PK_VERIFY, h->cfg.max_src);
+  };
+  if (!takes_few(full)) {
     int cap = few;
-    for (int c = few + 16; c < full; c += 16) {
-      const PassLayout at(h, PK_VERIFY, c, 0);
-      if (!attention_is_few(h, PK_VERIFY, h->cfg.max_src)) break;
-      cap = c;
-    }
+    while (cap + 16 < full && takes_few(cap + 16)) cap += 16;
     if (cap > few) b.cap[b.n++] = cap;
   }
   b.cap[b.n++] = full;
