@@ -322,20 +322,33 @@ void pass_shapes(const ad_model_cfg& c, PassCfg* pass, int* M_all) {
   *M_all = all;
 }
 
+// FP32 sublayers of few tokens (sublayer_f32.cuh): the model widths they are built for, and the width of their slices of hidden features of the feed-forward
+// sublayer (0: not covered).
+bool f32_sublayer_width(int d) { return d == 128 || d == 256; }
+int f32_ffn_slice(int F) { return F % 32 == 0 && F / 32 <= 16 ? 32 : F % 64 == 0 && F / 64 <= 32 ? 64 : 0; }
+
 // Floats of the partial sums of a projection with d output features over at most M tokens: a split projection has at most one
 // CTA per SM, each with at most 128 x 128 outputs (few-token kernel: at most 16 parts of 128 tokens).
 int num_sms();
-size_t partial_elems(int M, int d, bool bf16) {
+size_t partial_elems(const ad_model_cfg& c, int M) {
+  const int d = c.d_model;
   const size_t all = (size_t)M * d;
-  // (the feed-forward kernels of few tokens: up to 32 parts)
-  const size_t rows = bf16 ? std::min(few::FFN_MAX_PARTS * (size_t)M, (size_t)few::FFN_MAX_ROWS) : few::FFN_MAX_PARTS * (size_t)std::min(M, sub32::MAX_TOKENS);
-  const size_t ffn = d <= 64 * few::MAX_WARPS ? rows * d : 0;
+  // the feed-forward kernels of few tokens: a part per slice of hidden features
+  size_t ffn = 0;
+  if (c.dtype != AD_DTYPE_BF16) {
+    if (f32_sublayer_width(d) && f32_ffn_slice(c.d_ffn) > 0) ffn = (size_t)(c.d_ffn / f32_ffn_slice(c.d_ffn)) * std::min(M, sub32::MAX_TOKENS) * d;
+  } else if (few::ffn_few_fits(d, c.d_ffn, 1)) {
+    ffn = std::min((size_t)(c.d_ffn / few::FFN_SLICE) * M, (size_t)few::FFN_MAX_ROWS) * d;
+  }
   return std::max(std::max(all, ffn), std::min(16 * all, std::max((size_t)num_sms() * 128 * 128, (size_t)16 * few::MAX_TOKENS * d)));
 }
 
-// Models some of whose attention kernels leave a partial output projection per head.
-bool has_head_partials(const ad_model_cfg& c) {
-  return c.n_heads <= 16 && (c.dtype == AD_DTYPE_BF16 || c.d_model == 128 || c.d_model == 256);
+// Floats of the partial output projections, one per head, that some attention kernels leave (0: none of this model does).  The FP32 ones stop at
+// sub32::MAX_TOKENS tokens, whatever the handle can hold.
+size_t head_partial_elems(const ad_model_cfg& c, int M) {
+  if (c.n_heads > 16) return 0;
+  const size_t row = (size_t)c.n_heads * c.d_model;
+  return c.dtype == AD_DTYPE_BF16 ? row * M : f32_sublayer_width(c.d_model) ? row * std::min(M, sub32::MAX_TOKENS) : 0;
 }
 
 size_t layout(ad_handle* h, void* base) {
@@ -347,8 +360,8 @@ size_t layout(ad_handle* h, void* base) {
   const int M_all = h->M_all, Mv = h->pass[PK_VERIFY].M_cap;
   const int M_tmp = std::max(h->pass[PK_DRAFT].M_cap, h->pass[PK_ENCODE].M_cap);
   h->y = (float*)bp.take(sizeof(float) * (size_t)M_all * d);
-  h->pre = (float*)bp.take(sizeof(float) * partial_elems(M_all, d, h->bf16));
-  if (has_head_partials(c)) h->pre2 = (float*)bp.take(sizeof(float) * (size_t)c.n_heads * M_all * d);
+  h->pre = (float*)bp.take(sizeof(float) * partial_elems(c, M_all));
+  if (const size_t n = head_partial_elems(c, M_all)) h->pre2 = (float*)bp.take(sizeof(float) * n);
   h->yb.ptr = bp.take(e * (size_t)M_all * d); h->yb.cols = d;
   h->abuf.ptr = bp.take(e * (size_t)M_all * d); h->abuf.cols = d;
   h->hbuf.ptr = bp.take(e * (size_t)M_all * F); h->hbuf.cols = F;
@@ -371,8 +384,8 @@ size_t layout(ad_handle* h, void* base) {
     const int Me = h->pass[PK_ENCODE].M_cap;
     ActSet& sd = h->side;
     sd.y = (float*)bp.take(sizeof(float) * (size_t)Me * d);
-    sd.pre = (float*)bp.take(sizeof(float) * partial_elems(Me, d, h->bf16));
-    if (has_head_partials(c)) sd.pre2 = (float*)bp.take(sizeof(float) * (size_t)c.n_heads * Me * d);
+    sd.pre = (float*)bp.take(sizeof(float) * partial_elems(c, Me));
+    if (const size_t n = head_partial_elems(c, Me)) sd.pre2 = (float*)bp.take(sizeof(float) * n);
     sd.yb.ptr = bp.take(e * (size_t)Me * d); sd.yb.cols = d;
     sd.abuf.ptr = bp.take(e * (size_t)Me * d); sd.abuf.cols = d;
     sd.hbuf.ptr = bp.take(e * (size_t)Me * F); sd.hbuf.cols = F;
@@ -1085,8 +1098,6 @@ int embed(ad_handle* h, const PassCfg& pc, const Model& m) {
 }
 
 // ---- FP32 sublayers of few tokens (sublayer_f32.cuh) ----
-// Width of the slices of hidden features of the feed-forward sublayer (0: not covered).
-int f32_ffn_slice(int F) { return F % 32 == 0 && F / 32 <= 16 ? 32 : F % 64 == 0 && F / 64 <= 32 ? 64 : 0; }
 // Whether the sublayers of pass pc run on these kernels: what they cover, up to five waves of CTAs of the attention at capacity (two, three, five allowed:
 // 256 wide, batch 24 2522, 2494, 2494 us a call, 3256 without them).
 bool f32_sublayers(const ad_handle* h, const PassCfg& pc) {

@@ -36,7 +36,7 @@ def _cfg(shape, **kw):
     args.update(kw)
     return binding.ModelCfg(shape.d_model, shape.n_heads, shape.d_ffn, shape.vocab, shape.n_enc, shape.n_dec,
                             1 if shape.dtype == "bf16" else 0, args["max_batch"], args["max_src"], args["max_tgt"],
-                            args["kmax"], 0, 1, 2, 3, 1e-5, 0)
+                            args["kmax"], 0, 1, 2, 3, 1e-5, args.get("has_drafter", 0))
 
 
 def test_weight_counts_match_the_documented_layout(lib):
@@ -74,6 +74,26 @@ def test_workspace_query_and_config_checks(lib):
     bad = _cfg(synth.BASE)
     bad.eos = 40000
     assert lib.ad_query_workspace(C.byref(bad), C.byref(n)) == binding.AD_ERR_ARG
+
+
+def test_partial_sums_take_no_more_room_than_the_kernels_that_leave_them(lib):
+    """FP32 models: the sums per head and per slice of hidden features belong to kernels for passes of up to 1024 tokens and models 128 and
+    256 wide; a handle of thousands of tokens, or of another width, has no use for more of them."""
+    def size(d, heads, ffn, **kw):
+        n = C.c_size_t()
+        shape = synth.ModelShape("size", d, heads, ffn, 1000, 1, 1, "fp32")
+        assert lib.ad_query_workspace(C.byref(_cfg(shape, **kw)), C.byref(n)) == 0
+        return n.value
+
+    slack = 1 << 14                                           # alignment of the buffers
+    for d in (128, 256):                                      # twice the heads: so many more sums, with a drafter in both sets of buffers
+        for drafter in (0, 1):
+            large = dict(max_batch=256, max_src=256, max_tgt=64, kmax=64, has_drafter=drafter)
+            more = size(d, d // 32, 1024, **large) - size(d, d // 64, 1024, **large)
+            assert 0 < more <= (1 + drafter) * (d // 64) * 1024 * d * 4 + slack
+    # 512 wide: none at all, so a slightly wider model needs more room and not less
+    some = dict(max_batch=32, max_src=32, max_tgt=32, kmax=32)
+    assert size(512, 8, 2048, **some) < size(576, 9, 2048, **some)
 
 
 def test_struct_layouts():
