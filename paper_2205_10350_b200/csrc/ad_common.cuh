@@ -59,11 +59,12 @@ enum Epi : int {
 // (512 wide: base model, capacity 256 for the first line, 2048 for the others; 1024 wide: big model, capacity 1024):
 //   512 wide, 200 / 240 tokens: 32-token tiles 212 / 224 us, 64: 220 / 226, 128: 238 / 248, 16: 224 / 232;
 //   320 / 512 / 800 / 1024 tokens: 64-token tiles 293 / 309 / 344 / 363 us, 128: 340 / 351 / 379 / 388, 32: 334 / 362 / 435 / 455;
-//   2048 tokens: 128-token tiles 490 us, 64: 519, 256: 586 (256 is taken once it alone gives two CTAs per SM);
-//   1024 wide, 100 / 128 tokens: 64-token tiles 345 / 359 us, 128: 385 / 400, 32: 390 / 396.
+//   2048 tokens: 128-token tiles 490 us, 64: 519, 256: 586 (256 is taken once it alone gives two CTAs per SM).
 // The line at 1024 is the narrow models': 1024 wide, 128-token tiles already win there (648 us, 64: 717), and 64 at 200 (386, 32: 404).
-// 65 to 128 tokens inside a larger capacity: 32-token tiles too.  Whole calls of 512 wide models whose passes are of this size, the 16-feature form
-// of the few-token kernel in two rounds -> 64-token tiles -> 32: batch 3 with drafter 4560 -> 4236 -> 4073 us, batch 5 with drafter 4610 -> 4415 -> 4304.
+// 65 to 128 tokens inside a larger capacity: 32-token tiles too, while they are one wave of CTAs.  Verified blocks of 68 / 100 / 128 tokens of 200, 64-token tiles -> 32:
+// 768 wide 269 / 279 / 282 us -> 261 / 272 / 276, 1024 wide 305 / 318 / 324 -> 304 / 317 / 320; 512 wide, 72 / 96 / 128 tokens of 256, 182 / 186 / 193 -> 170 / 173 / 186 (the 16-feature
+// form of the few-token kernel in two rounds 191 / 202 / 212).  With more CTAs than SMs each of them reads its weights once more for nothing: arg-max over
+// a vocabulary of 16000, 512 wide, 100 tokens 10.3 -> 13.8 us, 65 tokens 10.9 -> 12.2; of 18816, 1024 wide, 12.5 -> 18.7; 8192, 768 wide, 8.2 -> 9.7.
 // Passes that never have more than 128 tokens take the few-token kernels and the rule is only asked for what those do not cover.
 // A projection whose feature tiles alone outnumber the SMs (the vocabulary) fills them with one token tile, and every further one
 // reads its weights again: one 128-token tile up to 128 tokens (90 tokens x 50265 x 768: 19.5 us with two of 64), then tiles of 128
@@ -95,7 +96,7 @@ __host__ __device__ inline Geo geometry(const GeoRule& r, int M) {
   } else if (nf >= r.sms) {
     g.tile = M <= 1536 ? 128 : 256;
   } else if (M <= 256) {
-    g.tile = 32;
+    g.tile = M > 128 || nf * ((M + 31) / 32) <= r.sms ? 32 : 64;
   } else if (M <= 1024) {
     g.tile = 64;
   } else {

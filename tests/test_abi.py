@@ -121,3 +121,14 @@ def test_projection_launches_cover_every_token_count(lib, d, heads, ffn, vocab):
         for i in range(n.value):
             epi, N, K, ctas, need_ctas, smem, need_smem = rows[7 * i: 7 * i + 7]
             assert ctas >= need_ctas and smem >= need_smem, (batch * kmax, epi, N, K, ctas, need_ctas, smem, need_smem)
+
+
+@pytest.mark.parametrize("d,vocab,batch,kmax,want", [(512, 16000, 2, 50, 2 * 125), (1024, 18816, 2, 64, 2 * 147), (768, 8192, 2, 33, 2 * 64), (512, 4096, 2, 64, 4 * 32),
+                                                     (512, 18944, 2, 64, 148)])
+def test_projections_of_65_to_128_tokens_read_their_weights_twice_where_tiles_of_32_tokens_outnumber_the_sms(lib, d, vocab, batch, kmax, want):
+    """CTAs of the projection onto vocabularies of fewer feature tiles than there are SMs (148 without a device), and of as many."""
+    cfg = binding.ModelCfg(d, d // 64, 2 * d, vocab, 2, 2, 1, batch, 64, 64, kmax, 0, 1, 2, 3, 1e-5, 0)
+    rows, n = (C.c_int32 * (7 * 16))(), C.c_int32()
+    assert lib.ad_debug_projection_shapes(C.byref(cfg), rows, 16, C.byref(n)) == 0
+    ctas = [rows[7 * i + 3] for i in range(n.value) if rows[7 * i] == 3]      # EPI_ARGMAX
+    assert ctas == [want]
