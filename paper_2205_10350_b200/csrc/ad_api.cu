@@ -1007,8 +1007,10 @@ int attention_few(ad_handle* h, const PassCfg& pc, const void* k, const void* v,
   }
   note_launch(h, wq ? "q_proj+attention+out_proj" : "attention+out_proj");
   cudaLaunchConfig_t cfg = {};
+  // A loop in place of a grid of more than one wave, even of one that has no work for most of its CTAs: a layout for 64 tokens of 14 rows with blocks of up
+  // to 64, 512 wide, launched 448 CTAs, an SM each, for at most 144 with work (verified blocks of 14 / 28 / 56 tokens 167 / 173 / 187 us, as a loop 156 / 160 / 176).
   // (CTAs of up to four warps fit an SM twice and keep their waves: 256 wide, encoder calls of four layers, 10 x 60 tokens 114 -> 125 us as a loop)
-  const long items = pc.pieces(c.max_batch, few::AQ), ctas = items * c.n_heads * split;
+  const long items = pc.pieces(h->dims.B, few::AQ), ctas = (long)h->dims.B * p.qchunks * c.n_heads * split;
   const bool loop = ctas > num_sms() && warps > 4 && c.n_heads * split <= num_sms();
   fp.rows = h->dims.B;
   const int groups = loop ? (int)std::min(items, (long)num_sms() / (c.n_heads * split)) : h->dims.B * p.qchunks;
