@@ -82,3 +82,43 @@ def test_sublayer_kernels_follow_the_checker(d, heads, ffn, batch, k, src, tgt):
     stats = lockstep(dec, model, srcs, lens, streams, k, [tgt] * batch, tol=1e-3, max_steps=12)
     assert stats["steps"] > 0
     dec.close()
+
+
+# of the checker's own error in FP32.  Measured with the partial sums added pairwise before the residual: at most 0.67 at 128 wide and 0.58 at 256; added to it one after
+# the other, 0.85 and 0.67 or more
+ERROR_BAR = {128: 0.75, 256: 0.62}
+
+
+@pytest.mark.parametrize("d,heads,ffn,batch,k,src", [(128, 4, 512, 1, 17, 16), (128, 4, 512, 4, 30, 30), (128, 2, 512, 3, 20, 100), (256, 8, 1024, 4, 30, 60),
+                                                     (256, 4, 2048, 2, 20, 130), (256, 8, 512, 3, 16, 40), (256, 4, 1024, 20, 40, 40)])
+def test_error_of_the_scores_against_64_bits(d, heads, ffn, batch, k, src):
+    """Scores of two verified blocks per row, one behind the other, against the checker in double precision: the many partial sums that sublayers in one kernel
+    each leave must not cost precision."""
+    shape = synth.ModelShape(f"f32err_{d}_{heads}_{ffn}", d, heads, ffn, 1000, 2, 2, "fp32")
+    w = synth.make_weights(shape, 0)
+    exact, plain = O.Model(shape, w, max_pos=256, real="f64"), O.Model(shape, w, max_pos=256)
+    r = np.random.default_rng(batch)
+    srcs = r.integers(4, shape.vocab, size=(batch, src)).astype(np.int32)
+    lens = r.integers(max(1, src // 2), src + 1, size=batch).astype(np.int32)
+    dec = binding.AggressiveDecoder(shape, w, max_batch=batch, max_src=src, max_tgt=2 * k, kmax=k)
+    dec.encode(srcs, lens)
+    rows = range(min(batch, 3))
+    states = [[m.state(srcs[b, : lens[b]], cap=2 * k) for m in (exact, plain)] for b in rows]
+    last = [exact.bos] * batch
+    err = own = 0.0
+    for _ in range(2):
+        drafts = r.integers(4, shape.vocab, size=(batch, k)).astype(np.int32)
+        ks = np.full(batch, k, np.int32)
+        dec.verify_block(drafts, ks)
+        lg = dec.debug_logits(batch * k).astype(np.float64)
+        for b in rows:
+            want, fp32 = (st.verify_block(last[b], drafts[b], want_logits=True)["logits"].astype(np.float64) for st in states[b])
+            err += ((lg[b * k: (b + 1) * k] - want) ** 2).sum()
+            own += ((fp32 - want) ** 2).sum()
+            for st in states[b]:
+                st.commit(k)
+            last[b] = int(drafts[b, -1])
+        dec.force_commit(drafts, ks)
+    dec.close()
+    print(f"{d} wide, {heads} heads, {ffn}, {batch} x {k}: error {(err / own) ** 0.5:.3f} of the checker's in FP32")
+    assert err <= ERROR_BAR[d] ** 2 * own
