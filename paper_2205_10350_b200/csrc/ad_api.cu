@@ -1201,9 +1201,13 @@ int ffn_sublayer(ad_handle* h, int pk, const Mat& w1, const float* b1, const Mat
     p.a.M_ptr = pc.plan.M;
     p.x = (const float*)h->yb.ptr; p.w_in = (const float*)w1.ptr; p.b_in = b1; p.w_out = (const float*)w2.ptr;
     p.out = h->pre; p.stride = (size_t)pc.M_cap * d; p.K2 = F;
-    AD_TRY(launch_sublayer_f32<sub32::FFN>(h, dim3((pc.M_cap + sub32::TOK - 1) / sub32::TOK, F / slice), slice, p, "ffn"));
+    // One wave of CTAs, which keep their weights from tile to tile.  With a CTA per tile, one an SM, every wave read them again: passes of 1024 tokens (four layers), the
+    // projections' own kernels -> a CTA per tile -> this: 256 wide, feed-forward width 1024 662 -> 670 -> 579 us, 2048 914 -> 979 -> 777, 128 wide, 2048 570 -> 623 -> 459; of 256
+    // 400 -> 302 -> 285, 508 -> 379 -> 330, 308 -> 272 -> 229.  Two waves: 597, 790, 470; 303, 349, 243.
+    const int slices = F / slice, groups = std::min((pc.M_cap + sub32::TOK - 1) / sub32::TOK, std::max(1, num_sms() / slices));
+    AD_TRY(launch_sublayer_f32<sub32::FFN>(h, dim3(groups, slices), slice, p, "ffn"));
     Partials ps = {};
-    ps.ptr = h->pre; ps.nsplit = F / slice; ps.stride = p.stride;
+    ps.ptr = h->pre; ps.nsplit = slices; ps.stride = p.stride;
     return layernorm(h, pc, ps, b2, lng, lnb, out);
   }
   GemmParams a = {};

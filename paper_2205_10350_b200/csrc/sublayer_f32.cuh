@@ -47,8 +47,8 @@ __device__ __forceinline__ void fma4(float4& s, float4 a, float4 b) {
 }
 __device__ __forceinline__ float sum4(float4 s) { return (s.x + s.y) + (s.z + s.w); }
 
-// S: width of a head, or of a slice of hidden features.  grid = (B * qchunks, heads) or (ceil(M_cap / 16), F / S); block = 256; dynamic shared
-// memory Layout<D, S>::FLOATS floats.
+// S: width of a head, or of a slice of hidden features.  grid = (B * qchunks, heads), or (groups, F / S): group i takes the tiles i, i + groups, ... of 16 tokens.
+// block = 256; dynamic shared memory Layout<D, S>::FLOATS floats (FFN: OS).
 template <Kind KIND, int D, int S>
 __global__ void __launch_bounds__(THREADS)
 sublayer_f32_kernel(const Params p) {
@@ -60,10 +60,11 @@ sublayer_f32_kernel(const Params p) {
   float *ks = sub_smem + L::KS, *vs = sub_smem + L::VS, *ps = sub_smem + L::PS;
   pdl_launch();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, h = blockIdx.y;
-  int m0, nt, kbase = 0, row_nk = 0;
+  int m0, nt, kbase = 0, row_nk = 0, M = 0;
   if (KIND == FFN) {
     m0 = blockIdx.x * TOK;
-    nt = min(TOK, plan_load(p.a.M_ptr) - m0);
+    M = plan_load(p.a.M_ptr);
+    nt = min(TOK, M - m0);
   } else {
     const int b = blockIdx.x / p.a.qchunks, i0 = (blockIdx.x - b * p.a.qchunks) * TOK;
     nt = min(TOK, plan_load(p.a.seg_len + b) - i0);
@@ -108,119 +109,131 @@ sublayer_f32_kernel(const Params p) {
     fetch_keys(0);
     const float* q = reinterpret_cast<const float*>(p.a.q);
     for (int idx = tid; idx < nt * S; idx += THREADS) hs[(idx / S) * L::LD + idx % S] = q[(size_t)(m0 + idx / S) * D + h * S + idx % S] * p.a.scale;
-  } else {
-    for (int idx = tid; idx < nt * (D / 4); idx += THREADS) {
+  }
+  auto fetch_x = [&](int m, int n) {                        // n tokens' input
+    for (int idx = tid; idx < n * (D / 4); idx += THREADS) {
       const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
-      simt::cp16(xs + r * D + c, p.x + (size_t)(m0 + r) * D + c, true);
+      simt::cp16(xs + r * D + c, p.x + (size_t)(m + r) * D + c, true);
     }
-  }
+  };
+  if (KIND != SELF) fetch_x(m0, nt);
   asm volatile("cp.async.commit_group;" ::: "memory");
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
-  if (KIND != SELF) {
-    // first projection: every part's share of the tokens' S features, then their sum
+  int m_next, n_next;
+  do {                                                      // (once, but for the feed-forward sublayer)
+    m_next = m0 + TOK * (int)gridDim.x;
+    n_next = KIND == FFN ? min(TOK, M - m_next) : 0;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (KIND != SELF) {
+      // first projection: every part's share of the tokens' S features, then their sum
 #pragma unroll 4
-    for (int r = 0; r < nt; ++r) {
-      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int r = 0; r < nt; ++r) {
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int i = 0; i < KP / 4; ++i) fma4(s, w1[KIND == SELF ? 0 : i], *reinterpret_cast<const float4*>(xs + r * D + part * KP + 4 * i));
-      red[(part * TOK + r) * S + f] = sum4(s);
-    }
-    __syncthreads();
-    for (int r = part; r < nt; r += PARTS) {
-      float s = red[r * S + f];
-#pragma unroll
-      for (int q = 1; q < PARTS; ++q) s += red[(q * TOK + r) * S + f];
-      s += bias;
-      hs[r * L::LD + f] = KIND == FFN ? fmaxf(s, 0.f) : s * p.a.scale;
-    }
-    __syncthreads();
-  }
-  if (KIND != FFN) {
-    // attention: two queries per warp, keys lane and lane + 32 of every tile, running maximum and sum
-    float mx[2] = {-INFINITY, -INFINITY}, den[2] = {0.f, 0.f}, acc[2][S / 32];
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-      for (int c = 0; c < S / 32; ++c) acc[u][c] = 0.f;
-    for (int j0 = 0; j0 < row_nk; j0 += KEYS) {
-      if (j0 > 0) {
-        __syncthreads();                                    // the previous tile has been read
-        fetch_keys(j0);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();
+        for (int i = 0; i < KP / 4; ++i) fma4(s, w1[KIND == SELF ? 0 : i], *reinterpret_cast<const float4*>(xs + r * D + part * KP + 4 * i));
+        red[(part * TOK + r) * S + f] = sum4(s);
       }
-      float s[2][2];
-      float4 s4[2][2];
+      __syncthreads();
+      if (KIND == FFN && n_next > 0) {                      // the next tile's input, under the rest of this one
+        fetch_x(m_next, n_next);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+      }
+      for (int r = part; r < nt; r += PARTS) {
+        float s = red[r * S + f];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) s4[u][0] = s4[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q = 1; q < PARTS; ++q) s += red[(q * TOK + r) * S + f];
+        s += bias;
+        hs[r * L::LD + f] = KIND == FFN ? fmaxf(s, 0.f) : s * p.a.scale;
+      }
+      __syncthreads();
+    }
+    if (KIND != FFN) {
+      // attention: two queries per warp, keys lane and lane + 32 of every tile, running maximum and sum
+      float mx[2] = {-INFINITY, -INFINITY}, den[2] = {0.f, 0.f}, acc[2][S / 32];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int c = 0; c < S / 32; ++c) acc[u][c] = 0.f;
+      for (int j0 = 0; j0 < row_nk; j0 += KEYS) {
+        if (j0 > 0) {
+          __syncthreads();                                    // the previous tile has been read
+          fetch_keys(j0);
+          asm volatile("cp.async.commit_group;" ::: "memory");
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          __syncthreads();
+        }
+        float s[2][2];
+        float4 s4[2][2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) s4[u][0] = s4[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
-      for (int c = 0; c < S; c += 4) {
-        const float4 k0 = *reinterpret_cast<const float4*>(ks + lane * L::LD + c), k1 = *reinterpret_cast<const float4*>(ks + (lane + 32) * L::LD + c);
+        for (int c = 0; c < S; c += 4) {
+          const float4 k0 = *reinterpret_cast<const float4*>(ks + lane * L::LD + c), k1 = *reinterpret_cast<const float4*>(ks + (lane + 32) * L::LD + c);
+#pragma unroll
+          for (int u = 0; u < 2; ++u) {
+            const float4 q = *reinterpret_cast<const float4*>(hs + (warp + 8 * u) * L::LD + c);
+            fma4(s4[u][0], q, k0);
+            fma4(s4[u][1], q, k1);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) { s[u][0] = sum4(s4[u][0]); s[u][1] = sum4(s4[u][1]); }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const float4 q = *reinterpret_cast<const float4*>(hs + (warp + 8 * u) * L::LD + c);
-          fma4(s4[u][0], q, k0);
-          fma4(s4[u][1], q, k1);
-        }
-      }
+          float p0 = 0.f, p1 = 0.f, corr = 1.f;
+          if (nk[u] > j0) {                                   // warp-uniform; otherwise the query sees no key of this tile
+            const float a0 = j0 + lane < nk[u] ? s[u][0] : -INFINITY, a1 = j0 + lane + 32 < nk[u] ? s[u][1] : -INFINITY;
+            float top = fmaxf(a0, a1);
 #pragma unroll
-      for (int u = 0; u < 2; ++u) { s[u][0] = sum4(s4[u][0]); s[u][1] = sum4(s4[u][1]); }
+            for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+            const float now = fmaxf(mx[u], top);              // finite: key j0 is visible
+            corr = expf(mx[u] - now);                         // exp(-inf) = 0 on the first tile
+            p0 = expf(a0 - now); p1 = expf(a1 - now);
+            float sum = p0 + p1;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            den[u] = den[u] * corr + sum;
+            mx[u] = now;
+          }
+          ps[(warp + 8 * u) * KEYS + lane] = p0;
+          ps[(warp + 8 * u) * KEYS + lane + 32] = p1;
+#pragma unroll
+          for (int c = 0; c < S / 32; ++c) acc[u][c] *= corr;
+        }
+        __syncwarp();
+        const int jn = min(KEYS, row_nk - j0);
+#pragma unroll 2
+        for (int j = 0; j < jn; j += 4) {                     // (keys beyond the last are zeros with probability 0)
+          const float4 pa = *reinterpret_cast<const float4*>(ps + warp * KEYS + j), pb = *reinterpret_cast<const float4*>(ps + (warp + 8) * KEYS + j);
+#pragma unroll
+          for (int c = 0; c < S / 32; ++c) {
+            const float* v = vs + j * L::LD + lane + 32 * c;
+            const float v0 = v[0], v1 = v[L::LD], v2 = v[2 * L::LD], v3 = v[3 * L::LD];
+            acc[0][c] = fmaf(pa.x, v0, acc[0][c]); acc[0][c] = fmaf(pa.y, v1, acc[0][c]); acc[0][c] = fmaf(pa.z, v2, acc[0][c]); acc[0][c] = fmaf(pa.w, v3, acc[0][c]);
+            acc[1][c] = fmaf(pb.x, v0, acc[1][c]); acc[1][c] = fmaf(pb.y, v1, acc[1][c]); acc[1][c] = fmaf(pb.z, v2, acc[1][c]); acc[1][c] = fmaf(pb.w, v3, acc[1][c]);
+          }
+        }
+        __syncwarp();
+      }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        float p0 = 0.f, p1 = 0.f, corr = 1.f;
-        if (nk[u] > j0) {                                   // warp-uniform; otherwise the query sees no key of this tile
-          const float a0 = j0 + lane < nk[u] ? s[u][0] : -INFINITY, a1 = j0 + lane + 32 < nk[u] ? s[u][1] : -INFINITY;
-          float top = fmaxf(a0, a1);
+        const float inv = nk[u] > 0 ? 1.f / den[u] : 0.f;
 #pragma unroll
-          for (int o = 16; o > 0; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
-          const float now = fmaxf(mx[u], top);              // finite: key j0 is visible
-          corr = expf(mx[u] - now);                         // exp(-inf) = 0 on the first tile
-          p0 = expf(a0 - now); p1 = expf(a1 - now);
-          float sum = p0 + p1;
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-          den[u] = den[u] * corr + sum;
-          mx[u] = now;
-        }
-        ps[(warp + 8 * u) * KEYS + lane] = p0;
-        ps[(warp + 8 * u) * KEYS + lane + 32] = p1;
-#pragma unroll
-        for (int c = 0; c < S / 32; ++c) acc[u][c] *= corr;
+        for (int c = 0; c < S / 32; ++c) os[(warp + 8 * u) * L::LD + lane + 32 * c] = acc[u][c] * inv;
       }
-      __syncwarp();
-      const int jn = min(KEYS, row_nk - j0);
-#pragma unroll 2
-      for (int j = 0; j < jn; j += 4) {                     // (keys beyond the last are zeros with probability 0)
-        const float4 pa = *reinterpret_cast<const float4*>(ps + warp * KEYS + j), pb = *reinterpret_cast<const float4*>(ps + (warp + 8) * KEYS + j);
-#pragma unroll
-        for (int c = 0; c < S / 32; ++c) {
-          const float* v = vs + j * L::LD + lane + 32 * c;
-          const float v0 = v[0], v1 = v[L::LD], v2 = v[2 * L::LD], v3 = v[3 * L::LD];
-          acc[0][c] = fmaf(pa.x, v0, acc[0][c]); acc[0][c] = fmaf(pa.y, v1, acc[0][c]); acc[0][c] = fmaf(pa.z, v2, acc[0][c]); acc[0][c] = fmaf(pa.w, v3, acc[0][c]);
-          acc[1][c] = fmaf(pb.x, v0, acc[1][c]); acc[1][c] = fmaf(pb.y, v1, acc[1][c]); acc[1][c] = fmaf(pb.z, v2, acc[1][c]); acc[1][c] = fmaf(pb.w, v3, acc[1][c]);
-        }
-      }
-      __syncwarp();
+      __syncthreads();
     }
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const float inv = nk[u] > 0 ? 1.f / den[u] : 0.f;
-#pragma unroll
-      for (int c = 0; c < S / 32; ++c) os[(warp + 8 * u) * L::LD + lane + 32 * c] = acc[u][c] * inv;
-    }
-    __syncthreads();
-  }
-  // second projection: this thread's output feature of every GROUPS-th token
-  float* dst = p.out + (size_t)h * p.stride + (size_t)m0 * D + n;
+    // second projection: this thread's output feature of every GROUPS-th token
+    float* dst = p.out + (size_t)h * p.stride + (size_t)m0 * D + n;
 #pragma unroll 4
-  for (int r = group; r < nt; r += GROUPS) {
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r = group; r < nt; r += GROUPS) {
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int i = 0; i < S / 4; ++i) fma4(s, w2[i], *reinterpret_cast<const float4*>(os + r * L::LD + 4 * i));
-    dst[(size_t)r * D] = sum4(s);
-  }
+      for (int i = 0; i < S / 4; ++i) fma4(s, w2[i], *reinterpret_cast<const float4*>(os + r * L::LD + 4 * i));
+      dst[(size_t)r * D] = sum4(s);
+    }
+    m0 = m_next; nt = n_next;
+  } while (KIND == FFN && nt > 0);
 }
 
 }  // namespace sub32

@@ -63,6 +63,9 @@ def test_passes_follow_the_checker(d, heads, ffn, batch, k):
     (128, 4, 1024, 2, 17, 40, 129),    # a tile and one query; 16 slices of 64; prefix keys in three tiles
     (256, 8, 512, 9, 33, 64, 40),      # 297 tokens of capacity, exactly one tile of source keys
     (256, 4, 2048, 2, 5, 130, 24),     # 64-wide heads, 32 partial sums for the LayerNorm, source keys in three tiles
+    (256, 4, 2048, 3, 30, 20, 60),     # the same with six tiles of tokens for four groups of CTAs
+    (128, 4, 1984, 5, 33, 20, 40),     # 31 partial sums, eleven tiles for four groups, the last one short
+    (256, 8, 512, 10, 33, 12, 34),     # 16 slices of 32 hidden features, 21 tiles for nine groups
     (256, 8, 1100, 2, 7, 20, 24),      # a feed-forward width that stays with the projections' own kernels
 ])
 def test_sublayer_kernels_follow_the_checker(d, heads, ffn, batch, k, src, tgt):
