@@ -200,7 +200,10 @@ def test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, r
     (256, 1024, 3, 5),       # 16 partial sums, 15 tokens: less than a tile
     (256, 2048, 1, 17),      # 32 partial sums, a tile and one token
     (384, 1536, 2, 40),      # 24 partial sums, six warps; five tiles
-    (512, 1088, 2, 64),      # 17 partial sums; eight tiles, two for each CTA
+    (512, 1088, 2, 64),      # 17 partial sums; eight tiles of tokens, a CTA each
+    (512, 2048, 2, 64),      # 32 partial sums; eight tiles for four groups of CTAs
+    (512, 2048, 3, 53),      # ten tiles for four groups, the last one short; 160 tokens are the most that 32 partial sums allow
+    (384, 1536, 4, 37),      # ten tiles for six groups
 ])
 def test_feed_forward_sublayer_in_one_kernel_follows_the_checker(d, ffn, batch, k):
     test_few_token_passes_follow_the_checker(d, ffn, batch, k, 9, k + 8)

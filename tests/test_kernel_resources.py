@@ -1,6 +1,8 @@
-"""Registers and spills of the small kernels that a pass runs between its projections, as the compiler reports them, and sizes of prefetches.
+"""Registers and spills of the small kernels that a pass runs between its projections and of the sublayers that hold their weights in registers, as the
+compiler reports them, and sizes of prefetches.
 
-They are bound by one memory round trip each, and the registers they hold are kept from the projection behind them."""
+The small ones are bound by one memory round trip each, and the registers they hold are kept from the projection behind them.  The sublayers' kernels sit close to
+the most that a thread can have."""
 import os
 import re
 import subprocess
@@ -16,12 +18,13 @@ pytestmark = pytest.mark.skipif(not os.path.exists(NVCC), reason="no CUDA compil
 def _report(tmp_path, kernels):
     """{kernel's symbol: (registers, bytes spilled)} of the kernels named."""
     src = tmp_path / "kernels.cu"
-    src.write_text('#include "accept.cuh"\nusing namespace ad;\nvoid* kernels[] = {%s};\n' % ", ".join(f"(void*){k}" for k in kernels))
+    src.write_text("".join(f'#include "{h}.cuh"\n' for h in ("accept", "attention_few", "ffn_few", "sublayer_f32")) +
+                   "using namespace ad;\nvoid* kernels[] = {%s};\n" % ", ".join(f"(void*){k}" for k in kernels))
     r = subprocess.run([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-rdc=true", "-I", build.CSRC, "-Xptxas", "-v",
                         "-c", str(src), "-o", str(tmp_path / "kernels.o")], check=True, capture_output=True, text=True)
     found = re.findall(r"Compiling entry function '(\S+)'.*?(\d+) bytes spill stores.*?Used (\d+) registers", r.stdout + r.stderr, re.S)
-    names = {re.match(r"\w+", k).group() for k in kernels}
-    return {sym: (int(regs), int(spill)) for sym, spill, regs in found if any(re.match(rf"_ZN2ad\d+{n}I", sym) for n in names)}
+    names = {re.match(r"(?:\w+::)*(\w+)", k).group(1) for k in kernels}
+    return {sym: (int(regs), int(spill)) for sym, spill, regs in found if any(re.match(rf"_ZN2ad\w*?\d+{n}(I|E)", sym) for n in names)}
 
 
 def test_layernorm_holds_what_its_partial_sums_need(tmp_path):
@@ -39,6 +42,18 @@ def test_accept_kernels_fit_a_thousand_threads_without_spills(tmp_path):
     assert len(found) == 3
     for sym, (regs, spill) in found.items():
         assert spill == 0 and regs <= 64, f"{sym}: {regs} registers, {spill} bytes spilled"
+
+
+def test_sublayers_with_their_weights_in_registers_do_not_spill(tmp_path):
+    few = [f"few::attention_few_kernel<{q}, {split}, {first}, {loop}>" for q in ("false", "true") for split in (1, 2) for first in ("false", "true")
+           for loop in ("false", "true")] + ["few::ffn_few_kernel"]
+    f32 = [f"sub32::sublayer_f32_kernel<sub32::{kind}, {d}, {s}>" for kind in ("SELF", "CROSS", "FFN") for d in (128, 256) for s in (32, 64)]
+    parts = [f"layernorm_parts_kernel<{a}>" for a in ("bf16", "float")]
+    found = _report(tmp_path, few + f32 + parts)
+    assert len(found) == len(few) + len(f32) + len(parts)
+    for sym, (regs, spill) in found.items():
+        limit = 128 if "layernorm" in sym else 255             # (two CTAs of 256 threads an SM; the most a thread can have)
+        assert spill == 0 and regs <= limit, f"{sym}: {regs} registers, {spill} bytes spilled"
 
 
 def test_prefetches_end(tmp_path):
