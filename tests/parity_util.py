@@ -16,9 +16,36 @@ from __future__ import annotations
 import numpy as np
 
 from oracle import ad_oracle as O
+from paper_2205_10350_b200 import synth
 
 MARGIN = 0.1
 OPS = O.Ops("f32")
+
+
+def following_weights(shape, seed=0):
+    """Weights of a model whose output follows its source, with clear gaps between the best and the second best score, where plain random weights
+    repeat one token whatever the source says.  The first head's dimensions carry nothing but the position; the last cross-attention looks the position being
+    decoded up in the source and carries its token over.  Ids divisible by eight are weaker variants of their successors: the output has the successor."""
+    w = synth.make_weights(shape, seed)
+    d, heads = shape.d_model, shape.n_heads
+    dh = d // heads
+    for n in w:
+        if n.endswith((".o.W", ".ffn2.W")):
+            w[n][:, :dh] = 0.0
+    emb = np.random.default_rng(seed).standard_normal(w["emb"].shape).astype(np.float32) / np.sqrt(d)
+    emb[:, :dh] = 0.0
+    variant = np.arange(8, shape.vocab - 1, 8)
+    emb[variant] = 0.8 * emb[variant + 1]
+    q = np.zeros((d, d), np.float32)
+    freq = 10000.0 ** (-np.arange(0, dh, 2) / d)
+    for h in range(heads):
+        for i in 2 * np.flatnonzero(freq >= 0.5):
+            q[i, h * dh + i] = q[i + 1, h * dh + i + 1] = 6.0
+    last = f"dec.{shape.n_dec - 1}.cross"
+    w["emb"] = emb
+    w[f"{last}.q.W"], w[f"{last}.k.W"] = q, q.copy()
+    w[f"{last}.v.W"], w[f"{last}.o.W"] = np.eye(d, dtype=np.float32), 4.0 * np.eye(d, dtype=np.float32)
+    return {n: synth.round_to_bf16(a) for n, a in w.items()} if shape.dtype == "bf16" else w
 
 
 def second_best(logits_row, best):
