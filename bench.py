@@ -277,7 +277,7 @@ def kernel_table(dec, shape, drafts, k, pk):
         elif name == "ffn":
             g["bytes"] += 2 * d * F * 2 + k * d * 2 + (F // 64) * k * d * 4
         elif "layernorm" in name:
-            g["bytes"] += 9 * k * d * 4 + k * d * 6
+            g["bytes"] += (int(name.rsplit("P", 1)[1]) + 1) * k * d * 4 + k * d * 6       # partial sums and residual; FP32 and BF16 result
     total = sum(g["us"] for g in groups.values())
     rows = []
     for g in sorted(groups.values(), key=lambda g: -g["us"]):

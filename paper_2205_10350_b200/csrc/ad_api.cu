@@ -739,7 +739,8 @@ const TcShape& cached_shape(ad_handle* h, const GeoRule& r, int M_cap) {
 // Whether a decoder pass reads more weights than stay in L2 (126 MB, shared with everything else) from one pass to the next.  Its kernels
 // then fetch them from HBM, and can begin to when an SM has room for them, one kernel ahead at most: the feed-forward projections, 128 CTAs
 // that fill an SM's registers each, waited 1.2 us for theirs.  So the QKV projection of a layer, three to four kernels ahead, brings
-// the layer's feed-forward weights into L2, its first feed-forward projection the next layer's attention weights.  Whole calls: 1024 wide
+// the layer's feed-forward weights into L2, its first feed-forward projection the next layer's attention weights (both in the form for wide slices of K
+// alone: models up to 512 wide prefetch nothing).  Whole calls: 1024 wide
 // (242 MB a pass), batch 4 greedy 7730 -> 7580 us, batch 1 with drafter 3810 -> 3760; 768 wide (176 MB) 2287 -> 2267.  The embedding matrix
 // fetched ahead in the last layers, or the first layer's weights at the end of the vocabulary kernel, gained nothing or lost it again.
 bool weights_stream(const ad_handle* h) {
@@ -1039,10 +1040,12 @@ int layernorm(ad_handle* h, const PassCfg& pc, const Partials& pre, const float*
               const ActBuf* out = nullptr) {
   const int d = h->cfg.d_model;
   const LnParams p = {pc.plan.M, pre, bias, h->y, g, b, d, h->cfg.ln_eps, h->y};
-  note_launch(h, "residual+layernorm");
   // P, the partial sums in flight, from the most that any token count of the pass brings (it sets the registers, see layernorm_kernel)
   const int most = pre.nsplit > 0 ? pre.nsplit : cached_shape(h, pre.rule, pc.M_cap).ksplit;
   if (most > 32 || (most > 16 && d > 512)) return fail(h, AD_ERR_ARG, "layernorm: too many partial sums");
+  char name[40];
+  snprintf(name, sizeof(name), "residual+layernorm P%d", most);
+  note_launch(h, name);
   auto go_n = [&](auto* yb, auto threads, auto parts) -> cudaError_t {
     using ActT = std::remove_pointer_t<decltype(yb)>;
     constexpr int T = decltype(threads)::value, P = decltype(parts)::value, per_cta = 256 / T;
