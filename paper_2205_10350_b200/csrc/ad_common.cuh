@@ -179,6 +179,12 @@ __device__ __forceinline__ int plan_load(const int* p) { return __ldcg(p); }
 // while the predecessor runs.  One CTA of the grid always waits, work or not: a grid that completed before its predecessor
 // would release its own successors too early.
 
+// 16-byte asynchronous copy global -> shared; zeros unless `there` (the source address must be valid all the same).
+__device__ __forceinline__ void cp16(void* smem_dst, const void* gmem_src, bool there) {
+  const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem_src), "r"(there ? 16 : 0) : "memory");
+}
+
 // 16 bytes of weights that one CTA reads once, kept out of L1 (whole calls: batch 1 1133 -> 1124 us, batch 8 3587 -> 3548; not for the
 // attention's weights, which the CTAs of a row's other query chunks read again: batch 8 with drafter 7865 -> 8090).
 __device__ __forceinline__ uint4 weight_load_once(const void* p) {

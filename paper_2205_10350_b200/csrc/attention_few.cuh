@@ -54,10 +54,6 @@ inline size_t att_few_smem(int warps, int rounds, bool loop_pair) {
 inline int att_few_split(int d) { return d > 64 * MAX_WARPS ? 2 : 1; }
 inline int att_few_warps(int d) { return d / 64 / att_few_split(d); }
 
-__device__ __forceinline__ void cp16(void* smem_dst, const void* gmem_src, bool there) {
-  const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem_src), "r"(there ? 16 : 0) : "memory");
-}
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);

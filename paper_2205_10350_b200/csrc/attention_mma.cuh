@@ -34,12 +34,6 @@ constexpr int AL_KLD = 96;             // key rows 192 bytes apart: conflict-fre
 constexpr int AL_VLD = 72;             // value rows 144 bytes apart: conflict-free ldmatrix
 constexpr int AL_TILE_BYTES = AM_KT * (AL_KLD + AL_VLD) * 2;   // 21 504
 
-// 16-byte asynchronous copy global -> shared; src_bytes = 0 writes zeros (the source address must still be valid).
-__device__ __forceinline__ void am_cp_async16(void* smem_dst, const void* gmem_src, int src_bytes) {
-  const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst));
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem_src), "r"(src_bytes) : "memory");
-}
-
 // One 64-key tile of K and V into `dst`; keys from row_nk on are written as zeros.
 template <int THREADS>
 __device__ __forceinline__ void fetch_kv_tile(uint8_t* dst, const bf16* k, const bf16* v, int first_key, int row_nk, int d, int tid) {
@@ -49,8 +43,8 @@ __device__ __forceinline__ void fetch_kv_tile(uint8_t* dst, const bf16* k, const
     const int idx = tid + THREADS * i, j = idx >> 3, c = (idx & 7) * 8;
     const bool there = first_key + j < row_nk;
     const size_t off = (size_t)(there ? first_key + j : 0) * d + c;
-    am_cp_async16(kd + j * AL_KLD + c, k + off, there ? 16 : 0);
-    am_cp_async16(kd + AM_KT * AL_KLD + j * AL_VLD + c, v + off, there ? 16 : 0);
+    cp16(kd + j * AL_KLD + c, k + off, there);
+    cp16(kd + AM_KT * AL_KLD + j * AL_VLD + c, v + off, there);
   }
 }
 

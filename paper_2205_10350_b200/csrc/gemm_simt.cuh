@@ -26,10 +26,6 @@ constexpr size_t smem_bytes() {
   return ring > sums ? ring : sums;
 }
 
-__device__ __forceinline__ void cp16(void* s, const void* g, bool there) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(s))), "l"(g),
-               "r"(there ? 16 : 0) : "memory");
-}
 __device__ __forceinline__ void cp4(void* s, const void* g, bool there) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(s))), "l"(g),
                "r"(there ? 4 : 0) : "memory");

@@ -10,7 +10,6 @@
 #pragma once
 
 #include "attention.cuh"
-#include "gemm_simt.cuh"   // cp16
 
 namespace ad {
 namespace sub32 {
@@ -92,8 +91,8 @@ sublayer_f32_kernel(const Params p) {
       const int j = idx / (S / 4), c = (idx % (S / 4)) * 4;
       const bool there = j0 + j < row_nk;
       const size_t off = (size_t)(kbase + (there ? j0 + j : 0)) * D + h * S + c;
-      simt::cp16(ks + j * L::LD + c, kk + off, there);
-      simt::cp16(vs + j * L::LD + c, vv + off, there);
+      cp16(ks + j * L::LD + c, kk + off, there);
+      cp16(vs + j * L::LD + c, vv + off, there);
     }
   };
   if (KIND == CROSS) fetch_keys(0);                         // the encoder's: older than the plan
@@ -113,7 +112,7 @@ sublayer_f32_kernel(const Params p) {
   auto fetch_x = [&](int m, int n) {                        // n tokens' input
     for (int idx = tid; idx < n * (D / 4); idx += THREADS) {
       const int r = idx / (D / 4), c = (idx % (D / 4)) * 4;
-      simt::cp16(xs + r * D + c, p.x + (size_t)(m + r) * D + c, true);
+      cp16(xs + r * D + c, p.x + (size_t)(m + r) * D + c, true);
     }
   };
   if (KIND != SELF) fetch_x(m0, nt);
