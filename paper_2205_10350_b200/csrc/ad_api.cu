@@ -1109,26 +1109,26 @@ bool f32_sublayers(const ad_handle* h, const PassCfg& pc) {
   const ad_model_cfg& c = h->cfg;
   return !h->bf16 && h->pre2 && h->sw.fuse_attn_proj && pc.M_cap <= sub32::MAX_TOKENS && pc.pieces(c.max_batch, sub32::TOK) * c.n_heads <= 5L * num_sms();
 }
-template <sub32::Kind KIND, int D, int S>
+template <sub32::Kind KIND, int D, int S, bool LOOP>
 cudaError_t launch_sublayer_f32_n(cudaStream_t st, dim3 grid, const sub32::Params& p) {
   typedef sub32::Layout<D, S> L;
   constexpr size_t smem = sizeof(float) * (KIND == sub32::FFN ? L::OS : L::FLOATS);
   static bool attr_set[kMaxDevices] = {};
   const int dev = current_device();
   if (!attr_set[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(sub32::sublayer_f32_kernel<KIND, D, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(sub32::sublayer_f32_kernel<KIND, D, S, LOOP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
   // (one CTA an SM, like the projections around it: 256 wide, batch 6 1364 us a call with the runtime's choice, 1295)
-  return launch_shared(one_cta_share(smem), sub32::sublayer_f32_kernel<KIND, D, S>, grid, dim3(sub32::THREADS), smem, st, p);
+  return launch_shared(one_cta_share(smem), sub32::sublayer_f32_kernel<KIND, D, S, LOOP>, grid, dim3(sub32::THREADS), smem, st, p);
 }
-template <sub32::Kind KIND>
+template <sub32::Kind KIND, bool LOOP = false>
 int launch_sublayer_f32(ad_handle* h, dim3 grid, int width, const sub32::Params& p, const char* what) {
   note_launch(h, what);
   const bool d128 = h->cfg.d_model == 128, s32 = width == 32;
-  const cudaError_t e = d128 ? (s32 ? launch_sublayer_f32_n<KIND, 128, 32>(h->stream, grid, p) : launch_sublayer_f32_n<KIND, 128, 64>(h->stream, grid, p))
-                             : (s32 ? launch_sublayer_f32_n<KIND, 256, 32>(h->stream, grid, p) : launch_sublayer_f32_n<KIND, 256, 64>(h->stream, grid, p));
+  const cudaError_t e = d128 ? (s32 ? launch_sublayer_f32_n<KIND, 128, 32, LOOP>(h->stream, grid, p) : launch_sublayer_f32_n<KIND, 128, 64, LOOP>(h->stream, grid, p))
+                             : (s32 ? launch_sublayer_f32_n<KIND, 256, 32, LOOP>(h->stream, grid, p) : launch_sublayer_f32_n<KIND, 256, 64, LOOP>(h->stream, grid, p));
   if (e != cudaSuccess) return fail(h, AD_ERR_CUDA, std::string("sublayer launch: ") + cudaGetErrorString(e));
   return AD_OK;
 }
@@ -1207,8 +1207,9 @@ int ffn_sublayer(ad_handle* h, int pk, const Mat& w1, const float* b1, const Mat
     // One wave of CTAs, which keep their weights from tile to tile.  With a CTA per tile, one an SM, every wave read them again: passes of 1024 tokens (four layers), the
     // projections' own kernels -> a CTA per tile -> this: 256 wide, feed-forward width 1024 662 -> 670 -> 579 us, 2048 914 -> 979 -> 777, 128 wide, 2048 570 -> 623 -> 459; of 256
     // 400 -> 302 -> 285, 508 -> 379 -> 330, 308 -> 272 -> 229.  Two waves: 597, 790, 470; 303, 349, 243.
-    const int slices = F / slice, groups = std::min((pc.M_cap + sub32::TOK - 1) / sub32::TOK, std::max(1, num_sms() / slices));
-    AD_TRY(launch_sublayer_f32<sub32::FFN>(h, dim3(groups, slices), slice, p, "ffn"));
+    const int slices = F / slice, tiles = (pc.M_cap + sub32::TOK - 1) / sub32::TOK, groups = std::max(1, num_sms() / slices);
+    if (tiles <= groups) AD_TRY(launch_sublayer_f32<sub32::FFN>(h, dim3(tiles, slices), slice, p, "ffn"));
+    else AD_TRY((launch_sublayer_f32<sub32::FFN, true>(h, dim3(groups, slices), slice, p, "ffn")));
     Partials ps = {};
     ps.ptr = h->pre; ps.nsplit = slices; ps.stride = p.stride;
     return layernorm(h, pc, ps, b2, lng, lnb, out);

@@ -47,7 +47,7 @@ def test_accept_kernels_fit_a_thousand_threads_without_spills(tmp_path):
 def test_sublayers_with_their_weights_in_registers_do_not_spill(tmp_path):
     few = [f"few::attention_few_kernel<{q}, {split}, {first}, {loop}>" for q in ("false", "true") for split in (1, 2) for first in ("false", "true")
            for loop in ("false", "true")] + ["few::ffn_few_kernel"]
-    f32 = [f"sub32::sublayer_f32_kernel<sub32::{kind}, {d}, {s}>" for kind in ("SELF", "CROSS", "FFN") for d in (128, 256) for s in (32, 64)]
+    f32 = [f"sub32::sublayer_f32_kernel<sub32::{kind}, {d}, {s}, {loop}>" for kind, loop in (("SELF", "false"), ("CROSS", "false"), ("FFN", "false"), ("FFN", "true")) for d in (128, 256) for s in (32, 64)]
     parts = [f"layernorm_parts_kernel<{a}>" for a in ("bf16", "float")]
     found = _report(tmp_path, few + f32 + parts)
     assert len(found) == len(few) + len(f32) + len(parts)
