@@ -1103,8 +1103,8 @@ int embed(ad_handle* h, const PassCfg& pc, const Model& m) {
 }
 
 // ---- FP32 sublayers of few tokens (sublayer_f32.cuh) ----
-// Whether the sublayers of pass pc run on these kernels: what they cover, up to five waves of CTAs of the attention at capacity (two, three, five allowed:
-// 256 wide, batch 24 2522, 2494, 2494 us a call, 3256 without them).
+// Whether the sublayers of pass pc run on these kernels: what they cover, up to five waves of CTAs of the attention at capacity.  256 wide, 3 + 3 layers, whole calls, the
+// projections' own kernels -> these: batch 24 (2.6 waves) 4834 -> 2977 us, 32 (3.5) 5430 -> 3457; full blocks of 1024 tokens (3.5 waves), four layers 689 -> 633.
 bool f32_sublayers(const ad_handle* h, const PassCfg& pc) {
   const ad_model_cfg& c = h->cfg;
   return !h->bf16 && h->pre2 && h->sw.fuse_attn_proj && pc.M_cap <= sub32::MAX_TOKENS && pc.pieces(c.max_batch, sub32::TOK) * c.n_heads <= 5L * num_sms();
@@ -1120,7 +1120,7 @@ cudaError_t launch_sublayer_f32_n(cudaStream_t st, dim3 grid, const sub32::Param
     if (e != cudaSuccess) return e;
     attr_set[dev] = true;
   }
-  // (one CTA an SM, like the projections around it: 256 wide, batch 6 1364 us a call with the runtime's choice, 1295)
+  // (one CTA an SM, like the projections around it; with the runtime's choice 256 wide, batch 6 1740 -> 1820 us a call, 128 wide, batch 6 776 -> 825, batch 32 1433 -> 1545)
   return launch_shared(one_cta_share(smem), sub32::sublayer_f32_kernel<KIND, D, S, LOOP>, grid, dim3(sub32::THREADS), smem, st, p);
 }
 template <sub32::Kind KIND, bool LOOP = false>

@@ -106,9 +106,9 @@ struct FewItems {
 // grid = (B * qchunks * SPLIT, H), qchunks = ceil(longest segment / 16); block = 32 * att_few_warps(d) threads; dynamic smem
 // att_few_smem; cluster (SPLIT, 1, 1) when QPROJ and SPLIT == 2.
 // LOOP: grid = (groups * SPLIT, H) of any size; the items that the pass has are dealt to the groups in runs, so that a CTA reads its weights
-// once and the keys and values of a row once for the queries of it that follow one another.  Taken where a grid that counts what the pass could
-// hold has more CTAs than there are SMs, one of which fits each: those came in waves, CTAs without work among them, and every one read 64 or
-// 128 KB of weights.  An item costs 2.7 us (128 keys) to 5.1 us (400 keys), the first as well as the following ones: it is a chain of five exchanges
+// once and the keys and values of a row once for the queries of it that follow one another.  Taken where the other grid, a CTA for every piece of the
+// longest block that a row could have, has more of them than there are SMs, one of which fits each: those came in waves, CTAs without work among them, and every one read
+// 64 or 128 KB of weights.  An item costs 2.7 us (128 keys) to 5.1 us (400 keys), the first as well as the following ones: it is a chain of five exchanges
 // between the warps with 1.3 us of MMAs in it.  Drafter's pass of 414 tokens, 512 wide, after the wait: self-attention 8.2 -> 7.6 us, cross-attention
 // over 400 keys 16.5 -> 12.2.  Whole calls: 768 wide, batch 6 4676 -> 4330 us, batch 8 with drafter 7732 -> 7464; 1024 wide, batch 4 5990 -> 5724, batch 3
 // with drafter 7233 -> 6991; 512 wide, batch 16, relaxed 2625 -> 2488.  Straight-line rounds (below) do not fit its registers: they spilled,

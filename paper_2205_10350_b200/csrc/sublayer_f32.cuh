@@ -4,9 +4,10 @@
 // As kernels of their own the projections are 2.1 us a piece, most of it boundary and round trips: eleven kernels a decoder layer.  With these it is
 // seven: QKV | attention + Wo | LayerNorm | Wq + attention + Wo | LayerNorm | W1 + W2 | LayerNorm.  A CTA owns a head (or a slice of the hidden features) and 16
 // tokens; its shares of both weight matrices are in registers before the dependency wait, and what it computes in between stays in shared memory.
-// What bounds them: one memory round trip, three to five barriers and, at 16 tokens, 512 to 1024 multiply-adds per thread.  Whole calls, before -> after, us: 128
-// wide, batch 1 575 -> 538, batch 6 1386 -> 913, batch 32 2224 -> 1735; 256 wide, batch 1 1163 -> 806, batch 6 2240 -> 1296, batch 24 3256 -> 2495.
-// All sums are FP32 multiply-adds.  The output projection leaves one partial sum per head (slice) for the LayerNorm to add.
+// What bounds them: one memory round trip, three to five barriers and, at 16 tokens, 512 to 1024 multiply-adds per thread.  Whole calls, sentences of 16 to 30
+// tokens, before -> after, us: 128 wide, 2 + 2 layers, batch 1 608 -> 551, batch 6 1155 -> 776, batch 32 1909 -> 1433, batch 5 with drafter 2022 -> 1240; 256 wide, 3 + 3 layers,
+// batch 1 1612 -> 1020, batch 6 2892 -> 1740, batch 24 4834 -> 2977.
+// All sums are FP32 multiply-adds.  The output projection leaves one partial sum per head (slice) for the LayerNorm to add (pairwise: see add_partials).
 #pragma once
 
 #include "attention.cuh"
@@ -39,8 +40,9 @@ struct Layout {
                        FLOATS = PS + TOK * KEYS;
 };
 
-// Products in four running sums, which keeps the chains of additions, and with them the rounding, as short as in the kernels that split K between half-warps (error
-// against 64 bits, 128 wide, batch 1 x 17: 4.9e-7 with those, 5.0e-7; in one running sum 5.8e-7, and a call takes 3 % less).
+// Products in four running sums, which keeps the chains of additions, and with them the rounding, as short as in the kernels that split K between half-warps.  Error of
+// the scores against 64 bits, two layers, rms, with those kernels / one running sum / four: 128 wide, batch 1 x 17 4.31e-8 / 4.33e-8 / 4.26e-8, 256 wide, batch 4 x 30 7.25e-8 /
+// 7.23e-8 / 7.17e-8.  In one sum a call takes 3 % less at 128 wide and up to 3 % more at 256.
 __device__ __forceinline__ void fma4(float4& s, float4 a, float4 b) {
   s.x = fmaf(a.x, b.x, s.x); s.y = fmaf(a.y, b.y, s.y); s.z = fmaf(a.z, b.z, s.z); s.w = fmaf(a.w, b.w, s.w);
 }
