@@ -153,19 +153,18 @@ def test_verified_blocks_see_their_own_keys_in_three_and_four_rounds(d, T, k, ke
     dec.close()
 
 
-@pytest.mark.parametrize("d,batch,k,src,rows,most", [
-    (512, 23, 1, 20, (0, 9, 22), 1),    # an item a row, more items than groups of CTAs by a handful
-    (512, 10, 33, 130, (0, 4, 9), 33),  # three items a row of which some are short, source keys in two rounds
-    (512, 40, 1, 260, (0, 31, 32, 39), 1),   # more rows than lanes; source keys in three rounds
-    (384, 35, 2, 10, (0, 17, 34), 2),   # six warps; the last lane's share of the rows is not full
-    (768, 4, 33, 100, (0, 1, 3), 33),   # pairs of CTAs whose halves of the queries meet once an item, keys in two rounds
-    (1024, 3, 40, 300, (0, 2), 40),     # the same with keys in three rounds
-    (512, 14, 64, 20, (0, 6, 13), 4),   # a layout for 64 tokens: fewer items than groups, long blocks are possible
-    (768, 9, 48, 70, (0, 8), 10),       # the same for 96 tokens and pairs of CTAs
+@pytest.mark.parametrize("d,batch,k,src,rows", [
+    (512, 23, 1, 20, (0, 9, 22)),       # an item a row, more items than groups of CTAs by a handful
+    (512, 10, 33, 130, (0, 4, 9)),      # three items a row of which some are short, source keys in two rounds
+    (512, 40, 1, 260, (0, 31, 32, 39)), # more rows than lanes; source keys in three rounds
+    (384, 35, 2, 10, (0, 17, 34)),      # six warps; the last lane's share of the rows is not full
+    (768, 4, 33, 100, (0, 1, 3)),       # pairs of CTAs whose halves of the queries meet once an item, keys in two rounds
+    (1024, 3, 40, 300, (0, 2)),         # the same with keys in three rounds
 ])
-def test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, rows, most):
+def test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, rows, most=None):
     """Attention of passes with more pieces of 16 queries than the device holds CTAs: one verified block of a ragged batch, idle rows among
-    the others, at an empty prefix and behind a committed one; sampled rows against the checker.  Blocks of at most `most` tokens."""
+    the others, at an empty prefix and behind a committed one; sampled rows against the checker.  Blocks of at most `most` tokens (None: k)."""
+    most = most or k
     from paper_2205_10350_b200 import binding
     shape = synth.ModelShape(f"loop_{d}", d, d // 64, 512, 1003, 1, 2, "bf16")
     w = synth.make_weights(shape, 0)
@@ -193,6 +192,14 @@ def test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, r
             last[b] = int(drafts[b, n[b] - 1])
         dec.force_commit(drafts, n)
     dec.close()
+
+
+@pytest.mark.parametrize("d,batch,k,src,rows,most", [
+    (512, 14, 64, 20, (0, 6, 13), 4),   # a layout for 64 tokens: fewer items than groups, long blocks are possible
+    (768, 9, 48, 70, (0, 8), 10),       # the same for 96 tokens and pairs of CTAs
+])
+def test_grids_that_loop_in_layouts_for_few_tokens_follow_the_checker(d, batch, k, src, rows, most):
+    test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, rows, most)
 
 
 @pytest.mark.parametrize("d,ffn,batch,k", [

@@ -233,8 +233,49 @@ def test_rows_of_a_loop_meet_in_a_cluster_or_through_global_memory(B, monkeypatc
     assert results[1] == results[0] and results[2] == results[0]
 
 
+BODY_CASES = [(512, 5, 13, "stream"), (512, 7, 14, "stream"), (512, 24, 40, "stream"), (512, 33, 9, "policy"), (512, 26, 40, "policy"), (768, 7, 14, "relaxed"),
+              (768, 20, 20, "policy"), (512, 5, 20, "drafter")]
+
+
+@pytest.mark.parametrize("d,B,k,how", BODY_CASES, ids=[f"{c[3]}-{c[0]}wide-{c[1]}rows-k{c[2]}" for c in BODY_CASES])
+def test_bodies_of_a_loop_for_few_and_many_tokens_give_the_same_sentences(d, B, k, how, monkeypatch):
+    """A decode loop picks its body by the tokens of each iteration; with one body for all of them (and with direct launches) the sentences and the
+    iterations are the same but for near-ties, and the launches that are counted are those of the bodies that ran."""
+    shape = synth.ModelShape(f"bodies_{d}", d, d // 64, 512, 1003, 1, 2, "bf16")
+    w = synth.make_weights(shape, 0)
+    wn = synth.make_weights(shape, 1) if how == "drafter" else None
+    r = np.random.default_rng(d + B * 7 + k)
+    T = max(24, k)
+    src = r.integers(4, 200, size=(B, T)).astype(np.int32)
+    lens = r.integers(T // 2, T + 1, size=B).astype(np.int32)
+    max_len = r.integers(4, T + 1, size=B).astype(np.int32)
+    max_len[0] = T
+    kw = dict(mode="IAD" if how == "policy" else "GAD", k=k, max_len=max_len)
+    if how == "drafter":
+        kw["run_drafter"] = True
+    elif how != "policy":
+        kw["draft_override"] = r.integers(4, shape.vocab, size=(B, T)).astype(np.int32)
+    runs = []
+    for one_body in ("0", "1"):
+        monkeypatch.setenv("AD_NO_FEW_BODY", one_body)
+        dec = binding.AggressiveDecoder(shape, w, wn, max_batch=B, max_src=T, max_tgt=T, kmax=k)
+        if how == "relaxed":
+            dec.set_acceptance(4, 0.5)
+        first, a = dec.generate(src, lens, **kw)
+        again, b = dec.generate(src, lens, **kw)
+        assert all(np.array_equal(x, y) for x, y in zip(first, again)) and a["kernel_launches"] == b["kernel_launches"]
+        direct, s = dec.generate(src, lens, use_graph=False, **kw)
+        runs += [(first, a), (direct, s)]
+        if one_body == "1":
+            assert a["kernel_launches"] >= a["iterations"] * 10
+        dec.close()
+    same = [sum(np.array_equal(x, y) for x, y in zip(runs[0][0], other[0])) for other in runs[1:]]
+    print(f"{how} {d} wide B={B} k={k}: rows the same {same}, iterations {[x[1]['iterations'] for x in runs]}, launches {[x[1]['kernel_launches'] for x in runs]}")
+    assert min(same) >= B - max(1, B // 4)
+
+
 # capacities just beyond what one form holds (96 tokens, 128 for the policy) and far beyond
-BODY_CASES = [(512, 7, 14, "stream"), (512, 24, 40, "stream"), (512, 33, 9, "policy"), (512, 10, 13, "policy"), (768, 7, 14, "relaxed"),
+FOLLOWING_CASES = [(512, 7, 14, "stream"), (512, 24, 40, "stream"), (512, 33, 9, "policy"), (512, 10, 13, "policy"), (768, 7, 14, "relaxed"),
               (768, 20, 20, "policy"), (512, 5, 20, "drafter")]
 BETA, TAU = 4, 0.5
 
@@ -256,8 +297,8 @@ def _parts_at_a_near_tie(model, src, a, b, draft):
     return min(abs(top[0] - d - TAU), abs(top[BETA - 1] - d), abs(top[BETA] - d)) <= 0.1
 
 
-@pytest.mark.parametrize("d,B,k,how", BODY_CASES, ids=[f"{c[3]}-{c[0]}wide-{c[1]}rows-k{c[2]}" for c in BODY_CASES])
-def test_bodies_of_a_loop_for_few_and_many_tokens_give_the_same_sentences(d, B, k, how, monkeypatch):
+@pytest.mark.parametrize("d,B,k,how", FOLLOWING_CASES, ids=[f"{c[3]}-{c[0]}wide-{c[1]}rows-k{c[2]}" for c in FOLLOWING_CASES])
+def test_bodies_of_a_loop_differ_at_near_ties_alone(d, B, k, how, monkeypatch):
     """A decode loop picks its body by the tokens of each iteration; with one body for all of them and with direct launches the sentences are the
     same or part at a near-tie, and so are the iterations where all sentences are the same and the drafts do not come from the drafter."""
     shape = synth.ModelShape(f"bodies_{d}", d, d // 64, 512, 1003, 1, 2, "bf16")
