@@ -837,9 +837,15 @@ cudaError_t launch_attention(dim3 grid, dim3 block, cudaStream_t st, const AttnP
   return launch_shared(share, attention_kernel<T, D, Q, FUSE, MINB>, grid, block, smem, st, p);
 }
 
-// Whether a pass of a model up to 512 wide has, at its capacity, work for at most three waves of the few-query kernel's CTAs (attention_few.cuh).
-bool within_three_waves(const ad_handle* h, const PassCfg& pc) {
-  return few::att_few_split(h->cfg.d_model) == 1 && pc.pieces(h->cfg.max_batch, few::AQ) * h->cfg.n_heads <= 3L * num_sms();
+// Whether a verification pass has, at its capacity, work for at most three waves (beyond 512 wide four) of the few-query kernel's CTAs (attention_few.cuh).
+bool within_few_waves(const ad_handle* h, const PassCfg& pc) {
+  const int split = few::att_few_split(h->cfg.d_model);
+  return pc.pieces(h->cfg.max_batch, few::AQ) * h->cfg.n_heads * split <= (split > 1 ? 4L : 3L) * num_sms();
+}
+// Whether the grid of the FFMA kernel, a CTA for every eight queries that a row could have, is too large for it.  It counts CTAs without work as well, in layouts for few tokens
+// most of them: 13 to 24 rows of one token in blocks of up to 64, 768 wide, counted by the work there can be (FFMA kernel) -> by the grid (MMA), four layers, 178 -> 138, 308 -> 149 us.
+bool many_queries(const ad_handle* h, const PassCfg& pc, int rows) {
+  return (long)rows * ((pc.seg_max + 7) / 8) * h->cfg.n_heads > 3L * num_sms();
 }
 
 int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, const void* v, void* out,
@@ -854,7 +860,7 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
   p.d = c.d_model;
   // one query per warp while the grid stays within a couple of waves, eight when there are many queries
   const int dh = c.d_model / c.n_heads;
-  const bool many = pc.pieces(h->dims.B, 8) * c.n_heads > 3L * num_sms();
+  const bool many = many_queries(h, pc, h->dims.B);
   p.scale = 1.0f / sqrtf((float)dh);
   // Tensor-core kernels when there are thousands of queries or rows may hold hundreds of keys (max_keys: the capacity, known on
   // the host); the FFMA kernel spreads few queries and few keys over more CTAs.
@@ -868,8 +874,9 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
     // What the FFMA kernel would do with FP32 probabilities keeps them (two BF16 numbers each; 0 to 5 us of such a call more than with one):
     // memory of one layer dominated by its attention, 27 sizes of 256 to 1024 wide: error against 64 bits within 0.03 % of the FFMA kernel's,
     // 0.3 to 1.8 % above it with probabilities rounded to BF16.
-    // So do verification passes that the few-query kernel takes where their tokens are not known (see attention_is_few).
-    const bool split_p = (!many || (&pc == &h->pass[PK_VERIFY] && within_three_waves(h, pc))) && max_keys < 256;
+    // So do layouts for few tokens whose grid alone is many, and verification passes within the most waves that the few-query kernel takes (see attention_is_few).
+    const bool many_work = pc.pieces(h->dims.B, 8) * c.n_heads > 3L * num_sms();
+    const bool split_p = (!many_work || (&pc == &h->pass[PK_VERIFY] && within_few_waves(h, pc))) && max_keys < 256;
     // Warps share a 16-query tile and split the keys (2 or 4 key groups) when rows have few queries; two groups also while
     // 64-query CTAs would not give every SM two.
     const long full = (long)h->dims.B * ((pc.seg_max + AM_Q - 1) / AM_Q) * c.n_heads;
@@ -941,13 +948,17 @@ int attention(ad_handle* h, const PassCfg& pc, const void* q, const void* k, con
 // Whether the few-query kernel (attention_few.cuh) serves an attention of pass pk: BF16, 64-wide heads, the keys within four rounds
 // of its warps, and work for a few waves of CTAs at most, counted by what the pass could hold (rows that have ended, shorter blocks and a
 // drafter's prefix that has not grown leave less).  A wave costs 4 to 7 us, the projections that
-// are kernels of their own otherwise 12 us a layer, so a verification pass may need three waves at capacity (four beyond 512 wide), a drafter's pass (on
+// are kernels of their own otherwise 12 us a layer, so a verification pass may need three waves at capacity, a drafter's pass (on
 // average half of its capacity) four.  Per decode iteration, one wave allowed -> this rule: base model, batch 12, blocks of 30:
 // 214 -> 174 us; batch 24, 12: 237 -> 196; batch 20, 1: 188 -> 160; batch of 5 with drafter 442 -> 373; 1024 wide, batch 2, 40: 272 -> 226;
 // batch 3 with drafter 662 -> 600.  Beyond: base batch 32 x 64 (seven waves) 270 -> 315, 1024 wide batch 16 x 1 (four) 239 -> 284.  Wide
 // models with fewer than eight queries a row stay at one wave: their CTAs read two weight slices each for a tile that is mostly padding
 // (768 wide, batch 12, 1: 202 against 210).  Looping grids, waves 2 / 2.5 / 3 / 3.5 / 4 / 4.5, whole calls: 512 wide, batch 20 5068 / 5046 / 5073 / 5147 / 5350 / 5443,
-// batch 16, relaxed 2379 / 2375 / 2482 / 2483 / 2481 / 2480; from 3 on, 1024 wide, batch 8 5350 / 4873 / 5028 / 5078, 768 wide, batch 16 4786 / 4781 / 4409 / 4479.
+// batch 16, relaxed 2379 / 2375 / 2482 / 2483 / 2481 / 2480.
+// Beyond 512 wide the few-query kernel is taken up to four waves only where the FFMA kernel would run instead, and not for blocks of eight, which fill that kernel's CTAs.
+// Full blocks of 130 source tokens, four layers, between three and four waves, few-query kernel / the other one, us: FFMA 768 wide 11 x 18 274 / 351, 1024 wide 8 x 18 298 / 380,
+// 768 wide 20 x 8 261 / 248; MMA 768 wide 8 x 48 293 / 243, 11 x 30 292 / 239, 20 x 10 277 / 233, 1024 wide 6 x 48 369 / 281, 8 x 30 324 / 276, 16 x 10 308 / 261.
+// With 256 keys or more, where the other kernels round the probabilities, four.
 // Layouts that the tokens pick hold as many as they are made for, and with 384 and 512 wide models two and a half waves are the line there; the MMA kernel
 // beyond keeps FP32's probabilities up to three waves, as this one does (split_p in attention).  It does so for fewer than 256 keys, with more the line stays at three waves.
 // A layout that has to hold whatever comes (device arrays) is mostly emptier than its capacity: verified blocks, two and a half waves for it as well -> three, 512 wide,
@@ -965,8 +976,9 @@ bool attention_is_few(const ad_handle* h, int pk, int max_keys) {
   if (max_keys > few::MAX_ROUNDS * few::AK * few::att_few_warps(c.d_model)) return false;
   // (in half waves)
   const bool one_wave = pk == PK_ENCODE ? split > 1 || max_keys >= 256 || (pc.seg_max <= 8 && c.d_model > 256) : split > 1 && pc.seg_max < 8;
-  const bool half_less = pc.few_cap == 0 && few::att_few_warps(c.d_model) > 4 && std::max(c.max_src, c.max_tgt) < 256;
-  const int waves = one_wave ? 2 : pk == PK_ENCODE ? 3 : pk == PK_DRAFT || split > 1 ? 8 : half_less ? 5 : 6;
+  const bool wide_four = split > 1 && (std::max(c.max_src, c.max_tgt) >= 256 || (pc.seg_max > 8 && !many_queries(h, pc, c.max_batch)));
+  const bool half_less = pc.few_cap == 0 && split == 1 && few::att_few_warps(c.d_model) > 4 && std::max(c.max_src, c.max_tgt) < 256;
+  const int waves = one_wave ? 2 : pk == PK_ENCODE ? 3 : pk == PK_DRAFT || wide_four ? 8 : half_less ? 5 : 6;
   return 2 * pc.pieces(c.max_batch, few::AQ) * c.n_heads * split <= (long)waves * num_sms();
 }
 

@@ -61,9 +61,10 @@ def _scores(w, tok, memory, heads, rounded):
 
 
 # between two and a half and three waves of CTAs at capacity (148 SMs): 47 to 55 pieces of 16 queries at eight heads, 62 to 74 at six; source keys in one and
-# in three rounds
+# in three rounds; 768 wide between three and four: 19 to 24 pieces
 @pytest.mark.parametrize("which", ["self", "cross"])
-@pytest.mark.parametrize("d,B,k,S", [(512, 12, 64, 60), (512, 16, 40, 30), (512, 25, 25, 60), (384, 17, 60, 60), (512, 12, 60, 300)])
+@pytest.mark.parametrize("d,B,k,S", [(512, 12, 64, 60), (512, 16, 40, 30), (512, 25, 25, 60), (384, 17, 60, 60), (512, 12, 60, 300), (768, 11, 30, 60),
+                                       (768, 20, 10, 60)])
 def test_verified_blocks_round_only_where_operands_are_stored(d, B, k, S, which):
     shape = synth.ModelShape(f"precision_{d}", d, d // 64, 128, 1003, 1, 1, "bf16")
     w = _weights(shape, which)

@@ -197,6 +197,9 @@ def test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, r
 @pytest.mark.parametrize("d,batch,k,src,rows,most", [
     (512, 14, 64, 20, (0, 6, 13), 4),   # a layout for 64 tokens: fewer items than groups, long blocks are possible
     (768, 9, 48, 70, (0, 8), 10),       # the same for 96 tokens and pairs of CTAs
+    (768, 13, 18, 70, (0, 7, 12), 4),   # too many items for it: the MMA kernel, few queries in a grid for long blocks
+    (1024, 13, 64, 100, (0, 12), 7),    # the same, keys in two tiles
+    (768, 24, 64, 70, (0, 11, 23), 1),  # a query a row
 ])
 def test_grids_that_loop_in_layouts_for_few_tokens_follow_the_checker(d, batch, k, src, rows, most):
     test_grids_that_loop_over_the_queries_follow_the_checker(d, batch, k, src, rows, most)
