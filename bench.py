@@ -80,8 +80,8 @@ def reduce_max_sum(dist, dev, seconds_or_ms, count):
 # DRAM counters of one verification step (dram__bytes_read.sum + dram__bytes_write.sum summed over the step's
 # kernels, ncu, caches flushed before every kernel) with the digest of the kernel sources they were taken on:
 # the figures are reported only while the sources still have that digest.
-NCU_COUNTERS = dict(sources_sha256="6fa5fa8fa929c1d2b6ec52a8e7b81b27148cb373268858ee96cfc23cf8900c8c",
-                    step_block40_bytes=104937216, projection_bytes=32865024,
+NCU_COUNTERS = dict(sources_sha256="c216cf0249969fb925acd873e37ad3e6636032a2dc8321bcc0510fa5401777c5",
+                    step_block40_bytes=104946176, projection_bytes=32872960,
                     summary="profiles/verify_step_base_b1_k40_dram_traffic.txt")
 
 
